@@ -3,23 +3,52 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libflora.so")
+NATIVE = os.path.join(HERE, "_native.so")                      # Python side of binding.py (argument marshalling), g++ only
+NATIVE_SOURCE = "flora_py.cpp"
 SOURCES = ["flora_api.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared", "--fmad=false", "-Xptxas", "-v"]
 
 
 def _newest_source_mtime() -> float:
-    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != NATIVE_SOURCE]
     paths.append(os.path.join(os.path.dirname(HERE), "include", "flora.h"))
     return max(os.path.getmtime(p) for p in paths)
 
 
+def build_native(force: bool = False) -> str:
+    """Compile csrc/flora_py.cpp into paper_2402_03293_b200/_native.so (needs libflora.so, which it calls)."""
+    src = os.path.join(CSRC, NATIVE_SOURCE)
+    newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(os.path.dirname(HERE), "include", "flora.h")))
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
+        return NATIVE
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f"-I{root}/include", f"-I{root}/include/torch/csrc/api/include", "-I/usr/local/cuda/include",
+           f"-I{sysconfig.get_paths()['include']}", src, "-o", NATIVE + ".tmp", f"-L{root}/lib", "-ltorch_python", "-ltorch_cpu", "-lc10",
+           "-lc10_cuda", f"-L{HERE}", "-l:libflora.so", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode:
+        print(res.stderr)
+        raise RuntimeError("g++ failed building _native.so")
+    os.replace(NATIVE + ".tmp", NATIVE)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu into paper_2402_03293_b200/libflora.so if it is missing or stale."""
+    """Compile csrc/*.cu into paper_2402_03293_b200/libflora.so, and the Python side, where missing or stale."""
+    lib = build_library(force, verbose)
+    build_native(force)
+    return lib
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

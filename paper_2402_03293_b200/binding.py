@@ -1,6 +1,7 @@
-"""ctypes binding of libflora.so: same names as include/flora.h, argument marshalling only.
+"""Python binding of libflora.so: same names as include/flora.h, argument marshalling only.
 
-Every operation runs in the CUDA library; there is no fallback.  If the library has not been
+The calls of a training step go through a small native module (csrc/flora_py.cpp: reading a tensor's C++ object takes tens of
+nanoseconds, building a flora_mat through ctypes microseconds); set-up and diagnostics use ctypes.  Every operation runs in the CUDA library; there is no fallback.  If the library has not been
 built (``python -c "import __graft_entry__ as g; g.build()"`` or
 ``python paper_2402_03293_b200/_build.py``) loading it raises.  PyTorch is used here for device
 memory (tensors) and streams only.
@@ -8,6 +9,8 @@ memory (tensors) and streams only.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import List, Optional, Sequence
 
@@ -97,6 +100,25 @@ def load() -> ctypes.CDLL:
     return _lib
 
 
+class _Unloaded:
+    """Stands for the native module until the first call: loads it (and the library) and puts it in its own place."""
+
+    def __getattr__(self, name):
+        global _native
+        load()
+        path = os.path.join(HERE, "_native.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build the library first (__graft_entry__.build())")
+        loader = importlib.machinery.ExtensionFileLoader("_native", path)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_native", loader))
+        loader.exec_module(module)
+        _native = module
+        return getattr(module, name)
+
+
+_native = _Unloaded()
+
+
 def status_string(status: int) -> str:
     return load().flora_status_string(status).decode()
 
@@ -142,33 +164,33 @@ def _dt(dtype) -> int:
 
 # ---------------------------------------------------------------------------------- single-matrix calls
 def flora_compress_accumulate(G: torch.Tensor, C: torch.Tensor, seed: int, r: int, stream=None) -> None:
-    g, c = mat(G), mat(C)
-    _check(load().flora_compress_accumulate(ctypes.byref(g), ctypes.byref(c), seed, r, _stream(stream)),
-           "flora_compress_accumulate")
+    st = _native.compress_accumulate(G, C, seed, r, stream)
+    if st:
+        raise FloraError(st, "flora_compress_accumulate")
 
 
 def flora_decompress_apply(W: torch.Tensor, C: torch.Tensor, seed: int, lr: float, scale: float, stream=None) -> None:
-    w, c = mat(W), mat(C)
-    _check(load().flora_decompress_apply(ctypes.byref(w), ctypes.byref(c), seed, lr, scale, _stream(stream)),
-           "flora_decompress_apply")
+    st = _native.decompress_apply(W, C, seed, lr, scale, stream)
+    if st:
+        raise FloraError(st, "flora_decompress_apply")
 
 
 def flora_momentum_step(G: torch.Tensor, M: torch.Tensor, beta: float, seed: int, stream=None) -> None:
-    g, m_ = mat(G), mat(M)
-    _check(load().flora_momentum_step(ctypes.byref(g), ctypes.byref(m_), beta, seed, _stream(stream)),
-           "flora_momentum_step")
+    st = _native.momentum_step(G, M, beta, seed, stream)
+    if st:
+        raise FloraError(st, "flora_momentum_step")
 
 
 def flora_momentum_step_resampled(G: torch.Tensor, M: torch.Tensor, beta: float, seed_old: int, seed_new: int, stream=None) -> None:
-    g, m_ = mat(G), mat(M)
-    _check(load().flora_momentum_step_resampled(ctypes.byref(g), ctypes.byref(m_), beta, seed_old, seed_new, _stream(stream)),
-           "flora_momentum_step_resampled")
+    st = _native.momentum_step_resampled(G, M, beta, seed_old, seed_new, stream)
+    if st:
+        raise FloraError(st, "flora_momentum_step_resampled")
 
 
 def flora_resample_transfer(M: torch.Tensor, m: int, operand, seed_old: int, seed_new: int, stream=None) -> None:
-    m_ = mat(M)
-    _check(load().flora_resample_transfer(ctypes.byref(m_), m, _dt(operand), seed_old, seed_new, _stream(stream)),
-           "flora_resample_transfer")
+    st = _native.resample_transfer(M, m, _dt(operand), seed_old, seed_new, stream)
+    if st:
+        raise FloraError(st, "flora_resample_transfer")
 
 
 def flora_resample_transfer_static(M: torch.Tensor, m: int, operand, seed_old: int, seed_new: int, stream=None) -> None:
@@ -181,9 +203,9 @@ def flora_resample_transfer_static(M: torch.Tensor, m: int, operand, seed_old: i
 
 def flora_transfer_axpby(dst: torch.Tensor, src: torch.Tensor, m: int, operand, seed_old: int, seed_new: int,
                          a: float, b: float, stream=None) -> None:
-    d, s = mat(dst), mat(src)
-    _check(load().flora_transfer_axpby(ctypes.byref(d), ctypes.byref(s), m, _dt(operand), seed_old, seed_new, a, b,
-                                       _stream(stream)), "flora_transfer_axpby")
+    st = _native.transfer_axpby(dst, src, m, _dt(operand), seed_old, seed_new, a, b, stream)
+    if st:
+        raise FloraError(st, "flora_transfer_axpby")
 
 
 def flora_materialize_A(out: torch.Tensor, seed: int, stream=None) -> None:
@@ -193,7 +215,15 @@ def flora_materialize_A(out: torch.Tensor, seed: int, stream=None) -> None:
 
 # ---------------------------------------------------------------------------------- host helpers
 def flora_derive_seed(base: int, matrix: int, epoch: int) -> int:
-    return int(load().flora_derive_seed(base, matrix, epoch))
+    return _native.derive_seed(base, matrix, epoch)
+
+
+def derive_seeds(base: int, count: int, epoch: int) -> "SeedList":
+    """flora_derive_seed for the matrices 0 .. count - 1, in one call."""
+    values, raw = _native.derive_seeds(base, count, epoch)
+    seeds = SeedList(values)
+    seeds._marshalled = (ctypes.c_uint64 * count).from_buffer_copy(raw) if count else (ctypes.c_uint64 * 0)()
+    return seeds
 
 
 def flora_resamples_at(t: int, kappa: int) -> bool:
@@ -301,39 +331,53 @@ class FloraSet:
             pass
 
     def rebind_gradients(self, G: List[torch.Tensor], stream=None) -> None:
-        _check(load().flora_set_rebind_gradients(self._h, _mat_array(G), _stream(stream)), "flora_set_rebind_gradients")
+        if len(G) != self.count:
+            raise ValueError("expected one gradient per matrix")
+        st = _native.set_rebind(self._handle(), G, stream)
+        if st:
+            raise FloraError(st, "flora_set_rebind_gradients")
         self.G = G
 
+    def _handle(self) -> int:
+        h = self._h
+        return h.value or 0 if h is not None else 0          # a closed set: the library answers FLORA_ERR_NULL
+
     def compress_accumulate(self, seeds: Sequence[int], stream=None) -> None:
-        _check(load().flora_set_compress_accumulate(self._h, _u64_array(seeds), _stream(stream)),
-               "flora_set_compress_accumulate")
+        st = _native.set_compress_accumulate(self._handle(), self.count, _u64_array(seeds), stream)
+        if st:
+            raise FloraError(st, "flora_set_compress_accumulate")
 
     def momentum_step(self, beta: float, seeds: Sequence[int], stream=None) -> None:
-        _check(load().flora_set_momentum_step(self._h, beta, _u64_array(seeds), _stream(stream)),
-               "flora_set_momentum_step")
+        st = _native.set_momentum_step(self._handle(), self.count, beta, _u64_array(seeds), stream)
+        if st:
+            raise FloraError(st, "flora_set_momentum_step")
 
     def compress_overwrite(self, seeds: Sequence[int], stream=None) -> None:
         """C <- G A^T: the first compression of an accumulation cycle, which makes zeroing C beforehand unnecessary
         (flora_set_momentum_step with beta = 0: the old sketch is neither read nor blended in)."""
-        _check(load().flora_set_momentum_step(self._h, 0.0, _u64_array(seeds), _stream(stream)),
-               "flora_set_momentum_step")
+        self.momentum_step(0.0, seeds, stream)
 
     def decompress_apply(self, seeds: Sequence[int], lr: float, scale: float, stream=None) -> None:
-        _check(load().flora_set_decompress_apply(self._h, _u64_array(seeds), lr, scale, _stream(stream)),
-               "flora_set_decompress_apply")
+        st = _native.set_decompress_apply(self._handle(), self.count, _u64_array(seeds), lr, scale, stream)
+        if st:
+            raise FloraError(st, "flora_set_decompress_apply")
 
     def resample_transfer(self, seeds_old: Sequence[int], seeds_new: Sequence[int], stream=None) -> None:
-        _check(load().flora_set_resample_transfer(self._h, _u64_array(seeds_old), _u64_array(seeds_new),
-                                                  _stream(stream)), "flora_set_resample_transfer")
+        st = _native.set_resample_transfer(self._handle(), self.count, _u64_array(seeds_old), _u64_array(seeds_new), stream)
+        if st:
+            raise FloraError(st, "flora_set_resample_transfer")
 
     def transfer_axpby_from(self, src: "FloraSet", seeds_old: Sequence[int], seeds_new: Sequence[int], a: float, b: float, stream=None) -> None:
         """self.S[i] <- b self.S[i] + a src.S[i] A(seeds_old[i]) A(seeds_new[i])^T for every matrix."""
-        _check(load().flora_set_transfer_axpby(self._h, src._h, _u64_array(seeds_old), _u64_array(seeds_new), a, b, _stream(stream)),
-               "flora_set_transfer_axpby")
+        h = src._h if isinstance(src._h, int) else (src._h.value if src._h is not None else 0)
+        st = _native.set_transfer_axpby(self._handle(), h or 0, self.count, _u64_array(seeds_old), _u64_array(seeds_new), a, b, stream)
+        if st:
+            raise FloraError(st, "flora_set_transfer_axpby")
 
     def momentum_step_resampled(self, beta: float, seeds_old: Sequence[int], seeds_new: Sequence[int], stream=None) -> None:
-        _check(load().flora_set_momentum_step_resampled(self._h, beta, _u64_array(seeds_old), _u64_array(seeds_new),
-                                                        _stream(stream)), "flora_set_momentum_step_resampled")
+        st = _native.set_momentum_step_resampled(self._handle(), self.count, beta, _u64_array(seeds_old), _u64_array(seeds_new), stream)
+        if st:
+            raise FloraError(st, "flora_set_momentum_step_resampled")
 
     def zero_state(self, stream=None) -> None:
         _check(load().flora_set_zero_state(self._h, _stream(stream)), "flora_set_zero_state")

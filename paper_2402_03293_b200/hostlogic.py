@@ -16,7 +16,7 @@ def _derived(cache: dict, base_seed: int, count: int, epoch: int):
     if epoch not in cache:
         if len(cache) > 4:
             cache.clear()
-        cache[epoch] = binding.SeedList(binding.flora_derive_seed(base_seed, i, epoch) for i in range(count))
+        cache[epoch] = binding.derive_seeds(base_seed, count, epoch)
     return cache[epoch]
 
 
