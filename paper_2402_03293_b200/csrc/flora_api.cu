@@ -1,7 +1,8 @@
 // C ABI of the Flora hot path (see include/flora.h for the contract of every entry point).
 // This file validates arguments, picks a kernel family and launches; all arithmetic of the path
-// lives in the kernels of flora_simt.cuh (fp32 SIMT), flora_tc.cuh (tcgen05 tensor cores; host side in flora_tc_host.cuh)
-// and flora_gram.cuh (momentum transfer).
+// lives in the kernels of flora_tc.cuh and flora_pair*.cuh (bf16 matrices that TMA can address; host side in
+// flora_tc_host.cuh), flora_gen.cuh (fp32, unaligned and small matrices; host side in flora_gen_host.cuh), flora_gram.cuh
+// (momentum transfer) and flora_simt.cuh (plain fp32 arithmetic: fp32 transfers, and a second opinion for tests).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -18,6 +19,7 @@
 #include "flora_simt.cuh"
 #include "flora_pool.cuh"
 #include "flora_tc_host.cuh"
+#include "flora_gen_host.cuh"
 #include "flora_gram.cuh"
 
 using namespace flora;
@@ -173,6 +175,7 @@ flora_status static_scratch_for_current_device(float** out)
     return FLORA_OK;
 }
 
+bool use_gen(const flora_mat* big) { return g_force_path.load(std::memory_order_relaxed) != 1 && gen_supported(*big); }
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 {
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch);
@@ -191,8 +194,50 @@ struct flora_set {
     std::vector<flora_mat> G, W, S;
     int r = 0;
     bool has_G = false, has_W = false;
-    TcSet tc;   // tensor-core work lists and descriptors (empty when the set is not eligible)
+    TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
+    GenSet gen_g[2], gen_w[2];     // the others, by dtype
 };
+
+// Below this many elements the matrices of a mixed set that TMA could serve are not worth a launch of their own (4 M
+// elements are 8 MB, a microsecond and a half of HBM time): all its matrices then go to the kernels of flora_gen.cuh.
+constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
+
+// Which matrices of one side (G or W) of a set the TMA kernels serve.
+static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S)
+{
+    std::vector<uint8_t> use = tc_eligible(big, S);
+    int64_t eligible = 0;
+    bool mixed = false;
+    for (size_t i = 0; i < big.size(); ++i) {
+        if (use[i]) eligible += big[i].rows * big[i].cols;
+        else mixed = mixed || big[i].rows > 0;
+    }
+    if (mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) std::fill(use.begin(), use.end(), (uint8_t)0);
+    return use;
+}
+
+// Builds (or builds again) the work lists of a set for its present pointers.
+static flora_status set_build(flora_set* s)
+{
+    tc_set_free(s->tc);
+    s->tc = TcSet();
+    for (int d = 0; d < 2; ++d) {
+        gen_set_free(s->gen_g[d]);
+        gen_set_free(s->gen_w[d]);
+    }
+    const std::vector<uint8_t> use_g = set_tma_side(s->G, s->S), use_w = set_tma_side(s->W, s->S);
+    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, false, nullptr, use_g, use_w);
+    for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
+        std::vector<int> g, w;
+        for (size_t i = 0; i < s->S.size(); ++i) {
+            if (s->has_G && !use_g[i] && s->G[i].dtype == d && s->G[i].rows > 0 && gen_supported(s->G[i])) g.push_back((int)i);
+            if (s->has_W && !use_w[i] && s->W[i].dtype == d && s->W[i].rows > 0 && gen_supported(s->W[i])) w.push_back((int)i);
+        }
+        st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g);
+        if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w);
+    }
+    return st;
+}
 
 extern "C" {
 
@@ -203,6 +248,7 @@ flora_status flora_compress_accumulate(const flora_mat* G, flora_mat* C, uint64_
     if (r != C->cols) return FLORA_ERR_RANK;
     if (G->rows == 0 || G->cols == 0) return FLORA_OK;
     if (use_tc_compress(G, C)) return tc_compress_single(G, C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
+    if (use_gen(G)) return gen_compress_single(*G, *C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
     return simt_compress(G, C, seed, 1.0f, 1.0f, as_stream(stream));
 }
 
@@ -212,6 +258,7 @@ flora_status flora_momentum_step(const flora_mat* G, flora_mat* M, float beta, u
     if (st) return st;
     if (G->rows == 0) return FLORA_OK;
     if (G->cols > 0 && use_tc_compress(G, M)) return tc_compress_single(G, M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
+    if (use_gen(G)) return gen_compress_single(*G, *M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
     return simt_compress(G, M, seed, 1.0f - beta, beta, as_stream(stream));
 }
 
@@ -224,6 +271,7 @@ flora_status flora_momentum_step_resampled(const flora_mat* G, flora_mat* M, flo
     st = flora_transfer_axpby(M, M, G->cols, G->dtype, seed_old, seed_new, beta, 0.0f, stream);
     if (st) return st;
     if (G->cols > 0 && use_tc_compress(G, M)) return tc_compress_single(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
+    if (use_gen(G)) return gen_compress_single(*G, *M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
     return simt_compress(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream));
 }
 
@@ -233,6 +281,7 @@ flora_status flora_decompress_apply(flora_mat* W, const flora_mat* C, uint64_t s
     if (st) return st;
     if (W->rows == 0 || W->cols == 0) return FLORA_OK;
     if (use_tc_decompress(W, C)) return tc_decompress_single(W, C, seed, lr * scale, as_stream(stream), g_launches);
+    if (use_gen(W)) return gen_decompress_single(*W, *C, seed, lr * scale, as_stream(stream), g_launches);
     return simt_decompress(W, C, seed, lr * scale, as_stream(stream));
 }
 
@@ -331,10 +380,9 @@ flora_status flora_set_create(int count, const flora_mat* G, const flora_mat* W,
     s->S.assign(S, S + count);
     if (G) s->G.assign(G, G + count);
     if (W) s->W.assign(W, W + count);
-    flora_status st = tc_set_build(s->tc, s->G, s->W, s->S);
+    flora_status st = set_build(s);
     if (st) {
-        tc_set_free(s->tc);
-        delete s;
+        flora_set_destroy(s);
         return st;
     }
     *out = s;
@@ -345,6 +393,10 @@ flora_status flora_set_destroy(flora_set* set)
 {
     if (!set) return FLORA_OK;
     tc_set_free(set->tc);
+    for (int d = 0; d < 2; ++d) {
+        gen_set_free(set->gen_g[d]);
+        gen_set_free(set->gen_w[d]);
+    }
     delete set;
     return FLORA_OK;
 }
@@ -361,6 +413,12 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
     }
     std::vector<flora_mat> newG(G, G + set->G.size());
     flora_status st = tc_set_rebind(set->tc, newG, as_stream(stream));
+    if (st == FLORA_ERR_ALIGN && (set->gen_g[0].ready() || set->gen_g[1].ready())) {
+        // a mixed set takes any address: the matrix changes sides (work that still reads the old tables ends first)
+        set->G.swap(newG);
+        return cudaStreamSynchronize(as_stream(stream)) == cudaSuccess ? set_build(set) : FLORA_ERR_CUDA;
+    }
+    for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_rebind(set->gen_g[d], newG, as_stream(stream));
     if (st) return st;
     set->G.swap(newG);
     return FLORA_OK;
@@ -371,10 +429,15 @@ static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a,
 {
     if (!set || !seeds) return FLORA_ERR_NULL;
     if (!set->has_G) return FLORA_ERR_UNSUPPORTED;
-    if (set->tc.compress_ready && g_force_path.load() != 1)
-        return tc_set_compress(set->tc, seeds, a, b, as_stream(stream), g_launches, behind_own_transfer);
+    const bool simt = g_force_path.load() == 1;
+    if (!simt) {
+        flora_status st = FLORA_OK;
+        if (set->tc.compress_ready) st = tc_set_compress(set->tc, seeds, a, b, as_stream(stream), g_launches, behind_own_transfer);
+        for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_compress(set->gen_g[d], seeds, a, b, as_stream(stream), g_launches);
+        if (st) return st;
+    }
     for (size_t i = 0; i < set->G.size(); ++i) {
-        if (set->G[i].rows == 0) continue;
+        if (set->G[i].rows == 0 || (!simt && gen_supported(set->G[i]))) continue;
         flora_status st = simt_compress(&set->G[i], &set->S[i], seeds[i], a, b, as_stream(stream));
         if (st) return st;
     }
@@ -395,10 +458,15 @@ flora_status flora_set_decompress_apply(flora_set* set, const uint64_t* seeds, f
 {
     if (!set || !seeds) return FLORA_ERR_NULL;
     if (!set->has_W) return FLORA_ERR_UNSUPPORTED;
-    if (set->tc.decompress_ready && g_force_path.load() != 1)
-        return tc_set_decompress(set->tc, seeds, lr * scale, as_stream(stream), g_launches);
+    const bool simt = g_force_path.load() == 1;
+    if (!simt) {
+        flora_status st = FLORA_OK;
+        if (set->tc.decompress_ready) st = tc_set_decompress(set->tc, seeds, lr * scale, as_stream(stream), g_launches);
+        for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_decompress(set->gen_w[d], seeds, lr * scale, as_stream(stream), g_launches);
+        if (st) return st;
+    }
     for (size_t i = 0; i < set->W.size(); ++i) {
-        if (set->W[i].rows == 0 || set->W[i].cols == 0) continue;
+        if (set->W[i].rows == 0 || set->W[i].cols == 0 || (!simt && gen_supported(set->W[i]))) continue;
         flora_status st = simt_decompress(&set->W[i], &set->S[i], seeds[i], lr * scale, as_stream(stream));
         if (st) return st;
     }

@@ -1,0 +1,711 @@
+// Tensor-core kernels for what the TMA kernels cannot take: fp32 matrices, and matrices or sketches whose rows start at
+// addresses that TMA cannot name, or that are smaller than a TMA tile.
+//
+//   gen_compress_kernel     S <- b S + a G A^T     (Algorithm 1 compression; Algorithm 2 update of M)
+//   gen_decompress_kernel   W <- W - step * S A    (Algorithm 1 decompression fused with the update)
+//
+// fp32 operands are cut into three bf16 parts, x = h + m + l, by truncation: h and m hold eight significant bits each, l
+// the remaining eight, so the cut loses nothing.  The product of two fp32 values is then the sum of six exact products of
+// parts (h h, h m, m h, m m, h l, l h; the three left out are together below 2^-23 of the product, under the rounding of
+// the fp32 sum they join), and the tensor core adds them up in fp32.  That is six bf16 MMAs where plain fp32 arithmetic
+// spent r multiply-adds per element of G on the ALUs.
+#pragma once
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "flora_ptx.cuh"
+#include "flora_rng.cuh"
+#include "flora_tc.cuh"
+
+namespace flora {
+
+struct GenMat {            // a matrix with its sketch
+    void* big;             // G or W
+    float* S;
+    int64_t ld, lds;
+    int32_t n, m;
+};
+struct GenItem {           // compression: one cluster
+    int32_t mat;
+    int32_t tile0;         // first 128-row tile
+    int32_t split;         // CTAs of the cluster that share the columns of one row group
+    int32_t pad;
+};
+
+constexpr int GEN_WORKERS = 8;                              // warps that load, convert, generate and write out
+constexpr int GEN_THREADS = 32 * (GEN_WORKERS + 1);         // and one that issues the MMAs
+constexpr int GEN_STAGES_MAX = 4;
+
+// Parts of an fp32 value.
+struct Parts {
+    uint32_t h, m, l;      // fp32 bit patterns whose low 16 bits are zero
+};
+__device__ __forceinline__ Parts split3(float x)
+{
+    Parts p;
+    p.h = __float_as_uint(x) & 0xFFFF0000u;
+    const float r1 = __fsub_rn(x, __uint_as_float(p.h));                            // exact
+    p.m = __float_as_uint(r1) & 0xFFFF0000u;
+    p.l = __float_as_uint(__fsub_rn(r1, __uint_as_float(p.m)));                     // exact
+    return p;
+}
+// Two bf16 values from the high halves of two fp32 bit patterns; `a` goes into the low half.
+__device__ __forceinline__ uint32_t pack_high(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
+
+// Operand tiles in shared memory: rows of ROWB = 64 or 128 bytes (K-major), swizzled over 16-byte chunks as the tensor core
+// expects (64-byte rows: chunk ^ (row / 2) % 4; 128-byte rows: chunk ^ row % 8).
+template <int ROWB>
+__device__ __forceinline__ uint32_t operand_offset(int row, int chunk)
+{
+    return (uint32_t)(row * ROWB + ((ROWB == 64 ? chunk ^ ((row >> 1) & 3) : chunk ^ (row & 7)) << 4));
+}
+template <int ROWB>
+__device__ __forceinline__ uint64_t operand_desc(uint32_t addr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFF);                  // start address
+    d |= (uint64_t)1 << 16;                                 // leading byte offset (unused for swizzled K-major)
+    d |= (uint64_t)((8 * ROWB) >> 4) << 32;                 // stride byte offset: next eight-row group
+    d |= (uint64_t)1 << 46;                                 // descriptor version of sm_100
+    d |= (uint64_t)(ROWB == 64 ? 4 : 2) << 61;              // 64- or 128-byte swizzle
+    return d;
+}
+// Stores four fp32 values as `PARTS` (3: exact cut, 1: rounded to bf16) bf16 quads; `part_bytes` apart.
+template <int PARTS>
+__device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, float x0, float x1, float x2, float x3)
+{
+    if (PARTS == 3) {
+        const Parts p0 = split3(x0), p1 = split3(x1), p2 = split3(x2), p3 = split3(x3);
+        ptx::st_shared_v2(addr, pack_high(p0.h, p1.h), pack_high(p2.h, p3.h));
+        ptx::st_shared_v2(addr + part_bytes, pack_high(p0.m, p1.m), pack_high(p2.m, p3.m));
+        ptx::st_shared_v2(addr + 2 * part_bytes, pack_high(p0.l, p1.l), pack_high(p2.l, p3.l));
+    } else {
+        __nv_bfloat162 lo = __floats2bfloat162_rn(x0, x1), hi = __floats2bfloat162_rn(x2, x3);
+        ptx::st_shared_v2(addr, *reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// compression
+//
+// A CTA takes T (1, 2 or 4) 128-row tiles of one matrix over a range of columns, a step of 128 bytes of every row (32 fp32 or
+// 64 bf16 values) at a time.  Worker warps fetch the rows with plain 16-byte loads, two tiles ahead in registers (rows that start
+// off a 16-byte boundary: two aligned loads per piece, shifted together), cut fp32 values into parts and write operand
+// tiles; the same warps generate the step's tile of A while the loads are under way.  One thread issues the MMAs.
+// Where a matrix has too few rows to fill the GPU, `split` CTAs of a cluster share its columns and add their partial sums
+// through distributed shared memory: one launch, one writer per element, and the sums do not depend on arrival order.
+// ------------------------------------------------------------------------------------------------
+template <bool F32>
+struct GenK1 {
+    static constexpr int K = F32 ? 32 : 64;                 // columns per step
+    static constexpr int PARTS = F32 ? 3 : 1;
+    static constexpr int ROWB = 2 * K;                      // bytes per operand row
+    static constexpr int TILE = 128 * ROWB;                 // one part of a 128-row tile
+};
+struct GenSmem {
+    uint64_t full[GEN_STAGES_MAX], empty[GEN_STAGES_MAX], acc_full;
+    uint32_t tmem_base;
+    int abort;
+};
+// The three parts of A side by side as one N operand (three MMAs per tile and K slice instead of six) while they fit.
+__host__ __device__ inline bool gen_side_by_side(bool f32, int r_pad) { return f32 && 3 * r_pad <= 256; }
+__host__ __device__ inline int gen_acc_cols(bool f32, int r_pad) { return gen_side_by_side(f32, r_pad) ? 3 * r_pad : r_pad; }
+inline size_t gen_k1_stage_bytes(bool f32, int r_pad, int T)
+{
+    return f32 ? (size_t)3 * 64 * (128 * T + r_pad) : (size_t)128 * (128 * T + r_pad);
+}
+// Row stride (in floats) of the staged accumulators: an odd multiple of 16 bytes, so that threads that own neighbouring
+// rows write to different banks.
+__host__ __device__ inline int gen_stage_stride(int r_pad) { return r_pad + 4; }
+
+// SINGLE: one matrix, passed by value; every cluster takes the next row groups of it.  (A template and not a test of `items`: the
+// choice between a table entry and a by-value parameter at run time was compiled into reads of the wrong one.)
+template <bool SINGLE, bool F32, bool ALIGNED>
+__global__ void __launch_bounds__(GEN_THREADS, 2)
+gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
+                    const __grid_constant__ GenMat single, int single_split, int seed_base, int r, float scale, float a, float b, int T, int stages,
+                    int cluster)
+{
+    using C = GenK1<F32>;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
+    uint8_t* const ring = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
+    __shared__ GenSmem ctl;
+    const int r_pad = (r + 15) & ~15;
+    const bool sbs = gen_side_by_side(F32, r_pad);
+    const int acc_cols = gen_acc_cols(F32, r_pad);
+    const uint32_t a_part = (uint32_t)r_pad * C::ROWB;
+    const uint32_t g_bytes = (uint32_t)(T * C::PARTS) * C::TILE, stage_bytes = g_bytes + C::PARTS * a_part;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int rank = cluster > 1 ? (int)ptx::cluster_ctarank() : 0;
+    const int cl = (int)blockIdx.x / cluster;
+    ptx::grid_launch_dependents();
+    GenItem item;
+    if (!SINGLE) {
+        item = items[cl];
+    } else {
+        item.mat = 0;
+        item.split = single_split;
+        item.tile0 = cl * (cluster / single_split) * T;
+    }
+    const GenMat mat = SINGLE ? single : mats[item.mat];
+    const int group = rank / item.split, part = rank % item.split;
+    const int tile0 = item.tile0 + group * T;
+    const int tiles = max(0, min(T, ((mat.n + 127) >> 7) - tile0));
+    const int all_steps = (mat.m + C::K - 1) / C::K;
+    const int ks0 = (int)((int64_t)part * all_steps / item.split), ks1 = (int)((int64_t)(part + 1) * all_steps / item.split);
+    const int steps = tiles > 0 ? ks1 - ks0 : 0;
+    uint32_t tmem_cols = 32;
+    while ((int)tmem_cols < T * acc_cols) tmem_cols <<= 1;
+
+    if (tid == 0) {
+        for (int s = 0; s < stages; ++s) {
+            ptx::mbar_init(ptx::smem_addr(&ctl.full[s]), GEN_WORKERS);
+            ptx::mbar_init(ptx::smem_addr(&ctl.empty[s]), 1);
+        }
+        ptx::mbar_init(ptx::smem_addr(&ctl.acc_full), 1);
+        ctl.abort = 0;
+        ptx::fence_barrier_init();
+        ptx::fence_proxy_async_smem();
+    }
+    if (warp == GEN_WORKERS) {
+        ptx::tmem_alloc(ptx::smem_addr(&ctl.tmem_base), tmem_cols);
+        ptx::tmem_relinquish();
+    }
+    // rows r .. r_pad of every part of every A tile stay zero for the whole kernel
+    if (r_pad > r)
+        for (int s = 0; s < stages; ++s)
+            for (int p = 0; p < C::PARTS; ++p)
+                for (int t = tid; t < (r_pad - r) * (C::ROWB / 16); t += GEN_THREADS)
+                    ptx::st_shared_v4(smem_base + s * stage_bytes + g_bytes + p * a_part + (uint32_t)r * C::ROWB + t * 16u, 0, 0, 0, 0);
+    ptx::fence_proxy_async_smem();
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    const uint32_t tmem = ctl.tmem_base;
+    volatile int* abort = &ctl.abort;
+
+    if (warp == GEN_WORKERS) {
+        // ------------------------------------------------------------------ MMA issuer
+        if (lane == 0 && steps > 0) {
+            RingPos p;
+            bool ok = true;
+            for (int ks = 0; ks < steps; ++ks, p.advance(stages)) {
+                ok = ptx::mbar_wait(ptx::smem_addr(&ctl.full[p.s]), p.wraps & 1u, abort);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                const uint32_t st = smem_base + p.s * stage_bytes;
+                const uint64_t da = operand_desc<C::ROWB>(st + g_bytes);
+                for (int t = 0; t < tiles; ++t) {
+                    const uint64_t dg = operand_desc<C::ROWB>(st + (uint32_t)(t * C::PARTS) * C::TILE);
+                    const uint32_t acc = tmem + (uint32_t)(t * acc_cols);
+#pragma unroll
+                    for (int kk = 0; kk < C::K / 16; ++kk) {
+                        const uint32_t on = (ks | kk) != 0;
+                        if (!F32) {
+                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, ptx::umma_idesc_bf16((uint32_t)r_pad), on);
+                        } else if (sbs) {
+                            // the blocks of the accumulator (one per part of A) are added up when they are read back
+                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(3u * r_pad), on);
+                            ptx::umma_bf16(acc, dg + (C::TILE >> 4) + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(2u * r_pad), 1u);
+                            ptx::umma_bf16(acc, dg + (2 * C::TILE >> 4) + kk * 2, da + kk * 2, ptx::umma_idesc_bf16((uint32_t)r_pad), 1u);
+                        } else {
+                            const uint32_t id = ptx::umma_idesc_bf16((uint32_t)r_pad);
+                            const uint64_t ap = (uint64_t)(a_part >> 4), gp = (uint64_t)(C::TILE >> 4);
+                            ptx::umma_bf16(acc, dg + 2 * gp + kk * 2, da + kk * 2, id, on);                // l h
+                            ptx::umma_bf16(acc, dg + kk * 2, da + 2 * ap + kk * 2, id, 1u);                // h l
+                            ptx::umma_bf16(acc, dg + gp + kk * 2, da + ap + kk * 2, id, 1u);               // m m
+                            ptx::umma_bf16(acc, dg + gp + kk * 2, da + kk * 2, id, 1u);                    // m h
+                            ptx::umma_bf16(acc, dg + kk * 2, da + ap + kk * 2, id, 1u);                    // h m
+                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, id, 1u);                         // h h
+                        }
+                    }
+                }
+                ptx::umma_commit(ptx::smem_addr(&ctl.empty[p.s]));
+            }
+            if (ok) ptx::umma_commit(ptx::smem_addr(&ctl.acc_full));
+        }
+    } else {
+        // ------------------------------------------------------------------ workers
+        // A step of a tile is 128 rows of eight 16-byte pieces; thread tid takes piece tid % 8 of the rows tid / 8 + 32 i.
+        const int piece = tid & 7, row_in = tid >> 3;
+        constexpr int ES = F32 ? 4 : 2, E = 16 / ES;                // element size, elements per piece
+        constexpr int BLK = ALIGNED ? 1 : 2;                        // 16-byte loads per piece
+        const uintptr_t g0 = reinterpret_cast<uintptr_t>(mat.big);
+        const uintptr_t g_end = g0 + ((int64_t)(mat.n - 1) * mat.ld + mat.m) * ES;
+        const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
+        bool ok = true;
+        auto piece_addr = [&](int row, int ks) { return g0 + ((int64_t)row * mat.ld + (int64_t)(ks0 + ks) * C::K + piece * E) * ES; };
+        auto fetch = [&](int u, uint4 (&x)[4][BLK]) {               // the four pieces of this thread of tile-step u = ks * tiles + t
+            const int ks = u / tiles, t = u - ks * tiles;
+            const int col = (ks0 + ks) * C::K + piece * E;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int row = (tile0 + t) * 128 + row_in + 32 * i;
+                const uintptr_t p = piece_addr(row, ks), p16 = p & ~(uintptr_t)15;
+#pragma unroll
+                for (int k = 0; k < BLK; ++k) x[i][k] = make_uint4(0, 0, 0, 0);
+                if (row >= mat.n || col >= mat.m) continue;
+                const bool two = !ALIGNED && p != p16;
+                if (p16 >= g0 && p16 + (two ? 32 : 16) <= g_end) {
+                    x[i][0] = *reinterpret_cast<const uint4*>(p16);
+                    if (two) x[i][BLK - 1] = *reinterpret_cast<const uint4*>(p16 + 16);
+                } else {
+                    // the ends of the buffer: element by element, as bytes of the same two blocks
+                    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const uintptr_t q = p + e * ES;
+                        if (col + e < mat.m) {
+                            const uint32_t v = F32 ? *reinterpret_cast<const uint32_t*>(q) : (uint32_t)*reinterpret_cast<const uint16_t*>(q);
+                            const int off = (int)(q - p16);
+#pragma unroll
+                            for (int k = 0; k < 4 * BLK; ++k)
+                                if (k == (off >> 2)) w[k] |= F32 ? v : v << ((off & 2) * 8);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < BLK; ++k) x[i][k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+                }
+            }
+        };
+        auto place = [&](int u, const uint4 (&x)[4][BLK], uint32_t st) {
+            const int ks = u / tiles, t = u - ks * tiles;
+            const int left = mat.m - ((ks0 + ks) * C::K + piece * E);            // valid elements from this piece on
+            const uint32_t tile = st + (uint32_t)(t * C::PARTS) * C::TILE;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int lr = row_in + 32 * i;
+                uint32_t w[4] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w};
+                if (!ALIGNED) {
+                    const uint4 y = x[i][BLK - 1];
+                    const uint32_t v[8] = {w[0], w[1], w[2], w[3], y.x, y.y, y.z, y.w};
+                    const int off = (int)(piece_addr((tile0 + t) * 128 + lr, ks) & 15);
+                    uint32_t s1[7], s2[5];
+#pragma unroll
+                    for (int k = 0; k < 7; ++k) s1[k] = (off & 4) ? v[k + 1] : v[k];
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) s2[k] = (off & 8) ? s1[k + 2] : s1[k];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) w[k] = (!F32 && (off & 2)) ? __byte_perm(s2[k], s2[k + 1], 0x5432) : s2[k];
+                }
+                if (left < E) {                                                  // columns at and beyond m contribute nothing
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (e >= left) w[e * ES / 4] &= F32 ? 0u : ((e & 1) ? 0x0000FFFFu : 0u);
+                }
+                if (F32) {
+                    store_quad<3>(tile + operand_offset<C::ROWB>(lr, piece >> 1) + (piece & 1) * 8, C::TILE, __uint_as_float(w[0]), __uint_as_float(w[1]),
+                                  __uint_as_float(w[2]), __uint_as_float(w[3]));
+                } else {
+                    ptx::st_shared_v4(tile + operand_offset<C::ROWB>(lr, piece), w[0], w[1], w[2], w[3]);
+                }
+            }
+        };
+        // the step's tile of A: one task is four columns of one row; which thread starts moves on from step to step, so that
+        // tiles with fewer tasks than threads keep all warps busy in turn
+        constexpr int QPR = C::K / 4;
+        const int tasks = r * QPR;
+        int first = tid;
+        auto generate = [&](int ks, uint32_t st) {
+            const uint32_t q0 = (uint32_t)(ks0 + ks) * QPR;
+            int t = first;
+            for (; t < tasks; t += 32 * GEN_WORKERS) {
+                const int j = t / QPR, q = t % QPR;
+                float v[4];
+                projection_quad(q0 + q, (uint32_t)j, key, scale, v);
+                store_quad<C::PARTS>(st + g_bytes + operand_offset<C::ROWB>(j, q >> 1) + (q & 1) * 8, a_part, v[0], v[1], v[2], v[3]);
+            }
+            first = t - tasks;
+        };
+        const int total = steps * tiles;
+        uint4 x0[4][BLK], x1[4][BLK];
+        // the first tile of A touches nothing that another kernel writes
+        if (steps > 0) generate(0, smem_base);
+        ptx::grid_dependency_wait();
+        if (total > 0) fetch(0, x0);
+        if (total > 1) fetch(1, x1);
+        RingPos p;
+        auto turn = [&](int u, uint4 (&x)[4][BLK]) {
+            const int ks = u / tiles, t = u - ks * tiles;
+            const uint32_t st = smem_base + p.s * stage_bytes;
+            if (t == 0 && ks > 0) {
+                ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl.empty[p.s]), (p.wraps & 1u) ^ 1u, abort);
+                if (ok) generate(ks, st);
+            }
+            if (!ok) return;
+            place(u, x, st);
+            if (u + 2 < total) fetch(u + 2, x);
+            if (t == tiles - 1) {
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl.full[p.s]));
+                p.advance(stages);
+            }
+        };
+        for (int u = 0; u < total && ok; u += 2) {
+            turn(u, x0);
+            if (u + 1 < total) turn(u + 1, x1);
+        }
+        if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
+        ptx::tc_fence_after_sync();
+        // ------------------------------------------------------------------ write-out
+        // Accumulators -> shared memory (the operand ring, free by now), one row of a tile per thread.  The other CTAs of a
+        // split add their sums before anything is written to the sketch, whose rows are then written by whole warps.
+        float* const stage = reinterpret_cast<float*>(ring);
+        const int stride = gen_stage_stride(r_pad);
+        auto stage_tile = [&](int t, float* to) {
+            const int row = (warp & 3) * 32 + lane;
+            __syncwarp();
+            for (int c = (warp >> 2) * 16; c < r_pad; c += 32) {
+                uint32_t v[16];
+                if (steps > 0) {
+                    const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(t * acc_cols + c);
+                    ptx::tmem_ld_16(at, v);
+                    if (sbs) {
+                        uint32_t v1[16], v2[16];
+                        ptx::tmem_ld_16(at + r_pad, v1);
+                        ptx::tmem_ld_16(at + 2 * r_pad, v2);
+                        ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            v[k] = __float_as_uint(__uint_as_float(v[k]) + (__uint_as_float(v1[k]) + __uint_as_float(v2[k])));
+                    } else {
+                        ptx::tmem_ld_wait();
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) v[k] = 0u;
+                }
+#pragma unroll
+                for (int k = 0; k < 16; k += 4)
+                    *reinterpret_cast<float4*>(to + row * stride + c + k) =
+                        make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]), __uint_as_float(v[k + 3]));
+            }
+        };
+        // rows [lr0, lr1) of the staged tiles (tile `t_first` on) -> sketch; `value(i, j)`: the finished sum
+        const bool vec = (r & 3) == 0 && (mat.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(mat.S) & 15) == 0;
+        auto write_rows = [&](int lr0, int lr1, int grow0, auto value4, auto value1) {
+            if (vec) {
+                const int per = r >> 2;                                      // pieces per row
+                const int total4 = (lr1 - lr0) * per;
+#pragma unroll 4
+                for (int e = tid; e < total4; e += 32 * GEN_WORKERS) {
+                    const int i = e / per, j = (e - i * per) * 4, lr = lr0 + i;
+                    if (grow0 + lr >= mat.n) break;
+                    float4 v = value4(lr, j);
+                    float4* dst = reinterpret_cast<float4*>(mat.S + (int64_t)(grow0 + lr) * mat.lds + j);
+                    v = make_float4(a * v.x, a * v.y, a * v.z, a * v.w);
+                    if (b != 0.0f) {                                         // b == 0 must not propagate whatever the state held before
+                        const float4 o = *dst;
+                        v = make_float4(fmaf(b, o.x, v.x), fmaf(b, o.y, v.y), fmaf(b, o.z, v.z), fmaf(b, o.w, v.w));
+                    }
+                    *dst = v;
+                }
+            } else {
+                const int total1 = (lr1 - lr0) * r;
+#pragma unroll 4
+                for (int e = tid; e < total1; e += 32 * GEN_WORKERS) {
+                    const int i = e / r, j = e - i * r, lr = lr0 + i;
+                    if (grow0 + lr >= mat.n) break;
+                    float* dst = mat.S + (int64_t)(grow0 + lr) * mat.lds + j;
+                    const float v = a * value1(lr, j);
+                    *dst = b != 0.0f ? fmaf(b, *dst, v) : v;
+                }
+            }
+        };
+        if (item.split == 1) {
+            for (int t = 0; t < tiles; ++t) {
+                if (t > 0) ptx::named_barrier_sync(1, 32 * GEN_WORKERS);
+                stage_tile(t, stage);
+                ptx::named_barrier_sync(1, 32 * GEN_WORKERS);
+                if (!*abort)
+                    write_rows(0, 128, (tile0 + t) * 128, [&](int i, int j) { return *reinterpret_cast<const float4*>(stage + i * stride + j); },
+                               [&](int i, int j) { return stage[i * stride + j]; });
+            }
+            if (cluster > 1) {
+                ptx::cluster_sync_some();
+                ptx::cluster_sync_some();
+            }
+        } else {
+            for (int t = 0; t < tiles; ++t) stage_tile(t, stage + t * 128 * stride);
+            ptx::cluster_sync_some();                                        // every partial sum of the cluster is staged
+            const int rows = tiles * 128, lr0 = part * rows / item.split, lr1 = (part + 1) * rows / item.split;
+            const uint32_t sbase = ptx::smem_addr(stage);
+            const int split = item.split, first_rank = group * split;
+            if (!*abort)
+                write_rows(lr0, lr1, tile0 * 128,
+                           [&](int i, int j) {
+                               float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                               for (int q = 0; q < split; ++q) {
+                                   const float4 w = ptx::ld_cluster_v4(ptx::map_to_cta(sbase + (uint32_t)(i * stride + j) * 4u, (uint32_t)(first_rank + q)));
+                                   v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+                               }
+                               return v;
+                           },
+                           [&](int i, int j) {
+                               float v = 0.f;
+                               for (int q = 0; q < split; ++q)
+                                   v += ptx::ld_cluster_f32(ptx::map_to_cta(sbase + (uint32_t)(i * stride + j) * 4u, (uint32_t)(first_rank + q)));
+                               return v;
+                           });
+            ptx::cluster_sync_some();                                        // nobody leaves while a peer may still read its sums
+        }
+    }
+    if (warp == GEN_WORKERS && cluster > 1) {
+        __syncwarp();
+        ptx::cluster_sync_some();
+        ptx::cluster_sync_some();
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (warp == GEN_WORKERS) {
+        ptx::tc_fence_after_sync();
+        ptx::tmem_dealloc(tmem, tmem_cols);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// decompression fused with the update
+//
+// A CTA takes a slab of GEN_BN columns of one matrix and a run of 128-row tiles.  The slab of A is generated once into
+// shared memory (parts of fp32 values, or bf16 values); per tile the rows of the sketch are cut into their three parts, the
+// MMAs run, and the accumulator goes through shared memory so that W is read and written along its rows whatever
+// their alignment.  Nothing is pipelined inside a CTA: two to four of them share an SM and fill each other's waits.
+// ------------------------------------------------------------------------------------------------
+constexpr int GEN_BN = 64;
+constexpr int GEN_K2_THREADS = 256;
+struct GenK2Item {
+    int32_t mat, col0, tile0, tiles;
+};
+struct GenK2Smem {
+    uint64_t done;
+    uint32_t tmem_base;
+    int abort;
+};
+template <int KB>
+__host__ __device__ inline size_t gen_k2_smem(bool f32, int r)
+{
+    const size_t chunks = (size_t)(r + KB - 1) / KB, slab = chunks * (f32 ? 3 : 1) * GEN_BN * (2 * KB);
+    const size_t sop = (size_t)3 * 128 * (2 * KB), staging = (size_t)128 * (GEN_BN + 4) * 4;
+    return slab + (sop > staging ? sop : staging) + 1024;
+}
+
+template <bool SINGLE, bool F32, int KB>
+__global__ void __launch_bounds__(GEN_K2_THREADS, 3)
+gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
+                      const __grid_constant__ GenMat single, int single_run, int seed_base, int r, float scale, float step)
+{
+    constexpr int PARTS = F32 ? 3 : 1, ROWB = 2 * KB, BN = GEN_BN;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
+    __shared__ GenK2Smem ctl;
+    const int chunks = (r + KB - 1) / KB;
+    constexpr uint32_t SLAB_PART = BN * ROWB, SOP_PART = 128 * ROWB;
+    const uint32_t slab = smem_base, sop = slab + (uint32_t)chunks * PARTS * SLAB_PART;
+    float* const staging = reinterpret_cast<float*>(smem_raw + (sop - ptx::smem_addr(smem_raw)));
+    constexpr int STRIDE = BN + 4;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    ptx::grid_launch_dependents();
+    GenK2Item item;
+    if (!SINGLE) {
+        item = items[blockIdx.x];
+    } else {
+        const int slabs = (single.m + BN - 1) / BN, rt = (single.n + 127) >> 7;
+        item.mat = 0;
+        item.col0 = ((int)blockIdx.x % slabs) * BN;
+        item.tile0 = ((int)blockIdx.x / slabs) * single_run;
+        item.tiles = min(single_run, rt - item.tile0);
+    }
+    const GenMat mat = SINGLE ? single : mats[item.mat];
+
+    if (tid == 0) {
+        ptx::mbar_init(ptx::smem_addr(&ctl.done), 1);
+        ctl.abort = 0;
+        ptx::fence_barrier_init();
+        ptx::fence_proxy_async_smem();
+    }
+    if (warp == 0) {
+        ptx::tmem_alloc(ptx::smem_addr(&ctl.tmem_base), BN);
+        ptx::tmem_relinquish();
+    }
+    {
+        // slab of A as the N x K operand: row = column of W, K = index j of the sketch; one task makes four columns x four j
+        const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
+        const int jq = ((r + 15) & ~15) >> 2;                     // the MMAs read whole 16-value slices
+        for (int t = tid; t < jq * (BN / 4); t += GEN_K2_THREADS) {
+            const int cq = t % (BN / 4), g = t / (BN / 4);
+            float v[4][4];
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                float q[4] = {0.f, 0.f, 0.f, 0.f};
+                if (g * 4 + jj < r) projection_quad((uint32_t)(item.col0 / 4 + cq), (uint32_t)(g * 4 + jj), key, scale, q);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u][jj] = q[u];
+            }
+            const int kc = g * 4 / KB, c16 = (g * 4 % KB) >> 3, half = g & 1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                store_quad<PARTS>(slab + (uint32_t)(kc * PARTS) * SLAB_PART + operand_offset<ROWB>(cq * 4 + u, c16) + half * 8, SLAB_PART, v[u][0], v[u][1],
+                                  v[u][2], v[u][3]);
+        }
+    }
+    ptx::fence_proxy_async_smem();
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    const uint32_t tmem = ctl.tmem_base;
+    volatile int* abort = &ctl.abort;
+    ptx::grid_dependency_wait();                                  // nothing above touches what another kernel writes
+
+    constexpr int ES = F32 ? 4 : 2, E = 16 / ES;                  // element size, elements per 16-byte piece
+    // W moves in 16-byte pieces where its rows and the slab allow it, element by element otherwise
+    const bool vec = item.col0 + BN <= mat.m && ((reinterpret_cast<uintptr_t>(mat.big) | (uintptr_t)(mat.ld * ES)) & 15) == 0;
+    const bool svec = ((reinterpret_cast<uintptr_t>(mat.S) | (uintptr_t)(mat.lds * 4)) & 15) == 0;
+    constexpr int PPR = BN / E;                                   // pieces per row of the tile
+    constexpr int NP = 128 * PPR / GEN_K2_THREADS;                // pieces per thread: 8 (fp32) or 4 (bf16)
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = 0; t < item.tiles && ok; ++t) {
+        const int row0 = (item.tile0 + t) * 128;
+        // old values of W, fetched before the MMAs
+        uint32_t w[32];
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                const int p = tid + GEN_K2_THREADS * i, row = row0 + p / PPR;
+                uint4 v = make_uint4(0, 0, 0, 0);
+                if (row < mat.n) v = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(mat.big) + ((int64_t)row * mat.ld + item.col0 + (p % PPR) * E) * ES);
+                w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const int row = row0 + warp * 16 + (i >> 1), col = item.col0 + lane + 32 * (i & 1);
+                w[i] = 0u;
+                if (row < mat.n && col < mat.m) {
+                    const int64_t at = (int64_t)row * mat.ld + col;
+                    w[i] = F32 ? reinterpret_cast<const uint32_t*>(mat.big)[at] : (uint32_t)reinterpret_cast<const uint16_t*>(mat.big)[at];
+                }
+            }
+        }
+        for (int kc = 0; kc < chunks && ok; ++kc) {
+            if (kc > 0) {                                         // the previous chunk of the sketch has been consumed
+                ok = __syncthreads_and(ptx::mbar_wait(ptx::smem_addr(&ctl.done), phase, abort)) != 0;      // uniform: nobody is left at a barrier
+                phase ^= 1u;
+                if (!ok) break;
+            }
+            constexpr int QPR = KB / 4;
+            const int live = min(KB, ((r - kc * KB) + 15) & ~15);  // columns of this chunk that the MMAs read
+#pragma unroll
+            for (int i = 0; i < 128 * QPR / GEN_K2_THREADS; ++i) {
+                const int p = tid + GEN_K2_THREADS * i, lr = p / QPR, q = p % QPR, row = row0 + lr, j = kc * KB + q * 4;
+                if (q * 4 >= live) continue;
+                float x[4] = {0.f, 0.f, 0.f, 0.f};
+                if (row < mat.n) {
+                    const float* src = mat.S + (int64_t)row * mat.lds + j;
+                    if (svec && j + 3 < r) {
+                        const float4 v = *reinterpret_cast<const float4*>(src);
+                        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (j + e < r) x[e] = src[e];
+                    }
+                }
+                store_quad<3>(sop + operand_offset<ROWB>(lr, q >> 1) + (q & 1) * 8, SOP_PART, x[0], x[1], x[2], x[3]);
+            }
+            ptx::fence_proxy_async_smem();
+            ptx::tc_fence_before_sync();
+            __syncthreads();
+            if (tid == 0) {
+                ptx::tc_fence_after_sync();
+                const uint32_t id = ptx::umma_idesc_bf16((uint32_t)BN);
+                const uint64_t ds = operand_desc<ROWB>(sop), da = operand_desc<ROWB>(slab + (uint32_t)(kc * PARTS) * SLAB_PART);
+                constexpr uint64_t sp = SOP_PART >> 4, ap = SLAB_PART >> 4;
+                for (int kk = 0; kk < live >> 4; ++kk) {
+                    const uint32_t on = (kc | kk) != 0;
+                    ptx::umma_bf16(tmem, ds + 2 * sp + kk * 2, da + kk * 2, id, on);                               // l h
+                    if (F32) {
+                        ptx::umma_bf16(tmem, ds + kk * 2, da + 2 * ap + kk * 2, id, 1u);                           // h l
+                        ptx::umma_bf16(tmem, ds + sp + kk * 2, da + ap + kk * 2, id, 1u);                          // m m
+                    }
+                    ptx::umma_bf16(tmem, ds + sp + kk * 2, da + kk * 2, id, 1u);                                   // m h
+                    if (F32) ptx::umma_bf16(tmem, ds + kk * 2, da + ap + kk * 2, id, 1u);                          // h m
+                    ptx::umma_bf16(tmem, ds + kk * 2, da + kk * 2, id, 1u);                                        // h h
+                }
+                ptx::umma_commit(ptx::smem_addr(&ctl.done));
+            }
+            __syncwarp();
+        }
+        if (!ok) break;
+        ok = __syncthreads_and(ptx::mbar_wait(ptx::smem_addr(&ctl.done), phase, abort)) != 0;
+        phase ^= 1u;
+        if (!ok) break;
+        ptx::tc_fence_after_sync();
+        {
+            // accumulator -> shared memory (over the sketch's operand, consumed by now): warp w takes rows 32 (w % 4) .. +31
+            uint32_t v[2][16];
+            const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 32);
+            __syncwarp();
+            ptx::tmem_ld_16(at, v[0]);
+            ptx::tmem_ld_16(at + 16, v[1]);
+            ptx::tmem_ld_wait();
+            float* to = staging + ((warp & 3) * 32 + lane) * STRIDE + (warp >> 2) * 32;
+#pragma unroll
+            for (int k = 0; k < 32; k += 4)
+                *reinterpret_cast<float4*>(to + k) = make_float4(__uint_as_float(v[k >> 4][k & 15]), __uint_as_float(v[k >> 4][(k & 15) + 1]),
+                                                                 __uint_as_float(v[k >> 4][(k & 15) + 2]), __uint_as_float(v[k >> 4][(k & 15) + 3]));
+        }
+        ptx::tc_fence_before_sync();
+        __syncthreads();
+        ptx::tc_fence_after_sync();
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                const int p = tid + GEN_K2_THREADS * i, lr = p / PPR, c = (p % PPR) * E, row = row0 + lr;
+                if (row >= mat.n) continue;
+                const float* acc = staging + lr * STRIDE + c;
+                uint32_t* x = &w[4 * i];
+                const float4 s0 = *reinterpret_cast<const float4*>(acc);
+                if (F32) {
+                    x[0] = __float_as_uint(fmaf(-step, s0.x, __uint_as_float(x[0])));
+                    x[1] = __float_as_uint(fmaf(-step, s0.y, __uint_as_float(x[1])));
+                    x[2] = __float_as_uint(fmaf(-step, s0.z, __uint_as_float(x[2])));
+                    x[3] = __float_as_uint(fmaf(-step, s0.w, __uint_as_float(x[3])));
+                } else {
+                    const float4 s1 = *reinterpret_cast<const float4*>(acc + 4);
+                    const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const __nv_bfloat162 old = *reinterpret_cast<__nv_bfloat162*>(&x[k]);
+                        __nv_bfloat162 nw = __floats2bfloat162_rn(fmaf(-step, s[2 * k], __low2float(old)), fmaf(-step, s[2 * k + 1], __high2float(old)));
+                        x[k] = *reinterpret_cast<uint32_t*>(&nw);
+                    }
+                }
+                *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(mat.big) + ((int64_t)row * mat.ld + item.col0 + c) * ES) = make_uint4(x[0], x[1], x[2], x[3]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const int lr = warp * 16 + (i >> 1), c = lane + 32 * (i & 1), row = row0 + lr, col = item.col0 + c;
+                if (row < mat.n && col < mat.m) {
+                    const int64_t at = (int64_t)row * mat.ld + col;
+                    const float s = staging[lr * STRIDE + c];
+                    if (F32) reinterpret_cast<float*>(mat.big)[at] = fmaf(-step, s, __uint_as_float(w[i]));
+                    else reinterpret_cast<__nv_bfloat16*>(mat.big)[at] = __float2bfloat16_rn(fmaf(-step, s, __uint_as_float(w[i] << 16)));
+                }
+            }
+        }
+        __syncthreads();                                          // the staged values have been read: the next tile's sketch rows may overwrite them
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) {
+        ptx::tc_fence_after_sync();
+        ptx::tmem_dealloc(tmem, BN);
+    }
+}
+
+}  // namespace flora

@@ -781,6 +781,7 @@ __global__ void __launch_bounds__(256) sketch_to_bf16_kernel(const TcMatrix* __r
     const float* S = mat->S;
     const int64_t lds = mat->lds;
     __nv_bfloat16* Sb = mat->Sb;
+    if (!Sb) return;                                      // a matrix that the decompression kernel does not serve
     for (int row = (int)blockIdx.x * rows_per_block + lr; row < mat->n; row += (int)gridDim.x * rows_per_block) {
         const float* src = S + (int64_t)row * lds + j;
         float v[8];

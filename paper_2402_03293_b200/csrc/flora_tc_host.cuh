@@ -39,6 +39,8 @@ struct TcSet {
     std::vector<K1Item> h_k1;
     std::vector<int> k1_launch_begin;   // item ranges per launch (at most SEEDS_PER_LAUNCH matrices each)
     std::vector<int> split_mats;        // matrices whose sketch is updated by several items
+    std::vector<int> members;           // matrices that compress_* serves; uploaded where that is not every matrix of the set
+    int* d_members = nullptr;
     // ranks above 64: the persistent CTA-pair kernel; a launch's clusters ("slots") each walk their own list of units
     bool k1_pair = false;
     int k1_n = 0;                       // accumulator columns: r rounded up to a multiple of 64
@@ -167,8 +169,9 @@ inline bool raise_smem_limit()
     }
     std::lock_guard<std::mutex> lock(mutex);
     if (done[dev]) return true;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess) {
+    cudaFuncAttributes fa;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || cudaFuncGetAttributes(&fa, Kernel) != cudaSuccess ||
+        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -802,6 +805,7 @@ inline void tc_set_free_stream(TcSet& s, cudaStream_t st)
         if (s.d_k1) cudaFreeAsync(s.d_k1, st);
         if (s.d_k2) cudaFreeAsync(s.d_k2, st);
         if (s.d_split) cudaFreeAsync(s.d_split, st);
+        if (s.d_members) cudaFreeAsync(s.d_members, st);
         if (s.d_slots) cudaFreeAsync(s.d_slots, st);
         if (s.d_sb) cudaFreeAsync(s.d_sb, st);
     } else {
@@ -809,6 +813,7 @@ inline void tc_set_free_stream(TcSet& s, cudaStream_t st)
         if (s.d_k1) cudaFree(s.d_k1);
         if (s.d_k2) cudaFree(s.d_k2);
         if (s.d_split) cudaFree(s.d_split);
+        if (s.d_members) cudaFree(s.d_members);
         if (s.d_slots) cudaFree(s.d_slots);
         if (s.d_sb) cudaFree(s.d_sb);
     }
@@ -816,6 +821,7 @@ inline void tc_set_free_stream(TcSet& s, cudaStream_t st)
     s.d_k1 = nullptr;
     s.d_k2 = nullptr;
     s.d_split = nullptr;
+    s.d_members = nullptr;
     s.d_slots = nullptr;
     s.d_sb = nullptr;
     s.compress_ready = s.decompress_ready = false;
@@ -848,32 +854,52 @@ inline flora_status tc_fill_matrices(TcSet& set, const std::vector<flora_mat>& G
         memset(&tm, 0, sizeof(tm));
         tm.S = (float*)S[i].data;
         tm.lds = S[i].ld;
-        const flora_mat& big = !G.empty() ? G[i] : W[i];
-        tm.n = (int32_t)big.rows;
-        tm.m = (int32_t)big.cols;
+        tm.n = (int32_t)S[i].rows;
+        tm.m = (int32_t)std::max(G.empty() ? (int64_t)0 : G[i].cols, W.empty() ? (int64_t)0 : W[i].cols);
         if (!G.empty() && G[i].rows && G[i].cols && !make_map(&tm.map_g, G[i])) return FLORA_ERR_CUDA;
         if (!W.empty() && W[i].rows && W[i].cols && !make_map(&tm.map_w, W[i])) return FLORA_ERR_CUDA;
-        if (S[i].rows && S[i].cols && !make_map_f32(&tm.map_s, S[i])) return FLORA_ERR_CUDA;
+        if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !make_map_f32(&tm.map_s, S[i])) return FLORA_ERR_CUDA;
     }
     return FLORA_OK;
 }
 
-// Builds the tensor-core side of a set; leaves it "not ready" (SIMT kernels are used) if any matrix is not eligible.
-inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G, const std::vector<flora_mat>& W,
-                                    const std::vector<flora_mat>& S, bool transient, cudaStream_t st)
+// What the TMA kernels can take of a set: the matrix has their type, size and alignment, and its sketch's rows can be addressed.
+inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S)
+{
+    std::vector<uint8_t> ok(big.size(), 0);
+    if (encode_tiled_fn())
+        for (size_t i = 0; i < big.size(); ++i) ok[i] = tc_mat_ok(big[i]) && tc_sketch_ok(S[i]);
+    return ok;
+}
+
+// Builds the tensor-core side of a set for the matrices marked in use_g (compression) and use_w (decompression); the planners
+// see the others as empty.  The descriptors of the sketches are made for every matrix whose sketch TMA can address.
+inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_all, const std::vector<flora_mat>& W_all,
+                                    const std::vector<flora_mat>& S, bool transient, cudaStream_t st, const std::vector<uint8_t>& use_g,
+                                    const std::vector<uint8_t>& use_w)
 {
     set.transient = transient;
     set.count = (int)S.size();
     if (S.empty() || !encode_tiled_fn()) return FLORA_OK;
     set.r = (int)S[0].cols;
-    bool g_ok = !G.empty(), w_ok = !W.empty();
+    std::vector<flora_mat> G = G_all, W = W_all;
+    bool g_ok = false, w_ok = false;
+    set.members.clear();
     for (size_t i = 0; i < S.size(); ++i) {
-        if (!G.empty() && (!tc_mat_ok(G[i]) || !tc_sketch_ok(S[i]))) g_ok = false;       // the epilogue writes S through its tensor map
-        if (!W.empty() && (!tc_mat_ok(W[i]) || !tc_sketch_ok(S[i]))) w_ok = false;
+        if (!G.empty()) {
+            if (use_g[i]) {
+                g_ok = true;
+                set.members.push_back((int)i);
+            } else {
+                G[i].rows = G[i].cols = 0;
+            }
+        }
+        if (!W.empty()) {
+            if (use_w[i]) w_ok = true;
+            else W[i].rows = W[i].cols = 0;
+        }
     }
-    if (!g_ok && !w_ok) return FLORA_OK;
-    std::vector<flora_mat> none;
-    flora_status rc = tc_fill_matrices(set, g_ok ? G : none, w_ok ? W : none, S);
+    flora_status rc = tc_fill_matrices(set, G, W, S);
     if (rc) return rc;
     if (w_ok) {
         plan_decompress(set, W, set.r);
@@ -884,7 +910,7 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G,
             std::vector<size_t> offset(S.size());
             for (size_t i = 0; i < S.size(); ++i) {
                 offset[i] = total;
-                total += (((size_t)S[i].rows * k_pad * 2) + 1023) & ~(size_t)1023;
+                total += (((size_t)W[i].rows * k_pad * 2) + 1023) & ~(size_t)1023;
             }
             if (total) {
                 cudaError_t e = transient ? scratch_alloc((void**)&set.d_sb, total, st) : cudaMalloc((void**)&set.d_sb, total);
@@ -894,7 +920,7 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G,
                 }
             }
             for (size_t i = 0; i < S.size(); ++i) {
-                if (S[i].rows == 0) continue;
+                if (W[i].rows == 0) continue;
                 TcMatrix& tm = set.h_mats[i];
                 tm.Sb = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<uint8_t*>(set.d_sb) + offset[i]);
                 flora_mat sb;
@@ -917,6 +943,8 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G,
         if (rc) return rc;
         rc = upload(&set.d_slots, set.h_slots, transient, st);
         if (rc) return rc;
+        if (set.members.size() < S.size()) rc = upload(&set.d_members, set.members, transient, st);
+        if (rc) return rc;
         set.compress_ready = true;
     }
     if (w_ok) {
@@ -927,18 +955,13 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G,
     return FLORA_OK;
 }
 
-inline flora_status tc_set_build(TcSet& set, const std::vector<flora_mat>& G, const std::vector<flora_mat>& W,
-                                 const std::vector<flora_mat>& S)
-{
-    return tc_set_build_on(set, G, W, S, false, nullptr);
-}
-
 // New gradient pointers, same shapes: only the tensor maps change.
 inline flora_status tc_set_rebind(TcSet& set, const std::vector<flora_mat>& G, cudaStream_t st)
 {
     if (!set.compress_ready) return FLORA_OK;
-    for (size_t i = 0; i < G.size(); ++i) {
+    for (int i : set.members)
         if (!tc_mat_ok(G[i])) return FLORA_ERR_ALIGN;
+    for (int i : set.members) {
         if (G[i].rows && G[i].cols && !make_map(&set.h_mats[i].map_g, G[i])) return FLORA_ERR_CUDA;
     }
     return upload(&set.d_mats, set.h_mats, false, st);
@@ -969,17 +992,18 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
     // L2 between the two (one 4096 x 11008 matrix at r = 256: 45.7 against 49.8 us; on 550 MB of sketches the pass
     // costs what it saves).  Every element still has one writer per launch, so the result does not depend on the schedule.
     int64_t state_bytes = 0;
-    for (const auto& tm : set.h_mats) state_bytes += (int64_t)tm.n * r * 4;
+    for (int i : set.members) state_bytes += (int64_t)set.h_mats[i].n * r * 4;
     const bool scale_all = pair && b != 0.0f && b != 1.0f && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES;
     if (scale_all || (b != 1.0f && !set.split_mats.empty())) {
         late_wait = tune_knob("FLORA_PDL", 1, 0, 1);
         // rows that receive adds (from several CTAs, or from the pair kernel's reducing write-out): scale them by b first
-        const size_t total = scale_all ? (size_t)set.count : set.split_mats.size();
+        const size_t total = scale_all ? set.members.size() : set.split_mats.size();
+        const int* ids = scale_all ? set.d_members : set.d_split;        // (no list: every matrix of the set)
         for (size_t begin = 0; begin < total; begin += 65535) {
             const size_t jobs_here = std::min<size_t>(65535, total - begin);
             // few enough blocks to be resident at once: the compression kernel may only start once all have started
             dim3 grid((unsigned)std::max<size_t>(1, std::min<size_t>(helper_blocks(set), (size_t)sm_count() * 6 / jobs_here)), (unsigned)jobs_here);
-            scale_sketches_kernel<<<grid, 256, 0, st>>>(set.d_mats, scale_all ? nullptr : set.d_split + begin, (int)begin, r, b);
+            scale_sketches_kernel<<<grid, 256, 0, st>>>(set.d_mats, ids ? ids + begin : nullptr, (int)begin, r, b);
             launches.fetch_add(1, std::memory_order_relaxed);
         }
         if (scale_all) b = 1.0f;
@@ -1085,7 +1109,8 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
     }
     plan->key = key;
     std::vector<flora_mat> b(1, big), s(1, sketch), none;
-    *rc = kind == 0 ? tc_set_build_on(plan->set, b, none, s, false, st) : tc_set_build_on(plan->set, none, b, s, false, st);
+    const std::vector<uint8_t> use = tc_eligible(b, s);
+    *rc = kind == 0 ? tc_set_build_on(plan->set, b, none, s, false, st, use, {}) : tc_set_build_on(plan->set, none, b, s, false, st, {}, use);
     if (*rc == FLORA_OK && cudaStreamSynchronize(st) != cudaSuccess) *rc = FLORA_ERR_CUDA;      // the tables are in place for every stream
     if (*rc != FLORA_OK) {
         tc_set_free(plan->set);

@@ -1,0 +1,79 @@
+"""The kernels for fp32, unaligned and small matrices (csrc/flora_gen.cuh) at the edges of their tiles, against the oracle.
+
+Tolerances: those of the other parity tests.  fp32: each product is exact to 2^-23 (three bf16 parts of 8 bits each, the
+products left out are below that) and up to 6 m of them are added in fp32, which for random signs leaves about
+sqrt(6 m) 2^-24 of the largest partial sum: 1e-5 holds with an order of magnitude to spare at the sizes here.  The weights
+carry one spacing of fp32 on top, since both sides store them rounded."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2402_03293_b200 import binding as fb
+from paper_2402_03293_b200 import workloads as wl
+from tests.parity_util import TOL, oracle_compress, oracle_decompress, rel_err, values
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _view(n, m, dtype, seed, offset, gap, std):
+    """An n x m view that starts `offset` elements into its buffer, rows m + gap apart."""
+    data = wl.gaussian_matrix(n, m, std * std, dtype, seed).to(DEV)
+    buf = torch.full((offset + n * (m + gap) + 8,), 3.0, dtype=data.dtype, device=DEV)
+    v = buf[offset:offset + n * (m + gap)].view(n, m + gap)[:, :m]
+    v.copy_(data)
+    return buf, v
+
+
+# rows around one and two tiles; columns around a step (32 fp32, 64 bf16 values) and a slab; ranks around a 16-column slice,
+# around where the three parts of A stop fitting one operand (80 | 96) and the largest; row groups shared by a cluster
+@pytest.mark.parametrize("n,m,r", [(1, 1, 1), (127, 31, 8), (128, 33, 16), (129, 65, 17), (257, 64, 80), (300, 130, 81), (40, 1029, 96), (64, 4100, 33),
+                                   (513, 257, 200), (130, 190, 256)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("offset,gap", [(0, 0), (1, 0), (3, 5)])
+def test_edges(n, m, r, dtype, offset, gap):
+    gbuf, G = _view(n, m, dtype, 5, offset, gap, 0.1)
+    wbuf, W = _view(n, m, dtype, 6, offset, gap, 0.02)
+    _, S = _view(n, r, "f32", 7, offset, gap, 1.0)
+    S0, W0 = S.clone(), W.clone()
+    around = wbuf.clone()
+    fb.flora_compress_accumulate(G, S, 11, r)
+    assert rel_err(S.cpu().numpy(), oracle_compress(G.contiguous(), S0, 11)) <= TOL[dtype]
+    S1 = S.clone()
+    fb.flora_momentum_step(G, S, 0.75, 12)
+    assert rel_err(S.cpu().numpy(), oracle_compress(G.contiguous(), S1, 12, a=0.25, b=0.75)) <= TOL[dtype]
+    fb.flora_decompress_apply(W, S, 13, 0.03, 1.0)
+    ref = oracle_decompress(W0, S.contiguous(), 13, 0.03, 1.0)
+    got, want, w0 = (values(x).astype(np.float64) for x in (wl.as_numpy(W.contiguous()), ref, wl.as_numpy(W0)))
+    spacing = float(np.spacing(np.float32(np.abs(want).max()))) * (1 if dtype == "f32" else 2 ** 16)
+    assert np.abs(got - want).max() <= TOL[dtype] * np.abs(want - w0).max() + spacing
+    W.copy_(W0)                                                       # nothing outside the view was written
+    assert torch.equal(wbuf, around)
+    assert fb.flora_device_status() == 0
+
+
+@pytest.mark.parametrize("r", [8, 33, 128])
+def test_mixed_sets(r):
+    """Both dtypes, odd rows and matrices that TMA serves in one set (enough of the latter that they get their own launch)."""
+    shapes = [(2048, 2304, "bf16"), (130, 515, "bf16"), (96, 200, "f32"), (10, 768, "bf16"), (300, 1000, "f32"), (50, 4099, "bf16")]
+    G = [wl.gaussian_matrix(n, m, 1e-2, d, 20 + i).to(DEV) for i, (n, m, d) in enumerate(shapes)]
+    W = [wl.gaussian_matrix(n, m, 4e-4, d, 40 + i).to(DEV) for i, (n, m, d) in enumerate(shapes)]
+    S = [torch.randn(n, r, device=DEV) for n, _, _ in shapes]
+    S0, W0 = [s.clone() for s in S], [w.clone() for w in W]
+    fset = fb.FloraSet([torch.zeros_like(g) for g in G], W, S)
+    fset.rebind_gradients(G)
+    seeds = [fb.flora_derive_seed(3, i, 0) for i in range(len(shapes))]
+    fset.momentum_step(0.5, seeds)
+    for i, (n, m, d) in enumerate(shapes):
+        assert rel_err(S[i].cpu().numpy(), oracle_compress(G[i], S0[i], seeds[i], a=0.5, b=0.5)) <= TOL[d], i
+    fset.decompress_apply(seeds, 0.03, 1.0)
+    for i, (n, m, d) in enumerate(shapes):
+        ref = oracle_decompress(W0[i], S[i], seeds[i], 0.03, 1.0)
+        assert rel_err(values(wl.as_numpy(W[i])), values(ref)) <= TOL[d], i
+    fset.compress_overwrite(seeds)
+    for i, (n, m, d) in enumerate(shapes):
+        assert rel_err(S[i].cpu().numpy(), oracle_compress(G[i], torch.zeros_like(S0[i]), seeds[i])) <= TOL[d], i
+    fset.zero_state()
+    assert all(bool(torch.all(s == 0)) for s in S)
+    fset.close()
+    assert fb.flora_device_status() == 0
