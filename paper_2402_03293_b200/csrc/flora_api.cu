@@ -178,11 +178,11 @@ flora_status static_scratch_for_current_device(float** out)
 bool use_gen(const flora_mat* big) { return g_force_path.load(std::memory_order_relaxed) != 1 && gen_supported(*big); }
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 {
-    return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch);
+    return g_force_path.load(std::memory_order_relaxed) != 1 && tune_knob("FLORA_GEN", 0, 0, 1) == 0 && tc_compress_supported(big, sketch);
 }
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
 {
-    return g_force_path.load(std::memory_order_relaxed) != 1 && tc_decompress_supported(big, sketch);
+    return g_force_path.load(std::memory_order_relaxed) != 1 && tune_knob("FLORA_GEN", 0, 0, 1) == 0 && tc_decompress_supported(big, sketch);
 }
 
 }  // namespace

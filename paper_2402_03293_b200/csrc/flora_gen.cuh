@@ -229,51 +229,48 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     } else {
         // ------------------------------------------------------------------ workers
         // A step of a tile is 128 rows of eight 16-byte pieces; thread tid takes piece tid % 8 of the rows tid / 8 + 32 i.
+        // What bounds a step is issue slots (16 KB of G take about 700 cycles of an SM's share of HBM), so the loop carries
+        // one pointer and tests one row count.  A piece that starts off a 16-byte boundary comes as the two aligned blocks it
+        // touches; a block is read whole as soon as one byte of it is wanted (it lies in one page with that byte).
         const int piece = tid & 7, row_in = tid >> 3;
         constexpr int ES = F32 ? 4 : 2, E = 16 / ES;                // element size, elements per piece
-        constexpr int BLK = ALIGNED ? 1 : 2;                        // 16-byte loads per piece
-        const uintptr_t g0 = reinterpret_cast<uintptr_t>(mat.big);
-        const uintptr_t g_end = g0 + ((int64_t)(mat.n - 1) * mat.ld + mat.m) * ES;
+        constexpr int BLK = ALIGNED ? 1 : 2;                        // 16-byte blocks per piece
         const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
         bool ok = true;
-        auto piece_addr = [&](int row, int ks) { return g0 + ((int64_t)row * mat.ld + (int64_t)(ks0 + ks) * C::K + piece * E) * ES; };
-        auto fetch = [&](int u, uint4 (&x)[4][BLK]) {               // the four pieces of this thread of tile-step u = ks * tiles + t
-            const int ks = u / tiles, t = u - ks * tiles;
-            const int col = (ks0 + ks) * C::K + piece * E;
+        const int64_t row_step = 32 * mat.ld * ES;                  // bytes between a thread's rows
+        const int rows_left = mat.n - tile0 * 128 - row_in;         // row t * 128 + 32 i of this thread exists if it is below this
+        const uint8_t* fp = reinterpret_cast<const uint8_t*>(mat.big) + ((int64_t)(tile0 * 128 + row_in) * mat.ld + (int64_t)ks0 * C::K + piece * E) * ES;
+        const uint32_t low0 = (uint32_t)reinterpret_cast<uintptr_t>(fp), low_step = (uint32_t)row_step;      // for the pieces' alignment
+        const uint8_t* fstep = fp;                                  // fetch cursor: this thread's piece of row 0 of the tile; of tile 0 of the step
+        int fks = 0, ft = 0, pks = 0, pt = 0;                       // fetch and place cursors: step, tile
+        auto left_at = [&](int ks) { return mat.m - ((ks0 + ks) * C::K + piece * E); };      // elements from this thread's piece on
+        auto fetch = [&](uint4 (&x)[4][BLK]) {                      // the four pieces of this thread of the tile at the fetch cursor
+            const int bytes = min(16, left_at(fks) * ES);
+            const uint8_t* p = fp;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int row = (tile0 + t) * 128 + row_in + 32 * i;
-                const uintptr_t p = piece_addr(row, ks), p16 = p & ~(uintptr_t)15;
-#pragma unroll
-                for (int k = 0; k < BLK; ++k) x[i][k] = make_uint4(0, 0, 0, 0);
-                if (row >= mat.n || col >= mat.m) continue;
-                const bool two = !ALIGNED && p != p16;
-                if (p16 >= g0 && p16 + (two ? 32 : 16) <= g_end) {
-                    x[i][0] = *reinterpret_cast<const uint4*>(p16);
-                    if (two) x[i][BLK - 1] = *reinterpret_cast<const uint4*>(p16 + 16);
-                } else {
-                    // the ends of the buffer: element by element, as bytes of the same two blocks
-                    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-                    for (int e = 0; e < E; ++e) {
-                        const uintptr_t q = p + e * ES;
-                        if (col + e < mat.m) {
-                            const uint32_t v = F32 ? *reinterpret_cast<const uint32_t*>(q) : (uint32_t)*reinterpret_cast<const uint16_t*>(q);
-                            const int off = (int)(q - p16);
-#pragma unroll
-                            for (int k = 0; k < 4 * BLK; ++k)
-                                if (k == (off >> 2)) w[k] |= F32 ? v : v << ((off & 2) * 8);
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < BLK; ++k) x[i][k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+            for (int i = 0; i < 4; ++i, p += row_step) {
+                const bool in = ft * 128 + 32 * i < rows_left && bytes > 0;
+                const uint8_t* const p16 = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)15);
+                x[i][0] = make_uint4(0, 0, 0, 0);
+                if (in) x[i][0] = *reinterpret_cast<const uint4*>(p16);
+                if (!ALIGNED) {
+                    x[i][BLK - 1] = make_uint4(0, 0, 0, 0);
+                    if (in && (int)(p - p16) + bytes > 16) x[i][BLK - 1] = *reinterpret_cast<const uint4*>(p16 + 16);
                 }
             }
+            if (++ft == tiles) {
+                ft = 0;
+                ++fks;
+                fstep += 128;
+                fp = fstep;
+            } else {
+                fp += 4 * row_step;
+            }
         };
-        auto place = [&](int u, const uint4 (&x)[4][BLK], uint32_t st) {
-            const int ks = u / tiles, t = u - ks * tiles;
-            const int left = mat.m - ((ks0 + ks) * C::K + piece * E);            // valid elements from this piece on
-            const uint32_t tile = st + (uint32_t)(t * C::PARTS) * C::TILE;
+        const uint32_t my_off = F32 ? (uint32_t)((piece & 1) * 8) : 0u;
+        auto place = [&](const uint4 (&x)[4][BLK], uint32_t st) {   // ... of the tile at the place cursor, as operand rows of stage st
+            const uint32_t tile = st + (uint32_t)(pt * C::PARTS) * C::TILE + my_off;
+            const int left = left_at(pks);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int lr = row_in + 32 * i;
@@ -281,14 +278,14 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 if (!ALIGNED) {
                     const uint4 y = x[i][BLK - 1];
                     const uint32_t v[8] = {w[0], w[1], w[2], w[3], y.x, y.y, y.z, y.w};
-                    const int off = (int)(piece_addr((tile0 + t) * 128 + lr, ks) & 15);
+                    const uint32_t off = low0 + (uint32_t)(pt * 4 + i) * low_step;
                     uint32_t s1[7], s2[5];
 #pragma unroll
                     for (int k = 0; k < 7; ++k) s1[k] = (off & 4) ? v[k + 1] : v[k];
 #pragma unroll
                     for (int k = 0; k < 5; ++k) s2[k] = (off & 8) ? s1[k + 2] : s1[k];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) w[k] = (!F32 && (off & 2)) ? __byte_perm(s2[k], s2[k + 1], 0x5432) : s2[k];
+                    for (int k = 0; k < 4; ++k) w[k] = F32 ? s2[k] : __byte_perm(s2[k], s2[k + 1], (off & 2) ? 0x5432 : 0x3210);
                 }
                 if (left < E) {                                                  // columns at and beyond m contribute nothing
 #pragma unroll
@@ -296,8 +293,8 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                         if (e >= left) w[e * ES / 4] &= F32 ? 0u : ((e & 1) ? 0x0000FFFFu : 0u);
                 }
                 if (F32) {
-                    store_quad<3>(tile + operand_offset<C::ROWB>(lr, piece >> 1) + (piece & 1) * 8, C::TILE, __uint_as_float(w[0]), __uint_as_float(w[1]),
-                                  __uint_as_float(w[2]), __uint_as_float(w[3]));
+                    store_quad<3>(tile + operand_offset<C::ROWB>(lr, piece >> 1), C::TILE, __uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]),
+                                  __uint_as_float(w[3]));
                 } else {
                     ptx::st_shared_v4(tile + operand_offset<C::ROWB>(lr, piece), w[0], w[1], w[2], w[3]);
                 }
@@ -324,20 +321,21 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         // the first tile of A touches nothing that another kernel writes
         if (steps > 0) generate(0, smem_base);
         ptx::grid_dependency_wait();
-        if (total > 0) fetch(0, x0);
-        if (total > 1) fetch(1, x1);
+        if (total > 0) fetch(x0);
+        if (total > 1) fetch(x1);
         RingPos p;
-        auto turn = [&](int u, uint4 (&x)[4][BLK]) {
-            const int ks = u / tiles, t = u - ks * tiles;
+        auto turn = [&](bool more, uint4 (&x)[4][BLK]) {
             const uint32_t st = smem_base + p.s * stage_bytes;
-            if (t == 0 && ks > 0) {
+            if (pt == 0 && pks > 0) {
                 ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl.empty[p.s]), (p.wraps & 1u) ^ 1u, abort);
-                if (ok) generate(ks, st);
+                if (ok) generate(pks, st);
             }
             if (!ok) return;
-            place(u, x, st);
-            if (u + 2 < total) fetch(u + 2, x);
-            if (t == tiles - 1) {
+            place(x, st);
+            if (more) fetch(x);
+            if (++pt == tiles) {
+                pt = 0;
+                ++pks;
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl.full[p.s]));
@@ -345,8 +343,8 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
             }
         };
         for (int u = 0; u < total && ok; u += 2) {
-            turn(u, x0);
-            if (u + 1 < total) turn(u + 1, x1);
+            turn(u + 2 < total, x0);
+            if (u + 1 < total) turn(u + 3 < total, x1);
         }
         if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
         ptx::tc_fence_after_sync();
@@ -469,12 +467,12 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
 // ------------------------------------------------------------------------------------------------
 // decompression fused with the update
 //
-// A CTA takes a slab of GEN_BN columns of one matrix and a run of 128-row tiles.  The slab of A is generated once into
-// shared memory (parts of fp32 values, or bf16 values); per tile the rows of the sketch are cut into their three parts, the
-// MMAs run, and the accumulator goes through shared memory so that W is read and written along its rows whatever
-// their alignment.  Nothing is pipelined inside a CTA: two to four of them share an SM and fill each other's waits.
+// The units of work are (slab of BN columns, 128-row tile); a CTA takes an equal, contiguous share of them, slab after slab,
+// and generates a slab of A (parts of fp32 values, or bf16 values) whenever its share enters one.  Per tile the rows of the
+// sketch are cut into their three parts, the MMAs run, and the accumulator goes through shared memory so that W is read and
+// written along its rows whatever their alignment.  The next tile's rows travel in registers meanwhile, and two
+// CTAs share an SM.
 // ------------------------------------------------------------------------------------------------
-constexpr int GEN_BN = 64;
 constexpr int GEN_K2_THREADS = 256;
 struct GenK2Item {
     int32_t mat, col0, tile0, tiles;
@@ -484,20 +482,20 @@ struct GenK2Smem {
     uint32_t tmem_base;
     int abort;
 };
-template <int KB>
+template <int KB, int BN>
 __host__ __device__ inline size_t gen_k2_smem(bool f32, int r)
 {
-    const size_t chunks = (size_t)(r + KB - 1) / KB, slab = chunks * (f32 ? 3 : 1) * GEN_BN * (2 * KB);
-    const size_t sop = (size_t)3 * 128 * (2 * KB), staging = (size_t)128 * (GEN_BN + 4) * 4;
+    const size_t chunks = (size_t)(r + KB - 1) / KB, slab = chunks * (f32 ? 3 : 1) * BN * (2 * KB);
+    const size_t sop = (size_t)3 * 128 * (2 * KB), staging = (size_t)128 * (BN + 4) * 4;
     return slab + (sop > staging ? sop : staging) + 1024;
 }
 
-template <bool SINGLE, bool F32, int KB>
-__global__ void __launch_bounds__(GEN_K2_THREADS, 3)
-gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
-                      const __grid_constant__ GenMat single, int single_run, int seed_base, int r, float scale, float step)
+template <bool SINGLE, bool F32, int KB, int BN>
+__global__ void __launch_bounds__(GEN_K2_THREADS, 2)
+gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restrict__ items, const int* __restrict__ begin,
+                      const __grid_constant__ SeedTable seeds, const __grid_constant__ GenMat single, int seed_base, int r, float scale, float step)
 {
-    constexpr int PARTS = F32 ? 3 : 1, ROWB = 2 * KB, BN = GEN_BN;
+    constexpr int PARTS = F32 ? 3 : 1, ROWB = 2 * KB;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     __shared__ GenK2Smem ctl;
@@ -508,17 +506,17 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
     constexpr int STRIDE = BN + 4;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     ptx::grid_launch_dependents();
-    GenK2Item item;
-    if (!SINGLE) {
-        item = items[blockIdx.x];
+    // this CTA's share: pieces of slabs (one matrix: units u .. u_end of the slab-major order)
+    int it = 0, it_end = 0, u = 0, u_end = 0, rt = 1;
+    if (SINGLE) {
+        rt = (single.n + 127) >> 7;
+        const int64_t total = (int64_t)rt * ((single.m + BN - 1) / BN);
+        u = (int)(blockIdx.x * total / gridDim.x);
+        u_end = (int)((blockIdx.x + 1) * total / gridDim.x);
     } else {
-        const int slabs = (single.m + BN - 1) / BN, rt = (single.n + 127) >> 7;
-        item.mat = 0;
-        item.col0 = ((int)blockIdx.x % slabs) * BN;
-        item.tile0 = ((int)blockIdx.x / slabs) * single_run;
-        item.tiles = min(single_run, rt - item.tile0);
+        it = begin[blockIdx.x];
+        it_end = begin[blockIdx.x + 1];
     }
-    const GenMat mat = SINGLE ? single : mats[item.mat];
 
     if (tid == 0) {
         ptx::mbar_init(ptx::smem_addr(&ctl.done), 1);
@@ -526,183 +524,228 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
     }
-    if (warp == 0) {
+    if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_addr(&ctl.tmem_base), BN);
         ptx::tmem_relinquish();
     }
-    {
-        // slab of A as the N x K operand: row = column of W, K = index j of the sketch; one task makes four columns x four j
-        const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
-        const int jq = ((r + 15) & ~15) >> 2;                     // the MMAs read whole 16-value slices
-        for (int t = tid; t < jq * (BN / 4); t += GEN_K2_THREADS) {
-            const int cq = t % (BN / 4), g = t / (BN / 4);
-            float v[4][4];
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                float q[4] = {0.f, 0.f, 0.f, 0.f};
-                if (g * 4 + jj < r) projection_quad((uint32_t)(item.col0 / 4 + cq), (uint32_t)(g * 4 + jj), key, scale, q);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u][jj] = q[u];
-            }
-            const int kc = g * 4 / KB, c16 = (g * 4 % KB) >> 3, half = g & 1;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                store_quad<PARTS>(slab + (uint32_t)(kc * PARTS) * SLAB_PART + operand_offset<ROWB>(cq * 4 + u, c16) + half * 8, SLAB_PART, v[u][0], v[u][1],
-                                  v[u][2], v[u][3]);
-        }
-    }
-    ptx::fence_proxy_async_smem();
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = ctl.tmem_base;
     volatile int* abort = &ctl.abort;
-    ptx::grid_dependency_wait();                                  // nothing above touches what another kernel writes
-
     constexpr int ES = F32 ? 4 : 2, E = 16 / ES;                  // element size, elements per 16-byte piece
-    // W moves in 16-byte pieces where its rows and the slab allow it, element by element otherwise
-    const bool vec = item.col0 + BN <= mat.m && ((reinterpret_cast<uintptr_t>(mat.big) | (uintptr_t)(mat.ld * ES)) & 15) == 0;
-    const bool svec = ((reinterpret_cast<uintptr_t>(mat.S) | (uintptr_t)(mat.lds * 4)) & 15) == 0;
-    constexpr int PPR = BN / E;                                   // pieces per row of the tile
-    constexpr int NP = 128 * PPR / GEN_K2_THREADS;                // pieces per thread: 8 (fp32) or 4 (bf16)
+    constexpr int PPR = BN / E;                                   // pieces per row of a tile
+    constexpr int NP = 128 * PPR / GEN_K2_THREADS;                // pieces per thread: 8, or 4 (bf16, BN = 64)
+    constexpr int NE = 128 * BN / GEN_K2_THREADS;                 // elements per thread
+    constexpr int QPR = KB / 4, NQ = 128 * QPR / GEN_K2_THREADS;   // four-value pieces of a row of the sketch's chunk; per thread
+    const int sq = tid % QPR, srow = tid / QPR, wp = tid % PPR, wrow = tid / PPR;
+    float x[NQ][4];                                               // the sketch's next chunk, under way
+    uint32_t w[32];                                               // old values of the tile of W, under way
     uint32_t phase = 0;
-    bool ok = true;
-    for (int t = 0; t < item.tiles && ok; ++t) {
-        const int row0 = (item.tile0 + t) * 128;
-        // old values of W, fetched before the MMAs
-        uint32_t w[32];
-        if (vec) {
-#pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                const int p = tid + GEN_K2_THREADS * i, row = row0 + p / PPR;
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (row < mat.n) v = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(mat.big) + ((int64_t)row * mat.ld + item.col0 + (p % PPR) * E) * ES);
-                w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
-            }
+    bool ok = true, waited = false;
+    while (ok && (SINGLE ? u < u_end : it < it_end)) {
+        GenK2Item item;
+        if (SINGLE) {
+            item.mat = 0;
+            item.col0 = u / rt * BN;
+            item.tile0 = u % rt;
+            item.tiles = min(rt - item.tile0, u_end - u);
+            u += item.tiles;
         } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int row = row0 + warp * 16 + (i >> 1), col = item.col0 + lane + 32 * (i & 1);
-                w[i] = 0u;
-                if (row < mat.n && col < mat.m) {
-                    const int64_t at = (int64_t)row * mat.ld + col;
-                    w[i] = F32 ? reinterpret_cast<const uint32_t*>(mat.big)[at] : (uint32_t)reinterpret_cast<const uint16_t*>(mat.big)[at];
-                }
-            }
+            item = items[it++];
         }
-        for (int kc = 0; kc < chunks && ok; ++kc) {
-            if (kc > 0) {                                         // the previous chunk of the sketch has been consumed
-                ok = __syncthreads_and(ptx::mbar_wait(ptx::smem_addr(&ctl.done), phase, abort)) != 0;      // uniform: nobody is left at a barrier
-                phase ^= 1u;
-                if (!ok) break;
-            }
-            constexpr int QPR = KB / 4;
-            const int live = min(KB, ((r - kc * KB) + 15) & ~15);  // columns of this chunk that the MMAs read
+        const GenMat mat = SINGLE ? single : mats[item.mat];
+        // W moves in 16-byte pieces where its rows and the slab allow it, element by element otherwise
+        const bool vec = item.col0 + BN <= mat.m && ((reinterpret_cast<uintptr_t>(mat.big) | (uintptr_t)(mat.ld * ES)) & 15) == 0;
+        const bool svec = ((reinterpret_cast<uintptr_t>(mat.S) | (uintptr_t)(mat.lds * 4)) & 15) == 0;
+        auto load_x = [&](int t, int kc) {
+            const int j = kc * KB + sq * 4, row = (item.tile0 + t) * 128 + srow;
+            const float* src = mat.S + (int64_t)row * mat.lds + j;
 #pragma unroll
-            for (int i = 0; i < 128 * QPR / GEN_K2_THREADS; ++i) {
-                const int p = tid + GEN_K2_THREADS * i, lr = p / QPR, q = p % QPR, row = row0 + lr, j = kc * KB + q * 4;
-                if (q * 4 >= live) continue;
-                float x[4] = {0.f, 0.f, 0.f, 0.f};
-                if (row < mat.n) {
-                    const float* src = mat.S + (int64_t)row * mat.lds + j;
+            for (int i = 0; i < NQ; ++i, src += (GEN_K2_THREADS / QPR) * mat.lds) {
+                x[i][0] = x[i][1] = x[i][2] = x[i][3] = 0.f;
+                if (row + (GEN_K2_THREADS / QPR) * i < mat.n) {
                     if (svec && j + 3 < r) {
                         const float4 v = *reinterpret_cast<const float4*>(src);
-                        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+                        x[i][0] = v.x; x[i][1] = v.y; x[i][2] = v.z; x[i][3] = v.w;
                     } else {
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
-                            if (j + e < r) x[e] = src[e];
+                            if (j + e < r) x[i][e] = src[e];
                     }
                 }
-                store_quad<3>(sop + operand_offset<ROWB>(lr, q >> 1) + (q & 1) * 8, SOP_PART, x[0], x[1], x[2], x[3]);
             }
-            ptx::fence_proxy_async_smem();
+        };
+        auto load_w = [&](int t) {
+            const int row0 = (item.tile0 + t) * 128;
+            if (vec) {
+                const uint8_t* src = reinterpret_cast<const uint8_t*>(mat.big) + ((int64_t)(row0 + wrow) * mat.ld + item.col0) * ES + wp * 16;
+#pragma unroll
+                for (int i = 0; i < NP; ++i, src += (GEN_K2_THREADS / PPR) * mat.ld * ES) {
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (row0 + wrow + (GEN_K2_THREADS / PPR) * i < mat.n) v = *reinterpret_cast<const uint4*>(src);
+                    w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+                }
+            } else if (NE <= 32) {
+                const int row = row0 + warp * 16, col = item.col0 + lane;
+                const uint8_t* src = reinterpret_cast<const uint8_t*>(mat.big) + ((int64_t)row * mat.ld + col) * ES;
+#pragma unroll
+                for (int i = 0; i < NE; ++i) {
+                    w[i & 31] = 0u;
+                    if (row + (i >> 1) < mat.n && col + 32 * (i & 1) < mat.m)
+                        w[i & 31] = F32 ? *reinterpret_cast<const uint32_t*>(src + 128 * (i & 1)) : (uint32_t)*reinterpret_cast<const uint16_t*>(src + 64 * (i & 1));
+                    if (i & 1) src += mat.ld * ES;
+                }
+            }
+        };
+        if (waited) {
+            load_x(0, 0);
+            load_w(0);
+        }
+        {
+            // slab of A as the N x K operand: row = column of W, K = index j of the sketch; one task makes four columns x four j
+            const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
+            const int jq = ((r + 15) & ~15) >> 2;                 // the MMAs read whole 16-value slices
+            for (int t = tid; t < jq * (BN / 4); t += GEN_K2_THREADS) {
+                const int cq = t % (BN / 4), g = t / (BN / 4);
+                float v[4][4];
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    float q[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (g * 4 + jj < r) projection_quad((uint32_t)(item.col0 / 4 + cq), (uint32_t)(g * 4 + jj), key, scale, q);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k][jj] = q[k];
+                }
+                const int kc = g * 4 / KB, c16 = (g * 4 % KB) >> 3, half = g & 1;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    store_quad<PARTS>(slab + (uint32_t)(kc * PARTS) * SLAB_PART + operand_offset<ROWB>(cq * 4 + k, c16) + half * 8, SLAB_PART, v[k][0],
+                                      v[k][1], v[k][2], v[k][3]);
+            }
+        }
+        if (!waited) {                                            // nothing so far touches what another kernel writes
+            ptx::grid_dependency_wait();
+            waited = true;
+            load_x(0, 0);
+            load_w(0);
+        }
+        for (int t = 0; t < item.tiles && ok; ++t) {
+            const int row0 = (item.tile0 + t) * 128;
+            for (int kc = 0; kc < chunks; ++kc) {
+                const int live = min(KB, ((r - kc * KB) + 15) & ~15);   // columns of this chunk that the MMAs read
+                if (kc > 0) {                                     // the previous chunk of the sketch has been consumed
+                    ok = __syncthreads_and(ptx::mbar_wait(ptx::smem_addr(&ctl.done), phase, abort)) != 0;      // uniform: nobody is left at a barrier
+                    phase ^= 1u;
+                    if (!ok) break;
+                }
+                if (sq * 4 < live) {
+#pragma unroll
+                    for (int i = 0; i < NQ; ++i)
+                        store_quad<3>(sop + operand_offset<ROWB>(srow + (GEN_K2_THREADS / QPR) * i, sq >> 1) + (sq & 1) * 8, SOP_PART, x[i][0], x[i][1], x[i][2],
+                                      x[i][3]);
+                }
+                ptx::fence_proxy_async_smem();
+                ptx::tc_fence_before_sync();
+                __syncthreads();
+                if (warp == 0) {
+                    if (lane == 0) {
+                        ptx::tc_fence_after_sync();
+                        const uint32_t id = ptx::umma_idesc_bf16((uint32_t)BN);
+                        const uint64_t ds = operand_desc<ROWB>(sop), da = operand_desc<ROWB>(slab + (uint32_t)(kc * PARTS) * SLAB_PART);
+                        constexpr uint64_t sp = SOP_PART >> 4, ap = SLAB_PART >> 4;
+                        for (int kk = 0; kk < live >> 4; ++kk) {
+                            const uint32_t on = (kc | kk) != 0;
+                            ptx::umma_bf16(tmem, ds + 2 * sp + kk * 2, da + kk * 2, id, on);                       // l h
+                            if (F32) {
+                                ptx::umma_bf16(tmem, ds + kk * 2, da + 2 * ap + kk * 2, id, 1u);                   // h l
+                                ptx::umma_bf16(tmem, ds + sp + kk * 2, da + ap + kk * 2, id, 1u);                  // m m
+                            }
+                            ptx::umma_bf16(tmem, ds + sp + kk * 2, da + kk * 2, id, 1u);                           // m h
+                            if (F32) ptx::umma_bf16(tmem, ds + kk * 2, da + ap + kk * 2, id, 1u);                  // h m
+                            ptx::umma_bf16(tmem, ds + kk * 2, da + kk * 2, id, 1u);                                // h h
+                        }
+                        ptx::umma_commit(ptx::smem_addr(&ctl.done));
+                    }
+                    __syncwarp();
+                }
+                if (kc + 1 < chunks) load_x(t, kc + 1);           // the next rows of the sketch travel while the tensor core works
+                else if (t + 1 < item.tiles) load_x(t + 1, 0);
+            }
+            if (!ok) break;
+            ok = __syncthreads_and(ptx::mbar_wait(ptx::smem_addr(&ctl.done), phase, abort)) != 0;
+            phase ^= 1u;
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            {
+                // accumulator -> shared memory (over the sketch's operand, consumed by now): warp w takes rows 32 (w % 4) .. +31
+                constexpr int NC = BN / 2;                        // columns per warp
+                const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * NC);
+                float* to = staging + ((warp & 3) * 32 + lane) * STRIDE + (warp >> 2) * NC;
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < NC; c += 16) {
+                    uint32_t v[16];
+                    ptx::tmem_ld_16(at + c, v);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int k = 0; k < 16; k += 4)
+                        *reinterpret_cast<float4*>(to + c + k) =
+                            make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]), __uint_as_float(v[k + 3]));
+                }
+            }
             ptx::tc_fence_before_sync();
             __syncthreads();
-            if (tid == 0) {
-                ptx::tc_fence_after_sync();
-                const uint32_t id = ptx::umma_idesc_bf16((uint32_t)BN);
-                const uint64_t ds = operand_desc<ROWB>(sop), da = operand_desc<ROWB>(slab + (uint32_t)(kc * PARTS) * SLAB_PART);
-                constexpr uint64_t sp = SOP_PART >> 4, ap = SLAB_PART >> 4;
-                for (int kk = 0; kk < live >> 4; ++kk) {
-                    const uint32_t on = (kc | kk) != 0;
-                    ptx::umma_bf16(tmem, ds + 2 * sp + kk * 2, da + kk * 2, id, on);                               // l h
+            ptx::tc_fence_after_sync();
+            if (vec) {
+                uint8_t* dst = reinterpret_cast<uint8_t*>(mat.big) + ((int64_t)(row0 + wrow) * mat.ld + item.col0) * ES + wp * 16;
+#pragma unroll
+                for (int i = 0; i < NP; ++i, dst += (GEN_K2_THREADS / PPR) * mat.ld * ES) {
+                    const int lr = wrow + (GEN_K2_THREADS / PPR) * i;
+                    if (row0 + lr >= mat.n) continue;
+                    const float* acc = staging + lr * STRIDE + wp * E;
+                    uint32_t* y = &w[4 * i];
+                    const float4 s0 = *reinterpret_cast<const float4*>(acc);
                     if (F32) {
-                        ptx::umma_bf16(tmem, ds + kk * 2, da + 2 * ap + kk * 2, id, 1u);                           // h l
-                        ptx::umma_bf16(tmem, ds + sp + kk * 2, da + ap + kk * 2, id, 1u);                          // m m
+                        y[0] = __float_as_uint(fmaf(-step, s0.x, __uint_as_float(y[0])));
+                        y[1] = __float_as_uint(fmaf(-step, s0.y, __uint_as_float(y[1])));
+                        y[2] = __float_as_uint(fmaf(-step, s0.z, __uint_as_float(y[2])));
+                        y[3] = __float_as_uint(fmaf(-step, s0.w, __uint_as_float(y[3])));
+                    } else {
+                        const float4 s1 = *reinterpret_cast<const float4*>(acc + 4);
+                        const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const __nv_bfloat162 old = *reinterpret_cast<__nv_bfloat162*>(&y[k]);
+                            __nv_bfloat162 nw = __floats2bfloat162_rn(fmaf(-step, s[2 * k], __low2float(old)), fmaf(-step, s[2 * k + 1], __high2float(old)));
+                            y[k] = *reinterpret_cast<uint32_t*>(&nw);
+                        }
                     }
-                    ptx::umma_bf16(tmem, ds + sp + kk * 2, da + kk * 2, id, 1u);                                   // m h
-                    if (F32) ptx::umma_bf16(tmem, ds + kk * 2, da + ap + kk * 2, id, 1u);                          // h m
-                    ptx::umma_bf16(tmem, ds + kk * 2, da + kk * 2, id, 1u);                                        // h h
+                    *reinterpret_cast<uint4*>(dst) = make_uint4(y[0], y[1], y[2], y[3]);
                 }
-                ptx::umma_commit(ptx::smem_addr(&ctl.done));
-            }
-            __syncwarp();
-        }
-        if (!ok) break;
-        ok = __syncthreads_and(ptx::mbar_wait(ptx::smem_addr(&ctl.done), phase, abort)) != 0;
-        phase ^= 1u;
-        if (!ok) break;
-        ptx::tc_fence_after_sync();
-        {
-            // accumulator -> shared memory (over the sketch's operand, consumed by now): warp w takes rows 32 (w % 4) .. +31
-            uint32_t v[2][16];
-            const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 32);
-            __syncwarp();
-            ptx::tmem_ld_16(at, v[0]);
-            ptx::tmem_ld_16(at + 16, v[1]);
-            ptx::tmem_ld_wait();
-            float* to = staging + ((warp & 3) * 32 + lane) * STRIDE + (warp >> 2) * 32;
-#pragma unroll
-            for (int k = 0; k < 32; k += 4)
-                *reinterpret_cast<float4*>(to + k) = make_float4(__uint_as_float(v[k >> 4][k & 15]), __uint_as_float(v[k >> 4][(k & 15) + 1]),
-                                                                 __uint_as_float(v[k >> 4][(k & 15) + 2]), __uint_as_float(v[k >> 4][(k & 15) + 3]));
-        }
-        ptx::tc_fence_before_sync();
-        __syncthreads();
-        ptx::tc_fence_after_sync();
-        if (vec) {
-#pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                const int p = tid + GEN_K2_THREADS * i, lr = p / PPR, c = (p % PPR) * E, row = row0 + lr;
-                if (row >= mat.n) continue;
-                const float* acc = staging + lr * STRIDE + c;
-                uint32_t* x = &w[4 * i];
-                const float4 s0 = *reinterpret_cast<const float4*>(acc);
-                if (F32) {
-                    x[0] = __float_as_uint(fmaf(-step, s0.x, __uint_as_float(x[0])));
-                    x[1] = __float_as_uint(fmaf(-step, s0.y, __uint_as_float(x[1])));
-                    x[2] = __float_as_uint(fmaf(-step, s0.z, __uint_as_float(x[2])));
-                    x[3] = __float_as_uint(fmaf(-step, s0.w, __uint_as_float(x[3])));
-                } else {
-                    const float4 s1 = *reinterpret_cast<const float4*>(acc + 4);
-                    const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const __nv_bfloat162 old = *reinterpret_cast<__nv_bfloat162*>(&x[k]);
-                        __nv_bfloat162 nw = __floats2bfloat162_rn(fmaf(-step, s[2 * k], __low2float(old)), fmaf(-step, s[2 * k + 1], __high2float(old)));
-                        x[k] = *reinterpret_cast<uint32_t*>(&nw);
+            } else {
+                constexpr int PER = BN / 32;
+                const int row = row0 + warp * 16, col = item.col0 + lane;
+                uint8_t* dst = reinterpret_cast<uint8_t*>(mat.big) + ((int64_t)row * mat.ld + col) * ES;
+#pragma unroll(NE <= 32 ? 32 : 8)
+                for (int i = 0; i < NE; ++i) {
+                    const int c = 32 * (i % PER);
+                    if (row + i / PER < mat.n && col + c < mat.m) {
+                        const float s = staging[(warp * 16 + i / PER) * STRIDE + lane + c];
+                        uint8_t* const q = dst + c * ES;
+                        const uint32_t old = NE <= 32 ? w[i & 31] : (uint32_t)*reinterpret_cast<const uint16_t*>(q);
+                        if (F32) *reinterpret_cast<float*>(q) = fmaf(-step, s, __uint_as_float(old));
+                        else *reinterpret_cast<__nv_bfloat16*>(q) = __float2bfloat16_rn(fmaf(-step, s, __uint_as_float(old << 16)));
                     }
-                }
-                *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(mat.big) + ((int64_t)row * mat.ld + item.col0 + c) * ES) = make_uint4(x[0], x[1], x[2], x[3]);
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int lr = warp * 16 + (i >> 1), c = lane + 32 * (i & 1), row = row0 + lr, col = item.col0 + c;
-                if (row < mat.n && col < mat.m) {
-                    const int64_t at = (int64_t)row * mat.ld + col;
-                    const float s = staging[lr * STRIDE + c];
-                    if (F32) reinterpret_cast<float*>(mat.big)[at] = fmaf(-step, s, __uint_as_float(w[i]));
-                    else reinterpret_cast<__nv_bfloat16*>(mat.big)[at] = __float2bfloat16_rn(fmaf(-step, s, __uint_as_float(w[i] << 16)));
+                    if (i % PER == PER - 1) dst += mat.ld * ES;
                 }
             }
+            if (t + 1 < item.tiles) load_w(t + 1);                // ... and the next tile of W while its product is made
+            __syncthreads();                                      // the staged values have been read: the next tile's sketch rows may overwrite them
         }
-        __syncthreads();                                          // the staged values have been read: the next tile's sketch rows may overwrite them
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == 1) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem, BN);
     }

@@ -11,7 +11,7 @@ namespace flora {
 
 // Launch shape of the compression for a list of matrices.
 struct GenK1Plan {
-    int T = 1, stages = 2, cluster = 1;
+    int T = 1, stages = 2, cluster = 1, per_sm = 1;
     size_t smem = 0;
     bool aligned = true;
 };
@@ -39,6 +39,7 @@ inline void gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split)
     // no more CTAs on an SM than its tensor memory serves: the CTAs of a cluster wait for one another, so none may wait for columns
     const int most = (int)(512 / cols);
     while (most < 8 && (size_t)(most + 1) * (p.smem + 1024) <= 227 * 1024) p.smem += 1024;
+    p.per_sm = two ? 2 : 1;
 }
 inline bool gen_k1_fits(bool f32, int r, int T, bool split)
 {
@@ -54,6 +55,17 @@ inline int gen_k1_tiles(bool f32, int r, int64_t max_tiles)
     int T = 1;
     while (T < 4 && gen > 0.5 * 700 * T && max_tiles >= 2 * T && gen_k1_fits(f32, r, 2 * T, false)) T *= 2;
     return T;
+}
+// Cost model of the compression (cycles of one SM): a step of T tiles takes its share of HBM (16 KB a tile, 700 cycles) or the
+// issue slots of generating and converting it, whichever is longer, and no less than the latency of one step; a CTA costs
+// about two microseconds before its first and after its last step, a little more when it adds up with others.
+inline double gen_k1_cost(bool f32, int r, int T, int per_sm, int64_t ctas, int64_t steps, int split)
+{
+    const double gen = (double)r * (f32 ? 32 : 64) * 54 / 128, issue = gen + (f32 ? 300.0 : 150.0) * T;
+    const double waves = (double)((ctas + (int64_t)per_sm * sm_count() - 1) / ((int64_t)per_sm * sm_count()));
+    const double together = std::min<double>(per_sm, (double)ctas / sm_count());
+    const double step = std::max(1000.0 + 1.5 * gen, std::max(1.0, together) * std::max(700.0 * T, issue));
+    return waves * (4000.0 + (split > 1 ? 1500.0 : 0.0) + (double)steps * step);
 }
 // CTAs that share the columns of one row group, so that `groups` of them fill the GPU; every CTA keeps at least two steps.
 inline int gen_k1_split(int64_t groups, int64_t steps, int64_t want)
@@ -112,15 +124,24 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
     const bool f32 = G.dtype == FLORA_F32;
     const int r = (int)S.cols;
     const int64_t tiles = (G.rows + 127) / 128, steps = (G.cols + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
-    const int64_t want = 2 * sm_count();
-    // few row groups: one tile each and the columns shared by a cluster
-    int T = gen_k1_tiles(f32, r, tiles);
-    while (T > 1 && (tiles + T - 1) / T * gen_k1_split((tiles + T - 1) / T, steps, want) < want / 2) T /= 2;
-    int split = gen_k1_split((tiles + T - 1) / T, steps, want);
-    while (split > 1 && T > 1 && !gen_k1_fits(f32, r, T, true)) T /= 2;
-    const int64_t groups = (tiles + T - 1) / T;
+    // tile shape and split with the shortest schedule: waves of CTAs times the steps of one
     GenK1Plan p;
-    gen_k1_shape(p, f32, r, T, split > 1);
+    int split = 1;
+    double best = 1e300;
+    for (int T = 1; T <= 4; T *= 2)
+        for (int k = 1; k <= 8; k *= 2) {
+            if (T > 1 && tiles < T) continue;
+            if ((k > 1 && steps < k) || !gen_k1_fits(f32, r, T, k > 1)) continue;
+            GenK1Plan cand;
+            gen_k1_shape(cand, f32, r, T, k > 1);
+            const double cost = gen_k1_cost(f32, r, T, cand.per_sm, ((tiles + T - 1) / T) * k, (steps + k - 1) / k, k);
+            if (cost < best * 0.98) {
+                best = cost;
+                p = cand;
+                split = k;
+            }
+        }
+    const int64_t groups = (tiles + p.T - 1) / p.T;
     p.cluster = split;
     p.aligned = gen_aligned(G);
     SeedTable table;
@@ -128,51 +149,72 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
     return gen_compress_launch(f32, p, (int)groups, nullptr, nullptr, table, gen_mat(G, S), split, 0, r, a, b, st, launches);
 }
 
-template <bool SINGLE, bool F32, int KB>
-inline cudaError_t gen_launch_k2(unsigned grid, const GenMat* mats, const GenK2Item* items, const SeedTable& seeds, const GenMat& one, int run,
-                                 int seed_base, int r, float step, cudaStream_t st)
+// Decompression: slabs of 128 columns for bf16 matrices whose rows move in 16-byte pieces, of 64 otherwise (an element-wise
+// thread holds its part of a tile in registers, and fp32 values take twice the room).
+struct GenK2Args {
+    unsigned grid;
+    const GenMat* mats;
+    const GenK2Item* items;
+    const int* begin;
+    const SeedTable* seeds;
+    GenMat one;
+    int seed_base, r;
+    float step;
+    cudaStream_t st;
+};
+inline int gen_k2_bn(bool f32, bool aligned) { return !f32 && aligned ? 128 : 64; }
+// CTAs that an SM holds (shared memory; registers allow two).
+inline int gen_k2_per_sm(bool f32, int r, int bn)
 {
-    if (!raise_smem_limit<gen_decompress_kernel<SINGLE, F32, KB>>()) return cudaErrorInvalidValue;
+    const size_t smem = r <= 32 ? (bn == 64 ? gen_k2_smem<32, 64>(f32, r) : gen_k2_smem<32, 128>(f32, r))
+                                : (bn == 64 ? gen_k2_smem<64, 64>(f32, r) : gen_k2_smem<64, 128>(f32, r));
+    return (int)std::max<size_t>(1, std::min<size_t>(2, 227 * 1024 / (smem + 1040)));
+}
+template <bool SINGLE, bool F32, int KB, int BN>
+inline cudaError_t gen_launch_k2(const GenK2Args& a)
+{
+    if (!raise_smem_limit<gen_decompress_kernel<SINGLE, F32, KB, BN>>()) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(a.grid);
     cfg.blockDim = dim3((unsigned)GEN_K2_THREADS);
-    cfg.dynamicSmemBytes = gen_k2_smem<KB>(F32, r);
-    cfg.stream = st;
+    cfg.dynamicSmemBytes = gen_k2_smem<KB, BN>(F32, a.r);
+    cfg.stream = a.st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gen_decompress_kernel<SINGLE, F32, KB>, mats, items, seeds, one, run, seed_base, r, 1.0f / sqrtf((float)r), step);
+    return cudaLaunchKernelEx(&cfg, gen_decompress_kernel<SINGLE, F32, KB, BN>, a.mats, a.items, a.begin, *a.seeds, a.one, a.seed_base, a.r,
+                              1.0f / sqrtf((float)a.r), a.step);
 }
-inline flora_status gen_decompress_launch(bool f32, unsigned grid, const GenMat* mats, const GenK2Item* items, const SeedTable& seeds, const GenMat& one,
-                                          int run, int seed_base, int r, float step, cudaStream_t st, std::atomic<uint64_t>& launches)
+template <bool SINGLE>
+inline cudaError_t gen_launch_k2_any(bool f32, int bn, const GenK2Args& a)
 {
-    auto go = [&](auto launch) { return launch(grid, mats, items, seeds, one, run, seed_base, r, step, st); };
-    cudaError_t e;
-    if (items) e = f32 ? (r <= 32 ? go(gen_launch_k2<false, true, 32>) : go(gen_launch_k2<false, true, 64>))
-                       : (r <= 32 ? go(gen_launch_k2<false, false, 32>) : go(gen_launch_k2<false, false, 64>));
-    else e = f32 ? (r <= 32 ? go(gen_launch_k2<true, true, 32>) : go(gen_launch_k2<true, true, 64>))
-                 : (r <= 32 ? go(gen_launch_k2<true, false, 32>) : go(gen_launch_k2<true, false, 64>));
+    if (f32) return a.r <= 32 ? gen_launch_k2<SINGLE, true, 32, 64>(a) : gen_launch_k2<SINGLE, true, 64, 64>(a);
+    if (bn == 64) return a.r <= 32 ? gen_launch_k2<SINGLE, false, 32, 64>(a) : gen_launch_k2<SINGLE, false, 64, 64>(a);
+    return a.r <= 32 ? gen_launch_k2<SINGLE, false, 32, 128>(a) : gen_launch_k2<SINGLE, false, 64, 128>(a);
+}
+inline flora_status gen_decompress_launch(bool f32, int bn, const GenK2Args& a, std::atomic<uint64_t>& launches)
+{
+    const cudaError_t e = a.items ? gen_launch_k2_any<false>(f32, bn, a) : gen_launch_k2_any<true>(f32, bn, a);
     launches.fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
-// Row tiles that share a generated slab: as many as still leave `want` CTAs.
-inline int64_t gen_k2_run(int64_t slabs, int64_t row_tiles, int64_t want)
-{
-    const int64_t runs = std::max<int64_t>(1, std::min(row_tiles, (want + slabs - 1) / slabs));
-    return (row_tiles + runs - 1) / runs;
-}
+// CTAs for `units` of (slab, tile): every one of them resident at once; where the generation of a slab outweighs a tile,
+// shares of fewer tiles than a slab has would repeat it, so the shares grow with the rank.
+inline int64_t gen_k2_grid(int64_t units, int64_t slots) { return std::max<int64_t>(1, std::min(units, slots)); }
 inline flora_status gen_decompress_single(const flora_mat& W, const flora_mat& S, uint64_t seed, float step, cudaStream_t st,
                                           std::atomic<uint64_t>& launches)
 {
-    const int64_t slabs = (W.cols + GEN_BN - 1) / GEN_BN, rt = (W.rows + 127) / 128;
-    const int64_t run = gen_k2_run(slabs, rt, 3 * sm_count());
-    const int64_t grid = slabs * ((rt + run - 1) / run);
-    if (grid > 0x7FFFFFFF) return FLORA_ERR_UNSUPPORTED;
+    const bool f32 = W.dtype == FLORA_F32;
+    const int bn = gen_k2_bn(f32, gen_aligned(W)), r = (int)S.cols;
+    const int64_t units = ((W.cols + bn - 1) / bn) * ((W.rows + 127) / 128);
+    if (units > 0x7FFFFFFF) return FLORA_ERR_UNSUPPORTED;
     SeedTable table;
     table.s[0] = seed;
-    return gen_decompress_launch(W.dtype == FLORA_F32, (unsigned)grid, nullptr, nullptr, table, gen_mat(W, S), (int)run, 0, (int)S.cols, step, st, launches);
+    const GenK2Args a{(unsigned)gen_k2_grid(units, (int64_t)sm_count() * gen_k2_per_sm(f32, r, bn)), nullptr, nullptr, nullptr, &table, gen_mat(W, S), 0, r,
+                      step, st};
+    return gen_decompress_launch(f32, bn, a, launches);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -184,7 +226,10 @@ struct GenSet {
     GenMat* d_mats = nullptr;
     GenItem* d_k1 = nullptr;
     GenK2Item* d_k2 = nullptr;
-    std::vector<int> begin, first_mat;         // ranges of items per launch
+    int* d_share = nullptr;                    // decompression: per launch, the first item of every CTA and the end
+    std::vector<int> begin, first_mat;         // compression: ranges of items per launch; decompression: where its table starts in d_share
+    std::vector<unsigned> grid;                // decompression: CTAs per launch
+    int bn = 64;
     GenK1Plan plan;
     int r = 0;
     bool f32 = false;
@@ -195,6 +240,7 @@ inline void gen_set_free(GenSet& s)
     if (s.d_mats) cudaFree(s.d_mats);
     if (s.d_k1) cudaFree(s.d_k1);
     if (s.d_k2) cudaFree(s.d_k2);
+    if (s.d_share) cudaFree(s.d_share);
     s = GenSet();
 }
 // kind 0: compression (big = G), 1: decompression (big = W)
@@ -208,7 +254,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     for (int i : ids) s.h_mats[i] = gen_mat(big[i], sketch[i]);
     flora_status rc = upload(&s.d_mats, s.h_mats, false, nullptr);
     if (rc) return rc;
-    struct Cut { int mat; int64_t work; GenItem k1; GenK2Item k2; };
+    struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
     auto launches_of = [&](auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
         size_t u0 = 0;
@@ -252,26 +298,50 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         for (int i : ids) {
             const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = (int64_t)(cluster / split[i]) * T;
             for (int64_t t0 = 0; t0 < tiles; t0 += per)
-                cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]), {i, (int32_t)t0, split[i], 0}, {}});
+                cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]), {i, (int32_t)t0, split[i], 0}});
         }
         std::vector<GenItem> items;
-        launches_of([&](const Cut& c) { items.push_back(c.k1); });
+        launches_of([&](const Cut& c) { items.push_back(c.item); });
         return upload(&s.d_k1, items, false, nullptr);
     }
-    int64_t total = 0;
-    for (int i : ids) total += ((big[i].rows + 127) / 128) * ((big[i].cols + GEN_BN - 1) / GEN_BN);
-    const int64_t run_max = std::max<int64_t>(1, total / (sms * 3 * 3));
-    for (int i : ids) {
-        const int64_t rt = (big[i].rows + 127) / 128, runs = (rt + run_max - 1) / run_max;
-        if (rt == 0 || big[i].cols == 0) continue;
-        const int64_t run = (rt + runs - 1) / runs;
-        for (int64_t c0 = 0; c0 < big[i].cols; c0 += GEN_BN)
-            for (int64_t t0 = 0; t0 < rt; t0 += run)
-                cuts.push_back({i, std::min(run, rt - t0), {}, {i, (int32_t)c0, (int32_t)t0, (int32_t)std::min(run, rt - t0)}});
-    }
+    // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
+    bool aligned = true;
+    for (int i : ids) aligned = aligned && gen_aligned(big[i]);
+    s.bn = gen_k2_bn(s.f32, aligned);
     std::vector<GenK2Item> items;
-    launches_of([&](const Cut& c) { items.push_back(c.k2); });
-    return upload(&s.d_k2, items, false, nullptr);
+    std::vector<int> share;
+    size_t k0 = 0;
+    while (k0 < ids.size()) {
+        size_t k1 = k0;
+        int64_t units = 0;
+        for (; k1 < ids.size() && ids[k1] < ids[k0] + SEEDS_PER_LAUNCH; ++k1)
+            units += ((big[ids[k1]].rows + 127) / 128) * ((big[ids[k1]].cols + s.bn - 1) / s.bn);
+        const int64_t ctas = gen_k2_grid(units, sms * gen_k2_per_sm(s.f32, s.r, s.bn));
+        s.begin.push_back((int)share.size());
+        s.first_mat.push_back(ids[k0]);
+        s.grid.push_back(units ? (unsigned)ctas : 0u);
+        int64_t pos = 0, c = 0;
+        share.push_back((int)items.size());
+        for (size_t k = k0; k < k1; ++k) {
+            const int i = ids[k];
+            const int64_t rt = (big[i].rows + 127) / 128;
+            for (int64_t c0 = 0; c0 < big[i].cols; c0 += s.bn)
+                for (int64_t t0 = 0; t0 < rt;) {
+                    while (pos == (c + 1) * units / ctas) {
+                        share.push_back((int)items.size());
+                        ++c;
+                    }
+                    const int64_t take = std::min(rt - t0, (c + 1) * units / ctas - pos);
+                    items.push_back({i, (int32_t)c0, (int32_t)t0, (int32_t)take});
+                    pos += take;
+                    t0 += take;
+                }
+        }
+        share.push_back((int)items.size());
+        k0 = k1;
+    }
+    rc = upload(&s.d_k2, items, false, nullptr);
+    return rc ? rc : upload(&s.d_share, share, false, nullptr);
 }
 inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
 {
@@ -290,9 +360,11 @@ inline flora_status gen_set_compress(const GenSet& s, const uint64_t* seeds, flo
 }
 inline flora_status gen_set_decompress(const GenSet& s, const uint64_t* seeds, float step, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
-    for (size_t l = 0; l + 1 < s.begin.size(); ++l) {
-        const flora_status rc = gen_decompress_launch(s.f32, (unsigned)(s.begin[l + 1] - s.begin[l]), s.d_mats, s.d_k2 + s.begin[l],
-                                                      gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 0, s.first_mat[l], s.r, step, st, launches);
+    for (size_t l = 0; l < s.grid.size(); ++l) {
+        if (s.grid[l] == 0) continue;
+        const SeedTable table = gen_seeds(s, seeds, s.first_mat[l]);
+        const GenK2Args a{s.grid[l], s.d_mats, s.d_k2, s.d_share + s.begin[l], &table, GenMat{}, s.first_mat[l], s.r, step, st};
+        const flora_status rc = gen_decompress_launch(s.f32, s.bn, a, launches);
         if (rc) return rc;
     }
     return FLORA_OK;
