@@ -81,8 +81,7 @@ __device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, f
         ptx::st_shared_v2(addr + part_bytes, pack_high(p0.m, p1.m), pack_high(p2.m, p3.m));
         ptx::st_shared_v2(addr + 2 * part_bytes, pack_high(p0.l, p1.l), pack_high(p2.l, p3.l));
     } else {
-        __nv_bfloat162 lo = __floats2bfloat162_rn(x0, x1), hi = __floats2bfloat162_rn(x2, x3);
-        ptx::st_shared_v2(addr, *reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+        ptx::st_shared_v2(addr, pack_bf16(x0, x1), pack_bf16(x2, x3));
     }
 }
 
@@ -308,11 +307,22 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         auto generate = [&](int ks, uint32_t st) {
             const uint32_t q0 = (uint32_t)(ks0 + ks) * QPR;
             int t = first;
-            for (; t < tasks; t += 32 * GEN_WORKERS) {
+            auto put = [&](int t, const float (&v)[4]) {
                 const int j = t / QPR, q = t % QPR;
-                float v[4];
-                projection_quad(q0 + q, (uint32_t)j, key, scale, v);
                 store_quad<C::PARTS>(st + g_bytes + operand_offset<C::ROWB>(j, q >> 1) + (q & 1) * 8, a_part, v[0], v[1], v[2], v[3]);
+            };
+            for (; t + 32 * GEN_WORKERS < tasks; t += 64 * GEN_WORKERS) {
+                const int u = t + 32 * GEN_WORKERS;
+                float v[4], w[4];
+                projection_two_quads(q0 + t % QPR, (uint32_t)(t / QPR), q0 + u % QPR, (uint32_t)(u / QPR), key, scale, v, w);
+                put(t, v);
+                put(u, w);
+            }
+            if (t < tasks) {
+                float v[4];
+                projection_quad(q0 + t % QPR, (uint32_t)(t / QPR), key, scale, v);
+                put(t, v);
+                t += 32 * GEN_WORKERS;
             }
             first = t - tasks;
         };
@@ -610,11 +620,15 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                 const int cq = t % (BN / 4), g = t / (BN / 4);
                 float v[4][4];
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) {
-                    float q[4] = {0.f, 0.f, 0.f, 0.f};
-                    if (g * 4 + jj < r) projection_quad((uint32_t)(item.col0 / 4 + cq), (uint32_t)(g * 4 + jj), key, scale, q);
+                for (int jj = 0; jj < 4; jj += 2) {
+                    float v0[4] = {0.f, 0.f, 0.f, 0.f}, v1[4] = {0.f, 0.f, 0.f, 0.f};
+                    const uint32_t q = (uint32_t)(item.col0 / 4 + cq), j = (uint32_t)(g * 4 + jj);
+                    if ((int)j < r) projection_two_quads(q, j, q, j + 1, key, scale, v0, v1);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) v[k][jj] = q[k];
+                    for (int k = 0; k < 4; ++k) {
+                        v[k][jj] = v0[k];
+                        v[k][jj + 1] = (int)j + 1 < r ? v1[k] : 0.0f;
+                    }
                 }
                 const int kc = g * 4 / KB, c16 = (g * 4 % KB) >> 3, half = g & 1;
 #pragma unroll

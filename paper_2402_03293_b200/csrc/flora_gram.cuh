@@ -156,16 +156,15 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
                 const int tt = is_new ? t - per_mat : t;
                 const int j = tt / cpr, c = tt % cpr;
                 const PhiloxKey key = is_new ? key_new : key_old;
-                uint2 lo = projection_quad_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
-                uint2 hi = projection_quad_bf16(q0 + 2 * c + 1, (uint32_t)j, key, scale);
+                uint4 v = projection_octet_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
                 if (ragged) {                              // columns >= m contribute nothing
                     const int64_t col = col_base + 8 * c;
-                    lo.x = mask_pair(lo.x, col, job.m);
-                    lo.y = mask_pair(lo.y, col + 2, job.m);
-                    hi.x = mask_pair(hi.x, col + 4, job.m);
-                    hi.y = mask_pair(hi.y, col + 6, job.m);
+                    v.x = mask_pair(v.x, col, job.m);
+                    v.y = mask_pair(v.y, col + 2, job.m);
+                    v.z = mask_pair(v.z, col + 4, job.m);
+                    v.w = mask_pair(v.w, col + 6, job.m);
                 }
-                ptx::st_shared_v4(st + (is_new ? old_bytes : 0u) + j * 128 + ((c ^ (j & 7)) << 4), lo.x, lo.y, hi.x, hi.y);
+                ptx::st_shared_v4(st + (is_new ? old_bytes : 0u) + j * 128 + ((c ^ (j & 7)) << 4), v.x, v.y, v.z, v.w);
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();

@@ -297,12 +297,9 @@ compress_pair_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict
             const int t = part * 32 + lane;
             if (t < my_tasks) {
                 const int lr = lrow0 + (t >> 3), j = j0 + (t >> 3), c = t & 7;
-                uint2 lo = make_uint2(0u, 0u), hi = make_uint2(0u, 0u);
-                if (j < r) {
-                    lo = projection_quad_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
-                    hi = projection_quad_bf16(q0 + 2 * c + 1, (uint32_t)j, key, scale);
-                }
-                ptx::st_shared_v4(a_tile + lr * 128 + ((c ^ (lr & 7)) << 4), lo.x, lo.y, hi.x, hi.y);
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (j < r) v = projection_octet_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
+                ptx::st_shared_v4(a_tile + lr * 128 + ((c ^ (lr & 7)) << 4), v.x, v.y, v.z, v.w);
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();

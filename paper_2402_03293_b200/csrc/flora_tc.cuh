@@ -96,7 +96,9 @@ struct K1Smem {                            // barriers and scalars, placed after
     int epi_go[4];
 };
 
-__global__ void __launch_bounds__(K1_MAX_THREADS, 1)
+// (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
+// 4096 x 11008 matrix takes 27 us instead of 20)
+__global__ void __maxnreg__(80)
 compress_tc_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
                    int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int S, int GW, int P, int late_wait)
 {
@@ -249,9 +251,8 @@ compress_tc_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict__
             if (S == 1) {
                 for (int t = g; t < tasks; t += team_threads) {
                     const int j = t >> 3, c = t & 7;
-                    const uint2 lo = projection_quad_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
-                    const uint2 hi = projection_quad_bf16(q0 + 2 * c + 1, (uint32_t)j, key, scale);
-                    ptx::st_shared_v4(a_tile + j * 128 + ((c ^ (j & 7)) << 4), lo.x, lo.y, hi.x, hi.y);
+                    const uint4 v = projection_octet_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
+                    ptx::st_shared_v4(a_tile + j * 128 + ((c ^ (j & 7)) << 4), v.x, v.y, v.z, v.w);
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
@@ -264,9 +265,8 @@ compress_tc_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict__
                 for (int t = g; t < my_tasks; t += team_threads) {
                     const int j = (int)rank * rows_per_cta + (t >> 3), c = t & 7;
                     if (j < r) {
-                        const uint2 lo = projection_quad_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
-                        const uint2 hi = projection_quad_bf16(q0 + 2 * c + 1, (uint32_t)j, key, scale);
-                        ptx::st_shared_v4(a_tile + j * 128 + ((c ^ (j & 7)) << 4), lo.x, lo.y, hi.x, hi.y);
+                        const uint4 v = projection_octet_bf16(q0 + 2 * c, (uint32_t)j, key, scale);
+                        ptx::st_shared_v4(a_tile + j * 128 + ((c ^ (j & 7)) << 4), v.x, v.y, v.z, v.w);
                     }
                 }
                 ptx::fence_proxy_async_smem();
@@ -426,13 +426,9 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
             for (int jj = 0; jj < 8; jj += 2) {
                 float v0[4] = {0.f, 0.f, 0.f, 0.f}, v1[4] = {0.f, 0.f, 0.f, 0.f};
                 const int j = jg * 8 + jj;
-                if (j < r) projection_quad((uint32_t)(col0 / 4 + cq), (uint32_t)j, key, scale, v0);
-                if (j + 1 < r) projection_quad((uint32_t)(col0 / 4 + cq), (uint32_t)(j + 1), key, scale, v1);
+                if (j < r) projection_two_quads((uint32_t)(col0 / 4 + cq), (uint32_t)j, (uint32_t)(col0 / 4 + cq), (uint32_t)(j + 1), key, scale, v0, v1);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    __nv_bfloat162 pr = __floats2bfloat162_rn(v0[u], v1[u]);
-                    packed[u][jj >> 1] = *reinterpret_cast<uint32_t*>(&pr);
-                }
+                for (int u = 0; u < 4; ++u) packed[u][jj >> 1] = pack_bf16(v0[u], j + 1 < r ? v1[u] : 0.0f);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -442,11 +438,15 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
         } else {
             float v[4][4];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                float q[4] = {0.f, 0.f, 0.f, 0.f};
-                if (jg * 4 + jj < r) projection_quad((uint32_t)(col0 / 4 + cq), (uint32_t)(jg * 4 + jj), key, scale, q);
+            for (int jj = 0; jj < 4; jj += 2) {
+                float v0[4] = {0.f, 0.f, 0.f, 0.f}, v1[4] = {0.f, 0.f, 0.f, 0.f};
+                const int j = jg * 4 + jj;
+                if (j < r) projection_two_quads((uint32_t)(col0 / 4 + cq), (uint32_t)j, (uint32_t)(col0 / 4 + cq), (uint32_t)(j + 1), key, scale, v0, v1);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v[u][jj] = bf16_round(q[u]);
+                for (int u = 0; u < 4; ++u) {
+                    v[u][jj] = bf16_round(v0[u]);
+                    v[u][jj + 1] = j + 1 < r ? bf16_round(v1[u]) : 0.0f;
+                }
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
