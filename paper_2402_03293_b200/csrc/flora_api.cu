@@ -220,13 +220,12 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
 static flora_status set_build(flora_set* s)
 {
     tc_set_free(s->tc);
-    s->tc = TcSet();
     for (int d = 0; d < 2; ++d) {
         gen_set_free(s->gen_g[d]);
         gen_set_free(s->gen_w[d]);
     }
     const std::vector<uint8_t> use_g = set_tma_side(s->G, s->S), use_w = set_tma_side(s->W, s->S);
-    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, false, nullptr, use_g, use_w);
+    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
         std::vector<int> g, w;
         for (size_t i = 0; i < s->S.size(); ++i) {

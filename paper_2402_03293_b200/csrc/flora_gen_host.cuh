@@ -252,7 +252,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     s.f32 = big[ids[0]].dtype == FLORA_F32;
     s.h_mats.assign(big.size(), GenMat{});
     for (int i : ids) s.h_mats[i] = gen_mat(big[i], sketch[i]);
-    flora_status rc = upload(&s.d_mats, s.h_mats, false, nullptr);
+    flora_status rc = upload(&s.d_mats, s.h_mats, nullptr);
     if (rc) return rc;
     struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
@@ -302,7 +302,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         }
         std::vector<GenItem> items;
         launches_of([&](const Cut& c) { items.push_back(c.item); });
-        return upload(&s.d_k1, items, false, nullptr);
+        return upload(&s.d_k1, items, nullptr);
     }
     // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
     bool aligned = true;
@@ -340,8 +340,8 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         share.push_back((int)items.size());
         k0 = k1;
     }
-    rc = upload(&s.d_k2, items, false, nullptr);
-    return rc ? rc : upload(&s.d_share, share, false, nullptr);
+    rc = upload(&s.d_k2, items, nullptr);
+    return rc ? rc : upload(&s.d_share, share, nullptr);
 }
 inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
 {
@@ -379,7 +379,7 @@ inline flora_status gen_set_rebind(GenSet& s, const std::vector<flora_mat>& big,
         aligned = aligned && gen_aligned(big[i]);
     }
     s.plan.aligned = aligned;
-    return upload(&s.d_mats, s.h_mats, false, st);
+    return upload(&s.d_mats, s.h_mats, st);
 }
 
 }  // namespace flora

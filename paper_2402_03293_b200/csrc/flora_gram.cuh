@@ -667,9 +667,7 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     // last kernel; nothing then stands between that kernel and the caller's next launch
     if (release_later) *release_later = nullptr;
     if (jobs.empty()) return FLORA_OK;
-    int sms = 148, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     // step width: 64 columns, or narrower while that leaves fewer than four steps per SM to balance
     int64_t total_cols = 0;
     int max_n = 1;

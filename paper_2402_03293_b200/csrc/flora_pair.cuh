@@ -48,11 +48,13 @@ struct PairSmem {
 // A CTA of rank q in its cluster belongs to pair q / 2 and holds half h = q % 2 of every A tile: rows
 // [h N/2, (h+1) N/2).  Of that half it generates the rows [pair * N/S, (pair+1) * N/S) and receives the rest from
 // the CTAs of the same parity.  The even CTA of a pair (the leader) issues the MMAs for both.
+template <bool SINGLE>
 __global__ void __launch_bounds__(PAIR_MAX_THREADS, 1)
-compress_pair_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict__ items, const int* __restrict__ slot_begin,
+compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K1Item* __restrict__ items, const int* __restrict__ slot_begin,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, int N, float scale, float a, float b, int gstages,
                      int astages, int S, int GW, int late_wait)
 {
+    const TcMatrix* mats = SINGLE ? &single : table;                   // (one matrix: every unit names matrix 0)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     const uint32_t g_bytes = (uint32_t)PAIR_T * G_TILE_BYTES;          // one stage of the G ring

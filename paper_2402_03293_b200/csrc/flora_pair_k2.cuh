@@ -51,10 +51,12 @@ struct K2Cursor {
 // 2p (leader) and 2p + 1 (follower; it may not exist, then the follower loads and stores nothing for that iteration).
 // Iterations are numbered through all items of the cluster (gt); the even ones belong to the first MMA thread, its
 // ring of sketch chunks (cstages / 2 stages) and accumulators 0 and 2, the odd ones to the second.
+template <bool SINGLE>
 __global__ void __launch_bounds__(K2P_THREADS, 1)
-decompress_pair_kernel(const TcMatrix* __restrict__ mats, const K2Item* __restrict__ items, int n_items, const __grid_constant__ SeedTable seeds,
+decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K2Item* __restrict__ items, int n_items, const __grid_constant__ SeedTable seeds,
                        int seed_base, int r, float scale, float step, int slots, int cstages)
 {
+    const TcMatrix* mats = SINGLE ? &single : table;            // (one matrix: every item names matrix 0)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     const int kchunks = (r + 63) >> 6;                          // 64 values of the rank per 128-byte row of bf16

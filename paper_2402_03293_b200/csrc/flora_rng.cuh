@@ -91,18 +91,18 @@ __device__ __forceinline__ f32x2 neg2_ln_u1(uint32_t xa0, uint32_t xa1)
 {
     const uint32_t b0 = __float_as_uint(__uint2float_rn((xa0 >> 8) + 1u)), b1 = __float_as_uint(__uint2float_rn((xa1 >> 8) + 1u));   // exact
     const uint32_t e0 = (b0 - 0x3F2AAAABu) & 0xFF800000u, e1 = (b1 - 0x3F2AAAABu) & 0xFF800000u;         // e * 2^23
-    const f32x2 t = fma2(pack2(__uint_as_float(b0 - e0), __uint_as_float(b1 - e1)), FLORA_BOTH(0xC0000000)/*-2.0*/, FLORA_BOTH(0x40000000)/*2.0*/);                        // exact
-    f32x2 q = FLORA_BOTH(0x3A0D84F4)/*0x1.1b09e8p-11*/;
-    q = fma2(q, t, FLORA_BOTH(0x3A9AD9F0)/*0x1.35b3ep-10*/);
-    q = fma2(q, t, FLORA_BOTH(0x3B0FCB11)/*0x1.1f9622p-9*/);
-    q = fma2(q, t, FLORA_BOTH(0x3BA8AD36)/*0x1.515a6cp-8*/);
-    q = fma2(q, t, FLORA_BOTH(0x3C4CE190)/*0x1.99c32p-7*/);
-    q = fma2(q, t, FLORA_BOTH(0x3D00058E)/*0x1.000b1cp-5*/);
-    q = fma2(q, t, FLORA_BOTH(0x3DAAAA94)/*0x1.555528p-4*/);
-    q = fma2(q, t, FLORA_BOTH(0x3E800000)/*0.25*/);
+    const f32x2 t = fma2(pack2(__uint_as_float(b0 - e0), __uint_as_float(b1 - e1)), FLORA_BOTH(0xC0000000) /* -2.0 */, FLORA_BOTH(0x40000000) /* 2.0 */);   // exact
+    f32x2 q = FLORA_BOTH(0x3A0D84F4) /* 0x1.1b09e8p-11 */;
+    q = fma2(q, t, FLORA_BOTH(0x3A9AD9F0) /* 0x1.35b3ep-10 */);
+    q = fma2(q, t, FLORA_BOTH(0x3B0FCB11) /* 0x1.1f9622p-9 */);
+    q = fma2(q, t, FLORA_BOTH(0x3BA8AD36) /* 0x1.515a6cp-8 */);
+    q = fma2(q, t, FLORA_BOTH(0x3C4CE190) /* 0x1.99c32p-7 */);
+    q = fma2(q, t, FLORA_BOTH(0x3D00058E) /* 0x1.000b1cp-5 */);
+    q = fma2(q, t, FLORA_BOTH(0x3DAAAA94) /* 0x1.555528p-4 */);
+    q = fma2(q, t, FLORA_BOTH(0x3E800000) /* 0.25 */);
     const f32x2 ln_mant = fma2(q, mul2(t, t), t);
-    const f32x2 steps = fma2(pack2(__int2float_rn((int)e0), __int2float_rn((int)e1)), FLORA_BOTH(0xB4000000)/*-0x1p-23*/, FLORA_BOTH(0x41C00000)/*24.0*/);                 // 24 - e, exact
-    return fma2(steps, FLORA_BOTH(0x3FB17218)/*0x1.62e43p+0*/, ln_mant);
+    const f32x2 steps = fma2(pack2(__int2float_rn((int)e0), __int2float_rn((int)e1)), FLORA_BOTH(0xB4000000) /* -0x1p-23 */, FLORA_BOTH(0x41C00000) /* 24.0 */);   // 24 - e, exact
+    return fma2(steps, FLORA_BOTH(0x3FB17218) /* 0x1.62e43p+0 */, ln_mant);
 }
 
 // Square roots of two values of neg2_ln_u1, rounded to nearest: one Newton (Heron) step g + (x - g^2) / (2 g) from the
@@ -115,7 +115,7 @@ __device__ __forceinline__ f32x2 sqrt_of_ln(f32x2 x)
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(fmaxf(x0, 1e-20f)));
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y1) : "f"(fmaxf(x1, 1e-20f)));
     const f32x2 y = pack2(y0, y1), g = mul2(x, y);
-    return fma2(fma2(mul2(g, FLORA_BOTH(0xBF800000)/*-1.0*/), g, x), mul2(y, FLORA_BOTH(0x3F000000)/*0.5*/), g);
+    return fma2(fma2(mul2(g, FLORA_BOTH(0xBF800000) /* -1.0 */), g, x), mul2(y, FLORA_BOTH(0x3F000000) /* 0.5 */), g);
 }
 
 // cos and sin of 2 pi (xb >> 8) / 2^24, of two words, without the exchange and the signs of their octants: fixed polynomials
@@ -123,14 +123,14 @@ __device__ __forceinline__ f32x2 sqrt_of_ln(f32x2 x)
 __device__ __forceinline__ void cos_sin_octant(uint32_t xb0, uint32_t xb1, f32x2& c, f32x2& s)
 {
     const float q0 = fabsf(__int2float_rn((int)((xb0 << 2) & 0xFFFFFC00u))), q1 = fabsf(__int2float_rn((int)((xb1 << 2) & 0xFFFFFC00u)));  // exact
-    const f32x2 x = mul2(pack2(q0, q1), FLORA_BOTH(0x2FC90FDB)/*0x1.921fb6p-32*/);
+    const f32x2 x = mul2(pack2(q0, q1), FLORA_BOTH(0x2FC90FDB) /* 0x1.921fb6p-32 */);
     const f32x2 z = mul2(x, x);
-    f32x2 sp = fma2(FLORA_BOTH(0xB94CA1F1)/*-0x1.9943e2p-13*/, z, FLORA_BOTH(0x3C08839D)/*0x1.11073ap-7*/);
-    sp = fma2(sp, z, FLORA_BOTH(0xBE2AAAA3)/*-0x1.555546p-3*/);
+    f32x2 sp = fma2(FLORA_BOTH(0xB94CA1F1) /* -0x1.9943e2p-13 */, z, FLORA_BOTH(0x3C08839D) /* 0x1.11073ap-7 */);
+    sp = fma2(sp, z, FLORA_BOTH(0xBE2AAAA3) /* -0x1.555546p-3 */);
     s = fma2(mul2(x, z), sp, x);
-    f32x2 cp = fma2(FLORA_BOTH(0xBAB226B1)/*-0x1.644d62p-10*/, z, FLORA_BOTH(0x3D2A9F40)/*0x1.553e8p-5*/);
-    cp = fma2(cp, z, FLORA_BOTH(0xBEFFFFD9)/*-0x1.ffffb2p-2*/);
-    c = fma2(z, cp, FLORA_BOTH(0x3F800000)/*1.0*/);
+    f32x2 cp = fma2(FLORA_BOTH(0xBAB226B1) /* -0x1.644d62p-10 */, z, FLORA_BOTH(0x3D2A9F40) /* 0x1.553e8p-5 */);
+    cp = fma2(cp, z, FLORA_BOTH(0xBEFFFFD9) /* -0x1.ffffb2p-2 */);
+    c = fma2(z, cp, FLORA_BOTH(0x3F800000) /* 1.0 */);
 }
 // One word's octant: cosine and sine change places in the odd half of each quarter turn, and take their signs.
 __device__ __forceinline__ f32x2 in_octant(uint32_t xb, float c, float s)

@@ -96,10 +96,12 @@ struct K1Smem {                            // barriers and scalars, placed after
     int epi_go[4];
 };
 
+// SINGLE: one matrix, its record passed by value (every item names matrix 0).
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
 // 4096 x 11008 matrix takes 27 us instead of 20)
+template <bool SINGLE>
 __global__ void __maxnreg__(80)
-compress_tc_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
+compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
                    int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int S, int GW, int P, int late_wait)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -115,7 +117,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ mats, const K1Item* __restrict__
 
     ptx::grid_launch_dependents();
     const K1Item item = items[blockIdx.x];                    // tables and descriptors are written at set creation, not by kernels
-    const TcMatrix* mat = mats + item.mat;
+    const TcMatrix* mat = SINGLE ? &single : table + item.mat;
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < T * r_pad) tmem_cols <<= 1;
 
@@ -458,12 +460,13 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
     }
 }
 
-template <bool BF16S>
+template <bool SINGLE, bool BF16S>
 __global__ void __launch_bounds__(K2_MAX_THREADS, 1)
-decompress_tc_kernel(const TcMatrix* __restrict__ mats, const K2Item* __restrict__ items, int n_items,
+decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K2Item* __restrict__ items, int n_items,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, float scale, float step, int bn, int slots,
                      int cstages, int GW, int nslabs)
 {
+    const TcMatrix* mats = SINGLE ? &single : table;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     // K chunks: one 128-byte row of S each (32 fp32 values, or 64 bf16 values when the bf16 copy of S is used)
@@ -739,10 +742,12 @@ decompress_tc_kernel(const TcMatrix* __restrict__ mats, const K2Item* __restrict
 
 // S <- b S for the listed matrices (those whose rows receive adds), or for matrix first + blockIdx.y of the table
 // where there is no list; blockIdx.y = list entry.
-__global__ void scale_sketches_kernel(const TcMatrix* __restrict__ mats, const int* __restrict__ ids, int first, int r, float b)
+template <bool SINGLE>
+__global__ void scale_sketches_kernel(const TcMatrix* __restrict__ mats, const __grid_constant__ TcMatrix single, const int* __restrict__ ids, int first, int r,
+                                      float b)
 {
     ptx::grid_launch_dependents();       // the compression kernel that follows may start streaming G right away
-    const TcMatrix* mat = mats + (ids ? ids[blockIdx.y] : first + (int)blockIdx.y);
+    const TcMatrix* mat = SINGLE ? &single : mats + (ids ? ids[blockIdx.y] : first + (int)blockIdx.y);
     float* S = mat->S;
     const int64_t total = (int64_t)mat->n * r;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
@@ -769,10 +774,11 @@ __global__ void scale_sketches_kernel(const TcMatrix* __restrict__ mats, const i
 // kernel for ranks above 64); blockIdx.y = matrix.  A thread converts eight neighbouring columns of one row: two
 // 16-byte loads (the sketches that reach this kernel have 16-byte aligned rows), one 16-byte store; a block of 256
 // threads covers 2048 / k_pad rows at a time.
-__global__ void __launch_bounds__(256) sketch_to_bf16_kernel(const TcMatrix* __restrict__ mats, int r, int k_pad)
+template <bool SINGLE>
+__global__ void __launch_bounds__(256) sketch_to_bf16_kernel(const TcMatrix* __restrict__ mats, const __grid_constant__ TcMatrix single, int r, int k_pad)
 {
     ptx::grid_launch_dependents();       // the decompression kernel that follows may set up and generate its first slabs meanwhile
-    const TcMatrix* mat = mats + blockIdx.y;
+    const TcMatrix* mat = SINGLE ? &single : mats + blockIdx.y;
     const int groups = k_pad >> 3;                        // 8-column groups per row: 8, 16, 24 or 32
     const int rows_per_block = 256 / groups;
     const int g = (int)threadIdx.x % groups, lr = (int)threadIdx.x / groups;

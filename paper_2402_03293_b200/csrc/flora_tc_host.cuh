@@ -27,7 +27,6 @@ namespace flora {
 struct TcSet {
     bool compress_ready = false;
     bool decompress_ready = false;
-    bool transient = false;             // device buffers come from the stream-ordered allocator
     int count = 0, r = 0;
     int T = 1, gstages = 2, astages = 2, S = 1, GW = 8, P = 1;
     std::vector<int> k1_launch_first_mat;
@@ -119,14 +118,22 @@ inline bool tc_compress_supported(const flora_mat* big, const flora_mat* sketch)
     return tc_mat_ok(*big) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
 }
 
-// SMs of the current device (queried on every call: a process may drive several devices).
+// SMs of the current device (a process may drive several devices), asked once per device.
 inline int sm_count()
 {
+    static std::atomic<int> known[POOL_MAX_DEVICES] = {};
     int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_MAX_DEVICES) {
         cudaGetLastError();
-        n = 148;
+        return 148;
     }
+    n = known[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
+        cudaGetLastError();
+        return 148;
+    }
+    known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -161,21 +168,21 @@ template <auto Kernel>
 inline bool raise_smem_limit()
 {
     static std::mutex mutex;
-    static bool done[POOL_MAX_DEVICES] = {};
+    static std::atomic<bool> done[POOL_MAX_DEVICES] = {};
     int dev = -1, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_MAX_DEVICES) {
         cudaGetLastError();
         return false;
     }
+    if (done[dev].load(std::memory_order_acquire)) return true;
     std::lock_guard<std::mutex> lock(mutex);
-    if (done[dev]) return true;
     cudaFuncAttributes fa;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || cudaFuncGetAttributes(&fa, Kernel) != cudaSuccess ||
         cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    done[dev] = true;
+    done[dev].store(true, std::memory_order_release);
     return true;
 }
 
@@ -275,7 +282,7 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
     set.gstages = gstages;
     set.astages = astages;
     set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + staging + sizeof(PairSmem) + 1024;
-    const int64_t slots = resident_clusters<compress_pair_kernel>(S, pair_threads(GW), set.k1_smem);
+    const int64_t slots = resident_clusters<compress_pair_kernel<false>>(S, pair_threads(GW), set.k1_smem);
     const int64_t group_tiles = (int64_t)S * T;
     struct Unit { int mat; int64_t tile0, tiles, kstep0, ksteps; bool direct; };
     auto build_units = [&](int64_t target, std::vector<Unit>& units, std::vector<int>& split) {
@@ -473,7 +480,7 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + sizeof(K1Smem) + 1024;
     // column chunks: aim at about `waves` items per slot (a slot is a CTA, or a cluster), at least 8 steps each
     int64_t slots = std::max<int64_t>(1, (int64_t)sm_count() * per_sm / S);
-    if (S > 1) slots = resident_clusters<compress_tc_kernel>(S, k1_threads(set.GW), set.k1_smem);
+    if (S > 1) slots = resident_clusters<compress_tc_kernel<false>>(S, k1_threads(set.GW), set.k1_smem);
     const int64_t group_tiles = (int64_t)S * T;                      // rows of one slot, in tiles
     struct Unit { int mat; int64_t tile0, tiles, kstep0, ksteps; bool direct; };
     auto build_units = [&](int64_t target, std::vector<Unit>& units, std::vector<int>& split) {
@@ -798,43 +805,25 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     set.k2_grid_max = balanced ? balanced_grid : grid_max;
 }
 
-inline void tc_set_free_stream(TcSet& s, cudaStream_t st)
+inline void tc_set_free(TcSet& s)
 {
-    if (s.transient) {
-        if (s.d_mats) cudaFreeAsync(s.d_mats, st);
-        if (s.d_k1) cudaFreeAsync(s.d_k1, st);
-        if (s.d_k2) cudaFreeAsync(s.d_k2, st);
-        if (s.d_split) cudaFreeAsync(s.d_split, st);
-        if (s.d_members) cudaFreeAsync(s.d_members, st);
-        if (s.d_slots) cudaFreeAsync(s.d_slots, st);
-        if (s.d_sb) cudaFreeAsync(s.d_sb, st);
-    } else {
-        if (s.d_mats) cudaFree(s.d_mats);
-        if (s.d_k1) cudaFree(s.d_k1);
-        if (s.d_k2) cudaFree(s.d_k2);
-        if (s.d_split) cudaFree(s.d_split);
-        if (s.d_members) cudaFree(s.d_members);
-        if (s.d_slots) cudaFree(s.d_slots);
-        if (s.d_sb) cudaFree(s.d_sb);
-    }
-    s.d_mats = nullptr;
-    s.d_k1 = nullptr;
-    s.d_k2 = nullptr;
-    s.d_split = nullptr;
-    s.d_members = nullptr;
-    s.d_slots = nullptr;
-    s.d_sb = nullptr;
-    s.compress_ready = s.decompress_ready = false;
+    if (s.d_mats) cudaFree(s.d_mats);
+    if (s.d_k1) cudaFree(s.d_k1);
+    if (s.d_k2) cudaFree(s.d_k2);
+    if (s.d_split) cudaFree(s.d_split);
+    if (s.d_members) cudaFree(s.d_members);
+    if (s.d_slots) cudaFree(s.d_slots);
+    if (s.d_sb) cudaFree(s.d_sb);
+    s = TcSet();
 }
-inline void tc_set_free(TcSet& s) { tc_set_free_stream(s, nullptr); }
 
 template <typename T>
-inline flora_status upload(T** dst, const std::vector<T>& src, bool transient, cudaStream_t st)
+inline flora_status upload(T** dst, const std::vector<T>& src, cudaStream_t st)
 {
     if (src.empty()) return FLORA_OK;
     const size_t bytes = src.size() * sizeof(T);
     if (!*dst) {
-        cudaError_t e = transient ? scratch_alloc((void**)dst, bytes, st) : cudaMalloc((void**)dst, bytes);
+        cudaError_t e = cudaMalloc((void**)dst, bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return FLORA_ERR_ALLOC;
@@ -875,10 +864,9 @@ inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const
 // Builds the tensor-core side of a set for the matrices marked in use_g (compression) and use_w (decompression); the planners
 // see the others as empty.  The descriptors of the sketches are made for every matrix whose sketch TMA can address.
 inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_all, const std::vector<flora_mat>& W_all,
-                                    const std::vector<flora_mat>& S, bool transient, cudaStream_t st, const std::vector<uint8_t>& use_g,
+                                    const std::vector<flora_mat>& S, cudaStream_t st, const std::vector<uint8_t>& use_g,
                                     const std::vector<uint8_t>& use_w)
 {
-    set.transient = transient;
     set.count = (int)S.size();
     if (S.empty() || !encode_tiled_fn()) return FLORA_OK;
     set.r = (int)S[0].cols;
@@ -913,7 +901,7 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_
                 total += (((size_t)W[i].rows * k_pad * 2) + 1023) & ~(size_t)1023;
             }
             if (total) {
-                cudaError_t e = transient ? scratch_alloc((void**)&set.d_sb, total, st) : cudaMalloc((void**)&set.d_sb, total);
+                cudaError_t e = cudaMalloc((void**)&set.d_sb, total);
                 if (e != cudaSuccess) {
                     cudaGetLastError();
                     return FLORA_ERR_ALLOC;
@@ -933,22 +921,22 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_
             }
         }
     }
-    rc = upload(&set.d_mats, set.h_mats, transient, st);
+    rc = upload(&set.d_mats, set.h_mats, st);
     if (rc) return rc;
     if (g_ok) {
         plan_compress(set, G, set.r);
-        rc = upload(&set.d_k1, set.h_k1, transient, st);
+        rc = upload(&set.d_k1, set.h_k1, st);
         if (rc) return rc;
-        rc = upload(&set.d_split, set.split_mats, transient, st);
+        rc = upload(&set.d_split, set.split_mats, st);
         if (rc) return rc;
-        rc = upload(&set.d_slots, set.h_slots, transient, st);
+        rc = upload(&set.d_slots, set.h_slots, st);
         if (rc) return rc;
-        if (set.members.size() < S.size()) rc = upload(&set.d_members, set.members, transient, st);
+        if (set.members.size() < S.size()) rc = upload(&set.d_members, set.members, st);
         if (rc) return rc;
         set.compress_ready = true;
     }
     if (w_ok) {
-        rc = upload(&set.d_k2, set.h_k2, transient, st);
+        rc = upload(&set.d_k2, set.h_k2, st);
         if (rc) return rc;
         set.decompress_ready = true;
     }
@@ -964,24 +952,27 @@ inline flora_status tc_set_rebind(TcSet& set, const std::vector<flora_mat>& G, c
     for (int i : set.members) {
         if (G[i].rows && G[i].cols && !make_map(&set.h_mats[i].map_g, G[i])) return FLORA_ERR_CUDA;
     }
-    return upload(&set.d_mats, set.h_mats, false, st);
+    return upload(&set.d_mats, set.h_mats, st);
 }
 
 // Blocks per matrix for the element-wise helper kernels (zero, scale): about four elements per thread of the
 // largest sketch.
 constexpr int64_t K1_SCALE_PASS_MAX_STATE_BYTES = 32ll << 20;   // sketches of a set up to this size are blended by a scaling pass (below)
 
+inline unsigned helper_blocks(int64_t most) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(1024, (most + 1023) / 1024)); }
 inline unsigned helper_blocks(const TcSet& set)
 {
     int64_t most = 1;
     for (const auto& tm : set.h_mats) most = std::max<int64_t>(most, (int64_t)tm.n * set.r);
-    return (unsigned)std::min<int64_t>(1024, (most + 1023) / 1024);
+    return helper_blocks(most);
 }
 
 // behind_own_kernel: the kernel before this call on the stream is one of the library's own that does not touch G and lets
 // its dependents start early (the transfer's apply kernel): only the write-out of the compression waits for it.
-inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st,
-                                    std::atomic<uint64_t>& launches, bool behind_own_kernel = false)
+// one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).
+template <bool SINGLE>
+inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, const uint64_t* seeds, float a, float b, cudaStream_t st,
+                                       std::atomic<uint64_t>& launches, bool behind_own_kernel)
 {
     const int r = set.r;
     const float scale = 1.0f / sqrtf((float)r);
@@ -992,23 +983,25 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
     // L2 between the two (one 4096 x 11008 matrix at r = 256: 45.7 against 49.8 us; on 550 MB of sketches the pass
     // costs what it saves).  Every element still has one writer per launch, so the result does not depend on the schedule.
     int64_t state_bytes = 0;
-    for (int i : set.members) state_bytes += (int64_t)set.h_mats[i].n * r * 4;
+    if (SINGLE) state_bytes = (int64_t)one.n * r * 4;
+    else
+        for (int i : set.members) state_bytes += (int64_t)set.h_mats[i].n * r * 4;
     const bool scale_all = pair && b != 0.0f && b != 1.0f && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES;
     if (scale_all || (b != 1.0f && !set.split_mats.empty())) {
         late_wait = tune_knob("FLORA_PDL", 1, 0, 1);
         // rows that receive adds (from several CTAs, or from the pair kernel's reducing write-out): scale them by b first
-        const size_t total = scale_all ? set.members.size() : set.split_mats.size();
+        const size_t total = SINGLE ? 1 : scale_all ? set.members.size() : set.split_mats.size();
         const int* ids = scale_all ? set.d_members : set.d_split;        // (no list: every matrix of the set)
         for (size_t begin = 0; begin < total; begin += 65535) {
             const size_t jobs_here = std::min<size_t>(65535, total - begin);
             // few enough blocks to be resident at once: the compression kernel may only start once all have started
-            dim3 grid((unsigned)std::max<size_t>(1, std::min<size_t>(helper_blocks(set), (size_t)sm_count() * 6 / jobs_here)), (unsigned)jobs_here);
-            scale_sketches_kernel<<<grid, 256, 0, st>>>(set.d_mats, ids ? ids + begin : nullptr, (int)begin, r, b);
+            dim3 grid((unsigned)std::max<size_t>(1, std::min<size_t>(SINGLE ? helper_blocks(state_bytes / 4) : helper_blocks(set), (size_t)sm_count() * 6 / jobs_here)), (unsigned)jobs_here);
+            scale_sketches_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats, one, ids ? ids + begin : nullptr, (int)begin, r, b);
             launches.fetch_add(1, std::memory_order_relaxed);
         }
         if (scale_all) b = 1.0f;
     }
-    if (!(pair ? raise_smem_limit<compress_pair_kernel>() : raise_smem_limit<compress_tc_kernel>())) return FLORA_ERR_CUDA;
+    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE>>() : raise_smem_limit<compress_tc_kernel<SINGLE>>())) return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k1_launch_begin.size(); ++l) {
         const int begin = set.k1_launch_begin[l], end = set.k1_launch_begin[l + 1];
         if (end == begin) continue;
@@ -1037,10 +1030,10 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
         cudaError_t e;
         if (pair) {
             const int* slot_table = set.d_slots + set.k1_slots_begin[l];
-            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel, mats, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
+            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE>, mats, one, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
                                    set.astages, set.S, set.GW, lw);
         } else {
-            e = cudaLaunchKernelEx(&cfg, compress_tc_kernel, mats, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.S,
+            e = cudaLaunchKernelEx(&cfg, compress_tc_kernel<SINGLE>, mats, one, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.S,
                                    set.GW, set.P, lw);
         }
         if (e != cudaSuccess) return FLORA_ERR_CUDA;
@@ -1049,26 +1042,31 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
     return cudaPeekAtLastError() == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
 
-// Single-matrix calls go through a set of one matrix.  Planning it (work split, tensor maps, device tables) costs far
-// more than the launch, and an optimizer calls with the same matrices step after step: the most recent plans are kept,
-// keyed by device, operation, addresses, shapes and rank.  A plan only names addresses and shapes, so it stays valid
-// when the caller's buffers are rewritten (or freed and handed out again with the same shape).  Calls that use the
+inline flora_status tc_set_compress(const TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
+                                    bool behind_own_kernel = false)
+{
+    return tc_compress_launch<false>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel);
+}
+
+// Plans of the single-matrix calls.  Planning (work split, device tables of the items) costs far more than a launch, and an
+// optimizer calls with the same shapes step after step: the most recent plans are kept, keyed by device, operation, shape and
+// rank.  A plan holds no addresses: the matrix's record with its tensor maps is made anew for every call (0.05 us a map) and
+// passed to the kernels by value, so a loop over a whole model's matrices, or over gradients at new addresses in every step,
+// plans once per shape (a cache keyed by addresses planned every call anew in such loops: 43 us each).  Calls that use the
 // cache are serialised by its mutex; a plan is built with a synchronous upload, so any stream may use it afterwards.
 struct SinglePlanKey {
     int dev, kind, r, det;
-    const void *big, *sketch;
-    int64_t rows, cols, ld, lds;
+    int64_t rows, cols;
     bool operator==(const SinglePlanKey& o) const
     {
-        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && big == o.big && sketch == o.sketch && rows == o.rows &&
-               cols == o.cols && ld == o.ld && lds == o.lds;
+        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && rows == o.rows && cols == o.cols;
     }
 };
 struct SinglePlan {
     SinglePlanKey key;
     TcSet set;
 };
-constexpr size_t SINGLE_PLAN_CACHE = 32;
+constexpr size_t SINGLE_PLAN_CACHE = 64;
 inline std::mutex& single_plan_mutex()
 {
     static std::mutex m;
@@ -1089,17 +1087,15 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
     key.kind = kind;
     key.r = (int)sketch.cols;
     key.det = deterministic_flag().load();
-    key.big = big.data;
-    key.sketch = sketch.data;
     key.rows = big.rows;
     key.cols = big.cols;
-    key.ld = big.ld;
-    key.lds = sketch.ld;
     for (size_t i = 0; i < cache.size(); ++i)
         if (cache[i]->key == key) {
             SinglePlan* hit = cache[i];
-            cache.erase(cache.begin() + i);
-            cache.insert(cache.begin(), hit);
+            if (i > 0) {
+                cache.erase(cache.begin() + i);
+                cache.insert(cache.begin(), hit);
+            }
             return &hit->set;
         }
     SinglePlan* plan = new (std::nothrow) SinglePlan();
@@ -1108,12 +1104,22 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
         return nullptr;
     }
     plan->key = key;
-    std::vector<flora_mat> b(1, big), s(1, sketch), none;
-    const std::vector<uint8_t> use = tc_eligible(b, s);
-    *rc = kind == 0 ? tc_set_build_on(plan->set, b, none, s, false, st, use, {}) : tc_set_build_on(plan->set, none, b, s, false, st, {}, use);
+    TcSet& set = plan->set;
+    set.count = 1;
+    set.r = key.r;
+    set.members.assign(1, 0);
+    const std::vector<flora_mat> b(1, big);
+    if (kind == 0) {
+        plan_compress(set, b, set.r);
+        *rc = upload(&set.d_k1, set.h_k1, st);
+        if (*rc == FLORA_OK) *rc = upload(&set.d_slots, set.h_slots, st);
+    } else {
+        plan_decompress(set, b, set.r);
+        *rc = upload(&set.d_k2, set.h_k2, st);
+    }
     if (*rc == FLORA_OK && cudaStreamSynchronize(st) != cudaSuccess) *rc = FLORA_ERR_CUDA;      // the tables are in place for every stream
     if (*rc != FLORA_OK) {
-        tc_set_free(plan->set);
+        tc_set_free(set);
         delete plan;
         return nullptr;
     }
@@ -1124,38 +1130,52 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
         tc_set_free(old->set);                                 // cudaFree waits for kernels that still read the tables
         delete old;
     }
-    return &plan->set;
+    return &set;
+}
+// The record of one matrix; g / w: which of the big matrix's two maps is wanted.
+inline bool single_record(TcMatrix* tm, const flora_mat& big, const flora_mat& sketch, bool is_g)
+{
+    memset(tm, 0, sizeof(*tm));
+    tm->S = (float*)sketch.data;
+    tm->lds = sketch.ld;
+    tm->n = (int32_t)big.rows;
+    tm->m = (int32_t)big.cols;
+    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && make_map_f32(&tm->map_s, sketch);
 }
 
 inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, float a, float b, cudaStream_t st,
                                        std::atomic<uint64_t>& launches)
 {
+    TcMatrix one;
+    if (!single_record(&one, *G, *S, true)) return FLORA_ERR_CUDA;
     std::lock_guard<std::mutex> lock(single_plan_mutex());
     flora_status rc;
     TcSet* set = single_plan(0, *G, *S, st, &rc);
-    if (!set) return rc;
-    return set->compress_ready ? tc_set_compress(*set, &seed, a, b, st, launches) : FLORA_ERR_UNSUPPORTED;
+    return set ? tc_compress_launch<true>(*set, one, &seed, a, b, st, launches, false) : rc;
 }
 
-inline flora_status tc_set_decompress(TcSet& set, const uint64_t* seeds, float step, cudaStream_t st,
-                                      std::atomic<uint64_t>& launches)
+template <bool SINGLE>
+inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, const uint64_t* seeds, float step, cudaStream_t st,
+                                         std::atomic<uint64_t>& launches)
 {
     const int r = set.r;
     const float scale = 1.0f / sqrtf((float)r);
     if (set.k2_bf16) {
         const int k_pad = (r + 63) & ~63;
         int max_rows = 1;
-        for (const auto& tm : set.h_mats) max_rows = std::max(max_rows, tm.n);
+        if (SINGLE) max_rows = one.n;
+        else
+            for (const auto& tm : set.h_mats) max_rows = std::max(max_rows, tm.n);
         const int rows_per_block = 256 / (k_pad / 8);
         const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(256, ((int64_t)max_rows + 4 * rows_per_block - 1) / (4 * rows_per_block)));   // about four rows per thread
         for (int begin = 0; begin < set.count; begin += 65535) {
             dim3 grid(bx, (unsigned)std::min(65535, set.count - begin));
-            sketch_to_bf16_kernel<<<grid, 256, 0, st>>>(set.d_mats + begin, r, k_pad);
+            sketch_to_bf16_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats + begin, one, r, k_pad);
             launches.fetch_add(1, std::memory_order_relaxed);
         }
     }
-    if (!(set.k2_pair ? raise_smem_limit<decompress_pair_kernel>()
-                      : set.k2_bf16 ? raise_smem_limit<decompress_tc_kernel<true>>() : raise_smem_limit<decompress_tc_kernel<false>>()))
+    if (!(set.k2_pair ? raise_smem_limit<decompress_pair_kernel<SINGLE>>()
+                      : set.k2_bf16 ? raise_smem_limit<decompress_tc_kernel<SINGLE, true>>() : raise_smem_limit<decompress_tc_kernel<SINGLE, false>>()))
         return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k2_launch_begin.size(); ++l) {
         const int begin = set.k2_launch_begin[l], end = set.k2_launch_begin[l + 1];
@@ -1181,28 +1201,47 @@ inline flora_status tc_set_decompress(TcSet& set, const uint64_t* seeds, float s
             cfg.numAttrs = 2;
             const TcMatrix* mats = set.d_mats;
             const K2Item* items = set.d_k2 + begin;
-            if (cudaLaunchKernelEx(&cfg, decompress_pair_kernel, mats, items, end - begin, table, seed_base, r, scale, step, set.slots, set.cstages) !=
+            if (cudaLaunchKernelEx(&cfg, decompress_pair_kernel<SINGLE>, mats, one, items, end - begin, table, seed_base, r, scale, step, set.slots, set.cstages) !=
                 cudaSuccess)
                 return FLORA_ERR_CUDA;
         } else if (set.k2_bf16)
-            decompress_tc_kernel<true><<<grid, 32 * (K2_FIXED_WARPS + set.k2_gw), set.k2_smem, st>>>(
-                set.d_mats, set.d_k2 + begin, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw, set.k2_nslabs);
+            decompress_tc_kernel<SINGLE, true><<<grid, 32 * (K2_FIXED_WARPS + set.k2_gw), set.k2_smem, st>>>(
+                set.d_mats, one, set.d_k2 + begin, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw, set.k2_nslabs);
         else
-            decompress_tc_kernel<false><<<grid, 32 * (K2_FIXED_WARPS + set.k2_gw), set.k2_smem, st>>>(
-                set.d_mats, set.d_k2 + begin, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw, set.k2_nslabs);
+            decompress_tc_kernel<SINGLE, false><<<grid, 32 * (K2_FIXED_WARPS + set.k2_gw), set.k2_smem, st>>>(
+                set.d_mats, one, set.d_k2 + begin, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw, set.k2_nslabs);
         launches.fetch_add(1, std::memory_order_relaxed);
     }
     return cudaPeekAtLastError() == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
 
+inline flora_status tc_set_decompress(const TcSet& set, const uint64_t* seeds, float step, cudaStream_t st, std::atomic<uint64_t>& launches)
+{
+    return tc_decompress_launch<false>(set, TcMatrix{}, seeds, step, st, launches);
+}
+
 inline flora_status tc_decompress_single(flora_mat* W, const flora_mat* S, uint64_t seed, float step, cudaStream_t st,
                                          std::atomic<uint64_t>& launches)
 {
+    TcMatrix one;
+    if (!single_record(&one, *W, *S, false)) return FLORA_ERR_CUDA;
     std::lock_guard<std::mutex> lock(single_plan_mutex());
     flora_status rc;
     TcSet* set = single_plan(1, *W, *S, st, &rc);
     if (!set) return rc;
-    return set->decompress_ready ? tc_set_decompress(*set, &seed, step, st, launches) : FLORA_ERR_UNSUPPORTED;
+    if (!set->k2_bf16) return tc_decompress_launch<true>(*set, one, &seed, step, st, launches);
+    // ranks above 64: scratch for the bf16 copy of the sketch, for the duration of the call
+    const int64_t k_pad = (S->cols + 63) & ~(int64_t)63;
+    void* sb = nullptr;
+    if (scratch_alloc(&sb, (size_t)(S->rows * k_pad * 2), st) != cudaSuccess) {
+        cudaGetLastError();
+        return FLORA_ERR_ALLOC;
+    }
+    one.Sb = reinterpret_cast<__nv_bfloat16*>(sb);
+    rc = make_map(&one.map_sb, flora_mat{sb, S->rows, k_pad, k_pad, FLORA_BF16}) ? tc_decompress_launch<true>(*set, one, &seed, step, st, launches)
+                                                                                 : FLORA_ERR_CUDA;
+    if (cudaFreeAsync(sb, st) != cudaSuccess && rc == FLORA_OK) rc = FLORA_ERR_CUDA;
+    return rc;
 }
 
 inline bool tc_decompress_supported(const flora_mat* big, const flora_mat* sketch)
