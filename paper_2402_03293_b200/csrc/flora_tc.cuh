@@ -672,30 +672,35 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t wrow = w_ring + s * slot_bytes + row * 128;
-                uint32_t acc[4][16];
+                // two 16-column chunks at a time: with all four of a warp in registers the kernel spills (96 registers for
+                // its 640 threads), which costs more than the second round trip to tensor memory
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (k < mine) ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + (gt & 1) * bn + (c_begin + k) * 16, acc[k]);
-                ptx::tmem_ld_wait();
+                for (int k0 = 0; k0 < 4; k0 += 2) {
+                    uint32_t acc[2][16];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (k < mine) {
-                        const int c16 = c_begin + k;
-                        const uint32_t box = wrow + (c16 >> 2) * W_BOX_BYTES;
+                    for (int k = 0; k < 2; ++k)
+                        if (k0 + k < mine) ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + (gt & 1) * bn + (c_begin + k0 + k) * 16, acc[k]);
+                    ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint32_t addr = box + (((((c16 & 3) << 1) + h) ^ (row & 7)) << 4);
-                            uint32_t x[4];
-                            ptx::ld_shared_v4(addr, x[0], x[1], x[2], x[3]);
+                    for (int k = 0; k < 2; ++k) {
+                        if (k0 + k < mine) {
+                            const int c16 = c_begin + k0 + k;
+                            const uint32_t box = wrow + (c16 >> 2) * W_BOX_BYTES;
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const __nv_bfloat162 old = *reinterpret_cast<__nv_bfloat162*>(&x[u]);
-                                const float lo = fmaf(-step, __uint_as_float(acc[k][h * 8 + 2 * u]), __low2float(old));
-                                const float hi = fmaf(-step, __uint_as_float(acc[k][h * 8 + 2 * u + 1]), __high2float(old));
-                                __nv_bfloat162 nw = __floats2bfloat162_rn(lo, hi);
-                                x[u] = *reinterpret_cast<uint32_t*>(&nw);
+                            for (int h = 0; h < 2; ++h) {
+                                const uint32_t addr = box + (((((c16 & 3) << 1) + h) ^ (row & 7)) << 4);
+                                uint32_t x[4];
+                                ptx::ld_shared_v4(addr, x[0], x[1], x[2], x[3]);
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    const __nv_bfloat162 old = *reinterpret_cast<__nv_bfloat162*>(&x[u]);
+                                    const float lo = fmaf(-step, __uint_as_float(acc[k][h * 8 + 2 * u]), __low2float(old));
+                                    const float hi = fmaf(-step, __uint_as_float(acc[k][h * 8 + 2 * u + 1]), __high2float(old));
+                                    __nv_bfloat162 nw = __floats2bfloat162_rn(lo, hi);
+                                    x[u] = *reinterpret_cast<uint32_t*>(&nw);
+                                }
+                                ptx::st_shared_v4(addr, x[0], x[1], x[2], x[3]);
                             }
-                            ptx::st_shared_v4(addr, x[0], x[1], x[2], x[3]);
                         }
                     }
                 }
