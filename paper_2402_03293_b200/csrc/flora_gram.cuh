@@ -380,9 +380,6 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
                 const ApplyUnit* __restrict__ units, const int* __restrict__ slot_begin, const __grid_constant__ ApplySingle single, int per_cluster,
                 int r, float aa, float bb)
 {
-    // A kernel launched behind this one with the programmatic-serialization attribute may start now (the compression of
-    // a resampling step does: it streams G, which this kernel does not touch, and waits itself before it reads a sketch).
-    ptx::grid_launch_dependents();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     const int N = (r + 15) & ~15, n_half = N >> 1, kchunks = (r + 31) >> 5;
@@ -444,6 +441,10 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
 
+    // A kernel launched behind this one with the programmatic-serialization attribute may start now that every CTA has its
+    // tensor memory (the compression of a resampling step does: it streams G, which this kernel does not touch, and waits itself
+    // before it reads a sketch).
+    ptx::grid_launch_dependents();
     if (warp == 0) {
         // ------------------------------------------------------------------ src loads: this CTA's tile, chunk by chunk
         if (lane == 0) {

@@ -76,7 +76,6 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < PAIR_T * N) tmem_cols <<= 1;
 
-    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
         for (int s = 0; s < gstages; ++s) {
             ptx::mbar_init(ptx::smem_addr(&ctl->full_g[s]), 1);
@@ -110,6 +109,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     __syncthreads();
     ptx::cluster_sync();                    // every CTA's barriers exist before anyone arrives on them remotely
     ptx::tc_fence_after_sync();
+    ptx::grid_launch_dependents();          // (after the allocation of tensor memory, as in compress_tc_kernel)
     // everything above touched only shared and tensor memory; G and S may have been written by the previous kernel
     // of the stream.  `late_wait`: that kernel is this library's own pre-scaling of S, which does not touch G.
     if (!late_wait) ptx::grid_dependency_wait();

@@ -115,7 +115,6 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     K1Smem* ctl = reinterpret_cast<K1Smem*>(smem_raw + (a_ring - ptx::smem_addr(smem_raw)) + (size_t)astages * a_bytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    ptx::grid_launch_dependents();
     const K1Item item = items[blockIdx.x];                    // tables and descriptors are written at set creation, not by kernels
     const TcMatrix* mat = SINGLE ? &single : table + item.mat;
     uint32_t tmem_cols = 32;
@@ -154,6 +153,9 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     __syncthreads();
     if (S > 1) ptx::cluster_sync();       // every CTA's barriers exist before anyone arrives on them remotely
     ptx::tc_fence_after_sync();
+    // Only now: the next kernel's CTAs may take tensor memory and hold it while they wait for this kernel, so every CTA of this
+    // one must have its own before they start.
+    ptx::grid_launch_dependents();
     // everything above touched only this CTA's shared and tensor memory; G and S may have been written by the
     // previous kernel of the stream.  `late_wait`: that kernel is this library's own pre-scaling of S, which was
     // itself ordered after everything before it and does not touch G, so only the accesses to S need to wait
