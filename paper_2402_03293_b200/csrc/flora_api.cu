@@ -178,11 +178,13 @@ flora_status static_scratch_for_current_device(float** out)
 bool use_gen(const flora_mat* big) { return g_force_path.load(std::memory_order_relaxed) != 1 && gen_supported(*big); }
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 {
-    return g_force_path.load(std::memory_order_relaxed) != 1 && tune_knob("FLORA_GEN", 0, 0, 1) == 0 && tc_compress_supported(big, sketch);
+    return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch) && 
+           !gen_compress_quicker(big->rows * big->cols, big->cols, (int)sketch->cols);
 }
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
 {
-    return g_force_path.load(std::memory_order_relaxed) != 1 && tune_knob("FLORA_GEN", 0, 0, 1) == 0 && tc_decompress_supported(big, sketch);
+    return g_force_path.load(std::memory_order_relaxed) != 1 && tc_decompress_supported(big, sketch) && 
+           !gen_decompress_quicker(big->rows * big->cols, (int)sketch->cols);
 }
 
 }  // namespace
@@ -202,17 +204,21 @@ struct flora_set {
 // elements are 8 MB, a microsecond and a half of HBM time): all its matrices then go to the kernels of flora_gen.cuh.
 constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
 
-// Which matrices of one side (G or W) of a set the TMA kernels serve.
-static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S)
+// Which matrices of one side (G: compression, or W: decompression) of a set the TMA kernels serve.
+static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression)
 {
     std::vector<uint8_t> use = tc_eligible(big, S);
-    int64_t eligible = 0;
+    int64_t eligible = 0, widest = 0;
     bool mixed = false;
     for (size_t i = 0; i < big.size(); ++i) {
         if (use[i]) eligible += big[i].rows * big[i].cols;
         else mixed = mixed || big[i].rows > 0;
+        widest = std::max(widest, big[i].cols);
     }
-    if (mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) std::fill(use.begin(), use.end(), (uint8_t)0);
+    const int r = S.empty() ? 1 : (int)S[0].cols;
+    const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
+    if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) || (compression ? gen_compress_quicker(counted, widest, r) : gen_decompress_quicker(counted, r)))
+        std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
 }
 
@@ -224,7 +230,7 @@ static flora_status set_build(flora_set* s)
         gen_set_free(s->gen_g[d]);
         gen_set_free(s->gen_w[d]);
     }
-    const std::vector<uint8_t> use_g = set_tma_side(s->G, s->S), use_w = set_tma_side(s->W, s->S);
+    const std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true), use_w = set_tma_side(s->W, s->S, false);
     flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
         std::vector<int> g, w;

@@ -33,21 +33,27 @@ struct GenItem {           // compression: one cluster
     int32_t pad;
 };
 
-constexpr int GEN_WORKERS = 8;                              // warps that load, convert, generate and write out
-constexpr int GEN_THREADS = 32 * (GEN_WORKERS + 1);         // and one that issues the MMAs
-constexpr int GEN_STAGES_MAX = 4;
+// Warps that load, convert, generate and write out (8, or 16 where a CTA has an SM to itself), and one that issues the MMAs.
+__host__ __device__ constexpr int gen_threads(int workers) { return 32 * (workers + 1); }
+constexpr int GEN_G_SLOTS_MAX = 8, GEN_A_SLOTS_MAX = 4;
+constexpr int GEN_MAX_SPLIT = 16;                           // CTAs that share the columns of a row group (above 8: not a portable cluster size)
 
-// Parts of an fp32 value.
-struct Parts {
-    uint32_t h, m, l;      // fp32 bit patterns whose low 16 bits are zero
+// The parts of two fp32 values, as fp32 bit patterns whose low 16 bits are to be dropped.
+struct Parts2 {
+    uint32_t h0, h1, m0, m1, l0, l1;
 };
-__device__ __forceinline__ Parts split3(float x)
+__device__ __forceinline__ Parts2 split3(float x0, float x1)
 {
-    Parts p;
-    p.h = __float_as_uint(x) & 0xFFFF0000u;
-    const float r1 = __fsub_rn(x, __uint_as_float(p.h));                            // exact
-    p.m = __float_as_uint(r1) & 0xFFFF0000u;
-    p.l = __float_as_uint(__fsub_rn(r1, __uint_as_float(p.m)));                     // exact
+    Parts2 p;
+    p.h0 = __float_as_uint(x0);
+    p.h1 = __float_as_uint(x1);
+    float r0, r1, l0, l1;
+    unpack2(fma2(pack2(__uint_as_float(p.h0 & 0xFFFF0000u), __uint_as_float(p.h1 & 0xFFFF0000u)), FLORA_BOTH(0xBF800000) /* -1 */, pack2(x0, x1)), r0, r1);   // exact
+    p.m0 = __float_as_uint(r0);
+    p.m1 = __float_as_uint(r1);
+    unpack2(fma2(pack2(__uint_as_float(p.m0 & 0xFFFF0000u), __uint_as_float(p.m1 & 0xFFFF0000u)), FLORA_BOTH(0xBF800000) /* -1 */, pack2(r0, r1)), l0, l1);   // exact
+    p.l0 = __float_as_uint(l0);
+    p.l1 = __float_as_uint(l1);
     return p;
 }
 // Two bf16 values from the high halves of two fp32 bit patterns; `a` goes into the low half.
@@ -76,10 +82,10 @@ template <int PARTS>
 __device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, float x0, float x1, float x2, float x3)
 {
     if (PARTS == 3) {
-        const Parts p0 = split3(x0), p1 = split3(x1), p2 = split3(x2), p3 = split3(x3);
-        ptx::st_shared_v2(addr, pack_high(p0.h, p1.h), pack_high(p2.h, p3.h));
-        ptx::st_shared_v2(addr + part_bytes, pack_high(p0.m, p1.m), pack_high(p2.m, p3.m));
-        ptx::st_shared_v2(addr + 2 * part_bytes, pack_high(p0.l, p1.l), pack_high(p2.l, p3.l));
+        const Parts2 p = split3(x0, x1), q = split3(x2, x3);
+        ptx::st_shared_v2(addr, pack_high(p.h0, p.h1), pack_high(q.h0, q.h1));
+        ptx::st_shared_v2(addr + part_bytes, pack_high(p.m0, p.m1), pack_high(q.m0, q.m1));
+        ptx::st_shared_v2(addr + 2 * part_bytes, pack_high(p.l0, p.l1), pack_high(q.l0, q.l1));
     } else {
         ptx::st_shared_v2(addr, pack_bf16(x0, x1), pack_bf16(x2, x3));
     }
@@ -103,43 +109,41 @@ struct GenK1 {
     static constexpr int TILE = 128 * ROWB;                 // one part of a 128-row tile
 };
 struct GenSmem {
-    uint64_t full[GEN_STAGES_MAX], empty[GEN_STAGES_MAX], acc_full;
+    uint64_t full[GEN_G_SLOTS_MAX], empty[GEN_G_SLOTS_MAX], a_empty[GEN_A_SLOTS_MAX], acc_full;
     uint32_t tmem_base;
     int abort;
 };
-// The three parts of A side by side as one N operand (three MMAs per tile and K slice instead of six) while they fit.
-__host__ __device__ inline bool gen_side_by_side(bool f32, int r_pad) { return f32 && 3 * r_pad <= 256; }
-__host__ __device__ inline int gen_acc_cols(bool f32, int r_pad) { return gen_side_by_side(f32, r_pad) ? 3 * r_pad : r_pad; }
-inline size_t gen_k1_stage_bytes(bool f32, int r_pad, int T)
-{
-    return f32 ? (size_t)3 * 64 * (128 * T + r_pad) : (size_t)128 * (128 * T + r_pad);
-}
+// Shared memory: a ring of tiles of G (parts of 128 rows x K) and a ring of tiles of A (one per step, used by all its tiles).
+inline size_t gen_k1_g_bytes(bool f32) { return f32 ? (size_t)3 * 64 * 128 : (size_t)128 * 128; }
+inline size_t gen_k1_a_bytes(bool f32, int r_pad) { return f32 ? (size_t)3 * 64 * r_pad : (size_t)128 * r_pad; }
 // Row stride (in floats) of the staged accumulators: an odd multiple of 16 bytes, so that threads that own neighbouring
 // rows write to different banks.
 __host__ __device__ inline int gen_stage_stride(int r_pad) { return r_pad + 4; }
 
-// SINGLE: one matrix, passed by value; every cluster takes the next row groups of it.  (A template and not a test of `items`: the
-// choice between a table entry and a by-value parameter at run time was compiled into reads of the wrong one.)
-template <bool SINGLE, bool F32, bool ALIGNED>
-__global__ void __launch_bounds__(GEN_THREADS, 2)
+// SINGLE: one matrix, passed by value; every cluster takes the next row groups of it.  (A template and not a test of `items`: with
+// a run-time choice between the table's entry and the by-value one the kernel was seen to read the other one's address.)
+// sbs (fp32): the three parts of A side by side as one N operand (three MMAs per tile and K slice instead of six), their products
+// in three blocks of the accumulator, which are added up when they are read back.
+template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
+__global__ void __launch_bounds__(gen_threads(WORKERS), WORKERS == 8 ? 2 : 1)
 gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
-                    const __grid_constant__ GenMat single, int single_split, int seed_base, int r, float scale, float a, float b, int T, int stages,
-                    int cluster)
+                    const __grid_constant__ GenMat single, int single_split, int seed_base, int r, float scale, float a, float b, int T, int sbs,
+                    int g_slots, int a_slots, int cluster)
 {
     using C = GenK1<F32>;
+    constexpr int NT = 32 * WORKERS;                              // worker threads
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t* const ring = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     __shared__ GenSmem ctl;
     const int r_pad = (r + 15) & ~15;
-    const bool sbs = gen_side_by_side(F32, r_pad);
-    const int acc_cols = gen_acc_cols(F32, r_pad);
+    const int acc_cols = F32 && sbs ? 3 * r_pad : r_pad;
     const uint32_t a_part = (uint32_t)r_pad * C::ROWB;
-    const uint32_t g_bytes = (uint32_t)(T * C::PARTS) * C::TILE, stage_bytes = g_bytes + C::PARTS * a_part;
+    constexpr uint32_t G_BYTES = (uint32_t)C::PARTS * C::TILE;
+    const uint32_t a_bytes = C::PARTS * a_part, a_ring = smem_base + (uint32_t)g_slots * G_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
     const int rank = cluster > 1 ? (int)ptx::cluster_ctarank() : 0;
     const int cl = (int)blockIdx.x / cluster;
-    ptx::grid_launch_dependents();
     GenItem item;
     if (!SINGLE) {
         item = items[cl];
@@ -149,69 +153,73 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         item.tile0 = cl * (cluster / single_split) * T;
     }
     const GenMat mat = SINGLE ? single : mats[item.mat];
-    const int group = rank / item.split, part = rank % item.split;
+    const int split = item.split, group = rank / split, part = rank % split;
     const int tile0 = item.tile0 + group * T;
     const int tiles = max(0, min(T, ((mat.n + 127) >> 7) - tile0));
     const int all_steps = (mat.m + C::K - 1) / C::K;
-    const int ks0 = (int)((int64_t)part * all_steps / item.split), ks1 = (int)((int64_t)(part + 1) * all_steps / item.split);
+    const int ks0 = (int)((int64_t)part * all_steps / split), ks1 = (int)((int64_t)(part + 1) * all_steps / split);
     const int steps = tiles > 0 ? ks1 - ks0 : 0;
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < T * acc_cols) tmem_cols <<= 1;
 
     if (tid == 0) {
-        for (int s = 0; s < stages; ++s) {
-            ptx::mbar_init(ptx::smem_addr(&ctl.full[s]), GEN_WORKERS);
+        for (int s = 0; s < g_slots; ++s) {
+            ptx::mbar_init(ptx::smem_addr(&ctl.full[s]), WORKERS);
             ptx::mbar_init(ptx::smem_addr(&ctl.empty[s]), 1);
         }
+        for (int s = 0; s < a_slots; ++s) ptx::mbar_init(ptx::smem_addr(&ctl.a_empty[s]), 1);
         ptx::mbar_init(ptx::smem_addr(&ctl.acc_full), 1);
         ctl.abort = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
     }
-    if (warp == GEN_WORKERS) {
+    if (warp == WORKERS) {
         ptx::tmem_alloc(ptx::smem_addr(&ctl.tmem_base), tmem_cols);
         ptx::tmem_relinquish();
     }
     // rows r .. r_pad of every part of every A tile stay zero for the whole kernel
     if (r_pad > r)
-        for (int s = 0; s < stages; ++s)
+        for (int s = 0; s < a_slots; ++s)
             for (int p = 0; p < C::PARTS; ++p)
-                for (int t = tid; t < (r_pad - r) * (C::ROWB / 16); t += GEN_THREADS)
-                    ptx::st_shared_v4(smem_base + s * stage_bytes + g_bytes + p * a_part + (uint32_t)r * C::ROWB + t * 16u, 0, 0, 0, 0);
+                for (int t = tid; t < (r_pad - r) * (C::ROWB / 16); t += gen_threads(WORKERS))
+                    ptx::st_shared_v4(a_ring + s * a_bytes + p * a_part + (uint32_t)r * C::ROWB + t * 16u, 0, 0, 0, 0);
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
+    // (only now: the next kernel's CTAs may take tensor memory and hold it while they wait for this kernel, so every CTA of this one
+    // must have its own before they start)
+    ptx::grid_launch_dependents();
     const uint32_t tmem = ctl.tmem_base;
     volatile int* abort = &ctl.abort;
 
-    if (warp == GEN_WORKERS) {
+    if (warp == WORKERS) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0 && steps > 0) {
-            RingPos p;
+            RingPos pg, pa;
             bool ok = true;
-            for (int ks = 0; ks < steps; ++ks, p.advance(stages)) {
-                ok = ptx::mbar_wait(ptx::smem_addr(&ctl.full[p.s]), p.wraps & 1u, abort);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const uint32_t st = smem_base + p.s * stage_bytes;
-                const uint64_t da = operand_desc<C::ROWB>(st + g_bytes);
-                for (int t = 0; t < tiles; ++t) {
-                    const uint64_t dg = operand_desc<C::ROWB>(st + (uint32_t)(t * C::PARTS) * C::TILE);
+            for (int ks = 0; ks < steps && ok; ++ks, pa.advance(a_slots)) {
+                const uint64_t da = operand_desc<C::ROWB>(a_ring + pa.s * a_bytes);
+                for (int t = 0; t < tiles; ++t, pg.advance(g_slots)) {
+                    // (the warps that filled a tile had written their share of the step's A before)
+                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl.full[pg.s]), pg.wraps & 1u, abort);
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+                    const uint64_t dg = operand_desc<C::ROWB>(smem_base + pg.s * G_BYTES);
                     const uint32_t acc = tmem + (uint32_t)(t * acc_cols);
 #pragma unroll
                     for (int kk = 0; kk < C::K / 16; ++kk) {
                         const uint32_t on = (ks | kk) != 0;
+                        const uint64_t ap = (uint64_t)(a_part >> 4);
+                        constexpr uint64_t gp = C::TILE >> 4;
+                        const uint32_t id = ptx::umma_idesc_bf16((uint32_t)r_pad);
                         if (!F32) {
-                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, ptx::umma_idesc_bf16((uint32_t)r_pad), on);
+                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, id, on);
                         } else if (sbs) {
-                            // the blocks of the accumulator (one per part of A) are added up when they are read back
                             ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(3u * r_pad), on);
-                            ptx::umma_bf16(acc, dg + (C::TILE >> 4) + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(2u * r_pad), 1u);
-                            ptx::umma_bf16(acc, dg + (2 * C::TILE >> 4) + kk * 2, da + kk * 2, ptx::umma_idesc_bf16((uint32_t)r_pad), 1u);
+                            ptx::umma_bf16(acc, dg + gp + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(2u * r_pad), 1u);
+                            ptx::umma_bf16(acc, dg + 2 * gp + kk * 2, da + kk * 2, id, 1u);
                         } else {
-                            const uint32_t id = ptx::umma_idesc_bf16((uint32_t)r_pad);
-                            const uint64_t ap = (uint64_t)(a_part >> 4), gp = (uint64_t)(C::TILE >> 4);
                             ptx::umma_bf16(acc, dg + 2 * gp + kk * 2, da + kk * 2, id, on);                // l h
                             ptx::umma_bf16(acc, dg + kk * 2, da + 2 * ap + kk * 2, id, 1u);                // h l
                             ptx::umma_bf16(acc, dg + gp + kk * 2, da + ap + kk * 2, id, 1u);               // m m
@@ -220,42 +228,43 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                             ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, id, 1u);                         // h h
                         }
                     }
+                    ptx::umma_commit(ptx::smem_addr(&ctl.empty[pg.s]));
                 }
-                ptx::umma_commit(ptx::smem_addr(&ctl.empty[p.s]));
+                if (ok) ptx::umma_commit(ptx::smem_addr(&ctl.a_empty[pa.s]));
             }
             if (ok) ptx::umma_commit(ptx::smem_addr(&ctl.acc_full));
         }
     } else {
         // ------------------------------------------------------------------ workers
-        // A step of a tile is 128 rows of eight 16-byte pieces; thread tid takes piece tid % 8 of the rows tid / 8 + 32 i.
+        // A step of a tile is 128 rows of eight 16-byte pieces; thread tid takes piece tid % 8 of the rows tid / 8 + RS i.
         // What bounds a step is issue slots (16 KB of G take about 700 cycles of an SM's share of HBM), so the loop carries
         // one pointer and tests one row count.  A piece that starts off a 16-byte boundary comes as the two aligned blocks it
         // touches; a block is read whole as soon as one byte of it is wanted (it lies in one page with that byte).
+        constexpr int RS = 4 * WORKERS, NI = 128 / RS;              // rows that the warps cover at a time; pieces per thread
+        constexpr int AHEAD = 8 / NI;                               // tiles under way in registers (32 KB of a CTA's G, or 64)
         const int piece = tid & 7, row_in = tid >> 3;
         constexpr int ES = F32 ? 4 : 2, E = 16 / ES;                // element size, elements per piece
         constexpr int BLK = ALIGNED ? 1 : 2;                        // 16-byte blocks per piece
         const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
         bool ok = true;
-        const int64_t row_step = 32 * mat.ld * ES;                  // bytes between a thread's rows
-        const int rows_left = mat.n - tile0 * 128 - row_in;         // row t * 128 + 32 i of this thread exists if it is below this
+        const int64_t row_step = RS * mat.ld * ES;                  // bytes between a thread's rows
+        const int rows_left = mat.n - tile0 * 128 - row_in;         // row t * 128 + RS i of this thread exists if it is below this
         const uint8_t* fp = reinterpret_cast<const uint8_t*>(mat.big) + ((int64_t)(tile0 * 128 + row_in) * mat.ld + (int64_t)ks0 * C::K + piece * E) * ES;
         const uint32_t low0 = (uint32_t)reinterpret_cast<uintptr_t>(fp), low_step = (uint32_t)row_step;      // for the pieces' alignment
         const uint8_t* fstep = fp;                                  // fetch cursor: this thread's piece of row 0 of the tile; of tile 0 of the step
         int fks = 0, ft = 0, pks = 0, pt = 0;                       // fetch and place cursors: step, tile
         auto left_at = [&](int ks) { return mat.m - ((ks0 + ks) * C::K + piece * E); };      // elements from this thread's piece on
-        auto fetch = [&](uint4 (&x)[4][BLK]) {                      // the four pieces of this thread of the tile at the fetch cursor
+        auto fetch = [&](uint4 (&x)[NI][BLK]) {                     // the pieces of this thread of the tile at the fetch cursor
             const int bytes = min(16, left_at(fks) * ES);
             const uint8_t* p = fp;
 #pragma unroll
-            for (int i = 0; i < 4; ++i, p += row_step) {
-                const bool in = ft * 128 + 32 * i < rows_left && bytes > 0;
-                const uint8_t* const p16 = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)15);
-                x[i][0] = make_uint4(0, 0, 0, 0);
-                if (in) x[i][0] = *reinterpret_cast<const uint4*>(p16);
-                if (!ALIGNED) {
-                    x[i][BLK - 1] = make_uint4(0, 0, 0, 0);
-                    if (in && (int)(p - p16) + bytes > 16) x[i][BLK - 1] = *reinterpret_cast<const uint4*>(p16 + 16);
-                }
+            for (int i = 0; i < NI; ++i, p += row_step) {
+                // (where there is nothing to fetch the registers keep what they held: rows beyond n are never written out, and
+                // columns beyond m are masked when they are placed)
+                const bool in = ft * 128 + RS * i < rows_left && bytes > 0;
+                const uint8_t* const p16 = ALIGNED ? p : reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)15);
+                ptx::ld_stream_v4(x[i][0], p16, in);
+                if (!ALIGNED) ptx::ld_stream_v4(x[i][BLK - 1], p16 + 16, in && (int)(p - p16) + bytes > 16);
             }
             if (++ft == tiles) {
                 ft = 0;
@@ -263,21 +272,21 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 fstep += 128;
                 fp = fstep;
             } else {
-                fp += 4 * row_step;
+                fp += NI * row_step;
             }
         };
         const uint32_t my_off = F32 ? (uint32_t)((piece & 1) * 8) : 0u;
-        auto place = [&](const uint4 (&x)[4][BLK], uint32_t st) {   // ... of the tile at the place cursor, as operand rows of stage st
-            const uint32_t tile = st + (uint32_t)(pt * C::PARTS) * C::TILE + my_off;
+        auto place = [&](const uint4 (&x)[NI][BLK], uint32_t slot) { // ... of the tile at the place cursor, as operand rows of a slot
+            const uint32_t tile = slot + my_off;
             const int left = left_at(pks);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int lr = row_in + 32 * i;
+            for (int i = 0; i < NI; ++i) {
+                const int lr = row_in + RS * i;
                 uint32_t w[4] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w};
                 if (!ALIGNED) {
                     const uint4 y = x[i][BLK - 1];
                     const uint32_t v[8] = {w[0], w[1], w[2], w[3], y.x, y.y, y.z, y.w};
-                    const uint32_t off = low0 + (uint32_t)(pt * 4 + i) * low_step;
+                    const uint32_t off = low0 + (uint32_t)(pt * NI + i) * low_step;
                     uint32_t s1[7], s2[5];
 #pragma unroll
                     for (int k = 0; k < 7; ++k) s1[k] = (off & 4) ? v[k + 1] : v[k];
@@ -309,10 +318,10 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
             int t = first;
             auto put = [&](int t, const float (&v)[4]) {
                 const int j = t / QPR, q = t % QPR;
-                store_quad<C::PARTS>(st + g_bytes + operand_offset<C::ROWB>(j, q >> 1) + (q & 1) * 8, a_part, v[0], v[1], v[2], v[3]);
+                store_quad<C::PARTS>(st + operand_offset<C::ROWB>(j, q >> 1) + (q & 1) * 8, a_part, v[0], v[1], v[2], v[3]);
             };
-            for (; t + 32 * GEN_WORKERS < tasks; t += 64 * GEN_WORKERS) {
-                const int u = t + 32 * GEN_WORKERS;
+            for (; t + NT < tasks; t += 2 * NT) {
+                const int u = t + NT;
                 float v[4], w[4];
                 projection_two_quads(q0 + t % QPR, (uint32_t)(t / QPR), q0 + u % QPR, (uint32_t)(u / QPR), key, scale, v, w);
                 put(t, v);
@@ -322,56 +331,72 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 float v[4];
                 projection_quad(q0 + t % QPR, (uint32_t)(t / QPR), key, scale, v);
                 put(t, v);
-                t += 32 * GEN_WORKERS;
+                t += NT;
             }
             first = t - tasks;
         };
         const int total = steps * tiles;
-        uint4 x0[4][BLK], x1[4][BLK];
-        // the first tile of A touches nothing that another kernel writes
-        if (steps > 0) generate(0, smem_base);
+        uint4 x[AHEAD][NI][BLK];
+#pragma unroll
+        for (int d = 0; d < AHEAD; ++d)
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+#pragma unroll
+                for (int k = 0; k < BLK; ++k) x[d][i][k] = make_uint4(0, 0, 0, 0);
+        // Tiles of A are made `lead` steps before they are used.  The first touches nothing that another kernel writes; the next
+        // ones are made while the first loads travel.
+        const int lead = a_slots - 2;
+        RingPos pa;                                                 // of the next tile to make
+        int made = 0;
+        auto make = [&]() {
+            generate(made, a_ring + pa.s * a_bytes);
+            ++made;
+            pa.advance(a_slots);
+        };
+        if (steps > 0) make();
         ptx::grid_dependency_wait();
-        if (total > 0) fetch(x0);
-        if (total > 1) fetch(x1);
-        RingPos p;
-        auto turn = [&](bool more, uint4 (&x)[4][BLK]) {
-            const uint32_t st = smem_base + p.s * stage_bytes;
-            if (pt == 0 && pks > 0) {
-                ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl.empty[p.s]), (p.wraps & 1u) ^ 1u, abort);
-                if (ok) generate(pks, st);
+#pragma unroll
+        for (int d = 0; d < AHEAD; ++d)
+            if (d < total) fetch(x[d]);
+        while (made < min(lead + 1, steps)) make();
+        RingPos pg;
+        auto turn = [&](bool more, uint4 (&x)[NI][BLK]) {
+            if (pt == 0 && pks > 0 && made < steps) {
+                ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl.a_empty[pa.s]), (pa.wraps & 1u) ^ 1u, abort);
+                if (ok) make();
             }
+            ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl.empty[pg.s]), (pg.wraps & 1u) ^ 1u, abort);
             if (!ok) return;
-            place(x, st);
+            place(x, smem_base + pg.s * G_BYTES);
             if (more) fetch(x);
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl.full[pg.s]));
+            pg.advance(g_slots);
             if (++pt == tiles) {
                 pt = 0;
                 ++pks;
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl.full[p.s]));
-                p.advance(stages);
             }
         };
-        for (int u = 0; u < total && ok; u += 2) {
-            turn(u + 2 < total, x0);
-            if (u + 1 < total) turn(u + 3 < total, x1);
+        for (int u = 0; u < total && ok; u += AHEAD) {
+#pragma unroll
+            for (int d = 0; d < AHEAD; ++d)
+                if (u + d < total) turn(u + d + AHEAD < total, x[d]);
         }
-        if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
-        ptx::tc_fence_after_sync();
         // ------------------------------------------------------------------ write-out
-        // Accumulators -> shared memory (the operand ring, free by now), one row of a tile per thread.  The other CTAs of a
+        // Accumulators -> shared memory (the operand rings, free by now), one row of a tile per thread.  The other CTAs of a
         // split add their sums before anything is written to the sketch, whose rows are then written by whole warps.
         float* const stage = reinterpret_cast<float*>(ring);
         const int stride = gen_stage_stride(r_pad);
         auto stage_tile = [&](int t, float* to) {
             const int row = (warp & 3) * 32 + lane;
             __syncwarp();
-            for (int c = (warp >> 2) * 16; c < r_pad; c += 32) {
+            for (int c = (warp >> 2) * 16; c < r_pad; c += 4 * WORKERS) {
                 uint32_t v[16];
                 if (steps > 0) {
                     const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(t * acc_cols + c);
                     ptx::tmem_ld_16(at, v);
-                    if (sbs) {
+                    if (F32 && sbs) {
                         uint32_t v1[16], v2[16];
                         ptx::tmem_ld_16(at + r_pad, v1);
                         ptx::tmem_ld_16(at + 2 * r_pad, v2);
@@ -392,45 +417,62 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                         make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]), __uint_as_float(v[k + 3]));
             }
         };
-        // rows [lr0, lr1) of the staged tiles (tile `t_first` on) -> sketch; `value(i, j)`: the finished sum
+        // Rows [lr0, lr1) of the CTA's tiles -> sketch; value(i, j): the finished sum.  The first values of the old sketch that a
+        // thread needs are fetched by `fetch_old`, before the sums are there.
+        constexpr int NOLD = 2;
         const bool vec = (r & 3) == 0 && (mat.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(mat.S) & 15) == 0;
-        auto write_rows = [&](int lr0, int lr1, int grow0, auto value4, auto value1) {
-            if (vec) {
-                const int per = r >> 2;                                      // pieces per row
-                const int total4 = (lr1 - lr0) * per;
-#pragma unroll 4
-                for (int e = tid; e < total4; e += 32 * GEN_WORKERS) {
-                    const int i = e / per, j = (e - i * per) * 4, lr = lr0 + i;
-                    if (grow0 + lr >= mat.n) break;
-                    float4 v = value4(lr, j);
-                    float4* dst = reinterpret_cast<float4*>(mat.S + (int64_t)(grow0 + lr) * mat.lds + j);
-                    v = make_float4(a * v.x, a * v.y, a * v.z, a * v.w);
-                    if (b != 0.0f) {                                         // b == 0 must not propagate whatever the state held before
-                        const float4 o = *dst;
-                        v = make_float4(fmaf(b, o.x, v.x), fmaf(b, o.y, v.y), fmaf(b, o.z, v.z), fmaf(b, o.w, v.w));
-                    }
-                    *dst = v;
-                }
-            } else {
-                const int total1 = (lr1 - lr0) * r;
-#pragma unroll 4
-                for (int e = tid; e < total1; e += 32 * GEN_WORKERS) {
-                    const int i = e / r, j = e - i * r, lr = lr0 + i;
-                    if (grow0 + lr >= mat.n) break;
-                    float* dst = mat.S + (int64_t)(grow0 + lr) * mat.lds + j;
-                    const float v = a * value1(lr, j);
-                    *dst = b != 0.0f ? fmaf(b, *dst, v) : v;
-                }
+        const int per = vec ? r >> 2 : r;                                    // pieces per row
+        float4 old[NOLD];
+        auto old_at = [&](int e, int lr0, int grow0) {
+            const int i = e / per, j = e - i * per;
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (grow0 + lr0 + i < mat.n) {
+                const float* src = mat.S + (int64_t)(grow0 + lr0 + i) * mat.lds;
+                if (vec) o = *reinterpret_cast<const float4*>(src + 4 * j);
+                else o.x = src[j];
+            }
+            return o;
+        };
+        auto fetch_old = [&](int lr0, int lr1, int grow0) {
+#pragma unroll
+            for (int k = 0; k < NOLD; ++k) {
+                old[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (b != 0.0f && tid + k * NT < (lr1 - lr0) * per) old[k] = old_at(tid + k * NT, lr0, grow0);
             }
         };
-        if (item.split == 1) {
+        auto write_rows = [&](int lr0, int lr1, int grow0, auto value) {
+            auto put = [&](int e, float4 o) {
+                const int i = e / per, j = e - i * per;
+                if (grow0 + lr0 + i >= mat.n) return;
+                float* dst = mat.S + (int64_t)(grow0 + lr0 + i) * mat.lds;
+                float4 v = value(lr0 + i, vec ? 4 * j : j);
+                v = make_float4(a * v.x, a * v.y, a * v.z, a * v.w);
+                if (b != 0.0f) v = make_float4(fmaf(b, o.x, v.x), fmaf(b, o.y, v.y), fmaf(b, o.z, v.z), fmaf(b, o.w, v.w));
+                if (vec) *reinterpret_cast<float4*>(dst + 4 * j) = v;        // (b == 0 must not propagate whatever the state held before)
+                else dst[j] = v.x;
+            };
+            const int total_e = (lr1 - lr0) * per;
+#pragma unroll
+            for (int k = 0; k < NOLD; ++k)
+                if (tid + k * NT < total_e) put(tid + k * NT, old[k]);
+#pragma unroll 4
+            for (int e = tid + NOLD * NT; e < total_e; e += NT) put(e, b != 0.0f ? old_at(e, lr0, grow0) : make_float4(0.f, 0.f, 0.f, 0.f));
+        };
+        const int rows = tiles * 128, lr0 = part * rows / split, lr1 = (part + 1) * rows / split;
+        if (split > 1) fetch_old(lr0, lr1, tile0 * 128);
+        if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
+        ptx::tc_fence_after_sync();
+        if (split == 1) {
             for (int t = 0; t < tiles; ++t) {
-                if (t > 0) ptx::named_barrier_sync(1, 32 * GEN_WORKERS);
+                fetch_old(0, 128, (tile0 + t) * 128);
+                if (t > 0) ptx::named_barrier_sync(1, NT);
                 stage_tile(t, stage);
-                ptx::named_barrier_sync(1, 32 * GEN_WORKERS);
+                ptx::named_barrier_sync(1, NT);
                 if (!*abort)
-                    write_rows(0, 128, (tile0 + t) * 128, [&](int i, int j) { return *reinterpret_cast<const float4*>(stage + i * stride + j); },
-                               [&](int i, int j) { return stage[i * stride + j]; });
+                    write_rows(0, 128, (tile0 + t) * 128, [&](int i, int j) {
+                        const float* p = stage + i * stride + j;
+                        return vec ? *reinterpret_cast<const float4*>(p) : make_float4(*p, 0.f, 0.f, 0.f);
+                    });
             }
             if (cluster > 1) {
                 ptx::cluster_sync_some();
@@ -439,36 +481,30 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         } else {
             for (int t = 0; t < tiles; ++t) stage_tile(t, stage + t * 128 * stride);
             ptx::cluster_sync_some();                                        // every partial sum of the cluster is staged
-            const int rows = tiles * 128, lr0 = part * rows / item.split, lr1 = (part + 1) * rows / item.split;
             const uint32_t sbase = ptx::smem_addr(stage);
-            const int split = item.split, first_rank = group * split;
+            const int first_rank = group * split;
             if (!*abort)
-                write_rows(lr0, lr1, tile0 * 128,
-                           [&](int i, int j) {
-                               float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                               for (int q = 0; q < split; ++q) {
-                                   const float4 w = ptx::ld_cluster_v4(ptx::map_to_cta(sbase + (uint32_t)(i * stride + j) * 4u, (uint32_t)(first_rank + q)));
-                                   v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
-                               }
-                               return v;
-                           },
-                           [&](int i, int j) {
-                               float v = 0.f;
-                               for (int q = 0; q < split; ++q)
-                                   v += ptx::ld_cluster_f32(ptx::map_to_cta(sbase + (uint32_t)(i * stride + j) * 4u, (uint32_t)(first_rank + q)));
-                               return v;
-                           });
+                write_rows(lr0, lr1, tile0 * 128, [&](int i, int j) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const uint32_t at = sbase + (uint32_t)(i * stride + j) * 4u;
+                    for (int q = 0; q < split; ++q) {
+                        const uint32_t p = ptx::map_to_cta(at, (uint32_t)(first_rank + q));
+                        const float4 w = vec ? ptx::ld_cluster_v4(p) : make_float4(ptx::ld_cluster_f32(p), 0.f, 0.f, 0.f);
+                        v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+                    }
+                    return v;
+                });
             ptx::cluster_sync_some();                                        // nobody leaves while a peer may still read its sums
         }
     }
-    if (warp == GEN_WORKERS && cluster > 1) {
+    if (warp == WORKERS && cluster > 1) {
         __syncwarp();
         ptx::cluster_sync_some();
         ptx::cluster_sync_some();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if (warp == GEN_WORKERS) {
+    if (warp == WORKERS) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem, tmem_cols);
     }
@@ -515,7 +551,6 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
     float* const staging = reinterpret_cast<float*>(smem_raw + (sop - ptx::smem_addr(smem_raw)));
     constexpr int STRIDE = BN + 4;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    ptx::grid_launch_dependents();
     // this CTA's share: pieces of slabs (one matrix: units u .. u_end of the slab-major order)
     int it = 0, it_end = 0, u = 0, u_end = 0, rt = 1;
     if (SINGLE) {
@@ -541,6 +576,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
+    ptx::grid_launch_dependents();                                // (after the allocation, as in the compression)
     const uint32_t tmem = ctl.tmem_base;
     volatile int* abort = &ctl.abort;
     constexpr int ES = F32 ? 4 : 2, E = 16 / ES;                  // element size, elements per 16-byte piece

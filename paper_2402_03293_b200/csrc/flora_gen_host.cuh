@@ -1,5 +1,7 @@
 // Host side of the kernels in flora_gen.cuh: tile shapes, work lists of sets, launches.
 #pragma once
+#include <math.h>
+
 #include <algorithm>
 #include <atomic>
 #include <vector>
@@ -11,7 +13,8 @@ namespace flora {
 
 // Launch shape of the compression for a list of matrices.
 struct GenK1Plan {
-    int T = 1, stages = 2, cluster = 1, per_sm = 1;
+    int T = 1, g_slots = 3, a_slots = 2, cluster = 1, per_sm = 1, workers = 8;
+    bool sbs = false;
     size_t smem = 0;
     bool aligned = true;
 };
@@ -22,67 +25,111 @@ inline bool gen_aligned(const flora_mat& g)
     return ((reinterpret_cast<uintptr_t>(g.data) | (uintptr_t)(g.ld * es)) & 15) == 0;
 }
 
-// CTAs of one SM: two where operand rings of two stages and the accumulators of both fit.
-inline void gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split)
+// Rings, accumulator layout and CTAs per SM for T tiles per CTA; false where they do not fit.  `per_sm` = 2: two CTAs with at
+// most 112 KB and 256 accumulator columns each.  At least three slots of G and two of A (with fewer the warps wait for the MMAs of
+// the step before: fp32 4096 x 11008 at r = 8 ran at half the speed).
+inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int per_sm)
 {
-    const int r_pad = (r + 15) & ~15, acc = gen_acc_cols(f32, r_pad);
-    uint32_t cols = 32;
-    while ((int)cols < T * acc) cols <<= 1;
-    const size_t stage = gen_k1_stage_bytes(f32, r_pad, T);
+    const int r_pad = (r + 15) & ~15, most_cols = per_sm == 2 ? 256 : 512;
+    p.sbs = f32 && 3 * r_pad <= 256 && T * 3 * r_pad <= most_cols;
+    const int cols_used = T * (p.sbs ? 3 * r_pad : r_pad);
+    if (cols_used > most_cols) return false;
+    const size_t budget = (per_sm == 2 ? 112 * 1024 : SMEM_BUDGET) - 1024;
+    const size_t g = gen_k1_g_bytes(f32), a = gen_k1_a_bytes(f32, r_pad);
     const size_t staged = (size_t)(split ? T : 1) * 128 * gen_stage_stride(r_pad) * 4;
-    const size_t half = 112 * 1024;                                       // two CTAs with their static parts share 227 KB
-    const bool two = cols <= 256 && 2 * stage + 1024 <= half && staged + 1024 <= half;
-    const size_t budget = (two ? half : SMEM_BUDGET) - 1024;
+    if (3 * g + 2 * a > budget || staged > budget) return false;
     p.T = T;
-    p.stages = (int)std::max<size_t>(1, std::min<size_t>(GEN_STAGES_MAX, budget / stage));
-    p.smem = std::max(p.stages * stage, staged) + 1024;
+    p.per_sm = per_sm;
+    p.a_slots = budget >= 4 * g + 3 * a ? 3 : 2;
+    p.g_slots = (int)std::min<size_t>(GEN_G_SLOTS_MAX, (budget - p.a_slots * a) / g);
+    p.smem = std::max(p.g_slots * g + p.a_slots * a, staged) + 1024;
     // no more CTAs on an SM than its tensor memory serves: the CTAs of a cluster wait for one another, so none may wait for columns
+    uint32_t cols = 32;
+    while ((int)cols < cols_used) cols <<= 1;
     const int most = (int)(512 / cols);
     while (most < 8 && (size_t)(most + 1) * (p.smem + 1024) <= 227 * 1024) p.smem += 1024;
-    p.per_sm = two ? 2 : 1;
+    return true;
 }
-inline bool gen_k1_fits(bool f32, int r, int T, bool split)
+// Cost model of the compression (cycles of one SM).  A step of T tiles takes its share of HBM (16 KB a tile, 700 cycles) or the
+// issue slots of generating and converting it, whichever is longer, and no less than the latency of one warp's part of it
+// (about 2100 cycles a tile with eight warps, 1500 with sixteen: measured); a CTA costs about two microseconds before its first
+// and after its last step, more with sixteen warps, and a little more when it adds up with others.
+inline double gen_k1_cost(bool f32, int r, int T, int workers, double together, int64_t waves, int64_t steps, int split)
 {
-    const int r_pad = (r + 15) & ~15;
-    const size_t staged = (size_t)(split ? T : 1) * 128 * gen_stage_stride(r_pad) * 4;
-    return T * gen_acc_cols(f32, r_pad) <= 512 && 2 * gen_k1_stage_bytes(f32, r_pad, T) + 1024 <= SMEM_BUDGET && staged + 1024 <= SMEM_BUDGET;
+    const int K = f32 ? 32 : 64;
+    const double issue = 0.5 * r * K + (f32 ? 900.0 : 600.0) * T;
+    const double quads = ceil((double)r * K / 4 / (32.0 * workers)), latency = (workers == 16 ? 1500.0 : 2100.0) * T + 330.0 * quads;
+    const double step = std::max(latency, std::max(1.0, together) * std::max(700.0 * T, issue));
+    return (double)waves * (4000.0 + (workers == 16 ? 2000.0 : 0.0) + (split > 1 ? 1000.0 + 50.0 * split : 0.0) + (double)steps * step);
 }
-// Tiles per CTA: the smallest count whose loads outlast the generation of A (one tile's 16 KB take about 700 cycles of an
-// SM's share of HBM; the r x K values of a step 54 issue slots each on 128 lanes), as far as memory goes.
-inline int gen_k1_tiles(bool f32, int r, int64_t max_tiles)
+// Clusters of `size` CTAs of the compression kernel that can be resident (asked once per kind of launch: the kernel's variants
+// need the same registers, so one stands for all).
+inline int gen_k1_resident(const GenK1Plan& p, int size)
 {
-    const double gen = (double)r * (f32 ? 32 : 64) * 54 / 128;
-    int T = 1;
-    while (T < 4 && gen > 0.5 * 700 * T && max_tiles >= 2 * T && gen_k1_fits(f32, r, 2 * T, false)) T *= 2;
-    return T;
+    if (size == 1) return sm_count() * p.per_sm;
+    struct Known { int dev, workers, size, clusters; size_t smem; };
+    static std::mutex mutex;
+    static std::vector<Known> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mutex);
+    for (const Known& k : known)
+        if (k.dev == dev && k.workers == p.workers && k.size == size && k.smem == p.smem) return k.clusters;
+    const int n = p.workers == 16 ? resident_clusters<gen_compress_kernel<true, true, false, 16>>(size, gen_threads(16), p.smem, true)
+                                  : resident_clusters<gen_compress_kernel<true, true, false, 8>>(size, gen_threads(8), p.smem, true);
+    known.push_back({dev, p.workers, size, n, p.smem});
+    return n;
 }
-// Cost model of the compression (cycles of one SM): a step of T tiles takes its share of HBM (16 KB a tile, 700 cycles) or the
-// issue slots of generating and converting it, whichever is longer, and no less than the latency of one step; a CTA costs
-// about two microseconds before its first and after its last step, a little more when it adds up with others.
-inline double gen_k1_cost(bool f32, int r, int T, int per_sm, int64_t ctas, int64_t steps, int split)
+// Tile shape and split with the shortest schedule.  Chosen once per shape and kept (64 of them).
+inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
 {
-    const double gen = (double)r * (f32 ? 32 : 64) * 54 / 128, issue = gen + (f32 ? 300.0 : 150.0) * T;
-    const double waves = (double)((ctas + (int64_t)per_sm * sm_count() - 1) / ((int64_t)per_sm * sm_count()));
-    const double together = std::min<double>(per_sm, (double)ctas / sm_count());
-    const double step = std::max(1000.0 + 1.5 * gen, std::max(1.0, together) * std::max(700.0 * T, issue));
-    return waves * (4000.0 + (split > 1 ? 1500.0 : 0.0) + (double)steps * step);
-}
-// CTAs that share the columns of one row group, so that `groups` of them fill the GPU; every CTA keeps at least two steps.
-inline int gen_k1_split(int64_t groups, int64_t steps, int64_t want)
-{
-    int split = 1;
-    while (split < 8 && groups * split * 2 <= want && steps >= 4 * split) split *= 2;
-    return split;
+    struct Known { int dev, r; bool f32; int64_t tiles, steps; GenK1Plan plan; };
+    static std::mutex mutex;
+    static std::vector<Known> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mutex);
+    if (tune_knob("FLORA_GEN_T", 0, 0, 4)) known.clear();        // (a sweep over shapes)
+    for (const Known& k : known)
+        if (k.dev == dev && k.r == r && k.f32 == f32 && k.tiles == tiles && k.steps == steps) return k.plan;
+    GenK1Plan best;
+    double least = 1e300;
+    for (int T = 1; T <= 4; T *= 2)
+        for (int split = 1; split <= GEN_MAX_SPLIT; ++split)
+            for (int workers = 8; workers <= 16; workers += 8) {
+                if ((T > 1 && tiles < T) || (split > 1 && steps < split)) continue;
+                if (tune_knob("FLORA_GEN_T", T, 1, 4) != T || tune_knob("FLORA_GEN_SPLIT", split, 1, 16) != split ||
+                    tune_knob("FLORA_GEN_WORKERS", workers, 8, 16) != workers)
+                    continue;
+                GenK1Plan p;
+                if (!gen_k1_shape(p, f32, r, T, split > 1, workers == 16 ? 1 : 2)) continue;    // (registers: one CTA of sixteen warps)
+                p.cluster = split;
+                p.workers = workers;
+                const int64_t clusters = (tiles + T - 1) / T, resident = gen_k1_resident(p, split);
+                const double together = std::min<double>(p.per_sm, (double)(std::min(clusters, resident) * split) / sm_count());
+                const double cost = gen_k1_cost(f32, r, T, workers, together, (clusters + resident - 1) / resident, (steps + split - 1) / split, split);
+                if (cost < least * 0.98) {
+                    least = cost;
+                    best = p;
+                }
+            }
+    if (least > 1e299) {                                          // (one tile, no split, one CTA per SM fits every rank)
+        gen_k1_shape(best, f32, r, 1, false, 1);
+        best.workers = 16;
+    }
+    if (known.size() >= 64) known.erase(known.begin());
+    known.push_back({dev, r, f32, tiles, steps, best});
+    return best;
 }
 
-template <bool SINGLE, bool F32, bool ALIGNED>
+template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds, const GenMat& one,
                                  int split, int seed_base, int r, float a, float b, cudaStream_t st)
 {
-    if (!raise_smem_limit<gen_compress_kernel<SINGLE, F32, ALIGNED>>()) return cudaErrorInvalidValue;
+    if (!raise_smem_limit<gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>>(true)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * p.cluster));
-    cfg.blockDim = dim3((unsigned)GEN_THREADS);
+    cfg.blockDim = dim3((unsigned)gen_threads(WORKERS));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -94,8 +141,8 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED>, mats, items, seeds, one, split, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
-                              p.stages, p.cluster);
+    return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, seeds, one, split, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
+                              (int)p.sbs, p.g_slots, p.a_slots, p.cluster);
 }
 inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds,
                                         const GenMat& one, int split, int seed_base, int r, float a, float b, cudaStream_t st,
@@ -103,10 +150,12 @@ inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int cluste
 {
     auto go = [&](auto launch) { return launch(p, clusters, mats, items, seeds, one, split, seed_base, r, a, b, st); };
     cudaError_t e;
-    if (items) e = f32 ? (p.aligned ? go(gen_launch_k1<false, true, true>) : go(gen_launch_k1<false, true, false>))
-                       : (p.aligned ? go(gen_launch_k1<false, false, true>) : go(gen_launch_k1<false, false, false>));
-    else e = f32 ? (p.aligned ? go(gen_launch_k1<true, true, true>) : go(gen_launch_k1<true, true, false>))
-                 : (p.aligned ? go(gen_launch_k1<true, false, true>) : go(gen_launch_k1<true, false, false>));
+#define FLORA_GEN_K1(SINGLE, F32, ALIGNED) (p.workers == 16 ? go(gen_launch_k1<SINGLE, F32, ALIGNED, 16>) : go(gen_launch_k1<SINGLE, F32, ALIGNED, 8>))
+    if (items) e = f32 ? (p.aligned ? FLORA_GEN_K1(false, true, true) : FLORA_GEN_K1(false, true, false))
+                       : (p.aligned ? FLORA_GEN_K1(false, false, true) : FLORA_GEN_K1(false, false, false));
+    else e = f32 ? (p.aligned ? FLORA_GEN_K1(true, true, true) : FLORA_GEN_K1(true, true, false))
+                 : (p.aligned ? FLORA_GEN_K1(true, false, true) : FLORA_GEN_K1(true, false, false));
+#undef FLORA_GEN_K1
     launches.fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
@@ -118,35 +167,39 @@ inline GenMat gen_mat(const flora_mat& big, const flora_mat& s)
 // What the kernels index with 32 bits.
 inline bool gen_supported(const flora_mat& big) { return big.rows < (1ll << 31) - 1024 && big.cols < (1ll << 31) - 1024; }
 
+// Small bf16 matrices that TMA could address are quicker here: these kernels start with less set-up (no tensor maps to fetch, no
+// zeroing or scaling launch for a split matrix) and share a row group among up to sixteen CTAs.  Measured, us per call with
+// the TMA kernels and with these: compress 768 x 768 at r = 16 10.9 / 4.9, 3072 x 768 at r = 16 11.2 / 6.6, 2048 x 2048 at r = 64
+// 19.1 / 17.0 (overwriting) and 15.9 / 17.1 (adding), 1024 x 1024 at r = 256 20.4 / 15.7, but 2048 x 2048 at r = 128 17.9 / 20.0 and
+// 512 x 8192 at r = 32 13.9 / 14.4; decompress 768 x 768 at r = 16 6.2 / 4.5, 1024 x 4096 at r = 16 8.0 / 7.2, 1024 x 1024 at
+// r = 128 11.6 / 9.9, but 2816 x 1024 at r = 64 8.9 / 9.4 and 2048 x 2048 at r = 256 15.5 / 31.4.
+// A set of small matrices stops gaining a little earlier (its TMA kernels start once for all): `elements` of a set are counted
+// as 5/3.  (4 x 768 x 768 at r = 16: compress 11.1 / 7.0, decompress 6.6 / 6.0; 7 M elements at r = 16: 13.6 / 12.9 and 10.4 / 13.8.)
+inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r)
+{
+    const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
+    if (knob >= 0) return knob == 1;
+    return cols <= 4096 && elements <= (r <= 64 ? 4 << 20 : 5 << 18);
+}
+inline bool gen_decompress_quicker(int64_t elements, int r)
+{
+    const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
+    if (knob >= 0) return knob == 1;
+    return elements <= (r <= 32 ? 5 << 20 : r <= 64 ? 2 << 20 : 5 << 18);
+}
+
 inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, uint64_t seed, float a, float b, cudaStream_t st,
                                         std::atomic<uint64_t>& launches)
 {
     const bool f32 = G.dtype == FLORA_F32;
     const int r = (int)S.cols;
     const int64_t tiles = (G.rows + 127) / 128, steps = (G.cols + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
-    // tile shape and split with the shortest schedule: waves of CTAs times the steps of one
-    GenK1Plan p;
-    int split = 1;
-    double best = 1e300;
-    for (int T = 1; T <= 4; T *= 2)
-        for (int k = 1; k <= 8; k *= 2) {
-            if (T > 1 && tiles < T) continue;
-            if ((k > 1 && steps < k) || !gen_k1_fits(f32, r, T, k > 1)) continue;
-            GenK1Plan cand;
-            gen_k1_shape(cand, f32, r, T, k > 1);
-            const double cost = gen_k1_cost(f32, r, T, cand.per_sm, ((tiles + T - 1) / T) * k, (steps + k - 1) / k, k);
-            if (cost < best * 0.98) {
-                best = cost;
-                p = cand;
-                split = k;
-            }
-        }
+    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps);
     const int64_t groups = (tiles + p.T - 1) / p.T;
-    p.cluster = split;
     p.aligned = gen_aligned(G);
     SeedTable table;
     table.s[0] = seed;
-    return gen_compress_launch(f32, p, (int)groups, nullptr, nullptr, table, gen_mat(G, S), split, 0, r, a, b, st, launches);
+    return gen_compress_launch(f32, p, (int)groups, nullptr, nullptr, table, gen_mat(G, S), p.cluster, 0, r, a, b, st, launches);
 }
 
 // Decompression: slabs of 128 columns for bf16 matrices whose rows move in 16-byte pieces, of 64 otherwise (an element-wise
@@ -274,27 +327,28 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     const int64_t sms = sm_count();
     if (kind == 0) {
         const int K = s.f32 ? 32 : 64;
-        int64_t max_tiles = 1, total = 0;
+        int64_t total = 0;
         for (int i : ids) {
             const int64_t tiles = (big[i].rows + 127) / 128;
-            max_tiles = std::max(max_tiles, tiles);
             total += tiles * ((big[i].cols + K - 1) / K);
             s.plan.aligned = s.plan.aligned && gen_aligned(big[i]);
         }
-        int T = gen_k1_tiles(s.f32, s.r, max_tiles);
-        // a CTA's share of the work, in tile-steps, with about three items per resident CTA; at least two steps of T tiles
-        const int64_t share = std::max<int64_t>(2 * T, total / (2 * sms * 3));
+        // One kind of CTA for the whole list: one tile, eight warps, two to an SM, where that fits (more tiles to share a tile of A
+        // lose more to the longer step than they save: measured); per matrix as many CTAs along the columns as leave each about a
+        // third of an SM's share of the work, and a single short wave on a small list.
+        const int per_sm = gen_k1_shape(s.plan, s.f32, s.r, 1, true, 2) ? 2 : 1;
+        const int64_t share = std::max<int64_t>(2, total / (per_sm * sms * 3));
         std::vector<int> split(big.size(), 1);
         int cluster = 1;
         for (int i : ids) {
-            const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K;
-            while (split[i] < 8 && std::min<int64_t>(T, tiles) * steps > 2 * share * split[i] && steps >= 4 * split[i]) split[i] *= 2;
+            const int64_t steps = (big[i].cols + K - 1) / K;
+            while (split[i] < 8 && steps > share * split[i] * 3 / 2 && steps >= 2 * split[i]) split[i] *= 2;
             cluster = std::max(cluster, split[i]);
         }
-        if (cluster > 1)
-            while (T > 1 && !gen_k1_fits(s.f32, s.r, T, true)) T /= 2;
-        gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1);
+        const int T = 1;
+        if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
+        s.plan.workers = per_sm == 2 ? 8 : 16;
         for (int i : ids) {
             const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = (int64_t)(cluster / split[i]) * T;
             for (int64_t t0 = 0; t0 < tiles; t0 += per)

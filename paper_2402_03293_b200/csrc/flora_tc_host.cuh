@@ -164,8 +164,9 @@ inline int tune_knob(const char*, int dflt, int, int) { return dflt; }
 // Lifts a kernel's limit on dynamic shared memory to what the device allows, once per kernel and device.  The
 // attribute belongs to the function, not to a launch: it is raised to the maximum once and never lowered, so sets
 // with different footprints can be alive, and launched in any order, at the same time.
+// wide: clusters of more than eight CTAs are wanted too.
 template <auto Kernel>
-inline bool raise_smem_limit()
+inline bool raise_smem_limit(bool wide = false)
 {
     static std::mutex mutex;
     static std::atomic<bool> done[POOL_MAX_DEVICES] = {};
@@ -178,7 +179,8 @@ inline bool raise_smem_limit()
     std::lock_guard<std::mutex> lock(mutex);
     cudaFuncAttributes fa;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || cudaFuncGetAttributes(&fa, Kernel) != cudaSuccess ||
-        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) != cudaSuccess) {
+        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) != cudaSuccess ||
+        (wide && cudaFuncSetAttribute(Kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
         return false;
     }
@@ -189,10 +191,10 @@ inline bool raise_smem_limit()
 // Clusters of `S` CTAs of `Kernel` that can be resident at once (fewer than SMs / S: a cluster sits inside one GPC);
 // SMs / S when there is no device to ask.
 template <auto Kernel>
-inline int resident_clusters(int S, int threads, size_t smem)
+inline int resident_clusters(int S, int threads, size_t smem, bool wide = false)
 {
     int slots = std::max(1, sm_count() / S);
-    if (!raise_smem_limit<Kernel>()) return slots;
+    if (!raise_smem_limit<Kernel>(wide)) return slots;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(S * 64));
     cfg.blockDim = dim3((unsigned)threads);
