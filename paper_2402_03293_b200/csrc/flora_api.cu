@@ -179,7 +179,7 @@ bool use_gen(const flora_mat* big) { return g_force_path.load(std::memory_order_
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 {
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch) && 
-           !gen_compress_quicker(big->rows * big->cols, big->cols, (int)sketch->cols);
+           !gen_compress_quicker(big->rows * big->cols, big->cols, (int)sketch->cols, big->dtype == FLORA_F32);
 }
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
 {
@@ -197,6 +197,7 @@ struct flora_set {
     int r = 0;
     bool has_G = false, has_W = false;
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
+    TcSet tcf;                     // the same for the compression of fp32 matrices
     GenSet gen_g[2], gen_w[2];     // the others, by dtype
 };
 
@@ -205,9 +206,9 @@ struct flora_set {
 constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
 
 // Which matrices of one side (G: compression, or W: decompression) of a set the TMA kernels serve.
-static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression)
+static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression, bool f32 = false)
 {
-    std::vector<uint8_t> use = tc_eligible(big, S);
+    std::vector<uint8_t> use = tc_eligible(big, S, f32);
     int64_t eligible = 0, widest = 0;
     bool mixed = false;
     for (size_t i = 0; i < big.size(); ++i) {
@@ -217,7 +218,7 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
     }
     const int r = S.empty() ? 1 : (int)S[0].cols;
     const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
-    if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) || (compression ? gen_compress_quicker(counted, widest, r) : gen_decompress_quicker(counted, r)))
+    if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) || (compression ? gen_compress_quicker(counted, widest, r, f32) : gen_decompress_quicker(counted, r)))
         std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
 }
@@ -226,12 +227,17 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
 static flora_status set_build(flora_set* s)
 {
     tc_set_free(s->tc);
+    tc_set_free(s->tcf);
     for (int d = 0; d < 2; ++d) {
         gen_set_free(s->gen_g[d]);
         gen_set_free(s->gen_w[d]);
     }
-    const std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true), use_w = set_tma_side(s->W, s->S, false);
+    std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true);
+    const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_w = set_tma_side(s->W, s->S, false);
     flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
+    if (st == FLORA_OK && std::find(use_f.begin(), use_f.end(), (uint8_t)1) != use_f.end())
+        st = tc_set_build_on(s->tcf, s->G, {}, s->S, nullptr, use_f, {});
+    for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
         std::vector<int> g, w;
         for (size_t i = 0; i < s->S.size(); ++i) {
@@ -398,6 +404,7 @@ flora_status flora_set_destroy(flora_set* set)
 {
     if (!set) return FLORA_OK;
     tc_set_free(set->tc);
+    tc_set_free(set->tcf);
     for (int d = 0; d < 2; ++d) {
         gen_set_free(set->gen_g[d]);
         gen_set_free(set->gen_w[d]);
@@ -418,8 +425,9 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
     }
     std::vector<flora_mat> newG(G, G + set->G.size());
     flora_status st = tc_set_rebind(set->tc, newG, as_stream(stream));
-    if (st == FLORA_ERR_ALIGN && (set->gen_g[0].ready() || set->gen_g[1].ready())) {
-        // a mixed set takes any address: the matrix changes sides (work that still reads the old tables ends first)
+    if (st == FLORA_OK) st = tc_set_rebind(set->tcf, newG, as_stream(stream));
+    if (st == FLORA_ERR_ALIGN && (set->gen_g[0].ready() || set->gen_g[1].ready() || set->tcf.compress_ready)) {
+        // a mixed (or fp32) set takes any address: the matrix changes sides (work that still reads the old tables ends first)
         set->G.swap(newG);
         return cudaStreamSynchronize(as_stream(stream)) == cudaSuccess ? set_build(set) : FLORA_ERR_CUDA;
     }
@@ -438,6 +446,7 @@ static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a,
     if (!simt) {
         flora_status st = FLORA_OK;
         if (set->tc.compress_ready) st = tc_set_compress(set->tc, seeds, a, b, as_stream(stream), g_launches, behind_own_transfer);
+        if (st == FLORA_OK && set->tcf.compress_ready) st = tc_set_compress(set->tcf, seeds, a, b, as_stream(stream), g_launches);
         for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_compress(set->gen_g[d], seeds, a, b, as_stream(stream), g_launches);
         if (st) return st;
     }

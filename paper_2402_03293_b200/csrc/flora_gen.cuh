@@ -122,8 +122,9 @@ __host__ __device__ inline int gen_stage_stride(int r_pad) { return r_pad + 4; }
 
 // SINGLE: one matrix, passed by value; every cluster takes the next row groups of it.  (A template and not a test of `items`: with
 // a run-time choice between the table's entry and the by-value one the kernel was seen to read the other one's address.)
-// sbs (fp32): the three parts of A side by side as one N operand (three MMAs per tile and K slice instead of six), their products
-// in three blocks of the accumulator, which are added up when they are read back.
+// sbs (fp32): the three parts of A side by side as one N operand (three MMAs per tile and K slice instead of six).  The tensor core
+// truncates its sums (2e-8 of the running sum lost per accumulation), so the large products, h h, have a block of the accumulator to
+// themselves and the small ones one or two others; the blocks are added up when they are read back.
 template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 __global__ void __launch_bounds__(gen_threads(WORKERS), WORKERS == 8 ? 2 : 1)
 gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
@@ -137,7 +138,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     uint8_t* const ring = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     __shared__ GenSmem ctl;
     const int r_pad = (r + 15) & ~15;
-    const int acc_cols = F32 && sbs ? 3 * r_pad : r_pad;
+    const int acc_cols = F32 ? (sbs ? 3 : 2) * r_pad : r_pad;
     const uint32_t a_part = (uint32_t)r_pad * C::ROWB;
     constexpr uint32_t G_BYTES = (uint32_t)C::PARTS * C::TILE;
     const uint32_t a_bytes = C::PARTS * a_part, a_ring = smem_base + (uint32_t)g_slots * G_BYTES;
@@ -216,16 +217,16 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                         if (!F32) {
                             ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, id, on);
                         } else if (sbs) {
-                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(3u * r_pad), on);
-                            ptx::umma_bf16(acc, dg + gp + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(2u * r_pad), 1u);
-                            ptx::umma_bf16(acc, dg + 2 * gp + kk * 2, da + kk * 2, id, 1u);
+                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(3u * r_pad), on);                  // h h | h m | h l
+                            ptx::umma_bf16(acc + r_pad, dg + gp + kk * 2, da + kk * 2, ptx::umma_idesc_bf16(2u * r_pad), 1u);     //     | m h | m m
+                            ptx::umma_bf16(acc + 2 * r_pad, dg + 2 * gp + kk * 2, da + kk * 2, id, 1u);                           //           | l h
                         } else {
-                            ptx::umma_bf16(acc, dg + 2 * gp + kk * 2, da + kk * 2, id, on);                // l h
-                            ptx::umma_bf16(acc, dg + kk * 2, da + 2 * ap + kk * 2, id, 1u);                // h l
-                            ptx::umma_bf16(acc, dg + gp + kk * 2, da + ap + kk * 2, id, 1u);               // m m
-                            ptx::umma_bf16(acc, dg + gp + kk * 2, da + kk * 2, id, 1u);                    // m h
-                            ptx::umma_bf16(acc, dg + kk * 2, da + ap + kk * 2, id, 1u);                    // h m
-                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, id, 1u);                         // h h
+                            ptx::umma_bf16(acc + r_pad, dg + 2 * gp + kk * 2, da + kk * 2, id, on);        // l h
+                            ptx::umma_bf16(acc + r_pad, dg + kk * 2, da + 2 * ap + kk * 2, id, 1u);        // h l
+                            ptx::umma_bf16(acc + r_pad, dg + gp + kk * 2, da + ap + kk * 2, id, 1u);       // m m
+                            ptx::umma_bf16(acc + r_pad, dg + gp + kk * 2, da + kk * 2, id, 1u);            // m h
+                            ptx::umma_bf16(acc + r_pad, dg + kk * 2, da + ap + kk * 2, id, 1u);            // h m
+                            ptx::umma_bf16(acc, dg + kk * 2, da + kk * 2, id, on);                         // h h
                         }
                     }
                     ptx::umma_commit(ptx::smem_addr(&ctl.empty[pg.s]));
@@ -396,14 +397,14 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 if (steps > 0) {
                     const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(t * acc_cols + c);
                     ptx::tmem_ld_16(at, v);
-                    if (F32 && sbs) {
+                    if (F32) {
                         uint32_t v1[16], v2[16];
                         ptx::tmem_ld_16(at + r_pad, v1);
-                        ptx::tmem_ld_16(at + 2 * r_pad, v2);
+                        if (sbs) ptx::tmem_ld_16(at + 2 * r_pad, v2);
                         ptx::tmem_ld_wait();
 #pragma unroll
                         for (int k = 0; k < 16; ++k)
-                            v[k] = __float_as_uint(__uint_as_float(v[k]) + (__uint_as_float(v1[k]) + __uint_as_float(v2[k])));
+                            v[k] = __float_as_uint(__uint_as_float(v[k]) + (__uint_as_float(v1[k]) + (sbs ? __uint_as_float(v2[k]) : 0.0f)));
                     } else {
                         ptx::tmem_ld_wait();
                     }
@@ -542,6 +543,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                       const __grid_constant__ SeedTable seeds, const __grid_constant__ GenMat single, int seed_base, int r, float scale, float step)
 {
     constexpr int PARTS = F32 ? 3 : 1, ROWB = 2 * KB;
+    constexpr uint32_t TMEM_COLS = F32 ? 2 * BN : BN;             // fp32: the large products, and the small ones (see the compression)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     __shared__ GenK2Smem ctl;
@@ -570,7 +572,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
         ptx::fence_proxy_async_smem();
     }
     if (warp == 1) {
-        ptx::tmem_alloc(ptx::smem_addr(&ctl.tmem_base), BN);
+        ptx::tmem_alloc(ptx::smem_addr(&ctl.tmem_base), TMEM_COLS);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before_sync();
@@ -705,14 +707,15 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                         constexpr uint64_t sp = SOP_PART >> 4, ap = SLAB_PART >> 4;
                         for (int kk = 0; kk < live >> 4; ++kk) {
                             const uint32_t on = (kc | kk) != 0;
-                            ptx::umma_bf16(tmem, ds + 2 * sp + kk * 2, da + kk * 2, id, on);                       // l h
+                            const uint32_t minor = tmem + (F32 ? BN : 0);
+                            ptx::umma_bf16(minor, ds + 2 * sp + kk * 2, da + kk * 2, id, on);                      // l h
                             if (F32) {
-                                ptx::umma_bf16(tmem, ds + kk * 2, da + 2 * ap + kk * 2, id, 1u);                   // h l
-                                ptx::umma_bf16(tmem, ds + sp + kk * 2, da + ap + kk * 2, id, 1u);                  // m m
+                                ptx::umma_bf16(minor, ds + kk * 2, da + 2 * ap + kk * 2, id, 1u);                  // h l
+                                ptx::umma_bf16(minor, ds + sp + kk * 2, da + ap + kk * 2, id, 1u);                 // m m
                             }
-                            ptx::umma_bf16(tmem, ds + sp + kk * 2, da + kk * 2, id, 1u);                           // m h
-                            if (F32) ptx::umma_bf16(tmem, ds + kk * 2, da + ap + kk * 2, id, 1u);                  // h m
-                            ptx::umma_bf16(tmem, ds + kk * 2, da + kk * 2, id, 1u);                                // h h
+                            ptx::umma_bf16(minor, ds + sp + kk * 2, da + kk * 2, id, 1u);                          // m h
+                            if (F32) ptx::umma_bf16(minor, ds + kk * 2, da + ap + kk * 2, id, 1u);                 // h m
+                            ptx::umma_bf16(tmem, ds + kk * 2, da + kk * 2, id, F32 ? on : 1u);                     // h h
                         }
                         ptx::umma_commit(ptx::smem_addr(&ctl.done));
                     }
@@ -736,7 +739,15 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                 for (int c = 0; c < NC; c += 16) {
                     uint32_t v[16];
                     ptx::tmem_ld_16(at + c, v);
-                    ptx::tmem_ld_wait();
+                    if (F32) {
+                        uint32_t y[16];
+                        ptx::tmem_ld_16(at + BN + c, y);
+                        ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(y[k]));
+                    } else {
+                        ptx::tmem_ld_wait();
+                    }
 #pragma unroll
                     for (int k = 0; k < 16; k += 4)
                         *reinterpret_cast<float4*>(to + c + k) =
@@ -797,7 +808,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
     __syncthreads();
     if (warp == 1) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, BN);
+        ptx::tmem_dealloc(tmem, TMEM_COLS);
     }
 }
 

@@ -25,6 +25,9 @@ inline bool gen_aligned(const flora_mat& g)
     return ((reinterpret_cast<uintptr_t>(g.data) | (uintptr_t)(g.ld * es)) & 15) == 0;
 }
 
+// Steps of 32 columns that a CTA adds up for fp32 matrices (two truncated accumulations of large products each, 2e-8 of the sum lost
+// in every one: 3e-6, what plain rounded fp32 loses over 10^4 products).
+constexpr int GEN_F32_CHAIN_STEPS = 72;
 // Rings, accumulator layout and CTAs per SM for T tiles per CTA; false where they do not fit.  `per_sm` = 2: two CTAs with at
 // most 112 KB and 256 accumulator columns each.  At least three slots of G and two of A (with fewer the warps wait for the MMAs of
 // the step before: fp32 4096 x 11008 at r = 8 ran at half the speed).
@@ -32,7 +35,7 @@ inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int p
 {
     const int r_pad = (r + 15) & ~15, most_cols = per_sm == 2 ? 256 : 512;
     p.sbs = f32 && 3 * r_pad <= 256 && T * 3 * r_pad <= most_cols;
-    const int cols_used = T * (p.sbs ? 3 * r_pad : r_pad);
+    const int cols_used = T * (!f32 ? r_pad : (p.sbs ? 3 : 2) * r_pad);
     if (cols_used > most_cols) return false;
     const size_t budget = (per_sm == 2 ? 112 * 1024 : SMEM_BUDGET) - 1024;
     const size_t g = gen_k1_g_bytes(f32), a = gen_k1_a_bytes(f32, r_pad);
@@ -98,6 +101,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
         for (int split = 1; split <= GEN_MAX_SPLIT; ++split)
             for (int workers = 8; workers <= 16; workers += 8) {
                 if ((T > 1 && tiles < T) || (split > 1 && steps < split)) continue;
+                if (f32 && split < GEN_MAX_SPLIT && steps > (int64_t)GEN_F32_CHAIN_STEPS * split) continue;
                 if (tune_knob("FLORA_GEN_T", T, 1, 4) != T || tune_knob("FLORA_GEN_SPLIT", split, 1, 16) != split ||
                     tune_knob("FLORA_GEN_WORKERS", workers, 8, 16) != workers)
                     continue;
@@ -175,10 +179,13 @@ inline bool gen_supported(const flora_mat& big) { return big.rows < (1ll << 31) 
 // r = 128 11.6 / 9.9, but 2816 x 1024 at r = 64 8.9 / 9.4 and 2048 x 2048 at r = 256 15.5 / 31.4.
 // A set of small matrices stops gaining a little earlier (its TMA kernels start once for all): `elements` of a set are counted
 // as 5/3.  (4 x 768 x 768 at r = 16: compress 11.1 / 7.0, decompress 6.6 / 6.0; 7 M elements at r = 16: 13.6 / 12.9 and 10.4 / 13.8.)
-inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r)
+inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32)
 {
     const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
     if (knob >= 0) return knob == 1;
+    // (fp32: 1024 x 1024 at r = 8 12.6 / 8.3, at r = 64 22 / 12; 768 x 3072 at r = 64 23 / 15.5; 2048 x 2048 at r = 64 23.5 / 21; 1024 x 4096 at
+    // r = 64 23.5 / 24.3.  Bit-reproducible results of long rows need the split over a cluster, which only these kernels have.)
+    if (f32) return (cols <= 3072 && elements <= 5 << 19) || deterministic_flag().load();
     return cols <= 4096 && elements <= (r <= 64 ? 4 << 20 : 5 << 18);
 }
 inline bool gen_decompress_quicker(int64_t elements, int r)
@@ -342,7 +349,8 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         int cluster = 1;
         for (int i : ids) {
             const int64_t steps = (big[i].cols + K - 1) / K;
-            while (split[i] < 8 && steps > share * split[i] * 3 / 2 && steps >= 2 * split[i]) split[i] *= 2;
+            while (split[i] < 8 && (steps > share * split[i] * 3 / 2 || (s.f32 && steps > (int64_t)GEN_F32_CHAIN_STEPS * split[i])) && steps >= 2 * split[i])
+                split[i] *= 2;
             cluster = std::max(cluster, split[i]);
         }
         const int T = 1;

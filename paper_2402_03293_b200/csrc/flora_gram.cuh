@@ -702,7 +702,7 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     memset(&single_arg, 0, sizeof(single_arg));
     if (tc_apply && single_job) {
         flora_mat md{jobs[0].dst, jobs[0].n, r, jobs[0].ldd, FLORA_F32}, ms{(void*)jobs[0].src, jobs[0].n, r, jobs[0].lds, FLORA_F32};
-        tc_apply = make_map_f32(&single_arg.map_dst, md) && make_map_f32(&single_arg.map_src, ms);
+        tc_apply = make_map(&single_arg.map_dst, md) && make_map(&single_arg.map_src, ms);
     }
     const bool single_maps = tc_apply && single_job;
     if (tc_apply)                            // the kernel wants T^T as its K-major operand: exchange the roles of the two projections

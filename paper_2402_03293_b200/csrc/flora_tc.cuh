@@ -89,45 +89,68 @@ inline int k1_threads(int gen_warps) { return 64 + 32 * gen_warps + 32; }
 constexpr int G_TILE_BYTES = 128 * 128;   // 128 rows x 64 bf16
 constexpr int S_CHUNK_BYTES_K1 = 128 * 128; // 128 rows x 32 fp32
 
-struct K1Smem {                            // barriers and scalars, placed after the tile ring
-    uint64_t full_g[8], empty_g[8], full_a[8], slice_ready[8], empty_a[8], acc_full, old_full[16];
+constexpr int K1_MAX_LSTAGES = 2;
+
+struct K1Smem {                            // barriers and scalars, placed after the tile rings
+    uint64_t full_g[8], empty_g[8], full_a[8], slice_ready[8], empty_a[8], full_l[K1_MAX_LSTAGES], empty_l[K1_MAX_LSTAGES], acc_full, old_full[16];
     uint32_t tmem_base;
     int abort;
     int epi_go[4];
 };
 
+// fp32 matrices (F32): G streams through the same ring (steps of 32 columns, tiles of the same 16 KB) and is multiplied as tf32,
+// whose operands are 32-bit words of which the tensor core takes the upper 19 bits: hi(G).  The generator warps write what that
+// leaves, lo(G) = G - hi(G) rounded to tf32, into a ring of its own, and A as hi(A) and lo(A) in two halves of its tile.  The sum of
+// hi hi, hi lo and lo hi carries 2^-22 of a product, below the rounding of the fp32 sum that it joins.  The tensor core's sums are
+// truncated, not rounded: every accumulation loses about 2e-8 of the running sum, always towards zero (measured: 6e-6 after 300), so
+// the small products have an accumulator of their own (`minor`), the steps of an item take up to `nsets` pairs of accumulators in
+// turn, the planner caps the steps of an item, and the parts are added up in rounded fp32 at the end.  What bounds a step then: the 16 KB of a tile from HBM (700 cycles of an SM's share) against 130 cycles of issue slots
+// for its lo(G), 11 r cycles for A and 400 of tensor pipe; the kernel that cut fp32 into three bf16 parts out of registers spent
+// 670 issue cycles on a tile.
 // SINGLE: one matrix, its record passed by value (every item names matrix 0).
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
 // 4096 x 11008 matrix takes 27 us instead of 20)
-template <bool SINGLE>
+template <bool SINGLE, bool F32>
 __global__ void __maxnreg__(80)
 compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
-                   int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int S, int GW, int P, int late_wait)
+                   int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int lstages, int nsets, int S, int GW, int P,
+                   int late_wait)
 {
+    constexpr int KC = F32 ? 32 : 64;                          // columns of a step
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     const int r_pad = (r + 15) & ~15;
-    const uint32_t a_bytes = (uint32_t)r_pad * 128u;
-    // two rings: G tiles (gstages x T tiles; the loads come from HBM and want many bytes in flight) and A tiles
+    const uint32_t a_part = (uint32_t)r_pad * 128u, a_bytes = F32 ? 2u * a_part : a_part;      // (F32: rows of hi(A), then rows of lo(A))
+    // accumulator of a tile; F32: hi hi in the first r_pad columns, the small products in the next
+    const int acc_cols = F32 ? 2 * r_pad : r_pad;
+    // F32: steps that share a pair of accumulators, and how many pairs an item uses
+    const int per_set = F32 ? max(16, (items[blockIdx.x].ksteps + nsets - 1) / nsets) : 1;
+    // two rings (F32: three): G tiles (gstages x T tiles; the loads come from HBM and want many bytes in flight) and A tiles
     // (astages x r_pad rows; produced on chip).  Each has its own full / empty barriers.
     const uint32_t g_bytes = (uint32_t)T * G_TILE_BYTES;
     const uint32_t a_ring = smem_base + (uint32_t)gstages * g_bytes;
-    K1Smem* ctl = reinterpret_cast<K1Smem*>(smem_raw + (a_ring - ptx::smem_addr(smem_raw)) + (size_t)astages * a_bytes);
+    const uint32_t l_ring = a_ring + (uint32_t)astages * a_bytes;
+    K1Smem* ctl = reinterpret_cast<K1Smem*>(smem_raw + (l_ring - ptx::smem_addr(smem_raw)) + (F32 ? (size_t)lstages * g_bytes : 0));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     const K1Item item = items[blockIdx.x];                    // tables and descriptors are written at set creation, not by kernels
     const TcMatrix* mat = SINGLE ? &single : table + item.mat;
     uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < T * r_pad) tmem_cols <<= 1;
+    while ((int)tmem_cols < T * acc_cols * (F32 ? nsets : 1)) tmem_cols <<= 1;
 
     if (threadIdx.x == 0) {
+        if (F32)
+            for (int s = 0; s < lstages; ++s) {
+                ptx::mbar_init(ptx::smem_addr(&ctl->full_l[s]), GW - P);
+                ptx::mbar_init(ptx::smem_addr(&ctl->empty_l[s]), 1);
+            }
         for (int s = 0; s < gstages; ++s) {
             ptx::mbar_init(ptx::smem_addr(&ctl->full_g[s]), 1);
             ptx::mbar_init(ptx::smem_addr(&ctl->empty_g[s]), 1);                   // this CTA's MMAs have consumed the G tiles
         }
         for (int s = 0; s < astages; ++s) {
-            ptx::mbar_init(ptx::smem_addr(&ctl->full_a[s]), S > 1 ? 1 : GW / P);   // cluster: one arrival + the peers' bytes
-            ptx::mbar_init(ptx::smem_addr(&ctl->slice_ready[s]), GW / P);
+            ptx::mbar_init(ptx::smem_addr(&ctl->full_a[s]), S > 1 ? 1 : F32 ? P : GW / P);   // cluster: one arrival + the peers' bytes
+            ptx::mbar_init(ptx::smem_addr(&ctl->slice_ready[s]), F32 ? P : GW / P);
             ptx::mbar_init(ptx::smem_addr(&ctl->empty_a[s]), S);                   // every CTA of the cluster has consumed the A tile
         }
         ptx::mbar_init(ptx::smem_addr(&ctl->acc_full), 1);
@@ -144,9 +167,9 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     // rows r .. r_pad of every A tile stay zero for the whole kernel
     if (r_pad > r) {
         const int pad_chunks = (r_pad - r) * 8;
-        for (int s = 0; s < astages; ++s)
+        for (int s = 0; s < astages * (F32 ? 2 : 1); ++s)
             for (int t = threadIdx.x; t < pad_chunks; t += (int)blockDim.x)
-                ptx::st_shared_v4(a_ring + s * a_bytes + (uint32_t)r * 128u + t * 16u, 0, 0, 0, 0);
+                ptx::st_shared_v4(a_ring + s * a_part + (uint32_t)r * 128u + t * 16u, 0, 0, 0, 0);
         ptx::fence_proxy_async_smem();
     }
     ptx::tc_fence_before_sync();
@@ -176,7 +199,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                 const uint32_t bar = ptx::smem_addr(&ctl->full_g[s]);
                 ptx::mbar_arrive_expect_tx(bar, (uint32_t)item.tiles * G_TILE_BYTES);
                 for (int t = 0; t < item.tiles; ++t)
-                    ptx::tma_load_2d(smem_base + s * g_bytes + t * G_TILE_BYTES, &mat->map_g, (item.kstep0 + ks) * 64, item.row0 + t * 128, bar);
+                    ptx::tma_load_2d(smem_base + s * g_bytes + t * G_TILE_BYTES, &mat->map_g, (item.kstep0 + ks) * KC, item.row0 + t * 128, bar);
                 issued = ks + 1;
             }
             if (*abort) {
@@ -188,14 +211,19 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = ptx::umma_idesc_bf16((uint32_t)r_pad);
+            const uint32_t idesc = F32 ? ptx::umma_idesc_tf32((uint32_t)r_pad) : ptx::umma_idesc_bf16((uint32_t)r_pad);
+            const bool sbs = 2 * r_pad <= 256;                       // F32: hi(A) and lo(A) side by side as one N operand
+            const uint32_t idesc2 = ptx::umma_idesc_tf32(2u * r_pad);
+            int in_set = 0, set = 0;                                 // F32: step within its pair of accumulators, and which pair
             const uint64_t desc_base = ptx::umma_desc_k_sw128(smem_base);
             bool ok = true;
-            RingPos rg, ra;
-            for (int ks = 0; ks < item.ksteps && ok; ++ks, rg.advance(gstages), ra.advance(astages)) {
+            RingPos rg, ra, rl;
+            for (int ks = 0; ks < item.ksteps && ok; ++ks, rg.advance(gstages), ra.advance(astages), rl.advance(F32 ? lstages : 1)) {
                 const int sg = rg.s, sa = ra.s;
                 const uint32_t pa = ra.wraps & 1u;
-                ok = (item.tiles == 0 || ptx::mbar_wait(ptx::smem_addr(&ctl->full_g[sg]), rg.wraps & 1u, abort)) &&
+                // (F32: lo(G) of the step is there, so G is, too)
+                ok = (item.tiles == 0 || (F32 ? ptx::mbar_wait(ptx::smem_addr(&ctl->full_l[rl.s]), rl.wraps & 1u, abort)
+                                              : ptx::mbar_wait(ptx::smem_addr(&ctl->full_g[sg]), rg.wraps & 1u, abort))) &&
                      (S > 1 ? ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->full_a[sa]), pa, abort)
                             : ptx::mbar_wait(ptx::smem_addr(&ctl->full_a[sa]), pa, abort));
                 if (!ok) break;
@@ -203,11 +231,41 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                 // descriptors differ from the ring base only in the start-address field (16-byte units)
                 const uint64_t dstage = desc_base + (uint64_t)((sg * g_bytes) >> 4);
                 const uint64_t da_tile = desc_base + (uint64_t)((a_ring - smem_base + sa * a_bytes) >> 4);
-                for (int t = 0; t < item.tiles; ++t) {
+                if (F32) {
+                    const uint64_t dlo = desc_base + (uint64_t)((l_ring - smem_base + rl.s * g_bytes) >> 4), da_lo = da_tile + (uint64_t)(a_part >> 4);
+                    // (grouped by shape: an MMA that writes a part of what the one before it wrote waits for that one's end)
+                    for (int t = 0; t < item.tiles; ++t) {
+                        const uint32_t acc = tmem + (set * T + t) * acc_cols, minor = acc + r_pad;
+                        const uint64_t dg = dstage + (uint64_t)((t * G_TILE_BYTES) >> 4);
+                        if (sbs) {
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        ptx::umma_bf16(tmem + t * r_pad, dstage + (uint64_t)((t * G_TILE_BYTES + kk * 32) >> 4), da_tile + (uint64_t)(kk * 2), idesc,
-                                       (ks | kk) != 0);
+                            for (int k8 = 0; k8 < 4; ++k8)                                                         // hi hi, hi lo
+                                ptx::umma_tf32(acc, dg + k8 * 2, da_tile + (uint64_t)(k8 * 2), idesc2, (in_set | k8) != 0);
+                        } else {
+#pragma unroll
+                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(acc, dg + k8 * 2, da_tile + (uint64_t)(k8 * 2), idesc, (in_set | k8) != 0);
+#pragma unroll
+                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(minor, dg + k8 * 2, da_lo + (uint64_t)(k8 * 2), idesc, (in_set | k8) != 0);
+                        }
+                    }
+                    for (int t = 0; t < item.tiles; ++t) {
+                        const uint32_t minor = tmem + (set * T + t) * acc_cols + r_pad;
+#pragma unroll
+                        for (int k8 = 0; k8 < 4; ++k8)                                                             // lo hi
+                            ptx::umma_tf32(minor, dlo + (uint64_t)((t * G_TILE_BYTES) >> 4) + k8 * 2, da_tile + (uint64_t)(k8 * 2), idesc, 1u);
+                    }
+                    if (++in_set == per_set) {
+                        in_set = 0;
+                        ++set;
+                    }
+                    if (item.tiles > 0) ptx::umma_commit(ptx::smem_addr(&ctl->empty_l[rl.s]));
+                } else {
+                    for (int t = 0; t < item.tiles; ++t) {
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            ptx::umma_bf16(tmem + t * r_pad, dstage + (uint64_t)((t * G_TILE_BYTES + kk * 32) >> 4), da_tile + (uint64_t)(kk * 2), idesc,
+                                           (ks | kk) != 0);
+                    }
                 }
                 if (item.tiles > 0) ptx::umma_commit(ptx::smem_addr(&ctl->empty_g[sg]));
                 // the A stage is free once every CTA of the cluster has consumed its copy of the tile
@@ -229,9 +287,12 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                 if (!ptx::mbar_wait(ptx::smem_addr(&ctl->slice_ready[s]), ra.wraps & 1u, abort)) break;
                 const uint32_t fbar = ptx::smem_addr(&ctl->full_a[s]);
                 const uint32_t src = a_ring + s * a_bytes + rank * slice_bytes;
-                ptx::mbar_arrive_expect_tx(fbar, (uint32_t)(S - 1) * slice_bytes);   // own slice is in place; peers' bytes to come
+                ptx::mbar_arrive_expect_tx(fbar, (uint32_t)(S - 1) * (F32 ? 2u : 1u) * slice_bytes);   // own slice is in place; peers' bytes to come
                 for (int d = 0; d < S; ++d)
-                    if (d != (int)rank) ptx::bulk_copy_to_peer(ptx::map_to_cta(src, d), src, slice_bytes, ptx::map_to_cta(fbar, d));
+                    if (d != (int)rank) {
+                        ptx::bulk_copy_to_peer(ptx::map_to_cta(src, d), src, slice_bytes, ptx::map_to_cta(fbar, d));
+                        if (F32) ptx::bulk_copy_to_peer(ptx::map_to_cta(src + a_part, d), src + a_part, slice_bytes, ptx::map_to_cta(fbar, d));
+                    }
             }
         }
     } else {
@@ -239,13 +300,77 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
         // The generator warps form P teams; team p writes the tiles of the steps p, p + P, ...: a thread's task (eight
         // values) is a long dependent chain, so with few tasks per thread it is latency, not issue rate, that bounds one
         // tile, and teams working on neighbouring steps at the same time hide it.
-        const int team_threads = 32 * (GW / P);
+        const int team_threads = F32 ? 32 * GW : 32 * (GW / P);
         const int team = (threadIdx.x - 64) / team_threads;
         const int g = (threadIdx.x - 64) - team * team_threads;   // 0 .. team_threads-1
         const PhiloxKey key = make_key(seeds.s[item.mat - seed_base]);
         const int tasks = r * 8;                              // (row j, 16-byte chunk c) pairs of one A tile
         bool ok = true;
-        for (int ks = team; ks < item.ksteps && ok; ks += P) {
+        if (F32) {
+            // The first P of these warps make A (this CTA's rows of it), the others lo(G): the two wait for different things, and warps
+            // that did both, one after the other, spent most of a step waiting (r = 64: 3000 cycles a step, of which HBM needs 1400).
+            if (g < 32 * P) {
+            RingPos ra;
+            const int nt = 32 * P, rows_here = S > 1 ? r_pad / S : r, j0 = S > 1 ? (int)rank * rows_here : 0;
+            const int tasks4 = min(rows_here, max(0, r - j0)) * 4;    // a task: eight columns of one row of A
+            int first = g;                                    // (moves on from step to step: with fewer tasks than threads the warps take turns)
+            for (int ks = 0; ks < item.ksteps && ok; ++ks, ra.advance(astages)) {
+                ok = ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->empty_a[ra.s]), (ra.wraps & 1u) ^ 1u, abort);
+                if (!ok) break;
+                const uint32_t a_tile = a_ring + ra.s * a_bytes;
+                const uint32_t q0 = (uint32_t)(item.kstep0 + ks) * 8u;
+                int t = first;
+                for (; t < tasks4; t += nt) {
+                    const int j = j0 + (t >> 2), c = t & 3;
+                    float v[2][4];
+                    projection_two_quads(q0 + 2 * c, (uint32_t)j, q0 + 2 * c + 1, (uint32_t)j, key, scale, v[0], v[1]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t hi[4], lo[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            hi[e] = (__float_as_uint(v[h][e]) + 0x1000u) & 0xFFFFE000u;               // rounded to tf32
+                            lo[e] = __float_as_uint(__fsub_rn(v[h][e], __uint_as_float(hi[e])));      // exact
+                        }
+                        const uint32_t at = a_tile + j * 128 + (((2 * c + h) ^ (j & 7)) << 4);
+                        ptx::st_shared_v4(at, hi[0], hi[1], hi[2], hi[3]);
+                        ptx::st_shared_v4(at + a_part, lo[0], lo[1], lo[2], lo[3]);
+                    }
+                }
+                first = t - tasks4;
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(S > 1 ? &ctl->slice_ready[ra.s] : &ctl->full_a[ra.s]));
+            }
+            } else if (item.tiles > 0) {
+            RingPos rg, rl;
+            const int l = g - 32 * P, nt = 32 * (GW - P);
+            for (int ks = 0; ks < item.ksteps && ok; ++ks, rg.advance(gstages), rl.advance(lstages)) {
+                ok = ptx::mbar_wait(ptx::smem_addr(&ctl->empty_l[rl.s]), (rl.wraps & 1u) ^ 1u, abort) &&
+                     ptx::mbar_wait(ptx::smem_addr(&ctl->full_g[rg.s]), rg.wraps & 1u, abort);
+                if (!ok) break;
+                const uint32_t src = smem_base + rg.s * g_bytes, dst = l_ring + rl.s * g_bytes;
+                const uint32_t end = (uint32_t)item.tiles * G_TILE_BYTES;
+                // same place in the tile, whatever its swizzle; four pieces of 16 bytes at a time (a tile has 1024; four times nt divides that)
+                for (uint32_t o = (uint32_t)l * 16u; o < end; o += (uint32_t)nt * 64u) {
+                    uint32_t x[4][4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) ptx::ld_shared_v4(src + o + (uint32_t)(u * nt) * 16u, x[u][0], x[u][1], x[u][2], x[u][3]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            x[u][e] = __float_as_uint(__fsub_rn(__uint_as_float(x[u][e]), __uint_as_float(x[u][e] & 0xFFFFE000u))) + 0x1000u;
+                        ptx::st_shared_v4(dst + o + (uint32_t)(u * nt) * 16u, x[u][0], x[u][1], x[u][2], x[u][3]);
+                    }
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->full_l[rl.s]));
+            }
+            }
+        }
+        for (int ks = team; !F32 && ks < item.ksteps && ok; ks += P) {
             const int s = ks % astages, it = ks / astages;
             ok = S > 1 ? ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->empty_a[s]), (it & 1) ^ 1, abort)
                        : ptx::mbar_wait(ptx::smem_addr(&ctl->empty_a[s]), (it & 1) ^ 1, abort);
@@ -339,14 +464,32 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                 if (!*(volatile int*)&ctl->epi_go[grp]) break;    // uniform: written before the barrier by one thread
                 const int t = i / nchunks, c = i % nchunks;
                 uint32_t v[32];
-                ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + t * r_pad + c * 32, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
-                if (c * 32 + 16 < r_pad)
-                    ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + t * r_pad + c * 32 + 16, *reinterpret_cast<uint32_t(*)[16]>(&v[16]));
-                else {
+                const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + t * acc_cols + c * 32;
+                const bool second = c * 32 + 16 < r_pad;
+                if (F32) {
 #pragma unroll
-                    for (int k = 16; k < 32; ++k) v[k] = 0u;
+                    for (int k = 0; k < 32; ++k) v[k] = 0u;
+                    for (int s = 0; s * per_set < item.ksteps; ++s)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if (h == 1 && !second) break;
+                            uint32_t x[16], y[16];
+                            ptx::tmem_ld_16(at + s * T * acc_cols + 16 * h, x);
+                            ptx::tmem_ld_16(at + s * T * acc_cols + r_pad + 16 * h, y);
+                            ptx::tmem_ld_wait();
+#pragma unroll
+                            for (int k = 0; k < 16; ++k)
+                                v[16 * h + k] = __float_as_uint(__uint_as_float(v[16 * h + k]) + (__uint_as_float(x[k]) + __uint_as_float(y[k])));
+                        }
+                } else {
+                    ptx::tmem_ld_16(at, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
+                    if (second) ptx::tmem_ld_16(at + 16, *reinterpret_cast<uint32_t(*)[16]>(&v[16]));
+                    else {
+#pragma unroll
+                        for (int k = 16; k < 32; ++k) v[k] = 0u;
+                    }
+                    ptx::tmem_ld_wait();
                 }
-                ptx::tmem_ld_wait();
                 const uint32_t brow = buffer(u) + (uint32_t)trow * 128u;
                 if (rmw) ptx::mbar_wait(ptx::smem_addr(&ctl->old_full[grp * 4 + u % NB]), (uint32_t)(u / NB) & 1u, abort);
 #pragma unroll

@@ -28,7 +28,8 @@ struct TcSet {
     bool compress_ready = false;
     bool decompress_ready = false;
     int count = 0, r = 0;
-    int T = 1, gstages = 2, astages = 2, S = 1, GW = 8, P = 1;
+    bool f32 = false;                   // fp32 matrices (compression only)
+    int T = 1, gstages = 2, astages = 2, lstages = 1, nsets = 1, S = 1, GW = 8, P = 1;
     std::vector<int> k1_launch_first_mat;
     size_t k1_smem = 0;
     TcMatrix* d_mats = nullptr;
@@ -76,30 +77,19 @@ inline EncodeTiledFn encode_tiled_fn()
     return fn;
 }
 
-// bf16 matrix, box = 64 columns x 128 rows, 128-byte swizzle, zero fill outside the matrix
+// A matrix in boxes of 128 bytes (64 bf16 or 32 fp32 columns) x 128 rows, 128-byte swizzle, zero fill outside the matrix
 inline bool make_map(CUtensorMap* out, const flora_mat& a)
 {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
+    const bool f32 = a.dtype == FLORA_F32;
     cuuint64_t dims[2] = {(cuuint64_t)a.cols, (cuuint64_t)a.rows};
-    cuuint64_t strides[1] = {(cuuint64_t)a.ld * 2};
-    cuuint32_t box[2] = {64, 128};
+    cuuint64_t strides[1] = {(cuuint64_t)a.ld * (f32 ? 4 : 2)};
+    cuuint32_t box[2] = {f32 ? 32u : 64u, 128};
     cuuint32_t estr[2] = {1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.data, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// fp32 sketch, box = 32 columns x 128 rows, 128-byte swizzle, zero fill outside the matrix
-inline bool make_map_f32(CUtensorMap* out, const flora_mat& a)
-{
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)a.cols, (cuuint64_t)a.rows};
-    cuuint64_t strides[1] = {(cuuint64_t)a.ld * 4};
-    cuuint32_t box[2] = {32, 128};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.data, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return fn(out, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.data, dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
 }
 
 inline bool tc_sketch_ok(const flora_mat& s)
@@ -113,9 +103,16 @@ inline bool tc_mat_ok(const flora_mat& a)
            (a.ld & 7) == 0 && a.rows < (1ll << 31) - 256 && a.cols < (1ll << 31) - 256;
 }
 
+// fp32 matrices for the compression kernel
+inline bool tc_f32_ok(const flora_mat& a)
+{
+    return a.dtype == FLORA_F32 && a.rows >= 128 && a.cols >= 32 && (reinterpret_cast<uintptr_t>(a.data) & 15) == 0 && (a.ld & 3) == 0 &&
+           a.rows < (1ll << 31) - 256 && a.cols < (1ll << 31) - 256;
+}
+
 inline bool tc_compress_supported(const flora_mat* big, const flora_mat* sketch)
 {
-    return tc_mat_ok(*big) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
+    return (tc_mat_ok(*big) || tc_f32_ok(*big)) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
 }
 
 // SMs of the current device (a process may drive several devices), asked once per device.
@@ -219,6 +216,9 @@ constexpr double K1_UNIT_OVERHEAD_STEPS = 6.0;
 // time that one element of a 128-row G tile costs its CTA (measured: an r x 64 tile takes about r * 64 * 0.18 ns of
 // one SM's ALUs, the 16 KB of a G tile 0.37 us of its share of HBM, and the ratio of the two per rank is about 0.045 / T).
 constexpr double K1_GENERATION_PER_RANK = 0.045;
+// Steps of 32 columns that an fp32 item may add into one accumulator: four accumulations each, 2e-8 of the sum lost in every one
+// of them, so at most 4e-6 and 1.2e-6 as measured (a sum of 10^4 products in plain rounded fp32 is off by 2.5e-6).
+constexpr int K1_F32_CHAIN_STEPS = 48;
 // Cost model of the decompression planner (microseconds on one SM): bytes an SM takes in per microsecond whatever their
 // source (about 60 GB/s with the tiles it can keep in flight), values of A per microsecond that the generator warps
 // make next to the streaming warps (8 or fewer warps), the share of a slab's generation that stays exposed with one
@@ -407,7 +407,11 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
 // so that the former stays under half of the latter.
 inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
 {
-    if (r > 64) {
+    set.f32 = false;
+    for (const auto& g : G) set.f32 = set.f32 || (g.rows > 0 && g.dtype == FLORA_F32);
+    const bool f32 = set.f32;
+    const int kc = f32 ? 32 : 64;                                // columns of a step
+    if (r > 64 && !f32) {
         plan_compress_pair(set, G, r);
         return;
     }
@@ -415,7 +419,7 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     const int r_pad = (r + 15) & ~15;
     int64_t max_tiles = 1, total_work = 0;       // work unit: one 128-row tile over one 64-column step
     for (const auto& g : G) {
-        const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + 63) / 64;
+        const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + kc - 1) / kc;
         max_tiles = std::max(max_tiles, tiles);
         total_work += tiles * ks;
     }
@@ -427,7 +431,7 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     auto padded_work = [&](int cand) {
         double padded = 0;
         for (const auto& g : G) {
-            const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + 63) / 64;
+            const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + kc - 1) / kc;
             padded += (double)((tiles + cand - 1) / cand * cand) * ks;
         }
         return padded;
@@ -436,15 +440,20 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     for (int cand = t_cap - 1; cand >= 1; --cand)
         if (padded_work(cand) < 0.8 * padded_work(T)) T = cand;
     T = tune_knob("FLORA_K1_T", T, 1, 512 / r_pad);
-    const size_t stage = (size_t)T * G_TILE_BYTES + (size_t)r_pad * 128;
+    // fp32: one tile per CTA and two CTAs per SM up to r = 32, where making A and lo(G) fits beside one tile's loads; two tiles above
+    // (one above r = 128, where the accumulators of two do not fit)
+    const int acc_cols = f32 ? 2 * r_pad : r_pad;
+    if (f32) T = tune_knob("FLORA_K1_T", (int)std::min<int64_t>(max_tiles, r_pad <= 32 || r_pad > 128 ? 1 : 2), 1, 512 / acc_cols);
+    const size_t stage = (size_t)T * G_TILE_BYTES * (f32 ? 2 : 1) + (size_t)r_pad * (f32 ? 256 : 128);
     uint32_t cols = 32;
-    while ((int)cols < T * r_pad) cols <<= 1;
+    while ((int)cols < T * acc_cols) cols <<= 1;
     // cluster size from the generation / load ratio
     const double ratio = r * K1_GENERATION_PER_RANK / T;
     int S = 1;
     while (S < 8 && ratio / S > 0.5) S <<= 1;
     while (S > 1 && (int64_t)S * T > 2 * max_tiles) S >>= 1;         // not more CTAs than there are rows to share
     S = tune_knob("FLORA_K1_CLUSTER", S, 1, 8);
+    if (f32) S = r_pad > 128 && max_tiles > 1 ? tune_knob("FLORA_K1_CLUSTER", 2, 1, 4) : 1;      // one tile per CTA: two CTAs make half of A each
     if (S & (S - 1)) S = 1;
     while (S > 1 && r_pad % (8 * S)) S >>= 1;                     // every CTA's slice of A is whole 8-row groups
     // two CTAs per SM when tensor memory allows it and each still gets two stages: the epilogue of one
@@ -455,17 +464,23 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     // link, bound the intake, so the G ring gets all the shared memory the A ring does not need.  A tiles are made on
     // chip: two stages; three (four for the large tiles of ranks above 128) where slices travel between the CTAs of a
     // cluster and the slowest CTA paces all of them.
-    const size_t g_stage = (size_t)T * G_TILE_BYTES, a_stage = (size_t)r_pad * 128;
-    const size_t ring_budget = SMEM_BUDGET / per_sm - sizeof(K1Smem) - 1024;
-    int astages = S > 1 ? (r_pad > 128 ? 4 : 3) : 2;
+    const size_t g_stage = (size_t)T * G_TILE_BYTES, a_stage = (size_t)r_pad * (f32 ? 256 : 128);
+    size_t ring_budget = SMEM_BUDGET / per_sm - sizeof(K1Smem) - 1024;
+    // fp32: lo(G) in two stages where that leaves G two; made on chip like A
+    set.lstages = f32 && ring_budget >= 4 * g_stage + 2 * a_stage ? 2 : 1;
+    if (f32) ring_budget -= set.lstages * g_stage;
+    int astages = f32 ? (ring_budget >= 3 * g_stage + 3 * a_stage ? 3 : 2) : S > 1 ? (r_pad > 128 ? 4 : 3) : 2;
     if ((ring_budget - astages * a_stage) / g_stage < 2) astages = 2;
     astages = tune_knob("FLORA_K1_ASTAGES", astages, 1, 8);
     int gstages = (int)std::min<size_t>(8, (ring_budget - std::min(ring_budget, astages * a_stage)) / g_stage);
     gstages = tune_knob("FLORA_K1_GSTAGES", std::max(1, gstages), 1, std::max(1, gstages));
     // generator warps: 16 where one CTA owns the SM and generation is a sizeable share of the work
-    int GW = (per_sm == 1 && ratio / S > 0.15) ? 16 : 8;
+    int GW = (per_sm == 1 && (ratio / S > 0.15 || f32)) ? 16 : 8;
     GW = tune_knob("FLORA_K1_GEN_WARPS", GW, 4, per_sm == 1 ? K1_MAX_GEN_WARPS : 8);
+    if (f32 && GW != 8 && GW != 16) GW = 8;                       // (the threads divide a tile's 16-byte pieces)
     set.GW = GW;
+    set.nsets = f32 ? std::max(1, std::min(8, (per_sm == 2 ? 256 : 512) / (T * acc_cols))) : 1;
+    const int64_t max_chunk = f32 && !deterministic_flag().load() ? (int64_t)K1_F32_CHAIN_STEPS * set.nsets : (int64_t)1 << 60;
     // generator teams: as many as keep every thread of a team busy with at least one task per tile
     {
         const int tile_tasks = (S > 1 ? r_pad / S : r) * 8;
@@ -473,16 +488,18 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
         while (2 * P <= astages && GW % (2 * P) == 0 && 32 * GW / (2 * P) >= tile_tasks) P *= 2;
         P = tune_knob("FLORA_K1_TEAMS", P, 1, 8);
         while (P > 1 && (GW % P || P > astages || (P & (P - 1)))) --P;
-        set.P = P;
+        // fp32: P warps make A, the others (4 or 8: their threads times four divide a tile's 1024 pieces of 16 bytes) lo(G)
+        set.P = f32 ? tune_knob("FLORA_K1_TEAMS", GW == 8 ? 4 : r_pad > 64 ? 12 : 8, 4, 12) : P;
     }
     set.T = T;
     set.S = S;
     set.gstages = gstages;
     set.astages = astages;
-    set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + sizeof(K1Smem) + 1024;
+    set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + (f32 ? (size_t)set.lstages * g_stage : 0) + sizeof(K1Smem) + 1024;
     // column chunks: aim at about `waves` items per slot (a slot is a CTA, or a cluster), at least 8 steps each
     int64_t slots = std::max<int64_t>(1, (int64_t)sm_count() * per_sm / S);
-    if (S > 1) slots = resident_clusters<compress_tc_kernel<false>>(S, k1_threads(set.GW), set.k1_smem);
+    if (S > 1) slots = f32 ? resident_clusters<compress_tc_kernel<false, true>>(S, k1_threads(set.GW), set.k1_smem)
+                           : resident_clusters<compress_tc_kernel<false, false>>(S, k1_threads(set.GW), set.k1_smem);
     const int64_t group_tiles = (int64_t)S * T;                      // rows of one slot, in tiles
     struct Unit { int mat; int64_t tile0, tiles, kstep0, ksteps; bool direct; };
     auto build_units = [&](int64_t target, std::vector<Unit>& units, std::vector<int>& split) {
@@ -491,12 +508,12 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
         for (size_t i = 0; i < G.size(); ++i) {
             const auto& g = G[i];
             if (g.rows == 0 || g.cols == 0) continue;
-            const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + 63) / 64;
+            const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + kc - 1) / kc;
             const int64_t groups = (tiles + group_tiles - 1) / group_tiles;
             const int64_t per_group = (tiles + groups - 1) / groups;     // rows spread evenly over the groups
-            int64_t chunk = std::max<int64_t>(8, target / per_group);
+            int64_t chunk = std::min(max_chunk, std::max<int64_t>(8, target / per_group));
             int64_t nchunks = (ks + chunk - 1) / chunk;
-            if (nchunks > 1 && ks - (nchunks - 1) * chunk < chunk / 2) --nchunks;    // no short tail item
+            if (nchunks > 1 && ks - (nchunks - 1) * chunk < chunk / 2 && (ks + nchunks - 2) / (nchunks - 1) <= max_chunk) --nchunks;    // no short tail item
             chunk = (ks + nchunks - 1) / nchunks;
             nchunks = (ks + chunk - 1) / chunk;
             if (nchunks > 1) split.push_back((int)i);
@@ -849,17 +866,17 @@ inline flora_status tc_fill_matrices(TcSet& set, const std::vector<flora_mat>& G
         tm.m = (int32_t)std::max(G.empty() ? (int64_t)0 : G[i].cols, W.empty() ? (int64_t)0 : W[i].cols);
         if (!G.empty() && G[i].rows && G[i].cols && !make_map(&tm.map_g, G[i])) return FLORA_ERR_CUDA;
         if (!W.empty() && W[i].rows && W[i].cols && !make_map(&tm.map_w, W[i])) return FLORA_ERR_CUDA;
-        if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !make_map_f32(&tm.map_s, S[i])) return FLORA_ERR_CUDA;
+        if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !make_map(&tm.map_s, S[i])) return FLORA_ERR_CUDA;
     }
     return FLORA_OK;
 }
 
 // What the TMA kernels can take of a set: the matrix has their type, size and alignment, and its sketch's rows can be addressed.
-inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S)
+inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool f32 = false)
 {
     std::vector<uint8_t> ok(big.size(), 0);
     if (encode_tiled_fn())
-        for (size_t i = 0; i < big.size(); ++i) ok[i] = tc_mat_ok(big[i]) && tc_sketch_ok(S[i]);
+        for (size_t i = 0; i < big.size(); ++i) ok[i] = (f32 ? tc_f32_ok(big[i]) : tc_mat_ok(big[i])) && tc_sketch_ok(S[i]);
     return ok;
 }
 
@@ -950,7 +967,7 @@ inline flora_status tc_set_rebind(TcSet& set, const std::vector<flora_mat>& G, c
 {
     if (!set.compress_ready) return FLORA_OK;
     for (int i : set.members)
-        if (!tc_mat_ok(G[i])) return FLORA_ERR_ALIGN;
+        if (!(set.f32 ? tc_f32_ok(G[i]) : tc_mat_ok(G[i]))) return FLORA_ERR_ALIGN;
     for (int i : set.members) {
         if (G[i].rows && G[i].cols && !make_map(&set.h_mats[i].map_g, G[i])) return FLORA_ERR_CUDA;
     }
@@ -1003,7 +1020,9 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
         }
         if (scale_all) b = 1.0f;
     }
-    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE>>() : raise_smem_limit<compress_tc_kernel<SINGLE>>())) return FLORA_ERR_CUDA;
+    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE>>()
+               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false>>()))
+        return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k1_launch_begin.size(); ++l) {
         const int begin = set.k1_launch_begin[l], end = set.k1_launch_begin[l + 1];
         if (end == begin) continue;
@@ -1035,8 +1054,11 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
             e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE>, mats, one, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
                                    set.astages, set.S, set.GW, lw);
         } else {
-            e = cudaLaunchKernelEx(&cfg, compress_tc_kernel<SINGLE>, mats, one, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.S,
-                                   set.GW, set.P, lw);
+            auto go = [&](auto kernel) {
+                return cudaLaunchKernelEx(&cfg, kernel, mats, one, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.lstages,
+                                          set.nsets, set.S, set.GW, set.P, lw);
+            };
+            e = set.f32 ? go(compress_tc_kernel<SINGLE, true>) : go(compress_tc_kernel<SINGLE, false>);
         }
         if (e != cudaSuccess) return FLORA_ERR_CUDA;
         launches.fetch_add(1, std::memory_order_relaxed);
@@ -1057,11 +1079,11 @@ inline flora_status tc_set_compress(const TcSet& set, const uint64_t* seeds, flo
 // plans once per shape (a cache keyed by addresses planned every call anew in such loops: 43 us each).  Calls that use the
 // cache are serialised by its mutex; a plan is built with a synchronous upload, so any stream may use it afterwards.
 struct SinglePlanKey {
-    int dev, kind, r, det;
+    int dev, kind, r, det, dtype;
     int64_t rows, cols;
     bool operator==(const SinglePlanKey& o) const
     {
-        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && rows == o.rows && cols == o.cols;
+        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && dtype == o.dtype && rows == o.rows && cols == o.cols;
     }
 };
 struct SinglePlan {
@@ -1089,6 +1111,7 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
     key.kind = kind;
     key.r = (int)sketch.cols;
     key.det = deterministic_flag().load();
+    key.dtype = big.dtype;
     key.rows = big.rows;
     key.cols = big.cols;
     for (size_t i = 0; i < cache.size(); ++i)
@@ -1142,7 +1165,7 @@ inline bool single_record(TcMatrix* tm, const flora_mat& big, const flora_mat& s
     tm->lds = sketch.ld;
     tm->n = (int32_t)big.rows;
     tm->m = (int32_t)big.cols;
-    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && make_map_f32(&tm->map_s, sketch);
+    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && make_map(&tm->map_s, sketch);
 }
 
 inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, float a, float b, cudaStream_t st,

@@ -77,3 +77,28 @@ def test_mixed_sets(r):
     assert all(bool(torch.all(s == 0)) for s in S)
     fset.close()
     assert fb.flora_device_status() == 0
+
+
+# fp32 matrices that the TMA compression takes (too wide or too large for the kernels above): rows and columns around a tile and a
+# step, ranks around where A stops fitting one operand (128 | 129) and where two tiles share it (32 | 33), one item and several per
+# accumulator set.  The bound is a third of the tolerance: hi/lo products carry 2^-22, and at most 192 truncated accumulations
+# (2e-8 of the running sum each, growing with the sum as its square root) stay under 3e-6.
+@pytest.mark.parametrize("n,m,r", [(128, 3104, 8), (257, 5000, 33), (130, 8196, 130), (385, 4100, 256), (2049, 2052, 96), (4096, 3076, 17), (129, 16380, 64),
+                                   (300, 3300, 128)])
+def test_fp32_through_tma(n, m, r):
+    G = wl.gaussian_matrix(n, m, 1e-2, "f32", 9).to(DEV)
+    S = torch.randn(n, r, device=DEV)
+    S0 = S.clone()
+    fb.flora_compress_accumulate(G, S, 31, r)
+    A = torch.empty(r, m, device=DEV)
+    fb.flora_materialize_A(A, 31)
+    product = G.double() @ A.double().T
+    assert ((S.double() - S0.double() - product).abs().max() / product.abs().max()).item() <= 3.3e-6 + 2.0 ** -22
+    fset = fb.FloraSet([torch.zeros_like(G), G[:, : m - 4].contiguous()], None, [S, S0])
+    fset.rebind_gradients([G, G[:, : m - 4].contiguous()])
+    S.fill_(float("nan"))
+    fset.compress_overwrite([32, 33])
+    fset.momentum_step(0.5, [32, 33])
+    assert rel_err(S.cpu().numpy(), oracle_compress(G, torch.zeros_like(S), 32)) <= TOL["f32"]
+    fset.close()
+    assert fb.flora_device_status() == 0
