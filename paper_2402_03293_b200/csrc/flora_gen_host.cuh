@@ -347,16 +347,25 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         const int64_t share = std::max<int64_t>(2, total / (per_sm * sms * 3));
         std::vector<int> split(big.size(), 1);
         int cluster = 1;
-        for (int i : ids) {
-            const int64_t steps = (big[i].cols + K - 1) / K;
-            while (split[i] < 8 && (steps > share * split[i] * 3 / 2 || (s.f32 && steps > (int64_t)GEN_F32_CHAIN_STEPS * split[i])) && steps >= 2 * split[i])
-                split[i] *= 2;
-            cluster = std::max(cluster, split[i]);
-        }
+        auto cut_columns = [&](int most) {       // CTAs along the columns per matrix, and clusters that makes
+            cluster = 1;
+            for (int i : ids) {
+                const int64_t steps = (big[i].cols + K - 1) / K;
+                split[i] = 1;
+                while (split[i] < most && (steps > share * split[i] * 3 / 2 || (s.f32 && steps > (int64_t)GEN_F32_CHAIN_STEPS * split[i])) && steps >= 2 * split[i])
+                    split[i] *= 2;
+                cluster = std::max(cluster, split[i]);
+            }
+            int64_t clusters = 0;
+            for (int i : ids) clusters += ((big[i].rows + 127) / 128 + cluster / split[i] - 1) / (cluster / split[i]);
+            return clusters;
+        };
+        // clusters of sixteen (not portable: they need a whole GPC's SMs) only where all of them are resident at once
+        s.plan.workers = per_sm == 2 ? 8 : 16;
+        if (cut_columns(GEN_MAX_SPLIT) > gen_k1_resident(s.plan, cluster) || cluster <= 8) cut_columns(8);
         const int T = 1;
         if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
-        s.plan.workers = per_sm == 2 ? 8 : 16;
         for (int i : ids) {
             const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = (int64_t)(cluster / split[i]) * T;
             for (int64_t t0 = 0; t0 < tiles; t0 += per)

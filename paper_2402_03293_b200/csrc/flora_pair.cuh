@@ -48,9 +48,9 @@ struct PairSmem {
 // A CTA of rank q in its cluster belongs to pair q / 2 and holds half h = q % 2 of every A tile: rows
 // [h N/2, (h+1) N/2).  Of that half it generates the rows [pair * N/S, (pair+1) * N/S) and receives the rest from
 // the CTAs of the same parity.  The even CTA of a pair (the leader) issues the MMAs for both.
-template <bool SINGLE>
+template <bool SINGLE, int MAPS>
 __global__ void __launch_bounds__(PAIR_MAX_THREADS, 1)
-compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K1Item* __restrict__ items, const int* __restrict__ slot_begin,
+compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const int* __restrict__ slot_begin,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, int N, float scale, float a, float b, int gstages,
                      int astages, int S, int GW, int late_wait)
 {
@@ -125,7 +125,9 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             for (int u = u_begin; u < u_end && ok; ++u) {
                 const K1Item item = items[(size_t)u * S + rank];
                 const TcMatrix* mat = mats + item.mat;
-                if (item.tiles > 0) ptx::prefetch_tensormap(&mat->map_g);
+                const CUtensorMap* map_g = &mat->map_g;
+                if constexpr (MAPS > 0) map_g = &gmaps.m[item.mat - seed_base];
+                if (item.tiles > 0) ptx::prefetch_tensormap(map_g);
                 for (int ks = 0; ks < item.ksteps; ++ks, ++g, pg.advance(gstages), pp.advance(PAIR_RELAY_DEPTH)) {
                     const int s = pg.s;
                     ok = ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->empty_g[s]), (pg.wraps & 1u) ^ 1u, abort);
@@ -135,7 +137,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                     if (item.tiles > 0) {
                         ptx::mbar_arrive_expect_tx(bar, (uint32_t)item.tiles * G_TILE_BYTES);
                         for (int t = 0; t < item.tiles; ++t)
-                            ptx::tma_load_2d(smem_base + s * g_bytes + t * G_TILE_BYTES, &mat->map_g, (item.kstep0 + ks) * 64, item.row0 + t * 128, bar);
+                            ptx::tma_load_2d(smem_base + s * g_bytes + t * G_TILE_BYTES, map_g, (item.kstep0 + ks) * 64, item.row0 + t * 128, bar);
                     } else {
                         ptx::mbar_arrive(bar);                                   // a CTA without rows loads nothing
                     }

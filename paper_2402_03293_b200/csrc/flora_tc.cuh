@@ -69,6 +69,18 @@ struct RingPos {
     }
 };
 
+// Tensor maps of gradients that were re-pointed since the set was made: they travel with the launch, by value, instead of by a copy
+// into the device table (a 30 KB copy from pageable memory between two kernels cost 8 us per micro-step on 48 matrices and kept the
+// second kernel from starting early; 6 KB of parameters add about one microsecond of host time, which the GPU does not see).
+template <int MAPS>
+struct alignas(64) GMaps {
+    CUtensorMap m[MAPS];
+};
+template <>
+struct GMaps<0> {
+};
+constexpr int GMAPS_FEW = 48, GMAPS_MANY = 192;      // (192 maps and the seeds stay below the 32 KB that a launch can carry)
+
 constexpr int SEEDS_PER_LAUNCH = 448;
 struct SeedTable {
     uint64_t s[SEEDS_PER_LAUNCH];
@@ -107,12 +119,12 @@ struct K1Smem {                            // barriers and scalars, placed after
 // turn, the planner caps the steps of an item, and the parts are added up in rounded fp32 at the end.  What bounds a step then: the 16 KB of a tile from HBM (700 cycles of an SM's share) against 130 cycles of issue slots
 // for its lo(G), 11 r cycles for A and 400 of tensor pipe; the kernel that cut fp32 into three bf16 parts out of registers spent
 // 670 issue cycles on a tile.
-// SINGLE: one matrix, its record passed by value (every item names matrix 0).
+// SINGLE: one matrix, its record passed by value (every item names matrix 0).  MAPS: the gradients' maps come with the launch.
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
 // 4096 x 11008 matrix takes 27 us instead of 20)
-template <bool SINGLE, bool F32>
+template <bool SINGLE, bool F32, int MAPS>
 __global__ void __maxnreg__(80)
-compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
+compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
                    int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int lstages, int nsets, int S, int GW, int P,
                    int late_wait)
 {
@@ -135,6 +147,8 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
 
     const K1Item item = items[blockIdx.x];                    // tables and descriptors are written at set creation, not by kernels
     const TcMatrix* mat = SINGLE ? &single : table + item.mat;
+    const CUtensorMap* map_g = &mat->map_g;
+    if constexpr (MAPS > 0) map_g = &gmaps.m[item.mat - seed_base];
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < T * acc_cols * (F32 ? nsets : 1)) tmem_cols <<= 1;
 
@@ -190,7 +204,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0 && item.tiles > 0) {
-            ptx::prefetch_tensormap(&mat->map_g);
+            ptx::prefetch_tensormap(map_g);
             int issued = 0;
             RingPos pg;
             for (int ks = 0; ks < item.ksteps; ++ks, pg.advance(gstages)) {
@@ -199,7 +213,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                 const uint32_t bar = ptx::smem_addr(&ctl->full_g[s]);
                 ptx::mbar_arrive_expect_tx(bar, (uint32_t)item.tiles * G_TILE_BYTES);
                 for (int t = 0; t < item.tiles; ++t)
-                    ptx::tma_load_2d(smem_base + s * g_bytes + t * G_TILE_BYTES, &mat->map_g, (item.kstep0 + ks) * KC, item.row0 + t * 128, bar);
+                    ptx::tma_load_2d(smem_base + s * g_bytes + t * G_TILE_BYTES, map_g, (item.kstep0 + ks) * KC, item.row0 + t * 128, bar);
                 issued = ks + 1;
             }
             if (*abort) {

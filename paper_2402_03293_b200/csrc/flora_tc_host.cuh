@@ -36,6 +36,7 @@ struct TcSet {
     K1Item* d_k1 = nullptr;
     int* d_split = nullptr;
     std::vector<TcMatrix> h_mats;
+    std::vector<CUtensorMap> g_maps;    // maps of re-pointed gradients (empty: the table's are valid)
     std::vector<K1Item> h_k1;
     std::vector<int> k1_launch_begin;   // item ranges per launch (at most SEEDS_PER_LAUNCH matrices each)
     std::vector<int> split_mats;        // matrices whose sketch is updated by several items
@@ -284,7 +285,7 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
     set.gstages = gstages;
     set.astages = astages;
     set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + staging + sizeof(PairSmem) + 1024;
-    const int64_t slots = resident_clusters<compress_pair_kernel<false>>(S, pair_threads(GW), set.k1_smem);
+    const int64_t slots = resident_clusters<compress_pair_kernel<false, 0>>(S, pair_threads(GW), set.k1_smem);
     const int64_t group_tiles = (int64_t)S * T;
     struct Unit { int mat; int64_t tile0, tiles, kstep0, ksteps; bool direct; };
     auto build_units = [&](int64_t target, std::vector<Unit>& units, std::vector<int>& split) {
@@ -498,8 +499,8 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + (f32 ? (size_t)set.lstages * g_stage : 0) + sizeof(K1Smem) + 1024;
     // column chunks: aim at about `waves` items per slot (a slot is a CTA, or a cluster), at least 8 steps each
     int64_t slots = std::max<int64_t>(1, (int64_t)sm_count() * per_sm / S);
-    if (S > 1) slots = f32 ? resident_clusters<compress_tc_kernel<false, true>>(S, k1_threads(set.GW), set.k1_smem)
-                           : resident_clusters<compress_tc_kernel<false, false>>(S, k1_threads(set.GW), set.k1_smem);
+    if (S > 1) slots = f32 ? resident_clusters<compress_tc_kernel<false, true, 0>>(S, k1_threads(set.GW), set.k1_smem)
+                           : resident_clusters<compress_tc_kernel<false, false, 0>>(S, k1_threads(set.GW), set.k1_smem);
     const int64_t group_tiles = (int64_t)S * T;                      // rows of one slot, in tiles
     struct Unit { int mat; int64_t tile0, tiles, kstep0, ksteps; bool direct; };
     auto build_units = [&](int64_t target, std::vector<Unit>& units, std::vector<int>& split) {
@@ -962,16 +963,18 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_
     return FLORA_OK;
 }
 
-// New gradient pointers, same shapes: only the tensor maps change.
+// New gradient pointers, same shapes: only the tensor maps change.  They are kept on the host and travel with the next launches;
+// sets of more matrices than a launch can carry maps for get them copied into their table.
 inline flora_status tc_set_rebind(TcSet& set, const std::vector<flora_mat>& G, cudaStream_t st)
 {
     if (!set.compress_ready) return FLORA_OK;
     for (int i : set.members)
         if (!(set.f32 ? tc_f32_ok(G[i]) : tc_mat_ok(G[i]))) return FLORA_ERR_ALIGN;
-    for (int i : set.members) {
-        if (G[i].rows && G[i].cols && !make_map(&set.h_mats[i].map_g, G[i])) return FLORA_ERR_CUDA;
-    }
-    return upload(&set.d_mats, set.h_mats, st);
+    const bool carried = set.count <= GMAPS_MANY;
+    if (carried) set.g_maps.resize((size_t)set.count);
+    for (int i : set.members)
+        if (!make_map(carried ? &set.g_maps[(size_t)i] : &set.h_mats[(size_t)i].map_g, G[i])) return FLORA_ERR_CUDA;
+    return carried ? FLORA_OK : upload(&set.d_mats, set.h_mats, st);
 }
 
 // Blocks per matrix for the element-wise helper kernels (zero, scale): about four elements per thread of the
@@ -989,7 +992,7 @@ inline unsigned helper_blocks(const TcSet& set)
 // behind_own_kernel: the kernel before this call on the stream is one of the library's own that does not touch G and lets
 // its dependents start early (the transfer's apply kernel): only the write-out of the compression waits for it.
 // one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).
-template <bool SINGLE>
+template <bool SINGLE, int MAPS>
 inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, const uint64_t* seeds, float a, float b, cudaStream_t st,
                                        std::atomic<uint64_t>& launches, bool behind_own_kernel)
 {
@@ -1020,8 +1023,8 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
         }
         if (scale_all) b = 1.0f;
     }
-    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE>>()
-               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false>>()))
+    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE, MAPS>>()
+               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true, MAPS>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false, MAPS>>()))
         return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k1_launch_begin.size(); ++l) {
         const int begin = set.k1_launch_begin[l], end = set.k1_launch_begin[l + 1];
@@ -1029,6 +1032,9 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
         const int seed_base = set.k1_launch_first_mat[l];
         SeedTable table;
         for (int i = 0; i < SEEDS_PER_LAUNCH; ++i) table.s[i] = seed_base + i < set.count ? seeds[seed_base + i] : 0;
+        GMaps<MAPS> gmaps;
+        if constexpr (MAPS > 0)
+            memcpy(gmaps.m, set.g_maps.data() + seed_base, sizeof(CUtensorMap) * std::min<size_t>(MAPS, (size_t)(set.count - seed_base)));
         // the pair kernel is persistent: one cluster per slot that has work; the other kernel runs one CTA per item
         const int n_slots = pair ? set.k1_slots_begin[l + 1] - set.k1_slots_begin[l] - 1 : 0;
         cudaLaunchConfig_t cfg = {};
@@ -1051,14 +1057,14 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
         cudaError_t e;
         if (pair) {
             const int* slot_table = set.d_slots + set.k1_slots_begin[l];
-            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE>, mats, one, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
+            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE, MAPS>, mats, one, gmaps, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
                                    set.astages, set.S, set.GW, lw);
         } else {
             auto go = [&](auto kernel) {
-                return cudaLaunchKernelEx(&cfg, kernel, mats, one, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.lstages,
+                return cudaLaunchKernelEx(&cfg, kernel, mats, one, gmaps, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.lstages,
                                           set.nsets, set.S, set.GW, set.P, lw);
             };
-            e = set.f32 ? go(compress_tc_kernel<SINGLE, true>) : go(compress_tc_kernel<SINGLE, false>);
+            e = set.f32 ? go(compress_tc_kernel<SINGLE, true, MAPS>) : go(compress_tc_kernel<SINGLE, false, MAPS>);
         }
         if (e != cudaSuccess) return FLORA_ERR_CUDA;
         launches.fetch_add(1, std::memory_order_relaxed);
@@ -1069,7 +1075,9 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
 inline flora_status tc_set_compress(const TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
                                     bool behind_own_kernel = false)
 {
-    return tc_compress_launch<false>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel);
+    return set.g_maps.empty() ? tc_compress_launch<false, 0>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel)
+           : set.count <= GMAPS_FEW ? tc_compress_launch<false, GMAPS_FEW>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel)
+                                    : tc_compress_launch<false, GMAPS_MANY>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel);
 }
 
 // Plans of the single-matrix calls.  Planning (work split, device tables of the items) costs far more than a launch, and an
@@ -1176,7 +1184,7 @@ inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_
     std::lock_guard<std::mutex> lock(single_plan_mutex());
     flora_status rc;
     TcSet* set = single_plan(0, *G, *S, st, &rc);
-    return set ? tc_compress_launch<true>(*set, one, &seed, a, b, st, launches, false) : rc;
+    return set ? tc_compress_launch<true, 0>(*set, one, &seed, a, b, st, launches, false) : rc;
 }
 
 template <bool SINGLE>
