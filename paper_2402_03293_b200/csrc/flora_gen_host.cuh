@@ -360,9 +360,9 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             for (int i : ids) clusters += ((big[i].rows + 127) / 128 + cluster / split[i] - 1) / (cluster / split[i]);
             return clusters;
         };
-        // clusters of sixteen (not portable: they need a whole GPC's SMs) only where all of them are resident at once
+        // clusters of sixteen (not portable: they need a whole GPC's SMs) only where one or two waves hold all of them
         s.plan.workers = per_sm == 2 ? 8 : 16;
-        if (cut_columns(GEN_MAX_SPLIT) > gen_k1_resident(s.plan, cluster) || cluster <= 8) cut_columns(8);
+        if (cut_columns(GEN_MAX_SPLIT) > 2 * gen_k1_resident(s.plan, cluster) || cluster <= 8) cut_columns(8);
         const int T = 1;
         if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
