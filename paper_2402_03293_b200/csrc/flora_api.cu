@@ -273,17 +273,46 @@ flora_status flora_momentum_step(const flora_mat* G, flora_mat* M, float beta, u
     return simt_compress(G, M, seed, 1.0f - beta, beta, as_stream(stream));
 }
 
+// dst <- b dst + a src (A_old A_new^T); release_later: see transfer_tc.
+static flora_status single_transfer(flora_mat* dst, const flora_mat* src, int64_t m, int32_t operand, uint64_t seed_old, uint64_t seed_new, float a,
+                                    float b, void* stream, void** release_later = nullptr)
+{
+    if (release_later) *release_later = nullptr;
+    flora_status st = check_transfer(dst, src, m, operand);
+    if (st) return st;
+    if (dst->rows == 0) return FLORA_OK;
+    const int r = (int)dst->cols;
+    if (g_force_path.load() != 1 && dst->rows <= 0x7FFFFFFF && m <= 0x7FFFFFFF) {
+        std::vector<GramJob> jobs(1);
+        jobs[0] = GramJob{nullptr, (float*)dst->data, (const float*)src->data, dst->ld, src->ld, (int32_t)dst->rows, (int32_t)m, seed_old, seed_new, 0, 0};
+        return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches, nullptr, nullptr, nullptr, release_later, operand == FLORA_F32);
+    }
+    float* T = nullptr;
+    if (scratch_alloc((void**)&T, sizeof(float) * r * r, as_stream(stream)) != cudaSuccess) {
+        cudaGetLastError();
+        return FLORA_ERR_ALLOC;
+    }
+    st = transfer_with_scratch(dst, src, m, operand, seed_old, seed_new, a, b, T, as_stream(stream));
+    if (cudaFreeAsync(T, as_stream(stream)) != cudaSuccess && st == FLORA_OK) st = FLORA_ERR_CUDA;
+    return st;
+}
+
 flora_status flora_momentum_step_resampled(const flora_mat* G, flora_mat* M, float beta, uint64_t seed_old, uint64_t seed_new, void* stream)
 {
     flora_status st = check_pair(G, M);
     if (st) return st;
     if (G->rows == 0) return FLORA_OK;
-    // M <- beta (M A_old A_new^T): the transfer's own scaling; then M <- M + (1 - beta) G A_new^T, a pure accumulation
-    st = flora_transfer_axpby(M, M, G->cols, G->dtype, seed_old, seed_new, beta, 0.0f, stream);
-    if (st) return st;
-    if (G->cols > 0 && use_tc_compress(G, M)) return tc_compress_single(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
-    if (use_gen(G)) return gen_compress_single(*G, *M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
-    return simt_compress(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream));
+    // M <- beta (M A_old A_new^T): the transfer's own scaling; then M <- M + (1 - beta) G A_new^T, a pure accumulation, which goes
+    // right behind the transfer's last kernel (the scratch is handed back after both)
+    void* scratch = nullptr;
+    st = single_transfer(M, M, G->cols, G->dtype, seed_old, seed_new, beta, 0.0f, stream, &scratch);
+    if (st == FLORA_OK) {
+        if (G->cols > 0 && use_tc_compress(G, M)) st = tc_compress_single(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
+        else if (use_gen(G)) st = gen_compress_single(*G, *M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
+        else st = simt_compress(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream));
+    }
+    if (scratch && cudaFreeAsync(scratch, as_stream(stream)) != cudaSuccess && st == FLORA_OK) st = FLORA_ERR_CUDA;
+    return st;
 }
 
 flora_status flora_decompress_apply(flora_mat* W, const flora_mat* C, uint64_t seed, float lr, float scale, void* stream)
@@ -299,23 +328,7 @@ flora_status flora_decompress_apply(flora_mat* W, const flora_mat* C, uint64_t s
 flora_status flora_transfer_axpby(flora_mat* dst, const flora_mat* src, int64_t m, int32_t operand, uint64_t seed_old,
                                   uint64_t seed_new, float a, float b, void* stream)
 {
-    flora_status st = check_transfer(dst, src, m, operand);
-    if (st) return st;
-    if (dst->rows == 0) return FLORA_OK;
-    const int r = (int)dst->cols;
-    if (operand == FLORA_BF16 && g_force_path.load() != 1) {
-        std::vector<GramJob> jobs(1);
-        jobs[0] = GramJob{nullptr, (float*)dst->data, (const float*)src->data, dst->ld, src->ld, (int32_t)dst->rows, (int32_t)m, seed_old, seed_new, 0, 0};
-        if (dst->rows <= 0x7FFFFFFF && m <= 0x7FFFFFFF) return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches);
-    }
-    float* T = nullptr;
-    if (scratch_alloc((void**)&T, sizeof(float) * r * r, as_stream(stream)) != cudaSuccess) {
-        cudaGetLastError();
-        return FLORA_ERR_ALLOC;
-    }
-    st = transfer_with_scratch(dst, src, m, operand, seed_old, seed_new, a, b, T, as_stream(stream));
-    if (cudaFreeAsync(T, as_stream(stream)) != cudaSuccess && st == FLORA_OK) st = FLORA_ERR_CUDA;
-    return st;
+    return single_transfer(dst, src, m, operand, seed_old, seed_new, a, b, stream);
 }
 
 flora_status flora_resample_transfer(flora_mat* M, int64_t m, int32_t operand, uint64_t seed_old, uint64_t seed_new, void* stream)
@@ -333,12 +346,12 @@ flora_status flora_resample_transfer_static(flora_mat* M, int64_t m, int32_t ope
     float* T = nullptr;
     st = static_scratch_for_current_device(&T);
     if (st) return st;
-    // T is cleared inside (it still holds the previous call's product), then filled and applied; bf16 operands take the
-    // tensor-core kernels of flora_resample_transfer (one matrix needs no tables: its job travels as a kernel parameter)
-    if (operand == FLORA_BF16 && g_force_path.load() != 1 && M->rows <= 0x7FFFFFFF && m <= 0x7FFFFFFF) {
+    // T is cleared inside (it still holds the previous call's product), then filled and applied by the kernels of
+    // flora_resample_transfer (one matrix needs no tables: its job travels as a kernel parameter)
+    if (g_force_path.load() != 1 && M->rows <= 0x7FFFFFFF && m <= 0x7FFFFFFF) {
         std::vector<GramJob> jobs(1);
         jobs[0] = GramJob{nullptr, (float*)M->data, (const float*)M->data, M->ld, M->ld, (int32_t)M->rows, (int32_t)m, seed_old, seed_new, 0, 0};
-        return transfer_tc(jobs, (int)r, 1.0f, 0.0f, as_stream(stream), g_launches, nullptr, nullptr, T);
+        return transfer_tc(jobs, (int)r, 1.0f, 0.0f, as_stream(stream), g_launches, nullptr, nullptr, T, nullptr, operand == FLORA_F32);
     }
     return transfer_with_scratch(M, M, m, operand, seed_old, seed_new, 1.0f, 0.0f, T, as_stream(stream));
 }
@@ -497,9 +510,10 @@ static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& s
     const int r = set->r;
     float* T = nullptr;
     if (set->S.empty()) return FLORA_OK;
-    bool all_bf16 = g_force_path.load() != 1;
-    for (const auto& g : big) all_bf16 = all_bf16 && g.dtype == FLORA_BF16 && g.cols <= 0x7FFFFFFF && g.rows <= 0x7FFFFFFF;
-    if (all_bf16) {
+    const int32_t dtype = big[0].dtype;
+    bool one_kind = g_force_path.load() != 1;
+    for (const auto& g : big) one_kind = one_kind && g.dtype == dtype && g.cols <= 0x7FFFFFFF && g.rows <= 0x7FFFFFFF;
+    if (one_kind) {
         // one gram launch and one apply launch over the whole set
         std::vector<GramJob> jobs;
         for (size_t i = 0; i < set->S.size(); ++i) {
@@ -507,7 +521,8 @@ static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& s
             jobs.push_back(GramJob{nullptr, (float*)set->S[i].data, (const float*)src[i].data, set->S[i].ld, src[i].ld,
                                    (int32_t)set->S[i].rows, (int32_t)big[i].cols, seeds_old[i], seeds_new[i], (int32_t)i, 0});
         }
-        return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches, set->tc.d_mats, src_mats, nullptr, release_later);
+        return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches, set->tc.d_mats, src_mats, nullptr, release_later,
+                           dtype == FLORA_F32);
     }
     if (scratch_alloc((void**)&T, sizeof(float) * r * r, as_stream(stream)) != cudaSuccess) {
         cudaGetLastError();

@@ -1,7 +1,9 @@
 // Momentum transfer on tensor cores (Algorithm 2, resampling branch):  dst <- b dst + a src (A_old A_new^T).
 //
 //   gram_tc_kernel        T += A_old[:, k-range] A_new[:, k-range]^T   (r x r, both operands generated in shared
-//                         memory as bf16, tcgen05 MMA into tensor memory, atomic adds of the partial products)
+//                         memory as bf16, tcgen05 MMA into tensor memory; the partial products are added up in clusters,
+//                         or atomically)
+//   gram_f32_kernel       the same for fp32 operands, in fp32 arithmetic
 //   apply_gram_jobs_kernel  dst <- b dst + a src T, row block by row block, for a list of matrices
 //
 // A whole weight set is handled by one launch of each kernel over a job table that is built per call.
@@ -60,11 +62,16 @@ __device__ __forceinline__ uint32_t mask_pair(uint32_t w, int64_t col, int64_t m
     return w;
 }
 
-// SINGLE: one matrix, passed by value; CTA b takes the steps [b * per_steps, (b + 1) * per_steps) (no tables in memory).
+// SINGLE: one matrix, passed by value (no tables in memory), the steps dealt evenly to all CTAs.  The CTAs work in clusters of
+// GRAM_CLUSTER, which add up their products through distributed shared memory before anything is written: 148 CTAs that each added
+// 256 KB atomically into one r x r matrix took 40 us of a transfer at r = 256 (4096 x 11008: 76 us for both kernels before, 52 now; what
+// remains of this kernel there is 7 us of generation and 25 us of sums through distributed shared memory and L2).  parts > 0: cluster p stores its sum as the p-th of
+// `parts` matrices at T (the apply kernel adds them up; nothing is zeroed beforehand); 0: the clusters add into T.
+constexpr int GRAM_CLUSTER = 8, GRAM_MAX_PARTS = 4;
 template <bool SINGLE>
 __global__ void __launch_bounds__(GRAM_THREADS, 1)
-gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ items, const __grid_constant__ GramJob single, int per_steps,
-               int r, float scale, int kw)
+gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ items, const __grid_constant__ GramJob single, int parts,
+               int64_t part_stride, int r, float scale, int kw)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
@@ -73,14 +80,15 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
     const int halves = r_m >> 7;
     const uint32_t old_bytes = (uint32_t)r_m * 128u, new_bytes = (uint32_t)r_n * 128u;
     const uint32_t stage_bytes = old_bytes + new_bytes;
-    GramSmem* ctl = reinterpret_cast<GramSmem*>(smem_raw + (smem_base - ptx::smem_addr(smem_raw)) + 2 * (size_t)stage_bytes);
+    const uint32_t ctl_at = SINGLE ? max(2u * stage_bytes, 128u * (uint32_t)(r_n + 4) * 4u) : 2u * stage_bytes;     // (behind the staged half of T, too)
+    GramSmem* ctl = reinterpret_cast<GramSmem*>(smem_raw + (smem_base - ptx::smem_addr(smem_raw)) + ctl_at);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     GramItem item;
     if (SINGLE) {
         const int total = (single.m + kw - 1) / kw;
         item.job = 0;
-        item.kstep0 = (int)blockIdx.x * per_steps;
-        item.ksteps = min(per_steps, total - item.kstep0);
+        item.kstep0 = (int)((int64_t)blockIdx.x * total / gridDim.x);
+        item.ksteps = (int)((int64_t)(blockIdx.x + 1) * total / gridDim.x) - item.kstep0;
         item.pad = 0;
     } else {
         item = items[blockIdx.x];
@@ -114,11 +122,12 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
+    if (SINGLE) ptx::grid_launch_dependents();            // (after the allocation: see compress_tc_kernel)
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (lane == 0 && item.ksteps > 0) {
             const uint32_t idesc = ptx::umma_idesc_bf16((uint32_t)r_n);
             const uint64_t desc_base = ptx::umma_desc_k_sw128(smem_base);
             bool ok = true;
@@ -170,7 +179,8 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->full[s]));
         }
-        if (warp <= 4 && ok) {
+        if (SINGLE && item.ksteps > 0) ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl->acc_full), 0, abort);
+        if (!SINGLE && warp <= 4 && ok) {
             // read back: warp w owns tensor-memory lanes 32*(w%4) .. +31 = rows of T within a 128-row half
             const int quarter = warp & 3;
             if (ptx::mbar_wait(ptx::smem_addr(&ctl->acc_full), 0, abort)) {
@@ -200,11 +210,127 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
             }
         }
     }
+    if (SINGLE) {
+        // per 128-row half: every CTA's product -> its shared memory (over the operand stages, consumed by now), each CTA of the
+        // cluster adds up its share of the rows over all of them and writes it
+        float* const stage = reinterpret_cast<float*>(smem_raw + (smem_base - ptx::smem_addr(smem_raw)));
+        const int stride = r_n + 4;                       // an odd multiple of 16 bytes: threads of neighbouring rows write to different banks
+        const int rank = (int)ptx::cluster_ctarank();
+        float* const out = job.T + (parts > 0 ? (int64_t)(blockIdx.x / GRAM_CLUSTER) * part_stride : 0);
+        const bool vec = (r & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+        ptx::grid_dependency_wait();                      // nothing so far touched what another kernel reads or writes
+        for (int h = 0; h < halves; ++h) {
+            ptx::tc_fence_after_sync();
+            if (warp > 0) {
+                __syncwarp();
+                const int row = (warp & 3) * 32 + lane;
+                for (int j0 = ((warp - 1) >> 2) * 16; j0 < r_n; j0 += 4 * GRAM_GEN_WARPS) {
+                    uint32_t v[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) v[u] = 0u;
+                    if (item.ksteps > 0) {
+                        ptx::tmem_ld_16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + h * r_n + j0, v);
+                        ptx::tmem_ld_wait();
+                    }
+#pragma unroll
+                    for (int u = 0; u < 16; u += 4)
+                        *reinterpret_cast<float4*>(stage + row * stride + j0 + u) =
+                            make_float4(__uint_as_float(v[u]), __uint_as_float(v[u + 1]), __uint_as_float(v[u + 2]), __uint_as_float(v[u + 3]));
+                }
+            }
+            ptx::cluster_sync_some();
+            constexpr int ROWS = 128 / GRAM_CLUSTER;
+            const int rows = max(0, min(ROWS, r - (h * 128 + rank * ROWS)));
+            const uint32_t base = ptx::smem_addr(stage);
+            if (!*abort) {
+                if (vec) {
+                    const int per = r >> 2;
+                    for (int e = (int)threadIdx.x; e < rows * per; e += GRAM_THREADS) {
+                        const int i = e / per, j = (e - i * per) * 4, lr = rank * ROWS + i;
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int q = 0; q < GRAM_CLUSTER; ++q) {
+                            const float4 w = ptx::ld_cluster_v4(ptx::map_to_cta(base + (uint32_t)(lr * stride + j) * 4u, (uint32_t)q));
+                            v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+                        }
+                        float* dst = out + (int64_t)(h * 128 + lr) * r + j;
+                        if (parts > 0) *reinterpret_cast<float4*>(dst) = v;
+                        else ptx::red_add_v4(dst, v.x, v.y, v.z, v.w);
+                    }
+                } else {
+                    for (int e = (int)threadIdx.x; e < rows * r; e += GRAM_THREADS) {
+                        const int i = e / r, j = e - i * r, lr = rank * ROWS + i;
+                        float v = 0.f;
+#pragma unroll
+                        for (int q = 0; q < GRAM_CLUSTER; ++q) v += ptx::ld_cluster_f32(ptx::map_to_cta(base + (uint32_t)(lr * stride + j) * 4u, (uint32_t)q));
+                        float* dst = out + (int64_t)(h * 128 + lr) * r + j;
+                        if (parts > 0) *dst = v;
+                        else atomicAdd(dst, v);
+                    }
+                }
+            }
+            ptx::cluster_sync_some();                     // nobody writes its next half, or leaves, while a peer still reads this one
+        }
+    }
     ptx::tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem, tmem_cols);
+    }
+}
+
+// The same products for fp32 operands, in fp32 arithmetic: blockIdx.y = 32 x 32 tile of T, item (or, SINGLE, blockIdx.x) = a range of
+// columns in steps of 32.  T is zeroed beforehand.
+template <bool SINGLE>
+__global__ void __launch_bounds__(256)
+gram_f32_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ items, const __grid_constant__ GramJob single, int per_steps, int r,
+                float scale)
+{
+    __shared__ float Ao[32][33];
+    __shared__ float An[32][33];
+    GramItem item;
+    if (SINGLE) {
+        item.job = 0;
+        item.kstep0 = (int)blockIdx.x * per_steps;
+        item.ksteps = min(per_steps, (single.m + 31) / 32 - item.kstep0);
+        item.pad = 0;
+    } else {
+        item = items[blockIdx.x];
+    }
+    const GramJob job = SINGLE ? single : jobs[item.job];
+    const PhiloxKey key_old = make_key(job.seed_old), key_new = make_key(job.seed_new);
+    const int tid = threadIdx.x, tiles = (r + 31) / 32;
+    const int a0 = ((int)blockIdx.y / tiles) * 32, b0 = ((int)blockIdx.y % tiles) * 32;
+    const int ta = tid >> 3, tb = tid & 7;                 // outputs (ta, tb + 8u), u < 4
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int ks = item.kstep0; ks < item.kstep0 + item.ksteps; ++ks) {
+        {
+            const int jj = tid >> 3, qq = tid & 7;         // 32 rows x 8 quads = 256 tasks per matrix
+            const uint32_t q = (uint32_t)ks * 8u + (uint32_t)qq;
+            float v[4] = {0.0f, 0.0f, 0.0f, 0.0f}, w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if (a0 + jj < r) projection_quad(q, (uint32_t)(a0 + jj), key_old, scale, v);
+            if (b0 + jj < r) projection_quad(q, (uint32_t)(b0 + jj), key_new, scale, w);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = (int64_t)ks * 32 + qq * 4 + u < job.m;
+                Ao[jj][qq * 4 + u] = in ? v[u] : 0.0f;
+                An[jj][qq * 4 + u] = in ? w[u] : 0.0f;
+            }
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int kk = 0; kk < 32; ++kk) {
+            const float av = Ao[ta][kk];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[u] = fmaf(av, An[tb + 8 * u][kk], acc[u]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int a = a0 + ta, b = b0 + tb + 8 * u;
+        if (a < r && b < r) atomicAdd(job.T + (int64_t)a * r + b, acc[u]);
     }
 }
 
@@ -353,7 +479,7 @@ apply_gram_jobs_kernel(const GramJob* __restrict__ jobs, const __grid_constant__
 struct ApplyUnit {
     int32_t job, tp0, ntp, pad;
 };
-constexpr int APPLY_TC_THREADS = 32 * 6;    // warp 0: src loads, 1: MMA issue (leader) / relay (follower), 2-5: T^T loads and epilogue
+constexpr int APPLY_TC_THREADS = 32 * 10;   // warp 0: src loads, 1: MMA issue (leader) / relay (follower), 2-5: T^T loads and epilogue, 6-9: T^T loads
 constexpr int APPLY_TC_STAGES = 4;
 constexpr int APPLY_TC_CHUNK = 128 * 128;   // 128 rows x 32 fp32
 struct ApplyTcSmem {
@@ -378,7 +504,7 @@ template <bool SINGLE>
 __global__ void __launch_bounds__(APPLY_TC_THREADS, 1)
 apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ dst_mats, const TcMatrix* __restrict__ src_mats,
                 const ApplyUnit* __restrict__ units, const int* __restrict__ slot_begin, const __grid_constant__ ApplySingle single, int per_cluster,
-                int r, float aa, float bb)
+                int parts, int64_t part_stride, int r, float aa, float bb)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
@@ -424,7 +550,7 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
             ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[k]), 8);      // the four epilogue warps of both CTAs
             ptx::mbar_init(ptx::smem_addr(&ctl->old_full[k]), 1);
         }
-        ptx::mbar_init(ptx::smem_addr(&ctl->b_full), 8);                // the four loader warps of both CTAs
+        ptx::mbar_init(ptx::smem_addr(&ctl->b_full), 16);               // the eight loader warps of both CTAs
         ctl->abort = 0;
         ctl->epi_go = 0;
         ptx::fence_barrier_init();
@@ -445,6 +571,7 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
     // tensor memory (the compression of a resampling step does: it streams G, which this kernel does not touch, and waits itself
     // before it reads a sketch).
     ptx::grid_launch_dependents();
+    if (SINGLE) ptx::grid_dependency_wait();    // the kernel that makes T lets this one set itself up meanwhile
     if (warp == 0) {
         // ------------------------------------------------------------------ src loads: this CTA's tile, chunk by chunk
         if (lane == 0) {
@@ -542,22 +669,34 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
             // previous unit have completed: this warp has seen the accumulators of its last tile complete.
             {
                 const int vec_per_row = kchunks * 8;                     // 16-byte pieces per row
-                for (int t = tid; t < n_half * vec_per_row; t += 128) {
-                    const int bl = t / vec_per_row, v = t - bl * vec_per_row;
-                    const int b = (int)half * n_half + bl, a0 = v * 4;
-                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (b < r) {
-                        const float* src = job.T + (int64_t)b * r + a0;
-                        if (a0 + 3 < r) x = *reinterpret_cast<const float4*>(src);
-                        else {
-                            if (a0 < r) x.x = src[0];
-                            if (a0 + 1 < r) x.y = src[1];
-                            if (a0 + 2 < r) x.z = src[2];
+                const int pieces = n_half * vec_per_row;
+                // Four pieces at a time, of all parts at once: it is the latency of these loads that a cluster with one unit waits
+                // for (r = 256, one after another: 25 of the kernel's 33 us).
+                constexpr int P = SINGLE ? GRAM_MAX_PARTS : 1;
+                for (int t0 = (int)threadIdx.x - 64; t0 < pieces; t0 += 4 * 256) {
+                    float4 x[4][P];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int t = t0 + 256 * u, bl = t / vec_per_row, v = t - bl * vec_per_row;
+                        const int b = (int)half * n_half + bl, a0 = v * 4;
+#pragma unroll
+                        for (int q = 0; q < P; ++q) {            // (r is a multiple of four here: a piece is whole or beyond r)
+                            x[u][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (t < pieces && b < r && a0 < r && q < parts)
+                                x[u][q] = *reinterpret_cast<const float4*>(job.T + q * part_stride + (int64_t)b * r + a0);
                         }
                     }
-                    const int kc = v >> 3, c = v & 7;
-                    ptx::st_shared_v4(smem_base + kc * b_block + bl * 128 + ((c ^ (bl & 7)) << 4), __float_as_uint(x.x), __float_as_uint(x.y),
-                                      __float_as_uint(x.z), __float_as_uint(x.w));
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int t = t0 + 256 * u, bl = t / vec_per_row, v = t - bl * vec_per_row;
+                        const int kc = v >> 3, c = v & 7;
+                        float4 y = x[u][0];
+#pragma unroll
+                        for (int q = 1; q < P; ++q) y = make_float4(y.x + x[u][q].x, y.y + x[u][q].y, y.z + x[u][q].z, y.w + x[u][q].w);
+                        if (t < pieces)
+                            ptx::st_shared_v4(smem_base + kc * b_block + bl * 128 + ((c ^ (bl & 7)) << 4), __float_as_uint(y.x), __float_as_uint(y.y),
+                                              __float_as_uint(y.z), __float_as_uint(y.w));
+                    }
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
@@ -566,26 +705,39 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
                     else ptx::mbar_arrive_cluster_release(ptx::map_to_cta(ptx::smem_addr(&ctl->b_full), 0u));
                 }
             }
+            if (warp >= 6) {
+                // the additional loader warps follow the tiles only to know when T^T may be overwritten
+                for (int tp = 0; tp < un.ntp; ++tp, ++gt)
+                    if (ok) ok = ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->acc_full[gt & 1]), ((uint32_t)gt >> 1) & 1u, abort);
+                continue;
+            }
             for (int tp = un.tp0; tp < un.tp0 + un.ntp; ++tp, ++gt) {
                 const int row0 = (2 * tp + (int)half) * 128;
                 const bool rows = row0 < job.n;
                 const bool rmw = bb != 0.0f;
+                // old values of dst come in by TMA, up to two chunks ahead (one per staging buffer), the first two under the MMAs
+                auto request_old = [&](int c) {
+                    const uint32_t bar = ptx::smem_addr(&ctl->old_full[c & 1]);
+                    ptx::mbar_arrive_expect_tx(bar, APPLY_TC_CHUNK);
+                    ptx::tma_load_2d(staging + (uint32_t)(c & 1) * APPLY_TC_CHUNK, map_d, c * 32, row0, bar);
+                };
+                bool requested = false;
+                if (rows && leader && ok && !*abort) {
+                    ptx::tma_store_wait_read<0>();                       // both buffers have been read out by the stores of the previous tile
+                    if (rmw) {
+                        request_old(0);
+                        if (nchunks > 1) request_old(1);
+                        requested = true;
+                    }
+                }
                 if (ok) ok = ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->acc_full[gt & 1]), ((uint32_t)gt >> 1) & 1u, abort);
                 ptx::tc_fence_after_sync();
+                if (requested && (!ok || *abort)) {                      // (an abandoned tile: its copies land before this CTA leaves)
+                    volatile int late = 0;
+                    ptx::mbar_wait(ptx::smem_addr(&ctl->old_full[0]), old_use[0] & 1u, &late);
+                    if (nchunks > 1) ptx::mbar_wait(ptx::smem_addr(&ctl->old_full[1]), old_use[1] & 1u, &late);
+                }
                 if (rows) {
-                    // old values of dst come in by TMA, up to two chunks ahead (one per staging buffer)
-                    auto request_old = [&](int c) {
-                        const uint32_t bar = ptx::smem_addr(&ctl->old_full[c & 1]);
-                        ptx::mbar_arrive_expect_tx(bar, APPLY_TC_CHUNK);
-                        ptx::tma_load_2d(staging + (uint32_t)(c & 1) * APPLY_TC_CHUNK, map_d, c * 32, row0, bar);
-                    };
-                    if (leader && ok && !*abort) {
-                        ptx::tma_store_wait_read<0>();                   // both buffers have been read out by the stores of the previous tile
-                        if (rmw) {
-                            request_old(0);
-                            if (nchunks > 1) request_old(1);
-                        }
-                    }
                     for (int c = 0; c < nchunks; ++c) {
                         const uint32_t buf = staging + (uint32_t)(c & 1) * APPLY_TC_CHUNK;
                         const uint32_t brow = buf + (uint32_t)trow * 128u;
@@ -660,10 +812,47 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
 // Host side.  A set: scratch (r x r per job, job and item tables) from the stream-ordered allocator, a memset, one
 // table upload, the two kernels, the release of the scratch.  A single matrix: only the r x r scratch; the job
 // travels as a kernel parameter.  `jobs` come without T; it is assigned here.
+// Shared memory of a staged 128-row half of T (gram_tc_kernel<true>).
+inline size_t single_gram_stage(int r_n) { return (size_t)128 * (r_n + 4) * 4; }
+inline int single_gram_clusters(int r_n, size_t smem)
+{
+    static std::atomic<int> known[POOL_MAX_DEVICES][17] = {};   // (the query takes microseconds)
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::atomic<int>& k = known[dev % POOL_MAX_DEVICES][r_n / 16];
+    int n = k.load();
+    if (n == 0) k.store(n = resident_clusters<gram_tc_kernel<true>>(GRAM_CLUSTER, GRAM_THREADS, smem));
+    return n;
+}
+
+// Step width and number of clusters of the gram kernel for one matrix: the cheapest pair in microseconds.  A step costs a latency of
+// about 0.5 us and 1 us for each 640 groups of eight values (one per generating thread); clusters beyond `most_parts` (one wave at
+// most) need a zeroed T, about 2 us, and add into it, about 0.3 us each at r = 256.
+inline int plan_single_gram(int r, int m, int most, int most_parts, int* kw)
+{
+    int best_c = 1;
+    double best = 1e30;
+    for (int w = 64; w >= 16; w >>= 1) {
+        const int steps = (m + w - 1) / w;
+        const double step = 0.5 + 2.0 * r * (w / 8) / 640.0;
+        for (int c = 1; c <= most; ++c) {
+            const int per = std::max(1, (steps + c * GRAM_CLUSTER - 1) / (c * GRAM_CLUSTER));
+            const double t = per * step + (c > most_parts ? 2.0 + c * (0.3 / 65536) * r * r : 0.1 * c);
+            if (t < best) {
+                best = t;
+                best_c = c;
+                *kw = w;
+            }
+        }
+    }
+    return best_c;
+}
+
 inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
                                 const TcMatrix* d_dst_mats = nullptr, const TcMatrix* d_src_mats = nullptr, float* static_T = nullptr,
-                                void** release_later = nullptr)
+                                void** release_later = nullptr, bool f32 = false)
 {
+    // f32: fp32 operands, in fp32 arithmetic throughout (gram_f32_kernel, then the fp32 apply kernels)
     // release_later: the caller frees the call's scratch (stream-ordered) itself, after it has put more work behind the
     // last kernel; nothing then stands between that kernel and the caller's next launch
     if (release_later) *release_later = nullptr;
@@ -676,18 +865,20 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
         total_cols += j.m;
         max_n = std::max(max_n, j.n);
     }
-    int kw = 64;
-    while (kw > 16 && total_cols / kw < 4 * (int64_t)sms) kw >>= 1;
+    const bool single = jobs.size() == 1, single_gram = single && !f32;
+    int kw = f32 ? 32 : 64, gram_clusters = 0, parts = 0;
+    while (!f32 && !single && kw > 16 && total_cols / kw < 4 * (int64_t)sms) kw >>= 1;
+    const int f32_tiles = ((r + 31) / 32) * ((r + 31) / 32);             // 32 x 32 tiles of T, each with its own blocks
     int64_t total_steps = 0;
     for (const auto& j : jobs) total_steps += (j.m + kw - 1) / kw;
-    const bool single = jobs.size() == 1;
-    // a single matrix: one wave of equal chunks; a set: about three items per SM, the largest first
+    // a set: about three items per SM, the largest first
     // (deterministic mode: one CTA per matrix, so that its r x r product is summed in one fixed order)
     const int64_t chunk = deterministic_flag().load() ? std::max<int64_t>(1, total_steps)
-                          : std::max<int64_t>(1, single ? (total_steps + sms - 1) / sms : (total_steps + 3 * sms - 1) / (3 * sms));
+                          : f32 ? std::max<int64_t>(1, total_steps * f32_tiles / (16 * sms))
+                          : std::max<int64_t>(1, (total_steps + 3 * sms - 1) / (3 * sms));
     const size_t t_bytes = (((size_t)r * r * sizeof(float)) + 255) & ~(size_t)255;
     const int r_m = (r + 127) & ~127, r_n = (r + 15) & ~15;
-    const size_t smem = 2 * (size_t)(r_m + r_n) * 128 + sizeof(GramSmem) + 1024;
+    const size_t smem = std::max(2 * (size_t)(r_m + r_n) * 128 + sizeof(GramSmem), single_gram_stage(r_n) + sizeof(GramSmem)) + 1024;
     const float scale = 1.0f / sqrtf((float)r);
     const unsigned apply_threads = (unsigned)((r + 31) & ~31);        // fallback kernel: one thread per sketch column
     bool tiled = (r & 3) == 0;                                        // register-tiled kernel: 16-byte aligned rows everywhere
@@ -697,7 +888,7 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     // the tensor-core apply kernel: rows addressable by TMA, and descriptors at hand (a set's tables, or, for one
     // matrix, two maps encoded here and passed as kernel parameters)
     const bool single_job = jobs.size() == 1;
-    bool tc_apply = tiled && encode_tiled_fn() != nullptr && (single_job || (d_dst_mats && d_src_mats));
+    bool tc_apply = !f32 && tiled && encode_tiled_fn() != nullptr && (single_job || (d_dst_mats && d_src_mats));
     ApplySingle single_arg;
     memset(&single_arg, 0, sizeof(single_arg));
     if (tc_apply && single_job) {
@@ -755,7 +946,13 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
         memcpy(tables.data() + units_off, units.data(), units.size() * sizeof(ApplyUnit));
         memcpy(tables.data() + slots_off, slot_begin.data(), slot_begin.size() * sizeof(int));
     }
-    const size_t tables_off = t_bytes * jobs.size();
+    if (single_gram) {
+        const int most_parts = tc_apply && !static_T ? GRAM_MAX_PARTS : 1;
+        if (deterministic_flag().load()) gram_clusters = most_parts;         // (parts are added up in one fixed order)
+        else gram_clusters = plan_single_gram(r, jobs[0].m, single_gram_clusters(r_n, smem), most_parts, &kw);
+        if (gram_clusters <= most_parts) parts = gram_clusters;
+    }
+    const size_t tables_off = t_bytes * (parts > 1 ? (size_t)parts : jobs.size());
     uint8_t* buf = nullptr;
     if (static_T) {
         if (!single_job || !tables.empty()) return FLORA_ERR_UNSUPPORTED;      // the fixed scratch serves one matrix, without tables
@@ -766,7 +963,10 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     }
     for (size_t i = 0; i < jobs.size(); ++i) jobs[i].T = reinterpret_cast<float*>(buf + i * t_bytes);
     flora_status rc = FLORA_OK;
-    bool ok = cudaMemsetAsync(buf, 0, tables_off, st) == cudaSuccess;
+    const bool empty_T = single && jobs[0].m == 0;                       // (no columns: T = 0)
+    if (empty_T) parts = std::min(parts, 1);
+    bool ok = (parts > 0 && !empty_T) || cudaMemsetAsync(buf, 0, tables_off, st) == cudaSuccess;
+    const int apply_parts = std::max(parts, 1);
     auto launch_apply_tc = [&](const GramJob* d_jobs, const ApplyUnit* d_units, const int* d_slots) {
         if (!(single_maps ? raise_smem_limit<apply_tc_kernel<true>>() : raise_smem_limit<apply_tc_kernel<false>>())) return false;
         cudaLaunchConfig_t cfg = {};
@@ -774,20 +974,22 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
         cfg.blockDim = dim3((unsigned)APPLY_TC_THREADS);
         cfg.dynamicSmemBytes = apply_tc_smem_bytes(r);
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (one matrix: the kernel waits for the gram kernel itself)
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = single_maps ? 2 : 1;
         cudaError_t e;
         if (single_maps) {
             single_arg.job = jobs[0];
             e = cudaLaunchKernelEx(&cfg, apply_tc_kernel<true>, (const GramJob*)nullptr, (const TcMatrix*)nullptr, (const TcMatrix*)nullptr,
-                                   (const ApplyUnit*)nullptr, (const int*)nullptr, single_arg, (int)pairs_per_cluster, r, a, b);
+                                   (const ApplyUnit*)nullptr, (const int*)nullptr, single_arg, (int)pairs_per_cluster, apply_parts, (int64_t)(t_bytes / sizeof(float)), r, a, b);
         } else {
-            e = cudaLaunchKernelEx(&cfg, apply_tc_kernel<false>, d_jobs, d_dst_mats, d_src_mats, d_units, d_slots, single_arg, 0, r, a, b);
+            e = cudaLaunchKernelEx(&cfg, apply_tc_kernel<false>, d_jobs, d_dst_mats, d_src_mats, d_units, d_slots, single_arg, 0, 1, (int64_t)0, r, a, b);
         }
         launches.fetch_add(1, std::memory_order_relaxed);
         return e == cudaSuccess;
@@ -798,8 +1000,26 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
         ok = ok && raise_smem_limit<gram_tc_kernel<true>>();
         if (ok) {
             const int ks = (jobs[0].m + kw - 1) / kw;
-            if (ks > 0) {
-                gram_tc_kernel<true><<<(unsigned)((ks + chunk - 1) / chunk), GRAM_THREADS, smem, st>>>(nullptr, nullptr, jobs[0], (int)chunk, r, scale, kw);
+            if (ks > 0 && f32) {
+                gram_f32_kernel<true><<<dim3((unsigned)((ks + chunk - 1) / chunk), (unsigned)f32_tiles), 256, 0, st>>>(nullptr, nullptr, jobs[0], (int)chunk, r, scale);
+                launches.fetch_add(1, std::memory_order_relaxed);
+            } else if (ks > 0) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)(gram_clusters * GRAM_CLUSTER));
+                cfg.blockDim = dim3((unsigned)GRAM_THREADS);
+                cfg.dynamicSmemBytes = smem;
+                cfg.stream = st;
+                cudaLaunchAttribute attr[2];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim.x = (unsigned)GRAM_CLUSTER;
+                attr[0].val.clusterDim.y = 1;
+                attr[0].val.clusterDim.z = 1;
+                attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // generation needs nothing of the kernel before
+                attr[1].val.programmaticStreamSerializationAllowed = 1;
+                cfg.attrs = attr;
+                cfg.numAttrs = 2;
+                ok = cudaLaunchKernelEx(&cfg, gram_tc_kernel<true>, (const GramJob*)nullptr, (const GramItem*)nullptr, jobs[0], parts,
+                                        (int64_t)(t_bytes / sizeof(float)), r, scale, kw) == cudaSuccess;
                 launches.fetch_add(1, std::memory_order_relaxed);
             }
             const dim3 grid((unsigned)((max_n + apply_rows - 1) / apply_rows), 1);
@@ -820,7 +1040,8 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
             const GramJob* d_jobs = reinterpret_cast<const GramJob*>(buf + tables_off);
             const GramItem* d_items = reinterpret_cast<const GramItem*>(buf + tables_off + jobs_bytes);
             if (n_items) {
-                gram_tc_kernel<false><<<(unsigned)n_items, GRAM_THREADS, smem, st>>>(d_jobs, d_items, jobs[0], 0, r, scale, kw);
+                if (f32) gram_f32_kernel<false><<<dim3((unsigned)n_items, (unsigned)f32_tiles), 256, 0, st>>>(d_jobs, d_items, jobs[0], 0, r, scale);
+                else gram_tc_kernel<false><<<(unsigned)n_items, GRAM_THREADS, smem, st>>>(d_jobs, d_items, jobs[0], 0, 0, r, scale, kw);
                 launches.fetch_add(1, std::memory_order_relaxed);
             }
             if (tc_apply)

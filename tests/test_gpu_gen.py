@@ -102,3 +102,35 @@ def test_fp32_through_tma(n, m, r):
     assert rel_err(S.cpu().numpy(), oracle_compress(G, torch.zeros_like(S), 32)) <= TOL["f32"]
     fset.close()
     assert fb.flora_device_status() == 0
+
+
+# Transfers: one cluster and several, with their sums stored side by side or added into one matrix (by columns and rank), ranks below,
+# at and above one and two 128-row halves, ranks that TMA cannot address (33, 250), pairs of row tiles around 256, and two units per
+# cluster.  Against the same product in fp64, in the Frobenius norm: with bf16 operands src and T are read as tf32 (2^-11 of each value,
+# at most twice that together), through the kernels without TMA and with fp32 operands everything is fp32 (1e-5 as elsewhere).
+@pytest.mark.parametrize("n,m,r", [(1, 1, 4), (255, 63, 8), (257, 20000, 8), (300, 700, 33), (256, 4100, 64), (513, 2049, 128), (130, 9000, 132), (64, 515, 250),
+                                   (40000, 300, 16), (385, 11008, 256)])
+@pytest.mark.parametrize("operand", ["f32", "bf16"])
+def test_transfer_edges(n, m, r, operand):
+    dtype = torch.float32 if operand == "f32" else torch.bfloat16
+    A, B = torch.empty(r, m, dtype=dtype, device=DEV), torch.empty(r, m, dtype=dtype, device=DEV)
+    fb.flora_materialize_A(A, 5)
+    fb.flora_materialize_A(B, 6)
+    T = A.double() @ B.double().T
+    tol = 2.0 ** -10 + 1e-5 if operand == "bf16" and r % 4 == 0 else 1e-5
+    src, old = torch.randn(n, r, device=DEV), torch.randn(n, r, device=DEV)
+    for a, b in ((1.0, 0.0), (0.25, 0.5)):
+        dst = old.clone()
+        fb.flora_transfer_axpby(dst, src, m, operand, 5, 6, a, b)
+        want = a * (src.double() @ T) + b * old.double()
+        assert ((dst.double() - want).norm() / want.norm()).item() <= tol
+    # a set of two, and in place with the scratch fixed at load time
+    S = [src.clone(), src[:1].clone()]
+    fset = fb.FloraSet([torch.zeros(n, m, dtype=dtype, device=DEV), torch.zeros(1, m, dtype=dtype, device=DEV)], None, S)
+    fset.resample_transfer([5, 7], [6, 8])
+    fixed = src.clone()
+    fb.flora_resample_transfer_static(fixed, m, operand, 5, 6)
+    want = src.double() @ T
+    assert all(((x.double() - want).norm() / want.norm()).item() <= tol for x in (S[0], fixed))
+    fset.close()
+    assert fb.flora_device_status() == 0
