@@ -27,13 +27,11 @@
  *  - `stream` is a cudaStream_t passed as void* (NULL = the default stream).
  *    Calls are asynchronous: they enqueue work on `stream` and return; they
  *    do not synchronise the device.  One exception: the first single-matrix
- *    call that meets a new (operation, addresses, shape, rank) on the
- *    tensor-core path builds its plan (work split, TMA descriptors, a few KB
- *    of device tables, for ranks above 64 a bf16 copy of the sketch for the
- *    decompression) with a device allocation and a synchronisation of
- *    `stream`; the 32 most recent plans are kept, so a training loop pays
- *    this once per matrix.  flora_set_* calls never do: a set is planned
- *    when it is created.
+ *    call that meets a new (operation, shape, dtype, rank) on the TMA path
+ *    builds its plan (work split, a few KB of device tables) with a device
+ *    allocation and a synchronisation of `stream`; the 64 most recent plans
+ *    are kept, so a training loop pays this once per shape.  flora_set_*
+ *    calls never do: a set is planned when it is created.
  *  - Stream capture: the set-level transfers (flora_set_resample_transfer,
  *    flora_set_transfer_axpby, flora_set_momentum_step_resampled),
  *    flora_set_rebind_gradients and a single-matrix call that plans upload
@@ -133,7 +131,7 @@ flora_status flora_momentum_step_resampled(const flora_mat* G, flora_mat* M, flo
  *  - The first call on each device looks up the device address of the array (cudaGetSymbolAddress, with
  *    that device current); make that first call outside any stream capture.  Later calls only launch.
  *  - All calls on a device share the one array, and it keeps what the last call left in it.  The call clears
- *    it first (a memset on `stream`), so back-to-back calls on one stream are fine; two calls that may run
+ *    or overwrites it first (on `stream`), so back-to-back calls on one stream are fine; two calls that may run
  *    concurrently on the same GPU (different streams, different threads) race on the array and must be
  *    serialised by the caller.
  * Arguments, result and error codes are otherwise those of flora_resample_transfer. */
