@@ -27,7 +27,9 @@ namespace flora {
 constexpr int PAIR_T = 2;                   // 128-row tiles per CTA (accumulators: PAIR_T x N <= 512 tensor-memory columns)
 constexpr int PAIR_FIXED_WARPS = 4;         // single-thread roles on warps 0, 4, 8, 12: G loads; MMA issue (tile 0); slice forwarding;
                                             // MMA issue (tile 1) in the leader, relay of the step's readiness in the follower
-constexpr int PAIR_EPI_WARPS = 8;           // two groups of four: group t writes out tile t; between two units they generate too
+constexpr int PAIR_EPI_WARPS = 8;           // two for each quarter of tensor memory's lanes; between two units they generate too
+constexpr int PAIR_EPI_BUFS = 1, PAIR_PIECE_BYTES = 32 * 128;    // staging buffers of a warp: 32 rows x 32 fp32
+constexpr int PAIR_STAGING_BYTES = PAIR_EPI_WARPS * PAIR_EPI_BUFS * PAIR_PIECE_BYTES;
 constexpr int PAIR_MAX_GEN_WARPS = 16;
 constexpr int PAIR_MAX_THREADS = 32 * (PAIR_FIXED_WARPS + PAIR_MAX_GEN_WARPS + PAIR_EPI_WARPS);
 constexpr int PAIR_RELAY_DEPTH = 8;         // ring of the leader's per-step "operands ready" barriers (deeper than either tile ring)
@@ -37,7 +39,6 @@ struct PairSmem {
     uint64_t full_g[8], empty_g[8], full_a[8], slice_ready[8], empty_a[8], ready[PAIR_RELAY_DEPTH], acc_full, acc_empty;
     uint32_t tmem_base;
     int abort;
-    int epi_go[2];
     int next_item;      // generation work items handed out so far (one item = 32 tasks of one step's slice)
     int total_steps;    // 64-column steps of all units of this cluster
 };
@@ -60,8 +61,8 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     const uint32_t g_bytes = (uint32_t)PAIR_T * G_TILE_BYTES;          // one stage of the G ring
     const uint32_t a_bytes = (uint32_t)(N >> 1) * 128u;                // one stage of the A ring: this CTA's half of a tile
     const uint32_t a_ring = smem_base + (uint32_t)gstages * g_bytes;
-    const uint32_t staging = a_ring + (uint32_t)astages * a_bytes;     // two 16 KB buffers, one per epilogue group
-    PairSmem* ctl = reinterpret_cast<PairSmem*>(smem_raw + (staging - ptx::smem_addr(smem_raw)) + 2 * (size_t)S_CHUNK_BYTES_K1);
+    const uint32_t staging = a_ring + (uint32_t)astages * a_bytes;     // the epilogue warps' buffers
+    PairSmem* ctl = reinterpret_cast<PairSmem*>(smem_raw + (staging - ptx::smem_addr(smem_raw)) + PAIR_STAGING_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Roles.  A warp is served by the scheduler warp % 4 of the SM.  The four single-thread roles (warps 0, 4, 8, 12)
     // share one scheduler, which gets only three of the 24 worker warps: the thread that issues the MMAs is on the
@@ -93,7 +94,6 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
         ptx::mbar_init(ptx::smem_addr(&ctl->acc_full), 2);
         ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty), 2 * PAIR_EPI_WARPS);        // the epilogue warps of both CTAs of the pair
         ctl->abort = 0;
-        ctl->epi_go[0] = ctl->epi_go[1] = 0;
         ctl->next_item = 0;
         int steps = 0;
         for (int u = u_begin; u < u_end; ++u) steps += items[(size_t)u * S + rank].ksteps;
@@ -319,24 +319,23 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 generate(w);
             }
         } else {
-            // Epilogue: group t writes out tile t of every unit.  Warp w of a group owns tensor-memory lanes
-            // 32*(w%4) .. +31, i.e. those rows of the tile.  The accumulator leaves in chunks of 32 columns x 128 rows
-            // (16 KB): registers -> the group's staging buffer in the 128-byte-swizzled layout of the sketch's tensor map
-            // -> one bulk tensor operation, clipped by the hardware at the sketch's last row and column:
+            // Epilogue.  A warp owns tensor-memory lanes 32*(w%4) .. +31, i.e. those rows of either tile; the warps that own
+            // the same rows take the 32-column chunks of both tiles in turn.  A piece (32 rows x 32 columns) goes through
+            // the warp's own staging buffers, in the 128-byte-swizzled layout of the sketch's tensor map, and leaves by one
+            // bulk tensor operation, clipped by the hardware at the sketch's last row and column:
             //   add   S <- S + a*acc   (b == 1, or several units share the rows and S was scaled by b beforehand):
             //         a bulk reduction, nothing is read back;
             //   store S <- a*acc       (b == 0 and the unit owns its rows);
             //   rmw   S <- b*S + a*acc (the unit owns its rows): each thread reads its row's old values straight from
             //         global memory.
+            // No warp waits for another one here: with pieces of 128 rows, staged by four warps between two barriers, a chunk
+            // took 2400 cycles and a unit's write-out 11 of its 33 us (r = 256), under which no MMA can run.
             const int ew = ww - GW;
             const int grp = ew >> 2;
             const int quarter = warp & 3;
-            const bool leader = (ew & 3) == 0 && lane == 0;
-            const int trow = quarter * 32 + lane;                     // row inside a tile
-            const uint32_t bar_a = 1u + 2u * (uint32_t)grp, bar_b = bar_a + 1u;
-            const uint32_t buf = staging + (uint32_t)grp * S_CHUNK_BYTES_K1;
-            const uint32_t brow = buf + (uint32_t)trow * 128u;
+            const uint32_t bufs = staging + (uint32_t)ew * (PAIR_EPI_BUFS * PAIR_PIECE_BYTES);
             const int nchunks = (r + 31) >> 5;
+            uint32_t piece = 0;                                       // pieces this warp has written
             bool waited = !late_wait, eok = true;
             for (int u = u_begin, done = 0; u < u_end; ++u, ++done) {
                 // until the accumulators of unit u are due, help with the generation of units up to u
@@ -363,66 +362,64 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                     ptx::grid_dependency_wait();
                     waited = true;
                 }
-                if (grp < item.tiles) {
-                    const bool add = item.direct == 0 || b == 1.0f;
-                    const bool rmw = !add && b != 0.0f;
-                    const int row = item.row0 + grp * 128 + trow;
+                const bool add = item.direct == 0 || b == 1.0f;
+                const bool rmw = !add && b != 0.0f;
+                for (int i = grp; i < item.tiles * nchunks && eok && !*abort; i += PAIR_EPI_WARPS / 4) {
+                    const int t = i / nchunks, c = i - t * nchunks;
+                    const int row0 = item.row0 + t * 128 + quarter * 32, row = row0 + lane;
                     const float* old_row = mat->S + (int64_t)row * mat->lds;
                     const bool row_ok = row < mat->n;
-                    for (int c = 0; c < nchunks; ++c) {
-                        if (leader) {
-                            const bool go = eok && !*abort;
-                            if (go) ptx::tma_store_wait_read<0>();    // the previous chunk has been read out of the staging buffer
-                            ctl->epi_go[grp] = go ? 1 : 0;
-                        }
-                        ptx::named_barrier_sync(bar_a, 128);
-                        if (!*(volatile int*)&ctl->epi_go[grp]) break;      // uniform: written before the barrier by one thread
+                    const uint32_t buf = bufs + (PAIR_EPI_BUFS > 1 ? piece % PAIR_EPI_BUFS : 0u) * PAIR_PIECE_BYTES;
+                    ++piece;
 #pragma unroll
-                        for (int hc = 0; hc < 2; ++hc) {
-                            const int col0 = c * 32 + hc * 16;
-                            float o[16];
-                            if (rmw) {
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    const int col = col0 + 4 * q;
-                                    if (row_ok && col + 3 < r) {
-                                        const float4 v4 = *reinterpret_cast<const float4*>(old_row + col);
-                                        o[4 * q] = v4.x; o[4 * q + 1] = v4.y; o[4 * q + 2] = v4.z; o[4 * q + 3] = v4.w;
-                                    } else {
-#pragma unroll
-                                        for (int e = 0; e < 4; ++e) o[4 * q + e] = (row_ok && col + e < r) ? old_row[col + e] : 0.0f;
-                                    }
-                                }
-                            }
-                            uint32_t v[16];
-                            if (col0 < N) {
-                                ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + grp * N + col0, v);
-                                ptx::tmem_ld_wait();
-                            } else {
-#pragma unroll
-                                for (int k = 0; k < 16; ++k) v[k] = 0u;
-                            }
+                    for (int hc = 0; hc < 2; ++hc) {
+                        const int col0 = c * 32 + hc * 16;
+                        float o[16];
+                        if (rmw) {
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                const uint32_t addr = brow + (uint32_t)(((hc * 4 + q) ^ (trow & 7)) << 4);
-                                float x0 = a * __uint_as_float(v[4 * q]), x1 = a * __uint_as_float(v[4 * q + 1]);
-                                float x2 = a * __uint_as_float(v[4 * q + 2]), x3 = a * __uint_as_float(v[4 * q + 3]);
-                                if (rmw) {
-                                    x0 = fmaf(b, o[4 * q], x0);
-                                    x1 = fmaf(b, o[4 * q + 1], x1);
-                                    x2 = fmaf(b, o[4 * q + 2], x2);
-                                    x3 = fmaf(b, o[4 * q + 3], x3);
+                                const int col = col0 + 4 * q;
+                                if (row_ok && col + 3 < r) {
+                                    const float4 v4 = *reinterpret_cast<const float4*>(old_row + col);
+                                    o[4 * q] = v4.x; o[4 * q + 1] = v4.y; o[4 * q + 2] = v4.z; o[4 * q + 3] = v4.w;
+                                } else {
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) o[4 * q + e] = (row_ok && col + e < r) ? old_row[col + e] : 0.0f;
                                 }
-                                ptx::st_shared_v4(addr, __float_as_uint(x0), __float_as_uint(x1), __float_as_uint(x2), __float_as_uint(x3));
                             }
                         }
-                        ptx::fence_proxy_async_smem();
-                        ptx::named_barrier_sync(bar_b, 128);
-                        if (leader && !*abort) {
-                            if (add) ptx::tma_reduce_add_2d(&mat->map_s, c * 32, item.row0 + grp * 128, buf);
-                            else ptx::tma_store_2d(&mat->map_s, c * 32, item.row0 + grp * 128, buf);
-                            ptx::tma_store_commit();
+                        uint32_t v[16];
+                        if (col0 < N) {
+                            ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + t * N + col0, v);
+                            ptx::tmem_ld_wait();
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) v[k] = 0u;
                         }
+                        if (hc == 0) {                                // the buffer's last piece has been read out
+                            if (lane == 0) ptx::tma_store_wait_read<PAIR_EPI_BUFS - 1>();
+                            __syncwarp();
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint32_t addr = buf + (uint32_t)lane * 128u + (uint32_t)(((hc * 4 + q) ^ (lane & 7)) << 4);
+                            float x0 = a * __uint_as_float(v[4 * q]), x1 = a * __uint_as_float(v[4 * q + 1]);
+                            float x2 = a * __uint_as_float(v[4 * q + 2]), x3 = a * __uint_as_float(v[4 * q + 3]);
+                            if (rmw) {
+                                x0 = fmaf(b, o[4 * q], x0);
+                                x1 = fmaf(b, o[4 * q + 1], x1);
+                                x2 = fmaf(b, o[4 * q + 2], x2);
+                                x3 = fmaf(b, o[4 * q + 3], x3);
+                            }
+                            ptx::st_shared_v4(addr, __float_as_uint(x0), __float_as_uint(x1), __float_as_uint(x2), __float_as_uint(x3));
+                        }
+                    }
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0 && row0 < mat->n) {
+                        if (add) ptx::tma_reduce_add_2d(&mat->map_sq, c * 32, row0, buf);
+                        else ptx::tma_store_2d(&mat->map_sq, c * 32, row0, buf);
+                        ptx::tma_store_commit();
                     }
                 }
                 // this warp has read all it needs from the accumulators of this unit: tell the pair's MMA issuer
@@ -434,7 +431,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                     else ptx::mbar_arrive_cluster(ptx::map_to_cta(ebar, rank - 1));
                 }
             }
-            if (leader) ptx::tma_store_wait_all<0>();                 // the sketches are complete in global memory before the CTA ends
+            if (lane == 0) ptx::tma_store_wait_all<0>();              // the sketches are complete in global memory before the CTA ends
         }
     }
     ptx::tc_fence_before_sync();

@@ -28,6 +28,7 @@ struct alignas(128) TcMatrix {
     CUtensorMap map_g;   // gradient G, box 64 columns x 128 rows, 128-byte swizzle
     CUtensorMap map_w;   // weight W, same box (loads and stores)
     CUtensorMap map_s;   // sketch S (fp32), box 32 columns x 128 rows, 128-byte swizzle
+    CUtensorMap map_sq;  // sketch S, box 32 columns x 32 rows (what one warp of an epilogue writes), 128-byte swizzle
     CUtensorMap map_sb;  // bf16 copy of S (scratch, n x k_pad), box 64 columns x 128 rows, 128-byte swizzle
     __nv_bfloat16* Sb;   // the bf16 copy (used by the decompression kernel for ranks above 64)
     float* S;            // sketch, n x r fp32

@@ -79,14 +79,14 @@ inline EncodeTiledFn encode_tiled_fn()
 }
 
 // A matrix in boxes of 128 bytes (64 bf16 or 32 fp32 columns) x 128 rows, 128-byte swizzle, zero fill outside the matrix
-inline bool make_map(CUtensorMap* out, const flora_mat& a)
+inline bool make_map(CUtensorMap* out, const flora_mat& a, int box_rows = 128)
 {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     const bool f32 = a.dtype == FLORA_F32;
     cuuint64_t dims[2] = {(cuuint64_t)a.cols, (cuuint64_t)a.rows};
     cuuint64_t strides[1] = {(cuuint64_t)a.ld * (f32 ? 4 : 2)};
-    cuuint32_t box[2] = {f32 ? 32u : 64u, 128};
+    cuuint32_t box[2] = {f32 ? 32u : 64u, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return fn(out, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.data, dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
@@ -251,7 +251,7 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
     while (S > 2 && (int64_t)S * T > 2 * max_tiles) S >>= 1;          // not more CTAs than there are rows to share
     S = tune_knob("FLORA_K1_CLUSTER", S, 2, 8);
     if (S & (S - 1)) S = 2;
-    const size_t g_stage = (size_t)T * G_TILE_BYTES, a_stage = (size_t)(N / 2) * 128, staging = 2 * (size_t)S_CHUNK_BYTES_K1;
+    const size_t g_stage = (size_t)T * G_TILE_BYTES, a_stage = (size_t)(N / 2) * 128, staging = PAIR_STAGING_BYTES;
     const size_t ring_budget = SMEM_BUDGET - sizeof(PairSmem) - 1024 - staging;
     // A tiles are made on chip by warps that each need about two microseconds for their share of a slice, and travel
     // between the CTAs of a cluster, whose slowest member paces all: six stages keep enough slices in the making
@@ -867,7 +867,7 @@ inline flora_status tc_fill_matrices(TcSet& set, const std::vector<flora_mat>& G
         tm.m = (int32_t)std::max(G.empty() ? (int64_t)0 : G[i].cols, W.empty() ? (int64_t)0 : W[i].cols);
         if (!G.empty() && G[i].rows && G[i].cols && !make_map(&tm.map_g, G[i])) return FLORA_ERR_CUDA;
         if (!W.empty() && W[i].rows && W[i].cols && !make_map(&tm.map_w, W[i])) return FLORA_ERR_CUDA;
-        if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !make_map(&tm.map_s, S[i])) return FLORA_ERR_CUDA;
+        if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !(make_map(&tm.map_s, S[i]) && make_map(&tm.map_sq, S[i], 32))) return FLORA_ERR_CUDA;
     }
     return FLORA_OK;
 }
@@ -1173,7 +1173,7 @@ inline bool single_record(TcMatrix* tm, const flora_mat& big, const flora_mat& s
     tm->lds = sketch.ld;
     tm->n = (int32_t)big.rows;
     tm->m = (int32_t)big.cols;
-    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && make_map(&tm->map_s, sketch);
+    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && make_map(&tm->map_s, sketch) && (!is_g || make_map(&tm->map_sq, sketch, 32));
 }
 
 inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, float a, float b, cudaStream_t st,
