@@ -112,7 +112,16 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     ptx::grid_launch_dependents();          // (after the allocation of tensor memory, as in compress_tc_kernel)
     // everything above touched only shared and tensor memory; G and S may have been written by the previous kernel
     // of the stream.  `late_wait`: that kernel is this library's own pre-scaling of S, which does not touch G.
-    if (!late_wait) ptx::grid_dependency_wait();
+    if (!late_wait) {
+        if (threadIdx.x == 0 && u_begin < u_end) {              // the first tiles into L2 meanwhile, as in compress_tc_kernel
+            const K1Item item = items[(size_t)u_begin * S + rank];
+            const CUtensorMap* map_g = &mats[item.mat].map_g;
+            if constexpr (MAPS > 0) map_g = &gmaps.m[item.mat - seed_base];
+            for (int ks = 0; ks < min(item.ksteps, K1_L2_AHEAD / PAIR_T); ++ks)
+                for (int t = 0; t < item.tiles; ++t) ptx::tma_prefetch_l2_2d(map_g, (item.kstep0 + ks) * 64, item.row0 + t * 128);
+        }
+        ptx::grid_dependency_wait();
+    }
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
 

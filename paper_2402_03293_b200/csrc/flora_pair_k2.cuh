@@ -104,6 +104,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
     __syncthreads();
     ptx::cluster_sync();                    // both CTAs' barriers exist before either arrives on the other's
     ptx::tc_fence_after_sync();
+    ptx::grid_launch_dependents();          // (after the allocation of tensor memory, as in compress_tc_kernel)
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
     // tile iterations of an item, and whether this CTA has a tile in iteration p

@@ -157,6 +157,8 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // Lets the next kernel of the stream begin its own set-up as soon as resources free up.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Asks for the line that holds an address to be brought into L2.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
 // Asks for a tile to be brought into L2 (no shared memory, no barrier): a later tma_load_2d of it finds it there.
 __device__ __forceinline__ void tma_prefetch_l2_2d(const void* tmap, int x, int y)
 {

@@ -100,6 +100,8 @@ constexpr int K1_MAX_THREADS = 64 + 32 * K1_MAX_GEN_WARPS + 32;
 // threads of a CTA: producer warp, MMA warp, GW generator warps, one warp that forwards slices to cluster peers
 inline int k1_threads(int gen_warps) { return 64 + 32 * gen_warps + 32; }
 constexpr int G_TILE_BYTES = 128 * 128;   // 128 rows x 64 bf16
+// Tiles of G that a CTA asks into L2 while it waits for the kernel before it to end (128 KB: what an SM gets of HBM in 3 us).
+constexpr int K1_L2_AHEAD = 8;
 constexpr int S_CHUNK_BYTES_K1 = 128 * 128; // 128 rows x 32 fp32
 
 constexpr int K1_MAX_LSTAGES = 2;
@@ -197,7 +199,15 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     // everything above touched only this CTA's shared and tensor memory; G and S may have been written by the
     // previous kernel of the stream.  `late_wait`: that kernel is this library's own pre-scaling of S, which was
     // itself ordered after everything before it and does not touch G, so only the accesses to S need to wait
-    if (!late_wait) ptx::grid_dependency_wait();
+    if (!late_wait) {
+        // (into L2 they may come before that kernel is done: a line that it writes is changed there)
+        if (threadIdx.x == 0) {
+            const int ahead = min(item.ksteps, K1_L2_AHEAD / max(1, item.tiles));
+            for (int ks = 0; ks < ahead; ++ks)
+                for (int t = 0; t < item.tiles; ++t) ptx::tma_prefetch_l2_2d(map_g, (item.kstep0 + ks) * KC, item.row0 + t * 128);
+        }
+        ptx::grid_dependency_wait();
+    }
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
     const uint32_t rank = S > 1 ? ptx::cluster_ctarank() : 0u;
@@ -670,15 +680,28 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
+    ptx::grid_launch_dependents();          // (after the allocation of tensor memory, as in compress_tc_kernel)
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
 
+    // The slabs of A touch nothing that another kernel writes.  The two loaders wait for the kernel before this one, and meanwhile
+    // the first tiles of W come into L2; BF16S: that kernel makes the bf16 sketches and was itself launched behind all earlier
+    // work, so only the sketch loader waits.
     if (warp == 0) {
         // ------------------------------------------------------------------ W tile loads
         if (lane == 0) {
             int gt = 0, pending_from = 0;                       // tiles issued so far over all items of this CTA
             RingPos pw;
             bool ok = true;
+            int ahead = 0;
+            for (int it = blockIdx.x; !BF16S && it < n_items && ahead < slots + 2; it += gridDim.x) {
+                const K2Item item = items[it];
+                const TcMatrix* mat = mats + item.mat;
+                const int live_boxes = min(boxes, (mat->m - item.col0 + 63) >> 6);
+                for (int i = 0; i < item.tiles && ahead < slots + 2; ++i, ++ahead)
+                    for (int bx = 0; bx < live_boxes; ++bx) ptx::tma_prefetch_l2_2d(&mat->map_w, item.col0 + bx * 64, item.row0 + i * 128);
+            }
+            if (!BF16S) ptx::grid_dependency_wait();
             for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
                 const K2Item item = items[it];
                 const TcMatrix* mat = mats + item.mat;
@@ -704,6 +727,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             int gc = 0;
             RingPos pc;
             bool ok = true;
+            ptx::grid_dependency_wait();
             for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
                 const K2Item item = items[it];
                 const TcMatrix* mat = mats + item.mat;

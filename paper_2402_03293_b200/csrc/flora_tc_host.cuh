@@ -1203,6 +1203,8 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
         const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(256, ((int64_t)max_rows + 4 * rows_per_block - 1) / (4 * rows_per_block)));   // about four rows per thread
         for (int begin = 0; begin < set.count; begin += 65535) {
             dim3 grid(bx, (unsigned)std::min(65535, set.count - begin));
+            // (launched behind all earlier work: started early, beside the compression's CTAs, its blocks would crowd on the SMs that
+            // those leave free)
             sketch_to_bf16_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats + begin, one, r, k_pad);
             launches.fetch_add(1, std::memory_order_relaxed);
         }
@@ -1217,32 +1219,30 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
         SeedTable table;
         for (int i = 0; i < SEEDS_PER_LAUNCH; ++i) table.s[i] = seed_base + i < set.count ? seeds[seed_base + i] : 0;
         const int grid = std::min(set.k2_grid_max, end - begin);
-        if (set.k2_pair) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)(2 * grid));                // `grid` pairs
-            cfg.blockDim = dim3((unsigned)K2P_THREADS);
-            cfg.dynamicSmemBytes = set.k2_smem;
-            cfg.stream = st;
-            cudaLaunchAttribute attr[2];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 2;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel's sketch loader waits for its predecessor itself
-            attr[1].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 2;
-            const TcMatrix* mats = set.d_mats;
-            const K2Item* items = set.d_k2 + begin;
-            if (cudaLaunchKernelEx(&cfg, decompress_pair_kernel<SINGLE>, mats, one, items, end - begin, table, seed_base, r, scale, step, set.slots, set.cstages) !=
-                cudaSuccess)
-                return FLORA_ERR_CUDA;
-        } else if (set.k2_bf16)
-            decompress_tc_kernel<SINGLE, true><<<grid, 32 * (K2_FIXED_WARPS + set.k2_gw), set.k2_smem, st>>>(
-                set.d_mats, one, set.d_k2 + begin, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw, set.k2_nslabs);
-        else
-            decompress_tc_kernel<SINGLE, false><<<grid, 32 * (K2_FIXED_WARPS + set.k2_gw), set.k2_smem, st>>>(
-                set.d_mats, one, set.d_k2 + begin, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw, set.k2_nslabs);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(set.k2_pair ? 2 * grid : grid));       // (`grid` pairs)
+        cfg.blockDim = dim3((unsigned)(set.k2_pair ? K2P_THREADS : 32 * (K2_FIXED_WARPS + set.k2_gw)));
+        cfg.dynamicSmemBytes = set.k2_smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // the kernel's loaders wait for its predecessor themselves
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = 2;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = set.k2_pair ? 2 : 1;
+        const TcMatrix* mats = set.d_mats;
+        const K2Item* items = set.d_k2 + begin;
+        auto go = [&](auto kernel) {
+            return cudaLaunchKernelEx(&cfg, kernel, mats, one, items, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw,
+                                      set.k2_nslabs);
+        };
+        const cudaError_t e = set.k2_pair ? cudaLaunchKernelEx(&cfg, decompress_pair_kernel<SINGLE>, mats, one, items, end - begin, table, seed_base, r, scale, step,
+                                                               set.slots, set.cstages)
+                              : set.k2_bf16 ? go(decompress_tc_kernel<SINGLE, true>) : go(decompress_tc_kernel<SINGLE, false>);
+        if (e != cudaSuccess) return FLORA_ERR_CUDA;
         launches.fetch_add(1, std::memory_order_relaxed);
     }
     return cudaPeekAtLastError() == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
