@@ -14,6 +14,8 @@
 
 #include <string.h>
 
+#include <type_traits>
+
 #include <algorithm>
 #include <atomic>
 #include <vector>
@@ -250,7 +252,7 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
                         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                         for (int q = 0; q < GRAM_CLUSTER; ++q) {
-                            const float4 w = ptx::ld_cluster_v4(ptx::map_to_cta(base + (uint32_t)(lr * stride + j) * 4u, (uint32_t)q));
+                            const float4 w = ptx::ld_cluster_v4(ptx::map_to_cta(base + (uint32_t)(lr * stride + j) * 4u, (uint32_t)(q + rank) % GRAM_CLUSTER));
                             v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
                         }
                         float* dst = out + (int64_t)(h * 128 + lr) * r + j;
@@ -262,7 +264,7 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
                         const int i = e / r, j = e - i * r, lr = rank * ROWS + i;
                         float v = 0.f;
 #pragma unroll
-                        for (int q = 0; q < GRAM_CLUSTER; ++q) v += ptx::ld_cluster_f32(ptx::map_to_cta(base + (uint32_t)(lr * stride + j) * 4u, (uint32_t)q));
+                        for (int q = 0; q < GRAM_CLUSTER; ++q) v += ptx::ld_cluster_f32(ptx::map_to_cta(base + (uint32_t)(lr * stride + j) * 4u, (uint32_t)(q + rank) % GRAM_CLUSTER));
                         float* dst = out + (int64_t)(h * 128 + lr) * r + j;
                         if (parts > 0) *dst = v;
                         else atomicAdd(dst, v);
@@ -479,14 +481,13 @@ apply_gram_jobs_kernel(const GramJob* __restrict__ jobs, const __grid_constant__
 struct ApplyUnit {
     int32_t job, tp0, ntp, pad;
 };
-constexpr int APPLY_TC_THREADS = 32 * 10;   // warp 0: src loads, 1: MMA issue (leader) / relay (follower), 2-5: T^T loads and epilogue, 6-9: T^T loads
+constexpr int APPLY_TC_THREADS = 32 * 10;   // warp 0: src loads, 1: MMA issue (leader) / relay (follower), 2-9: T^T loads and epilogue
 constexpr int APPLY_TC_STAGES = 4;
 constexpr int APPLY_TC_CHUNK = 128 * 128;   // 128 rows x 32 fp32
 struct ApplyTcSmem {
-    uint64_t full_a[APPLY_TC_STAGES], empty_a[APPLY_TC_STAGES], peer_full[APPLY_TC_STAGES], acc_full[2], acc_empty[2], b_full, old_full[2];
+    uint64_t full_a[APPLY_TC_STAGES], empty_a[APPLY_TC_STAGES], peer_full[APPLY_TC_STAGES], acc_full[2], acc_empty[2], b_full;
     uint32_t tmem_base;
     int abort;
-    int epi_go;
 };
 inline size_t apply_tc_smem_bytes(int r)
 {
@@ -511,7 +512,7 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
     const int N = (r + 15) & ~15, n_half = N >> 1, kchunks = (r + 31) >> 5;
     const uint32_t b_block = (uint32_t)n_half * 128u;                    // one 32-column chunk of this CTA's half of T^T
     const uint32_t a_ring = smem_base + (uint32_t)kchunks * b_block;
-    const uint32_t staging = a_ring + APPLY_TC_STAGES * APPLY_TC_CHUNK;  // two chunk buffers of the epilogue
+    const uint32_t staging = a_ring + APPLY_TC_STAGES * APPLY_TC_CHUNK;  // the epilogue warps' buffers, 4 KB each
     ApplyTcSmem* ctl = reinterpret_cast<ApplyTcSmem*>(smem_raw + (staging - ptx::smem_addr(smem_raw)) + 2 * (size_t)APPLY_TC_CHUNK);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t half = ptx::cluster_ctarank();
@@ -547,12 +548,10 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
         }
         for (int k = 0; k < 2; ++k) {
             ptx::mbar_init(ptx::smem_addr(&ctl->acc_full[k]), 1);
-            ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[k]), 8);      // the four epilogue warps of both CTAs
-            ptx::mbar_init(ptx::smem_addr(&ctl->old_full[k]), 1);
+            ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[k]), 16);     // the eight epilogue warps of both CTAs
         }
         ptx::mbar_init(ptx::smem_addr(&ctl->b_full), 16);               // the eight loader warps of both CTAs
         ctl->abort = 0;
-        ctl->epi_go = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
     }
@@ -653,51 +652,53 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
         // ------------------------------------------------------------------ T^T loads, then the epilogue of every tile
         // Warp w owns tensor-memory lanes 32*(w%4) .. +31, i.e. those rows of the CTA's tile.
         const int quarter = warp & 3;
-        const int tid = (int)threadIdx.x - 64;                           // 0 .. 127
-        const bool leader = tid == 0;
-        const int trow = quarter * 32 + lane;
+        const int grp = warp < 6 ? 0 : 1;
+        const uint32_t buf = staging + (uint32_t)(warp - 2) * 4096u;
         const int nchunks = (r + 31) >> 5;
         bool ok = true;
         int gt = 0;                                                      // tiles done
-        uint32_t old_use[2] = {0u, 0u};                                  // how often each staging buffer has received an old chunk
         for (int u = u_begin; u < u_end; ++u) {
             const ApplyUnit un = unit_at(u);
             const GramJob job = SINGLE ? single.job : jobs[un.job];
-            const CUtensorMap* map_d = SINGLE ? &single.map_dst : &dst_mats[job.mat].map_s;
+            const CUtensorMap* map_d = SINGLE ? &single.map_dst : &dst_mats[job.mat].map_sq;
             // this CTA's half of T^T: rows [half * n_half, +n_half) of the r x r matrix job.T, as the N x K operand
             // (K-major, 128-byte swizzle, chunks of 32 columns); rows and columns beyond r are zero.  The MMAs of the
             // previous unit have completed: this warp has seen the accumulators of its last tile complete.
             {
                 const int vec_per_row = kchunks * 8;                     // 16-byte pieces per row
                 const int pieces = n_half * vec_per_row;
-                // Four pieces at a time, of all parts at once: it is the latency of these loads that a cluster with one unit waits
-                // for (r = 256, one after another: 25 of the kernel's 33 us).
-                constexpr int P = SINGLE ? GRAM_MAX_PARTS : 1;
-                for (int t0 = (int)threadIdx.x - 64; t0 < pieces; t0 += 4 * 256) {
-                    float4 x[4][P];
+                // Sixteen loads under way per thread (four parts of four pieces, or sixteen pieces): it is their latency that a cluster
+                // with one unit waits for (r = 256: one after another 25 of the kernel's 33 us, four at a time 6).
+                auto load_t = [&](auto pieces_at_once, auto parts_at_once) {
+                    constexpr int U = decltype(pieces_at_once)::value, P = decltype(parts_at_once)::value;
+                    for (int t0 = (int)threadIdx.x - 64; t0 < pieces; t0 += U * 256) {
+                        float4 x[U][P];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int t = t0 + 256 * u, bl = t / vec_per_row, v = t - bl * vec_per_row;
-                        const int b = (int)half * n_half + bl, a0 = v * 4;
+                        for (int u = 0; u < U; ++u) {
+                            const int t = t0 + 256 * u, bl = t / vec_per_row, v = t - bl * vec_per_row;
+                            const int b = (int)half * n_half + bl, a0 = v * 4;
 #pragma unroll
-                        for (int q = 0; q < P; ++q) {            // (r is a multiple of four here: a piece is whole or beyond r)
-                            x[u][q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (t < pieces && b < r && a0 < r && q < parts)
-                                x[u][q] = *reinterpret_cast<const float4*>(job.T + q * part_stride + (int64_t)b * r + a0);
+                            for (int q = 0; q < P; ++q) {        // (r is a multiple of four here: a piece is whole or beyond r)
+                                x[u][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                if (t < pieces && b < r && a0 < r && q < parts)
+                                    x[u][q] = *reinterpret_cast<const float4*>(job.T + q * part_stride + (int64_t)b * r + a0);
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const int t = t0 + 256 * u, bl = t / vec_per_row, v = t - bl * vec_per_row;
+                            const int kc = v >> 3, c = v & 7;
+                            float4 y = x[u][0];
+#pragma unroll
+                            for (int q = 1; q < P; ++q) y = make_float4(y.x + x[u][q].x, y.y + x[u][q].y, y.z + x[u][q].z, y.w + x[u][q].w);
+                            if (t < pieces)
+                                ptx::st_shared_v4(smem_base + kc * b_block + bl * 128 + ((c ^ (bl & 7)) << 4), __float_as_uint(y.x), __float_as_uint(y.y),
+                                                  __float_as_uint(y.z), __float_as_uint(y.w));
                         }
                     }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int t = t0 + 256 * u, bl = t / vec_per_row, v = t - bl * vec_per_row;
-                        const int kc = v >> 3, c = v & 7;
-                        float4 y = x[u][0];
-#pragma unroll
-                        for (int q = 1; q < P; ++q) y = make_float4(y.x + x[u][q].x, y.y + x[u][q].y, y.z + x[u][q].z, y.w + x[u][q].w);
-                        if (t < pieces)
-                            ptx::st_shared_v4(smem_base + kc * b_block + bl * 128 + ((c ^ (bl & 7)) << 4), __float_as_uint(y.x), __float_as_uint(y.y),
-                                              __float_as_uint(y.z), __float_as_uint(y.w));
-                    }
-                }
+                };
+                if (SINGLE && parts > 1) load_t(std::integral_constant<int, 4>(), std::integral_constant<int, GRAM_MAX_PARTS>());
+                else load_t(std::integral_constant<int, 16>(), std::integral_constant<int, 1>());
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -705,87 +706,50 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
                     else ptx::mbar_arrive_cluster_release(ptx::map_to_cta(ptx::smem_addr(&ctl->b_full), 0u));
                 }
             }
-            if (warp >= 6) {
-                // the additional loader warps follow the tiles only to know when T^T may be overwritten
-                for (int tp = 0; tp < un.ntp; ++tp, ++gt)
-                    if (ok) ok = ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->acc_full[gt & 1]), ((uint32_t)gt >> 1) & 1u, abort);
-                continue;
-            }
             for (int tp = un.tp0; tp < un.tp0 + un.ntp; ++tp, ++gt) {
-                const int row0 = (2 * tp + (int)half) * 128;
-                const bool rows = row0 < job.n;
-                const bool rmw = bb != 0.0f;
-                // old values of dst come in by TMA, up to two chunks ahead (one per staging buffer), the first two under the MMAs
-                auto request_old = [&](int c) {
-                    const uint32_t bar = ptx::smem_addr(&ctl->old_full[c & 1]);
-                    ptx::mbar_arrive_expect_tx(bar, APPLY_TC_CHUNK);
-                    ptx::tma_load_2d(staging + (uint32_t)(c & 1) * APPLY_TC_CHUNK, map_d, c * 32, row0, bar);
-                };
-                bool requested = false;
-                if (rows && leader && ok && !*abort) {
-                    ptx::tma_store_wait_read<0>();                       // both buffers have been read out by the stores of the previous tile
-                    if (rmw) {
-                        request_old(0);
-                        if (nchunks > 1) request_old(1);
-                        requested = true;
+                // A warp's pieces are 32 rows x 32 columns, chunks grp, grp + 2, ... of its rows, staged in its own 4 KB; no warp waits
+                // for another one.  The old values of the next piece are on their way while this one is written.
+                const int row0 = (2 * tp + (int)half) * 128 + quarter * 32, row = row0 + lane;
+                const bool rmw = bb != 0.0f, row_ok = row < job.n;
+                const float* const old_row = job.dst + (int64_t)row * job.ldd;
+                float4 old[8];
+                auto fetch_old = [&](int c) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {                        // (r is a multiple of four here)
+                        old[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (rmw && row_ok && c * 32 + 4 * q < r) old[q] = *reinterpret_cast<const float4*>(old_row + c * 32 + 4 * q);
                     }
-                }
+                };
+                fetch_old(grp);
                 if (ok) ok = ptx::mbar_wait_cluster(ptx::smem_addr(&ctl->acc_full[gt & 1]), ((uint32_t)gt >> 1) & 1u, abort);
                 ptx::tc_fence_after_sync();
-                if (requested && (!ok || *abort)) {                      // (an abandoned tile: its copies land before this CTA leaves)
-                    volatile int late = 0;
-                    ptx::mbar_wait(ptx::smem_addr(&ctl->old_full[0]), old_use[0] & 1u, &late);
-                    if (nchunks > 1) ptx::mbar_wait(ptx::smem_addr(&ctl->old_full[1]), old_use[1] & 1u, &late);
-                }
-                if (rows) {
-                    for (int c = 0; c < nchunks; ++c) {
-                        const uint32_t buf = staging + (uint32_t)(c & 1) * APPLY_TC_CHUNK;
-                        const uint32_t brow = buf + (uint32_t)trow * 128u;
-                        if (leader) {
-                            const bool go = ok && !*abort;
-                            if (go && !rmw) ptx::tma_store_wait_read<1>();   // the store of chunk c - 2 has read this buffer
-                            ctl->epi_go = go ? 1 : 0;
-                        }
-                        ptx::named_barrier_sync(1, 128);
-                        if (!*(volatile int*)&ctl->epi_go) break;         // uniform: written before the barrier by one thread
-                        uint32_t v[32];
-                        const int col0 = c * 32;
-                        if (col0 < N) ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(gt & 1) * N + col0, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
-                        if (col0 + 16 < N) ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(gt & 1) * N + col0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&v[16]));
-                        ptx::tmem_ld_wait();
-                        if (col0 + 16 >= N) {
+                for (int c = grp; c < nchunks && ok && !*abort; c += 2) {
+                    uint32_t v[32];
+                    const int col0 = c * 32;
+                    __syncwarp();
+                    ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(gt & 1) * N + col0, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
+                    if (col0 + 16 < N) ptx::tmem_ld_16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(gt & 1) * N + col0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&v[16]));
+                    ptx::tmem_ld_wait();
+                    if (col0 + 16 >= N) {
 #pragma unroll
-                            for (int k = 16; k < 32; ++k) v[k] = 0u;
-                        }
-                        if (rmw) {
-                            if (!ptx::mbar_wait(ptx::smem_addr(&ctl->old_full[c & 1]), old_use[c & 1] & 1u, abort)) ok = false;
-                            ++old_use[c & 1];
-                        }
+                        for (int k = 16; k < 32; ++k) v[k] = 0u;
+                    }
+                    if (lane == 0) ptx::tma_store_wait_read<0>();        // the piece before has been read out
+                    __syncwarp();
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const uint32_t addr = brow + (uint32_t)((q ^ (trow & 7)) << 4);
-                            float x0 = aa * __uint_as_float(v[4 * q]), x1 = aa * __uint_as_float(v[4 * q + 1]);
-                            float x2 = aa * __uint_as_float(v[4 * q + 2]), x3 = aa * __uint_as_float(v[4 * q + 3]);
-                            if (rmw) {
-                                uint32_t o0, o1, o2, o3;
-                                ptx::ld_shared_v4(addr, o0, o1, o2, o3);
-                                x0 = fmaf(bb, __uint_as_float(o0), x0);
-                                x1 = fmaf(bb, __uint_as_float(o1), x1);
-                                x2 = fmaf(bb, __uint_as_float(o2), x2);
-                                x3 = fmaf(bb, __uint_as_float(o3), x3);
-                            }
-                            ptx::st_shared_v4(addr, __float_as_uint(x0), __float_as_uint(x1), __float_as_uint(x2), __float_as_uint(x3));
-                        }
-                        ptx::fence_proxy_async_smem();
-                        ptx::named_barrier_sync(2, 128);
-                        if (leader && !*abort) {
-                            ptx::tma_store_2d(map_d, c * 32, row0, buf);
-                            ptx::tma_store_commit();
-                            if (rmw && c + 2 < nchunks) {
-                                ptx::tma_store_wait_read<0>();           // this buffer has been read out: the old chunk after next may land in it
-                                request_old(c + 2);
-                            }
-                        }
+                    for (int q = 0; q < 8; ++q) {
+                        float4 x = make_float4(aa * __uint_as_float(v[4 * q]), aa * __uint_as_float(v[4 * q + 1]), aa * __uint_as_float(v[4 * q + 2]),
+                                               aa * __uint_as_float(v[4 * q + 3]));
+                        if (rmw) x = make_float4(fmaf(bb, old[q].x, x.x), fmaf(bb, old[q].y, x.y), fmaf(bb, old[q].z, x.z), fmaf(bb, old[q].w, x.w));
+                        ptx::st_shared_v4(buf + (uint32_t)lane * 128u + (uint32_t)((q ^ (lane & 7)) << 4), __float_as_uint(x.x), __float_as_uint(x.y),
+                                          __float_as_uint(x.z), __float_as_uint(x.w));
+                    }
+                    if (c + 2 < nchunks) fetch_old(c + 2);
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0 && row0 < job.n) {
+                        ptx::tma_store_2d(map_d, c * 32, row0, buf);
+                        ptx::tma_store_commit();
                     }
                 }
                 // this warp has read all it needs from the accumulator: the MMAs of the tile after next may overwrite it
@@ -798,7 +762,7 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
                 }
             }
         }
-        if (leader) ptx::tma_store_wait_all<0>();
+        if (lane == 0) ptx::tma_store_wait_all<0>();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -893,7 +857,7 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     memset(&single_arg, 0, sizeof(single_arg));
     if (tc_apply && single_job) {
         flora_mat md{jobs[0].dst, jobs[0].n, r, jobs[0].ldd, FLORA_F32}, ms{(void*)jobs[0].src, jobs[0].n, r, jobs[0].lds, FLORA_F32};
-        tc_apply = make_map(&single_arg.map_dst, md) && make_map(&single_arg.map_src, ms);
+        tc_apply = make_map(&single_arg.map_dst, md, 32) && make_map(&single_arg.map_src, ms);
     }
     const bool single_maps = tc_apply && single_job;
     if (tc_apply)                            // the kernel wants T^T as its K-major operand: exchange the roles of the two projections
