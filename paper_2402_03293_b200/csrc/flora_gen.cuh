@@ -499,10 +499,21 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 write_rows(lr0, lr1, tile0 * 128, [&](int i, int j) {
                     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
                     const uint32_t at = sbase + (uint32_t)(i * stride + j) * 4u;
-                    for (int q = 0; q < split; ++q) {
-                        const uint32_t p = ptx::map_to_cta(at, (uint32_t)(first_rank + q));
-                        const float4 w = vec ? ptx::ld_cluster_v4(p) : make_float4(ptx::ld_cluster_f32(p), 0.f, 0.f, 0.f);
-                        v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+                    // (eight at a time under way, each CTA from its own neighbour on: it is their latency that counts)
+                    for (int q0 = 0; q0 < split; q0 += 8) {
+                        float4 w[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const int q = q0 + u + part;
+                            w[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (q0 + u < split) {
+                                const uint32_t p = ptx::map_to_cta(at, (uint32_t)(first_rank + (q < split ? q : q - split)));
+                                if (vec) w[u] = ptx::ld_cluster_v4(p);
+                                else w[u].x = ptx::ld_cluster_f32(p);
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) v = make_float4(v.x + w[u].x, v.y + w[u].y, v.z + w[u].z, v.w + w[u].w);
                     }
                     return v;
                 });
