@@ -106,8 +106,9 @@ def test_fp32_through_tma(n, m, r):
 
 # Transfers: one cluster and several, with their sums stored side by side or added into one matrix (by columns and rank), ranks below,
 # at and above one and two 128-row halves, ranks that TMA cannot address (33, 250), pairs of row tiles around 256, and two units per
-# cluster.  Against the same product in fp64, in the Frobenius norm: with bf16 operands src and T are read as tf32 (2^-11 of each value,
-# at most twice that together), through the kernels without TMA and with fp32 operands everything is fp32 (1e-5 as elsewhere).
+# cluster.  Against the same product in fp64, in the Frobenius norm: with bf16 operands src and T are read as tf32, whose ten
+# mantissa bits are cut off and not rounded (each value loses less than 2^-10 of itself, a product less than 2^-9, and one element of
+# one row can show all of it), through the kernels without TMA and with fp32 operands everything is fp32 (1e-5 as elsewhere).
 @pytest.mark.parametrize("n,m,r", [(1, 1, 4), (255, 63, 8), (257, 20000, 8), (300, 700, 33), (256, 4100, 64), (513, 2049, 128), (130, 9000, 132), (64, 515, 250),
                                    (40000, 300, 16), (385, 11008, 256)])
 @pytest.mark.parametrize("operand", ["f32", "bf16"])
@@ -117,7 +118,7 @@ def test_transfer_edges(n, m, r, operand):
     fb.flora_materialize_A(A, 5)
     fb.flora_materialize_A(B, 6)
     T = A.double() @ B.double().T
-    tol = 2.0 ** -10 + 1e-5 if operand == "bf16" and r % 4 == 0 else 1e-5
+    tol = 2.0 ** -9 + 1e-5 if operand == "bf16" and r % 4 == 0 else 1e-5
     src, old = torch.randn(n, r, device=DEV), torch.randn(n, r, device=DEV)
     for a, b in ((1.0, 0.0), (0.25, 0.5)):
         dst = old.clone()
