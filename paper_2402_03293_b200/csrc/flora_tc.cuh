@@ -935,7 +935,8 @@ template <bool SINGLE>
 __global__ void scale_sketches_kernel(const TcMatrix* __restrict__ mats, const __grid_constant__ TcMatrix single, const int* __restrict__ ids, int first, int r,
                                       float b)
 {
-    ptx::grid_launch_dependents();       // the compression kernel that follows may start streaming G right away
+    ptx::grid_launch_dependents();       // the compression kernel that follows may set up and ask for its first tiles meanwhile
+    ptx::grid_dependency_wait();
     const TcMatrix* mat = SINGLE ? &single : mats + (ids ? ids[blockIdx.y] : first + (int)blockIdx.y);
     float* S = mat->S;
     const int64_t total = (int64_t)mat->n * r;

@@ -980,6 +980,7 @@ inline flora_status tc_set_rebind(TcSet& set, const std::vector<flora_mat>& G, c
 // Blocks per matrix for the element-wise helper kernels (zero, scale): about four elements per thread of the
 // largest sketch.
 constexpr int64_t K1_SCALE_PASS_MAX_STATE_BYTES = 32ll << 20;   // sketches of a set up to this size are blended by a scaling pass (below)
+constexpr int64_t K1_EARLY_SCALE_MAX_STATE_BYTES = 16ll << 20;
 
 inline unsigned helper_blocks(int64_t most) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(1024, (most + 1023) / 1024)); }
 inline unsigned helper_blocks(const TcSet& set)
@@ -1010,7 +1011,11 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
         for (int i : set.members) state_bytes += (int64_t)set.h_mats[i].n * r * 4;
     const bool scale_all = pair && b != 0.0f && b != 1.0f && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES;
     if (scale_all || (b != 1.0f && !set.split_mats.empty())) {
-        late_wait = tune_knob("FLORA_PDL", 1, 0, 1);
+        // A short pass is itself launched early, and the compression waits for it with everything (momentum step of one 4096 x 11008
+        // matrix at r = 8 22.7 -> 21.4 us, with b = 0 22.9 -> 20.8; fp32 1024 x 4096 at r = 64 20.6 -> 18.5).  A long one starts behind
+        // all earlier work, and the compression streams G under it (42 MB of sketches: 98.4 us, 101 the other way).
+        const bool early = state_bytes <= K1_EARLY_SCALE_MAX_STATE_BYTES;
+        late_wait = early ? 0 : tune_knob("FLORA_PDL", 1, 0, 1);
         // rows that receive adds (from several CTAs, or from the pair kernel's reducing write-out): scale them by b first
         const size_t total = SINGLE ? 1 : scale_all ? set.members.size() : set.split_mats.size();
         const int* ids = scale_all ? set.d_members : set.d_split;        // (no list: every matrix of the set)
@@ -1018,7 +1023,17 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
             const size_t jobs_here = std::min<size_t>(65535, total - begin);
             // few enough blocks to be resident at once: the compression kernel may only start once all have started
             dim3 grid((unsigned)std::max<size_t>(1, std::min<size_t>(SINGLE ? helper_blocks(state_bytes / 4) : helper_blocks(set), (size_t)sm_count() * 6 / jobs_here)), (unsigned)jobs_here);
-            scale_sketches_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats, one, ids ? ids + begin : nullptr, (int)begin, r, b);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = grid;
+            cfg.blockDim = dim3(256);
+            cfg.stream = st;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = early ? 1 : 0;
+            if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<SINGLE>, (const TcMatrix*)set.d_mats, one, ids ? ids + begin : (const int*)nullptr, (int)begin, r, b) != cudaSuccess)
+                return FLORA_ERR_CUDA;
             launches.fetch_add(1, std::memory_order_relaxed);
         }
         if (scale_all) b = 1.0f;
