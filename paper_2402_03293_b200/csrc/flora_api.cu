@@ -184,7 +184,7 @@ bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
 {
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_decompress_supported(big, sketch) && 
-           !gen_decompress_quicker(big->rows * big->cols, (int)sketch->cols);
+           !gen_decompress_quicker(big->rows * big->cols, (int)sketch->cols, big->dtype == FLORA_F32);
 }
 
 }  // namespace
@@ -197,7 +197,7 @@ struct flora_set {
     int r = 0;
     bool has_G = false, has_W = false;
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
-    TcSet tcf;                     // the same for the compression of fp32 matrices
+    TcSet tcf;                     // the same for fp32 matrices
     GenSet gen_g[2], gen_w[2];     // the others, by dtype
 };
 
@@ -218,7 +218,7 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
     }
     const int r = S.empty() ? 1 : (int)S[0].cols;
     const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
-    if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) || (compression ? gen_compress_quicker(counted, widest, r, f32) : gen_decompress_quicker(counted, r)))
+    if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) || (compression ? gen_compress_quicker(counted, widest, r, f32) : gen_decompress_quicker(counted, r, f32)))
         std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
 }
@@ -233,11 +233,14 @@ static flora_status set_build(flora_set* s)
         gen_set_free(s->gen_w[d]);
     }
     std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true);
-    const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_w = set_tma_side(s->W, s->S, false);
+    const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_wf = set_tma_side(s->W, s->S, false, true);
+    std::vector<uint8_t> use_w = set_tma_side(s->W, s->S, false);
+    auto any = [](const std::vector<uint8_t>& use) { return std::find(use.begin(), use.end(), (uint8_t)1) != use.end(); };
     flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
-    if (st == FLORA_OK && std::find(use_f.begin(), use_f.end(), (uint8_t)1) != use_f.end())
-        st = tc_set_build_on(s->tcf, s->G, {}, s->S, nullptr, use_f, {});
+    if (st == FLORA_OK && (any(use_f) || any(use_wf)))
+        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, nullptr, use_f, use_wf);
     for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
+    for (size_t i = 0; i < use_w.size(); ++i) use_w[i] |= use_wf[i];
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
         std::vector<int> g, w;
         for (size_t i = 0; i < s->S.size(); ++i) {
@@ -489,6 +492,7 @@ flora_status flora_set_decompress_apply(flora_set* set, const uint64_t* seeds, f
     if (!simt) {
         flora_status st = FLORA_OK;
         if (set->tc.decompress_ready) st = tc_set_decompress(set->tc, seeds, lr * scale, as_stream(stream), g_launches);
+        if (st == FLORA_OK && set->tcf.decompress_ready) st = tc_set_decompress(set->tcf, seeds, lr * scale, as_stream(stream), g_launches);
         for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_decompress(set->gen_w[d], seeds, lr * scale, as_stream(stream), g_launches);
         if (st) return st;
     }

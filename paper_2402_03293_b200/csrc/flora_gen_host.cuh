@@ -188,10 +188,13 @@ inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32
     if (f32) return (cols <= 3072 && elements <= 5 << 19) || deterministic_flag().load();
     return cols <= 4096 && elements <= (r <= 64 ? 4 << 20 : 5 << 18);
 }
-inline bool gen_decompress_quicker(int64_t elements, int r)
+inline bool gen_decompress_quicker(int64_t elements, int r, bool f32)
 {
     const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
     if (knob >= 0) return knob == 1;
+    // (fp32, with these and with the TMA kernel: 512 x 512 at r = 8 3.8 / 4.2, 1024 x 1024 at r = 8 4.6 / 5.3, at r = 64 6.6 / 6.7, at r = 128
+    // 10.5 / 8.7, 1024 x 4096 at r = 64 15.6 / 12.0, 4096 x 11008 at r = 8 81 / 63.5)
+    if (f32) return elements <= (r <= 32 ? 1 << 20 : 1 << 19) || r > K2_F32_MAX_R;
     return elements <= (r <= 32 ? 5 << 20 : r <= 64 ? 2 << 20 : 5 << 18);
 }
 

@@ -324,7 +324,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
             const K2Item first = items[cluster];
             const int helper = ((warp >= 8 ? warp - 4 : warp - 2) << 5) + lane;           // 0 .. 255
             if (first.tiles > 0)
-                k2_generate_slab<true>(slab0, slab_block, kchunks, 64, first.col0 + 64 * (int)half, r, make_key(seeds.s[first.mat - seed_base]), scale,
+                k2_generate_slab<true, false>(slab0, slab_block, kchunks, 64, first.col0 + 64 * (int)half, r, make_key(seeds.s[first.mat - seed_base]), scale,
                                        32 * K2P_GEN_WARPS + helper, 32 * (K2P_GEN_WARPS + 8));
             ptx::fence_proxy_async_smem();
             __syncwarp();
@@ -402,7 +402,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
             ok = ptx::mbar_wait(ptx::smem_addr(&ctl->slab_empty[sb]), (((uint32_t)k >> 1) & 1u) ^ 1u, abort);
             if (!ok) break;
             if (item.tiles > 0)         // (an empty item pads a CTA's list: its slab is never read)
-                k2_generate_slab<true>(slab0 + sb * slab_bytes, slab_block, kchunks, 64, item.col0 + 64 * (int)half, r, key, scale, g,
+                k2_generate_slab<true, false>(slab0 + sb * slab_bytes, slab_block, kchunks, 64, item.col0 + 64 * (int)half, r, key, scale, g,
                                        k == 0 ? 32 * (K2P_GEN_WARPS + 8) : 32 * K2P_GEN_WARPS);      // the first slab is shared with the combine warps
             ptx::fence_proxy_async_smem();
             __syncwarp();

@@ -568,6 +568,7 @@ constexpr int K2_FIXED_WARPS = 12;  // warp 0: W loads, 1: MMA, 2-5 and 8-11: co
 constexpr int K2_MAX_GEN_WARPS = 8;
 constexpr int K2_HELPER_WARPS = 8;    // the combine warps, idle until the first tile arrives, generate part of the CTA's first slab
 constexpr int K2_MAX_THREADS = 32 * (K2_FIXED_WARPS + K2_MAX_GEN_WARPS);
+constexpr int K2_CUT_WARPS = 4, K2_LSTAGES = 2;   // fp32 W: warps that cut the sketch's chunks (behind the generators), ring of the lower parts
 constexpr int K2_MAX_SLOTS = 6;
 constexpr int K2_MAX_CSTAGES = 8;
 constexpr int W_BOX_BYTES = 128 * 128;     // 128 rows x 64 bf16
@@ -576,6 +577,7 @@ constexpr int S_CHUNK_BYTES = 128 * 128;   // 128 rows x 32 fp32
 struct K2Smem {
     uint64_t w_full[K2_MAX_SLOTS], w_free[K2_MAX_SLOTS], out_ready[K2_MAX_SLOTS];
     uint64_t c_full[K2_MAX_CSTAGES], c_empty[K2_MAX_CSTAGES], acc_full[2], acc_empty[2], slab_full[2], slab_empty[2], slab_help;
+    uint64_t l_full[K2_LSTAGES], l_empty[K2_LSTAGES];
     uint32_t tmem_base;
     int abort;
 };
@@ -583,7 +585,9 @@ struct K2Smem {
 // Writes the tasks first, first + stride, ... of one r x bn slab of A as the N x K operand: row = column of W,
 // K = index j of the sketch, values rounded to bf16 (kept in 32-bit containers, exact in tf32, for the fp32 sketch
 // path).  One task makes a 4-column x 4-j (or 8-j) block and stores one 16-byte chunk per column; j >= r is zero.
-template <bool BF16S>
+// F32: rows 0 .. bn hold A rounded to tf32, rows bn .. 2 bn what that leaves of A (exact).
+__device__ __forceinline__ uint32_t round_tf32(uint32_t x) { return (x + 0x1000u) & 0xFFFFE000u; }
+template <bool BF16S, bool F32>
 __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_block, int kchunks, int bn, int col0, int r, const PhiloxKey key,
                                                  float scale, int first, int stride)
 {
@@ -616,13 +620,23 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
                 if (j < r) projection_two_quads((uint32_t)(col0 / 4 + cq), (uint32_t)j, (uint32_t)(col0 / 4 + cq), (uint32_t)(j + 1), key, scale, v0, v1);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    v[u][jj] = bf16_round(v0[u]);
-                    v[u][jj + 1] = j + 1 < r ? bf16_round(v1[u]) : 0.0f;
+                    v[u][jj] = F32 ? v0[u] : bf16_round(v0[u]);
+                    v[u][jj + 1] = j + 1 < r ? (F32 ? v1[u] : bf16_round(v1[u])) : 0.0f;
                 }
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int c = cq * 4 + u;
+                if (F32) {
+                    uint32_t lo[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float hi = __uint_as_float(round_tf32(__float_as_uint(v[u][k])));
+                        lo[k] = __float_as_uint(v[u][k] - hi);
+                        v[u][k] = hi;
+                    }
+                    ptx::st_shared_v4(blk + (bn + c) * 128 + (((jg & 7) ^ (c & 7)) << 4), lo[0], lo[1], lo[2], lo[3]);
+                }
                 ptx::st_shared_v4(blk + c * 128 + (((jg & 7) ^ (c & 7)) << 4), __float_as_uint(v[u][0]), __float_as_uint(v[u][1]),
                                   __float_as_uint(v[u][2]), __float_as_uint(v[u][3]));
             }
@@ -630,7 +644,10 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
     }
 }
 
-template <bool SINGLE, bool BF16S>
+// F32: W is fp32.  Both operands are cut into what tf32 holds, rounded, and the rest, x = hi + lo; of the four products lo lo is left
+// out (2^-23), S_hi multiplies hi and lo of A side by side as one operand of 2 bn rows, and the small products have an accumulator to
+// themselves (the tensor core truncates its sums).  Four warps cut the sketch's chunks in shared memory.  W's boxes are 32 columns wide.
+template <bool SINGLE, bool BF16S, bool F32>
 __global__ void __launch_bounds__(K2_MAX_THREADS, 1)
 decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K2Item* __restrict__ items, int n_items,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, float scale, float step, int bn, int slots,
@@ -641,16 +658,19 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     // K chunks: one 128-byte row of S each (32 fp32 values, or 64 bf16 values when the bf16 copy of S is used)
     const int kchunks = BF16S ? (r + 63) >> 6 : (r + 31) >> 5;
-    const int boxes = bn >> 6;                                 // 64-column boxes per W tile
-    const uint32_t slab_block = (uint32_t)bn * 128u;           // one K chunk of a slab
+    constexpr int WC = F32 ? 32 : 64;                          // columns of a box of W
+    const int boxes = bn / WC;                                 // boxes per W tile
+    const uint32_t slab_block = (uint32_t)bn * (F32 ? 256u : 128u);   // one K chunk of a slab
     const uint32_t slab_bytes = kchunks * slab_block;
     const uint32_t slab0 = smem_base;
     const uint32_t c_ring = slab0 + nslabs * slab_bytes;
-    const uint32_t w_ring = c_ring + cstages * (uint32_t)S_CHUNK_BYTES;
+    const uint32_t l_ring = c_ring + cstages * (uint32_t)S_CHUNK_BYTES;
+    const uint32_t w_ring = l_ring + (F32 ? K2_LSTAGES : 0) * (uint32_t)S_CHUNK_BYTES;
     const uint32_t slot_bytes = (uint32_t)boxes * W_BOX_BYTES;
     K2Smem* ctl = reinterpret_cast<K2Smem*>(smem_raw + (w_ring - ptx::smem_addr(smem_raw)) + (size_t)slots * slot_bytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t tmem_cols = 2u * (uint32_t)bn;              // 256 or 128: a power of two >= 32
+    const int acc_cols = F32 ? 2 * bn : bn;                    // columns of one of the two accumulators
+    const uint32_t tmem_cols = 2u * (uint32_t)acc_cols;        // 256 or 128: a power of two >= 32
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < slots; ++s) {
@@ -669,6 +689,10 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             ptx::mbar_init(ptx::smem_addr(&ctl->slab_empty[s]), 1);
         }
         ptx::mbar_init(ptx::smem_addr(&ctl->slab_help), K2_HELPER_WARPS);
+        for (int s = 0; s < K2_LSTAGES; ++s) {
+            ptx::mbar_init(ptx::smem_addr(&ctl->l_full[s]), K2_CUT_WARPS);
+            ptx::mbar_init(ptx::smem_addr(&ctl->l_empty[s]), 1);
+        }
         ctl->abort = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
@@ -697,15 +721,15 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             for (int it = blockIdx.x; !BF16S && it < n_items && ahead < slots + 2; it += gridDim.x) {
                 const K2Item item = items[it];
                 const TcMatrix* mat = mats + item.mat;
-                const int live_boxes = min(boxes, (mat->m - item.col0 + 63) >> 6);
+                const int live_boxes = min(boxes, (mat->m - item.col0 + WC - 1) / WC);
                 for (int i = 0; i < item.tiles && ahead < slots + 2; ++i, ++ahead)
-                    for (int bx = 0; bx < live_boxes; ++bx) ptx::tma_prefetch_l2_2d(&mat->map_w, item.col0 + bx * 64, item.row0 + i * 128);
+                    for (int bx = 0; bx < live_boxes; ++bx) ptx::tma_prefetch_l2_2d(&mat->map_w, item.col0 + bx * WC, item.row0 + i * 128);
             }
             if (!BF16S) ptx::grid_dependency_wait();
             for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
                 const K2Item item = items[it];
                 const TcMatrix* mat = mats + item.mat;
-                const int live_boxes = min(boxes, (mat->m - item.col0 + 63) >> 6);
+                const int live_boxes = min(boxes, (mat->m - item.col0 + WC - 1) / WC);
                 for (int i = 0; i < item.tiles; ++i, ++gt, pw.advance(slots)) {
                     const int s = pw.s;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->w_free[s]), (pw.wraps & 1u) ^ 1u, abort);
@@ -713,7 +737,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                     const uint32_t bar = ptx::smem_addr(&ctl->w_full[s]);
                     ptx::mbar_arrive_expect_tx(bar, (uint32_t)live_boxes * W_BOX_BYTES);
                     for (int bx = 0; bx < live_boxes; ++bx)
-                        ptx::tma_load_2d(w_ring + s * slot_bytes + bx * W_BOX_BYTES, &mat->map_w, item.col0 + bx * 64, item.row0 + i * 128, bar);
+                        ptx::tma_load_2d(w_ring + s * slot_bytes + bx * W_BOX_BYTES, &mat->map_w, item.col0 + bx * WC, item.row0 + i * 128, bar);
                 }
             }
             if (*abort) {   // loads that nobody consumed: wait (bounded) until they have landed
@@ -752,7 +776,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             const uint32_t idesc = BF16S ? ptx::umma_idesc_bf16((uint32_t)bn) : ptx::umma_idesc_tf32((uint32_t)bn);
             const uint64_t desc_ring = ptx::umma_desc_k_sw128(c_ring);
             int gt = 0, gc = 0, k = 0;
-            RingPos pc;
+            RingPos pc, pl;
             bool ok = true;
             for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++k) {
                 const K2Item item = items[it];
@@ -762,10 +786,26 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 // the combine warps' share: of the first slab, or of every slab when there is only one buffer
                 if ((k == 0 || nslabs == 1) && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl->slab_help), k & 1, abort);
                 for (int i = 0; i < item.tiles && ok; ++i, ++gt) {
-                    const uint32_t acc_addr = tmem + (gt & 1) * bn;
+                    const uint32_t acc_addr = tmem + (gt & 1) * acc_cols;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[gt & 1]), ((gt >> 1) & 1) ^ 1, abort);
                     for (int kc = 0; kc < kchunks && ok; ++kc, ++gc, pc.advance(cstages)) {
                         const int s = pc.s;
+                        if (F32) {
+                            // (the chunk's lower part is there, so the chunk is, too)
+                            ok = ptx::mbar_wait(ptx::smem_addr(&ctl->l_full[pl.s]), pl.wraps & 1u, abort);
+                            if (!ok) break;
+                            ptx::tc_fence_after_sync();
+                            const uint64_t da = desc_ring + (uint64_t)((s * S_CHUNK_BYTES) >> 4), dl = desc_ring + (uint64_t)((l_ring - c_ring + pl.s * S_CHUNK_BYTES) >> 4);
+                            const uint64_t db = desc_slab + (uint64_t)((kc * slab_block) >> 4);
+#pragma unroll
+                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(acc_addr, da + k8 * 2, db + k8 * 2, ptx::umma_idesc_tf32(2u * bn), (kc | k8) != 0);   // hi hi | hi lo
+#pragma unroll
+                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(acc_addr + bn, dl + k8 * 2, db + k8 * 2, idesc, 1u);                                  //       | lo hi
+                            ptx::umma_commit(ptx::smem_addr(&ctl->c_empty[s]));
+                            ptx::umma_commit(ptx::smem_addr(&ctl->l_empty[pl.s]));
+                            pl.advance(K2_LSTAGES);
+                            continue;
+                        }
                         ok = ptx::mbar_wait(ptx::smem_addr(&ctl->c_full[s]), pc.wraps & 1u, abort);
                         if (!ok) break;
                         ptx::tc_fence_after_sync();
@@ -795,13 +835,13 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
                 const K2Item item = items[it];
                 const TcMatrix* mat = mats + item.mat;
-                const int live_boxes = min(boxes, (mat->m - item.col0 + 63) >> 6);
+                const int live_boxes = min(boxes, (mat->m - item.col0 + WC - 1) / WC);
                 for (int i = 0; i < item.tiles; ++i, ++gt, pw.advance(slots)) {
                     const int s = pw.s;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->out_ready[s]), pw.wraps & 1u, abort);
                     if (!ok) break;
                     for (int bx = 0; bx < live_boxes; ++bx)
-                        ptx::tma_store_2d(&mat->map_w, item.col0 + bx * 64, item.row0 + i * 128, w_ring + s * slot_bytes + bx * W_BOX_BYTES);
+                        ptx::tma_store_2d(&mat->map_w, item.col0 + bx * WC, item.row0 + i * 128, w_ring + s * slot_bytes + bx * W_BOX_BYTES);
                     ptx::tma_store_commit();
                     if (lag) {
                         // one store stays in flight: wait until all but the newest have read their slot, free that one
@@ -826,7 +866,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
         const int quarter = warp & 3;
         const int half = warp >= 8 ? 1 : 0;
         const int row = quarter * 32 + lane;
-        const int per_half = boxes << 1;                       // 16-column chunks per half: 2 (bn 64) or 4 (bn 128)
+        const int per_half = bn >> 5;                          // 16-column chunks per half: 2 (bn 64) or 4 (bn 128)
         int gt = 0;
         RingPos pw;
         bool ok = true;
@@ -840,13 +880,13 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 ok = ptx::mbar_wait(ptx::smem_addr(&ctl->slab_empty[0]), (((nslabs == 2 ? (k >> 1) : k) & 1) ^ 1), abort);
                 if (!ok) break;
                 if (item.tiles > 0)     // (an empty item pads a CTA's list: its slab is never read)
-                    k2_generate_slab<BF16S>(slab0, slab_block, kchunks, bn, item.col0, r, make_key(seeds.s[item.mat - seed_base]), scale,
+                    k2_generate_slab<BF16S, F32>(slab0, slab_block, kchunks, bn, item.col0, r, make_key(seeds.s[item.mat - seed_base]), scale,
                                             32 * GW + helper, 32 * (GW + K2_HELPER_WARPS));
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->slab_help));
             }
-            const int live_chunks = min(boxes, (mats[item.mat].m - item.col0 + 63) >> 6) << 2;
+            const int live_chunks = min(boxes, (mats[item.mat].m - item.col0 + WC - 1) / WC) * (WC / 16);
             const int c_begin = half * per_half;
             const int mine = max(0, min(per_half, live_chunks - c_begin));
             for (int i = 0; i < item.tiles; ++i, ++gt, pw.advance(slots)) {
@@ -856,10 +896,32 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t wrow = w_ring + s * slot_bytes + row * 128;
+                if (F32) {
+#pragma unroll 1
+                    for (int k = 0; k < mine; ++k) {
+                        const int c16 = c_begin + k;
+                        const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (gt & 1) * acc_cols + c16 * 16;
+                        uint32_t v[16], y[16];
+                        ptx::tmem_ld_16(at, v);
+                        ptx::tmem_ld_16(at + bn, y);
+                        ptx::tmem_ld_wait();
+                        const uint32_t box = wrow + (c16 >> 1) * W_BOX_BYTES;
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            const uint32_t addr = box + (((((c16 & 1) << 2) + h) ^ (row & 7)) << 4);
+                            uint32_t x[4];
+                            ptx::ld_shared_v4(addr, x[0], x[1], x[2], x[3]);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                x[u] = __float_as_uint(fmaf(-step, __uint_as_float(v[4 * h + u]) + __uint_as_float(y[4 * h + u]), __uint_as_float(x[u])));
+                            ptx::st_shared_v4(addr, x[0], x[1], x[2], x[3]);
+                        }
+                    }
+                }
                 // two 16-column chunks at a time: with all four of a warp in registers the kernel spills (96 registers for
                 // its 640 threads), which costs more than the second round trip to tensor memory
 #pragma unroll
-                for (int k0 = 0; k0 < 4; k0 += 2) {
+                for (int k0 = 0; k0 < (F32 ? 0 : 4); k0 += 2) {
                     uint32_t acc[2][16];
 #pragma unroll
                     for (int k = 0; k < 2; ++k)
@@ -897,6 +959,35 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 }
             }
         }
+    } else if (F32 && warp >= K2_FIXED_WARPS + GW) {
+        // ------------------------------------------------------------------ sketch chunks: rounded to tf32 in place, the rest beside them
+        const int tid = (int)threadIdx.x - 32 * (K2_FIXED_WARPS + GW);
+        RingPos pc, pl;
+        bool ok = true;
+        for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+            const int chunks = items[it].tiles * kchunks;
+            for (int c = 0; c < chunks; ++c, pc.advance(cstages), pl.advance(K2_LSTAGES)) {
+                ok = ptx::mbar_wait(ptx::smem_addr(&ctl->c_full[pc.s]), pc.wraps & 1u, abort) &&
+                     ptx::mbar_wait(ptx::smem_addr(&ctl->l_empty[pl.s]), (pl.wraps & 1u) ^ 1u, abort);
+                if (!ok) break;
+                const uint32_t at = c_ring + pc.s * S_CHUNK_BYTES + tid * 16, to = l_ring + pl.s * S_CHUNK_BYTES + tid * 16;
+#pragma unroll
+                for (int i = 0; i < S_CHUNK_BYTES / (16 * 32 * K2_CUT_WARPS); ++i) {
+                    uint32_t x[4], hi[4], lo[4];
+                    ptx::ld_shared_v4(at + i * (16 * 32 * K2_CUT_WARPS), x[0], x[1], x[2], x[3]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        hi[u] = round_tf32(x[u]);
+                        lo[u] = __float_as_uint(__uint_as_float(x[u]) - __uint_as_float(hi[u]));
+                    }
+                    ptx::st_shared_v4(at + i * (16 * 32 * K2_CUT_WARPS), hi[0], hi[1], hi[2], hi[3]);
+                    ptx::st_shared_v4(to + i * (16 * 32 * K2_CUT_WARPS), lo[0], lo[1], lo[2], lo[3]);
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->l_full[pl.s]));
+            }
+        }
     } else {
         // ------------------------------------------------------------------ slab generators
         // Slab of A as the N x K operand: row = column of W, K = index j of the sketch, values rounded to bf16
@@ -914,7 +1005,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             const uint32_t slab = slab0 + sb * slab_bytes;
             // the first slab (every slab, with a single buffer) is shared with the combine warps
             if (item.tiles > 0)
-                k2_generate_slab<BF16S>(slab, slab_block, kchunks, bn, item.col0, r, key, scale, g,
+                k2_generate_slab<BF16S, F32>(slab, slab_block, kchunks, bn, item.col0, r, key, scale, g,
                                         (k == 0 || nslabs == 1) ? 32 * (GW + K2_HELPER_WARPS) : 32 * GW);
             ptx::fence_proxy_async_smem();
             __syncwarp();

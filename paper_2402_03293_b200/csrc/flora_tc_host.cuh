@@ -50,6 +50,7 @@ struct TcSet {
     int* d_slots = nullptr;
     // decompression
     int bn = 128, slots = 2, cstages = 2, k2_gw = 8, k2_nslabs = 2, k2_grid_max = 148;
+    bool k2_f32 = false;                // the weights are fp32
     bool k2_bf16 = false;               // ranks above 64: the kernel reads a bf16 copy of the sketches
     bool k2_pair = false;               // ... and runs on CTA pairs (decompress_pair_kernel); k2_grid_max then counts pairs
     __nv_bfloat16* d_sb = nullptr;      // that copy (scratch owned by the set)
@@ -104,7 +105,9 @@ inline bool tc_mat_ok(const flora_mat& a)
            (a.ld & 7) == 0 && a.rows < (1ll << 31) - 256 && a.cols < (1ll << 31) - 256;
 }
 
-// fp32 matrices for the compression kernel
+// fp32 weights: the slabs of A (two parts, 64 columns) of larger ranks leave no room for two tiles of W and four chunks of the sketch
+constexpr int K2_F32_MAX_R = 128;
+// fp32 matrices
 inline bool tc_f32_ok(const flora_mat& a)
 {
     return a.dtype == FLORA_F32 && a.rows >= 128 && a.cols >= 32 && (reinterpret_cast<uintptr_t>(a.data) & 15) == 0 && (a.ld & 3) == 0 &&
@@ -613,15 +616,19 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     // ranks up to 64 read the fp32 sketch directly (tf32 MMA); above that the bytes of S that a CTA pulls per W
     // tile exceed what shared memory can keep in flight, so a bf16 copy of S is made first (half the bytes,
     // twice the K depth per 128-byte row) and the MMA runs in bf16
-    const bool bf16s = tune_knob("FLORA_K2_BF16S", r > 64 ? 1 : 0, 0, 1) != 0;
+    bool f32 = false;
+    for (const auto& w : W) f32 = f32 || (w.rows > 0 && w.dtype == FLORA_F32);
+    set.k2_f32 = f32;
+    const bool bf16s = !f32 && tune_knob("FLORA_K2_BF16S", r > 64 ? 1 : 0, 0, 1) != 0;
     set.k2_bf16 = bf16s;
     const int kchunks = bf16s ? (r + 63) / 64 : (r + 31) / 32;
     // slabs of 128 columns (every chunk of S then serves twice the columns of W) whenever two slabs, two W slots and
     // two S chunks of that width fit; 64 columns otherwise
     const size_t ctl = sizeof(K2Smem) + 1024;
     int bn = (2 * (size_t)kchunks * 128 * 128 + 2 * S_CHUNK_BYTES + 2 * 2 * (size_t)W_BOX_BYTES + ctl <= SMEM_BUDGET) ? 128 : 64;
-    bn = tune_knob("FLORA_K2_BN", bn, 64, 128) >= 128 ? 128 : 64;
-    const size_t slab_bytes = (size_t)kchunks * bn * 128, slot = (size_t)(bn / 64) * W_BOX_BYTES;
+    bn = !f32 && tune_knob("FLORA_K2_BN", bn, 64, 128) >= 128 ? 128 : 64;
+    const size_t slab_bytes = (size_t)kchunks * bn * (f32 ? 256 : 128), slot = (size_t)(bn / (f32 ? 32 : 64)) * W_BOX_BYTES;
+    const size_t lower = f32 ? (size_t)K2_LSTAGES * S_CHUNK_BYTES : 0;      // ring of the sketch's lower parts
     // two CTAs per SM when two of them fit (each with two slabs, two W slots and one S chunk)
     const size_t per_cta_max = 113 * 1024;                       // half of an SM's shared memory minus the reserve
     int per_sm = (2 * slab_bytes + S_CHUNK_BYTES + 2 * slot + ctl <= per_cta_max) ? 2 : 1;
@@ -630,22 +637,24 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     // than four S chunks in flight: the chunks of one W tile are kchunks x 16 KB, and with too few of them under way
     // the loads' latency, not bandwidth, sets the pace.  With one buffer every warp that is idle between two items
     // (the combine warps) shares the generation.
-    int nslabs = (2 * slab_bytes + 4 * S_CHUNK_BYTES + 2 * slot + ctl <= SMEM_BUDGET) ? 2 : 1;
+    // (fp32 W: a chunk is cut before it is multiplied, so its slot goes round slowly: with two of them 4096 x 11008 took 94 us at
+    // r = 64, with four and one slab buffer 72, and a third W slot is worth less than the fourth chunk: 77.)
+    int nslabs = (2 * slab_bytes + 4 * S_CHUNK_BYTES + (f32 ? 3 : 2) * slot + lower + ctl <= SMEM_BUDGET) ? 2 : 1;
     nslabs = tune_knob("FLORA_K2_SLABS", nslabs, 1, 2);
-    const size_t budget = (per_sm == 2 ? per_cta_max : SMEM_BUDGET) - ctl - nslabs * slab_bytes;
+    const size_t budget = (per_sm == 2 ? per_cta_max : SMEM_BUDGET) - ctl - nslabs * slab_bytes - lower;
     int cstages = std::max(2, std::min(nslabs == 1 ? 2 * kchunks : kchunks + 1, nslabs == 1 ? K2_MAX_CSTAGES : 4));
     cstages = tune_knob("FLORA_K2_CSTAGES", cstages, 1, K2_MAX_CSTAGES);
-    while (cstages > 1 && (size_t)cstages * S_CHUNK_BYTES + 2 * slot > budget) --cstages;
+    while (cstages > 1 && (size_t)cstages * S_CHUNK_BYTES + (f32 && cstages > 4 ? 3 : 2) * slot > budget) --cstages;
     int slots = (int)std::min<size_t>(K2_MAX_SLOTS, (budget - (size_t)cstages * S_CHUNK_BYTES) / slot);
     slots = tune_knob("FLORA_K2_SLOTS", slots, 1, std::max(1, slots));
-    int GW = 8;
+    int GW = f32 ? K2_MAX_GEN_WARPS - K2_CUT_WARPS : 8;
     GW = tune_knob("FLORA_K2_GEN_WARPS", GW, 1, K2_MAX_GEN_WARPS);
     set.bn = bn;
     set.slots = slots;
     set.cstages = cstages;
     set.k2_gw = GW;
     set.k2_nslabs = nslabs;
-    set.k2_smem = nslabs * slab_bytes + (size_t)cstages * S_CHUNK_BYTES + (size_t)slots * slot + sizeof(K2Smem) + 1024;
+    set.k2_smem = nslabs * slab_bytes + (size_t)cstages * S_CHUNK_BYTES + (size_t)slots * slot + lower + sizeof(K2Smem) + 1024;
     int grid_max = sm_count() * per_sm;
     // Ranks above 128 run on CTA pairs: each CTA holds half of a 128-column slab (two buffers of kchunks x 8 KB), the
     // sketch chunks of its own tiles (as many stages as fit beside two W tiles, at most two tiles' worth) and its W tiles.
@@ -675,8 +684,8 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     // cost model (microseconds of one SM): a tile streams bn*128*4 bytes at the SM's share of HBM; a slab costs
     // r*bn normals at the generator warps' rate and overlaps the previous item's streaming
     // (an SM takes in about 60 GB/s whatever the source: the chunks of S count like the W tile itself)
-    const double t_tile = std::max((double)bn * 128 * 4 / (6.5e6 / sm_count()),
-                                   ((double)bn * 128 * 2 + (double)kchunks * S_CHUNK_BYTES) / K2_SM_BYTES_PER_US);
+    const double t_tile = std::max((double)bn * 128 * (f32 ? 8 : 4) / (6.5e6 / sm_count()),
+                                   ((double)bn * 128 * (f32 ? 4 : 2) + (double)kchunks * S_CHUNK_BYTES) / K2_SM_BYTES_PER_US);
     const double t_slab = (double)r * bn / (GW >= 8 ? K2_VALUES_PER_US_8_WARPS : K2_VALUES_PER_US_FEWER);   // generator warps share the SM with the streaming warps
     auto build = [&](int run, std::vector<K2Item>& out) {
         out.clear();
@@ -1225,7 +1234,9 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
         }
     }
     if (!(set.k2_pair ? raise_smem_limit<decompress_pair_kernel<SINGLE>>()
-                      : set.k2_bf16 ? raise_smem_limit<decompress_tc_kernel<SINGLE, true>>() : raise_smem_limit<decompress_tc_kernel<SINGLE, false>>()))
+                      : set.k2_bf16 ? raise_smem_limit<decompress_tc_kernel<SINGLE, true, false>>()
+                      : set.k2_f32  ? raise_smem_limit<decompress_tc_kernel<SINGLE, false, true>>()
+                                    : raise_smem_limit<decompress_tc_kernel<SINGLE, false, false>>()))
         return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k2_launch_begin.size(); ++l) {
         const int begin = set.k2_launch_begin[l], end = set.k2_launch_begin[l + 1];
@@ -1236,7 +1247,7 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
         const int grid = std::min(set.k2_grid_max, end - begin);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(set.k2_pair ? 2 * grid : grid));       // (`grid` pairs)
-        cfg.blockDim = dim3((unsigned)(set.k2_pair ? K2P_THREADS : 32 * (K2_FIXED_WARPS + set.k2_gw)));
+        cfg.blockDim = dim3((unsigned)(set.k2_pair ? K2P_THREADS : 32 * (K2_FIXED_WARPS + set.k2_gw + (set.k2_f32 ? K2_CUT_WARPS : 0))));
         cfg.dynamicSmemBytes = set.k2_smem;
         cfg.stream = st;
         cudaLaunchAttribute attr[2];
@@ -1256,7 +1267,9 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
         };
         const cudaError_t e = set.k2_pair ? cudaLaunchKernelEx(&cfg, decompress_pair_kernel<SINGLE>, mats, one, items, end - begin, table, seed_base, r, scale, step,
                                                                set.slots, set.cstages)
-                              : set.k2_bf16 ? go(decompress_tc_kernel<SINGLE, true>) : go(decompress_tc_kernel<SINGLE, false>);
+                              : set.k2_bf16 ? go(decompress_tc_kernel<SINGLE, true, false>)
+                              : set.k2_f32  ? go(decompress_tc_kernel<SINGLE, false, true>)
+                                            : go(decompress_tc_kernel<SINGLE, false, false>);
         if (e != cudaSuccess) return FLORA_ERR_CUDA;
         launches.fetch_add(1, std::memory_order_relaxed);
     }
@@ -1294,7 +1307,7 @@ inline flora_status tc_decompress_single(flora_mat* W, const flora_mat* S, uint6
 
 inline bool tc_decompress_supported(const flora_mat* big, const flora_mat* sketch)
 {
-    return tc_mat_ok(*big) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
+    return (tc_mat_ok(*big) || (tc_f32_ok(*big) && sketch->cols <= K2_F32_MAX_R)) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
 }
 
 inline flora_status tc_set_zero(TcSet& set, cudaStream_t st, std::atomic<uint64_t>& launches)

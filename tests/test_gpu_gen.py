@@ -104,6 +104,31 @@ def test_fp32_through_tma(n, m, r):
     assert fb.flora_device_status() == 0
 
 
+# fp32 weights that the TMA decompression takes: rows and columns around a tile, a slab and a box of 32 columns, ranks around where a
+# second slab buffer stops fitting (32 | 33), with odd numbers of chunks, and the largest; next to a matrix that stays with the kernels
+# above.  Per element, of sum |C| |A|: the products carry 2^-22 (lo lo left out, lo cut to tf32), and each of the r / 8 + 2 truncated
+# accumulations loses less than 2^-22 of the running sum; the store of W rounds to 2^-24.
+@pytest.mark.parametrize("n,m,r", [(129, 8260, 8), (1000, 2100, 33), (4097, 1028, 1), (300, 5004, 96), (2049, 3076, 128), (8200, 164, 64), (128, 8224, 100)])
+def test_fp32_weights_through_tma(n, m, r):
+    W = wl.gaussian_matrix(n, m, 4e-4, "f32", 9).to(DEV)
+    C = torch.randn(n, r, device=DEV)
+    A = torch.empty(r, m, device=DEV)
+    fb.flora_materialize_A(A, 17)
+    update, size = 0.05 * (C.double() @ A.double()), 0.05 * (C.double().abs() @ A.double().abs())
+    bound = size * (r / 8 + 3) * 2.0 ** -22 + (W.double().abs() + update.abs()) * 2.0 ** -24
+    buf = torch.full((n, m + 4), 3.0, device=DEV)
+    buf[:, :m] = W
+    fb.flora_decompress_apply(buf[:, :m], C, 17, 0.05, 1.0)
+    assert bool(((buf[:, :m].double() - (W.double() - update)).abs() <= bound).all()) and torch.all(buf[:, m:] == 3.0)
+    small = torch.zeros(40, 70, device=DEV)
+    W2 = W.clone()
+    fset = fb.FloraSet(None, [W2, small], [C, torch.randn(40, r, device=DEV)])
+    fset.decompress_apply([17, 18], 0.05, 1.0)
+    assert bool(((W2.double() - (W.double() - update)).abs() <= bound).all()) and bool(small.abs().sum() > 0)
+    fset.close()
+    assert fb.flora_device_status() == 0
+
+
 # Transfers: one cluster and several, with their sums stored side by side or added into one matrix (by columns and rank), ranks below,
 # at and above one and two 128-row halves, ranks that TMA cannot address (33, 250), pairs of row tiles around 256, and two units per
 # cluster.  Against the same product in fp64, in the Frobenius norm: with bf16 operands src and T are read as tf32, whose ten
