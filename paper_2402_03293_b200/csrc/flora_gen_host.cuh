@@ -363,9 +363,42 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             for (int i : ids) clusters += ((big[i].rows + 127) / 128 + cluster / split[i] - 1) / (cluster / split[i]);
             return clusters;
         };
-        // clusters of sixteen (not portable: they need a whole GPC's SMs) only where one or two waves hold all of them
         s.plan.workers = per_sm == 2 ? 8 : 16;
-        if (cut_columns(GEN_MAX_SPLIT) > 2 * gen_k1_resident(s.plan, cluster) || cluster <= 8) cut_columns(8);
+        // How many CTAs at most: the shortest schedule of the clusters, longest first, on as many as can be resident (sixteen to a
+        // cluster need a whole GPC's SMs, so few are).  Measured, us per compression with at most 2, 4, 8, 16: the ragged set of eight matrices
+        // of up to 257 x 4097 at r = 32 68, 37, 21, 13.7 (bf16) and 156, 83, 44, 23.5 (fp32); 3000 x 1001, 2000 x 515 and 5000 x 129 in fp32 46, 25.9,
+        // 27.7, 33.5; 24 matrices of GPT-2-small shapes, rows off 16 bytes, 70, 77, 86, 85 (bf16).
+        int most = 8;
+        double shortest = 1e300;
+        for (int cand = 1; cand <= GEN_MAX_SPLIT; cand *= 2) {
+            cut_columns(cand);
+            if (cluster < cand && cand > 1) break;                // (the last one already had all it could use)
+            std::vector<double> work;
+            bool chains = true;                                   // no fp32 sum longer than it may be
+            for (int i : ids) {
+                const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = cluster / split[i];
+                if (tiles == 0) continue;
+                chains = chains && !(s.f32 && split[i] < GEN_MAX_SPLIT && steps > (int64_t)GEN_F32_CHAIN_STEPS * split[i]);
+                const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, per_sm, 1, (steps + split[i] - 1) / split[i], cluster);
+                work.insert(work.end(), (size_t)((tiles + per - 1) / per), cost);
+            }
+            if (work.empty() || (!chains && cand < GEN_MAX_SPLIT)) continue;
+            std::sort(work.begin(), work.end(), [](double x, double y) { return x > y; });
+            std::vector<double> ends((size_t)std::max(1, gen_k1_resident(s.plan, cluster)), 0.0);     // a heap, the earliest end on top
+            double span = 0.0;
+            for (double w : work) {
+                std::pop_heap(ends.begin(), ends.end(), [](double x, double y) { return x > y; });
+                ends.back() += w;
+                span = std::max(span, ends.back());
+                std::push_heap(ends.begin(), ends.end(), [](double x, double y) { return x > y; });
+            }
+            if (span < shortest * 1.02) {                         // (where two come out alike the longer chains are the slower)
+                shortest = std::min(shortest, span);
+                most = cand;
+            }
+        }
+        most = tune_knob("FLORA_GEN_MOST", most, 1, GEN_MAX_SPLIT);
+        cut_columns(most);
         const int T = 1;
         if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
