@@ -124,7 +124,7 @@ gram_tc_kernel(const GramJob* __restrict__ jobs, const GramItem* __restrict__ it
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
-    if (SINGLE) ptx::grid_launch_dependents();            // (after the allocation: see compress_tc_kernel)
+    ptx::grid_launch_dependents();                        // (after the allocation: see compress_tc_kernel)
     const uint32_t tmem = ctl->tmem_base;
     volatile int* abort = &ctl->abort;
 
@@ -570,7 +570,7 @@ apply_tc_kernel(const GramJob* __restrict__ jobs, const TcMatrix* __restrict__ d
     // tensor memory (the compression of a resampling step does: it streams G, which this kernel does not touch, and waits itself
     // before it reads a sketch).
     ptx::grid_launch_dependents();
-    if (SINGLE) ptx::grid_dependency_wait();    // the kernel that makes T lets this one set itself up meanwhile
+    ptx::grid_dependency_wait();                // the kernel that makes T lets this one set itself up meanwhile
     if (warp == 0) {
         // ------------------------------------------------------------------ src loads: this CTA's tile, chunk by chunk
         if (lane == 0) {
@@ -943,10 +943,10 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
         attr[0].val.clusterDim.x = 2;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (one matrix: the kernel waits for the gram kernel itself)
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (the kernel waits for the gram kernel itself)
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = single_maps ? 2 : 1;
+        cfg.numAttrs = 2;
         cudaError_t e;
         if (single_maps) {
             single_arg.job = jobs[0];
