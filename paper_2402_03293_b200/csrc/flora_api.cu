@@ -453,7 +453,8 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
     return FLORA_OK;
 }
 
-// behind_own_transfer: the kernel before this call on the stream is the library's own transfer, which does not touch G
+// behind_own_transfer: the work before this call on the stream is the library's own transfer, which does not touch G and whose first
+// operation waited for all earlier work (transfer_tc's `ordered`)
 static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a, float b, void* stream, bool behind_own_transfer = false)
 {
     if (!set || !seeds) return FLORA_ERR_NULL;
@@ -506,9 +507,10 @@ flora_status flora_set_decompress_apply(flora_set* set, const uint64_t* seeds, f
 
 // dst.S[i] <- b dst.S[i] + a src[i] (A(old_i) A(new_i)^T) for every matrix of the set `dst`.
 static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& src, const TcMatrix* src_mats, const uint64_t* seeds_old,
-                                 const uint64_t* seeds_new, float a, float b, void* stream, void** release_later = nullptr)
+                                 const uint64_t* seeds_new, float a, float b, void* stream, void** release_later = nullptr, bool* ordered = nullptr)
 {
     if (release_later) *release_later = nullptr;
+    if (ordered) *ordered = false;
     if (!set || !seeds_old || !seeds_new) return FLORA_ERR_NULL;
     const std::vector<flora_mat>& big = set->has_G ? set->G : set->W;
     const int r = set->r;
@@ -526,7 +528,7 @@ static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& s
                                    (int32_t)set->S[i].rows, (int32_t)big[i].cols, seeds_old[i], seeds_new[i], (int32_t)i, 0});
         }
         return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches, set->tc.d_mats, src_mats, nullptr, release_later,
-                           dtype == FLORA_F32);
+                           dtype == FLORA_F32, ordered);
     }
     if (scratch_alloc((void**)&T, sizeof(float) * r * r, as_stream(stream)) != cudaSuccess) {
         cudaGetLastError();
@@ -562,10 +564,12 @@ flora_status flora_set_momentum_step_resampled(flora_set* set, float beta, const
     if (!set || !seeds_old || !seeds_new) return FLORA_ERR_NULL;
     if (!set->has_G) return FLORA_ERR_UNSUPPORTED;
     // the compression goes right behind the transfer's last kernel and starts while that one still runs (it waits itself
-    // before it touches a sketch); the transfer's scratch is handed back after it has been launched
+    // before it touches a sketch, and before it reads G unless the transfer's first operation waited for G's writer); the
+    // transfer's scratch is handed back after it has been launched
     void* scratch = nullptr;
-    flora_status st = set_transfer(set, set->S, set->tc.d_mats, seeds_old, seeds_new, beta, 0.0f, stream, &scratch);
-    if (st == FLORA_OK) st = set_compress(set, seeds_new, 1.0f - beta, 1.0f, stream, scratch != nullptr);
+    bool ordered = false;
+    flora_status st = set_transfer(set, set->S, set->tc.d_mats, seeds_old, seeds_new, beta, 0.0f, stream, &scratch, &ordered);
+    if (st == FLORA_OK) st = set_compress(set, seeds_new, 1.0f - beta, 1.0f, stream, ordered);
     if (scratch && cudaFreeAsync(scratch, as_stream(stream)) != cudaSuccess && st == FLORA_OK) st = FLORA_ERR_CUDA;
     return st;
 }

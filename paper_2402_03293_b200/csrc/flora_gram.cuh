@@ -814,12 +814,16 @@ inline int plan_single_gram(int r, int m, int most, int most_parts, int* kw)
 
 inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
                                 const TcMatrix* d_dst_mats = nullptr, const TcMatrix* d_src_mats = nullptr, float* static_T = nullptr,
-                                void** release_later = nullptr, bool f32 = false)
+                                void** release_later = nullptr, bool f32 = false, bool* ordered = nullptr)
 {
     // f32: fp32 operands, in fp32 arithmetic throughout (gram_f32_kernel, then the fp32 apply kernels)
     // release_later: the caller frees the call's scratch (stream-ordered) itself, after it has put more work behind the
     // last kernel; nothing then stands between that kernel and the caller's next launch
+    // ordered: set to true where the call's first work on the stream waits for everything before it (the table copy of several
+    // matrices).  One matrix has no such work: its gram kernel is launched early and waits itself, after its successor may have
+    // started, so a kernel behind the transfer may not take for granted that anything before the call is done.
     if (release_later) *release_later = nullptr;
+    if (ordered) *ordered = false;
     if (jobs.empty()) return FLORA_OK;
     const int sms = sm_count();
     // step width: 64 columns, or narrower while that leaves fewer than four steps per SM to balance
@@ -1000,6 +1004,7 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
         // pageable source: staged by the runtime before the call returns
         ok = ok && cudaMemcpyAsync(buf + tables_off, tables.data(), tables.size(), cudaMemcpyHostToDevice, st) == cudaSuccess &&
              raise_smem_limit<gram_tc_kernel<false>>();
+        if (ordered) *ordered = ok;
         if (ok) {
             const GramJob* d_jobs = reinterpret_cast<const GramJob*>(buf + tables_off);
             const GramItem* d_items = reinterpret_cast<const GramItem*>(buf + tables_off + jobs_bytes);

@@ -111,7 +111,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     ptx::tc_fence_after_sync();
     ptx::grid_launch_dependents();          // (after the allocation of tensor memory, as in compress_tc_kernel)
     // everything above touched only shared and tensor memory; G and S may have been written by the previous kernel
-    // of the stream.  `late_wait`: that kernel is this library's own pre-scaling of S, which does not touch G.
+    // of the stream.  `late_wait`: the kernels before this one do not touch G, and its writer is done (see compress_tc_kernel).
     if (!late_wait) {
         if (threadIdx.x == 0 && u_begin < u_end) {              // the first tiles into L2 meanwhile, as in compress_tc_kernel
             const K1Item item = items[(size_t)u_begin * S + rank];

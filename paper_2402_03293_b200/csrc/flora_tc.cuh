@@ -197,8 +197,9 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     // one must have its own before they start.
     ptx::grid_launch_dependents();
     // everything above touched only this CTA's shared and tensor memory; G and S may have been written by the
-    // previous kernel of the stream.  `late_wait`: that kernel is this library's own pre-scaling of S, which was
-    // itself ordered after everything before it and does not touch G, so only the accesses to S need to wait
+    // previous kernel of the stream.  `late_wait`: the kernels before this one are this library's own (the pre-scaling of S, or a
+    // transfer), do not touch G, and the first of them was itself ordered after everything before it - a full dependency, not an
+    // early launch whose own wait may still be under way -, so only the accesses to S need to wait
     if (!late_wait) {
         // (into L2 they may come before that kernel is done: a line that it writes is changed there)
         if (threadIdx.x == 0) {

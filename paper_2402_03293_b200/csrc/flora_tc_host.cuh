@@ -999,8 +999,9 @@ inline unsigned helper_blocks(const TcSet& set)
     return helper_blocks(most);
 }
 
-// behind_own_kernel: the kernel before this call on the stream is one of the library's own that does not touch G and lets
-// its dependents start early (the transfer's apply kernel): only the write-out of the compression waits for it.
+// behind_own_kernel: the kernels before this call on the stream, back to one that everything earlier was complete before, are the
+// library's own (a transfer of several matrices), do not touch G and let their dependents start early: only the write-out of the
+// compression waits for them.
 // one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).
 template <bool SINGLE, int MAPS>
 inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, const uint64_t* seeds, float a, float b, cudaStream_t st,

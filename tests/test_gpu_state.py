@@ -226,3 +226,28 @@ def test_first_compression_of_a_cycle_overwrites_whatever_the_sketch_held(r):
         two = oracle_compress(G[i], torch.from_numpy(oracle_compress(G[i], torch.zeros(n, r), s_used[i])), s_used[i])
         assert rel_err(S[i].cpu().numpy(), two) <= TOL["bf16"], i
     fset.close()
+
+
+@pytest.mark.parametrize("n,m,r", [(2048, 4224, 32), (2048, 4096, 256)])
+def test_resampled_step_of_one_matrix_waits_for_the_writer_of_its_gradient(n, m, r):
+    """A set of one matrix whose gradient was written by a kernel that lets its successors start early (here the library's own
+    weight update, on the same stream): the transfer's kernels start early, too, so the compression behind them must wait itself
+    before it reads G."""
+    G = torch.zeros(n, m, device=DEV, dtype=torch.bfloat16)
+    D = torch.randn(n, r, device=DEV)
+    M = torch.randn(n, r, device=DEV)
+    M0 = M.clone()
+    fset = fb.FloraSet([G], None, [M])
+    fb.flora_decompress_apply(G, D, 7, 0.0, 1.0)                      # (plans)
+    for k in range(4):
+        G.zero_()
+        M.copy_(M0)
+        fb.flora_decompress_apply(G, D, 8 + k, -1.0, 1.0)             # G <- D A
+        fset.momentum_step_resampled(0.5, [21], [22])
+        want = M0.clone()
+        fb.flora_resample_transfer(want, m, "bf16", 21, 22)
+        torch.cuda.synchronize()
+        fb.flora_momentum_step(G, want, 0.5, 22)
+        assert rel_err(M.cpu().numpy(), want.cpu().numpy()) <= 1e-4, k      # (sums in another order; an old G would be off by its size)
+    fset.close()
+    assert fb.flora_device_status() == 0
