@@ -250,6 +250,13 @@ static flora_status set_build(flora_set* s)
         st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g);
         if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w);
     }
+    // The tables were copied from pageable memory on the legacy stream, to which streams made with the non-blocking flag are not
+    // ordered: they are in place before any stream may use them.
+    const bool copied = s->tc.d_mats || s->tcf.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats;
+    if (copied && cudaStreamSynchronize(nullptr) != cudaSuccess) {
+        cudaGetLastError();
+        if (st == FLORA_OK) st = FLORA_ERR_CUDA;
+    }
     return st;
 }
 

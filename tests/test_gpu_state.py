@@ -251,3 +251,26 @@ def test_resampled_step_of_one_matrix_waits_for_the_writer_of_its_gradient(n, m,
         assert rel_err(M.cpu().numpy(), want.cpu().numpy()) <= 1e-4, k      # (sums in another order; an old G would be off by its size)
     fset.close()
     assert fb.flora_device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_a_set_may_be_used_from_any_stream_as_soon_as_it_exists(dtype):
+    """The tables of a set are copied behind whatever the default stream holds; a stream that is not ordered to it may use the set
+    at once."""
+    shapes, r = [(512, 4224), (2048, 2304), (40, 70)], 32
+    G = [wl.gaussian_matrix(n, m, 1e-2, dtype, 3 + i).to(DEV) for i, (n, m) in enumerate(shapes)]
+    W = [torch.zeros_like(g) for g in G]
+    S = [torch.zeros(n, r, device=DEV) for n, _ in shapes]
+    side = torch.cuda.Stream()                                        # (torch's streams are non-blocking)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(40_000_000)                                     # some 20 ms of the default stream
+    fset = fb.FloraSet(G, W, S)
+    seeds = [fb.flora_derive_seed(2, i, 0) for i in range(len(shapes))]
+    fset.compress_accumulate(seeds, stream=side)
+    fset.decompress_apply(seeds, 0.1, 1.0, stream=side)
+    torch.cuda.synchronize()
+    for i, (n, m) in enumerate(shapes):
+        assert rel_err(S[i].cpu().numpy(), oracle_compress(G[i], torch.zeros(n, r), seeds[i])) <= TOL[dtype], i
+        ref = oracle_decompress(torch.zeros_like(W[i]).cpu(), S[i].cpu(), seeds[i], 0.1, 1.0)
+        assert rel_err(values(wl.as_numpy(W[i])), values(ref)) <= TOL[dtype], i
+    fset.close()
