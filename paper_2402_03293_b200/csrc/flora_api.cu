@@ -223,15 +223,9 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
     return use;
 }
 
-// Builds (or builds again) the work lists of a set for its present pointers.
+// Builds the work lists of a set.
 static flora_status set_build(flora_set* s)
 {
-    tc_set_free(s->tc);
-    tc_set_free(s->tcf);
-    for (int d = 0; d < 2; ++d) {
-        gen_set_free(s->gen_g[d]);
-        gen_set_free(s->gen_w[d]);
-    }
     std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true);
     const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_wf = set_tma_side(s->W, s->S, false, true);
     std::vector<uint8_t> use_w = set_tma_side(s->W, s->S, false);
@@ -447,17 +441,35 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
         if (G[i].dtype != set->G[i].dtype) return FLORA_ERR_DTYPE;
     }
     std::vector<flora_mat> newG(G, G + set->G.size());
-    flora_status st = tc_set_rebind(set->tc, newG, as_stream(stream));
-    if (st == FLORA_OK) st = tc_set_rebind(set->tcf, newG, as_stream(stream));
-    if (st == FLORA_ERR_ALIGN && (set->gen_g[0].ready() || set->gen_g[1].ready() || set->tcf.compress_ready)) {
-        // a mixed (or fp32) set takes any address: the matrix changes sides (work that still reads the old tables ends first)
-        set->G.swap(newG);
-        return cudaStreamSynchronize(as_stream(stream)) == cudaSuccess ? set_build(set) : FLORA_ERR_CUDA;
-    }
+    // A set of any other kind than bf16 matrices that TMA serves takes any address.  Where TMA cannot address one of the new
+    // gradients, the matrices of its kind are compressed one by one until a later call brings addresses that it can: those launches
+    // carry the matrix by value, so nothing is allocated, planned or waited for here.
+    const bool tc_ok = tc_set_addressable(set->tc, newG), tcf_ok = tc_set_addressable(set->tcf, newG);
+    if ((!tc_ok || !tcf_ok) && !(set->gen_g[0].ready() || set->gen_g[1].ready() || set->tcf.compress_ready)) return FLORA_ERR_ALIGN;
+    std::vector<CUtensorMap> maps, maps_f;
+    if ((tc_ok && !tc_set_make_maps(set->tc, newG, maps)) || (tcf_ok && !tc_set_make_maps(set->tcf, newG, maps_f))) return FLORA_ERR_CUDA;
+    flora_status st = tc_ok ? tc_set_rebind(set->tc, maps, as_stream(stream)) : FLORA_OK;
+    if (st == FLORA_OK && tcf_ok) st = tc_set_rebind(set->tcf, maps_f, as_stream(stream));
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_rebind(set->gen_g[d], newG, as_stream(stream));
     if (st) return st;
+    set->tc.off_tma = !tc_ok;
+    set->tcf.off_tma = !tcf_ok;
     set->G.swap(newG);
     return FLORA_OK;
+}
+
+// The matrices of a set that the TMA kernels serve.
+static flora_status tma_compress(const flora_set* set, const TcSet& tc, const uint64_t* seeds, float a, float b, cudaStream_t st, bool behind_own_transfer)
+{
+    if (!tc.compress_ready) return FLORA_OK;
+    if (!tc.off_tma) return tc_set_compress(tc, seeds, a, b, st, g_launches, behind_own_transfer);
+    flora_status rc = FLORA_OK;
+    for (size_t k = 0; k < tc.members.size() && rc == FLORA_OK; ++k) {
+        const size_t i = (size_t)tc.members[k];
+        flora_mat S = set->S[i];
+        rc = gen_supported(set->G[i]) ? gen_compress_single(set->G[i], S, seeds[i], a, b, st, g_launches) : simt_compress(&set->G[i], &S, seeds[i], a, b, st);
+    }
+    return rc;
 }
 
 // behind_own_transfer: the work before this call on the stream is the library's own transfer, which does not touch G and whose first
@@ -468,9 +480,8 @@ static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a,
     if (!set->has_G) return FLORA_ERR_UNSUPPORTED;
     const bool simt = g_force_path.load() == 1;
     if (!simt) {
-        flora_status st = FLORA_OK;
-        if (set->tc.compress_ready) st = tc_set_compress(set->tc, seeds, a, b, as_stream(stream), g_launches, behind_own_transfer);
-        if (st == FLORA_OK && set->tcf.compress_ready) st = tc_set_compress(set->tcf, seeds, a, b, as_stream(stream), g_launches);
+        flora_status st = tma_compress(set, set->tc, seeds, a, b, as_stream(stream), behind_own_transfer);
+        if (st == FLORA_OK) st = tma_compress(set, set->tcf, seeds, a, b, as_stream(stream), false);
         for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_compress(set->gen_g[d], seeds, a, b, as_stream(stream), g_launches);
         if (st) return st;
     }

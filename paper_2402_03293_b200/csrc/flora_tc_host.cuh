@@ -37,6 +37,7 @@ struct TcSet {
     int* d_split = nullptr;
     std::vector<TcMatrix> h_mats;
     std::vector<CUtensorMap> g_maps;    // maps of re-pointed gradients (empty: the table's are valid)
+    bool off_tma = false;               // a gradient was re-pointed to where TMA cannot address it: compressed matrix by matrix (set_compress)
     std::vector<K1Item> h_k1;
     std::vector<int> k1_launch_begin;   // item ranges per launch (at most SEEDS_PER_LAUNCH matrices each)
     std::vector<int> split_mats;        // matrices whose sketch is updated by several items
@@ -972,17 +973,34 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_
     return FLORA_OK;
 }
 
+// Whether TMA can address the new gradients of all members.
+inline bool tc_set_addressable(const TcSet& set, const std::vector<flora_mat>& G)
+{
+    if (set.compress_ready)
+        for (int i : set.members)
+            if (!(set.f32 ? tc_f32_ok(G[i]) : tc_mat_ok(G[i]))) return false;
+    return true;
+}
+// Tensor maps of the members' new gradients, in the members' order.
+inline bool tc_set_make_maps(const TcSet& set, const std::vector<flora_mat>& G, std::vector<CUtensorMap>& maps)
+{
+    if (!set.compress_ready) return true;
+    maps.resize(set.members.size());
+    for (size_t k = 0; k < maps.size(); ++k)
+        if (!make_map(&maps[k], G[(size_t)set.members[k]])) return false;
+    return true;
+}
 // New gradient pointers, same shapes: only the tensor maps change.  They are kept on the host and travel with the next launches;
 // sets of more matrices than a launch can carry maps for get them copied into their table.
-inline flora_status tc_set_rebind(TcSet& set, const std::vector<flora_mat>& G, cudaStream_t st)
+inline flora_status tc_set_rebind(TcSet& set, const std::vector<CUtensorMap>& maps, cudaStream_t st)
 {
     if (!set.compress_ready) return FLORA_OK;
-    for (int i : set.members)
-        if (!(set.f32 ? tc_f32_ok(G[i]) : tc_mat_ok(G[i]))) return FLORA_ERR_ALIGN;
     const bool carried = set.count <= GMAPS_MANY;
     if (carried) set.g_maps.resize((size_t)set.count);
-    for (int i : set.members)
-        if (!make_map(carried ? &set.g_maps[(size_t)i] : &set.h_mats[(size_t)i].map_g, G[i])) return FLORA_ERR_CUDA;
+    for (size_t k = 0; k < maps.size(); ++k) {
+        const size_t i = (size_t)set.members[k];
+        (carried ? set.g_maps[i] : set.h_mats[i].map_g) = maps[k];
+    }
     return carried ? FLORA_OK : upload(&set.d_mats, set.h_mats, st);
 }
 

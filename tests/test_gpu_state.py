@@ -274,3 +274,48 @@ def test_a_set_may_be_used_from_any_stream_as_soon_as_it_exists(dtype):
         ref = oracle_decompress(torch.zeros_like(W[i]).cpu(), S[i].cpu(), seeds[i], 0.1, 1.0)
         assert rel_err(values(wl.as_numpy(W[i])), values(ref)) <= TOL[dtype], i
     fset.close()
+
+
+@pytest.mark.parametrize("kind", ["f32", "mixed"])
+def test_gradients_may_move_to_where_tma_cannot_address_them_and_back(kind):
+    """A set that holds fp32 or mixed matrices takes gradients at any address.  The call neither allocates nor waits for anything,
+    and what follows on the stream uses the new addresses."""
+    shapes = [(512, 4224, "f32"), (2048, 1536, "f32")] if kind == "f32" else [(2048, 2304, "bf16"), (130, 515, "bf16"), (512, 4224, "f32")]
+    r = 24
+    W = [torch.zeros(n, m, device=DEV, dtype=wl.torch_dtype(d)) for n, m, d in shapes]
+    S = [torch.zeros(n, r, device=DEV) for n, _, _ in shapes]
+    seeds = [fb.flora_derive_seed(5, i, 0) for i in range(len(shapes))]
+
+    def grads(t, off):
+        out = []
+        for i, (n, m, d) in enumerate(shapes):
+            buf = torch.zeros(n * m + 8, device=DEV, dtype=wl.torch_dtype(d))
+            v = buf[off:off + n * m].view(n, m)
+            v.copy_(wl.gaussian_matrix(n, m, 1e-2, d, 10 * t + i))
+            out.append(v)
+        return out
+
+    G = [grads(t, off) for t, off in enumerate((0, 1, 0, 1))]
+    fset = fb.FloraSet(G[0], W, S)
+    side = torch.cuda.Stream()
+    for t, g in enumerate(G):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(20_000_000)
+            busy = torch.cuda.Event()
+            busy.record()
+        fset.rebind_gradients(g, stream=side)
+        assert not busy.query()                                       # (the stream is still at work: nothing has been waited for)
+        fset.compress_overwrite(seeds, stream=side)
+        fset.momentum_step(0.75, [s + 1 for s in seeds], stream=side)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+        for i, (n, m, d) in enumerate(shapes):
+            first = torch.from_numpy(oracle_compress(g[i], torch.zeros(n, r), seeds[i]))
+            assert rel_err(S[i].cpu().numpy(), oracle_compress(g[i], first, seeds[i] + 1, a=0.25, b=0.75)) <= TOL[d], (t, i)
+    fset.decompress_apply(seeds, 0.1, 1.0)
+    for i, (n, m, d) in enumerate(shapes):
+        ref = oracle_decompress(torch.zeros_like(W[i]).cpu(), S[i].cpu(), seeds[i], 0.1, 1.0)
+        assert rel_err(values(wl.as_numpy(W[i])), values(ref)) <= TOL[d], i
+    fset.close()
