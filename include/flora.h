@@ -163,9 +163,12 @@ typedef struct flora_set flora_set;
 flora_status flora_set_create(int count, const flora_mat* G, const flora_mat* W, const flora_mat* S, flora_set** out);
 flora_status flora_set_destroy(flora_set* set);
 
-/* Re-point the gradient matrices of a set (same shapes, dtypes and leading dimensions).  The update of
- * the device-side descriptors is enqueued on `stream`: it is ordered after the set's earlier launches on
- * that stream and before its later ones.  */
+/* Re-point the gradient matrices of a set (same shapes, dtypes and leading dimensions).  Ordered as work on `stream`: the set's
+ * earlier launches on that stream use the old gradients, its later ones the new, and so do compressions of the set that a CUDA
+ * graph holds when the graph is launched behind the call on that stream.  Two limits, FLORA_ERR_ALIGN otherwise (nothing changes
+ * then): the gradients of a set of bf16 matrices that were all aligned to 16 bytes (pointer and ld) and large enough for the
+ * TMA kernels must stay so, and once a compression has been recorded into a graph no set may lose that alignment.
+ * (Compressions recorded while a gradient of a set with fp32 or mixed matrices lay off 16 bytes keep that address.) */
 flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void* stream);
 
 /* seeds: host array of `count` 64-bit seeds, one per matrix (copied before the call returns). */

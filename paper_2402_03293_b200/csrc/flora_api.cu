@@ -446,6 +446,9 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
     // carry the matrix by value, so nothing is allocated, planned or waited for here.
     const bool tc_ok = tc_set_addressable(set->tc, newG), tcf_ok = tc_set_addressable(set->tcf, newG);
     if ((!tc_ok || !tcf_ok) && !(set->gen_g[0].ready() || set->gen_g[1].ready() || set->tcf.compress_ready)) return FLORA_ERR_ALIGN;
+    // launches that a graph holds read the gradients through the set's tables, with the kernels of the time they were recorded at
+    if ((!tc_ok && set->tc.captured) || (!tcf_ok && set->tcf.captured) || !gen_set_rebindable(set->gen_g[0], newG) || !gen_set_rebindable(set->gen_g[1], newG))
+        return FLORA_ERR_ALIGN;
     std::vector<CUtensorMap> maps, maps_f;
     if ((tc_ok && !tc_set_make_maps(set->tc, newG, maps)) || (tcf_ok && !tc_set_make_maps(set->tcf, newG, maps_f))) return FLORA_ERR_CUDA;
     flora_status st = tc_ok ? tc_set_rebind(set->tc, maps, as_stream(stream)) : FLORA_OK;
@@ -459,7 +462,7 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
 }
 
 // The matrices of a set that the TMA kernels serve.
-static flora_status tma_compress(const flora_set* set, const TcSet& tc, const uint64_t* seeds, float a, float b, cudaStream_t st, bool behind_own_transfer)
+static flora_status tma_compress(const flora_set* set, TcSet& tc, const uint64_t* seeds, float a, float b, cudaStream_t st, bool behind_own_transfer)
 {
     if (!tc.compress_ready) return FLORA_OK;
     if (!tc.off_tma) return tc_set_compress(tc, seeds, a, b, st, g_launches, behind_own_transfer);

@@ -296,6 +296,7 @@ struct GenSet {
     GenK1Plan plan;
     int r = 0;
     bool f32 = false;
+    bool captured_aligned = false;             // a launch that relies on whole 16-byte pieces has been recorded into a graph
     bool ready() const { return !ids.empty(); }
 };
 inline void gen_set_free(GenSet& s)
@@ -456,8 +457,9 @@ inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
     for (int i = 0; i < SEEDS_PER_LAUNCH; ++i) t.s[i] = base + i < (int)s.h_mats.size() ? seeds[base + i] : 0;
     return t;
 }
-inline flora_status gen_set_compress(const GenSet& s, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches)
+inline flora_status gen_set_compress(GenSet& s, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
+    if (s.ready() && s.plan.aligned && !s.captured_aligned) s.captured_aligned = capturing(st);
     for (size_t l = 0; l + 1 < s.begin.size(); ++l) {
         const flora_status rc = gen_compress_launch(s.f32, s.plan, s.begin[l + 1] - s.begin[l], s.d_mats, s.d_k1 + s.begin[l],
                                                     gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, s.first_mat[l], s.r, a, b, st, launches);
@@ -475,6 +477,14 @@ inline flora_status gen_set_decompress(const GenSet& s, const uint64_t* seeds, f
         if (rc) return rc;
     }
     return FLORA_OK;
+}
+// Whether launches recorded into a graph can read the new gradients.
+inline bool gen_set_rebindable(const GenSet& s, const std::vector<flora_mat>& big)
+{
+    if (s.captured_aligned)
+        for (int i : s.ids)
+            if (!gen_aligned(big[i])) return false;
+    return true;
 }
 // New gradient pointers, same shapes.
 inline flora_status gen_set_rebind(GenSet& s, const std::vector<flora_mat>& big, cudaStream_t st)

@@ -53,7 +53,7 @@ template <bool SINGLE, int MAPS>
 __global__ void __launch_bounds__(PAIR_MAX_THREADS, 1)
 compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const int* __restrict__ slot_begin,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, int N, float scale, float a, float b, int gstages,
-                     int astages, int S, int GW, int late_wait)
+                     int astages, int S, int GW, int late_wait, int new_maps)
 {
     const TcMatrix* mats = SINGLE ? &single : table;                   // (one matrix: every unit names matrix 0)
     extern __shared__ uint8_t smem_raw[];
@@ -117,6 +117,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
             const K1Item item = items[(size_t)u_begin * S + rank];
             const CUtensorMap* map_g = &mats[item.mat].map_g;
             if constexpr (MAPS > 0) map_g = &gmaps.m[item.mat - seed_base];
+            if (!SINGLE && MAPS == 0 && new_maps) ptx::fence_tensormap_acquire(map_g);
             for (int ks = 0; ks < min(item.ksteps, K1_L2_AHEAD / PAIR_T); ++ks)
                 for (int t = 0; t < item.tiles; ++t) ptx::tma_prefetch_l2_2d(map_g, (item.kstep0 + ks) * 64, item.row0 + t * 128);
         }
@@ -136,6 +137,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 const TcMatrix* mat = mats + item.mat;
                 const CUtensorMap* map_g = &mat->map_g;
                 if constexpr (MAPS > 0) map_g = &gmaps.m[item.mat - seed_base];
+                if (!SINGLE && MAPS == 0 && new_maps) ptx::fence_tensormap_acquire(map_g);
                 if (item.tiles > 0) ptx::prefetch_tensormap(map_g);
                 for (int ks = 0; ks < item.ksteps; ++ks, ++g, pg.advance(gstages), pp.advance(PAIR_RELAY_DEPTH)) {
                     const int s = pg.s;

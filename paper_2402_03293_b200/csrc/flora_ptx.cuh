@@ -213,6 +213,12 @@ __device__ __forceinline__ void tma_store_wait_all()
 {
     asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
 }
+// Makes a tensor map in global memory that was written since the last kernel (a copy into a table, a graph launched behind it)
+// visible to the TMA operations of this thread: they read maps through a cache of their own.
+__device__ __forceinline__ void fence_tensormap_acquire(const void* tmap)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tmap) : "memory");
+}
 __device__ __forceinline__ void prefetch_tensormap(const void* tmap)
 {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");

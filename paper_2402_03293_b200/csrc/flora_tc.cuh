@@ -123,13 +123,14 @@ struct K1Smem {                            // barriers and scalars, placed after
 // for its lo(G), 11 r cycles for A and 400 of tensor pipe; the kernel that cut fp32 into three bf16 parts out of registers spent
 // 670 issue cycles on a tile.
 // SINGLE: one matrix, its record passed by value (every item names matrix 0).  MAPS: the gradients' maps come with the launch.
+// new_maps: those in the table may have been written since the kernel before.
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
 // 4096 x 11008 matrix takes 27 us instead of 20)
 template <bool SINGLE, bool F32, int MAPS>
 __global__ void __maxnreg__(80)
 compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
                    int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int lstages, int nsets, int S, int GW, int P,
-                   int late_wait)
+                   int late_wait, int new_maps)
 {
     constexpr int KC = F32 ? 32 : 64;                          // columns of a step
     extern __shared__ uint8_t smem_raw[];
@@ -200,6 +201,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     // previous kernel of the stream.  `late_wait`: the kernels before this one are this library's own (the pre-scaling of S, or a
     // transfer), do not touch G, and the first of them was itself ordered after everything before it - a full dependency, not an
     // early launch whose own wait may still be under way -, so only the accesses to S need to wait
+    if (!SINGLE && MAPS == 0 && new_maps && threadIdx.x == 0) ptx::fence_tensormap_acquire(map_g);       // (the thread that issues the loads)
     if (!late_wait) {
         // (into L2 they may come before that kernel is done: a line that it writes is changed there)
         if (threadIdx.x == 0) {

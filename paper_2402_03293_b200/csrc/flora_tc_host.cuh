@@ -37,6 +37,9 @@ struct TcSet {
     int* d_split = nullptr;
     std::vector<TcMatrix> h_mats;
     std::vector<CUtensorMap> g_maps;    // maps of re-pointed gradients (empty: the table's are valid)
+    TcMatrix* d_graph = nullptr;        // the table that launches recorded into graphs read (g_maps travel with the others)
+    bool new_maps = false;              // the table's maps have been written since it was made
+    bool captured = false;              // such a launch exists
     bool off_tma = false;               // a gradient was re-pointed to where TMA cannot address it: compressed matrix by matrix (set_compress)
     std::vector<K1Item> h_k1;
     std::vector<int> k1_launch_begin;   // item ranges per launch (at most SEEDS_PER_LAUNCH matrices each)
@@ -844,6 +847,7 @@ inline void tc_set_free(TcSet& s)
     if (s.d_members) cudaFree(s.d_members);
     if (s.d_slots) cudaFree(s.d_slots);
     if (s.d_sb) cudaFree(s.d_sb);
+    if (s.d_graph) cudaFree(s.d_graph);
     s = TcSet();
 }
 
@@ -991,7 +995,8 @@ inline bool tc_set_make_maps(const TcSet& set, const std::vector<flora_mat>& G, 
     return true;
 }
 // New gradient pointers, same shapes: only the tensor maps change.  They are kept on the host and travel with the next launches;
-// sets of more matrices than a launch can carry maps for get them copied into their table.
+// sets of more matrices than a launch can carry maps for get them copied into their table.  Launches recorded into a graph read a
+// table of their own, which is brought up to date on the stream.
 inline flora_status tc_set_rebind(TcSet& set, const std::vector<CUtensorMap>& maps, cudaStream_t st)
 {
     if (!set.compress_ready) return FLORA_OK;
@@ -999,9 +1004,49 @@ inline flora_status tc_set_rebind(TcSet& set, const std::vector<CUtensorMap>& ma
     if (carried) set.g_maps.resize((size_t)set.count);
     for (size_t k = 0; k < maps.size(); ++k) {
         const size_t i = (size_t)set.members[k];
-        (carried ? set.g_maps[i] : set.h_mats[i].map_g) = maps[k];
+        set.h_mats[i].map_g = maps[k];
+        if (carried) set.g_maps[i] = maps[k];
     }
-    return carried ? FLORA_OK : upload(&set.d_mats, set.h_mats, st);
+    if (!carried) {
+        set.new_maps = true;
+        return upload(&set.d_mats, set.h_mats, st);
+    }
+    return set.d_graph ? upload(&set.d_graph, set.h_mats, st) : FLORA_OK;
+}
+
+// Whether work put on the stream is recorded into a graph instead of run.
+inline bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return status == cudaStreamCaptureStatusActive;
+}
+// The table for launches that are recorded into a graph.  Maps that travel with a launch would be recorded with it, and a replay
+// would go on reading the gradients of that time.  The copy may not become a part of the graph either, so it is made on a
+// stream of its own and waited for; nothing else reads the table yet.
+inline flora_status tc_graph_table(TcSet& set)
+{
+    set.captured = true;
+    if (set.count > GMAPS_MANY || set.d_graph) return FLORA_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaStream_t own = nullptr;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return FLORA_ERR_CUDA;
+    }
+    flora_status rc = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) == cudaSuccess ? upload(&set.d_graph, set.h_mats, own) : FLORA_ERR_CUDA;
+    if (rc == FLORA_OK && cudaStreamSynchronize(own) != cudaSuccess) rc = FLORA_ERR_CUDA;
+    if (own) cudaStreamDestroy(own);
+    if (rc != FLORA_OK) {
+        if (set.d_graph) cudaFree(set.d_graph);
+        set.d_graph = nullptr;
+        cudaGetLastError();
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return rc;
 }
 
 // Blocks per matrix for the element-wise helper kernels (zero, scale): about four elements per thread of the
@@ -1020,10 +1065,11 @@ inline unsigned helper_blocks(const TcSet& set)
 // behind_own_kernel: the kernels before this call on the stream, back to one that everything earlier was complete before, are the
 // library's own (a transfer of several matrices), do not touch G and let their dependents start early: only the write-out of the
 // compression waits for them.
-// one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).
+// one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).  mats: the table of the
+// others; new_maps: its maps may have been written since the kernel before.
 template <bool SINGLE, int MAPS>
-inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, const uint64_t* seeds, float a, float b, cudaStream_t st,
-                                       std::atomic<uint64_t>& launches, bool behind_own_kernel)
+inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
+                                       cudaStream_t st, std::atomic<uint64_t>& launches, bool behind_own_kernel, bool new_maps = false)
 {
     const int r = set.r;
     const float scale = 1.0f / sqrtf((float)r);
@@ -1060,7 +1106,7 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
             attr[0].val.programmaticStreamSerializationAllowed = 1;
             cfg.attrs = attr;
             cfg.numAttrs = early ? 1 : 0;
-            if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<SINGLE>, (const TcMatrix*)set.d_mats, one, ids ? ids + begin : (const int*)nullptr, (int)begin, r, b) != cudaSuccess)
+            if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<SINGLE>, mats, one, ids ? ids + begin : (const int*)nullptr, (int)begin, r, b) != cudaSuccess)
                 return FLORA_ERR_CUDA;
             launches.fetch_add(1, std::memory_order_relaxed);
         }
@@ -1094,18 +1140,17 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
         attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = set.S > 1 ? 2 : 1;
-        const TcMatrix* mats = set.d_mats;
         const K1Item* items = set.d_k1 + begin;
         const int lw = l == 0 ? late_wait : 0;
         cudaError_t e;
         if (pair) {
             const int* slot_table = set.d_slots + set.k1_slots_begin[l];
             e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE, MAPS>, mats, one, gmaps, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
-                                   set.astages, set.S, set.GW, lw);
+                                   set.astages, set.S, set.GW, lw, (int)new_maps);
         } else {
             auto go = [&](auto kernel) {
                 return cudaLaunchKernelEx(&cfg, kernel, mats, one, gmaps, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.lstages,
-                                          set.nsets, set.S, set.GW, set.P, lw);
+                                          set.nsets, set.S, set.GW, set.P, lw, (int)new_maps);
             };
             e = set.f32 ? go(compress_tc_kernel<SINGLE, true, MAPS>) : go(compress_tc_kernel<SINGLE, false, MAPS>);
         }
@@ -1115,12 +1160,16 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix& one, co
     return cudaPeekAtLastError() == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
 
-inline flora_status tc_set_compress(const TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
+inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
                                     bool behind_own_kernel = false)
 {
-    return set.g_maps.empty() ? tc_compress_launch<false, 0>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel)
-           : set.count <= GMAPS_FEW ? tc_compress_launch<false, GMAPS_FEW>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel)
-                                    : tc_compress_launch<false, GMAPS_MANY>(set, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel);
+    if (capturing(st)) {
+        const flora_status rc = tc_graph_table(set);
+        return rc ? rc : tc_compress_launch<false, 0>(set, set.d_graph ? set.d_graph : set.d_mats, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel, true);
+    }
+    return set.g_maps.empty() ? tc_compress_launch<false, 0>(set, set.d_mats, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel, set.new_maps)
+           : set.count <= GMAPS_FEW ? tc_compress_launch<false, GMAPS_FEW>(set, set.d_mats, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel)
+                                    : tc_compress_launch<false, GMAPS_MANY>(set, set.d_mats, TcMatrix{}, seeds, a, b, st, launches, behind_own_kernel);
 }
 
 // Plans of the single-matrix calls.  Planning (work split, device tables of the items) costs far more than a launch, and an
@@ -1227,7 +1276,7 @@ inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_
     std::lock_guard<std::mutex> lock(single_plan_mutex());
     flora_status rc;
     TcSet* set = single_plan(0, *G, *S, st, &rc);
-    return set ? tc_compress_launch<true, 0>(*set, one, &seed, a, b, st, launches, false) : rc;
+    return set ? tc_compress_launch<true, 0>(*set, nullptr, one, &seed, a, b, st, launches, false) : rc;
 }
 
 template <bool SINGLE>

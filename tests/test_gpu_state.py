@@ -319,3 +319,49 @@ def test_gradients_may_move_to_where_tma_cannot_address_them_and_back(kind):
         ref = oracle_decompress(torch.zeros_like(W[i]).cpu(), S[i].cpu(), seeds[i], 0.1, 1.0)
         assert rel_err(values(wl.as_numpy(W[i])), values(ref)) <= TOL[d], i
     fset.close()
+
+
+@pytest.mark.parametrize("dtype,r,shapes", [("bf16", 32, [(512, 4224), (2048, 1536), (1600, 1600)]), ("bf16", 128, [(2048, 2304), (512, 4224)]),
+                                            ("f32", 24, [(512, 4224), (2048, 1536)]), ("bf16", 16, [(256, 384), (200, 136)]), ("f32", 16, [(256, 384), (200, 136)]),
+                                            ("bf16", 8, [(128, 64)] * 193 + [(4096, 2048)])])
+def test_a_graph_of_compressions_follows_rebound_gradients(dtype, r, shapes):
+    """A graph that holds a set's compression reads the gradients that the set has when the graph is launched: recorded before and
+    after a rebind, replayed after others, with ordinary launches in between, on every kernel family and on sets of more matrices
+    than a launch carries addresses for."""
+    count = len(shapes)
+    check = list(range(count)) if count < 10 else [0, 100, count - 1]
+    G = [[wl.gaussian_matrix(n, m, 1e-2, dtype, 10 * t + i).to(DEV) for i, (n, m) in enumerate(shapes)] for t in range(4)]
+    S = [torch.zeros(n, r, device=DEV) for n, _ in shapes]
+    seeds = [fb.flora_derive_seed(5, i, 0) for i in range(count)]
+    fset = fb.FloraSet(G[0], None, S)
+    fset.compress_overwrite(seeds)
+    if dtype == "bf16":
+        fset.rebind_gradients(G[1])                                   # (recorded behind a rebind, or as created)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        fset.compress_overwrite(seeds)
+        fset.compress_accumulate(seeds)
+
+    def holds(t):
+        torch.cuda.synchronize()
+        for i in check:
+            once = torch.from_numpy(oracle_compress(G[t][i], torch.zeros(shapes[i][0], r), seeds[i]))
+            assert rel_err(S[i].cpu().numpy(), oracle_compress(G[t][i], once, seeds[i])) <= TOL[dtype], (t, i)
+
+    graph.replay()
+    holds(1 if dtype == "bf16" else 0)
+    for t in (2, 3):
+        fset.rebind_gradients(G[t])
+        graph.replay()
+        holds(t)
+        fset.compress_overwrite(seeds)
+        fset.compress_accumulate(seeds)
+        holds(t)
+    off = [torch.zeros(n * m + 8, device=DEV, dtype=g.dtype)[1:1 + n * m].view(n, m) for g, (n, m) in zip(G[0], shapes)]
+    with pytest.raises(fb.FloraError, match="FLORA_ERR_ALIGN"):
+        fset.rebind_gradients(off)
+    graph.replay()
+    holds(3)
+    del graph
+    fset.close()
