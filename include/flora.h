@@ -30,8 +30,9 @@
  *    call that meets a new (operation, shape, dtype, rank) on the TMA path
  *    builds its plan (work split, a few KB of device tables) with a device
  *    allocation and a synchronisation of `stream`; the 64 most recent plans
- *    are kept, so a training loop pays this once per shape.  flora_set_*
- *    calls never do: a set is planned when it is created.
+ *    are kept (and those that a CUDA graph uses), so a training loop pays
+ *    this once per shape.  flora_set_* calls never do: a set is planned when
+ *    it is created.
  *  - Stream capture: the set-level transfers (flora_set_resample_transfer,
  *    flora_set_transfer_axpby, flora_set_momentum_step_resampled),
  *    flora_set_rebind_gradients and a single-matrix call that plans upload

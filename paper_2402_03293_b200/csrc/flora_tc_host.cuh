@@ -1176,7 +1176,7 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
 // optimizer calls with the same shapes step after step: the most recent plans are kept, keyed by device, operation, shape and
 // rank.  A plan holds no addresses: the matrix's record with its tensor maps is made anew for every call (0.05 us a map) and
 // passed to the kernels by value, so a loop over a whole model's matrices, or over gradients at new addresses in every step,
-// plans once per shape (a cache keyed by addresses planned every call anew in such loops: 43 us each).  Calls that use the
+// plans once per shape (a plan whose launches have been recorded into a graph is never dropped: the graph reads its tables; a cache keyed by addresses planned every call anew in such loops: 43 us each).  Calls that use the
 // cache are serialised by its mutex; a plan is built with a synchronous upload, so any stream may use it afterwards.
 struct SinglePlanKey {
     int dev, kind, r, det, dtype;
@@ -1189,6 +1189,7 @@ struct SinglePlanKey {
 struct SinglePlan {
     SinglePlanKey key;
     TcSet set;
+    bool recorded = false;                 // a graph holds launches that read its tables: it stays
 };
 constexpr size_t SINGLE_PLAN_CACHE = 64;
 inline std::mutex& single_plan_mutex()
@@ -1221,6 +1222,7 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
                 cache.erase(cache.begin() + i);
                 cache.insert(cache.begin(), hit);
             }
+            hit->recorded = hit->recorded || capturing(st);
             return &hit->set;
         }
     SinglePlan* plan = new (std::nothrow) SinglePlan();
@@ -1249,12 +1251,14 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
         return nullptr;
     }
     cache.insert(cache.begin(), plan);
-    if (cache.size() > SINGLE_PLAN_CACHE) {
-        SinglePlan* old = cache.back();
-        cache.pop_back();
-        tc_set_free(old->set);                                 // cudaFree waits for kernels that still read the tables
-        delete old;
-    }
+    if (cache.size() > SINGLE_PLAN_CACHE)
+        for (size_t i = cache.size(); i-- > 1;)
+            if (!cache[i]->recorded) {
+                tc_set_free(cache[i]->set);                    // cudaFree waits for kernels that still read the tables
+                delete cache[i];
+                cache.erase(cache.begin() + i);
+                break;
+            }
     return &set;
 }
 // The record of one matrix; g / w: which of the big matrix's two maps is wanted.

@@ -365,3 +365,52 @@ def test_a_graph_of_compressions_follows_rebound_gradients(dtype, r, shapes):
     holds(3)
     del graph
     fset.close()
+
+
+def test_graphs_keep_the_plans_of_single_matrix_calls():
+    """A graph reads the device tables of the plans that its calls used: they outlive any number of later shapes."""
+    n, m, r = 512, 8192, 32
+    G, W, S = _g(n, m, 3), torch.zeros(n, m, device=DEV, dtype=torch.bfloat16), torch.zeros(n, r, device=DEV)
+
+    def calls():
+        fb.flora_momentum_step(G, S, 0.0, 9)
+        fb.flora_decompress_apply(W, S, 9, -1.0, 1.0)
+
+    calls()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    for k in range(80):                                               # more shapes than plans are kept of
+        fb.flora_momentum_step(torch.zeros(128, 4224 + 64 * k, device=DEV, dtype=torch.bfloat16), torch.zeros(128, r, device=DEV), 0.0, 9)
+    W.zero_()
+    S.fill_(7.0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert rel_err(S.cpu().numpy(), oracle_compress(G, torch.zeros(n, r), 9)) <= TOL["bf16"]
+    ref = oracle_decompress(torch.zeros_like(W).cpu(), S.cpu(), 9, -1.0, 1.0)
+    assert rel_err(values(wl.as_numpy(W)), values(ref)) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("r", [96, 256])
+def test_single_matrix_calls_of_high_rank_can_be_recorded(r):
+    """Above rank 64 the decompression takes the bf16 copy of the sketch from the pool, also inside a graph."""
+    n, m = 2048, 2304
+    G, W, S = _g(n, m, 3), torch.zeros(n, m, device=DEV, dtype=torch.bfloat16), torch.zeros(n, r, device=DEV)
+
+    def calls():
+        fb.flora_momentum_step(G, S, 0.0, 9)
+        fb.flora_momentum_step_resampled(G, S, 0.5, 9, 10)
+        fb.flora_decompress_apply(W, S, 10, -1.0, 1.0)
+
+    calls()
+    torch.cuda.synchronize()
+    once = W.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    for _ in range(2):
+        W.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert rel_err(values(wl.as_numpy(W)), values(wl.as_numpy(once))) <= 1e-2      # (sums in another order, one bf16 spacing)
