@@ -8,7 +8,9 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include <vector>
 
@@ -120,13 +122,18 @@ bool args(Py_ssize_t n, Py_ssize_t want)
 }
 // Runs a call of the C ABI without the interpreter lock (a first call that plans, or a launch into a full queue, may block)
 // and returns its status.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
 template <typename F>
 PyObject* run(F&& call)
 {
     flora_status s;
-    Py_BEGIN_ALLOW_THREADS
-    s = call();
-    Py_END_ALLOW_THREADS
+    {
+        Unlocked unlocked;
+        s = call();
+    }
     return PyLong_FromLong((long)s);
 }
 
@@ -227,15 +234,11 @@ FN(set_rebind)                       // handle, tensors, stream
     flora_set* h;
     void* st;
     if (!args(n, 3) || !handle(a[0], &h) || !stream(a[2], &st)) return nullptr;
-    PyObject* seq = PySequence_Fast(a[1], "expected a sequence of tensors");
+    THPObjectPtr seq(PySequence_Fast(a[1], "expected a sequence of tensors"));
     if (!seq) return nullptr;
-    std::vector<flora_mat> g((size_t)PySequence_Fast_GET_SIZE(seq));
+    std::vector<flora_mat> g((size_t)PySequence_Fast_GET_SIZE(seq.get()));
     for (size_t i = 0; i < g.size(); ++i)
-        if (!mat(PySequence_Fast_GET_ITEM(seq, (Py_ssize_t)i), &g[i])) {
-            Py_DECREF(seq);
-            return nullptr;
-        }
-    Py_DECREF(seq);
+        if (!mat(PySequence_Fast_GET_ITEM(seq.get(), (Py_ssize_t)i), &g[i])) return nullptr;
     return run([&] { return flora_set_rebind_gradients(h, g.data(), st); });
 }
 FN(set_compress_accumulate)          // handle, count, seeds, stream
@@ -303,7 +306,17 @@ FN(set_momentum_step_resampled)      // handle, count, beta, seeds_old, seeds_ne
     return run([&] { return flora_set_momentum_step_resampled(h, beta, so.data(), sn.data(), st); });
 }
 
-#define ROW(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+// Reading a tensor or asking for the current stream may throw (a tensor without strides, a machine without a GPU): the C++ exception
+// becomes a Python one here, instead of passing through the interpreter's C frames, which ends the process.
+template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    return F(self, a, n);
+    END_HANDLE_TH_ERRORS
+}
+
+#define ROW(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
     ROW(compress_accumulate), ROW(decompress_apply), ROW(momentum_step), ROW(momentum_step_resampled), ROW(resample_transfer),
     ROW(transfer_axpby), ROW(derive_seed), ROW(derive_seeds), ROW(set_rebind), ROW(set_compress_accumulate), ROW(set_momentum_step),

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2402_03293_b200 import binding as fb
 from paper_2402_03293_b200 import hostlogic
@@ -165,3 +166,14 @@ def test_accumulation_feeding_momentum_order():
     assert mom.calls[1][2:] == (0.5, 1.0)
     with pytest.raises(RuntimeError):
         both.apply(0.5)
+
+
+def test_errors_of_torch_reach_the_caller_as_exceptions():
+    """What reading a tensor or asking for the current stream throws in C++ becomes a Python exception (it would end the process)."""
+    empty = torch.zeros(0, 4)
+    if not torch.cuda.is_available():
+        with pytest.raises(Exception):                                # there is no current stream
+            fb.flora_compress_accumulate(empty, empty, 1, 4)
+    with pytest.raises(Exception):
+        fb.flora_momentum_step(torch.eye(4).to_sparse(), empty, 0.5, 1, stream=0)
+    fb.flora_compress_accumulate(empty, empty, 1, 4, stream=0)        # (an empty problem is fine)
