@@ -8,7 +8,6 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libflora.so")
-NATIVE = os.path.join(HERE, "_native.so")                      # Python side of binding.py (argument marshalling), g++ only
 NATIVE_SOURCE = "flora_py.cpp"
 SOURCES = ["flora_api.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -21,24 +20,32 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
+def native_path() -> str:
+    """The Python side of binding.py (argument marshalling).  It reads torch's C++ objects, whose layout belongs to one build of torch
+    and Python: the name says for which it was made, so another one does not load it."""
+    import torch
+    return os.path.join(HERE, f"_native-{sysconfig.get_config_var('SOABI')}-torch{torch.__version__}.so")
+
+
 def build_native(force: bool = False) -> str:
-    """Compile csrc/flora_py.cpp into paper_2402_03293_b200/_native.so (needs libflora.so, which it calls)."""
+    """Compile csrc/flora_py.cpp (g++ only; needs libflora.so, which it calls) where missing or stale."""
+    native = native_path()
     src = os.path.join(CSRC, NATIVE_SOURCE)
     newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(os.path.dirname(HERE), "include", "flora.h")))
-    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
-        return NATIVE
+    if not force and os.path.exists(native) and os.path.getmtime(native) >= newest:
+        return native
     import torch
     root = os.path.dirname(torch.__file__)
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            f"-I{root}/include", f"-I{root}/include/torch/csrc/api/include", "-I/usr/local/cuda/include",
-           f"-I{sysconfig.get_paths()['include']}", src, "-o", NATIVE + ".tmp", f"-L{root}/lib", "-ltorch_python", "-ltorch_cpu", "-lc10",
+           f"-I{sysconfig.get_paths()['include']}", src, "-o", native + ".tmp", f"-L{root}/lib", "-ltorch_python", "-ltorch_cpu", "-lc10",
            "-lc10_cuda", f"-L{HERE}", "-l:libflora.so", "-Wl,-rpath,$ORIGIN"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode:
         print(res.stderr)
-        raise RuntimeError("g++ failed building _native.so")
-    os.replace(NATIVE + ".tmp", NATIVE)
-    return NATIVE
+        raise RuntimeError("g++ failed building the native side of binding.py")
+    os.replace(native + ".tmp", native)
+    return native
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -16,6 +16,8 @@ from typing import List, Optional, Sequence
 
 import torch
 
+from . import _build
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libflora.so")
 
@@ -106,7 +108,7 @@ class _Unloaded:
     def __getattr__(self, name):
         global _native
         load()
-        path = os.path.join(HERE, "_native.so")
+        path = _build.native_path()
         if not os.path.exists(path):
             raise RuntimeError(f"{path} is missing: build the library first (__graft_entry__.build())")
         loader = importlib.machinery.ExtensionFileLoader("_native", path)

@@ -177,3 +177,14 @@ def test_errors_of_torch_reach_the_caller_as_exceptions():
     with pytest.raises(Exception):
         fb.flora_momentum_step(torch.eye(4).to_sparse(), empty, 0.5, 1, stream=0)
     fb.flora_compress_accumulate(empty, empty, 1, 4, stream=0)        # (an empty problem is fine)
+
+
+def test_the_native_side_of_another_torch_is_not_loaded(monkeypatch):
+    from paper_2402_03293_b200 import _build
+    here = _build.native_path()
+    assert os.path.exists(here)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert _build.native_path() != here
+    monkeypatch.setattr(fb, "_native", fb._Unloaded())
+    with pytest.raises(RuntimeError, match="is missing"):
+        fb.flora_derive_seed(1, 2, 3)
