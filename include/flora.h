@@ -167,8 +167,8 @@ flora_status flora_set_destroy(flora_set* set);
 /* Re-point the gradient matrices of a set (same shapes, dtypes and leading dimensions).  Ordered as work on `stream`: the set's
  * earlier launches on that stream use the old gradients, its later ones the new, and so do compressions of the set that a CUDA
  * graph holds when the graph is launched behind the call on that stream.  Two limits, FLORA_ERR_ALIGN otherwise (nothing changes
- * then): the gradients of a set of bf16 matrices that were all aligned to 16 bytes (pointer and ld) and large enough for the
- * TMA kernels must stay so, and once a compression has been recorded into a graph no set may lose that alignment.
+ * then): where all matrices of a set are bf16 with at least 128 rows and 64 columns, the gradients (pointer and ld) and the
+ * sketches aligned to 16 bytes, they must stay so, and once a compression has been recorded into a graph no set may lose that alignment.
  * (Compressions recorded while a gradient of a set with fp32 or mixed matrices lay off 16 bytes keep that address.) */
 flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void* stream);
 

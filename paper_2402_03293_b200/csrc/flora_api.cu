@@ -196,6 +196,7 @@ struct flora_set {
     std::vector<flora_mat> G, W, S;
     int r = 0;
     bool has_G = false, has_W = false;
+    bool aligned_G = false;        // made of bf16 gradients that TMA can address, all of them: such a set takes no others
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
     TcSet tcf;                     // the same for fp32 matrices
     GenSet gen_g[2], gen_w[2];     // the others, by dtype
@@ -221,6 +222,12 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
     if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS) || (compression ? gen_compress_quicker(counted, widest, r, f32) : gen_decompress_quicker(counted, r, f32)))
         std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
+}
+
+static bool all_addressable(const std::vector<flora_mat>& G, const std::vector<flora_mat>& S)
+{
+    const std::vector<uint8_t> ok = tc_eligible(G, S);
+    return !ok.empty() && std::find(ok.begin(), ok.end(), (uint8_t)0) == ok.end();
 }
 
 // Builds the work lists of a set.
@@ -408,6 +415,7 @@ flora_status flora_set_create(int count, const flora_mat* G, const flora_mat* W,
     s->S.assign(S, S + count);
     if (G) s->G.assign(G, G + count);
     if (W) s->W.assign(W, W + count);
+    s->aligned_G = s->has_G && all_addressable(s->G, s->S);
     flora_status st = set_build(s);
     if (st) {
         flora_set_destroy(s);
@@ -441,11 +449,12 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
         if (G[i].dtype != set->G[i].dtype) return FLORA_ERR_DTYPE;
     }
     std::vector<flora_mat> newG(G, G + set->G.size());
-    // A set of any other kind than bf16 matrices that TMA serves takes any address.  Where TMA cannot address one of the new
-    // gradients, the matrices of its kind are compressed one by one until a later call brings addresses that it can: those launches
-    // carry the matrix by value, so nothing is allocated, planned or waited for here.
+    // A set whose gradients were all bf16 matrices that TMA can address takes no others, whichever kernels serve it; any other set
+    // takes any address.  Where TMA cannot address one of its new gradients, the matrices of the kind are compressed one by one until
+    // a later call brings addresses that it can: those launches carry the matrix by value, so nothing is allocated, planned or waited
+    // for here.
+    if (set->aligned_G && !all_addressable(newG, set->S)) return FLORA_ERR_ALIGN;
     const bool tc_ok = tc_set_addressable(set->tc, newG), tcf_ok = tc_set_addressable(set->tcf, newG);
-    if ((!tc_ok || !tcf_ok) && !(set->gen_g[0].ready() || set->gen_g[1].ready() || set->tcf.compress_ready)) return FLORA_ERR_ALIGN;
     // launches that a graph holds read the gradients through the set's tables, with the kernels of the time they were recorded at
     if ((!tc_ok && set->tc.captured) || (!tcf_ok && set->tcf.captured) || !gen_set_rebindable(set->gen_g[0], newG) || !gen_set_rebindable(set->gen_g[1], newG))
         return FLORA_ERR_ALIGN;

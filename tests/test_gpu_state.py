@@ -414,3 +414,19 @@ def test_single_matrix_calls_of_high_rank_can_be_recorded(r):
         graph.replay()
         torch.cuda.synchronize()
         assert rel_err(values(wl.as_numpy(W)), values(wl.as_numpy(once))) <= 1e-2      # (sums in another order, one bf16 spacing)
+
+
+@pytest.mark.parametrize("shapes", [[(256, 384), (200, 136)], [(512, 4224), (2048, 2304)]])
+def test_a_set_of_aligned_bf16_matrices_takes_aligned_gradients_only(shapes):
+    """Large or small, whichever kernels serve it; a refused call leaves the set as it was."""
+    r = 16
+    G = [_g(n, m, 3 + i) for i, (n, m) in enumerate(shapes)]
+    S = [torch.zeros(n, r, device=DEV) for n, _ in shapes]
+    fset = fb.FloraSet(G, None, S)
+    off = [torch.zeros(n * m + 8, device=DEV, dtype=torch.bfloat16)[1:1 + n * m].view(n, m) for n, m in shapes]
+    with pytest.raises(fb.FloraError, match="FLORA_ERR_ALIGN"):
+        fset.rebind_gradients([G[0], off[1]])
+    fset.compress_overwrite([5, 6])
+    for i, (n, m) in enumerate(shapes):
+        assert rel_err(S[i].cpu().numpy(), oracle_compress(G[i], torch.zeros(n, r), 5 + i)) <= TOL["bf16"], i
+    fset.close()
