@@ -210,6 +210,8 @@ constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
 static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression, bool f32 = false)
 {
     std::vector<uint8_t> use = tc_eligible(big, S, f32);
+    if (compression && f32)
+        for (size_t i = 0; i < big.size(); ++i) use[i] = use[i] && big[i].cols >= K1_F32_MIN_COLS;
     int64_t eligible = 0, widest = 0;
     bool mixed = false;
     for (size_t i = 0; i < big.size(); ++i) {

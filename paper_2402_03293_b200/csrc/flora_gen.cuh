@@ -37,6 +37,7 @@ struct GenItem {           // compression: one cluster
 __host__ __device__ constexpr int gen_threads(int workers) { return 32 * (workers + 1); }
 constexpr int GEN_G_SLOTS_MAX = 8, GEN_A_SLOTS_MAX = 4;
 constexpr int GEN_L2_AHEAD = 8;                             // steps of a tile that a CTA asks into L2 before it may load them
+constexpr int GEN_F32_CHAIN_STEPS = 72;                     // steps of an fp32 matrix that a CTA adds up at most
 constexpr int GEN_MAX_SPLIT = 16;                           // CTAs that share the columns of a row group (above 8: not a portable cluster size)
 
 // The parts of two fp32 values, as fp32 bit patterns whose low 16 bits are to be dropped.

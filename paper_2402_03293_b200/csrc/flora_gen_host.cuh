@@ -25,9 +25,9 @@ inline bool gen_aligned(const flora_mat& g)
     return ((reinterpret_cast<uintptr_t>(g.data) | (uintptr_t)(g.ld * es)) & 15) == 0;
 }
 
-// Steps of 32 columns that a CTA adds up for fp32 matrices (two truncated accumulations of large products each, 2e-8 of the sum lost
-// in every one: 3e-6, what plain rounded fp32 loses over 10^4 products).
-constexpr int GEN_F32_CHAIN_STEPS = 72;
+// Steps of 32 columns that a CTA adds up for fp32 matrices: two truncated accumulations of large products each, 3.7e-8 of the sum
+// lost in every step as measured; the three-part products are off by 6e-8.
+inline int64_t gen_f32_chain(int64_t steps) { return std::min<int64_t>(GEN_F32_CHAIN_STEPS, f32_chain(32 * steps, 3.7e-8, 6e-8)); }
 // Rings, accumulator layout and CTAs per SM for T tiles per CTA; false where they do not fit.  `per_sm` = 2: two CTAs with at
 // most 112 KB and 256 accumulator columns each.  At least three slots of G and two of A (with fewer the warps wait for the MMAs of
 // the step before: fp32 4096 x 11008 at r = 8 ran at half the speed).
@@ -101,7 +101,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
         for (int split = 1; split <= GEN_MAX_SPLIT; ++split)
             for (int workers = 8; workers <= 16; workers += 8) {
                 if ((T > 1 && tiles < T) || (split > 1 && steps < split)) continue;
-                if (f32 && split < GEN_MAX_SPLIT && steps > (int64_t)GEN_F32_CHAIN_STEPS * split) continue;
+                if (f32 && split < GEN_MAX_SPLIT && steps > gen_f32_chain(steps) * split) continue;
                 if (tune_knob("FLORA_GEN_T", T, 1, 4) != T || tune_knob("FLORA_GEN_SPLIT", split, 1, 16) != split ||
                     tune_knob("FLORA_GEN_WORKERS", workers, 8, 16) != workers)
                     continue;
@@ -356,7 +356,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             for (int i : ids) {
                 const int64_t steps = (big[i].cols + K - 1) / K;
                 split[i] = 1;
-                while (split[i] < most && (steps > share * split[i] * 3 / 2 || (s.f32 && steps > (int64_t)GEN_F32_CHAIN_STEPS * split[i])) && steps >= 2 * split[i])
+                while (split[i] < most && (steps > share * split[i] * 3 / 2 || (s.f32 && steps > gen_f32_chain(steps) * split[i])) && steps >= 2 * split[i])
                     split[i] *= 2;
                 cluster = std::max(cluster, split[i]);
             }
@@ -379,7 +379,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             for (int i : ids) {
                 const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = cluster / split[i];
                 if (tiles == 0) continue;
-                chains = chains && !(s.f32 && split[i] < GEN_MAX_SPLIT && steps > (int64_t)GEN_F32_CHAIN_STEPS * split[i]);
+                chains = chains && !(s.f32 && split[i] < GEN_MAX_SPLIT && steps > gen_f32_chain(steps) * split[i]);
                 const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, per_sm, 1, (steps + split[i] - 1) / split[i], cluster);
                 work.insert(work.end(), (size_t)((tiles + per - 1) / per), cost);
             }

@@ -140,7 +140,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
     // accumulator of a tile; F32: hi hi in the first r_pad columns, the small products in the next
     const int acc_cols = F32 ? 2 * r_pad : r_pad;
     // F32: steps that share a pair of accumulators, and how many pairs an item uses
-    const int per_set = F32 ? max(16, (items[blockIdx.x].ksteps + nsets - 1) / nsets) : 1;
+    const int per_set = F32 ? max(4, (items[blockIdx.x].ksteps + nsets - 1) / nsets) : 1;
     // two rings (F32: three): G tiles (gstages x T tiles; the loads come from HBM and want many bytes in flight) and A tiles
     // (astages x r_pad rows; produced on chip).  Each has its own full / empty barriers.
     const uint32_t g_bytes = (uint32_t)T * G_TILE_BYTES;

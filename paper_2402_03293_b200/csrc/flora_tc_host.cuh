@@ -28,7 +28,7 @@ struct TcSet {
     bool compress_ready = false;
     bool decompress_ready = false;
     int count = 0, r = 0;
-    bool f32 = false;                   // fp32 matrices (compression only)
+    bool f32 = false;                   // fp32 gradients
     int T = 1, gstages = 2, astages = 2, lstages = 1, nsets = 1, S = 1, GW = 8, P = 1;
     std::vector<int> k1_launch_first_mat;
     size_t k1_smem = 0;
@@ -111,6 +111,9 @@ inline bool tc_mat_ok(const flora_mat& a)
 
 // fp32 weights: the slabs of A (two parts, 64 columns) of larger ranks leave no room for two tiles of W and four chunks of the sketch
 constexpr int K2_F32_MAX_R = 128;
+// fp32 gradients: the products of compress_tc_kernel<F32> alone are off by as much as a plain fp32 sum of some 60 columns, which leaves
+// narrow matrices too little room for its truncated sums (k1_f32_chain); gen_compress_kernel takes those.
+constexpr int64_t K1_F32_MIN_COLS = 512;
 // fp32 matrices
 inline bool tc_f32_ok(const flora_mat& a)
 {
@@ -120,7 +123,7 @@ inline bool tc_f32_ok(const flora_mat& a)
 
 inline bool tc_compress_supported(const flora_mat* big, const flora_mat* sketch)
 {
-    return (tc_mat_ok(*big) || tc_f32_ok(*big)) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
+    return (tc_mat_ok(*big) || (tc_f32_ok(*big) && big->cols >= K1_F32_MIN_COLS)) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
 }
 
 // SMs of the current device (a process may drive several devices), asked once per device.
@@ -224,9 +227,18 @@ constexpr double K1_UNIT_OVERHEAD_STEPS = 6.0;
 // time that one element of a 128-row G tile costs its CTA (measured: an r x 64 tile takes about r * 64 * 0.18 ns of
 // one SM's ALUs, the 16 KB of a G tile 0.37 us of its share of HBM, and the ratio of the two per rank is about 0.045 / T).
 constexpr double K1_GENERATION_PER_RANK = 0.045;
-// Steps of 32 columns that an fp32 item may add into one accumulator: four accumulations each, 2e-8 of the sum lost in every one
-// of them, so at most 4e-6 and 1.2e-6 as measured (a sum of 10^4 products in plain rounded fp32 is off by 2.5e-6).
-constexpr int K1_F32_CHAIN_STEPS = 48;
+// Steps of 32 columns that an fp32 compression over `cols` columns may add into one accumulator.  The tensor core truncates its sums:
+// each accumulation loses a little of the running sum, always towards zero, so the loss grows with their number.  Errors against
+// 64 bits in the 2-norm, measured on normal G: plain fp32 arithmetic 1.8e-8 sqrt(cols), so the chain is kept so short that the loss
+// (`per_step`) and the error of the products (`products`) together stay below that.  (Chains of 48 steps whatever the columns,
+// 40000 x 3072 at r = 96: 3.6e-6, plain fp32 1.0e-6.)
+inline int64_t f32_chain(int64_t cols, double per_step, double products)
+{
+    const double plain = 0.9 * 1.8e-8, room = plain * plain * (double)cols - products * products;
+    return std::max<int64_t>(1, room > 0 ? (int64_t)(sqrt(room) / per_step) : 0);
+}
+// compress_tc_kernel<F32>: four accumulations a step, 6.7e-8; its products are hi hi + hi lo + lo hi, 1.4e-7
+inline int64_t k1_f32_chain(int64_t cols) { return std::min<int64_t>(48, f32_chain(cols, 6.7e-8, 1.4e-7)); }
 // Cost model of the decompression planner (microseconds on one SM): bytes an SM takes in per microsecond whatever their
 // source (about 60 GB/s with the tiles it can keep in flight), values of A per microsecond that the generator warps
 // make next to the streaming warps (8 or fewer warps), the share of a slab's generation that stays exposed with one
@@ -488,7 +500,6 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
     if (f32 && GW != 8 && GW != 16) GW = 8;                       // (the threads divide a tile's 16-byte pieces)
     set.GW = GW;
     set.nsets = f32 ? std::max(1, std::min(8, (per_sm == 2 ? 256 : 512) / (T * acc_cols))) : 1;
-    const int64_t max_chunk = f32 && !deterministic_flag().load() ? (int64_t)K1_F32_CHAIN_STEPS * set.nsets : (int64_t)1 << 60;
     // generator teams: as many as keep every thread of a team busy with at least one task per tile
     {
         const int tile_tasks = (S > 1 ? r_pad / S : r) * 8;
@@ -519,6 +530,7 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
             const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + kc - 1) / kc;
             const int64_t groups = (tiles + group_tiles - 1) / group_tiles;
             const int64_t per_group = (tiles + groups - 1) / groups;     // rows spread evenly over the groups
+            const int64_t max_chunk = f32 ? k1_f32_chain(g.cols) * set.nsets : (int64_t)1 << 60;
             int64_t chunk = std::min(max_chunk, std::max<int64_t>(8, target / per_group));
             int64_t nchunks = (ks + chunk - 1) / chunk;
             if (nchunks > 1 && ks - (nchunks - 1) * chunk < chunk / 2 && (ks + nchunks - 2) / (nchunks - 1) <= max_chunk) --nchunks;    // no short tail item
