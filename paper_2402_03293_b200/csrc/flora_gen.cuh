@@ -566,7 +566,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                       const __grid_constant__ SeedTable seeds, const __grid_constant__ GenMat single, int seed_base, int r, float scale, float step)
 {
     constexpr int PARTS = F32 ? 3 : 1, ROWB = 2 * KB;
-    constexpr uint32_t TMEM_COLS = F32 ? 2 * BN : BN;             // fp32: the large products, and the small ones (see the compression)
+    constexpr uint32_t TMEM_COLS = F32 ? 4 * BN : BN;             // fp32: the large products of even slices, the small ones, the large of odd slices
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     __shared__ GenK2Smem ctl;
@@ -746,7 +746,8 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                             }
                             ptx::umma_bf16(minor, ds + sp + kk * 2, da + kk * 2, id, 1u);                          // m h
                             if (F32) ptx::umma_bf16(minor, ds + kk * 2, da + ap + kk * 2, id, 1u);                 // h m
-                            ptx::umma_bf16(tmem, ds + kk * 2, da + kk * 2, id, F32 ? on : 1u);                     // h h
+                            // h h (fp32: two accumulators in turn, which halves what their truncated sums lose)
+                            ptx::umma_bf16(tmem + (F32 ? (kk & 1) * 2 * BN : 0), ds + kk * 2, da + kk * 2, id, F32 ? (uint32_t)(kc != 0 || kk > 1) : 1u);
                         }
                         ptx::umma_commit(ptx::smem_addr(&ctl.done));
                     }
@@ -771,11 +772,17 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                     uint32_t v[16];
                     ptx::tmem_ld_16(at + c, v);
                     if (F32) {
-                        uint32_t y[16];
+                        uint32_t y[16], z[16];
                         ptx::tmem_ld_16(at + BN + c, y);
+                        if (r > 16) {
+                            ptx::tmem_ld_16(at + 2 * BN + c, z);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) z[k] = 0u;
+                        }
                         ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int k = 0; k < 16; ++k) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(y[k]));
+                        for (int k = 0; k < 16; ++k) v[k] = __float_as_uint((__uint_as_float(v[k]) + __uint_as_float(z[k])) + __uint_as_float(y[k]));
                     } else {
                         ptx::tmem_ld_wait();
                     }

@@ -648,8 +648,10 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
 }
 
 // F32: W is fp32.  Both operands are cut into what tf32 holds, rounded, and the rest, x = hi + lo; of the four products lo lo is left
-// out (2^-23), S_hi multiplies hi and lo of A side by side as one operand of 2 bn rows, and the small products have an accumulator to
-// themselves (the tensor core truncates its sums).  Four warps cut the sketch's chunks in shared memory.  W's boxes are 32 columns wide.
+// out (2^-24 at most, the products together are off by 7e-8 in the 2-norm), S_hi multiplies hi and lo of A side by side as one operand of 2 bn
+// rows, and the small products have accumulators to themselves.  The tensor core truncates its sums, and the loss grows with the length
+// of the chain: slices of eight columns take two pairs of accumulators in turn (W after a step of 5 %, against 64 bits: r = 128 3.06e-8
+// with one pair, plain fp32 arithmetic 2.70e-8).  Four warps cut the sketch's chunks in shared memory.  W's boxes are 32 columns wide.
 template <bool SINGLE, bool BF16S, bool F32>
 __global__ void __launch_bounds__(K2_MAX_THREADS, 1)
 decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K2Item* __restrict__ items, int n_items,
@@ -672,8 +674,8 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     const uint32_t slot_bytes = (uint32_t)boxes * W_BOX_BYTES;
     K2Smem* ctl = reinterpret_cast<K2Smem*>(smem_raw + (w_ring - ptx::smem_addr(smem_raw)) + (size_t)slots * slot_bytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int acc_cols = F32 ? 2 * bn : bn;                    // columns of one of the two accumulators
-    const uint32_t tmem_cols = 2u * (uint32_t)acc_cols;        // 256 or 128: a power of two >= 32
+    const int acc_cols = F32 ? 4 * bn : bn;                    // columns of one of the two accumulators (F32: two pairs, large and small products)
+    const uint32_t tmem_cols = 2u * (uint32_t)acc_cols;        // 512, 256 or 128
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < slots; ++s) {
@@ -801,9 +803,10 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                             const uint64_t da = desc_ring + (uint64_t)((s * S_CHUNK_BYTES) >> 4), dl = desc_ring + (uint64_t)((l_ring - c_ring + pl.s * S_CHUNK_BYTES) >> 4);
                             const uint64_t db = desc_slab + (uint64_t)((kc * slab_block) >> 4);
 #pragma unroll
-                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(acc_addr, da + k8 * 2, db + k8 * 2, ptx::umma_idesc_tf32(2u * bn), (kc | k8) != 0);   // hi hi | hi lo
+                            for (int k8 = 0; k8 < 4; ++k8)                                                                         // hi hi | hi lo
+                                ptx::umma_tf32(acc_addr + (k8 & 1) * 2 * bn, da + k8 * 2, db + k8 * 2, ptx::umma_idesc_tf32(2u * bn), kc != 0 || k8 > 1);
 #pragma unroll
-                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(acc_addr + bn, dl + k8 * 2, db + k8 * 2, idesc, 1u);                                  //       | lo hi
+                            for (int k8 = 0; k8 < 4; ++k8) ptx::umma_tf32(acc_addr + (k8 & 1) * 2 * bn + bn, dl + k8 * 2, db + k8 * 2, idesc, 1u);   // | lo hi
                             ptx::umma_commit(ptx::smem_addr(&ctl->c_empty[s]));
                             ptx::umma_commit(ptx::smem_addr(&ctl->l_empty[pl.s]));
                             pl.advance(K2_LSTAGES);
@@ -906,8 +909,16 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                         const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + (gt & 1) * acc_cols + c16 * 16;
                         uint32_t v[16], y[16];
                         ptx::tmem_ld_16(at, v);
-                        ptx::tmem_ld_16(at + bn, y);
+                        ptx::tmem_ld_16(at + 2 * bn, y);
                         ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) v[u] = __float_as_uint(__uint_as_float(v[u]) + __uint_as_float(y[u]));
+                        uint32_t z[16];
+                        ptx::tmem_ld_16(at + bn, y);
+                        ptx::tmem_ld_16(at + 3 * bn, z);
+                        ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) y[u] = __float_as_uint(__uint_as_float(y[u]) + __uint_as_float(z[u]));
                         const uint32_t box = wrow + (c16 >> 1) * W_BOX_BYTES;
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
