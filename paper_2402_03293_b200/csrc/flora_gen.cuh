@@ -30,7 +30,7 @@ struct GenItem {           // compression: one cluster
     int32_t mat;
     int32_t tile0;         // first 128-row tile
     int32_t split;         // CTAs of the cluster that share the columns of one row group
-    int32_t pad;
+    int32_t col0;          // first column (fp32: a launch takes GEN_F32_PASS_COLS columns)
 };
 
 // Warps that load, convert, generate and write out (8, or 16 where a CTA has an SM to itself), and one that issues the MMAs.
@@ -39,6 +39,9 @@ constexpr int GEN_G_SLOTS_MAX = 8, GEN_A_SLOTS_MAX = 4;
 constexpr int GEN_L2_AHEAD = 8;                             // steps of a tile that a CTA asks into L2 before it may load them
 constexpr int GEN_F32_CHAIN_STEPS = 72;                     // steps of an fp32 matrix that a CTA adds up at most
 constexpr int GEN_MAX_SPLIT = 16;                           // CTAs that share the columns of a row group (above 8: not a portable cluster size)
+// Columns of an fp32 matrix that one launch adds up: as many as keep every CTA's chain within its limit.  Wider matrices take several
+// launches, whose sums are added in rounded fp32 (one after another, so in a fixed order).
+constexpr int GEN_F32_PASS_COLS = 32 * GEN_MAX_SPLIT * GEN_F32_CHAIN_STEPS;
 
 // The parts of two fp32 values, as fp32 bit patterns whose low 16 bits are to be dropped.
 struct Parts2 {
@@ -130,7 +133,7 @@ __host__ __device__ inline int gen_stage_stride(int r_pad) { return r_pad + 4; }
 template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 __global__ void __launch_bounds__(gen_threads(WORKERS), WORKERS == 8 ? 2 : 1)
 gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
-                    const __grid_constant__ GenMat single, int single_split, int seed_base, int r, float scale, float a, float b, int T, int sbs,
+                    const __grid_constant__ GenMat single, int single_split, int single_col0, int seed_base, int r, float scale, float a, float b, int T, int sbs,
                     int g_slots, int a_slots, int cluster)
 {
     using C = GenK1<F32>;
@@ -154,13 +157,15 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         item.mat = 0;
         item.split = single_split;
         item.tile0 = cl * (cluster / single_split) * T;
+        item.col0 = single_col0;
     }
     const GenMat mat = SINGLE ? single : mats[item.mat];
     const int split = item.split, group = rank / split, part = rank % split;
     const int tile0 = item.tile0 + group * T;
     const int tiles = max(0, min(T, ((mat.n + 127) >> 7) - tile0));
-    const int all_steps = (mat.m + C::K - 1) / C::K;
-    const int ks0 = (int)((int64_t)part * all_steps / split), ks1 = (int)((int64_t)(part + 1) * all_steps / split);
+    const int m_end = F32 ? item.col0 + min(mat.m - item.col0, GEN_F32_PASS_COLS) : mat.m;      // columns beyond it are another launch's
+    const int all_steps = (m_end - item.col0 + C::K - 1) / C::K, step0 = item.col0 / C::K;
+    const int ks0 = step0 + (int)((int64_t)part * all_steps / split), ks1 = step0 + (int)((int64_t)(part + 1) * all_steps / split);
     const int steps = tiles > 0 ? ks1 - ks0 : 0;
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < T * acc_cols) tmem_cols <<= 1;
@@ -256,7 +261,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         const uint32_t low0 = (uint32_t)reinterpret_cast<uintptr_t>(fp), low_step = (uint32_t)row_step;      // for the pieces' alignment
         const uint8_t* fstep = fp;                                  // fetch cursor: this thread's piece of row 0 of the tile; of tile 0 of the step
         int fks = 0, ft = 0, pks = 0, pt = 0;                       // fetch and place cursors: step, tile
-        auto left_at = [&](int ks) { return mat.m - ((ks0 + ks) * C::K + piece * E); };      // elements from this thread's piece on
+        auto left_at = [&](int ks) { return m_end - ((ks0 + ks) * C::K + piece * E); };      // elements from this thread's piece on
         auto fetch = [&](uint4 (&x)[NI][BLK]) {                     // the pieces of this thread of the tile at the fetch cursor
             const int bytes = min(16, left_at(fks) * ES);
             const uint8_t* p = fp;

@@ -128,7 +128,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
 
 template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds, const GenMat& one,
-                                 int split, int seed_base, int r, float a, float b, cudaStream_t st)
+                                 int split, int col0, int seed_base, int r, float a, float b, cudaStream_t st)
 {
     if (!raise_smem_limit<gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>>(true)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
@@ -145,14 +145,14 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, seeds, one, split, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
+    return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, seeds, one, split, col0, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
                               (int)p.sbs, p.g_slots, p.a_slots, p.cluster);
 }
 inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds,
-                                        const GenMat& one, int split, int seed_base, int r, float a, float b, cudaStream_t st,
+                                        const GenMat& one, int split, int col0, int seed_base, int r, float a, float b, cudaStream_t st,
                                         std::atomic<uint64_t>& launches)
 {
-    auto go = [&](auto launch) { return launch(p, clusters, mats, items, seeds, one, split, seed_base, r, a, b, st); };
+    auto go = [&](auto launch) { return launch(p, clusters, mats, items, seeds, one, split, col0, seed_base, r, a, b, st); };
     cudaError_t e;
 #define FLORA_GEN_K1(SINGLE, F32, ALIGNED) (p.workers == 16 ? go(gen_launch_k1<SINGLE, F32, ALIGNED, 16>) : go(gen_launch_k1<SINGLE, F32, ALIGNED, 8>))
     if (items) e = f32 ? (p.aligned ? FLORA_GEN_K1(false, true, true) : FLORA_GEN_K1(false, true, false))
@@ -203,13 +203,21 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
 {
     const bool f32 = G.dtype == FLORA_F32;
     const int r = (int)S.cols;
-    const int64_t tiles = (G.rows + 127) / 128, steps = (G.cols + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
+    const int64_t pass = f32 ? GEN_F32_PASS_COLS : G.cols;
+    const int64_t tiles = (G.rows + 127) / 128, steps = (std::min(G.cols, pass) + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
     GenK1Plan p = gen_k1_choose(f32, r, tiles, steps);
     const int64_t groups = (tiles + p.T - 1) / p.T;
     p.aligned = gen_aligned(G);
     SeedTable table;
     table.s[0] = seed;
-    return gen_compress_launch(f32, p, (int)groups, nullptr, nullptr, table, gen_mat(G, S), p.cluster, 0, r, a, b, st, launches);
+    int64_t col0 = 0;
+    do {                                                          // (a matrix without columns: one launch, S <- b S)
+        const flora_status rc = gen_compress_launch(f32, p, (int)groups, nullptr, nullptr, table, gen_mat(G, S), p.cluster, (int)col0, 0, r, a,
+                                                    col0 ? 1.0f : b, st, launches);
+        if (rc) return rc;
+        col0 += pass;
+    } while (col0 < G.cols);
+    return FLORA_OK;
 }
 
 // Decompression: slabs of 128 columns for bf16 matrices whose rows move in 16-byte pieces, of 64 otherwise (an element-wise
@@ -291,6 +299,7 @@ struct GenSet {
     GenK2Item* d_k2 = nullptr;
     int* d_share = nullptr;                    // decompression: per launch, the first item of every CTA and the end
     std::vector<int> begin, first_mat;         // compression: ranges of items per launch; decompression: where its table starts in d_share
+    std::vector<uint8_t> adds;                 // compression: launches behind the first columns of their matrices, which add to them
     std::vector<unsigned> grid;                // decompression: CTAs per launch
     int bn = 64;
     GenK1Plan plan;
@@ -320,9 +329,9 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     if (rc) return rc;
     struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
-    auto launches_of = [&](auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
+    int count = 0;
+    auto launches_of = [&](bool adds, auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
         size_t u0 = 0;
-        int count = 0;
         while (u0 < cuts.size()) {
             size_t u1 = u0;
             const int first = cuts[u0].mat;
@@ -330,18 +339,24 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             std::stable_sort(cuts.begin() + u0, cuts.begin() + u1, [](const Cut& x, const Cut& y) { return x.work > y.work; });
             s.begin.push_back(count);
             s.first_mat.push_back(first);
+            s.adds.push_back(adds ? 1 : 0);
             for (size_t u = u0; u < u1; ++u, ++count) emit(cuts[u]);
             u0 = u1;
         }
-        s.begin.push_back(count);
     };
     const int64_t sms = sm_count();
     if (kind == 0) {
         const int K = s.f32 ? 32 : 64;
-        int64_t total = 0;
+        // columns of matrix i that launch `pass` takes, in steps
+        auto steps_of = [&](int i, int64_t pass) {
+            const int64_t left = s.f32 ? std::min<int64_t>(big[i].cols - pass * GEN_F32_PASS_COLS, GEN_F32_PASS_COLS) : big[i].cols;
+            return (std::max<int64_t>(0, left) + K - 1) / K;
+        };
+        int64_t total = 0, passes = 1;
         for (int i : ids) {
             const int64_t tiles = (big[i].rows + 127) / 128;
-            total += tiles * ((big[i].cols + K - 1) / K);
+            total += tiles * steps_of(i, 0);
+            if (s.f32) passes = std::max(passes, (big[i].cols + GEN_F32_PASS_COLS - 1) / GEN_F32_PASS_COLS);
             s.plan.aligned = s.plan.aligned && gen_aligned(big[i]);
         }
         // One kind of CTA for the whole list: one tile, eight warps, two to an SM, where that fits (more tiles to share a tile of A
@@ -354,7 +369,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         auto cut_columns = [&](int most) {       // CTAs along the columns per matrix, and clusters that makes
             cluster = 1;
             for (int i : ids) {
-                const int64_t steps = (big[i].cols + K - 1) / K;
+                const int64_t steps = steps_of(i, 0);
                 split[i] = 1;
                 while (split[i] < most && (steps > share * split[i] * 3 / 2 || (s.f32 && steps > gen_f32_chain(steps) * split[i])) && steps >= 2 * split[i])
                     split[i] *= 2;
@@ -377,7 +392,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             std::vector<double> work;
             bool chains = true;                                   // no fp32 sum longer than it may be
             for (int i : ids) {
-                const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = cluster / split[i];
+                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, 0), per = cluster / split[i];
                 if (tiles == 0) continue;
                 chains = chains && !(s.f32 && split[i] < GEN_MAX_SPLIT && steps > gen_f32_chain(steps) * split[i]);
                 const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, per_sm, 1, (steps + split[i] - 1) / split[i], cluster);
@@ -403,13 +418,19 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         const int T = 1;
         if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
-        for (int i : ids) {
-            const int64_t tiles = (big[i].rows + 127) / 128, steps = (big[i].cols + K - 1) / K, per = (int64_t)(cluster / split[i]) * T;
-            for (int64_t t0 = 0; t0 < tiles; t0 += per)
-                cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]), {i, (int32_t)t0, split[i], 0}});
-        }
         std::vector<GenItem> items;
-        launches_of([&](const Cut& c) { items.push_back(c.item); });
+        for (int64_t pass = 0; pass < passes; ++pass) {
+            cuts.clear();
+            for (int i : ids) {
+                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass), per = (int64_t)(cluster / split[i]) * T;
+                if (pass > 0 && steps == 0) continue;
+                for (int64_t t0 = 0; t0 < tiles; t0 += per)
+                    cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]),
+                                    {i, (int32_t)t0, split[i], s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0}});
+            }
+            launches_of(pass > 0, [&](const Cut& c) { items.push_back(c.item); });
+        }
+        s.begin.push_back(count);
         return upload(&s.d_k1, items, nullptr);
     }
     // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
@@ -462,7 +483,8 @@ inline flora_status gen_set_compress(GenSet& s, const uint64_t* seeds, float a, 
     if (s.ready() && s.plan.aligned && !s.captured_aligned) s.captured_aligned = capturing(st);
     for (size_t l = 0; l + 1 < s.begin.size(); ++l) {
         const flora_status rc = gen_compress_launch(s.f32, s.plan, s.begin[l + 1] - s.begin[l], s.d_mats, s.d_k1 + s.begin[l],
-                                                    gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, s.first_mat[l], s.r, a, b, st, launches);
+                                                    gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, 0, s.first_mat[l], s.r, a, s.adds[l] ? 1.0f : b, st,
+                                                    launches);
         if (rc) return rc;
     }
     return FLORA_OK;

@@ -167,3 +167,34 @@ def test_transfer_edges(n, m, r, operand):
     assert all(((x.double() - want).norm() / size(want, 1.0, 0.0)).item() <= tol for x in (S[0], fixed))
     fset.close()
     assert fb.flora_device_status() == 0
+
+
+# Rows longer than one launch may add up (36864 columns: sixteen CTAs of 72 steps), around its end and over many of them, off 16 bytes
+# and, in bit-reproducible mode, on; the result stays as near to 64 bits as plain fp32 arithmetic (1.8e-8 sqrt(m) in the 2-norm; one
+# chain of truncated sums over 600001 columns would lose 4e-5).
+@pytest.mark.parametrize("n,m,r", [(3, 36863, 8), (130, 36865, 33), (16, 73729, 8), (5, 600001, 4), (128, 50256, 16)])
+def test_long_fp32_rows(n, m, r):
+    G = wl.gaussian_matrix(n, m, 1e-2, "f32", 9).to(DEV)
+    A = torch.empty(r, m, device=DEV)
+    fb.flora_materialize_A(A, 31)
+    product = G.double() @ A.double().T
+    S0 = torch.randn(n, r, generator=torch.Generator(device=DEV).manual_seed(m), device=DEV)
+    fb.flora_set_deterministic(True)
+    try:
+        alone, again = S0.clone(), S0.clone()
+        fb.flora_momentum_step(G, alone, 0.75, 31)
+        fb.flora_momentum_step(G, again, 0.75, 31)
+        member, other = S0.clone(), torch.ones(40, r, device=DEV)
+        small = wl.gaussian_matrix(40, 300, 1e-2, "f32", 8).to(DEV)
+        other0 = other.clone()
+        fset = fb.FloraSet([small, G], None, [other, member])
+        fset.momentum_step(0.75, [32, 31])
+    finally:
+        fb.flora_set_deterministic(False)
+    want = 0.75 * S0.double() + 0.25 * product
+    for x in (alone, member):
+        assert ((x.double() - want).norm() / want.norm()).item() <= 1.8e-8 * m ** 0.5 + 2.0 ** -23
+    assert torch.equal(alone, again)
+    assert rel_err(other.cpu().numpy(), oracle_compress(small, other0, 32, a=0.25, b=0.75)) <= TOL["f32"]
+    fset.close()
+    assert fb.flora_device_status() == 0
