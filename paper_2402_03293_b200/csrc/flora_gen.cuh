@@ -82,12 +82,19 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t addr)
     d |= (uint64_t)(ROWB == 64 ? 4 : 2) << 61;              // 64- or 128-byte swizzle
     return d;
 }
-// Stores four fp32 values as `PARTS` (3: exact cut, 1: rounded to bf16) bf16 quads; `part_bytes` apart.
-template <int PARTS>
+// Stores four fp32 values as `PARTS` (3: exact cut, 1: rounded to bf16) bf16 quads; `part_bytes` apart.  ONE_SUM: the products of all
+// parts go into one sum (see join_parts for the other way), so the lower parts of an infinity are stored as zero.
+template <int PARTS, bool ONE_SUM = false>
 __device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, float x0, float x1, float x2, float x3)
 {
     if (PARTS == 3) {
-        const Parts2 p = split3(x0, x1), q = split3(x2, x3);
+        Parts2 p = split3(x0, x1), q = split3(x2, x3);
+        if (ONE_SUM && largest(x0, x1, x2, x3) == __int_as_float(0x7F800000)) {
+            p.m0 = isinf(x0) ? 0u : p.m0, p.l0 = isinf(x0) ? 0u : p.l0;
+            p.m1 = isinf(x1) ? 0u : p.m1, p.l1 = isinf(x1) ? 0u : p.l1;
+            q.m0 = isinf(x2) ? 0u : q.m0, q.l0 = isinf(x2) ? 0u : q.l0;
+            q.m1 = isinf(x3) ? 0u : q.m1, q.l1 = isinf(x3) ? 0u : q.l1;
+        }
         ptx::st_shared_v2(addr, pack_high(p.h0, p.h1), pack_high(q.h0, q.h1));
         ptx::st_shared_v2(addr + part_bytes, pack_high(p.m0, p.m1), pack_high(q.m0, q.m1));
         ptx::st_shared_v2(addr + 2 * part_bytes, pack_high(p.l0, p.l1), pack_high(q.l0, q.l1));
@@ -421,7 +428,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                         ptx::tmem_ld_wait();
 #pragma unroll
                         for (int k = 0; k < 16; ++k)
-                            v[k] = __float_as_uint(__uint_as_float(v[k]) + (__uint_as_float(v1[k]) + (sbs ? __uint_as_float(v2[k]) : 0.0f)));
+                            v[k] = __float_as_uint(join_parts(__uint_as_float(v[k]), __uint_as_float(v1[k]) + (sbs ? __uint_as_float(v2[k]) : 0.0f)));
                     } else {
                         ptx::tmem_ld_wait();
                     }
@@ -729,7 +736,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                 if (sq * 4 < live) {
 #pragma unroll
                     for (int i = 0; i < NQ; ++i)
-                        store_quad<3>(sop + operand_offset<ROWB>(srow + (GEN_K2_THREADS / QPR) * i, sq >> 1) + (sq & 1) * 8, SOP_PART, x[i][0], x[i][1], x[i][2],
+                        store_quad<3, !F32>(sop + operand_offset<ROWB>(srow + (GEN_K2_THREADS / QPR) * i, sq >> 1) + (sq & 1) * 8, SOP_PART, x[i][0], x[i][1], x[i][2],
                                       x[i][3]);
                 }
                 ptx::fence_proxy_async_smem();
@@ -787,7 +794,8 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
                         }
                         ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int k = 0; k < 16; ++k) v[k] = __float_as_uint((__uint_as_float(v[k]) + __uint_as_float(z[k])) + __uint_as_float(y[k]));
+                        for (int k = 0; k < 16; ++k)
+                            v[k] = __float_as_uint(join_parts(__uint_as_float(v[k]) + __uint_as_float(z[k]), __uint_as_float(y[k])));
                     } else {
                         ptx::tmem_ld_wait();
                     }

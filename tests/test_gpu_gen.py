@@ -198,3 +198,81 @@ def test_long_fp32_rows(n, m, r):
     assert rel_err(other.cpu().numpy(), oracle_compress(small, other0, 32, a=0.25, b=0.75)) <= TOL["f32"]
     fset.close()
     assert fb.flora_device_status() == 0
+
+
+def _special(t, seed):
+    """Puts infinities, NaN and the largest numbers into some rows of t, the rest of which stays as it is; the rows that hold any."""
+    n, m = t.shape
+    gen = torch.Generator().manual_seed(seed)
+    rows = sorted(set(torch.randint(0, n, (9,), generator=gen).tolist()) | {0, n - 1})
+    for k, i in enumerate(rows):
+        at = torch.randint(0, m, (3,), generator=gen).tolist() + [m - 1]
+        if k % 4 == 0:
+            t[i, at[0]] = float("inf")
+        elif k % 4 == 1:
+            t[i, at[0]], t[i, at[3]] = float("inf"), float("-inf")
+        elif k % 4 == 2:
+            t[i, at[1]] = float("nan")
+        else:
+            t[i, at[0]], t[i, at[1]] = float("-inf"), float("-inf")
+    return rows
+
+
+def _same(got, want, tol, what):
+    """Infinities and NaN in the same places with the same signs; the numbers within tol of the largest."""
+    got, want = got.double(), want.double()
+    fin = torch.isfinite(want)
+    assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(got[torch.isinf(want)], want[torch.isinf(want)]), what
+    assert bool((got[fin] - want[fin]).abs().max() <= tol * want[fin].abs().max()), what
+
+
+# Infinities and NaN come out as plain arithmetic gives them wherever fp32 values are multiplied in parts: fp32 gradients in the kernels
+# without TMA (split over a cluster or not, off 16 bytes or on) and with it (one item or several per row, one operand or two, a
+# cluster), sketches in both decompressions and for bf16 weights of the kernels without TMA.
+@pytest.mark.parametrize("n,m,r,offset", [(200, 300, 8, 0), (130, 1029, 33, 1), (64, 4100, 96, 0), (300, 5000, 17, 0), (257, 4100, 130, 0), (2049, 2052, 64, 0)])
+def test_infinities_in_gradients(n, m, r, offset):
+    _, G = _view(n, m, "f32", 3, offset, 0, 0.1)
+    _special(G, 1)
+    A = torch.empty(r, m, device=DEV)
+    fb.flora_materialize_A(A, 31)
+    product = torch.stack([(G.double() * A[j].double()).sum(1) for j in range(r)], 1)       # (no zeros are multiplied in)
+    S = torch.randn(n, r, generator=torch.Generator(device=DEV).manual_seed(5), device=DEV)
+    S0 = S.clone()
+    fb.flora_compress_accumulate(G, S, 31, r)
+    _same(S, S0.double() + product, 1e-5, "add")
+    S.fill_(float("nan"))
+    fb.flora_momentum_step(G, S, 0.0, 31)
+    _same(S, product, 1e-5, "overwrite")
+    T = S0.clone()
+    fset = fb.FloraSet([torch.zeros_like(G), torch.zeros_like(G)], None, [T, S])
+    fset.rebind_gradients([G, G])
+    fset.momentum_step(0.75, [31, 32])
+    _same(T, 0.75 * S0.double() + 0.25 * product, 1e-5, "momentum of a set")
+    fset.close()
+
+
+@pytest.mark.parametrize("n,m,r,dtype", [(200, 300, 8, "f32"), (130, 1029, 96, "f32"), (2049, 3076, 64, "f32"), (600, 5004, 128, "f32"), (130, 1029, 33, "bf16"),
+                                         (300, 384, 16, "bf16"), (2049, 3080, 32, "bf16")])
+def test_infinities_in_sketches(n, m, r, dtype):
+    C = torch.randn(n, r, generator=torch.Generator(device=DEV).manual_seed(6), device=DEV)
+    rows = _special(C, 2)
+    if dtype == "f32" and r >= 64:                                    # (|A| < 5.8 / sqrt(r): the sum stays finite)
+        C[rows[1]] = 1e-3
+        C[rows[1], r - 1] = 3.4028234e38                              # rounds to infinity in tf32
+    A = torch.empty(r, m, device=DEV, dtype=wl.torch_dtype(dtype))
+    fb.flora_materialize_A(A, 17)
+    W = wl.gaussian_matrix(n, m, 4e-4, dtype, 9).to(DEV)
+    update = torch.zeros(n, m, device=DEV, dtype=torch.float64)
+    for j in range(r):
+        update += C[:, j:j + 1].double() * A[j].double()
+    want = W.double() - 1e-3 * update
+    W2 = W.clone()
+    fb.flora_decompress_apply(W, C, 17, 1e-3, 1.0)
+    fset = fb.FloraSet(None, [W2, W2.clone()], [C, C])
+    fset.decompress_apply([17, 18], 1e-3, 1.0)
+    big = want.abs() > 1e30
+    for x in (W, W2):
+        _same(torch.where(big, 0.0, x.double()), torch.where(big, 0.0, want), 1e-5 if dtype == "f32" else 4e-3, "numbers")
+        _same(torch.where(big, x.double(), 0.0), torch.where(big, want, 0.0), 1e-5 if dtype == "f32" else 4e-3, "large")
+    fset.close()
+    assert fb.flora_device_status() == 0
