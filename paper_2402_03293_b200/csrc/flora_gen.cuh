@@ -89,7 +89,7 @@ __device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, f
 {
     if (PARTS == 3) {
         Parts2 p = split3(x0, x1), q = split3(x2, x3);
-        if (ONE_SUM && largest(x0, x1, x2, x3) == __int_as_float(0x7F800000)) {
+        if (ONE_SUM && fmaxf(fmaxf(fabsf(x0), fabsf(x1)), fmaxf(fabsf(x2), fabsf(x3))) == __int_as_float(0x7F800000)) {
             p.m0 = isinf(x0) ? 0u : p.m0, p.l0 = isinf(x0) ? 0u : p.l0;
             p.m1 = isinf(x1) ? 0u : p.m1, p.l1 = isinf(x1) ? 0u : p.l1;
             q.m0 = isinf(x2) ? 0u : q.m0, q.l0 = isinf(x2) ? 0u : q.l0;

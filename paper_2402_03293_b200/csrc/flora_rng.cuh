@@ -192,7 +192,6 @@ __device__ __forceinline__ float bf16_round(float v)
 // Adds up what fp32 products made in parts come to: the sum of the large products (upper part times upper part) and that of the others.
 // Where an operand is infinite its lower parts are NaN, or meet an upper part of either sign; the large products alone are then what
 // plain arithmetic gives, sign by sign (the upper part of an infinity is that infinity, of a NaN a NaN, and A is never zero).
-__device__ __forceinline__ float largest(float a, float b, float c, float d) { return fmaxf(fmaxf(fabsf(a), fabsf(b)), fmaxf(fabsf(c), fabsf(d))); }
 __device__ __forceinline__ float join_parts(float large, float rest) { return fabsf(large) < __int_as_float(0x7F800000) ? large + rest : large; }
 
 }  // namespace flora

@@ -927,7 +927,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                             ptx::ld_shared_v4(addr, x[0], x[1], x[2], x[3]);
 #pragma unroll
                             for (int u = 0; u < 4; ++u)
-                                x[u] = __float_as_uint(fmaf(-step, join_parts(__uint_as_float(v[4 * h + u]), __uint_as_float(y[4 * h + u])), __uint_as_float(x[u])));
+                                x[u] = __float_as_uint(fmaf(-step, __uint_as_float(v[4 * h + u]) + __uint_as_float(y[4 * h + u]), __uint_as_float(x[u])));
                             ptx::st_shared_v4(addr, x[0], x[1], x[2], x[3]);
                         }
                     }
@@ -990,13 +990,12 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                     uint32_t x[4], hi[4], lo[4];
                     ptx::ld_shared_v4(at + i * (16 * 32 * K2_CUT_WARPS), x[0], x[1], x[2], x[3]);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) hi[u] = round_tf32(x[u]);
-                    // (the largest numbers are cut off: rounding would carry them to infinity)
-                    if (largest(__uint_as_float(x[0]), __uint_as_float(x[1]), __uint_as_float(x[2]), __uint_as_float(x[3])) >= __uint_as_float(0x7F7FF000u))
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) hi[u] = (hi[u] & 0x7FFFFFFFu) == 0x7F800000u ? x[u] & 0xFFFFE000u : hi[u];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) lo[u] = __float_as_uint(__uint_as_float(x[u]) - __uint_as_float(hi[u]));
+                    for (int u = 0; u < 4; ++u) {
+                        // Upper parts stay finite: the lower part of an infinity is then that infinity and meets the upper parts of A
+                        // alone, so that the sums come out with the signs of plain arithmetic (and the largest numbers stay numbers).
+                        hi[u] = __float_as_uint(fminf(fmaxf(__uint_as_float(round_tf32(x[u])), __uint_as_float(0xFF7FE000u)), __uint_as_float(0x7F7FE000u)));
+                        lo[u] = __float_as_uint(__uint_as_float(x[u]) - __uint_as_float(hi[u]));
+                    }
                     ptx::st_shared_v4(at + i * (16 * 32 * K2_CUT_WARPS), hi[0], hi[1], hi[2], hi[3]);
                     ptx::st_shared_v4(to + i * (16 * 32 * K2_CUT_WARPS), lo[0], lo[1], lo[2], lo[3]);
                 }
