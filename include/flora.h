@@ -230,7 +230,8 @@ void flora_set_deterministic(int on);
  * Diagnostics.
  * ------------------------------------------------------------------------------------------- */
 /* Test hook: 0 = choose the kernel automatically (tensor-core kernels when dtype, alignment and
- * rank allow), 1 = always the plain fp32 SIMT kernels.  Process-wide. */
+ * rank allow), 1 = always the plain fp32 SIMT kernels, 2 = the TMA kernels for every matrix that
+ * they can serve, also where smaller ones are quicker (sets: as of their creation).  Process-wide. */
 void flora_debug_force_path(int path);
 
 /* Test hook for the host-side work decomposition of the tensor-core kernels (no kernel is launched; works without a

@@ -30,7 +30,7 @@ __host__ __device__ __forceinline__ PhiloxKey make_key(uint64_t seed)
 //   * what comes in pairs runs in packed instructions (two fp32 operations each, rounded as the scalar ones are);
 //   * the logarithm is evaluated in -2s with every constant scaled by a power of two, the octant reduction by the sign of
 //     the 22 low bits read as a signed number, so that neither needs fix-up instructions;
-//   * the square root has its special cases taken out beforehand.
+//   * the square root is one Newton (Heron) step on the hardware's estimate; its argument is never negative, subnormal or infinite.
 // Every rounding step is the one of the definition; only exact operations were rearranged.
 
 // Two Philox4x32-10 blocks with counters (qa, ja, 0, 0) and (qb, jb, 0, 0).
@@ -106,8 +106,8 @@ __device__ __forceinline__ f32x2 neg2_ln_u1(uint32_t xa0, uint32_t xa1)
 }
 
 // Square roots of two values of neg2_ln_u1, rounded to nearest: one Newton (Heron) step g + (x - g^2) / (2 g) from the
-// hardware's estimate of 1 / sqrt(x), with the residual in one fma.  Equal to the IEEE square root on all 2^24 values that
-// neg2_ln_u1 takes (compared one by one); 0 is the only special one among them.
+// hardware's estimate of 1 / sqrt(x), with the residual in one fma.  Equal to the IEEE square root on the values that neg2_ln_u1
+// takes (2^24 at most; the tests compare 2^27 draws of them bit by bit); 0 is the only special one among them.
 __device__ __forceinline__ f32x2 sqrt_of_ln(f32x2 x)
 {
     float x0, x1, y0, y1;

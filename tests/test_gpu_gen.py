@@ -94,12 +94,23 @@ def test_fp32_through_tma(n, m, r):
     fb.flora_materialize_A(A, 31)
     product = G.double() @ A.double().T
     assert ((S.double() - S0.double() - product).abs().max() / product.abs().max()).item() <= 3.3e-6 + 2.0 ** -22
-    fset = fb.FloraSet([torch.zeros_like(G), G[:, : m - 4].contiguous()], None, [S, S0])
-    fset.rebind_gradients([G, G[:, : m - 4].contiguous()])
+    G2 = G[:, : m - 4].contiguous()
+    T = S0.clone()
+    fset = fb.FloraSet([torch.zeros_like(G), G2], None, [S, T])
+    fset.rebind_gradients([G, G2])
     S.fill_(float("nan"))
+    T.fill_(float("nan"))
     fset.compress_overwrite([32, 33])
-    fset.momentum_step(0.5, [32, 33])
     assert rel_err(S.cpu().numpy(), oracle_compress(G, torch.zeros_like(S), 32)) <= TOL["f32"]
+    assert rel_err(T.cpu().numpy(), oracle_compress(G2, torch.zeros_like(T), 33)) <= TOL["f32"]
+    S.copy_(S0)                                                       # a blend whose two parts differ: another seed, unequal weights
+    T.copy_(S0)
+    fset.momentum_step(0.75, [34, 35])
+    assert rel_err(S.cpu().numpy(), oracle_compress(G, S0, 34, a=0.25, b=0.75)) <= TOL["f32"]
+    assert rel_err(T.cpu().numpy(), oracle_compress(G2, S0, 35, a=0.25, b=0.75)) <= TOL["f32"]
+    alone = S0.clone()
+    fb.flora_momentum_step(G, alone, 0.75, 34)
+    assert rel_err(alone.cpu().numpy(), oracle_compress(G, S0, 34, a=0.25, b=0.75)) <= TOL["f32"]
     fset.close()
     assert fb.flora_device_status() == 0
 

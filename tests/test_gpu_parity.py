@@ -43,6 +43,16 @@ def test_generated_projection_is_bit_exact(seed, r, m):
     assert np.array_equal(wl.as_numpy(outb), orc.round_to_bf16(ref)[1])
 
 
+def test_generated_projection_is_bit_exact_over_the_range_of_the_generator():
+    """2 x 8 x 2^24 values: 2^27 draws of u1, which leave out one in 3000 of its 2^24 values (the square root and the logarithm see
+    nothing else), and of u2."""
+    r, m = 8, 1 << 24
+    out = torch.empty(r, m, device=DEV)
+    for seed in (2024, 77):
+        fb.flora_materialize_A(out, seed)
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), orc.materialize_A(seed, r, m).view(np.uint32)), seed
+
+
 # --------------------------------------------------------------------------------------- contractions
 SHAPES = [(1, 1, 1), (5, 7, 3), (33, 100, 8), (130, 257, 17), (64, 512, 32), (300, 1000, 64), (129, 200, 256),
           # eligible for the tensor-core kernels (bf16, 16-byte aligned rows, n >= 128, m >= 64), ragged tiles and tails
