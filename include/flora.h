@@ -18,11 +18,18 @@
  *    elements (ld >= cols).  `data` is a DEVICE pointer that the caller owns;
  *    the library never frees, reallocates or keeps it beyond the call (a
  *    flora_set keeps the pointers it was created with until it is destroyed).
+ *    A compression whose G is not aligned to 16 bytes (pointer and ld) reads
+ *    whole 16-byte blocks, up to 15 bytes before and behind the matrix or
+ *    its rows: never beyond the page of a byte of G, and what is read there
+ *    is not used.  Nothing outside the matrices is written.
  *  - G and W may be FLORA_F32 or FLORA_BF16; the sketches C and M are always
  *    FLORA_F32.  The dtype of G / W also fixes the precision of the projection
  *    as the contraction sees it: fp32 values of A for FLORA_F32, those values
  *    rounded to bf16 (nearest even) for FLORA_BF16.  Products are accumulated
- *    in fp32.
+ *    in fp32.  fp32 results are as near to exact ones as sums in plain fp32
+ *    arithmetic; infinities and NaN in G or in a sketch come out as that
+ *    arithmetic gives them (a NaN whose payload lies in the low 16 bits only,
+ *    which no operation makes, may come out as an infinity).
  *  - The rank r is the column count of the sketch, 1 <= r <= 256.
  *  - `stream` is a cudaStream_t passed as void* (NULL = the default stream).
  *    Calls are asynchronous: they enqueue work on `stream` and return; they
@@ -223,7 +230,8 @@ flora_status flora_set_read_weights_to_host(flora_set* set, void* const* host_W,
  * order (compression over column ranges of a wide matrix; the r x r product of the transfer over column ranges),
  * which can change the last bits from run to run.  on != 0: sets created from now on give every row of a sketch a
  * single owner, and every transfer from now on sums its r x r product in one CTA per matrix, so that repeated runs
- * on the same inputs are bit-identical (slower on few, wide matrices).  Process-wide; default off. */
+ * on the same inputs are bit-identical (slower on few, wide matrices).  (The r x r product of a single bf16 matrix is summed by up to
+ * four clusters of CTAs and added up in a fixed order; that of a member of a set, or of fp32 operands, by one CTA per tile of it.)  Process-wide; default off. */
 void flora_set_deterministic(int on);
 
 /* ---------------------------------------------------------------------------------------------

@@ -2,7 +2,8 @@
 // This file validates arguments, picks a kernel family and launches; all arithmetic of the path
 // lives in the kernels of flora_tc.cuh and flora_pair*.cuh (bf16 matrices that TMA can address; host side in
 // flora_tc_host.cuh), flora_gen.cuh (fp32, unaligned and small matrices; host side in flora_gen_host.cuh), flora_gram.cuh
-// (momentum transfer) and flora_simt.cuh (plain fp32 arithmetic: fp32 transfers, and a second opinion for tests).
+// (momentum transfer) and flora_simt.cuh (plain fp32 arithmetic: matrices beyond 2^31 rows or columns, transfers of sets that mix
+// dtypes, and a second opinion for tests).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -245,16 +246,16 @@ static bool all_addressable(const std::vector<flora_mat>& G, const std::vector<f
     return !ok.empty() && std::find(ok.begin(), ok.end(), (uint8_t)0) == ok.end();
 }
 
-// Builds the work lists of a set.
-static flora_status set_build(flora_set* s)
+// Builds the work lists of a set; its tables are copied on `own`.
+static flora_status set_build_on(flora_set* s, cudaStream_t own)
 {
     std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true);
     const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_wf = set_tma_side(s->W, s->S, false, true);
     std::vector<uint8_t> use_w = set_tma_side(s->W, s->S, false);
     auto any = [](const std::vector<uint8_t>& use) { return std::find(use.begin(), use.end(), (uint8_t)1) != use.end(); };
-    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
+    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, own, use_g, use_w);
     if (st == FLORA_OK && (any(use_f) || any(use_wf)))
-        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, nullptr, use_f, use_wf);
+        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, own, use_f, use_wf);
     for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
     for (size_t i = 0; i < use_w.size(); ++i) use_w[i] |= use_wf[i];
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
@@ -263,16 +264,28 @@ static flora_status set_build(flora_set* s)
             if (s->has_G && !use_g[i] && s->G[i].dtype == d && s->G[i].rows > 0 && gen_supported(s->G[i])) g.push_back((int)i);
             if (s->has_W && !use_w[i] && s->W[i].dtype == d && s->W[i].rows > 0 && gen_supported(s->W[i])) w.push_back((int)i);
         }
-        st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g);
-        if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w);
+        st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g, own);
+        if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w, own);
     }
-    // The tables were copied from pageable memory on the legacy stream, to which streams made with the non-blocking flag are not
-    // ordered: they are in place before any stream may use them.
-    const bool copied = s->tc.d_mats || s->tcf.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats;
-    if (copied && cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    return st;
+}
+// The tables are in place when this returns, for every stream.  They are copied on a stream of their own and waited for: the legacy
+// default stream would have the call wait for whatever the program has put on it, and streams made with the non-blocking flag are
+// not ordered to it.  (The tables are new memory, which nothing reads yet.)
+static flora_status set_build(flora_set* s)
+{
+    if (s->S.empty()) return FLORA_OK;
+    cudaStream_t own = nullptr;
+    if (cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        return FLORA_ERR_CUDA;
+    }
+    flora_status st = set_build_on(s, own);
+    if (cudaStreamSynchronize(own) != cudaSuccess) {
         cudaGetLastError();
         if (st == FLORA_OK) st = FLORA_ERR_CUDA;
     }
+    cudaStreamDestroy(own);
     return st;
 }
 

@@ -6,9 +6,10 @@
 //
 // fp32 operands are cut into three bf16 parts, x = h + m + l, by truncation: h and m hold eight significant bits each, l
 // the remaining eight, so the cut loses nothing.  The product of two fp32 values is then the sum of six exact products of
-// parts (h h, h m, m h, m m, h l, l h; the three left out are together below 2^-23 of the product, under the rounding of
-// the fp32 sum they join), and the tensor core adds them up in fp32.  That is six bf16 MMAs where plain fp32 arithmetic
-// spent r multiply-adds per element of G on the ALUs.
+// parts (h h, h m, m h, m m, h l, l h), which the tensor core adds up in fp32.  The three left out reach 2^-21 of a product
+// (the parts are cut off: m is below 2^-7 of x, l below 2^-15), in the 2-norm over normal values 6e-8 of a sum, as much as
+// rounding every product to fp32 would.  That is six bf16 MMAs where plain fp32 arithmetic spent r multiply-adds per
+// element of G on the ALUs.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -254,7 +255,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         // A step of a tile is 128 rows of eight 16-byte pieces; thread tid takes piece tid % 8 of the rows tid / 8 + RS i.
         // What bounds a step is issue slots (16 KB of G take about 700 cycles of an SM's share of HBM), so the loop carries
         // one pointer and tests one row count.  A piece that starts off a 16-byte boundary comes as the two aligned blocks it
-        // touches; a block is read whole as soon as one byte of it is wanted (it lies in one page with that byte).
+        // touches; a block is read whole as soon as one byte of it is wanted (it lies in one page with that byte; the header says so).
         constexpr int RS = 4 * WORKERS, NI = 128 / RS;              // rows that the warps cover at a time; pieces per thread
         constexpr int AHEAD = 8 / NI;                               // tiles under way in registers (32 KB of a CTA's G, or 64)
         const int piece = tid & 7, row_in = tid >> 3;

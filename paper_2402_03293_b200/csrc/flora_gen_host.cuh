@@ -271,8 +271,7 @@ inline flora_status gen_decompress_launch(bool f32, int bn, const GenK2Args& a, 
     launches.fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
-// CTAs for `units` of (slab, tile): every one of them resident at once; where the generation of a slab outweighs a tile,
-// shares of fewer tiles than a slab has would repeat it, so the shares grow with the rank.
+// CTAs for `units` of (slab, tile): as many as can be resident at once, at every rank.
 inline int64_t gen_k2_grid(int64_t units, int64_t slots) { return std::max<int64_t>(1, std::min(units, slots)); }
 inline flora_status gen_decompress_single(const flora_mat& W, const flora_mat& S, uint64_t seed, float step, cudaStream_t st,
                                           std::atomic<uint64_t>& launches)
@@ -317,7 +316,8 @@ inline void gen_set_free(GenSet& s)
     s = GenSet();
 }
 // kind 0: compression (big = G), 1: decompression (big = W)
-inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_mat>& big, const std::vector<flora_mat>& sketch, const std::vector<int>& ids)
+inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_mat>& big, const std::vector<flora_mat>& sketch, const std::vector<int>& ids,
+                                  cudaStream_t st)
 {
     s.ids = ids;
     if (ids.empty()) return FLORA_OK;
@@ -325,7 +325,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     s.f32 = big[ids[0]].dtype == FLORA_F32;
     s.h_mats.assign(big.size(), GenMat{});
     for (int i : ids) s.h_mats[i] = gen_mat(big[i], sketch[i]);
-    flora_status rc = upload(&s.d_mats, s.h_mats, nullptr);
+    flora_status rc = upload(&s.d_mats, s.h_mats, st);
     if (rc) return rc;
     struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
@@ -431,7 +431,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             launches_of(pass > 0, [&](const Cut& c) { items.push_back(c.item); });
         }
         s.begin.push_back(count);
-        return upload(&s.d_k1, items, nullptr);
+        return upload(&s.d_k1, items, st);
     }
     // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
     bool aligned = true;
@@ -469,8 +469,8 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         share.push_back((int)items.size());
         k0 = k1;
     }
-    rc = upload(&s.d_k2, items, nullptr);
-    return rc ? rc : upload(&s.d_share, share, nullptr);
+    rc = upload(&s.d_k2, items, st);
+    return rc ? rc : upload(&s.d_share, share, st);
 }
 inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
 {

@@ -80,7 +80,9 @@ struct alignas(64) GMaps {
 template <>
 struct GMaps<0> {
 };
-constexpr int GMAPS_FEW = 48, GMAPS_MANY = 192;      // (192 maps and the seeds stay below the 32 KB that a launch can carry)
+// Two sizes: 192 maps and the seeds stay below the 32 KB that a launch can carry, and cost 1.4 us of host time a launch whatever the
+// set; a third of that costs 0.3.  (Host time of a launch without maps, with 48, with 192: 3.2, 3.4, 4.6 us; the GPU's is the same.)
+constexpr int GMAPS_FEW = 64, GMAPS_MANY = 192;
 
 constexpr int SEEDS_PER_LAUNCH = 448;
 struct SeedTable {
@@ -116,12 +118,13 @@ struct K1Smem {                            // barriers and scalars, placed after
 // fp32 matrices (F32): G streams through the same ring (steps of 32 columns, tiles of the same 16 KB) and is multiplied as tf32,
 // whose operands are 32-bit words of which the tensor core takes the upper 19 bits: hi(G).  The generator warps write what that
 // leaves, lo(G) = G - hi(G) rounded to tf32, into a ring of its own, and A as hi(A) and lo(A) in two halves of its tile.  The sum of
-// hi hi, hi lo and lo hi carries 2^-22 of a product, below the rounding of the fp32 sum that it joins.  The tensor core's sums are
-// truncated, not rounded: every accumulation loses about 2e-8 of the running sum, always towards zero (measured: 6e-6 after 300), so
-// the small products have an accumulator of their own (`minor`), the steps of an item take up to `nsets` pairs of accumulators in
-// turn, the planner caps the steps of an item, and the parts are added up in rounded fp32 at the end.  What bounds a step then: the 16 KB of a tile from HBM (700 cycles of an SM's share) against 130 cycles of issue slots
-// for its lo(G), 11 r cycles for A and 400 of tensor pipe; the kernel that cut fp32 into three bf16 parts out of registers spent
-// 670 issue cycles on a tile.
+// hi hi, hi lo and lo hi is off by up to 2^-20 of a product (hi(G) is cut off, not rounded), by 1.4e-7 of a sum over normal values in
+// the 2-norm: less than the rounding of a plain fp32 sum over more than 60 columns.  The tensor core's sums are truncated: every
+// accumulation loses about 2e-8 of the running sum, always towards zero (measured: 6e-6 after 300), so the small products have an
+// accumulator of their own (`minor`), the steps of an item are spread over up to `nsets` pairs of accumulators, the planner caps the
+// steps of an item by the width of the matrix (k1_f32_chain), and the parts are added up in rounded fp32 at the end.  What bounds a
+// step then: the 16 KB of a tile from HBM (700 cycles of an SM's share) against 130 cycles of issue slots for its lo(G), 11 r cycles for
+// A and 400 of tensor pipe; the kernel that cut fp32 into three bf16 parts out of registers spent 670 issue cycles on a tile.
 // SINGLE: one matrix, its record passed by value (every item names matrix 0).  MAPS: the gradients' maps come with the launch.
 // new_maps: those in the table may have been written since the kernel before.
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one

@@ -263,7 +263,7 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
         total_work += tiles * ks;
     }
     // Clusters of eight wherever the matrices have the rows for them: a slice of A then serves 2048 rows, and a 1600-row
-    // matrix is one unit (at N = 128 clusters of four keep a CTA's share of a slice within what its generators make
+    // matrix is one unit (times with an earlier, slower generator of A: at N = 128 clusters of four keep a CTA's share of a slice within what its generators make
     // during a step, and fit 132 SMs instead of 120, but generate every slice of such a matrix twice: 824 against 714 us
     // on config 5's set at r = 128, 32.8 against 28.9 us on one 4096 x 11008 matrix).
     int S = 8;
@@ -645,10 +645,7 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     bn = !f32 && tune_knob("FLORA_K2_BN", bn, 64, 128) >= 128 ? 128 : 64;
     const size_t slab_bytes = (size_t)kchunks * bn * (f32 ? 256 : 128), slot = (size_t)(bn / (f32 ? 32 : 64)) * W_BOX_BYTES;
     const size_t lower = f32 ? (size_t)K2_LSTAGES * S_CHUNK_BYTES : 0;      // ring of the sketch's lower parts
-    // two CTAs per SM when two of them fit (each with two slabs, two W slots and one S chunk)
-    const size_t per_cta_max = 113 * 1024;                       // half of an SM's shared memory minus the reserve
-    int per_sm = (2 * slab_bytes + S_CHUNK_BYTES + 2 * slot + ctl <= per_cta_max) ? 2 : 1;
-    per_sm = 1;   // twelve fixed warps plus generators: one CTA per SM
+    // (twelve fixed warps plus generators: one CTA per SM)
     // Two slab buffers (the next item's slab is generated while the current item streams) unless that leaves fewer
     // than four S chunks in flight: the chunks of one W tile are kchunks x 16 KB, and with too few of them under way
     // the loads' latency, not bandwidth, sets the pace.  With one buffer every warp that is idle between two items
@@ -657,7 +654,7 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     // r = 64, with four and one slab buffer 72, and a third W slot is worth less than the fourth chunk: 77.)
     int nslabs = (2 * slab_bytes + 4 * S_CHUNK_BYTES + (f32 ? 3 : 2) * slot + lower + ctl <= SMEM_BUDGET) ? 2 : 1;
     nslabs = tune_knob("FLORA_K2_SLABS", nslabs, 1, 2);
-    const size_t budget = (per_sm == 2 ? per_cta_max : SMEM_BUDGET) - ctl - nslabs * slab_bytes - lower;
+    const size_t budget = SMEM_BUDGET - ctl - nslabs * slab_bytes - lower;
     int cstages = std::max(2, std::min(nslabs == 1 ? 2 * kchunks : kchunks + 1, nslabs == 1 ? K2_MAX_CSTAGES : 4));
     cstages = tune_knob("FLORA_K2_CSTAGES", cstages, 1, K2_MAX_CSTAGES);
     while (cstages > 1 && (size_t)cstages * S_CHUNK_BYTES + (f32 && cstages > 4 ? 3 : 2) * slot > budget) --cstages;
@@ -671,7 +668,7 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     set.k2_gw = GW;
     set.k2_nslabs = nslabs;
     set.k2_smem = nslabs * slab_bytes + (size_t)cstages * S_CHUNK_BYTES + (size_t)slots * slot + lower + sizeof(K2Smem) + 1024;
-    int grid_max = sm_count() * per_sm;
+    int grid_max = sm_count();
     // Ranks above 128 run on CTA pairs: each CTA holds half of a 128-column slab (two buffers of kchunks x 8 KB), the
     // sketch chunks of its own tiles (as many stages as fit beside two W tiles, at most two tiles' worth) and its W tiles.
     // Above r = 192 one CTA has room for a single slab buffer only; from r = 129 to 192 it has room for two, and the pair

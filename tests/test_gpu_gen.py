@@ -1,8 +1,8 @@
 """The kernels for fp32, unaligned and small matrices (csrc/flora_gen.cuh) at the edges of their tiles, against the oracle.
 
-Tolerances: those of the other parity tests.  fp32: each product is exact to 2^-23 (three bf16 parts of 8 bits each, the
-products left out are below that) and up to 6 m of them are added in fp32, which for random signs leaves about
-sqrt(6 m) 2^-24 of the largest partial sum: 1e-5 holds with an order of magnitude to spare at the sizes here.  The weights
+Tolerances: those of the other parity tests.  fp32: each product is exact to 2^-21 (three bf16 parts, the products left out
+are below that, and 2^-24 of a sum in the 2-norm), and chains of truncated sums are kept so short that a sum over m columns is off
+by less than 1.8e-8 sqrt(m): 1e-5 holds with an order of magnitude to spare at the sizes here.  The weights
 carry one spacing of fp32 on top, since both sides store them rounded."""
 import numpy as np
 import pytest
@@ -81,8 +81,8 @@ def test_mixed_sets(r):
 
 # fp32 matrices that the TMA compression takes (too wide or too large for the kernels above): rows and columns around a tile and a
 # step, ranks around where A stops fitting one operand (128 | 129) and where two tiles share it (32 | 33), one item and several per
-# accumulator set.  The bound is a third of the tolerance: hi/lo products carry 2^-22, and at most 192 truncated accumulations
-# (2e-8 of the running sum each, growing with the sum as its square root) stay under 3e-6.
+# accumulator set.  The bound is a third of the tolerance: hi/lo products are off by 2^-20 at most and 1.4e-7 of a sum in
+# the 2-norm, and the chains of truncated sums stay below what plain fp32 sums lose, 1.8e-8 sqrt(m) in the 2-norm (2.3e-6 at 16380).
 @pytest.mark.parametrize("n,m,r", [(128, 3104, 8), (257, 5000, 33), (130, 8196, 130), (385, 4100, 256), (2049, 2052, 96), (4096, 3076, 17), (129, 16380, 64),
                                    (300, 3300, 128)])
 def test_fp32_through_tma(n, m, r):
@@ -117,7 +117,7 @@ def test_fp32_through_tma(n, m, r):
 
 # fp32 weights that the TMA decompression takes: rows and columns around a tile, a slab and a box of 32 columns, ranks around where a
 # second slab buffer stops fitting (32 | 33), with odd numbers of chunks, and the largest; next to a matrix that stays with the kernels
-# above.  Per element, of sum |C| |A|: the products carry 2^-22 (lo lo left out, lo cut to tf32), and each of the r / 8 + 2 truncated
+# above.  Per element, of sum |C| |A|: the products carry 2^-21 (lo lo left out: 2^-24; both lo cut to tf32: 2^-22 each at most), and each of the r / 8 + 2 truncated
 # accumulations loses less than 2^-22 of the running sum; the store of W rounds to 2^-24.
 @pytest.mark.parametrize("n,m,r", [(129, 8260, 8), (1000, 2100, 33), (4097, 1028, 1), (300, 5004, 96), (2049, 3076, 128), (8200, 164, 64), (128, 8224, 100)])
 def test_fp32_weights_through_tma(n, m, r):
