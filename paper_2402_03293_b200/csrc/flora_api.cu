@@ -209,6 +209,8 @@ struct flora_set {
     std::vector<flora_mat> G, W, S;
     int r = 0;
     bool has_G = false, has_W = false;
+    cudaEvent_t copied = nullptr;          // the tables' copies
+    std::atomic<bool> in_place{false};     // ... are known to be done
     bool aligned_G = false;        // made of bf16 gradients that TMA can address, all of them: such a set takes no others
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
     TcSet tcf;                     // the same for fp32 matrices
@@ -246,16 +248,17 @@ static bool all_addressable(const std::vector<flora_mat>& G, const std::vector<f
     return !ok.empty() && std::find(ok.begin(), ok.end(), (uint8_t)0) == ok.end();
 }
 
-// Builds the work lists of a set; its tables are copied on `own`.
-static flora_status set_build_on(flora_set* s, cudaStream_t own)
+// Builds the work lists of a set.  Its tables are copied from pageable memory on the legacy default stream, to which streams made
+// with the non-blocking flag are not ordered: set_ready puts every stream behind the copies.
+static flora_status set_build(flora_set* s)
 {
     std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true);
     const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_wf = set_tma_side(s->W, s->S, false, true);
     std::vector<uint8_t> use_w = set_tma_side(s->W, s->S, false);
     auto any = [](const std::vector<uint8_t>& use) { return std::find(use.begin(), use.end(), (uint8_t)1) != use.end(); };
-    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, own, use_g, use_w);
+    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
     if (st == FLORA_OK && (any(use_f) || any(use_wf)))
-        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, own, use_f, use_wf);
+        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, nullptr, use_f, use_wf);
     for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
     for (size_t i = 0; i < use_w.size(); ++i) use_w[i] |= use_wf[i];
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
@@ -264,29 +267,37 @@ static flora_status set_build_on(flora_set* s, cudaStream_t own)
             if (s->has_G && !use_g[i] && s->G[i].dtype == d && s->G[i].rows > 0 && gen_supported(s->G[i])) g.push_back((int)i);
             if (s->has_W && !use_w[i] && s->W[i].dtype == d && s->W[i].rows > 0 && gen_supported(s->W[i])) w.push_back((int)i);
         }
-        st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g, own);
-        if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w, own);
+        st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g, nullptr);
+        if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w, nullptr);
     }
+    if (s->tc.d_mats || s->tcf.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats)
+        if (cudaEventCreateWithFlags(&s->copied, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(s->copied, nullptr) != cudaSuccess) {
+            cudaGetLastError();
+            if (st == FLORA_OK) st = FLORA_ERR_CUDA;
+        }
     return st;
 }
-// The tables are in place when this returns, for every stream.  They are copied on a stream of their own and waited for: the legacy
-// default stream would have the call wait for whatever the program has put on it, and streams made with the non-blocking flag are
-// not ordered to it.  (The tables are new memory, which nothing reads yet.)
-static flora_status set_build(flora_set* s)
+// Before a call puts work that reads the set's tables on a stream.  Nothing waits on the host for the copies (creating a set would
+// wait for whatever the program has queued: GPT-2-XL set 26 -> 30 ms), except where the stream is being recorded into a graph, which
+// cannot depend on an event of outside.
+static flora_status set_ready(flora_set* s, cudaStream_t st)
 {
-    if (s->S.empty()) return FLORA_OK;
-    cudaStream_t own = nullptr;
-    if (cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) != cudaSuccess) {
+    if (!s->copied || s->in_place.load(std::memory_order_acquire)) return FLORA_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;        // (asking for an event is not allowed during a capture otherwise)
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const bool recording = capturing(st);
+    const cudaError_t e = recording ? cudaEventSynchronize(s->copied) : cudaEventQuery(s->copied);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) {
+        s->in_place.store(true, std::memory_order_release);
+        return FLORA_OK;
+    }
+    cudaGetLastError();
+    if (e != cudaErrorNotReady || cudaStreamWaitEvent(st, s->copied, 0) != cudaSuccess) {
         cudaGetLastError();
         return FLORA_ERR_CUDA;
     }
-    flora_status st = set_build_on(s, own);
-    if (cudaStreamSynchronize(own) != cudaSuccess) {
-        cudaGetLastError();
-        if (st == FLORA_OK) st = FLORA_ERR_CUDA;
-    }
-    cudaStreamDestroy(own);
-    return st;
+    return FLORA_OK;
 }
 
 extern "C" {
@@ -462,6 +473,7 @@ flora_status flora_set_destroy(flora_set* set)
         gen_set_free(set->gen_g[d]);
         gen_set_free(set->gen_w[d]);
     }
+    if (set->copied) cudaEventDestroy(set->copied);
     delete set;
     return FLORA_OK;
 }
@@ -488,7 +500,9 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
         return FLORA_ERR_ALIGN;
     std::vector<CUtensorMap> maps, maps_f;
     if ((tc_ok && !tc_set_make_maps(set->tc, newG, maps)) || (tcf_ok && !tc_set_make_maps(set->tcf, newG, maps_f))) return FLORA_ERR_CUDA;
-    flora_status st = tc_ok ? tc_set_rebind(set->tc, maps, as_stream(stream)) : FLORA_OK;
+    flora_status st = set_ready(set, as_stream(stream));
+    if (st) return st;
+    st = tc_ok ? tc_set_rebind(set->tc, maps, as_stream(stream)) : FLORA_OK;
     if (st == FLORA_OK && tcf_ok) st = tc_set_rebind(set->tcf, maps_f, as_stream(stream));
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_rebind(set->gen_g[d], newG, as_stream(stream));
     if (st) return st;
@@ -518,6 +532,7 @@ static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a,
 {
     if (!set || !seeds) return FLORA_ERR_NULL;
     if (!set->has_G) return FLORA_ERR_UNSUPPORTED;
+    if (const flora_status st = set_ready(set, as_stream(stream))) return st;
     const bool simt = g_force_path.load() == 1;
     if (!simt) {
         flora_status st = tma_compress(set, set->tc, seeds, a, b, as_stream(stream), behind_own_transfer);
@@ -547,6 +562,7 @@ flora_status flora_set_decompress_apply(flora_set* set, const uint64_t* seeds, f
 {
     if (!set || !seeds) return FLORA_ERR_NULL;
     if (!set->has_W) return FLORA_ERR_UNSUPPORTED;
+    if (const flora_status st = set_ready(set, as_stream(stream))) return st;
     const bool simt = g_force_path.load() == 1;
     if (!simt) {
         flora_status st = FLORA_OK;
@@ -570,6 +586,7 @@ static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& s
     if (release_later) *release_later = nullptr;
     if (ordered) *ordered = false;
     if (!set || !seeds_old || !seeds_new) return FLORA_ERR_NULL;
+    if (const flora_status st = set_ready(set, as_stream(stream))) return st;
     const std::vector<flora_mat>& big = set->has_G ? set->G : set->W;
     const int r = set->r;
     float* T = nullptr;
@@ -614,6 +631,7 @@ flora_status flora_set_transfer_axpby(flora_set* dst, const flora_set* src, cons
     if (src->S.size() != dst->S.size() || src->r != dst->r) return FLORA_ERR_SHAPE;
     for (size_t i = 0; i < dst->S.size(); ++i)
         if (src->S[i].rows != dst->S[i].rows) return FLORA_ERR_SHAPE;
+    if (const flora_status st = set_ready(const_cast<flora_set*>(src), as_stream(stream))) return st;
     return set_transfer(dst, src->S, src->tc.d_mats, seeds_old, seeds_new, a, b, stream);
 }
 
@@ -635,6 +653,7 @@ flora_status flora_set_momentum_step_resampled(flora_set* set, float beta, const
 flora_status flora_set_zero_state(flora_set* set, void* stream)
 {
     if (!set) return FLORA_ERR_NULL;
+    if (const flora_status st = set_ready(set, as_stream(stream))) return st;
     if (set->tc.d_mats && g_force_path.load() != 1) return tc_set_zero(set->tc, as_stream(stream), g_launches);
     for (auto& s : set->S) {
         if (s.rows == 0) continue;
