@@ -211,6 +211,7 @@ struct flora_set {
     bool has_G = false, has_W = false;
     cudaEvent_t copied = nullptr;          // the tables' copies
     std::atomic<bool> in_place{false};     // ... are known to be done
+    bool tf32_transfer = false;    // all its matrices (on one side) are bf16 and can be addressed by TMA: see transfer_tables
     bool aligned_G = false;        // made of bf16 gradients that TMA can address, all of them: such a set takes no others
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
     TcSet tcf;                     // the same for fp32 matrices
@@ -455,6 +456,7 @@ flora_status flora_set_create(int count, const flora_mat* G, const flora_mat* W,
     if (G) s->G.assign(G, G + count);
     if (W) s->W.assign(W, W + count);
     s->aligned_G = s->has_G && all_addressable(s->G, s->S);
+    s->tf32_transfer = s->aligned_G || (s->has_W && all_addressable(s->W, s->S));
     flora_status st = set_build(s);
     if (st) {
         flora_set_destroy(s);
@@ -579,6 +581,10 @@ flora_status flora_set_decompress_apply(flora_set* set, const uint64_t* seeds, f
     return FLORA_OK;
 }
 
+// The tables through which the transfer of several matrices may read sketches as tf32 (apply_tc_kernel).  Sets of bf16 matrices that
+// TMA serves have always been read so; for any other set the product stays in fp32 (sketch against the oracle: 8e-4 as tf32, 1e-6).
+static const TcMatrix* transfer_tables(const flora_set* set) { return set->tf32_transfer ? set->tc.d_mats : nullptr; }
+
 // dst.S[i] <- b dst.S[i] + a src[i] (A(old_i) A(new_i)^T) for every matrix of the set `dst`.
 static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& src, const TcMatrix* src_mats, const uint64_t* seeds_old,
                                  const uint64_t* seeds_new, float a, float b, void* stream, void** release_later = nullptr, bool* ordered = nullptr)
@@ -602,7 +608,7 @@ static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& s
             jobs.push_back(GramJob{nullptr, (float*)set->S[i].data, (const float*)src[i].data, set->S[i].ld, src[i].ld,
                                    (int32_t)set->S[i].rows, (int32_t)big[i].cols, seeds_old[i], seeds_new[i], (int32_t)i, 0});
         }
-        return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches, set->tc.d_mats, src_mats, nullptr, release_later,
+        return transfer_tc(jobs, r, a, b, as_stream(stream), g_launches, transfer_tables(set), src_mats, nullptr, release_later,
                            dtype == FLORA_F32, ordered);
     }
     if (scratch_alloc((void**)&T, sizeof(float) * r * r, as_stream(stream)) != cudaSuccess) {
@@ -621,7 +627,7 @@ static flora_status set_transfer(flora_set* set, const std::vector<flora_mat>& s
 flora_status flora_set_resample_transfer(flora_set* set, const uint64_t* seeds_old, const uint64_t* seeds_new, void* stream)
 {
     if (!set) return FLORA_ERR_NULL;
-    return set_transfer(set, set->S, set->tc.d_mats, seeds_old, seeds_new, 1.0f, 0.0f, stream);
+    return set_transfer(set, set->S, transfer_tables(set), seeds_old, seeds_new, 1.0f, 0.0f, stream);
 }
 
 flora_status flora_set_transfer_axpby(flora_set* dst, const flora_set* src, const uint64_t* seeds_old, const uint64_t* seeds_new, float a, float b,
@@ -632,7 +638,7 @@ flora_status flora_set_transfer_axpby(flora_set* dst, const flora_set* src, cons
     for (size_t i = 0; i < dst->S.size(); ++i)
         if (src->S[i].rows != dst->S[i].rows) return FLORA_ERR_SHAPE;
     if (const flora_status st = set_ready(const_cast<flora_set*>(src), as_stream(stream))) return st;
-    return set_transfer(dst, src->S, src->tc.d_mats, seeds_old, seeds_new, a, b, stream);
+    return set_transfer(dst, src->S, transfer_tables(src), seeds_old, seeds_new, a, b, stream);
 }
 
 flora_status flora_set_momentum_step_resampled(flora_set* set, float beta, const uint64_t* seeds_old, const uint64_t* seeds_new, void* stream)
@@ -644,7 +650,7 @@ flora_status flora_set_momentum_step_resampled(flora_set* set, float beta, const
     // transfer's scratch is handed back after it has been launched
     void* scratch = nullptr;
     bool ordered = false;
-    flora_status st = set_transfer(set, set->S, set->tc.d_mats, seeds_old, seeds_new, beta, 0.0f, stream, &scratch, &ordered);
+    flora_status st = set_transfer(set, set->S, transfer_tables(set), seeds_old, seeds_new, beta, 0.0f, stream, &scratch, &ordered);
     if (st == FLORA_OK) st = set_compress(set, seeds_new, 1.0f - beta, 1.0f, stream, ordered);
     if (scratch && cudaFreeAsync(scratch, as_stream(stream)) != cudaSuccess && st == FLORA_OK) st = FLORA_ERR_CUDA;
     return st;

@@ -287,3 +287,23 @@ def test_infinities_in_sketches(n, m, r, dtype):
         _same(torch.where(big, x.double(), 0.0), torch.where(big, want, 0.0), 1e-5 if dtype == "f32" else 4e-3, "large")
     fset.close()
     assert fb.flora_device_status() == 0
+
+
+# A set with matrices that TMA cannot address: its transfer is computed in fp32 throughout (as tf32 the sketches would be off by 8e-4).
+@pytest.mark.parametrize("r", [32, 64])
+def test_transfers_of_mixed_sets_stay_in_fp32(r):
+    shapes = [(130, 70), (1000, 515), (257, 4097), (768, 768), (48, 3072)]
+    src = [torch.randn(n, r, generator=torch.Generator(device=DEV).manual_seed(i), device=DEV) for i, (n, _) in enumerate(shapes)]
+    dst = [torch.randn(n, r, generator=torch.Generator(device=DEV).manual_seed(9 + i), device=DEV) for i, (n, _) in enumerate(shapes)]
+    dst0 = [x.clone() for x in dst]
+    G = [torch.zeros(n, m, device=DEV, dtype=torch.bfloat16) for n, m in shapes]
+    acc, mom = fb.FloraSet(G, None, src), fb.FloraSet(None, [g.clone() for g in G], dst)
+    mom.transfer_axpby_from(acc, [1, 2, 3, 4, 5], [11, 12, 13, 14, 15], 0.25, 0.5)
+    for i, (n, m) in enumerate(shapes):
+        A, B = torch.empty(r, m, dtype=torch.bfloat16, device=DEV), torch.empty(r, m, dtype=torch.bfloat16, device=DEV)
+        fb.flora_materialize_A(A, 1 + i)
+        fb.flora_materialize_A(B, 11 + i)
+        want = 0.25 * (src[i].double() @ (A.double() @ B.double().T)) + 0.5 * dst0[i].double()
+        assert ((dst[i].double() - want).norm() / want.norm()).item() <= 1e-5, i
+    acc.close()
+    mom.close()
