@@ -179,10 +179,10 @@ flora_status static_scratch_for_current_device(float** out)
 bool use_gen(const flora_mat* big) { return g_force_path.load(std::memory_order_relaxed) != 1 && gen_supported(*big); }
 // Whether matrices of this size go to the kernels without TMA although TMA can address them (flora_debug_force_path(2): only where
 // those alone give bit-reproducible fp32 results).
-bool small_compress(int64_t elements, int64_t cols, int r, bool f32)
+bool small_compress(int64_t elements, int64_t cols, int r, bool f32, bool set)
 {
     if (g_force_path.load(std::memory_order_relaxed) == 2) return f32 && deterministic_flag().load();
-    return gen_compress_quicker(elements, cols, r, f32);
+    return gen_compress_quicker(elements, cols, r, f32, set);
 }
 bool small_decompress(int64_t elements, int r, bool f32)
 {
@@ -192,7 +192,7 @@ bool small_decompress(int64_t elements, int r, bool f32)
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 {
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch) &&
-           !small_compress(big->rows * big->cols, big->cols, (int)sketch->cols, big->dtype == FLORA_F32);
+           !small_compress(big->rows * big->cols, big->cols, (int)sketch->cols, big->dtype == FLORA_F32, false);
 }
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
 {
@@ -238,7 +238,7 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
     const int r = S.empty() ? 1 : (int)S[0].cols;
     const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
     if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS && g_force_path.load() != 2) ||
-        (compression ? small_compress(counted, widest, r, f32) : small_decompress(counted, r, f32)))
+        (compression ? small_compress(counted, widest, r, f32, true) : small_decompress(counted, r, f32)))
         std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
 }

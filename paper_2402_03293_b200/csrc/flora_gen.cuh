@@ -36,10 +36,20 @@ struct GenItem {           // compression: one cluster
 
 // Warps that load, convert, generate and write out (8, or 16 where a CTA has an SM to itself), and one that issues the MMAs.
 __host__ __device__ constexpr int gen_threads(int workers) { return 32 * (workers + 1); }
-constexpr int GEN_G_SLOTS_MAX = 8, GEN_A_SLOTS_MAX = 4;
+constexpr int GEN_G_SLOTS_MAX = 8, GEN_A_SLOTS_MAX = 6;
 constexpr int GEN_L2_AHEAD = 8;                             // steps of a tile that a CTA asks into L2 before it may load them
 constexpr int GEN_F32_CHAIN_STEPS = 72;                     // steps of an fp32 matrix that a CTA adds up at most
 constexpr int GEN_MAX_SPLIT = 16;                           // CTAs that share the columns of a row group (above 8: not a portable cluster size)
+// How the CTAs of a split bring their sums together.
+//   Ordered   through distributed shared memory: every row has one writer, which adds the peers' sums in a fixed order.  Bit-reproducible
+//             mode only: reading the peers and the two cluster barriers around that took half of a small launch.
+//   Scaled    every CTA adds its sums to the sketch in global memory (red.global), after the cluster has scaled the rows: each CTA its
+//             share of them while its first loads travel, and a barrier whose wait is over before the sums are there.
+//   Plain     the same where there is nothing to scale (b = 1): no barrier, and no clusters.
+// Measured with Ordered / Scaled / Plain, us a launch in a chain: 512 x 512 at r = 8 in fp32 5.9 / 4.4 / 3.6, 256 x 384 at r = 32 5.0 / 4.4 / 3.6,
+// 768 x 768 at r = 16 5.5 / 4.7 / 3.7, 768 x 2304 at r = 16 7.6 / 6.1 / 5.3.  (Of the 6 us of the first one 1.3 passed before it could read
+// anything, 1.6 until its product was there, 3.1 with the sums of sixteen CTAs, the write-out and the way out.)
+enum GenJoin { GEN_JOIN_ORDERED, GEN_JOIN_SCALED, GEN_JOIN_PLAIN };
 // Columns of an fp32 matrix that one launch adds up: as many as keep every CTA's chain within its limit.  Wider matrices take several
 // launches, whose sums are added in rounded fp32 (one after another, so in a fixed order).
 constexpr int GEN_F32_PASS_COLS = 32 * GEN_MAX_SPLIT * GEN_F32_CHAIN_STEPS;
@@ -133,6 +143,27 @@ inline size_t gen_k1_a_bytes(bool f32, int r_pad) { return f32 ? (size_t)3 * 64 
 // rows write to different banks.
 __host__ __device__ inline int gen_stage_stride(int r_pad) { return r_pad + 4; }
 
+// `rows` rows of the sketch from row0 on, times b (b = 0: cleared, whatever they held), by NT threads.
+template <int NT>
+__device__ __forceinline__ void scale_rows(const GenMat& mat, int row0, int rows, int r, float b, int tid)
+{
+    const bool vec = (r & 3) == 0 && (mat.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(mat.S) & 15) == 0;
+    const int per = vec ? r >> 2 : r, total = rows * per;                    // pieces
+    float* const S = mat.S + (int64_t)row0 * mat.lds;
+#pragma unroll 4
+    for (int e = tid; e < total; e += NT) {
+        const int i = e / per, j = e - i * per;
+        float* const p = S + (int64_t)i * mat.lds + (vec ? 4 * j : j);
+        if (vec) {
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (b != 0.0f) o = *reinterpret_cast<const float4*>(p);
+            *reinterpret_cast<float4*>(p) = make_float4(b * o.x, b * o.y, b * o.z, b * o.w);
+        } else {
+            *p = b != 0.0f ? b * *p : 0.0f;
+        }
+    }
+}
+
 // SINGLE: one matrix, passed by value; every cluster takes the next row groups of it.  (A template and not a test of `items`: with
 // a run-time choice between the table's entry and the by-value one the kernel was seen to read the other one's address.)
 // sbs (fp32): the three parts of A side by side as one N operand (three MMAs per tile and K slice instead of six).  The tensor core
@@ -142,7 +173,7 @@ template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 __global__ void __launch_bounds__(gen_threads(WORKERS), WORKERS == 8 ? 2 : 1)
 gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
                     const __grid_constant__ GenMat single, int single_split, int single_col0, int seed_base, int r, float scale, float a, float b, int T, int sbs,
-                    int g_slots, int a_slots, int cluster)
+                    int g_slots, int a_slots, int cluster, int joining, int ahead)
 {
     using C = GenK1<F32>;
     constexpr int NT = 32 * WORKERS;                              // worker threads
@@ -156,8 +187,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     constexpr uint32_t G_BYTES = (uint32_t)C::PARTS * C::TILE;
     const uint32_t a_bytes = C::PARTS * a_part, a_ring = smem_base + (uint32_t)g_slots * G_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-    const int rank = cluster > 1 ? (int)ptx::cluster_ctarank() : 0;
-    const int cl = (int)blockIdx.x / cluster;
+    const int cl = (int)blockIdx.x / cluster, rank = (int)blockIdx.x - cl * cluster;
     GenItem item;
     if (!SINGLE) {
         item = items[cl];
@@ -173,8 +203,10 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     const int tiles = max(0, min(T, ((mat.n + 127) >> 7) - tile0));
     const int m_end = F32 ? item.col0 + min(mat.m - item.col0, GEN_F32_PASS_COLS) : mat.m;      // columns beyond it are another launch's
     const int all_steps = (m_end - item.col0 + C::K - 1) / C::K, step0 = item.col0 / C::K;
-    const int ks0 = step0 + (int)((int64_t)part * all_steps / split), ks1 = step0 + (int)((int64_t)(part + 1) * all_steps / split);
+    // (at most 2^25 steps and 16 parts: a 64-bit division takes a quarter of a microsecond)
+    const int ks0 = step0 + (int)((uint32_t)part * (uint32_t)all_steps / (uint32_t)split), ks1 = step0 + (int)((uint32_t)(part + 1) * (uint32_t)all_steps / (uint32_t)split);
     const int steps = tiles > 0 ? ks1 - ks0 : 0;
+    const bool barrier = cluster > 1 && joining == GEN_JOIN_SCALED;
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < T * acc_cols) tmem_cols <<= 1;
 
@@ -211,6 +243,12 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
 
     if (warp == WORKERS) {
         // ------------------------------------------------------------------ MMA issuer
+        if (barrier) {
+            // the workers have scaled this CTA's rows; the release is this warp's, as it has nothing else to do until the first tile is
+            // there (by the workers, behind the main loop, it took 0.9 us of a small launch)
+            ptx::named_barrier_sync(2, NT + 32);
+            ptx::cluster_arrive_release();
+        }
         if (lane == 0 && steps > 0) {
             RingPos pg, pa;
             bool ok = true;
@@ -359,8 +397,9 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
             for (int i = 0; i < NI; ++i)
 #pragma unroll
                 for (int k = 0; k < BLK; ++k) x[d][i][k] = make_uint4(0, 0, 0, 0);
-        // Tiles of A are made `lead` steps before they are used.  The first touches nothing that another kernel writes; the next
-        // ones are made while the first loads travel.
+        // Tiles of A are made up to `lead` steps before they are used (the MMAs that read the slot before are then done).  They touch
+        // nothing that another kernel writes: the first `ahead` are made while the kernel before this one runs, the next while the first
+        // loads travel.
         const int lead = a_slots - 2;
         RingPos pa;                                                 // of the next tile to make
         int made = 0;
@@ -379,15 +418,23 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 if ((tile0 + t) * 128 + (tid & 127) < mat.n) ptx::prefetch_l2(first + (int64_t)t * 128 * mat.ld * ES + ks * 128);
             }
         }
-        if (steps > 0) make();
+        while (made < min(ahead, steps)) make();
         ptx::grid_dependency_wait();
 #pragma unroll
         for (int d = 0; d < AHEAD; ++d)
             if (d < total) fetch(x[d]);
         while (made < min(lead + 1, steps)) make();
+        if (barrier && split > 1) {
+            const int lr0 = part * (tiles * 128) / split, lr1 = (part + 1) * (tiles * 128) / split;
+            scale_rows<NT>(mat, tile0 * 128 + lr0, min(lr1 - lr0, mat.n - tile0 * 128 - lr0), r, b, tid);
+        }
+        if (barrier) {
+            ptx::named_barrier_arrive(2, NT + 32);
+            ptx::cluster_arrive_relaxed();
+        }
         RingPos pg;
         auto turn = [&](bool more, uint4 (&x)[NI][BLK]) {
-            if (pt == 0 && pks > 0 && made < steps) {
+            if (pt == 0 && made < steps && made <= pks + lead) {
                 ok = ok && ptx::mbar_wait(ptx::smem_addr(&ctl.a_empty[pa.s]), (pa.wraps & 1u) ^ 1u, abort);
                 if (ok) make();
             }
@@ -414,37 +461,40 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         // split add their sums before anything is written to the sketch, whose rows are then written by whole warps.
         float* const stage = reinterpret_cast<float*>(ring);
         const int stride = gen_stage_stride(r_pad);
+        auto load_sums = [&](int t, int c, uint32_t (&v)[16]) {              // sixteen columns of a tile, a row per thread
+            if (steps > 0) {
+                const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(t * acc_cols + c);
+                ptx::tmem_ld_16(at, v);
+                if (F32) {
+                    uint32_t v1[16], v2[16];
+                    ptx::tmem_ld_16(at + r_pad, v1);
+                    if (sbs) ptx::tmem_ld_16(at + 2 * r_pad, v2);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int k = 0; k < 16; ++k)
+                        v[k] = __float_as_uint(join_parts(__uint_as_float(v[k]), __uint_as_float(v1[k]) + (sbs ? __uint_as_float(v2[k]) : 0.0f)));
+                } else {
+                    ptx::tmem_ld_wait();
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) v[k] = 0u;
+            }
+        };
         auto stage_tile = [&](int t, float* to) {
             const int row = (warp & 3) * 32 + lane;
             __syncwarp();
             for (int c = (warp >> 2) * 16; c < r_pad; c += 4 * WORKERS) {
                 uint32_t v[16];
-                if (steps > 0) {
-                    const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(t * acc_cols + c);
-                    ptx::tmem_ld_16(at, v);
-                    if (F32) {
-                        uint32_t v1[16], v2[16];
-                        ptx::tmem_ld_16(at + r_pad, v1);
-                        if (sbs) ptx::tmem_ld_16(at + 2 * r_pad, v2);
-                        ptx::tmem_ld_wait();
-#pragma unroll
-                        for (int k = 0; k < 16; ++k)
-                            v[k] = __float_as_uint(join_parts(__uint_as_float(v[k]), __uint_as_float(v1[k]) + (sbs ? __uint_as_float(v2[k]) : 0.0f)));
-                    } else {
-                        ptx::tmem_ld_wait();
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) v[k] = 0u;
-                }
+                load_sums(t, c, v);
 #pragma unroll
                 for (int k = 0; k < 16; k += 4)
                     *reinterpret_cast<float4*>(to + row * stride + c + k) =
                         make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]), __uint_as_float(v[k + 3]));
             }
         };
-        // Rows [lr0, lr1) of the CTA's tiles -> sketch; value(i, j): the finished sum.  The first values of the old sketch that a
-        // thread needs are fetched by `fetch_old`, before the sums are there.
+        // The sketch's old values, in pieces of four where its rows allow that.  The first ones that a thread needs are fetched by
+        // `fetch_old`, before they are used.
         constexpr int NOLD = 2;
         const bool vec = (r & 3) == 0 && (mat.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(mat.S) & 15) == 0;
         const int per = vec ? r >> 2 : r;                                    // pieces per row
@@ -466,6 +516,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 if (b != 0.0f && tid + k * NT < (lr1 - lr0) * per) old[k] = old_at(tid + k * NT, lr0, grow0);
             }
         };
+        // Rows [lr0, lr1) of the CTA's tiles -> sketch; value(i, j): the finished sum.
         auto write_rows = [&](int lr0, int lr1, int grow0, auto value) {
             auto put = [&](int e, float4 o) {
                 const int i = e / per, j = e - i * per;
@@ -484,10 +535,9 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
 #pragma unroll 4
             for (int e = tid + NOLD * NT; e < total_e; e += NT) put(e, b != 0.0f ? old_at(e, lr0, grow0) : make_float4(0.f, 0.f, 0.f, 0.f));
         };
-        const int rows = tiles * 128, lr0 = part * rows / split, lr1 = (part + 1) * rows / split;
-        if (split > 1) fetch_old(lr0, lr1, tile0 * 128);
         if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
         ptx::tc_fence_after_sync();
+        if (barrier) ptx::cluster_wait_some();
         if (split == 1) {
             for (int t = 0; t < tiles; ++t) {
                 fetch_old(0, 128, (tile0 + t) * 128);
@@ -500,11 +550,41 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                         return vec ? *reinterpret_cast<const float4*>(p) : make_float4(*p, 0.f, 0.f, 0.f);
                     });
             }
-            if (cluster > 1) {
+            if (cluster > 1 && joining == GEN_JOIN_ORDERED) {
                 ptx::cluster_sync_some();
                 ptx::cluster_sync_some();
             }
+        } else if (joining != GEN_JOIN_ORDERED) {
+            const bool adds = steps > 0 && !*abort;
+            for (int t = 0; t < tiles; ++t) {
+                if (vec) {
+                    const int row = (tile0 + t) * 128 + (warp & 3) * 32 + lane;
+                    float* const dst = mat.S + (int64_t)row * mat.lds;
+                    for (int c = (warp >> 2) * 16; c < r_pad; c += 4 * WORKERS) {
+                        uint32_t v[16];
+                        __syncwarp();
+                        load_sums(t, c, v);
+#pragma unroll
+                        for (int k = 0; k < 16; k += 4)
+                            if (adds && row < mat.n && c + k < r)
+                                ptx::red_add_v4(dst + c + k, a * __uint_as_float(v[k]), a * __uint_as_float(v[k + 1]), a * __uint_as_float(v[k + 2]), a * __uint_as_float(v[k + 3]));
+                    }
+                } else {
+                    // (through shared memory: neighbouring threads then add to neighbouring values)
+                    if (t > 0) ptx::named_barrier_sync(1, NT);
+                    stage_tile(t, stage);
+                    ptx::named_barrier_sync(1, NT);
+                    const int grow0 = (tile0 + t) * 128, total_e = adds ? min(128, mat.n - grow0) * r : 0;
+#pragma unroll 4
+                    for (int e = tid; e < total_e; e += NT) {
+                        const int i = e / r, j = e - i * r;
+                        ptx::red_add(mat.S + (int64_t)(grow0 + i) * mat.lds + j, a * stage[i * stride + j]);
+                    }
+                }
+            }
         } else {
+            const int lr0 = part * (tiles * 128) / split, lr1 = (part + 1) * (tiles * 128) / split;
+            fetch_old(lr0, lr1, tile0 * 128);
             for (int t = 0; t < tiles; ++t) stage_tile(t, stage + t * 128 * stride);
             ptx::cluster_sync_some();                                        // every partial sum of the cluster is staged
             const uint32_t sbase = ptx::smem_addr(stage);
@@ -534,10 +614,12 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
             ptx::cluster_sync_some();                                        // nobody leaves while a peer may still read its sums
         }
     }
-    if (warp == WORKERS && cluster > 1) {
-        __syncwarp();
-        ptx::cluster_sync_some();
-        ptx::cluster_sync_some();
+    if (warp == WORKERS) {
+        if (barrier) ptx::cluster_wait_some();
+        else if (cluster > 1 && joining == GEN_JOIN_ORDERED) {
+            ptx::cluster_sync_some();
+            ptx::cluster_sync_some();
+        }
     }
     ptx::tc_fence_before_sync();
     __syncthreads();

@@ -17,6 +17,7 @@ struct GenK1Plan {
     bool sbs = false;
     size_t smem = 0;
     bool aligned = true;
+    bool ordered = false;      // bit-reproducible sums
 };
 
 inline bool gen_aligned(const flora_mat& g)
@@ -31,7 +32,7 @@ inline int64_t gen_f32_chain(int64_t steps) { return std::min<int64_t>(GEN_F32_C
 // Rings, accumulator layout and CTAs per SM for T tiles per CTA; false where they do not fit.  `per_sm` = 2: two CTAs with at
 // most 112 KB and 256 accumulator columns each.  At least three slots of G and two of A (with fewer the warps wait for the MMAs of
 // the step before: fp32 4096 x 11008 at r = 8 ran at half the speed).
-inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int per_sm)
+inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int per_sm, int64_t steps)
 {
     const int r_pad = (r + 15) & ~15, most_cols = per_sm == 2 ? 256 : 512;
     p.sbs = f32 && 3 * r_pad <= 256 && T * 3 * r_pad <= most_cols;
@@ -43,7 +44,10 @@ inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int p
     if (3 * g + 2 * a > budget || staged > budget) return false;
     p.T = T;
     p.per_sm = per_sm;
+    // Slots of A: three, or one for each step of a short run, so that all may be made while the kernel before this one runs (24 KB at
+    // most, and four slots of G stay).
     p.a_slots = budget >= 4 * g + 3 * a ? 3 : 2;
+    if (p.a_slots == 3 && steps <= GEN_A_SLOTS_MAX && steps * a <= std::min<size_t>(24 * 1024, budget - 4 * g)) p.a_slots = (int)std::max<int64_t>(3, steps);
     p.g_slots = (int)std::min<size_t>(GEN_G_SLOTS_MAX, (budget - p.a_slots * a) / g);
     p.smem = std::max(p.g_slots * g + p.a_slots * a, staged) + 1024;
     // no more CTAs on an SM than its tensor memory serves: the CTAs of a cluster wait for one another, so none may wait for columns
@@ -56,14 +60,17 @@ inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int p
 // Cost model of the compression (cycles of one SM).  A step of T tiles takes its share of HBM (16 KB a tile, 700 cycles) or the
 // issue slots of generating and converting it, whichever is longer, and no less than the latency of one warp's part of it
 // (about 2100 cycles a tile with eight warps, 1500 with sixteen: measured); a CTA costs about two microseconds before its first
-// and after its last step, more with sixteen warps, and a little more when it adds up with others.
-inline double gen_k1_cost(bool f32, int r, int T, int workers, double together, int64_t waves, int64_t steps, int split)
+// and after its last step, more with sixteen warps, and a little more when it adds up with others.  premade: all its tiles of A are
+// made beside the kernel before it (700 x 2001 at r = 255, us a launch in a chain with 8, 10, 12, 14, 16 CTAs along the columns: 20.0, 19.9,
+// 15.1, 22.8, 19.9; with twelve two launches fit side by side).
+inline double gen_k1_cost(bool f32, int r, int T, int workers, double together, int64_t waves, int64_t steps, int split, bool premade = false)
 {
+    if (premade) return 4000.0 + (workers == 16 ? 2000.0 : 0.0) + (split > 1 ? 200.0 : 0.0) + (double)steps * 1500.0 * T;
     const int K = f32 ? 32 : 64;
     const double issue = 0.5 * r * K + (f32 ? 900.0 : 600.0) * T;
     const double quads = ceil((double)r * K / 4 / (32.0 * workers)), latency = (workers == 16 ? 1500.0 : 2100.0) * T + 330.0 * quads;
     const double step = std::max(latency, std::max(1.0, together) * std::max(700.0 * T, issue));
-    return (double)waves * (4000.0 + (workers == 16 ? 2000.0 : 0.0) + (split > 1 ? 1000.0 + 50.0 * split : 0.0) + (double)steps * step);
+    return (double)waves * (4000.0 + (workers == 16 ? 2000.0 : 0.0) + (split > 1 ? 200.0 : 0.0) + (double)steps * step);
 }
 // Clusters of `size` CTAs of the compression kernel that can be resident (asked once per kind of launch: the kernel's variants
 // need the same registers, so one stands for all).
@@ -83,10 +90,14 @@ inline int gen_k1_resident(const GenK1Plan& p, int size)
     known.push_back({dev, p.workers, size, n, p.smem});
     return n;
 }
+// Whether a launch of so many CTAs leaves half of the GPU free: in a chain of such launches it starts beside its predecessor and has the time
+// to fill its ring of A.
+inline bool gen_k1_beside(const GenK1Plan& p, int64_t ctas) { return 2 * ctas <= (int64_t)sm_count() * p.per_sm; }
 // Tile shape and split with the shortest schedule.  Chosen once per shape and kept (64 of them).
-inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
+// clusters: the CTAs of a split form one (see GenJoin); without, any free slot will do, and more CTAs are resident.
+inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bool clusters)
 {
-    struct Known { int dev, r; bool f32; int64_t tiles, steps; GenK1Plan plan; };
+    struct Known { int dev, r; bool f32, clusters; int64_t tiles, steps; GenK1Plan plan; };
     static std::mutex mutex;
     static std::vector<Known> known;
     int dev = 0;
@@ -94,7 +105,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
     std::lock_guard<std::mutex> lock(mutex);
     if (tune_knob("FLORA_GEN_T", 0, 0, 4)) known.clear();        // (a sweep over shapes)
     for (const Known& k : known)
-        if (k.dev == dev && k.r == r && k.f32 == f32 && k.tiles == tiles && k.steps == steps) return k.plan;
+        if (k.dev == dev && k.r == r && k.f32 == f32 && k.clusters == clusters && k.tiles == tiles && k.steps == steps) return k.plan;
     GenK1Plan best;
     double least = 1e300;
     for (int T = 1; T <= 4; T *= 2)
@@ -106,23 +117,27 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps)
                     tune_knob("FLORA_GEN_WORKERS", workers, 8, 16) != workers)
                     continue;
                 GenK1Plan p;
-                if (!gen_k1_shape(p, f32, r, T, split > 1, workers == 16 ? 1 : 2)) continue;    // (registers: one CTA of sixteen warps)
+                if (!gen_k1_shape(p, f32, r, T, split > 1, workers == 16 ? 1 : 2, (steps + split - 1) / split)) continue;    // (registers: one CTA of sixteen warps)
                 p.cluster = split;
                 p.workers = workers;
-                const int64_t clusters = (tiles + T - 1) / T, resident = gen_k1_resident(p, split);
-                const double together = std::min<double>(p.per_sm, (double)(std::min(clusters, resident) * split) / sm_count());
-                const double cost = gen_k1_cost(f32, r, T, workers, together, (clusters + resident - 1) / resident, (steps + split - 1) / split, split);
+                const int64_t groups = (tiles + T - 1) / T;
+                // (waves of row groups: what is left of a wave that is not full counts as one)
+                const int64_t resident = clusters ? gen_k1_resident(p, split) : (int64_t)sm_count() * p.per_sm;
+                const int64_t units = clusters ? groups : groups * split;
+                const double together = std::min<double>(p.per_sm, (double)(std::min(units, resident) * (clusters ? split : 1)) / sm_count());
+                const double cost = gen_k1_cost(f32, r, T, workers, together, (units + resident - 1) / resident, (steps + split - 1) / split, split,
+                                                gen_k1_beside(p, groups * split) && (steps + split - 1) / split <= p.a_slots);
                 if (cost < least * 0.98) {
                     least = cost;
                     best = p;
                 }
             }
     if (least > 1e299) {                                          // (one tile, no split, one CTA per SM fits every rank)
-        gen_k1_shape(best, f32, r, 1, false, 1);
+        gen_k1_shape(best, f32, r, 1, false, 1, steps);
         best.workers = 16;
     }
     if (known.size() >= 64) known.erase(known.begin());
-    known.push_back({dev, r, f32, tiles, steps, best});
+    known.push_back({dev, r, f32, clusters, tiles, steps, best});
     return best;
 }
 
@@ -136,6 +151,11 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     cfg.blockDim = dim3((unsigned)gen_threads(WORKERS));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = st;
+    const int joining = p.ordered ? GEN_JOIN_ORDERED : b != 1.0f ? GEN_JOIN_SCALED : GEN_JOIN_PLAIN;
+    // Tiles of A made before the wait: all slots where there is time for it, or where that takes half a microsecond a tile at most; one
+    // otherwise, and the loads go out as soon as they may (1000 x 4097 at r = 64, all slots / one: 15.6 / 13.8 us; the ragged set of eight matrices at
+    // r = 32, a compression: 11.2 / 13.5).
+    const int ahead = gen_k1_beside(p, (int64_t)clusters * p.cluster) || r * (F32 ? 32 : 64) <= 2048 ? p.a_slots : 1;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // the kernel waits for its predecessor itself
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -144,9 +164,9 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = p.cluster > 1 ? 2 : 1;
+    cfg.numAttrs = p.cluster > 1 && joining != GEN_JOIN_PLAIN ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, seeds, one, split, col0, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
-                              (int)p.sbs, p.g_slots, p.a_slots, p.cluster);
+                              (int)p.sbs, p.g_slots, p.a_slots, p.cluster, joining, ahead);
 }
 inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds,
                                         const GenMat& one, int split, int col0, int seed_base, int r, float a, float b, cudaStream_t st,
@@ -179,14 +199,18 @@ inline bool gen_supported(const flora_mat& big) { return big.rows < (1ll << 31) 
 // r = 128 11.6 / 9.9, but 2816 x 1024 at r = 64 8.9 / 9.4 and 2048 x 2048 at r = 256 15.5 / 31.4.
 // A set of small matrices stops gaining a little earlier (its TMA kernels start once for all): `elements` of a set are counted
 // as 5/3.  (4 x 768 x 768 at r = 16: compress 11.1 / 7.0, decompress 6.6 / 6.0; 7 M elements at r = 16: 13.6 / 12.9 and 10.4 / 13.8.)
-inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32)
+// One matrix at a time, in a chain (with the TMA kernels and with these): bf16 1600 x 4800 at r = 16 12.2 / 9.2 (momentum 13.2 / 12.5), at r = 64 17.8 / 16.8, 6400 x 1600 at
+// r = 32 14.3 / 12.8, but 768 x 9216 10.8 / 11.5 and 4096 x 4096 at r = 64 17.3 / 22.0; 2048 x 2048 at r = 128 14.0 / 14.4; fp32 2048 x 2048 at r = 8 11.4 / 9.0, at
+// r = 128 21.3 / 19.7, but at r = 256 25.5 / 32.3 and 1024 x 4096 at r = 8 11.6 / 12.2.
+inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32, bool set)
 {
     const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
     if (knob >= 0) return knob == 1;
-    // (fp32: 1024 x 1024 at r = 8 12.6 / 8.3, at r = 64 22 / 12; 768 x 3072 at r = 64 23 / 15.5; 2048 x 2048 at r = 64 23.5 / 21; 1024 x 4096 at
-    // r = 64 23.5 / 24.3.  Bit-reproducible results of long rows need the split over a cluster, which only these kernels have.)
-    if (f32) return (cols <= 3072 && elements <= 5 << 19) || deterministic_flag().load();
-    return cols <= 4096 && elements <= (r <= 64 ? 4 << 20 : 5 << 18);
+    // (fp32: 1024 x 1024 at r = 8 12.6 / 8.3, at r = 64 22 / 12; 768 x 3072 at r = 64 23 / 15.5.  Bit-reproducible results of long rows need the
+    // split over a cluster, which only these kernels have.)
+    if (f32) return (cols <= 3072 && elements <= (set || r > 128 ? 5 << 19 : 4 << 20)) || deterministic_flag().load();
+    if (r > 64) return cols <= 4096 && elements <= 5 << 18;
+    return set ? cols <= 4096 && elements <= 4 << 20 : cols <= 5120 && elements <= 10 << 20;
 }
 inline bool gen_decompress_quicker(int64_t elements, int r, bool f32)
 {
@@ -205,9 +229,33 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
     const int r = (int)S.cols;
     const int64_t pass = f32 ? GEN_F32_PASS_COLS : G.cols;
     const int64_t tiles = (G.rows + 127) / 128, steps = (std::min(G.cols, pass) + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
-    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps);
+    const bool ordered = deterministic_flag().load() != 0;
+    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps, ordered);
     const int64_t groups = (tiles + p.T - 1) / p.T;
     p.aligned = gen_aligned(G);
+    p.ordered = ordered;
+    // Rows that several CTAs add to are scaled by the launch itself where its clusters fit beside a predecessor, by a pass of its own in front
+    // of it otherwise.  (Momentum step, in one launch of clusters / with a pass, us: 768 x 2304 at r = 16 5.5 / 7.3, but 2048 x 2048 at
+    // r = 32 11.3 / 10.1, 3000 x 5001 at r = 18 in fp32 52.7 / 41.5.)
+    if (!ordered && p.cluster > 1 && b != 1.0f && !(gen_k1_beside(p, groups * p.cluster) && gen_k1_resident(p, p.cluster) >= groups)) {
+        TcMatrix one;
+        memset(&one, 0, sizeof(one));
+        one.S = (float*)S.data;
+        one.lds = S.ld;
+        one.n = (int32_t)G.rows;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(std::min(helper_blocks(G.rows * r), (unsigned)sm_count() * 6));
+        cfg.blockDim = dim3(256);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<true>, (const TcMatrix*)nullptr, one, (const int*)nullptr, 0, r, b) != cudaSuccess) return FLORA_ERR_CUDA;
+        launches.fetch_add(1, std::memory_order_relaxed);
+        b = 1.0f;
+    }
     SeedTable table;
     table.s[0] = seed;
     int64_t col0 = 0;
@@ -362,7 +410,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         // One kind of CTA for the whole list: one tile, eight warps, two to an SM, where that fits (more tiles to share a tile of A
         // lose more to the longer step than they save: measured); per matrix as many CTAs along the columns as leave each about a
         // third of an SM's share of the work, and a single short wave on a small list.
-        const int per_sm = gen_k1_shape(s.plan, s.f32, s.r, 1, true, 2) ? 2 : 1;
+        const int per_sm = gen_k1_shape(s.plan, s.f32, s.r, 1, true, 2, GEN_A_SLOTS_MAX + 1) ? 2 : 1;
         const int64_t share = std::max<int64_t>(2, total / (per_sm * sms * 3));
         std::vector<int> split(big.size(), 1);
         int cluster = 1;
@@ -416,8 +464,11 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         most = tune_knob("FLORA_GEN_MOST", most, 1, GEN_MAX_SPLIT);
         cut_columns(most);
         const int T = 1;
-        if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm)) return FLORA_ERR_UNSUPPORTED;
+        int64_t longest = 1;
+        for (int i : ids) longest = std::max(longest, (steps_of(i, 0) + split[i] - 1) / split[i]);
+        if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm, longest)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
+        s.plan.ordered = deterministic_flag().load() != 0;
         std::vector<GenItem> items;
         for (int64_t pass = 0; pass < passes; ++pass) {
             cuts.clear();

@@ -100,6 +100,23 @@ __device__ __forceinline__ void cluster_sync_some()
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
+// The two halves of that barrier, in the same manner.  relaxed: of threads whose writes another thread's release covers (it has met
+// them at a barrier of the CTA before).
+__device__ __forceinline__ void cluster_arrive_release()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait_some()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
 // Reads of another CTA's shared memory (address from map_to_cta).
 __device__ __forceinline__ float4 ld_cluster_v4(uint32_t cluster_addr)
 {
@@ -202,6 +219,12 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+// Counts this thread at such a barrier without waiting there.
+__device__ __forceinline__ void named_barrier_arrive(uint32_t id, uint32_t nthreads)
+{
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 template <int N>
 __device__ __forceinline__ void tma_store_wait_read()
@@ -378,6 +401,7 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
 {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
+__device__ __forceinline__ void red_add(float* p, float a) { asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory"); }
 // 16-byte asynchronous copy global -> shared by the calling thread (both addresses 16-byte aligned), grouped and
 // awaited per thread.
 __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src)
