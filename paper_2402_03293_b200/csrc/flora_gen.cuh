@@ -27,11 +27,12 @@ struct GenMat {            // a matrix with its sketch
     int64_t ld, lds;
     int32_t n, m;
 };
-struct GenItem {           // compression: one cluster
+struct GenItem {           // compression: one cluster, or one CTA of a split whose CTAs form none
     int32_t mat;
     int32_t tile0;         // first 128-row tile
     int32_t split;         // CTAs of the cluster that share the columns of one row group
     int32_t col0;          // first column (fp32: a launch takes GEN_F32_PASS_COLS columns)
+    int32_t part;          // without clusters: which part of the split
 };
 
 // Warps that load, convert, generate and write out (8, or 16 where a CTA has an SM to itself), and one that issues the MMAs.
@@ -121,8 +122,7 @@ __device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, f
 // 64 bf16 values) at a time.  Worker warps fetch the rows with plain 16-byte loads, two tiles ahead in registers (rows that start
 // off a 16-byte boundary: two aligned loads per piece, shifted together), cut fp32 values into parts and write operand
 // tiles; the same warps generate the step's tile of A while the loads are under way.  One thread issues the MMAs.
-// Where a matrix has too few rows to fill the GPU, `split` CTAs of a cluster share its columns and add their partial sums
-// through distributed shared memory: one launch, one writer per element, and the sums do not depend on arrival order.
+// Where a matrix has too few rows to fill the GPU, `split` CTAs share its columns and add their sums to the sketch (GenJoin).
 // ------------------------------------------------------------------------------------------------
 template <bool F32>
 struct GenK1 {
@@ -196,9 +196,10 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         item.split = single_split;
         item.tile0 = cl * (cluster / single_split) * T;
         item.col0 = single_col0;
+        item.part = 0;
     }
     const GenMat mat = SINGLE ? single : mats[item.mat];
-    const int split = item.split, group = rank / split, part = rank % split;
+    const int split = item.split, group = rank / split, part = item.part + rank % split;
     const int tile0 = item.tile0 + group * T;
     const int tiles = max(0, min(T, ((mat.n + 127) >> 7) - tile0));
     const int m_end = F32 ? item.col0 + min(mat.m - item.col0, GEN_F32_PASS_COLS) : mat.m;      // columns beyond it are another launch's
@@ -457,8 +458,8 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 if (u + d < total) turn(u + d + AHEAD < total, x[d]);
         }
         // ------------------------------------------------------------------ write-out
-        // Accumulators -> shared memory (the operand rings, free by now), one row of a tile per thread.  The other CTAs of a
-        // split add their sums before anything is written to the sketch, whose rows are then written by whole warps.
+        // A split: accumulators -> sketch, added in global memory, a row of a tile per thread.  Otherwise, and where rows have no 16-byte
+        // pieces: accumulators -> shared memory (the operand rings, free by now), whose rows whole warps then add or write.
         float* const stage = reinterpret_cast<float*>(ring);
         const int stride = gen_stage_stride(r_pad);
         auto load_sums = [&](int t, int c, uint32_t (&v)[16]) {              // sixteen columns of a tile, a row per thread

@@ -18,6 +18,8 @@ struct GenK1Plan {
     size_t smem = 0;
     bool aligned = true;
     bool ordered = false;      // bit-reproducible sums
+    bool beside = false;       // two such launches fit side by side (see gen_k1_choose)
+    double cost = 0;           // by gen_k1_cost
 };
 
 inline bool gen_aligned(const flora_mat& g)
@@ -90,14 +92,15 @@ inline int gen_k1_resident(const GenK1Plan& p, int size)
     known.push_back({dev, p.workers, size, n, p.smem});
     return n;
 }
-// Whether a launch of so many CTAs leaves half of the GPU free: in a chain of such launches it starts beside its predecessor and has the time
-// to fill its ring of A.
-inline bool gen_k1_beside(const GenK1Plan& p, int64_t ctas) { return 2 * ctas <= (int64_t)sm_count() * p.per_sm; }
 // Tile shape and split with the shortest schedule.  Chosen once per shape and kept (64 of them).
-// clusters: the CTAs of a split form one (see GenJoin); without, any free slot will do, and more CTAs are resident.
-inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bool clusters)
+// clusters: the CTAs of a split form one (see GenJoin); without, any free slot will do, and more CTAs are resident.  A launch that leaves
+// half of the GPU free (beside) starts, in a chain of such launches, beside its predecessor and has the time to fill its ring of A; clusters
+// that do not also lose what single CTAs find in the gaps, about the time of making two tiles of A (1000 x 4097 at r = 64, a momentum step: 17.7 us in
+// clusters, 14.0 without and with a pass that scales the sketch).
+// chain: it stands behind launches like itself (compressions of a cycle).
+inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bool clusters, bool chain)
 {
-    struct Known { int dev, r; bool f32, clusters; int64_t tiles, steps; GenK1Plan plan; };
+    struct Known { int dev, r; bool f32, clusters, chain; int64_t tiles, steps; GenK1Plan plan; };
     static std::mutex mutex;
     static std::vector<Known> known;
     int dev = 0;
@@ -105,7 +108,8 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
     std::lock_guard<std::mutex> lock(mutex);
     if (tune_knob("FLORA_GEN_T", 0, 0, 4)) known.clear();        // (a sweep over shapes)
     for (const Known& k : known)
-        if (k.dev == dev && k.r == r && k.f32 == f32 && k.clusters == clusters && k.tiles == tiles && k.steps == steps) return k.plan;
+        if (k.dev == dev && k.r == r && k.f32 == f32 && k.clusters == clusters && k.chain == chain && k.tiles == tiles && k.steps == steps) return k.plan;
+    const int K = f32 ? 32 : 64;
     GenK1Plan best;
     double least = 1e300;
     for (int T = 1; T <= 4; T *= 2)
@@ -125,10 +129,12 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
                 const int64_t resident = clusters ? gen_k1_resident(p, split) : (int64_t)sm_count() * p.per_sm;
                 const int64_t units = clusters ? groups : groups * split;
                 const double together = std::min<double>(p.per_sm, (double)(std::min(units, resident) * (clusters ? split : 1)) / sm_count());
-                const double cost = gen_k1_cost(f32, r, T, workers, together, (units + resident - 1) / resident, (steps + split - 1) / split, split,
-                                                gen_k1_beside(p, groups * split) && (steps + split - 1) / split <= p.a_slots);
+                p.beside = 2 * groups * split <= (int64_t)sm_count() * p.per_sm;
+                double cost = gen_k1_cost(f32, r, T, workers, together, (units + resident - 1) / resident, (steps + split - 1) / split, split,
+                                          !clusters && (chain || r * K <= 2048) && p.beside && (steps + split - 1) / split <= p.a_slots);
+                if (clusters && split > 1 && !p.beside) cost += 1.25 * r * K;
                 if (cost < least * 0.98) {
-                    least = cost;
+                    least = p.cost = cost;
                     best = p;
                 }
             }
@@ -137,7 +143,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
         best.workers = 16;
     }
     if (known.size() >= 64) known.erase(known.begin());
-    known.push_back({dev, r, f32, clusters, tiles, steps, best});
+    known.push_back({dev, r, f32, clusters, chain, tiles, steps, best});
     return best;
 }
 
@@ -155,7 +161,7 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     // Tiles of A made before the wait: all slots where there is time for it, or where that takes half a microsecond a tile at most; one
     // otherwise, and the loads go out as soon as they may (1000 x 4097 at r = 64, all slots / one: 15.6 / 13.8 us; the ragged set of eight matrices at
     // r = 32, a compression: 11.2 / 13.5).
-    const int ahead = gen_k1_beside(p, (int64_t)clusters * p.cluster) || r * (F32 ? 32 : 64) <= 2048 ? p.a_slots : 1;
+    const int ahead = p.beside || r * (F32 ? 32 : 64) <= 2048 ? p.a_slots : 1;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // the kernel waits for its predecessor itself
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -230,14 +236,20 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
     const int64_t pass = f32 ? GEN_F32_PASS_COLS : G.cols;
     const int64_t tiles = (G.rows + 127) / 128, steps = (std::min(G.cols, pass) + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
     const bool ordered = deterministic_flag().load() != 0;
-    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps, ordered);
+    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps, ordered, b == 1.0f);
+    // Rows that several CTAs add to are scaled by the launch itself, in clusters, or by a pass of its own in front of it, which takes one or two
+    // microseconds of a chain and the time of its bytes.  (Momentum step, in clusters / with a pass, us: 768 x 2304 at r = 16 5.5 / 6.4, but 2048 x 2048
+    // at r = 32 11.3 / 9, 3000 x 5001 at r = 18 in fp32 52.7 / 37.6.)
+    bool scale_first = false;
+    if (!ordered && p.cluster > 1 && b != 1.0f) {
+        const GenK1Plan c = gen_k1_choose(f32, r, tiles, steps, true, false);
+        scale_first = c.cost > p.cost + 3000.0 + 0.01 * (double)(G.rows * r);
+        if (!scale_first) p = c;
+    }
     const int64_t groups = (tiles + p.T - 1) / p.T;
     p.aligned = gen_aligned(G);
     p.ordered = ordered;
-    // Rows that several CTAs add to are scaled by the launch itself where its clusters fit beside a predecessor, by a pass of its own in front
-    // of it otherwise.  (Momentum step, in one launch of clusters / with a pass, us: 768 x 2304 at r = 16 5.5 / 7.3, but 2048 x 2048 at
-    // r = 32 11.3 / 10.1, 3000 x 5001 at r = 18 in fp32 52.7 / 41.5.)
-    if (!ordered && p.cluster > 1 && b != 1.0f && !(gen_k1_beside(p, groups * p.cluster) && gen_k1_resident(p, p.cluster) >= groups)) {
+    if (scale_first) {
         TcMatrix one;
         memset(&one, 0, sizeof(one));
         one.S = (float*)S.data;
@@ -343,9 +355,12 @@ struct GenSet {
     std::vector<GenMat> h_mats;                // one entry per matrix of the set (members filled in)
     GenMat* d_mats = nullptr;
     GenItem* d_k1 = nullptr;
+    GenItem* d_plain = nullptr;                // compression that only adds (b = 1): CTAs of a split form no clusters there
     GenK2Item* d_k2 = nullptr;
     int* d_share = nullptr;                    // decompression: per launch, the first item of every CTA and the end
     std::vector<int> begin, first_mat;         // compression: ranges of items per launch; decompression: where its table starts in d_share
+    std::vector<int> plain_begin, plain_first; // ... its ranges and first matrices
+    GenK1Plan plain;
     std::vector<uint8_t> adds;                 // compression: launches behind the first columns of their matrices, which add to them
     std::vector<unsigned> grid;                // decompression: CTAs per launch
     int bn = 64;
@@ -359,6 +374,7 @@ inline void gen_set_free(GenSet& s)
 {
     if (s.d_mats) cudaFree(s.d_mats);
     if (s.d_k1) cudaFree(s.d_k1);
+    if (s.d_plain) cudaFree(s.d_plain);
     if (s.d_k2) cudaFree(s.d_k2);
     if (s.d_share) cudaFree(s.d_share);
     s = GenSet();
@@ -378,16 +394,15 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
     int count = 0;
-    auto launches_of = [&](bool adds, auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
+    auto launches_of = [&](std::vector<int>& begin, std::vector<int>& first_mat, auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
         size_t u0 = 0;
         while (u0 < cuts.size()) {
             size_t u1 = u0;
             const int first = cuts[u0].mat;
             while (u1 < cuts.size() && cuts[u1].mat < first + SEEDS_PER_LAUNCH) ++u1;
             std::stable_sort(cuts.begin() + u0, cuts.begin() + u1, [](const Cut& x, const Cut& y) { return x.work > y.work; });
-            s.begin.push_back(count);
-            s.first_mat.push_back(first);
-            s.adds.push_back(adds ? 1 : 0);
+            begin.push_back(count);
+            first_mat.push_back(first);
             for (size_t u = u0; u < u1; ++u, ++count) emit(cuts[u]);
             u0 = u1;
         }
@@ -477,12 +492,60 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
                 if (pass > 0 && steps == 0) continue;
                 for (int64_t t0 = 0; t0 < tiles; t0 += per)
                     cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]),
-                                    {i, (int32_t)t0, split[i], s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0}});
+                                    {i, (int32_t)t0, split[i], s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0, 0}});
             }
-            launches_of(pass > 0, [&](const Cut& c) { items.push_back(c.item); });
+            launches_of(s.begin, s.first_mat, [&](const Cut& c) { items.push_back(c.item); });
+            s.adds.resize(s.begin.size(), pass > 0 ? 1 : 0);
         }
         s.begin.push_back(count);
-        return upload(&s.d_k1, items, st);
+        rc = upload(&s.d_k1, items, st);
+        if (rc || s.plan.ordered) return rc;
+        // Where nothing is to be scaled: single CTAs, and as many steps for each as make the shortest sum of waves.  (The ragged set of eight matrices
+        // at r = 32, a compression: 9.6 -> 8.4 us, in fp32 20.3 -> 11.7; 24 matrices of GPT-2-small shapes with an odd column 70.9 -> 65.4)
+        int64_t most_steps = 1;
+        for (int i : ids) most_steps = std::max(most_steps, steps_of(i, 0));
+        auto parts_of = [&](int i, int64_t per, int64_t pass) {
+            const int64_t steps = steps_of(i, pass);
+            if (s.f32) per = std::min(per, gen_f32_chain(steps_of(i, 0)));
+            return std::max<int64_t>(1, (steps + per - 1) / per);
+        };
+        int64_t best_per = most_steps;
+        double least = 1e300;
+        for (int64_t per = 1; per <= most_steps; per += std::max<int64_t>(1, per / 8)) {
+            int64_t ctas = 0, longest_run = 1;
+            for (int i : ids) {
+                const int64_t parts = parts_of(i, per, 0);
+                ctas += (big[i].rows + 127) / 128 * parts;
+                longest_run = std::max(longest_run, (steps_of(i, 0) + parts - 1) / parts);
+            }
+            const int64_t slots = sms * per_sm, waves = (ctas + slots - 1) / slots;
+            const double together = std::min<double>(per_sm, (double)ctas / sms);
+            const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, together, waves, longest_run, 2);
+            if (cost < least * 0.98) {
+                least = cost;
+                best_per = per;
+            }
+        }
+        s.plain = s.plan;
+        int64_t longest_run = 1;
+        for (int i : ids) longest_run = std::max(longest_run, (steps_of(i, 0) + parts_of(i, best_per, 0) - 1) / parts_of(i, best_per, 0));
+        if (!gen_k1_shape(s.plain, s.f32, s.r, 1, true, per_sm, longest_run)) return FLORA_ERR_UNSUPPORTED;
+        s.plain.cluster = 1;
+        std::vector<GenItem> plain;
+        count = 0;
+        for (int64_t pass = 0; pass < passes; ++pass) {
+            cuts.clear();
+            for (int i : ids) {
+                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass), parts = parts_of(i, best_per, pass);
+                if (pass > 0 && steps == 0) continue;
+                for (int64_t t0 = 0; t0 < tiles; ++t0)
+                    for (int64_t part = 0; part < parts; ++part)
+                        cuts.push_back({i, (steps + parts - 1) / parts, {i, (int32_t)t0, (int32_t)parts, s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0, (int32_t)part}});
+            }
+            launches_of(s.plain_begin, s.plain_first, [&](const Cut& c) { plain.push_back(c.item); });
+        }
+        s.plain_begin.push_back(count);
+        return upload(&s.d_plain, plain, st);
     }
     // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
     bool aligned = true;
@@ -532,6 +595,14 @@ inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
 inline flora_status gen_set_compress(GenSet& s, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
     if (s.ready() && s.plan.aligned && !s.captured_aligned) s.captured_aligned = capturing(st);
+    if (b == 1.0f && s.d_plain) {
+        for (size_t l = 0; l + 1 < s.plain_begin.size(); ++l) {
+            const flora_status rc = gen_compress_launch(s.f32, s.plain, s.plain_begin[l + 1] - s.plain_begin[l], s.d_mats, s.d_plain + s.plain_begin[l],
+                                                        gen_seeds(s, seeds, s.plain_first[l]), GenMat{}, 1, 0, s.plain_first[l], s.r, a, b, st, launches);
+            if (rc) return rc;
+        }
+        return FLORA_OK;
+    }
     for (size_t l = 0; l + 1 < s.begin.size(); ++l) {
         const flora_status rc = gen_compress_launch(s.f32, s.plan, s.begin[l + 1] - s.begin[l], s.d_mats, s.d_k1 + s.begin[l],
                                                     gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, 0, s.first_mat[l], s.r, a, s.adds[l] ? 1.0f : b, st,
@@ -568,7 +639,7 @@ inline flora_status gen_set_rebind(GenSet& s, const std::vector<flora_mat>& big,
         s.h_mats[i].big = big[i].data;
         aligned = aligned && gen_aligned(big[i]);
     }
-    s.plan.aligned = aligned;
+    s.plan.aligned = s.plain.aligned = aligned;
     return upload(&s.d_mats, s.h_mats, st);
 }
 
