@@ -184,10 +184,10 @@ bool small_compress(int64_t elements, int64_t cols, int r, bool f32, bool set)
     if (g_force_path.load(std::memory_order_relaxed) == 2) return f32 && deterministic_flag().load();
     return gen_compress_quicker(elements, cols, r, f32, set);
 }
-bool small_decompress(int64_t elements, int r, bool f32)
+bool small_decompress(int64_t elements, int r, bool f32, bool loose)
 {
     if (g_force_path.load(std::memory_order_relaxed) == 2) return f32 && r > K2_F32_MAX_R;
-    return gen_decompress_quicker(elements, r, f32);
+    return gen_decompress_quicker(elements, r, f32, loose);
 }
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 {
@@ -197,7 +197,7 @@ bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
 {
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_decompress_supported(big, sketch) &&
-           !small_decompress(big->rows * big->cols, (int)sketch->cols, big->dtype == FLORA_F32);
+           !small_decompress(big->rows * big->cols, (int)sketch->cols, big->dtype == FLORA_F32, !tc_sketch_ok(*sketch));
 }
 
 }  // namespace
@@ -221,24 +221,28 @@ struct flora_set {
 // Below this many elements the matrices of a mixed set that TMA could serve are not worth a launch of their own (4 M
 // elements are 8 MB, a microsecond and a half of HBM time): all its matrices then go to the kernels of flora_gen.cuh.
 constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
+// The same for sets with sketches that TMA cannot address, which also want a scaling pass and a copy of the sketches: eleven matrices of which three
+// with 4.5 M elements are TMA's, r = 7, momentum step and update: 85.7 us with launches of their own, 72.9 without; twelve with 30 M, r = 37: 63 and 206.
+constexpr int64_t LOOSE_SET_TMA_MIN_ELEMENTS = 16ll << 20;
 
 // Which matrices of one side (G: compression, or W: decompression) of a set the TMA kernels serve.
 static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression, bool f32 = false)
 {
-    std::vector<uint8_t> use = tc_eligible(big, S, f32);
+    std::vector<uint8_t> use = tc_eligible(big, S, f32, !f32);
     if (compression && f32)
-        for (size_t i = 0; i < big.size(); ++i) use[i] = use[i] && big[i].cols >= K1_F32_MIN_COLS;
+        for (size_t i = 0; i < big.size(); ++i) use[i] = use[i] && big[i].cols >= K1_F32_MIN_COLS && sketch_writable(S[i]);
     int64_t eligible = 0, widest = 0;
-    bool mixed = false;
+    bool mixed = false, loose = false;
     for (size_t i = 0; i < big.size(); ++i) {
         if (use[i]) eligible += big[i].rows * big[i].cols;
         else mixed = mixed || big[i].rows > 0;
         widest = std::max(widest, big[i].cols);
+        loose = loose || (!f32 && !tc_sketch_ok(S[i]));
     }
     const int r = S.empty() ? 1 : (int)S[0].cols;
     const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
-    if ((mixed && eligible < MIXED_SET_TMA_MIN_ELEMENTS && g_force_path.load() != 2) ||
-        (compression ? small_compress(counted, widest, r, f32, true) : small_decompress(counted, r, f32)))
+    if (((mixed || loose) && eligible < (loose && big.size() > 1 ? LOOSE_SET_TMA_MIN_ELEMENTS : mixed ? MIXED_SET_TMA_MIN_ELEMENTS : 0) && g_force_path.load() != 2) ||
+        (compression ? small_compress(counted, widest, r, f32, true) : small_decompress(counted, r, f32, loose)))
         std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
 }
@@ -258,6 +262,12 @@ static flora_status set_build(flora_set* s)
     std::vector<uint8_t> use_w = set_tma_side(s->W, s->S, false);
     auto any = [](const std::vector<uint8_t>& use) { return std::find(use.begin(), use.end(), (uint8_t)1) != use.end(); };
     flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
+    if (st == FLORA_ERR_ALLOC && !s->S.empty() && !tc_sketch_ok(s->S[0]) && any(use_w)) {
+        // no room for the copy of sketches that TMA cannot address: the kernels that need none take the weights
+        tc_set_free(s->tc);
+        std::fill(use_w.begin(), use_w.end(), (uint8_t)0);
+        st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
+    }
     if (st == FLORA_OK && (any(use_f) || any(use_wf)))
         st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, nullptr, use_f, use_wf);
     for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
@@ -371,7 +381,10 @@ flora_status flora_decompress_apply(flora_mat* W, const flora_mat* C, uint64_t s
     flora_status st = check_pair(W, C);
     if (st) return st;
     if (W->rows == 0 || W->cols == 0) return FLORA_OK;
-    if (use_tc_decompress(W, C)) return tc_decompress_single(W, C, seed, lr * scale, as_stream(stream), g_launches);
+    if (use_tc_decompress(W, C)) {
+        st = tc_decompress_single(W, C, seed, lr * scale, as_stream(stream), g_launches);
+        if (st != FLORA_ERR_ALLOC || tc_sketch_ok(*C)) return st;      // (no room for the copy of a sketch that TMA cannot address: without one)
+    }
     if (use_gen(W)) return gen_decompress_single(*W, *C, seed, lr * scale, as_stream(stream), g_launches);
     return simt_decompress(W, C, seed, lr * scale, as_stream(stream));
 }

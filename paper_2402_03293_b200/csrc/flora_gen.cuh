@@ -55,27 +55,6 @@ enum GenJoin { GEN_JOIN_ORDERED, GEN_JOIN_SCALED, GEN_JOIN_PLAIN };
 // launches, whose sums are added in rounded fp32 (one after another, so in a fixed order).
 constexpr int GEN_F32_PASS_COLS = 32 * GEN_MAX_SPLIT * GEN_F32_CHAIN_STEPS;
 
-// The parts of two fp32 values, as fp32 bit patterns whose low 16 bits are to be dropped.
-struct Parts2 {
-    uint32_t h0, h1, m0, m1, l0, l1;
-};
-__device__ __forceinline__ Parts2 split3(float x0, float x1)
-{
-    Parts2 p;
-    p.h0 = __float_as_uint(x0);
-    p.h1 = __float_as_uint(x1);
-    float r0, r1, l0, l1;
-    unpack2(fma2(pack2(__uint_as_float(p.h0 & 0xFFFF0000u), __uint_as_float(p.h1 & 0xFFFF0000u)), FLORA_BOTH(0xBF800000) /* -1 */, pack2(x0, x1)), r0, r1);   // exact
-    p.m0 = __float_as_uint(r0);
-    p.m1 = __float_as_uint(r1);
-    unpack2(fma2(pack2(__uint_as_float(p.m0 & 0xFFFF0000u), __uint_as_float(p.m1 & 0xFFFF0000u)), FLORA_BOTH(0xBF800000) /* -1 */, pack2(r0, r1)), l0, l1);   // exact
-    p.l0 = __float_as_uint(l0);
-    p.l1 = __float_as_uint(l1);
-    return p;
-}
-// Two bf16 values from the high halves of two fp32 bit patterns; `a` goes into the low half.
-__device__ __forceinline__ uint32_t pack_high(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
-
 // Operand tiles in shared memory: rows of ROWB = 64 or 128 bytes (K-major), swizzled over 16-byte chunks as the tensor core
 // expects (64-byte rows: chunk ^ (row / 2) % 4; 128-byte rows: chunk ^ row % 8).
 template <int ROWB>
@@ -722,8 +701,11 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
             item = items[it++];
         }
         const GenMat mat = SINGLE ? single : mats[item.mat];
-        // W moves in 16-byte pieces where its rows and the slab allow it, element by element otherwise
-        const bool vec = item.col0 + BN <= mat.m && ((reinterpret_cast<uintptr_t>(mat.big) | (uintptr_t)(mat.ld * ES)) & 15) == 0;
+        // W moves in 16-byte pieces where its rows and the slab's end allow it, element by element otherwise.  (The last slab element by
+        // element although its columns are whole pieces: 1224 x 4896 at r = 11 17.4 us instead of 10.9, 32 matrices of GPT-2 shapes of width 1192
+        // at r = 11 472 instead of 199)
+        const bool vec = (item.col0 + BN <= mat.m || mat.m % E == 0) && ((reinterpret_cast<uintptr_t>(mat.big) | (uintptr_t)(mat.ld * ES)) & 15) == 0;
+        const bool piece_in = item.col0 + wp * E < mat.m;
         const bool svec = ((reinterpret_cast<uintptr_t>(mat.S) | (uintptr_t)(mat.lds * 4)) & 15) == 0;
         auto load_x = [&](int t, int kc) {
             const int j = kc * KB + sq * 4, row = (item.tile0 + t) * 128 + srow;
@@ -750,7 +732,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
 #pragma unroll
                 for (int i = 0; i < NP; ++i, src += (GEN_K2_THREADS / PPR) * mat.ld * ES) {
                     uint4 v = make_uint4(0, 0, 0, 0);
-                    if (row0 + wrow + (GEN_K2_THREADS / PPR) * i < mat.n) v = *reinterpret_cast<const uint4*>(src);
+                    if (piece_in && row0 + wrow + (GEN_K2_THREADS / PPR) * i < mat.n) v = *reinterpret_cast<const uint4*>(src);
                     w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
                 }
             } else if (NE <= 32) {
@@ -897,7 +879,7 @@ gen_decompress_kernel(const GenMat* __restrict__ mats, const GenK2Item* __restri
 #pragma unroll
                 for (int i = 0; i < NP; ++i, dst += (GEN_K2_THREADS / PPR) * mat.ld * ES) {
                     const int lr = wrow + (GEN_K2_THREADS / PPR) * i;
-                    if (row0 + lr >= mat.n) continue;
+                    if (!piece_in || row0 + lr >= mat.n) continue;
                     const float* acc = staging + lr * STRIDE + wp * E;
                     uint32_t* y = &w[4 * i];
                     const float4 s0 = *reinterpret_cast<const float4*>(acc);

@@ -218,14 +218,17 @@ inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32
     if (r > 64) return cols <= 4096 && elements <= 5 << 18;
     return set ? cols <= 4096 && elements <= 4 << 20 : cols <= 5120 && elements <= 10 << 20;
 }
-inline bool gen_decompress_quicker(int64_t elements, int r, bool f32)
+// loose: TMA cannot address the sketch; the TMA kernel then reads a copy of its three parts.  (bf16 1224 x 4896 at r = 7 14.5 / 10.8, at r = 45 16.5 / 17.4, at r =
+// 255 28.7 / 49; 4096 x 11008 at r = 7 39.0 / 52.9.  Tight, 768 x 3072 at r = 96 14.4 / 11.2, 2048 x 2048 at r = 128 14.5 / 16.3.)
+inline bool gen_decompress_quicker(int64_t elements, int r, bool f32, bool loose)
 {
     const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
     if (knob >= 0) return knob == 1;
     // (fp32, with these and with the TMA kernel: 512 x 512 at r = 8 3.8 / 4.2, 1024 x 1024 at r = 8 4.6 / 5.3, at r = 64 6.6 / 6.7, at r = 128
     // 10.5 / 8.7, 1024 x 4096 at r = 64 15.6 / 12.0, 4096 x 11008 at r = 8 81 / 63.5)
     if (f32) return elements <= (r <= 32 ? 1 << 20 : 1 << 19) || r > K2_F32_MAX_R;
-    return elements <= (r <= 32 ? 5 << 20 : r <= 64 ? 2 << 20 : 5 << 18);
+    if (r > 64) return elements <= (r <= 128 ? 5 << 19 : 5 << 18);
+    return elements <= (loose ? (r <= 32 ? 14 << 20 : 5 << 20) : r <= 32 ? 5 << 20 : 2 << 20);
 }
 
 inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, uint64_t seed, float a, float b, cudaStream_t st,

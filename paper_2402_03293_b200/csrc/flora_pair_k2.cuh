@@ -51,7 +51,7 @@ struct K2Cursor {
 // 2p (leader) and 2p + 1 (follower; it may not exist, then the follower loads and stores nothing for that iteration).
 // Iterations are numbered through all items of the cluster (gt); the even ones belong to the first MMA thread, its
 // ring of sketch chunks (cstages / 2 stages) and accumulators 0 and 2, the odd ones to the second.
-template <bool SINGLE>
+template <bool SINGLE, int PARTS = 1>
 __global__ void __launch_bounds__(K2P_THREADS, 1)
 decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K2Item* __restrict__ items, int n_items, const __grid_constant__ SeedTable seeds,
                        int seed_base, int r, float scale, float step, int slots, int cstages)
@@ -60,6 +60,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     const int kchunks = (r + 63) >> 6;                          // 64 values of the rank per 128-byte row of bf16
+    const int schunks = kchunks * PARTS;                        // (PARTS: see sketch_to_parts_kernel)
     const uint32_t slab_block = 64u * 128u;                     // one K chunk of this CTA's half of a slab: 64 columns of W
     const uint32_t slab_bytes = (uint32_t)kchunks * slab_block;
     const uint32_t slab0 = smem_base;
@@ -209,7 +210,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
             // (programmatic dependent launch): nothing else here reads what that kernel writes
             ptx::grid_dependency_wait();
             while (ok && (cs[0].it < n_items || cs[1].it < n_items)) {
-                for (int kc = 0; kc < kchunks && ok; ++kc) {
+                for (int kc = 0; kc < schunks && ok; ++kc) {
 #pragma unroll
                     for (int x = 0; x < 2; ++x) {
                         if (cs[x].it >= n_items) continue;
@@ -267,7 +268,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
                     const int a = gt & (K2P_ACCS - 1);
                     const uint32_t acc_addr = tmem + (uint32_t)a * K2P_BN;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[a]), (((uint32_t)gt >> 2) & 1u) ^ 1u, abort);
-                    for (int kc = 0; kc < kchunks && ok; ++kc, pc.advance(ring_stages)) {
+                    for (int kc = 0, kq = 0; kc < schunks && ok; ++kc, pc.advance(ring_stages)) {
                         const int s = pc.s;
                         const uint32_t full = ptx::smem_addr(&ctl->c_full[x * ring_stages + s]);
                         ok = ptx::mbar_wait(full, pc.wraps & 1u, abort);
@@ -278,10 +279,12 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
                             // descriptors differ from the ring / slab base only in the start-address field (16-byte units); the
                             // same offsets address the follower's chunk and its half of the slab
                             const uint64_t da = desc_ring + (uint64_t)((s * S_CHUNK_BYTES + k16 * 32) >> 4);
-                            const uint64_t db = desc_slab + (uint64_t)((kc * slab_block + k16 * 32) >> 4);
+                            const uint64_t db = desc_slab + (uint64_t)(((PARTS > 1 ? kq : kc) * slab_block + k16 * 32) >> 4);
+                            if (PARTS > 1 && kq * 64 + k16 * 16 >= r) break;               // (zeros)
                             ptx::umma_bf16_pair(acc_addr, da, db, idesc, (kc | k16) != 0);
                         }
                         ptx::umma_commit_pair(ptx::smem_addr(&ctl->c_empty[x * ring_stages + s]), (uint16_t)3u);
+                        if (PARTS > 1 && ++kq == kchunks) kq = 0;
                     }
                     if (ok) ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[a]), (uint16_t)3u);
                 }
@@ -298,7 +301,7 @@ decompress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant
             RingPos pc;
             bool ok = true;
             while (ok && c.it < n_items) {
-                for (int kc = 0; kc < kchunks; ++kc, pc.advance(ring_stages)) {
+                for (int kc = 0; kc < schunks; ++kc, pc.advance(ring_stages)) {
                     const uint32_t bar = ptx::smem_addr(&ctl->c_full[x * ring_stages + pc.s]);
                     ok = ptx::mbar_wait(bar, pc.wraps & 1u, abort);
                     if (!ok) break;

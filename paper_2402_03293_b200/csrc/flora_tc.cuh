@@ -21,6 +21,27 @@
 
 namespace flora {
 
+// The parts of two fp32 values, as fp32 bit patterns whose low 16 bits are to be dropped.
+struct Parts2 {
+    uint32_t h0, h1, m0, m1, l0, l1;
+};
+__device__ __forceinline__ Parts2 split3(float x0, float x1)
+{
+    Parts2 p;
+    p.h0 = __float_as_uint(x0);
+    p.h1 = __float_as_uint(x1);
+    float r0, r1, l0, l1;
+    unpack2(fma2(pack2(__uint_as_float(p.h0 & 0xFFFF0000u), __uint_as_float(p.h1 & 0xFFFF0000u)), FLORA_BOTH(0xBF800000) /* -1 */, pack2(x0, x1)), r0, r1);   // exact
+    p.m0 = __float_as_uint(r0);
+    p.m1 = __float_as_uint(r1);
+    unpack2(fma2(pack2(__uint_as_float(p.m0 & 0xFFFF0000u), __uint_as_float(p.m1 & 0xFFFF0000u)), FLORA_BOTH(0xBF800000) /* -1 */, pack2(r0, r1)), l0, l1);   // exact
+    p.l0 = __float_as_uint(l0);
+    p.l1 = __float_as_uint(l1);
+    return p;
+}
+// Two bf16 values from the high halves of two fp32 bit patterns; `a` goes into the low half.
+__device__ __forceinline__ uint32_t pack_high(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
+
 // ------------------------------------------------------------------------------------------------
 // device-side tables
 // ------------------------------------------------------------------------------------------------
@@ -29,12 +50,13 @@ struct alignas(128) TcMatrix {
     CUtensorMap map_w;   // weight W, same box (loads and stores)
     CUtensorMap map_s;   // sketch S (fp32), box 32 columns x 128 rows, 128-byte swizzle
     CUtensorMap map_sq;  // sketch S, box 32 columns x 32 rows (what one warp of an epilogue writes), 128-byte swizzle
-    CUtensorMap map_sb;  // bf16 copy of S (scratch, n x k_pad), box 64 columns x 128 rows, 128-byte swizzle
+    CUtensorMap map_sb;  // bf16 copy of S (scratch, n x k_pad, or its three parts side by side), box 64 columns x 128 rows, 128-byte swizzle
     __nv_bfloat16* Sb;   // the bf16 copy (used by the decompression kernel for ranks above 64)
     float* S;            // sketch, n x r fp32
     int64_t lds;
     int32_t n, m;
-    int32_t pad[24];
+    int32_t loose;       // TMA cannot address the rows of S (no map_s, map_sq): the compression writes them with plain accesses
+    int32_t pad[23];
 };
 static_assert(sizeof(TcMatrix) % 128 == 0, "matrix records hold TMA descriptors");
 
@@ -84,6 +106,25 @@ struct GMaps<0> {
 // set; a third of that costs 0.3.  (Host time of a launch without maps, with 48, with 192: 3.2, 3.4, 4.6 us; the GPU's is the same.)
 constexpr int GMAPS_FEW = 64, GMAPS_MANY = 192;
 
+// Writes 32 rows x 32 columns of accumulators, staged in shared memory as a sketch's tensor map would have them (128-byte rows,
+// swizzled), into a sketch that TMA cannot address: ranks that are no multiple of four, or bases off 16 bytes.  One warp; its lanes
+// take the columns of a row, or of two or four rows where there are few, and add to them or store them.  (A sketch that is to be
+// blended has been scaled before: reading the old values here took a momentum step of 96 matrices at r = 255 from 502 to 746 us.)
+__device__ __forceinline__ void write_piece(uint32_t buf, float* S, int64_t lds, int n, int r, int row0, int col0, int lane, bool add)
+{
+    const int cols = min(32, r - col0), rows = min(32, n - row0);
+    const int shift = cols > 16 ? 5 : cols > 8 ? 4 : 3, j = lane & ((1 << shift) - 1), step = 32 >> shift;
+    float* p = S + (int64_t)(row0 + (lane >> shift)) * lds + col0 + j;
+#pragma unroll 4
+    for (int i = lane >> shift; i < rows; i += step, p += step * lds) {
+        if (j >= cols) continue;
+        float v;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(buf + (uint32_t)(i * 128 + ((((j >> 2) ^ (i & 7)) << 4) | ((j & 3) << 2)))));
+        if (add) ptx::red_add(p, v);
+        else *p = v;
+    }
+}
+
 constexpr int SEEDS_PER_LAUNCH = 448;
 struct SeedTable {
     uint64_t s[SEEDS_PER_LAUNCH];
@@ -129,7 +170,8 @@ struct K1Smem {                            // barriers and scalars, placed after
 // new_maps: those in the table may have been written since the kernel before.
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
 // 4096 x 11008 matrix takes 27 us instead of 20)
-template <bool SINGLE, bool F32, int MAPS>
+// LOOSE: a sketch may be one that TMA cannot address (a template parameter: tested at run time it cost the others 1 to 2 %).
+template <bool SINGLE, bool F32, int MAPS, bool LOOSE = false>
 __global__ void __maxnreg__(80)
 compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
                    int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int lstages, int nsets, int S, int GW, int P,
@@ -458,7 +500,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
             ptx::tc_fence_after_sync();
             if (late_wait) ptx::grid_dependency_wait();
             const bool add = item.direct == 0 || b == 1.0f;
-            const bool rmw = !add && b != 0.0f;
+            const bool loose = LOOSE && mat->loose != 0, rmw = !add && b != 0.0f;
             const int nchunks = (r + 31) >> 5;
             const int total = item.tiles * nchunks;               // chunks of this CTA; the group takes grp, grp + EG, ...
             const int NB = min(areas / EG, 4);                    // buffers of this group
@@ -537,6 +579,12 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                         x3 = fmaf(b, __uint_as_float(o3), x3);
                     }
                     ptx::st_shared_v4(addr, __float_as_uint(x0), __float_as_uint(x1), __float_as_uint(x2), __float_as_uint(x3));
+                }
+                if (loose) {                                          // every warp writes out the rows that it staged
+                    __syncwarp();
+                    write_piece(buffer(u) + (uint32_t)(quarter * 32) * 128u, mat->S, mat->lds, mat->n, r, item.row0 + t * 128 + quarter * 32, c * 32, lane,
+                                add);
+                    continue;
                 }
                 ptx::fence_proxy_async_smem();
                 ptx::named_barrier_sync(bar_b, 128);
@@ -655,7 +703,8 @@ __device__ __forceinline__ void k2_generate_slab(uint32_t slab, uint32_t slab_bl
 // rows, and the small products have accumulators to themselves.  The tensor core truncates its sums, and the loss grows with the length
 // of the chain: slices of eight columns take two pairs of accumulators in turn (W after a step of 5 %, against 64 bits: r = 128 3.06e-8
 // with one pair, plain fp32 arithmetic 2.70e-8).  Four warps cut the sketch's chunks in shared memory.  W's boxes are 32 columns wide.
-template <bool SINGLE, bool BF16S, bool F32>
+// PARTS: 3 where the copy of the sketch holds its parts.
+template <bool SINGLE, bool BF16S, bool F32, int PARTS = 1>
 __global__ void __launch_bounds__(K2_MAX_THREADS, 1)
 decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const K2Item* __restrict__ items, int n_items,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, float scale, float step, int bn, int slots,
@@ -666,6 +715,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     // K chunks: one 128-byte row of S each (32 fp32 values, or 64 bf16 values when the bf16 copy of S is used)
     const int kchunks = BF16S ? (r + 63) >> 6 : (r + 31) >> 5;
+    const int schunks = kchunks * PARTS;                       // (the parts follow one another and meet the same slab)
     constexpr int WC = F32 ? 32 : 64;                          // columns of a box of W
     const int boxes = bn / WC;                                 // boxes per W tile
     const uint32_t slab_block = (uint32_t)bn * (F32 ? 256u : 128u);   // one K chunk of a slab
@@ -764,7 +814,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 const K2Item item = items[it];
                 const TcMatrix* mat = mats + item.mat;
                 for (int i = 0; i < item.tiles && ok; ++i) {
-                    for (int kc = 0; kc < kchunks; ++kc, ++gc, pc.advance(cstages)) {
+                    for (int kc = 0; kc < schunks; ++kc, ++gc, pc.advance(cstages)) {
                         const int s = pc.s;
                         ok = ptx::mbar_wait(ptx::smem_addr(&ctl->c_empty[s]), (pc.wraps & 1u) ^ 1u, abort);
                         if (!ok) break;
@@ -796,7 +846,7 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                 for (int i = 0; i < item.tiles && ok; ++i, ++gt) {
                     const uint32_t acc_addr = tmem + (gt & 1) * acc_cols;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[gt & 1]), ((gt >> 1) & 1) ^ 1, abort);
-                    for (int kc = 0; kc < kchunks && ok; ++kc, ++gc, pc.advance(cstages)) {
+                    for (int kc = 0, kq = 0; kc < schunks && ok; ++kc, ++gc, pc.advance(cstages)) {
                         const int s = pc.s;
                         if (F32) {
                             // (the chunk's lower part is there, so the chunk is, too)
@@ -822,11 +872,13 @@ decompress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                         for (int k8 = 0; k8 < 4; ++k8) {
                             // descriptors differ from the ring / slab base only in the start-address field (16-byte units)
                             const uint64_t da = desc_ring + (uint64_t)((s * S_CHUNK_BYTES + k8 * 32) >> 4);
-                            const uint64_t db = desc_slab + (uint64_t)((kc * slab_block + k8 * 32) >> 4);
+                            const uint64_t db = desc_slab + (uint64_t)(((PARTS > 1 ? kq : kc) * slab_block + k8 * 32) >> 4);
+                            if (PARTS > 1 && kq * 64 + k8 * 16 >= r) break;               // (zeros)
                             if (BF16S) ptx::umma_bf16(acc_addr, da, db, idesc, (kc | k8) != 0);
                             else ptx::umma_tf32(acc_addr, da, db, idesc, (kc | k8) != 0);
                         }
                         ptx::umma_commit(ptx::smem_addr(&ctl->c_empty[s]));
+                        if (PARTS > 1 && ++kq == kchunks) kq = 0;
                     }
                     if (ok) ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[gt & 1]));
                 }
@@ -1106,6 +1158,42 @@ __global__ void __launch_bounds__(256) sketch_to_bf16_kernel(const TcMatrix* __r
         out.z = *reinterpret_cast<uint32_t*>(&p2);
         out.w = *reinterpret_cast<uint32_t*>(&p3);
         *reinterpret_cast<uint4*>(Sb + (int64_t)row * k_pad + j) = out;
+    }
+}
+
+// The same for sketches that TMA cannot address (ranks that are no multiple of four, bases off 16 bytes): their decompression has always
+// multiplied the whole fp32 value, so the copy holds its three exact parts side by side (the smallest first), n x 3 k_pad, and the
+// kernel runs over all of them.  The lower parts of an infinity are stored as zero: all products go into one sum.
+template <bool SINGLE>
+__global__ void __launch_bounds__(256) sketch_to_parts_kernel(const TcMatrix* __restrict__ mats, const __grid_constant__ TcMatrix single, int r, int k_pad)
+{
+    ptx::grid_launch_dependents();
+    const TcMatrix* mat = SINGLE ? &single : mats + blockIdx.y;
+    const int groups = k_pad >> 3, rows_per_block = 256 / groups;
+    const int g = (int)threadIdx.x % groups, lr = (int)threadIdx.x / groups;
+    if (lr >= rows_per_block) return;
+    const int j = g * 8;
+    __nv_bfloat16* Sb = mat->Sb;
+    if (!Sb) return;
+    for (int row = (int)blockIdx.x * rows_per_block + lr; row < mat->n; row += (int)gridDim.x * rows_per_block) {
+        const float* src = mat->S + (int64_t)row * mat->lds + j;
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = j + e < r ? src[e] : 0.0f;
+        uint32_t h[4], m[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            Parts2 p = split3(v[2 * e], v[2 * e + 1]);
+            if (isinf(v[2 * e])) p.m0 = p.l0 = 0u;
+            if (isinf(v[2 * e + 1])) p.m1 = p.l1 = 0u;
+            h[e] = pack_high(p.h0, p.h1);
+            m[e] = pack_high(p.m0, p.m1);
+            l[e] = pack_high(p.l0, p.l1);
+        }
+        uint4* const out = reinterpret_cast<uint4*>(Sb + (int64_t)row * (3 * k_pad) + j);
+        out[0] = make_uint4(l[0], l[1], l[2], l[3]);
+        out[k_pad / 8] = make_uint4(m[0], m[1], m[2], m[3]);
+        out[k_pad / 4] = make_uint4(h[0], h[1], h[2], h[3]);
     }
 }
 

@@ -29,6 +29,7 @@ struct TcSet {
     bool decompress_ready = false;
     int count = 0, r = 0;
     bool f32 = false;                   // fp32 gradients
+    bool loose = false;                 // a sketch whose rows TMA cannot address
     int T = 1, gstages = 2, astages = 2, lstages = 1, nsets = 1, S = 1, GW = 8, P = 1;
     std::vector<int> k1_launch_first_mat;
     size_t k1_smem = 0;
@@ -55,7 +56,8 @@ struct TcSet {
     // decompression
     int bn = 128, slots = 2, cstages = 2, k2_gw = 8, k2_nslabs = 2, k2_grid_max = 148;
     bool k2_f32 = false;                // the weights are fp32
-    bool k2_bf16 = false;               // ranks above 64: the kernel reads a bf16 copy of the sketches
+    bool k2_bf16 = false;               // ranks above 64, and sketches that TMA cannot address: the kernel reads a bf16 copy of the sketches
+    int k2_parts = 1;                   // ... of this many parts (three: the fp32 values as they are)
     bool k2_pair = false;               // ... and runs on CTA pairs (decompress_pair_kernel); k2_grid_max then counts pairs
     __nv_bfloat16* d_sb = nullptr;      // that copy (scratch owned by the set)
     std::vector<int> k2_launch_first_mat;
@@ -103,6 +105,10 @@ inline bool tc_sketch_ok(const flora_mat& s)
     return (reinterpret_cast<uintptr_t>(s.data) & 15) == 0 && (s.ld & 3) == 0 && s.cols >= 1 && s.cols <= 256;
 }
 
+// Whether the compression may write the sketch's rows by TMA: it clips a row's end to 16 bytes only, so a rank that is no multiple of four must not
+// have anything else behind it.
+inline bool sketch_writable(const flora_mat& s) { return tc_sketch_ok(s) && (s.cols & 3) == 0; }
+
 inline bool tc_mat_ok(const flora_mat& a)
 {
     return a.dtype == FLORA_BF16 && a.rows >= 128 && a.cols >= 64 && (reinterpret_cast<uintptr_t>(a.data) & 15) == 0 &&
@@ -123,7 +129,8 @@ inline bool tc_f32_ok(const flora_mat& a)
 
 inline bool tc_compress_supported(const flora_mat* big, const flora_mat* sketch)
 {
-    return (tc_mat_ok(*big) || (tc_f32_ok(*big) && big->cols >= K1_F32_MIN_COLS)) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
+    // (a bf16 matrix may have a sketch that TMA cannot address: the write-out then takes plain accesses)
+    return (tc_mat_ok(*big) || (tc_f32_ok(*big) && big->cols >= K1_F32_MIN_COLS && sketch_writable(*sketch))) && encode_tiled_fn() != nullptr;
 }
 
 // SMs of the current device (a process may drive several devices), asked once per device.
@@ -627,7 +634,7 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
 
 // Work decomposition of the decompression kernel: column slabs of bn columns, cut into runs of row tiles; the
 // persistent CTAs take the items round-robin, largest first.
-inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
+inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r, bool loose = false)
 {
     // ranks up to 64 read the fp32 sketch directly (tf32 MMA); above that the bytes of S that a CTA pulls per W
     // tile exceed what shared memory can keep in flight, so a bf16 copy of S is made first (half the bytes,
@@ -635,9 +642,10 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     bool f32 = false;
     for (const auto& w : W) f32 = f32 || (w.rows > 0 && w.dtype == FLORA_F32);
     set.k2_f32 = f32;
-    const bool bf16s = !f32 && tune_knob("FLORA_K2_BF16S", r > 64 ? 1 : 0, 0, 1) != 0;
+    const bool bf16s = !f32 && tune_knob("FLORA_K2_BF16S", r > 64 || loose ? 1 : 0, 0, 1) != 0;
+    set.k2_parts = loose ? 3 : 1;
     set.k2_bf16 = bf16s;
-    const int kchunks = bf16s ? (r + 63) / 64 : (r + 31) / 32;
+    const int kchunks = bf16s ? (r + 63) / 64 : (r + 31) / 32, schunks = kchunks * set.k2_parts;      // of a slab, and of the sketch's rows of a tile
     // slabs of 128 columns (every chunk of S then serves twice the columns of W) whenever two slabs, two W slots and
     // two S chunks of that width fit; 64 columns otherwise
     const size_t ctl = sizeof(K2Smem) + 1024;
@@ -655,7 +663,7 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     int nslabs = (2 * slab_bytes + 4 * S_CHUNK_BYTES + (f32 ? 3 : 2) * slot + lower + ctl <= SMEM_BUDGET) ? 2 : 1;
     nslabs = tune_knob("FLORA_K2_SLABS", nslabs, 1, 2);
     const size_t budget = SMEM_BUDGET - ctl - nslabs * slab_bytes - lower;
-    int cstages = std::max(2, std::min(nslabs == 1 ? 2 * kchunks : kchunks + 1, nslabs == 1 ? K2_MAX_CSTAGES : 4));
+    int cstages = std::max(2, std::min(nslabs == 1 ? 2 * schunks : schunks + 1, nslabs == 1 ? K2_MAX_CSTAGES : 4));
     cstages = tune_knob("FLORA_K2_CSTAGES", cstages, 1, K2_MAX_CSTAGES);
     while (cstages > 1 && (size_t)cstages * S_CHUNK_BYTES + (f32 && cstages > 4 ? 3 : 2) * slot > budget) --cstages;
     int slots = (int)std::min<size_t>(K2_MAX_SLOTS, (budget - (size_t)cstages * S_CHUNK_BYTES) / slot);
@@ -679,7 +687,7 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     if (pair) {
         const size_t half_slab = (size_t)kchunks * 64 * 128, pslot = 2 * (size_t)W_BOX_BYTES;
         const size_t pbudget = SMEM_BUDGET - sizeof(K2PairSmem) - 1024 - 2 * half_slab;
-        int pc = std::min(K2_MAX_CSTAGES, 2 * kchunks);
+        int pc = std::min(K2_MAX_CSTAGES, 2 * schunks);
         pc = tune_knob("FLORA_K2_CSTAGES", pc, 2, K2_MAX_CSTAGES);
         while (pc > 2 && (size_t)pc * S_CHUNK_BYTES + 2 * pslot > pbudget) --pc;
         pc &= ~1;                                        // two rings of equal depth, one per MMA-issuing thread
@@ -698,7 +706,7 @@ inline void plan_decompress(TcSet& set, const std::vector<flora_mat>& W, int r)
     // r*bn normals at the generator warps' rate and overlaps the previous item's streaming
     // (an SM takes in about 60 GB/s whatever the source: the chunks of S count like the W tile itself)
     const double t_tile = std::max((double)bn * 128 * (f32 ? 8 : 4) / (6.5e6 / sm_count()),
-                                   ((double)bn * 128 * (f32 ? 4 : 2) + (double)kchunks * S_CHUNK_BYTES) / K2_SM_BYTES_PER_US);
+                                   ((double)bn * 128 * (f32 ? 4 : 2) + (double)schunks * S_CHUNK_BYTES) / K2_SM_BYTES_PER_US);
     const double t_slab = (double)r * bn / (GW >= 8 ? K2_VALUES_PER_US_8_WARPS : K2_VALUES_PER_US_FEWER);   // generator warps share the SM with the streaming warps
     auto build = [&](int run, std::vector<K2Item>& out) {
         out.clear();
@@ -890,17 +898,20 @@ inline flora_status tc_fill_matrices(TcSet& set, const std::vector<flora_mat>& G
         tm.m = (int32_t)std::max(G.empty() ? (int64_t)0 : G[i].cols, W.empty() ? (int64_t)0 : W[i].cols);
         if (!G.empty() && G[i].rows && G[i].cols && !make_map(&tm.map_g, G[i])) return FLORA_ERR_CUDA;
         if (!W.empty() && W[i].rows && W[i].cols && !make_map(&tm.map_w, W[i])) return FLORA_ERR_CUDA;
+        tm.loose = !sketch_writable(S[i]);
+        set.loose = set.loose || (tm.loose && !G.empty() && G[i].rows > 0);
         if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !(make_map(&tm.map_s, S[i]) && make_map(&tm.map_sq, S[i], 32))) return FLORA_ERR_CUDA;
     }
     return FLORA_OK;
 }
 
-// What the TMA kernels can take of a set: the matrix has their type, size and alignment, and its sketch's rows can be addressed.
-inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool f32 = false)
+// What the TMA kernels can take of a set: the matrix has their type, size and alignment, and its sketch's rows can be addressed
+// (any_sketch: or not).
+inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool f32 = false, bool any_sketch = false)
 {
     std::vector<uint8_t> ok(big.size(), 0);
     if (encode_tiled_fn())
-        for (size_t i = 0; i < big.size(); ++i) ok[i] = (f32 ? tc_f32_ok(big[i]) : tc_mat_ok(big[i])) && tc_sketch_ok(S[i]);
+        for (size_t i = 0; i < big.size(); ++i) ok[i] = (f32 ? tc_f32_ok(big[i]) : tc_mat_ok(big[i])) && (any_sketch || tc_sketch_ok(S[i]));
     return ok;
 }
 
@@ -933,10 +944,12 @@ inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_
     flora_status rc = tc_fill_matrices(set, G, W, S);
     if (rc) return rc;
     if (w_ok) {
-        plan_decompress(set, W, set.r);
+        bool loose = false;
+        for (size_t i = 0; i < S.size(); ++i) loose = loose || (W[i].rows > 0 && !tc_sketch_ok(S[i]));
+        plan_decompress(set, W, set.r, loose);
         if (set.k2_bf16) {
-            // scratch for the bf16 copies of the sketches: n x k_pad each, 1 KB aligned
-            const int k_pad = (set.r + 63) & ~63;
+            // scratch for the bf16 copies of the sketches: n x k_pad (three times that in parts) each, 1 KB aligned
+            const int k_pad = ((set.r + 63) & ~63) * set.k2_parts;
             size_t total = 0;
             std::vector<size_t> offset(S.size());
             for (size_t i = 0; i < S.size(); ++i) {
@@ -1076,8 +1089,8 @@ inline unsigned helper_blocks(const TcSet& set)
 // compression waits for them.
 // one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).  mats: the table of the
 // others; new_maps: its maps may have been written since the kernel before.
-template <bool SINGLE, int MAPS>
-inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
+template <bool SINGLE, int MAPS, bool LOOSE>
+inline flora_status tc_compress_launch_as(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
                                        cudaStream_t st, std::atomic<uint64_t>& launches, bool behind_own_kernel, bool new_maps = false)
 {
     const int r = set.r;
@@ -1092,7 +1105,8 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, c
     if (SINGLE) state_bytes = (int64_t)one.n * r * 4;
     else
         for (int i : set.members) state_bytes += (int64_t)set.h_mats[i].n * r * 4;
-    const bool scale_all = pair && b != 0.0f && b != 1.0f && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES;
+    // Sketches that TMA cannot address are always scaled first (see write_piece).
+    const bool scale_all = b != 0.0f && b != 1.0f && (LOOSE || (pair && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES));
     if (scale_all || (b != 1.0f && !set.split_mats.empty())) {
         // A short pass is itself launched early, and the compression waits for it with everything (momentum step of one 4096 x 11008
         // matrix at r = 8 22.7 -> 21.4 us, with b = 0 22.9 -> 20.8; fp32 1024 x 4096 at r = 64 20.6 -> 18.5).  A long one starts behind
@@ -1121,8 +1135,8 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, c
         }
         if (scale_all) b = 1.0f;
     }
-    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE, MAPS>>()
-               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true, MAPS>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false, MAPS>>()))
+    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE, MAPS, LOOSE>>()
+               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true, MAPS>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false, MAPS, LOOSE>>()))
         return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k1_launch_begin.size(); ++l) {
         const int begin = set.k1_launch_begin[l], end = set.k1_launch_begin[l + 1];
@@ -1154,19 +1168,27 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, c
         cudaError_t e;
         if (pair) {
             const int* slot_table = set.d_slots + set.k1_slots_begin[l];
-            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE, MAPS>, mats, one, gmaps, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
+            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE, MAPS, LOOSE>, mats, one, gmaps, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
                                    set.astages, set.S, set.GW, lw, (int)new_maps);
         } else {
             auto go = [&](auto kernel) {
                 return cudaLaunchKernelEx(&cfg, kernel, mats, one, gmaps, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.lstages,
                                           set.nsets, set.S, set.GW, set.P, lw, (int)new_maps);
             };
-            e = set.f32 ? go(compress_tc_kernel<SINGLE, true, MAPS>) : go(compress_tc_kernel<SINGLE, false, MAPS>);
+            e = set.f32 ? go(compress_tc_kernel<SINGLE, true, MAPS>) : go(compress_tc_kernel<SINGLE, false, MAPS, LOOSE>);
         }
         if (e != cudaSuccess) return FLORA_ERR_CUDA;
         launches.fetch_add(1, std::memory_order_relaxed);
     }
     return cudaPeekAtLastError() == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
+}
+
+template <bool SINGLE, int MAPS>
+inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
+                                       cudaStream_t st, std::atomic<uint64_t>& launches, bool behind_own_kernel, bool new_maps = false)
+{
+    return (SINGLE ? one.loose != 0 : set.loose) ? tc_compress_launch_as<SINGLE, MAPS, true>(set, mats, one, seeds, a, b, st, launches, behind_own_kernel, new_maps)
+                                                 : tc_compress_launch_as<SINGLE, MAPS, false>(set, mats, one, seeds, a, b, st, launches, behind_own_kernel, new_maps);
 }
 
 inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
@@ -1188,11 +1210,11 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
 // plans once per shape (a plan whose launches have been recorded into a graph is never dropped: the graph reads its tables; a cache keyed by addresses planned every call anew in such loops: 43 us each).  Calls that use the
 // cache are serialised by its mutex; a plan is built with a synchronous upload, so any stream may use it afterwards.
 struct SinglePlanKey {
-    int dev, kind, r, det, dtype;
+    int dev, kind, r, det, dtype, loose;
     int64_t rows, cols;
     bool operator==(const SinglePlanKey& o) const
     {
-        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && dtype == o.dtype && rows == o.rows && cols == o.cols;
+        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && dtype == o.dtype && loose == o.loose && rows == o.rows && cols == o.cols;
     }
 };
 struct SinglePlan {
@@ -1222,6 +1244,7 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
     key.r = (int)sketch.cols;
     key.det = deterministic_flag().load();
     key.dtype = big.dtype;
+    key.loose = kind == 1 && !tc_sketch_ok(sketch);
     key.rows = big.rows;
     key.cols = big.cols;
     for (size_t i = 0; i < cache.size(); ++i)
@@ -1250,7 +1273,7 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
         *rc = upload(&set.d_k1, set.h_k1, st);
         if (*rc == FLORA_OK) *rc = upload(&set.d_slots, set.h_slots, st);
     } else {
-        plan_decompress(set, b, set.r);
+        plan_decompress(set, b, set.r, key.loose != 0);
         *rc = upload(&set.d_k2, set.h_k2, st);
     }
     if (*rc == FLORA_OK && cudaStreamSynchronize(st) != cudaSuccess) *rc = FLORA_ERR_CUDA;      // the tables are in place for every stream
@@ -1278,7 +1301,8 @@ inline bool single_record(TcMatrix* tm, const flora_mat& big, const flora_mat& s
     tm->lds = sketch.ld;
     tm->n = (int32_t)big.rows;
     tm->m = (int32_t)big.cols;
-    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && make_map(&tm->map_s, sketch) && (!is_g || make_map(&tm->map_sq, sketch, 32));
+    tm->loose = !sketch_writable(sketch);
+    return make_map(is_g ? &tm->map_g : &tm->map_w, big) && (!tc_sketch_ok(sketch) || (make_map(&tm->map_s, sketch) && (!is_g || make_map(&tm->map_sq, sketch, 32))));
 }
 
 inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, float a, float b, cudaStream_t st,
@@ -1310,11 +1334,14 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
             dim3 grid(bx, (unsigned)std::min(65535, set.count - begin));
             // (launched behind all earlier work: started early, beside the compression's CTAs, its blocks would crowd on the SMs that
             // those leave free)
-            sketch_to_bf16_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats + begin, one, r, k_pad);
+            if (set.k2_parts == 3) sketch_to_parts_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats + begin, one, r, k_pad);
+            else sketch_to_bf16_kernel<SINGLE><<<grid, 256, 0, st>>>(set.d_mats + begin, one, r, k_pad);
             launches.fetch_add(1, std::memory_order_relaxed);
         }
     }
-    if (!(set.k2_pair ? raise_smem_limit<decompress_pair_kernel<SINGLE>>()
+    const bool parts = set.k2_parts == 3;
+    if (!(set.k2_pair ? (parts ? raise_smem_limit<decompress_pair_kernel<SINGLE, 3>>() : raise_smem_limit<decompress_pair_kernel<SINGLE>>())
+                      : parts       ? raise_smem_limit<decompress_tc_kernel<SINGLE, true, false, 3>>()
                       : set.k2_bf16 ? raise_smem_limit<decompress_tc_kernel<SINGLE, true, false>>()
                       : set.k2_f32  ? raise_smem_limit<decompress_tc_kernel<SINGLE, false, true>>()
                                     : raise_smem_limit<decompress_tc_kernel<SINGLE, false, false>>()))
@@ -1346,8 +1373,11 @@ inline flora_status tc_decompress_launch(const TcSet& set, const TcMatrix& one, 
             return cudaLaunchKernelEx(&cfg, kernel, mats, one, items, end - begin, table, seed_base, r, scale, step, set.bn, set.slots, set.cstages, set.k2_gw,
                                       set.k2_nslabs);
         };
-        const cudaError_t e = set.k2_pair ? cudaLaunchKernelEx(&cfg, decompress_pair_kernel<SINGLE>, mats, one, items, end - begin, table, seed_base, r, scale, step,
-                                                               set.slots, set.cstages)
+        auto go_pair = [&](auto kernel) {
+            return cudaLaunchKernelEx(&cfg, kernel, mats, one, items, end - begin, table, seed_base, r, scale, step, set.slots, set.cstages);
+        };
+        const cudaError_t e = set.k2_pair ? (parts ? go_pair(decompress_pair_kernel<SINGLE, 3>) : go_pair(decompress_pair_kernel<SINGLE>))
+                              : parts       ? go(decompress_tc_kernel<SINGLE, true, false, 3>)
                               : set.k2_bf16 ? go(decompress_tc_kernel<SINGLE, true, false>)
                               : set.k2_f32  ? go(decompress_tc_kernel<SINGLE, false, true>)
                                             : go(decompress_tc_kernel<SINGLE, false, false>);
@@ -1373,7 +1403,7 @@ inline flora_status tc_decompress_single(flora_mat* W, const flora_mat* S, uint6
     if (!set) return rc;
     if (!set->k2_bf16) return tc_decompress_launch<true>(*set, one, &seed, step, st, launches);
     // ranks above 64: scratch for the bf16 copy of the sketch, for the duration of the call
-    const int64_t k_pad = (S->cols + 63) & ~(int64_t)63;
+    const int64_t k_pad = ((S->cols + 63) & ~(int64_t)63) * set->k2_parts;
     void* sb = nullptr;
     if (scratch_alloc(&sb, (size_t)(S->rows * k_pad * 2), st) != cudaSuccess) {
         cudaGetLastError();
@@ -1388,7 +1418,8 @@ inline flora_status tc_decompress_single(flora_mat* W, const flora_mat* S, uint6
 
 inline bool tc_decompress_supported(const flora_mat* big, const flora_mat* sketch)
 {
-    return (tc_mat_ok(*big) || (tc_f32_ok(*big) && sketch->cols <= K2_F32_MAX_R)) && tc_sketch_ok(*sketch) && encode_tiled_fn() != nullptr;
+    // (bf16 weights may have a sketch that TMA cannot address: the kernel then reads a copy of it)
+    return (tc_mat_ok(*big) || (tc_f32_ok(*big) && sketch->cols <= K2_F32_MAX_R && tc_sketch_ok(*sketch))) && encode_tiled_fn() != nullptr;
 }
 
 inline flora_status tc_set_zero(TcSet& set, cudaStream_t st, std::atomic<uint64_t>& launches)
