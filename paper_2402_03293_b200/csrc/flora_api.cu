@@ -189,13 +189,17 @@ bool small_decompress(int64_t elements, int r, bool f32, bool loose)
     if (g_force_path.load(std::memory_order_relaxed) == 2) return f32 && r > K2_F32_MAX_R;
     return gen_decompress_quicker(elements, r, f32, loose);
 }
-bool use_tc_compress(const flora_mat* big, const flora_mat* sketch)
+// A first call of a shape makes its plan, which a stream that is being recorded into a graph does not allow; with a sketch that TMA cannot
+// address the general kernels, which need none, are recorded instead.
+bool use_tc_compress(const flora_mat* big, const flora_mat* sketch, void* stream)
 {
+    if (!sketch_writable(*sketch) && capturing(as_stream(stream))) return false;
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch) &&
            !small_compress(big->rows * big->cols, big->cols, (int)sketch->cols, big->dtype == FLORA_F32, false);
 }
-bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch)
+bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch, void* stream)
 {
+    if (!tc_sketch_ok(*sketch) && capturing(as_stream(stream))) return false;
     return g_force_path.load(std::memory_order_relaxed) != 1 && tc_decompress_supported(big, sketch) &&
            !small_decompress(big->rows * big->cols, (int)sketch->cols, big->dtype == FLORA_F32, !tc_sketch_ok(*sketch));
 }
@@ -319,7 +323,7 @@ flora_status flora_compress_accumulate(const flora_mat* G, flora_mat* C, uint64_
     if (st) return st;
     if (r != C->cols) return FLORA_ERR_RANK;
     if (G->rows == 0 || G->cols == 0) return FLORA_OK;
-    if (use_tc_compress(G, C)) return tc_compress_single(G, C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
+    if (use_tc_compress(G, C, stream)) return tc_compress_single(G, C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
     if (use_gen(G)) return gen_compress_single(*G, *C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
     return simt_compress(G, C, seed, 1.0f, 1.0f, as_stream(stream));
 }
@@ -329,7 +333,7 @@ flora_status flora_momentum_step(const flora_mat* G, flora_mat* M, float beta, u
     flora_status st = check_pair(G, M);
     if (st) return st;
     if (G->rows == 0) return FLORA_OK;
-    if (G->cols > 0 && use_tc_compress(G, M)) return tc_compress_single(G, M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
+    if (G->cols > 0 && use_tc_compress(G, M, stream)) return tc_compress_single(G, M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
     if (use_gen(G)) return gen_compress_single(*G, *M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
     return simt_compress(G, M, seed, 1.0f - beta, beta, as_stream(stream));
 }
@@ -368,7 +372,7 @@ flora_status flora_momentum_step_resampled(const flora_mat* G, flora_mat* M, flo
     void* scratch = nullptr;
     st = single_transfer(M, M, G->cols, G->dtype, seed_old, seed_new, beta, 0.0f, stream, &scratch);
     if (st == FLORA_OK) {
-        if (G->cols > 0 && use_tc_compress(G, M)) st = tc_compress_single(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
+        if (G->cols > 0 && use_tc_compress(G, M, stream)) st = tc_compress_single(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
         else if (use_gen(G)) st = gen_compress_single(*G, *M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
         else st = simt_compress(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream));
     }
@@ -381,7 +385,7 @@ flora_status flora_decompress_apply(flora_mat* W, const flora_mat* C, uint64_t s
     flora_status st = check_pair(W, C);
     if (st) return st;
     if (W->rows == 0 || W->cols == 0) return FLORA_OK;
-    if (use_tc_decompress(W, C)) {
+    if (use_tc_decompress(W, C, stream)) {
         st = tc_decompress_single(W, C, seed, lr * scale, as_stream(stream), g_launches);
         if (st != FLORA_ERR_ALLOC || tc_sketch_ok(*C)) return st;      // (no room for the copy of a sketch that TMA cannot address: without one)
     }

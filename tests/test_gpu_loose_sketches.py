@@ -89,3 +89,25 @@ def test_sets(r):
     assert not torch.isfinite(W[0].float()).any()
     assert torch.isfinite(W[1].float()).all()
     fset.close()
+
+
+def test_first_calls_of_a_shape_inside_a_graph():
+    """Nothing is planned for such sketches while a stream is being recorded (and a replay reads what the buffers hold by then)."""
+    n, m, r = 4112, 4104, 75                                          # (a shape of its own: no plan of another test)
+    G, W = wl.gaussian_matrix(n, m, 1e-2, "bf16", 1).to(DEV), wl.gaussian_matrix(n, m, 4e-4, "bf16", 2).to(DEV)
+    S = torch.zeros(n, r, device=DEV)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        fb.flora_momentum_step(G, S, 0.0, 3)
+        fb.flora_compress_accumulate(G, S, 3, r)
+        fb.flora_decompress_apply(W, S, 3, 0.01, 0.5)
+    W0, G2 = W.clone(), wl.gaussian_matrix(n, m, 1e-2, "bf16", 4).to(DEV)
+    G.copy_(G2)
+    graph.replay()
+    rows = np.arange(0, n, 257)
+    want = 2.0 * oracle_compress(G2[rows].contiguous(), torch.zeros(len(rows), r), 3)
+    assert rel_err(S[rows].cpu().numpy(), want) <= TOL["f32"]
+    wref = oracle_decompress(W0[rows].contiguous(), S[rows].contiguous(), 3, 0.01, 0.5)
+    assert rel_err(values(wl.as_numpy(W[rows].contiguous())), values(wref)) <= TOL["bf16"]
+    del graph
