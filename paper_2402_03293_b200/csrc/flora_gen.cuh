@@ -40,7 +40,11 @@ __host__ __device__ constexpr int gen_threads(int workers) { return 32 * (worker
 constexpr int GEN_G_SLOTS_MAX = 8, GEN_A_SLOTS_MAX = 6;
 constexpr int GEN_L2_AHEAD = 8;                             // steps of a tile that a CTA asks into L2 before it may load them
 constexpr int GEN_F32_CHAIN_STEPS = 72;                     // steps of an fp32 matrix that a CTA adds up at most
-constexpr int GEN_MAX_SPLIT = 16;                           // CTAs that share the columns of a row group (above 8: not a portable cluster size)
+constexpr int GEN_MAX_SPLIT = 16;                           // CTAs of a cluster that share the columns of a row group (above 8: not a portable cluster size)
+// Parts that single CTAs make of a row group's columns.  A bf16 matrix of a set has up to 2^25 steps and a part's range is found as part * steps /
+// parts in 32 bits, so no more than 64 (without a limit a member of 1 x 31,765,017 got 9732 of them, a ninth over the wrong columns).
+constexpr int GEN_MAX_PARTS = 64;
+static_assert((uint64_t)GEN_MAX_PARTS << 25 < 1ull << 32 && GEN_MAX_SPLIT <= GEN_MAX_PARTS, "column ranges are found in 32 bits");
 // How the CTAs of a split bring their sums together.
 //   Ordered   through distributed shared memory: every row has one writer, which adds the peers' sums in a fixed order.  Bit-reproducible
 //             mode only: reading the peers and the two cluster barriers around that took half of a small launch.
@@ -183,7 +187,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     const int tiles = max(0, min(T, ((mat.n + 127) >> 7) - tile0));
     const int m_end = F32 ? item.col0 + min(mat.m - item.col0, GEN_F32_PASS_COLS) : mat.m;      // columns beyond it are another launch's
     const int all_steps = (m_end - item.col0 + C::K - 1) / C::K, step0 = item.col0 / C::K;
-    // (at most 2^25 steps and 16 parts: a 64-bit division takes a quarter of a microsecond)
+    // (in 32 bits, see GEN_MAX_PARTS: a 64-bit division takes a quarter of a microsecond)
     const int ks0 = step0 + (int)((uint32_t)part * (uint32_t)all_steps / (uint32_t)split), ks1 = step0 + (int)((uint32_t)(part + 1) * (uint32_t)all_steps / (uint32_t)split);
     const int steps = tiles > 0 ? ks1 - ks0 : 0;
     const bool barrier = cluster > 1 && joining == GEN_JOIN_SCALED;

@@ -510,7 +510,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         auto parts_of = [&](int i, int64_t per, int64_t pass) {
             const int64_t steps = steps_of(i, pass);
             if (s.f32) per = std::min(per, gen_f32_chain(steps_of(i, 0)));
-            return std::max<int64_t>(1, (steps + per - 1) / per);
+            return std::max<int64_t>(1, std::min<int64_t>(GEN_MAX_PARTS, (steps + per - 1) / per));
         };
         int64_t best_per = most_steps;
         double least = 1e300;
