@@ -219,33 +219,44 @@ struct flora_set {
     bool aligned_G = false;        // made of bf16 gradients that TMA can address, all of them: such a set takes no others
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
     TcSet tcf;                     // the same for fp32 matrices
+    TcSet tcl;                     // ... and for bf16 matrices whose sketch TMA cannot address
     GenSet gen_g[2], gen_w[2];     // the others, by dtype
 };
 
 // Below this many elements the matrices of a mixed set that TMA could serve are not worth a launch of their own (4 M
 // elements are 8 MB, a microsecond and a half of HBM time): all its matrices then go to the kernels of flora_gen.cuh.
 constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
-// The same for sets with sketches that TMA cannot address, which also want a scaling pass and a copy of the sketches: eleven matrices of which three
+// The same for the matrices of a set whose sketches TMA cannot address, which also want passes over the sketches: eleven matrices of which three
 // with 4.5 M elements are TMA's, r = 7, momentum step and update: 85.7 us with launches of their own, 72.9 without; twelve with 30 M, r = 37: 63 and 206.
 constexpr int64_t LOOSE_SET_TMA_MIN_ELEMENTS = 16ll << 20;
 
+// What the TMA kernels may take of a set: fp32 matrices, bf16 matrices, and (decompression only) bf16 matrices whose sketch TMA cannot address.  Each
+// kind has work lists of its own, so an odd sketch takes nothing but its own matrix to the kernel that reads three parts (24 matrices of GPT-2-small
+// shapes of which one has a sketch off 16 bytes, r = 32 / 64 / 256, update: 40.9 / 44.9 / 94.4 us with all of them there, 33.8 / 43.0 / 85.8 this way;
+// 25.7 / 30.6 / 61.1 without the odd one.  Three of 2048 x 2048 and a small one with such a sketch, r = 64: 27.9 and 18.0).
+enum class Side { F32, BF16, LOOSE };
+
 // Which matrices of one side (G: compression, or W: decompression) of a set the TMA kernels serve.
-static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression, bool f32 = false)
+static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool compression, Side side)
 {
-    std::vector<uint8_t> use = tc_eligible(big, S, f32, !f32);
-    if (compression && f32)
-        for (size_t i = 0; i < big.size(); ++i) use[i] = use[i] && big[i].cols >= K1_F32_MIN_COLS && sketch_writable(S[i]);
-    int64_t eligible = 0, widest = 0;
-    bool mixed = false, loose = false;
+    const bool f32 = side == Side::F32, loose = side == Side::LOOSE;
+    std::vector<uint8_t> use(big.size(), 0);
+    int64_t eligible = 0, widest = 0, odd = 0;           // (odd: with sketches that TMA cannot address)
+    bool mixed = false;
     for (size_t i = 0; i < big.size(); ++i) {
+        const bool kind = f32           ? tc_f32_ok(big[i]) && (compression ? big[i].cols >= K1_F32_MIN_COLS && sketch_writable(S[i]) : tc_sketch_ok(S[i]))
+                          : compression ? tc_mat_ok(big[i])
+                                        : tc_mat_ok(big[i]) && tc_sketch_ok(S[i]) != loose;
+        use[i] = encode_tiled_fn() && kind;
         if (use[i]) eligible += big[i].rows * big[i].cols;
         else mixed = mixed || big[i].rows > 0;
         widest = std::max(widest, big[i].cols);
-        loose = loose || (!f32 && !tc_sketch_ok(S[i]));
+        odd += use[i] && !f32 && !tc_sketch_ok(S[i]) ? big[i].rows * big[i].cols : 0;
     }
     const int r = S.empty() ? 1 : (int)S[0].cols;
     const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
-    if (((mixed || loose) && eligible < (loose && big.size() > 1 ? LOOSE_SET_TMA_MIN_ELEMENTS : mixed ? MIXED_SET_TMA_MIN_ELEMENTS : 0) && g_force_path.load() != 2) ||
+    const int64_t least = 2 * odd > eligible && big.size() > 1 ? LOOSE_SET_TMA_MIN_ELEMENTS : mixed ? MIXED_SET_TMA_MIN_ELEMENTS : 0;
+    if ((eligible < least && g_force_path.load() != 2) ||
         (compression ? small_compress(counted, widest, r, f32, true) : small_decompress(counted, r, f32, loose)))
         std::fill(use.begin(), use.end(), (uint8_t)0);
     return use;
@@ -253,29 +264,34 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
 
 static bool all_addressable(const std::vector<flora_mat>& G, const std::vector<flora_mat>& S)
 {
-    const std::vector<uint8_t> ok = tc_eligible(G, S);
-    return !ok.empty() && std::find(ok.begin(), ok.end(), (uint8_t)0) == ok.end();
+    if (G.empty() || !encode_tiled_fn()) return false;
+    for (size_t i = 0; i < G.size(); ++i)
+        if (!tc_mat_ok(G[i]) || !tc_sketch_ok(S[i])) return false;
+    return true;
 }
 
 // Builds the work lists of a set.  Its tables are copied from pageable memory on the legacy default stream, to which streams made
 // with the non-blocking flag are not ordered: set_ready puts every stream behind the copies.
 static flora_status set_build(flora_set* s)
 {
-    std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true);
-    const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, true), use_wf = set_tma_side(s->W, s->S, false, true);
-    std::vector<uint8_t> use_w = set_tma_side(s->W, s->S, false);
+    const std::vector<flora_mat> none;
     auto any = [](const std::vector<uint8_t>& use) { return std::find(use.begin(), use.end(), (uint8_t)1) != use.end(); };
+    std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true, Side::BF16), use_w = set_tma_side(s->W, s->S, false, Side::BF16);
     flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
-    if (st == FLORA_ERR_ALLOC && !s->S.empty() && !tc_sketch_ok(s->S[0]) && any(use_w)) {
-        // no room for the copy of sketches that TMA cannot address: the kernels that need none take the weights
-        tc_set_free(s->tc);
-        std::fill(use_w.begin(), use_w.end(), (uint8_t)0);
-        st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
+    for (const Side side : {Side::F32, Side::LOOSE}) {
+        TcSet& tc = side == Side::F32 ? s->tcf : s->tcl;
+        const std::vector<uint8_t> g = side == Side::F32 ? set_tma_side(s->G, s->S, true, side) : std::vector<uint8_t>(s->G.size(), 0);
+        std::vector<uint8_t> w = set_tma_side(s->W, s->S, false, side);
+        if (st == FLORA_OK && (any(g) || any(w))) st = tc_set_build_on(tc, any(g) ? s->G : none, any(w) ? s->W : none, s->S, nullptr, g, w);
+        if (st == FLORA_ERR_ALLOC && side == Side::LOOSE && any(w)) {
+            // no room for the copy of these sketches: the kernels that need none take the weights
+            tc_set_free(tc);
+            std::fill(w.begin(), w.end(), (uint8_t)0);
+            st = any(g) ? tc_set_build_on(tc, s->G, none, s->S, nullptr, g, w) : FLORA_OK;
+        }
+        for (size_t i = 0; i < g.size(); ++i) use_g[i] |= g[i];
+        for (size_t i = 0; i < w.size(); ++i) use_w[i] |= w[i];
     }
-    if (st == FLORA_OK && (any(use_f) || any(use_wf)))
-        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : std::vector<flora_mat>(), any(use_wf) ? s->W : std::vector<flora_mat>(), s->S, nullptr, use_f, use_wf);
-    for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
-    for (size_t i = 0; i < use_w.size(); ++i) use_w[i] |= use_wf[i];
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
         std::vector<int> g, w;
         for (size_t i = 0; i < s->S.size(); ++i) {
@@ -285,7 +301,7 @@ static flora_status set_build(flora_set* s)
         st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g, nullptr);
         if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w, nullptr);
     }
-    if (s->tc.d_mats || s->tcf.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats)
+    if (s->tc.d_mats || s->tcf.d_mats || s->tcl.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats)
         if (cudaEventCreateWithFlags(&s->copied, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(s->copied, nullptr) != cudaSuccess) {
             cudaGetLastError();
             if (st == FLORA_OK) st = FLORA_ERR_CUDA;
@@ -488,6 +504,7 @@ flora_status flora_set_destroy(flora_set* set)
     if (!set) return FLORA_OK;
     tc_set_free(set->tc);
     tc_set_free(set->tcf);
+    tc_set_free(set->tcl);
     for (int d = 0; d < 2; ++d) {
         gen_set_free(set->gen_g[d]);
         gen_set_free(set->gen_w[d]);
@@ -513,20 +530,23 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
     // a later call brings addresses that it can: those launches carry the matrix by value, so nothing is allocated, planned or waited
     // for here.
     if (set->aligned_G && !all_addressable(newG, set->S)) return FLORA_ERR_ALIGN;
-    const bool tc_ok = tc_set_addressable(set->tc, newG), tcf_ok = tc_set_addressable(set->tcf, newG);
+    TcSet* const kinds[] = {&set->tc, &set->tcf, &set->tcl};
+    bool addressable[3];
+    std::vector<CUtensorMap> maps[3];
     // launches that a graph holds read the gradients through the set's tables, with the kernels of the time they were recorded at
-    if ((!tc_ok && set->tc.captured) || (!tcf_ok && set->tcf.captured) || !gen_set_rebindable(set->gen_g[0], newG) || !gen_set_rebindable(set->gen_g[1], newG))
-        return FLORA_ERR_ALIGN;
-    std::vector<CUtensorMap> maps, maps_f;
-    if ((tc_ok && !tc_set_make_maps(set->tc, newG, maps)) || (tcf_ok && !tc_set_make_maps(set->tcf, newG, maps_f))) return FLORA_ERR_CUDA;
+    for (int k = 0; k < 3; ++k) {
+        addressable[k] = tc_set_addressable(*kinds[k], newG);
+        if (!addressable[k] && kinds[k]->captured) return FLORA_ERR_ALIGN;
+    }
+    if (!gen_set_rebindable(set->gen_g[0], newG) || !gen_set_rebindable(set->gen_g[1], newG)) return FLORA_ERR_ALIGN;
+    for (int k = 0; k < 3; ++k)
+        if (addressable[k] && !tc_set_make_maps(*kinds[k], newG, maps[k])) return FLORA_ERR_CUDA;
     flora_status st = set_ready(set, as_stream(stream));
-    if (st) return st;
-    st = tc_ok ? tc_set_rebind(set->tc, maps, as_stream(stream)) : FLORA_OK;
-    if (st == FLORA_OK && tcf_ok) st = tc_set_rebind(set->tcf, maps_f, as_stream(stream));
+    for (int k = 0; k < 3 && st == FLORA_OK; ++k)
+        if (addressable[k]) st = tc_set_rebind(*kinds[k], maps[k], as_stream(stream));
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_rebind(set->gen_g[d], newG, as_stream(stream));
     if (st) return st;
-    set->tc.off_tma = !tc_ok;
-    set->tcf.off_tma = !tcf_ok;
+    for (int k = 0; k < 3; ++k) kinds[k]->off_tma = !addressable[k];
     set->G.swap(newG);
     return FLORA_OK;
 }
@@ -556,6 +576,7 @@ static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a,
     if (!simt) {
         flora_status st = tma_compress(set, set->tc, seeds, a, b, as_stream(stream), behind_own_transfer);
         if (st == FLORA_OK) st = tma_compress(set, set->tcf, seeds, a, b, as_stream(stream), false);
+        if (st == FLORA_OK) st = tma_compress(set, set->tcl, seeds, a, b, as_stream(stream), false);
         for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_compress(set->gen_g[d], seeds, a, b, as_stream(stream), g_launches);
         if (st) return st;
     }
@@ -585,8 +606,8 @@ flora_status flora_set_decompress_apply(flora_set* set, const uint64_t* seeds, f
     const bool simt = g_force_path.load() == 1;
     if (!simt) {
         flora_status st = FLORA_OK;
-        if (set->tc.decompress_ready) st = tc_set_decompress(set->tc, seeds, lr * scale, as_stream(stream), g_launches);
-        if (st == FLORA_OK && set->tcf.decompress_ready) st = tc_set_decompress(set->tcf, seeds, lr * scale, as_stream(stream), g_launches);
+        for (const TcSet* tc : {&set->tc, &set->tcf, &set->tcl})
+            if (st == FLORA_OK && tc->decompress_ready) st = tc_set_decompress(*tc, seeds, lr * scale, as_stream(stream), g_launches);
         for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_decompress(set->gen_w[d], seeds, lr * scale, as_stream(stream), g_launches);
         if (st) return st;
     }

@@ -905,16 +905,6 @@ inline flora_status tc_fill_matrices(TcSet& set, const std::vector<flora_mat>& G
     return FLORA_OK;
 }
 
-// What the TMA kernels can take of a set: the matrix has their type, size and alignment, and its sketch's rows can be addressed
-// (any_sketch: or not).
-inline std::vector<uint8_t> tc_eligible(const std::vector<flora_mat>& big, const std::vector<flora_mat>& S, bool f32 = false, bool any_sketch = false)
-{
-    std::vector<uint8_t> ok(big.size(), 0);
-    if (encode_tiled_fn())
-        for (size_t i = 0; i < big.size(); ++i) ok[i] = (f32 ? tc_f32_ok(big[i]) : tc_mat_ok(big[i])) && (any_sketch || tc_sketch_ok(S[i]));
-    return ok;
-}
-
 // Builds the tensor-core side of a set for the matrices marked in use_g (compression) and use_w (decompression); the planners
 // see the others as empty.  The descriptors of the sketches are made for every matrix whose sketch TMA can address.
 inline flora_status tc_set_build_on(TcSet& set, const std::vector<flora_mat>& G_all, const std::vector<flora_mat>& W_all,

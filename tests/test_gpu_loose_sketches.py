@@ -111,3 +111,48 @@ def test_first_calls_of_a_shape_inside_a_graph():
     wref = oracle_decompress(W0[rows].contiguous(), S[rows].contiguous(), 3, 0.01, 0.5)
     assert rel_err(values(wl.as_numpy(W[rows].contiguous())), values(wref)) <= TOL["bf16"]
     del graph
+
+
+@pytest.mark.parametrize("path", [0, 2])
+def test_one_odd_sketch_among_others(path):
+    """It takes its own matrix to other kernels, and only that one: the others' results are those of a set without it, bit for bit."""
+    fb.flora_debug_force_path(path)
+    r, shapes = 64, [(2048, 1024), (1000, 2048), (2048, 1024), (512, 2048)]
+    G = [wl.gaussian_matrix(n, m, 1e-2, "bf16", 80 + i).to(DEV) for i, (n, m) in enumerate(shapes)]
+    W0 = [wl.gaussian_matrix(n, m, 4e-4, "bf16", 90 + i).to(DEV) for i, (n, m) in enumerate(shapes)]
+    results = []
+    for odd in (0, 1):
+        W = [w.clone() for w in W0]
+        S = [_sketch(n, r, odd if i == 0 else 0, 0, 100 + i)[1] for i, (n, _) in enumerate(shapes)]
+        fset = fb.FloraSet(G[1:], W[1:], S[1:]) if odd == 0 else fb.FloraSet(G, W, S)
+        seeds = [110 + i for i in range(1 - odd, len(shapes))]
+        fset.decompress_apply(seeds, 0.03, 1.0)
+        if odd:
+            _weights_match(W[0], W0[0], S[0], 110, 0.03)
+        want = [oracle_compress(G[i], S[i], 110 + i) for i in range(len(shapes))]
+        fset.compress_accumulate(seeds)
+        for i in range(1 - odd, len(shapes)):
+            assert rel_err(S[i].cpu().numpy(), want[i]) <= TOL["f32"], i
+        fset.close()
+        results.append(W[1:])
+    assert all(torch.equal(x, y) for x, y in zip(*results))
+
+
+def test_no_memory_for_the_copy_of_the_sketches():
+    """A set is made all the same, whichever of its sketches wants the copy (1.6 GB here)."""
+    n, m = 1 << 22, 64
+    W = [torch.zeros(128, m, dtype=torch.bfloat16, device=DEV), torch.zeros(n, m, dtype=torch.bfloat16, device=DEV)]
+    S = [torch.ones(128, 4, device=DEV)[:, :1], torch.ones(n, 1, device=DEV)]
+    torch.cuda.empty_cache()
+    rest = torch.empty(max(0, torch.cuda.mem_get_info()[0] - (1 << 30)), dtype=torch.uint8, device=DEV)
+    try:
+        fset = fb.FloraSet(None, W, S)
+    finally:
+        del rest
+        torch.cuda.empty_cache()
+    fset.decompress_apply([3, 4], 0.5, 1.0)
+    fset.close()
+    for i in range(2):
+        A = torch.empty(1, m, device=DEV)
+        fb.flora_materialize_A(A, 3 + i)
+        assert torch.equal(W[i], (-0.5 * A.bfloat16().float()).bfloat16().expand_as(W[i]))
