@@ -21,6 +21,7 @@
 #include "flora_pool.cuh"
 #include "flora_tc_host.cuh"
 #include "flora_gen_host.cuh"
+#include "flora_fold.cuh"
 #include "flora_gram.cuh"
 
 using namespace flora;
@@ -204,6 +205,30 @@ bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch, void* stre
            !small_decompress(big->rows * big->cols, (int)sketch->cols, big->dtype == FLORA_F32, !tc_sketch_ok(*sketch));
 }
 
+// S <- b S + a G A^T.  TMA's kernels where they take the matrix; with a sketch that TMA cannot address they make the sums in scratch, which are then blended in
+// (flora_fold.cuh), or, where there is no memory for it, the general kernels take the call.
+flora_status compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, float a, float b, void* stream)
+{
+    const cudaStream_t st = as_stream(stream);
+    const int r = (int)S->cols;
+    if (G->cols > 0 && use_tc_compress(G, S, stream)) {
+        if (sketch_writable(*S)) return tc_compress_single(G, S, seed, a, b, st, g_launches);
+        flora_mat sums{nullptr, S->rows, S->cols, fold_ld(r), FLORA_F32};
+        if (scratch_alloc(&sums.data, sizeof(float) * (size_t)(sums.rows * sums.ld), st) == cudaSuccess) {
+            // (sums as short as those of the general kernels: the tensor core truncates them, 7e-8 of a sum lost per step of 64 columns)
+            const int64_t steps = (G->cols + 63) / 64, parts = gen_k1_choose(false, r, (G->rows + 127) / 128, steps, true, false).cluster;
+            flora_status rc = tc_compress_single(G, &sums, seed, 1.0f, 0.0f, st, g_launches, (steps + parts - 1) / parts);
+            const FoldMat fold{(float*)S->data, (const float*)sums.data, S->ld, (int32_t)S->rows, (int32_t)sums.ld, 1, 0};
+            if (rc == FLORA_OK) rc = fold_single(fold, r, a, b, sm_count(), st, g_launches);
+            if (cudaFreeAsync(sums.data, st) != cudaSuccess && rc == FLORA_OK) rc = FLORA_ERR_CUDA;
+            return rc;
+        }
+        cudaGetLastError();
+    }
+    if (use_gen(G)) return gen_compress_single(*G, *S, seed, a, b, st, g_launches);
+    return simt_compress(G, S, seed, a, b, st);
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------------------------------------
@@ -219,7 +244,15 @@ struct flora_set {
     bool aligned_G = false;        // made of bf16 gradients that TMA can address, all of them: such a set takes no others
     TcSet tc;                      // work lists and descriptors of the TMA kernels, for the matrices they serve
     TcSet tcf;                     // the same for fp32 matrices
-    TcSet tcl;                     // ... and for bf16 matrices whose sketch TMA cannot address
+    TcSet tcl;                     // ... decompression of bf16 matrices whose sketch TMA cannot address
+    // Compression of a set that has such sketches: the lists of all its bf16 matrices, with scratch in the place of those sketches (flora_fold.cuh)
+    TcSet tcg;
+    float* d_sums = nullptr;
+    FoldItem* d_fold = nullptr;
+    int fold_items = 0;
+    int* d_beside = nullptr;       // their indexes
+    int beside = 0;
+    int64_t beside_most = 0;       // floats of the largest
     GenSet gen_g[2], gen_w[2];     // the others, by dtype
 };
 
@@ -230,8 +263,8 @@ constexpr int64_t MIXED_SET_TMA_MIN_ELEMENTS = 4ll << 20;
 // with 4.5 M elements are TMA's, r = 7, momentum step and update: 85.7 us with launches of their own, 72.9 without; twelve with 30 M, r = 37: 63 and 206.
 constexpr int64_t LOOSE_SET_TMA_MIN_ELEMENTS = 16ll << 20;
 
-// What the TMA kernels may take of a set: fp32 matrices, bf16 matrices, and (decompression only) bf16 matrices whose sketch TMA cannot address.  Each
-// kind has work lists of its own, so an odd sketch takes nothing but its own matrix to the kernel that reads three parts (24 matrices of GPT-2-small
+// What the TMA kernels may take of a set: fp32 matrices, bf16 matrices, and bf16 matrices whose sketch TMA cannot address (compression: the others, too).
+// In the decompression each kind has work lists of its own, so an odd sketch takes nothing but its own matrix to the kernel that reads three parts (24 matrices of GPT-2-small
 // shapes of which one has a sketch off 16 bytes, r = 32 / 64 / 256, update: 40.9 / 44.9 / 94.4 us with all of them there, 33.8 / 43.0 / 85.8 this way;
 // 25.7 / 30.6 / 61.1 without the odd one.  Three of 2048 x 2048 and a small one with such a sketch, r = 64: 27.9 and 18.0).
 enum class Side { F32, BF16, LOOSE };
@@ -245,13 +278,13 @@ static std::vector<uint8_t> set_tma_side(const std::vector<flora_mat>& big, cons
     bool mixed = false;
     for (size_t i = 0; i < big.size(); ++i) {
         const bool kind = f32           ? tc_f32_ok(big[i]) && (compression ? big[i].cols >= K1_F32_MIN_COLS && sketch_writable(S[i]) : tc_sketch_ok(S[i]))
-                          : compression ? tc_mat_ok(big[i])
+                          : compression ? tc_mat_ok(big[i]) && (loose || sketch_writable(S[i]))
                                         : tc_mat_ok(big[i]) && tc_sketch_ok(S[i]) != loose;
         use[i] = encode_tiled_fn() && kind;
         if (use[i]) eligible += big[i].rows * big[i].cols;
         else mixed = mixed || big[i].rows > 0;
         widest = std::max(widest, big[i].cols);
-        odd += use[i] && !f32 && !tc_sketch_ok(S[i]) ? big[i].rows * big[i].cols : 0;
+        odd += use[i] && !(compression ? sketch_writable(S[i]) : tc_sketch_ok(S[i])) ? big[i].rows * big[i].cols : 0;
     }
     const int r = S.empty() ? 1 : (int)S[0].cols;
     const int64_t counted = big.size() > 1 ? eligible * 5 / 3 : eligible;
@@ -270,28 +303,76 @@ static bool all_addressable(const std::vector<flora_mat>& G, const std::vector<f
     return true;
 }
 
+// The lists of a compression with sketches that TMA cannot address, where it has such matrices and there is memory for their sums; otherwise
+// s->beside stays 0.
+static flora_status set_build_beside(flora_set* s, const std::vector<uint8_t>& use)
+{
+    const int ld = fold_ld(s->r);
+    std::vector<int> ids;
+    int64_t rows = 0;
+    for (size_t i = 0; i < use.size(); ++i)
+        if (use[i] && !sketch_writable(s->S[i])) {
+            ids.push_back((int)i);
+            rows += s->S[i].rows;
+        }
+    if (ids.empty()) return FLORA_OK;
+    if (cudaMalloc((void**)&s->d_sums, sizeof(float) * (size_t)rows * ld) != cudaSuccess) {
+        cudaGetLastError();
+        s->d_sums = nullptr;
+        return FLORA_OK;
+    }
+    std::vector<flora_mat> S = s->S;
+    std::vector<FoldItem> fold;
+    float* D = s->d_sums;
+    for (int i : ids) {
+        flora_mat& m = S[(size_t)i];
+        fold_cut(fold, FoldMat{(float*)m.data, D, m.ld, (int32_t)m.rows, ld, 1, 0}, m.rows, fold_rows(rows, s->r, sm_count()));
+        m.data = D;
+        m.ld = ld;
+        D += m.rows * ld;
+        s->beside_most = std::max(s->beside_most, m.rows * m.cols);
+    }
+    // (sums as short as the general kernels', which are cut where they exceed half of an SM's share of the set; see compress_single.  Eight blocks of GPT-2
+    // shapes of width 1192 at r = 101: sketch off by 5.2e-6 with whole rows of 4768 columns, 2.5e-6 with halves)
+    int64_t work = 0;
+    for (size_t i = 0; i < use.size(); ++i)
+        if (use[i]) work += (s->G[i].rows + 127) / 128 * ((s->G[i].cols + 63) / 64);
+    s->tcg.max_chain = std::max<int64_t>(8, work / (2 * sm_count()));
+    s->beside = (int)ids.size();
+    flora_status st = tc_set_build_on(s->tcg, s->G, std::vector<flora_mat>(), S, nullptr, use, std::vector<uint8_t>(use.size(), 0));
+    s->fold_items = (int)fold.size();
+    if (st == FLORA_OK) st = upload(&s->d_fold, fold, nullptr);
+    return st ? st : upload(&s->d_beside, ids, nullptr);
+}
+
 // Builds the work lists of a set.  Its tables are copied from pageable memory on the legacy default stream, to which streams made
 // with the non-blocking flag are not ordered: set_ready puts every stream behind the copies.
 static flora_status set_build(flora_set* s)
 {
     const std::vector<flora_mat> none;
     auto any = [](const std::vector<uint8_t>& use) { return std::find(use.begin(), use.end(), (uint8_t)1) != use.end(); };
-    std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true, Side::BF16), use_w = set_tma_side(s->W, s->S, false, Side::BF16);
-    flora_status st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
-    for (const Side side : {Side::F32, Side::LOOSE}) {
-        TcSet& tc = side == Side::F32 ? s->tcf : s->tcl;
-        const std::vector<uint8_t> g = side == Side::F32 ? set_tma_side(s->G, s->S, true, side) : std::vector<uint8_t>(s->G.size(), 0);
-        std::vector<uint8_t> w = set_tma_side(s->W, s->S, false, side);
-        if (st == FLORA_OK && (any(g) || any(w))) st = tc_set_build_on(tc, any(g) ? s->G : none, any(w) ? s->W : none, s->S, nullptr, g, w);
-        if (st == FLORA_ERR_ALLOC && side == Side::LOOSE && any(w)) {
-            // no room for the copy of these sketches: the kernels that need none take the weights
-            tc_set_free(tc);
-            std::fill(w.begin(), w.end(), (uint8_t)0);
-            st = any(g) ? tc_set_build_on(tc, s->G, none, s->S, nullptr, g, w) : FLORA_OK;
-        }
-        for (size_t i = 0; i < g.size(); ++i) use_g[i] |= g[i];
-        for (size_t i = 0; i < w.size(); ++i) use_w[i] |= w[i];
+    std::vector<uint8_t> use_g = set_tma_side(s->G, s->S, true, Side::LOOSE), use_w = set_tma_side(s->W, s->S, false, Side::BF16);
+    flora_status st = set_build_beside(s, use_g);
+    if (!s->beside) {
+        use_g = set_tma_side(s->G, s->S, true, Side::BF16);
+        if (st == FLORA_OK) st = tc_set_build_on(s->tc, s->G, s->W, s->S, nullptr, use_g, use_w);
+    } else if (st == FLORA_OK) {
+        st = tc_set_build_on(s->tc, none, s->W, s->S, nullptr, use_g, use_w);
     }
+    const std::vector<uint8_t> use_f = set_tma_side(s->G, s->S, true, Side::F32), use_wf = set_tma_side(s->W, s->S, false, Side::F32);
+    if (st == FLORA_OK && (any(use_f) || any(use_wf)))
+        st = tc_set_build_on(s->tcf, any(use_f) ? s->G : none, any(use_wf) ? s->W : none, s->S, nullptr, use_f, use_wf);
+    std::vector<uint8_t> use_wl = set_tma_side(s->W, s->S, false, Side::LOOSE);
+    if (st == FLORA_OK && any(use_wl)) {
+        st = tc_set_build_on(s->tcl, none, s->W, s->S, nullptr, use_g, use_wl);
+        if (st == FLORA_ERR_ALLOC) {                   // no room for the copy of these sketches: the kernels that need none take the weights
+            tc_set_free(s->tcl);
+            std::fill(use_wl.begin(), use_wl.end(), (uint8_t)0);
+            st = FLORA_OK;
+        }
+    }
+    for (size_t i = 0; i < use_g.size(); ++i) use_g[i] |= use_f[i];
+    for (size_t i = 0; i < use_w.size(); ++i) use_w[i] |= use_wf[i] | use_wl[i];
     for (int d = 0; d < 2 && st == FLORA_OK; ++d) {
         std::vector<int> g, w;
         for (size_t i = 0; i < s->S.size(); ++i) {
@@ -301,7 +382,7 @@ static flora_status set_build(flora_set* s)
         st = gen_set_build(s->gen_g[d], 0, s->G, s->S, g, nullptr);
         if (st == FLORA_OK) st = gen_set_build(s->gen_w[d], 1, s->W, s->S, w, nullptr);
     }
-    if (s->tc.d_mats || s->tcf.d_mats || s->tcl.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats)
+    if (s->tc.d_mats || s->tcf.d_mats || s->tcl.d_mats || s->tcg.d_mats || s->gen_g[0].d_mats || s->gen_g[1].d_mats || s->gen_w[0].d_mats || s->gen_w[1].d_mats)
         if (cudaEventCreateWithFlags(&s->copied, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(s->copied, nullptr) != cudaSuccess) {
             cudaGetLastError();
             if (st == FLORA_OK) st = FLORA_ERR_CUDA;
@@ -339,9 +420,7 @@ flora_status flora_compress_accumulate(const flora_mat* G, flora_mat* C, uint64_
     if (st) return st;
     if (r != C->cols) return FLORA_ERR_RANK;
     if (G->rows == 0 || G->cols == 0) return FLORA_OK;
-    if (use_tc_compress(G, C, stream)) return tc_compress_single(G, C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
-    if (use_gen(G)) return gen_compress_single(*G, *C, seed, 1.0f, 1.0f, as_stream(stream), g_launches);
-    return simt_compress(G, C, seed, 1.0f, 1.0f, as_stream(stream));
+    return compress_single(G, C, seed, 1.0f, 1.0f, stream);
 }
 
 flora_status flora_momentum_step(const flora_mat* G, flora_mat* M, float beta, uint64_t seed, void* stream)
@@ -349,9 +428,7 @@ flora_status flora_momentum_step(const flora_mat* G, flora_mat* M, float beta, u
     flora_status st = check_pair(G, M);
     if (st) return st;
     if (G->rows == 0) return FLORA_OK;
-    if (G->cols > 0 && use_tc_compress(G, M, stream)) return tc_compress_single(G, M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
-    if (use_gen(G)) return gen_compress_single(*G, *M, seed, 1.0f - beta, beta, as_stream(stream), g_launches);
-    return simt_compress(G, M, seed, 1.0f - beta, beta, as_stream(stream));
+    return compress_single(G, M, seed, 1.0f - beta, beta, stream);
 }
 
 // dst <- b dst + a src (A_old A_new^T); release_later: see transfer_tc.
@@ -388,9 +465,7 @@ flora_status flora_momentum_step_resampled(const flora_mat* G, flora_mat* M, flo
     void* scratch = nullptr;
     st = single_transfer(M, M, G->cols, G->dtype, seed_old, seed_new, beta, 0.0f, stream, &scratch);
     if (st == FLORA_OK) {
-        if (G->cols > 0 && use_tc_compress(G, M, stream)) st = tc_compress_single(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
-        else if (use_gen(G)) st = gen_compress_single(*G, *M, seed_new, 1.0f - beta, 1.0f, as_stream(stream), g_launches);
-        else st = simt_compress(G, M, seed_new, 1.0f - beta, 1.0f, as_stream(stream));
+        st = compress_single(G, M, seed_new, 1.0f - beta, 1.0f, stream);
     }
     if (scratch && cudaFreeAsync(scratch, as_stream(stream)) != cudaSuccess && st == FLORA_OK) st = FLORA_ERR_CUDA;
     return st;
@@ -505,6 +580,10 @@ flora_status flora_set_destroy(flora_set* set)
     tc_set_free(set->tc);
     tc_set_free(set->tcf);
     tc_set_free(set->tcl);
+    tc_set_free(set->tcg);
+    if (set->d_sums) cudaFree(set->d_sums);
+    if (set->d_fold) cudaFree(set->d_fold);
+    if (set->d_beside) cudaFree(set->d_beside);
     for (int d = 0; d < 2; ++d) {
         gen_set_free(set->gen_g[d]);
         gen_set_free(set->gen_w[d]);
@@ -530,7 +609,7 @@ flora_status flora_set_rebind_gradients(flora_set* set, const flora_mat* G, void
     // a later call brings addresses that it can: those launches carry the matrix by value, so nothing is allocated, planned or waited
     // for here.
     if (set->aligned_G && !all_addressable(newG, set->S)) return FLORA_ERR_ALIGN;
-    TcSet* const kinds[] = {&set->tc, &set->tcf, &set->tcl};
+    TcSet* const kinds[] = {&set->tc, &set->tcf, &set->tcg};
     bool addressable[3];
     std::vector<CUtensorMap> maps[3];
     // launches that a graph holds read the gradients through the set's tables, with the kernels of the time they were recorded at
@@ -565,6 +644,19 @@ static flora_status tma_compress(const flora_set* set, TcSet& tc, const uint64_t
     return rc;
 }
 
+// The bf16 matrices of a set that has sketches which TMA cannot address: their sums are made in scratch, b = 0 where there are no others, beside them from
+// zeros, and blended in.
+static flora_status beside_compress(flora_set* set, const uint64_t* seeds, float a, float b, cudaStream_t st, bool behind_own_transfer)
+{
+    TcSet& tc = set->tcg;
+    if (!tc.compress_ready || tc.off_tma) return tma_compress(set, tc, seeds, a, b, st, false);
+    const bool alone = (size_t)set->beside == tc.members.size();
+    flora_status rc = FLORA_OK;
+    if (!alone && b != 0.0f) rc = tc_scale_launch<false>(tc.d_mats, TcMatrix{}, set->d_beside, (size_t)set->beside, set->beside_most, set->r, 0.0f, true, st, g_launches);
+    if (rc == FLORA_OK) rc = tc_set_compress(tc, seeds, a, alone ? 0.0f : b, st, g_launches, behind_own_transfer);
+    return rc ? rc : fold_launch(false, set->d_fold, set->fold_items, FoldMat{}, 0, 0, set->r, 1.0f, b, sm_count(), st, g_launches);
+}
+
 // behind_own_transfer: the work before this call on the stream is the library's own transfer, which does not touch G and whose first
 // operation waited for all earlier work (transfer_tc's `ordered`)
 static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a, float b, void* stream, bool behind_own_transfer = false)
@@ -576,7 +668,7 @@ static flora_status set_compress(flora_set* set, const uint64_t* seeds, float a,
     if (!simt) {
         flora_status st = tma_compress(set, set->tc, seeds, a, b, as_stream(stream), behind_own_transfer);
         if (st == FLORA_OK) st = tma_compress(set, set->tcf, seeds, a, b, as_stream(stream), false);
-        if (st == FLORA_OK) st = tma_compress(set, set->tcl, seeds, a, b, as_stream(stream), false);
+        if (st == FLORA_OK) st = beside_compress(set, seeds, a, b, as_stream(stream), behind_own_transfer);
         for (int d = 0; d < 2 && st == FLORA_OK; ++d) st = gen_set_compress(set->gen_g[d], seeds, a, b, as_stream(stream), g_launches);
         if (st) return st;
     }

@@ -49,7 +49,7 @@ struct PairSmem {
 // A CTA of rank q in its cluster belongs to pair q / 2 and holds half h = q % 2 of every A tile: rows
 // [h N/2, (h+1) N/2).  Of that half it generates the rows [pair * N/S, (pair+1) * N/S) and receives the rest from
 // the CTAs of the same parity.  The even CTA of a pair (the leader) issues the MMAs for both.
-template <bool SINGLE, int MAPS, bool LOOSE = false>
+template <bool SINGLE, int MAPS>
 __global__ void __launch_bounds__(PAIR_MAX_THREADS, 1)
 compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const int* __restrict__ slot_begin,
                      const __grid_constant__ SeedTable seeds, int seed_base, int r, int N, float scale, float a, float b, int gstages,
@@ -374,7 +374,7 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                     waited = true;
                 }
                 const bool add = item.direct == 0 || b == 1.0f;
-                const bool loose = LOOSE && mat->loose != 0, rmw = !add && b != 0.0f;
+                const bool rmw = !add && b != 0.0f;
                 for (int i = grp; i < item.tiles * nchunks && eok && !*abort; i += PAIR_EPI_WARPS / 4) {
                     const int t = i / nchunks, c = i - t * nchunks;
                     const int row0 = item.row0 + t * 128 + quarter * 32, row = row0 + lane;
@@ -424,12 +424,6 @@ compress_pair_kernel(const TcMatrix* __restrict__ table, const __grid_constant__
                             }
                             ptx::st_shared_v4(addr, __float_as_uint(x0), __float_as_uint(x1), __float_as_uint(x2), __float_as_uint(x3));
                         }
-                    }
-                    if (loose) {
-                        __syncwarp();
-                        write_piece(buf, mat->S, mat->lds, mat->n, r, row0, c * 32, lane, add);
-                        __syncwarp();                                 // the next piece goes into the same buffer
-                        continue;
                     }
                     ptx::fence_proxy_async_smem();
                     __syncwarp();

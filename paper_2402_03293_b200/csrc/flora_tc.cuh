@@ -55,8 +55,7 @@ struct alignas(128) TcMatrix {
     float* S;            // sketch, n x r fp32
     int64_t lds;
     int32_t n, m;
-    int32_t loose;       // TMA cannot address the rows of S (no map_s, map_sq): the compression writes them with plain accesses
-    int32_t pad[23];
+    int32_t pad[24];
 };
 static_assert(sizeof(TcMatrix) % 128 == 0, "matrix records hold TMA descriptors");
 
@@ -106,25 +105,6 @@ struct GMaps<0> {
 // set; a third of that costs 0.3.  (Host time of a launch without maps, with 48, with 192: 3.2, 3.4, 4.6 us; the GPU's is the same.)
 constexpr int GMAPS_FEW = 64, GMAPS_MANY = 192;
 
-// Writes 32 rows x 32 columns of accumulators, staged in shared memory as a sketch's tensor map would have them (128-byte rows,
-// swizzled), into a sketch that TMA cannot address: ranks that are no multiple of four, or bases off 16 bytes.  One warp; its lanes
-// take the columns of a row, or of two or four rows where there are few, and add to them or store them.  (A sketch that is to be
-// blended has been scaled before: reading the old values here took a momentum step of 96 matrices at r = 255 from 502 to 746 us.)
-__device__ __forceinline__ void write_piece(uint32_t buf, float* S, int64_t lds, int n, int r, int row0, int col0, int lane, bool add)
-{
-    const int cols = min(32, r - col0), rows = min(32, n - row0);
-    const int shift = cols > 16 ? 5 : cols > 8 ? 4 : 3, j = lane & ((1 << shift) - 1), step = 32 >> shift;
-    float* p = S + (int64_t)(row0 + (lane >> shift)) * lds + col0 + j;
-#pragma unroll 4
-    for (int i = lane >> shift; i < rows; i += step, p += step * lds) {
-        if (j >= cols) continue;
-        float v;
-        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(buf + (uint32_t)(i * 128 + ((((j >> 2) ^ (i & 7)) << 4) | ((j & 3) << 2)))));
-        if (add) ptx::red_add(p, v);
-        else *p = v;
-    }
-}
-
 constexpr int SEEDS_PER_LAUNCH = 448;
 struct SeedTable {
     uint64_t s[SEEDS_PER_LAUNCH];
@@ -170,8 +150,7 @@ struct K1Smem {                            // barriers and scalars, placed after
 // new_maps: those in the table may have been written since the kernel before.
 // (80 registers: two CTAs of eight generator warps then fit an SM; with 88 the second one does not, and r = 8 on one
 // 4096 x 11008 matrix takes 27 us instead of 20)
-// LOOSE: a sketch may be one that TMA cannot address (a template parameter: tested at run time it cost the others 1 to 2 %).
-template <bool SINGLE, bool F32, int MAPS, bool LOOSE = false>
+template <bool SINGLE, bool F32, int MAPS>
 __global__ void __maxnreg__(80)
 compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ TcMatrix single, const __grid_constant__ GMaps<MAPS> gmaps, const K1Item* __restrict__ items, const __grid_constant__ SeedTable seeds,
                    int seed_base, int r, float scale, float a, float b, int T, int gstages, int astages, int lstages, int nsets, int S, int GW, int P,
@@ -500,7 +479,7 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
             ptx::tc_fence_after_sync();
             if (late_wait) ptx::grid_dependency_wait();
             const bool add = item.direct == 0 || b == 1.0f;
-            const bool loose = LOOSE && mat->loose != 0, rmw = !add && b != 0.0f;
+            const bool rmw = !add && b != 0.0f;
             const int nchunks = (r + 31) >> 5;
             const int total = item.tiles * nchunks;               // chunks of this CTA; the group takes grp, grp + EG, ...
             const int NB = min(areas / EG, 4);                    // buffers of this group
@@ -579,12 +558,6 @@ compress_tc_kernel(const TcMatrix* __restrict__ table, const __grid_constant__ T
                         x3 = fmaf(b, __uint_as_float(o3), x3);
                     }
                     ptx::st_shared_v4(addr, __float_as_uint(x0), __float_as_uint(x1), __float_as_uint(x2), __float_as_uint(x3));
-                }
-                if (loose) {                                          // every warp writes out the rows that it staged
-                    __syncwarp();
-                    write_piece(buffer(u) + (uint32_t)(quarter * 32) * 128u, mat->S, mat->lds, mat->n, r, item.row0 + t * 128 + quarter * 32, c * 32, lane,
-                                add);
-                    continue;
                 }
                 ptx::fence_proxy_async_smem();
                 ptx::named_barrier_sync(bar_b, 128);
@@ -1113,11 +1086,12 @@ __global__ void scale_sketches_kernel(const TcMatrix* __restrict__ mats, const _
         }
         for (int64_t t = (total & ~(int64_t)3) + tid; t < total; t += nthreads) S[t] = (b == 0.0f) ? 0.0f : S[t] * b;
     } else {
-        for (int64_t row = blockIdx.x; row < mat->n; row += gridDim.x)
-            for (int j = (int)threadIdx.x; j < r; j += (int)blockDim.x) {
-                float* p = S + row * mat->lds + j;
-                *p = (b == 0.0f) ? 0.0f : *p * b;
-            }
+        // (a block to a row left most of its threads idle at small ranks: 20 us on 4096 rows of 7)
+        for (int64_t t = tid; t < total; t += nthreads) {
+            const int64_t row = total < (1ll << 32) ? (int64_t)((uint32_t)t / (uint32_t)r) : t / r;
+            float* p = S + row * mat->lds + (t - row * r);
+            *p = (b == 0.0f) ? 0.0f : *p * b;
+        }
     }
 }
 

@@ -29,8 +29,8 @@ struct TcSet {
     bool decompress_ready = false;
     int count = 0, r = 0;
     bool f32 = false;                   // fp32 gradients
-    bool loose = false;                 // a sketch whose rows TMA cannot address
     int T = 1, gstages = 2, astages = 2, lstages = 1, nsets = 1, S = 1, GW = 8, P = 1;
+    int64_t max_chain = (int64_t)1 << 60;        // steps that a CTA of a compression adds up at most (kept to unless every row is to have one owner)
     std::vector<int> k1_launch_first_mat;
     size_t k1_smem = 0;
     TcMatrix* d_mats = nullptr;
@@ -312,7 +312,7 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
     set.astages = astages;
     set.k1_smem = (size_t)gstages * g_stage + (size_t)astages * a_stage + staging + sizeof(PairSmem) + 1024;
     const int64_t slots = resident_clusters<compress_pair_kernel<false, 0>>(S, pair_threads(GW), set.k1_smem);
-    const int64_t group_tiles = (int64_t)S * T;
+    const int64_t group_tiles = (int64_t)S * T, max_chunk = deterministic_flag().load() ? (int64_t)1 << 60 : set.max_chain;
     struct Unit { int mat; int64_t tile0, tiles, kstep0, ksteps; bool direct; };
     auto build_units = [&](int64_t target, std::vector<Unit>& units, std::vector<int>& split) {
         units.clear();
@@ -323,9 +323,9 @@ inline void plan_compress_pair(TcSet& set, const std::vector<flora_mat>& G, int 
             const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + 63) / 64;
             const int64_t groups = (tiles + group_tiles - 1) / group_tiles;
             const int64_t per_group = (tiles + groups - 1) / groups;     // rows spread evenly over the groups
-            int64_t chunk = std::max<int64_t>(8, target / per_group);
+            int64_t chunk = std::min(max_chunk, std::max<int64_t>(8, target / per_group));
             int64_t nchunks = (ks + chunk - 1) / chunk;
-            if (nchunks > 1 && ks - (nchunks - 1) * chunk < chunk / 2) --nchunks;    // no short tail unit
+            if (nchunks > 1 && ks - (nchunks - 1) * chunk < chunk / 2 && (ks + nchunks - 2) / (nchunks - 1) <= max_chunk) --nchunks;    // no short tail unit
             chunk = (ks + nchunks - 1) / nchunks;
             nchunks = (ks + chunk - 1) / chunk;
             if (nchunks > 1) split.push_back((int)i);
@@ -537,7 +537,7 @@ inline void plan_compress(TcSet& set, const std::vector<flora_mat>& G, int r)
             const int64_t tiles = (g.rows + 127) / 128, ks = (g.cols + kc - 1) / kc;
             const int64_t groups = (tiles + group_tiles - 1) / group_tiles;
             const int64_t per_group = (tiles + groups - 1) / groups;     // rows spread evenly over the groups
-            const int64_t max_chunk = f32 ? k1_f32_chain(g.cols) * set.nsets : (int64_t)1 << 60;
+            const int64_t max_chunk = f32 ? k1_f32_chain(g.cols) * set.nsets : deterministic_flag().load() ? (int64_t)1 << 60 : set.max_chain;
             int64_t chunk = std::min(max_chunk, std::max<int64_t>(8, target / per_group));
             int64_t nchunks = (ks + chunk - 1) / chunk;
             if (nchunks > 1 && ks - (nchunks - 1) * chunk < chunk / 2 && (ks + nchunks - 2) / (nchunks - 1) <= max_chunk) --nchunks;    // no short tail item
@@ -898,8 +898,6 @@ inline flora_status tc_fill_matrices(TcSet& set, const std::vector<flora_mat>& G
         tm.m = (int32_t)std::max(G.empty() ? (int64_t)0 : G[i].cols, W.empty() ? (int64_t)0 : W[i].cols);
         if (!G.empty() && G[i].rows && G[i].cols && !make_map(&tm.map_g, G[i])) return FLORA_ERR_CUDA;
         if (!W.empty() && W[i].rows && W[i].cols && !make_map(&tm.map_w, W[i])) return FLORA_ERR_CUDA;
-        tm.loose = !sketch_writable(S[i]);
-        set.loose = set.loose || (tm.loose && !G.empty() && G[i].rows > 0);
         if (S[i].rows && S[i].cols && tc_sketch_ok(S[i]) && !(make_map(&tm.map_s, S[i]) && make_map(&tm.map_sq, S[i], 32))) return FLORA_ERR_CUDA;
     }
     return FLORA_OK;
@@ -1067,11 +1065,36 @@ constexpr int64_t K1_SCALE_PASS_MAX_STATE_BYTES = 32ll << 20;   // sketches of a
 constexpr int64_t K1_EARLY_SCALE_MAX_STATE_BYTES = 16ll << 20;
 
 inline unsigned helper_blocks(int64_t most) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(1024, (most + 1023) / 1024)); }
-inline unsigned helper_blocks(const TcSet& set)
+inline int64_t most_sketch(const TcSet& set)
 {
     int64_t most = 1;
     for (const auto& tm : set.h_mats) most = std::max<int64_t>(most, (int64_t)tm.n * set.r);
-    return helper_blocks(most);
+    return most;
+}
+inline unsigned helper_blocks(const TcSet& set) { return helper_blocks(most_sketch(set)); }
+// S <- b S for `total` matrices of the table (ids, or the first ones), or for the one; most: floats of the largest sketch.
+template <bool SINGLE>
+inline flora_status tc_scale_launch(const TcMatrix* mats, const TcMatrix& one, const int* ids, size_t total, int64_t most, int r, float b, bool early,
+                                    cudaStream_t st, std::atomic<uint64_t>& launches)
+{
+    for (size_t begin = 0; begin < total; begin += 65535) {
+        const size_t jobs_here = std::min<size_t>(65535, total - begin);
+        // few enough blocks to be resident at once: the compression kernel may only start once all have started
+        dim3 grid((unsigned)std::max<size_t>(1, std::min<size_t>(helper_blocks(most), (size_t)sm_count() * 6 / jobs_here)), (unsigned)jobs_here);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(256);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = early ? 1 : 0;
+        if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<SINGLE>, mats, one, ids ? ids + begin : (const int*)nullptr, (int)begin, r, b) != cudaSuccess)
+            return FLORA_ERR_CUDA;
+        launches.fetch_add(1, std::memory_order_relaxed);
+    }
+    return FLORA_OK;
 }
 
 // behind_own_kernel: the kernels before this call on the stream, back to one that everything earlier was complete before, are the
@@ -1079,8 +1102,8 @@ inline unsigned helper_blocks(const TcSet& set)
 // compression waits for them.
 // one: the record of the matrix where the plan is that of a single one (it then holds no addresses itself).  mats: the table of the
 // others; new_maps: its maps may have been written since the kernel before.
-template <bool SINGLE, int MAPS, bool LOOSE>
-inline flora_status tc_compress_launch_as(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
+template <bool SINGLE, int MAPS>
+inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
                                        cudaStream_t st, std::atomic<uint64_t>& launches, bool behind_own_kernel, bool new_maps = false)
 {
     const int r = set.r;
@@ -1095,8 +1118,7 @@ inline flora_status tc_compress_launch_as(const TcSet& set, const TcMatrix* mats
     if (SINGLE) state_bytes = (int64_t)one.n * r * 4;
     else
         for (int i : set.members) state_bytes += (int64_t)set.h_mats[i].n * r * 4;
-    // Sketches that TMA cannot address are always scaled first (see write_piece).
-    const bool scale_all = b != 0.0f && b != 1.0f && (LOOSE || (pair && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES));
+    const bool scale_all = pair && b != 0.0f && b != 1.0f && state_bytes <= K1_SCALE_PASS_MAX_STATE_BYTES;
     if (scale_all || (b != 1.0f && !set.split_mats.empty())) {
         // A short pass is itself launched early, and the compression waits for it with everything (momentum step of one 4096 x 11008
         // matrix at r = 8 22.7 -> 21.4 us, with b = 0 22.9 -> 20.8; fp32 1024 x 4096 at r = 64 20.6 -> 18.5).  A long one starts behind
@@ -1106,27 +1128,12 @@ inline flora_status tc_compress_launch_as(const TcSet& set, const TcMatrix* mats
         // rows that receive adds (from several CTAs, or from the pair kernel's reducing write-out): scale them by b first
         const size_t total = SINGLE ? 1 : scale_all ? set.members.size() : set.split_mats.size();
         const int* ids = scale_all ? set.d_members : set.d_split;        // (no list: every matrix of the set)
-        for (size_t begin = 0; begin < total; begin += 65535) {
-            const size_t jobs_here = std::min<size_t>(65535, total - begin);
-            // few enough blocks to be resident at once: the compression kernel may only start once all have started
-            dim3 grid((unsigned)std::max<size_t>(1, std::min<size_t>(SINGLE ? helper_blocks(state_bytes / 4) : helper_blocks(set), (size_t)sm_count() * 6 / jobs_here)), (unsigned)jobs_here);
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = grid;
-            cfg.blockDim = dim3(256);
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = early ? 1 : 0;
-            if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<SINGLE>, mats, one, ids ? ids + begin : (const int*)nullptr, (int)begin, r, b) != cudaSuccess)
-                return FLORA_ERR_CUDA;
-            launches.fetch_add(1, std::memory_order_relaxed);
-        }
+        const flora_status rc = tc_scale_launch<SINGLE>(mats, one, ids, total, SINGLE ? state_bytes / 4 : most_sketch(set), r, b, early, st, launches);
+        if (rc) return rc;
         if (scale_all) b = 1.0f;
     }
-    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE, MAPS, LOOSE>>()
-               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true, MAPS>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false, MAPS, LOOSE>>()))
+    if (!(pair ? raise_smem_limit<compress_pair_kernel<SINGLE, MAPS>>()
+               : set.f32 ? raise_smem_limit<compress_tc_kernel<SINGLE, true, MAPS>>() : raise_smem_limit<compress_tc_kernel<SINGLE, false, MAPS>>()))
         return FLORA_ERR_CUDA;
     for (size_t l = 0; l + 1 < set.k1_launch_begin.size(); ++l) {
         const int begin = set.k1_launch_begin[l], end = set.k1_launch_begin[l + 1];
@@ -1158,27 +1165,19 @@ inline flora_status tc_compress_launch_as(const TcSet& set, const TcMatrix* mats
         cudaError_t e;
         if (pair) {
             const int* slot_table = set.d_slots + set.k1_slots_begin[l];
-            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE, MAPS, LOOSE>, mats, one, gmaps, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
+            e = cudaLaunchKernelEx(&cfg, compress_pair_kernel<SINGLE, MAPS>, mats, one, gmaps, items, slot_table, table, seed_base, r, set.k1_n, scale, a, b, set.gstages,
                                    set.astages, set.S, set.GW, lw, (int)new_maps);
         } else {
             auto go = [&](auto kernel) {
                 return cudaLaunchKernelEx(&cfg, kernel, mats, one, gmaps, items, table, seed_base, r, scale, a, b, set.T, set.gstages, set.astages, set.lstages,
                                           set.nsets, set.S, set.GW, set.P, lw, (int)new_maps);
             };
-            e = set.f32 ? go(compress_tc_kernel<SINGLE, true, MAPS>) : go(compress_tc_kernel<SINGLE, false, MAPS, LOOSE>);
+            e = set.f32 ? go(compress_tc_kernel<SINGLE, true, MAPS>) : go(compress_tc_kernel<SINGLE, false, MAPS>);
         }
         if (e != cudaSuccess) return FLORA_ERR_CUDA;
         launches.fetch_add(1, std::memory_order_relaxed);
     }
     return cudaPeekAtLastError() == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
-}
-
-template <bool SINGLE, int MAPS>
-inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, const TcMatrix& one, const uint64_t* seeds, float a, float b,
-                                       cudaStream_t st, std::atomic<uint64_t>& launches, bool behind_own_kernel, bool new_maps = false)
-{
-    return (SINGLE ? one.loose != 0 : set.loose) ? tc_compress_launch_as<SINGLE, MAPS, true>(set, mats, one, seeds, a, b, st, launches, behind_own_kernel, new_maps)
-                                                 : tc_compress_launch_as<SINGLE, MAPS, false>(set, mats, one, seeds, a, b, st, launches, behind_own_kernel, new_maps);
 }
 
 inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches,
@@ -1201,10 +1200,11 @@ inline flora_status tc_set_compress(TcSet& set, const uint64_t* seeds, float a, 
 // cache are serialised by its mutex; a plan is built with a synchronous upload, so any stream may use it afterwards.
 struct SinglePlanKey {
     int dev, kind, r, det, dtype, loose;
+    int64_t max_chain;
     int64_t rows, cols;
     bool operator==(const SinglePlanKey& o) const
     {
-        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && dtype == o.dtype && loose == o.loose && rows == o.rows && cols == o.cols;
+        return dev == o.dev && kind == o.kind && r == o.r && det == o.det && dtype == o.dtype && loose == o.loose && max_chain == o.max_chain && rows == o.rows && cols == o.cols;
     }
 };
 struct SinglePlan {
@@ -1219,7 +1219,7 @@ inline std::mutex& single_plan_mutex()
     return m;
 }
 // Call with single_plan_mutex() held.  kind 0: compression (big = G), 1: decompression (big = W).
-inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketch, cudaStream_t st, flora_status* rc)
+inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketch, cudaStream_t st, flora_status* rc, int64_t max_chain = (int64_t)1 << 60)
 {
     static std::vector<SinglePlan*> cache;                     // most recently used first
     *rc = FLORA_OK;
@@ -1235,6 +1235,7 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
     key.det = deterministic_flag().load();
     key.dtype = big.dtype;
     key.loose = kind == 1 && !tc_sketch_ok(sketch);
+    key.max_chain = max_chain;
     key.rows = big.rows;
     key.cols = big.cols;
     for (size_t i = 0; i < cache.size(); ++i)
@@ -1259,6 +1260,7 @@ inline TcSet* single_plan(int kind, const flora_mat& big, const flora_mat& sketc
     set.members.assign(1, 0);
     const std::vector<flora_mat> b(1, big);
     if (kind == 0) {
+        set.max_chain = max_chain;
         plan_compress(set, b, set.r);
         *rc = upload(&set.d_k1, set.h_k1, st);
         if (*rc == FLORA_OK) *rc = upload(&set.d_slots, set.h_slots, st);
@@ -1291,18 +1293,17 @@ inline bool single_record(TcMatrix* tm, const flora_mat& big, const flora_mat& s
     tm->lds = sketch.ld;
     tm->n = (int32_t)big.rows;
     tm->m = (int32_t)big.cols;
-    tm->loose = !sketch_writable(sketch);
     return make_map(is_g ? &tm->map_g : &tm->map_w, big) && (!tc_sketch_ok(sketch) || (make_map(&tm->map_s, sketch) && (!is_g || make_map(&tm->map_sq, sketch, 32))));
 }
 
 inline flora_status tc_compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, float a, float b, cudaStream_t st,
-                                       std::atomic<uint64_t>& launches)
+                                       std::atomic<uint64_t>& launches, int64_t max_chain = (int64_t)1 << 60)
 {
     TcMatrix one;
     if (!single_record(&one, *G, *S, true)) return FLORA_ERR_CUDA;
     std::lock_guard<std::mutex> lock(single_plan_mutex());
     flora_status rc;
-    TcSet* set = single_plan(0, *G, *S, st, &rc);
+    TcSet* set = single_plan(0, *G, *S, st, &rc, max_chain);
     return set ? tc_compress_launch<true, 0>(*set, nullptr, one, &seed, a, b, st, launches, false) : rc;
 }
 
