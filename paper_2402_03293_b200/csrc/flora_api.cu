@@ -216,7 +216,7 @@ flora_status compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, fl
         flora_mat sums{nullptr, S->rows, S->cols, fold_ld(r), FLORA_F32};
         if (scratch_alloc(&sums.data, sizeof(float) * (size_t)(sums.rows * sums.ld), st) == cudaSuccess) {
             // (sums as short as those of the general kernels: the tensor core truncates them, 7e-8 of a sum lost per step of 64 columns)
-            const int64_t steps = (G->cols + 63) / 64, parts = gen_k1_choose(false, r, (G->rows + 127) / 128, steps, true, false).cluster;
+            const int64_t steps = (G->cols + 63) / 64, parts = gen_k1_choose(false, r, (G->rows + 127) / 128, steps, true).cluster;
             flora_status rc = tc_compress_single(G, &sums, seed, 1.0f, 0.0f, st, g_launches, (steps + parts - 1) / parts);
             const FoldMat fold{(float*)S->data, (const float*)sums.data, S->ld, (int32_t)S->rows, (int32_t)sums.ld, 1, 0};
             if (rc == FLORA_OK) rc = fold_single(fold, r, a, b, sm_count(), st, g_launches);

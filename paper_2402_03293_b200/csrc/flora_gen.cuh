@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "flora_fold.cuh"
 #include "flora_ptx.cuh"
 #include "flora_rng.cuh"
 #include "flora_tc.cuh"
@@ -26,6 +27,7 @@ struct GenMat {            // a matrix with its sketch
     float* S;
     int64_t ld, lds;
     int32_t n, m;
+    float* D;              // compression: scratch for the sums of its parts (GEN_JOIN_SLICES)
 };
 struct GenItem {           // compression: one cluster, or one CTA of a split whose CTAs form none
     int32_t mat;
@@ -45,16 +47,15 @@ constexpr int GEN_MAX_SPLIT = 16;                           // CTAs of a cluster
 // parts in 32 bits, so no more than 64 (without a limit a member of 1 x 31,765,017 got 9732 of them, a ninth over the wrong columns).
 constexpr int GEN_MAX_PARTS = 64;
 static_assert((uint64_t)GEN_MAX_PARTS << 25 < 1ull << 32 && GEN_MAX_SPLIT <= GEN_MAX_PARTS, "column ranges are found in 32 bits");
-// How the CTAs of a split bring their sums together.
-//   Ordered   through distributed shared memory: every row has one writer, which adds the peers' sums in a fixed order.  Bit-reproducible
-//             mode only: reading the peers and the two cluster barriers around that took half of a small launch.
-//   Scaled    every CTA adds its sums to the sketch in global memory (red.global), after the cluster has scaled the rows: each CTA its
-//             share of them while its first loads travel, and a barrier whose wait is over before the sums are there.
-//   Plain     the same where there is nothing to scale (b = 1): no barrier, and no clusters.
-// Measured with Ordered / Scaled / Plain, us a launch in a chain: 512 x 512 at r = 8 in fp32 5.9 / 4.4 / 3.6, 256 x 384 at r = 32 5.0 / 4.4 / 3.6,
-// 768 x 768 at r = 16 5.5 / 4.7 / 3.7, 768 x 2304 at r = 16 7.6 / 6.1 / 5.3.  (Of the 6 us of the first one 1.3 passed before it could read
-// anything, 1.6 until its product was there, 3.1 with the sums of sixteen CTAs, the write-out and the way out.)
-enum GenJoin { GEN_JOIN_ORDERED, GEN_JOIN_SCALED, GEN_JOIN_PLAIN };
+// How the CTAs of a split bring their sums together.  In either way the sums are added in a fixed order and rounded into the sketch once.  (Every CTA
+// added its sums to the sketch by itself before: 512 x 512 at r = 8 in fp32 3.6 us instead of 4.7, but a step was off by up to four times as much once the
+// state was as large as what is added to it, and differed from run to run.)
+//   Push     the CTAs of a cluster: each sends every row's sums to the CTA that owns the row (st.async, counted by the owner's mbarrier), which adds them up
+//            and blends them into the sketch.  Nothing waits for a peer but for its sums.  (Reading the peers' sums, between two cluster barriers, took
+//            half of a small launch: 5.9 us there.)
+//   Slices   single CTAs store the sums of their part in scratch, and a kernel behind them blends them in (flora_fold.cuh).  No clusters, so
+//            any free slot of an SM will do and more CTAs are resident: larger matrices.
+enum GenJoin { GEN_JOIN_PUSH, GEN_JOIN_SLICES };
 // Columns of an fp32 matrix that one launch adds up: as many as keep every CTA's chain within its limit.  Wider matrices take several
 // launches, whose sums are added in rounded fp32 (one after another, so in a fixed order).
 constexpr int GEN_F32_PASS_COLS = 32 * GEN_MAX_SPLIT * GEN_F32_CHAIN_STEPS;
@@ -115,9 +116,12 @@ struct GenK1 {
     static constexpr int TILE = 128 * ROWB;                 // one part of a 128-row tile
 };
 struct GenSmem {
-    uint64_t full[GEN_G_SLOTS_MAX], empty[GEN_G_SLOTS_MAX], a_empty[GEN_A_SLOTS_MAX], acc_full;
+    uint64_t full[GEN_G_SLOTS_MAX], empty[GEN_G_SLOTS_MAX], a_empty[GEN_A_SLOTS_MAX], acc_full, landed;
     uint32_t tmem_base;
     int abort;
+    // what only the write-out needs: in registers over the main loop it costs that loop spills (fp32 8192 x 8191 at r = 32: 140 -> 163 us)
+    GenMat mat;
+    int32_t split, part, group, tile0, tiles, steps;
 };
 // Shared memory: a ring of tiles of G (parts of 128 rows x K) and a ring of tiles of A (one per step, used by all its tiles).
 inline size_t gen_k1_g_bytes(bool f32) { return f32 ? (size_t)3 * 64 * 128 : (size_t)128 * 128; }
@@ -126,25 +130,14 @@ inline size_t gen_k1_a_bytes(bool f32, int r_pad) { return f32 ? (size_t)3 * 64 
 // rows write to different banks.
 __host__ __device__ inline int gen_stage_stride(int r_pad) { return r_pad + 4; }
 
-// `rows` rows of the sketch from row0 on, times b (b = 0: cleared, whatever they held), by NT threads.
-template <int NT>
-__device__ __forceinline__ void scale_rows(const GenMat& mat, int row0, int rows, int r, float b, int tid)
+// The rows of a group's tiles that a CTA of it owns (push), and the most that any of them does.
+struct GenRows {
+    int begin, end, share;
+};
+__device__ __forceinline__ GenRows gen_rows(int tiles, int part, int split)
 {
-    const bool vec = (r & 3) == 0 && (mat.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(mat.S) & 15) == 0;
-    const int per = vec ? r >> 2 : r, total = rows * per;                    // pieces
-    float* const S = mat.S + (int64_t)row0 * mat.lds;
-#pragma unroll 4
-    for (int e = tid; e < total; e += NT) {
-        const int i = e / per, j = e - i * per;
-        float* const p = S + (int64_t)i * mat.lds + (vec ? 4 * j : j);
-        if (vec) {
-            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (b != 0.0f) o = *reinterpret_cast<const float4*>(p);
-            *reinterpret_cast<float4*>(p) = make_float4(b * o.x, b * o.y, b * o.z, b * o.w);
-        } else {
-            *p = b != 0.0f ? b * *p : 0.0f;
-        }
-    }
+    const int rows = tiles * 128;
+    return GenRows{part * rows / split, (part + 1) * rows / split, (rows + split - 1) / split};
 }
 
 // SINGLE: one matrix, passed by value; every cluster takes the next row groups of it.  (A template and not a test of `items`: with
@@ -156,7 +149,7 @@ template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 __global__ void __launch_bounds__(gen_threads(WORKERS), WORKERS == 8 ? 2 : 1)
 gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
                     const __grid_constant__ GenMat single, int single_split, int single_col0, int seed_base, int r, float scale, float a, float b, int T, int sbs,
-                    int g_slots, int a_slots, int cluster, int joining, int ahead)
+                    int g_slots, int a_slots, int cluster, int joining, int land, int ahead)
 {
     using C = GenK1<F32>;
     constexpr int NT = 32 * WORKERS;                              // worker threads
@@ -190,7 +183,9 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     // (in 32 bits, see GEN_MAX_PARTS: a 64-bit division takes a quarter of a microsecond)
     const int ks0 = step0 + (int)((uint32_t)part * (uint32_t)all_steps / (uint32_t)split), ks1 = step0 + (int)((uint32_t)(part + 1) * (uint32_t)all_steps / (uint32_t)split);
     const int steps = tiles > 0 ? ks1 - ks0 : 0;
-    const bool barrier = cluster > 1 && joining == GEN_JOIN_SCALED;
+    // Push: the sums of the group's CTAs for the rows that this one owns land in shared memory behind the rings, or, where there is no room, in them,
+    // once the peers know that they are free.
+    const bool push = cluster > 1 && joining == GEN_JOIN_PUSH, apart = land != 0;
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < T * acc_cols) tmem_cols <<= 1;
 
@@ -201,8 +196,18 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         }
         for (int s = 0; s < a_slots; ++s) ptx::mbar_init(ptx::smem_addr(&ctl.a_empty[s]), 1);
         ptx::mbar_init(ptx::smem_addr(&ctl.acc_full), 1);
+        ptx::mbar_init(ptx::smem_addr(&ctl.landed), 1);
         ctl.abort = 0;
+        ctl.mat = mat;
+        ctl.split = split;
+        ctl.part = part;
+        ctl.group = group;
+        ctl.tile0 = tile0;
+        ctl.tiles = tiles;
+        ctl.steps = steps;
         ptx::fence_barrier_init();
+        const GenRows own = gen_rows(tiles, part, split);
+        if (push && split > 1) ptx::mbar_arrive_expect_tx(ptx::smem_addr(&ctl.landed), (uint32_t)(split * max(0, min(own.end, mat.n - tile0 * 128) - own.begin) * ((r + 3) >> 2) * 16));
         ptx::fence_proxy_async_smem();
     }
     if (warp == WORKERS) {
@@ -224,15 +229,10 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
     ptx::grid_launch_dependents();
     const uint32_t tmem = ctl.tmem_base;
     volatile int* abort = &ctl.abort;
+    if (push && apart) ptx::cluster_arrive_release();
 
     if (warp == WORKERS) {
         // ------------------------------------------------------------------ MMA issuer
-        if (barrier) {
-            // the workers have scaled this CTA's rows; the release is this warp's, as it has nothing else to do until the first tile is
-            // there (by the workers, behind the main loop, it took 0.9 us of a small launch)
-            ptx::named_barrier_sync(2, NT + 32);
-            ptx::cluster_arrive_release();
-        }
         if (lane == 0 && steps > 0) {
             RingPos pg, pa;
             bool ok = true;
@@ -408,14 +408,6 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         for (int d = 0; d < AHEAD; ++d)
             if (d < total) fetch(x[d]);
         while (made < min(lead + 1, steps)) make();
-        if (barrier && split > 1) {
-            const int lr0 = part * (tiles * 128) / split, lr1 = (part + 1) * (tiles * 128) / split;
-            scale_rows<NT>(mat, tile0 * 128 + lr0, min(lr1 - lr0, mat.n - tile0 * 128 - lr0), r, b, tid);
-        }
-        if (barrier) {
-            ptx::named_barrier_arrive(2, NT + 32);
-            ptx::cluster_arrive_relaxed();
-        }
         RingPos pg;
         auto turn = [&](bool more, uint4 (&x)[NI][BLK]) {
             if (pt == 0 && made < steps && made <= pks + lead) {
@@ -441,8 +433,21 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                 if (u + d < total) turn(u + d + AHEAD < total, x[d]);
         }
         // ------------------------------------------------------------------ write-out
-        // A split: accumulators -> sketch, added in global memory, a row of a tile per thread.  Otherwise, and where rows have no 16-byte
-        // pieces: accumulators -> shared memory (the operand rings, free by now), whose rows whole warps then add or write.
+        constexpr bool STORED = !SINGLE || F32 || ALIGNED;                     // (GenSmem; single unaligned bf16 matrices spill less without)
+        const GenMat& mat_ = mat;
+        const int split_ = split, part_ = part, group_ = group, tile0_ = tile0, tiles_ = tiles, steps_ = steps;
+        {
+        // A split: accumulators -> the row's owner, or scratch, a row of a tile per thread.  Otherwise accumulators -> shared memory (the operand
+        // rings, free by now), whose rows whole warps then write.
+        if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
+        ptx::tc_fence_after_sync();
+        if (push) {
+            if (!apart) ptx::cluster_arrive_release();                       // this CTA's rings are free
+            ptx::cluster_wait_some();                                        // its peers' are, and their barriers are set up
+        }
+        const GenMat mat = STORED ? ctl.mat : mat_;
+        const int split = STORED ? ctl.split : split_, part = STORED ? ctl.part : part_, group = STORED ? ctl.group : group_,
+                  tile0 = STORED ? ctl.tile0 : tile0_, tiles = STORED ? ctl.tiles : tiles_, steps = STORED ? ctl.steps : steps_;
         float* const stage = reinterpret_cast<float*>(ring);
         const int stride = gen_stage_stride(r_pad);
         auto load_sums = [&](int t, int c, uint32_t (&v)[16]) {              // sixteen columns of a tile, a row per thread
@@ -519,9 +524,6 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
 #pragma unroll 4
             for (int e = tid + NOLD * NT; e < total_e; e += NT) put(e, b != 0.0f ? old_at(e, lr0, grow0) : make_float4(0.f, 0.f, 0.f, 0.f));
         };
-        if (total > 0 && ok) ok = ptx::mbar_wait(ptx::smem_addr(&ctl.acc_full), 0, abort);
-        ptx::tc_fence_after_sync();
-        if (barrier) ptx::cluster_wait_some();
         if (split == 1) {
             for (int t = 0; t < tiles; ++t) {
                 fetch_old(0, 128, (tile0 + t) * 128);
@@ -534,76 +536,80 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
                         return vec ? *reinterpret_cast<const float4*>(p) : make_float4(*p, 0.f, 0.f, 0.f);
                     });
             }
-            if (cluster > 1 && joining == GEN_JOIN_ORDERED) {
-                ptx::cluster_sync_some();
-                ptx::cluster_sync_some();
-            }
-        } else if (joining != GEN_JOIN_ORDERED) {
-            const bool adds = steps > 0 && !*abort;
-            for (int t = 0; t < tiles; ++t) {
-                if (vec) {
-                    const int row = (tile0 + t) * 128 + (warp & 3) * 32 + lane;
-                    float* const dst = mat.S + (int64_t)row * mat.lds;
-                    for (int c = (warp >> 2) * 16; c < r_pad; c += 4 * WORKERS) {
-                        uint32_t v[16];
-                        __syncwarp();
-                        load_sums(t, c, v);
+        } else if (push) {
+            // Sums land as [sender][piece of four columns][row]: neighbouring rows, which a warp's lanes hold, go to neighbouring addresses.
+            const GenRows own = gen_rows(tiles, part, split);
+            const int rows = tiles * 128, share = own.share, lr0 = own.begin, quads = (r + 3) >> 2, mine = min(own.end, mat.n - tile0 * 128) - lr0, total_e = share * quads;
+            auto place_of = [&](int e, int& left) {                          // a thread's piece e of the rows that this CTA owns
+                const int p = e / share, i = e - p * share;
+                left = i < mine ? r - 4 * p : 0;
+                return mat.S + (int64_t)(tile0 * 128 + lr0 + i) * mat.lds + 4 * p;
+            };
+            auto old_of = [&](int e) {
+                int left;
+                const float* src = place_of(e, left);
+                return b != 0.0f ? load_some(src, vec, left) : make_float4(0.f, 0.f, 0.f, 0.f);
+            };
 #pragma unroll
-                        for (int k = 0; k < 16; k += 4)
-                            if (adds && row < mat.n && c + k < r)
-                                ptx::red_add_v4(dst + c + k, a * __uint_as_float(v[k]), a * __uint_as_float(v[k + 1]), a * __uint_as_float(v[k + 2]), a * __uint_as_float(v[k + 3]));
-                    }
-                } else {
-                    // (through shared memory: neighbouring threads then add to neighbouring values)
-                    if (t > 0) ptx::named_barrier_sync(1, NT);
-                    stage_tile(t, stage);
-                    ptx::named_barrier_sync(1, NT);
-                    const int grow0 = (tile0 + t) * 128, total_e = adds ? min(128, mat.n - grow0) * r : 0;
-#pragma unroll 4
-                    for (int e = tid; e < total_e; e += NT) {
-                        const int i = e / r, j = e - i * r;
-                        ptx::red_add(mat.S + (int64_t)(grow0 + i) * mat.lds + j, a * stage[i * stride + j]);
-                    }
+            for (int k = 0; k < NOLD; ++k) old[k] = tid + k * NT < total_e ? old_of(tid + k * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
+            // (also of a CTA that has given up: its peers count on the bytes)
+            for (int t = 0; t < tiles; ++t) {
+                const int row = t * 128 + (warp & 3) * 32 + lane, owner = ((row + 1) * split - 1) / rows, at = row - owner * rows / split;
+                const uint32_t to = (uint32_t)(group * split + owner), bar = ptx::map_to_cta(ptx::smem_addr(&ctl.landed), to);
+                const uint32_t dst = ptx::map_to_cta(smem_base + (uint32_t)land + (uint32_t)(part * quads * share + at) * 16u, to);
+                for (int c = (warp >> 2) * 16; c < r_pad; c += 4 * WORKERS) {
+                    uint32_t v[16];
+                    __syncwarp();
+                    load_sums(t, c, v);
+#pragma unroll
+                    for (int k = 0; k < 16; k += 4)
+                        if (tile0 * 128 + row < mat.n && c + k < r)
+                            ptx::st_async_v4(dst + (uint32_t)((c + k) >> 2) * (uint32_t)share * 16u, v[k], v[k + 1], v[k + 2], v[k + 3], bar);
                 }
             }
+            // (a peer that gives up sends its sums after one time limit, so this one waits longer: it must not leave before they are here)
+            ok = ptx::mbar_wait_peers(ptx::smem_addr(&ctl.landed), 0, abort, 4 * ptx::WAIT_LIMIT_NS) && ok;
+            const float4* const landing = reinterpret_cast<const float4*>(ring + land);
+            auto put = [&](int e, const float4& o) {
+                int left;
+                float* const dst = place_of(e, left);
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+                for (int q = 0; q < split; ++q) {
+                    const float4 w = landing[q * total_e + e];
+                    v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+                }
+                store_some(dst, fold_blend(v, o, a, b), vec, left);
+            };
+            if (!*abort) {
+#pragma unroll
+                for (int k = 0; k < NOLD; ++k)
+                    if (tid + k * NT < total_e) put(tid + k * NT, old[k]);
+                for (int e = tid + NOLD * NT; e < total_e; e += NT) put(e, old_of(e));
+            }
         } else {
-            const int lr0 = part * (tiles * 128) / split, lr1 = (part + 1) * (tiles * 128) / split;
-            fetch_old(lr0, lr1, tile0 * 128);
-            for (int t = 0; t < tiles; ++t) stage_tile(t, stage + t * 128 * stride);
-            ptx::cluster_sync_some();                                        // every partial sum of the cluster is staged
-            const uint32_t sbase = ptx::smem_addr(stage);
-            const int first_rank = group * split;
-            if (!*abort)
-                write_rows(lr0, lr1, tile0 * 128, [&](int i, int j) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const uint32_t at = sbase + (uint32_t)(i * stride + j) * 4u;
-                    // (eight at a time under way, each CTA from its own neighbour on: it is their latency that counts)
-                    for (int q0 = 0; q0 < split; q0 += 8) {
-                        float4 w[8];
+            // (laid out for the kernel that adds the slices up, in lines of eight rows' pieces: FoldMat)
+            const int quads = (r + 3) >> 2;
+            float4* const slice = reinterpret_cast<float4*>(mat.D) + (int64_t)part * fold_slice(mat.n, r);
+            for (int t = 0; t < tiles; ++t) {
+                const int row = (tile0 + t) * 128 + (warp & 3) * 32 + lane;
+                float4* const dst = slice + (int64_t)(row >> 3) * quads * 8 + (row & 7);
+                for (int c = (warp >> 2) * 16; c < r_pad; c += 4 * WORKERS) {
+                    uint32_t v[16];
+                    __syncwarp();
+                    load_sums(t, c, v);
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int q = q0 + u + part;
-                            w[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (q0 + u < split) {
-                                const uint32_t p = ptx::map_to_cta(at, (uint32_t)(first_rank + (q < split ? q : q - split)));
-                                if (vec) w[u] = ptx::ld_cluster_v4(p);
-                                else w[u].x = ptx::ld_cluster_f32(p);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) v = make_float4(v.x + w[u].x, v.y + w[u].y, v.z + w[u].z, v.w + w[u].w);
-                    }
-                    return v;
-                });
-            ptx::cluster_sync_some();                                        // nobody leaves while a peer may still read its sums
+                    for (int k = 0; k < 16; k += 4)
+                        if (row < mat.n && c + k < r)
+                            dst[((c + k) >> 2) * 8] = make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]), __uint_as_float(v[k + 3]));
+                }
+            }
+        }
         }
     }
-    if (warp == WORKERS) {
-        if (barrier) ptx::cluster_wait_some();
-        else if (cluster > 1 && joining == GEN_JOIN_ORDERED) {
-            ptx::cluster_sync_some();
-            ptx::cluster_sync_some();
-        }
+    if (warp == WORKERS && push) {
+        if (!apart) ptx::cluster_arrive_release();
+        ptx::cluster_wait_some();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();

@@ -6,7 +6,9 @@
 #include <atomic>
 #include <vector>
 
+#include "flora_fold.cuh"
 #include "flora_gen.cuh"
+#include "flora_pool.cuh"
 #include "flora_tc_host.cuh"
 
 namespace flora {
@@ -17,7 +19,8 @@ struct GenK1Plan {
     bool sbs = false;
     size_t smem = 0;
     bool aligned = true;
-    bool ordered = false;      // bit-reproducible sums
+    bool push = false;         // GEN_JOIN_PUSH: `cluster` CTAs form one
+    uint32_t land = 0;         // ... where peers' sums land in shared memory (0: in the rings)
     bool beside = false;       // two such launches fit side by side (see gen_k1_choose)
     double cost = 0;           // by gen_k1_cost
 };
@@ -34,7 +37,7 @@ inline int64_t gen_f32_chain(int64_t steps) { return std::min<int64_t>(GEN_F32_C
 // Rings, accumulator layout and CTAs per SM for T tiles per CTA; false where they do not fit.  `per_sm` = 2: two CTAs with at
 // most 112 KB and 256 accumulator columns each.  At least three slots of G and two of A (with fewer the warps wait for the MMAs of
 // the step before: fp32 4096 x 11008 at r = 8 ran at half the speed).
-inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int per_sm, int64_t steps)
+inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, bool push, int per_sm, int64_t steps)
 {
     const int r_pad = (r + 15) & ~15, most_cols = per_sm == 2 ? 256 : 512;
     p.sbs = f32 && 3 * r_pad <= 256 && T * 3 * r_pad <= most_cols;
@@ -42,16 +45,25 @@ inline bool gen_k1_shape(GenK1Plan& p, bool f32, int r, int T, bool split, int p
     if (cols_used > most_cols) return false;
     const size_t budget = (per_sm == 2 ? 112 * 1024 : SMEM_BUDGET) - 1024;
     const size_t g = gen_k1_g_bytes(f32), a = gen_k1_a_bytes(f32, r_pad);
-    const size_t staged = (size_t)(split ? T : 1) * 128 * gen_stage_stride(r_pad) * 4;
+    // (single CTAs of a split stage nothing, but two tiles at r = 128 with two slots of A, which then fit two CTAs on an SM, ran 3000 x 5001 in 48 us instead of 38)
+    const size_t staged = ((size_t)(split ? T : 1) * 128 + (push ? GEN_MAX_SPLIT : 0)) * gen_stage_stride(r_pad) * 4;
     if (3 * g + 2 * a > budget || staged > budget) return false;
     p.T = T;
     p.per_sm = per_sm;
     // Slots of A: three, or one for each step of a short run, so that all may be made while the kernel before this one runs (24 KB at
     // most, and four slots of G stay).
-    p.a_slots = budget >= 4 * g + 3 * a ? 3 : 2;
-    if (p.a_slots == 3 && steps <= GEN_A_SLOTS_MAX && steps * a <= std::min<size_t>(24 * 1024, budget - 4 * g)) p.a_slots = (int)std::max<int64_t>(3, steps);
-    p.g_slots = (int)std::min<size_t>(GEN_G_SLOTS_MAX, (budget - p.a_slots * a) / g);
-    p.smem = std::max(p.g_slots * g + p.a_slots * a, staged) + 1024;
+    auto rings = [&](size_t room) {
+        p.a_slots = room >= 4 * g + 3 * a ? 3 : 2;
+        if (p.a_slots == 3 && steps <= GEN_A_SLOTS_MAX && steps * a <= std::min<size_t>(24 * 1024, room - 4 * g)) p.a_slots = (int)std::max<int64_t>(3, steps);
+        p.g_slots = (int)std::min<size_t>(GEN_G_SLOTS_MAX, (room - p.a_slots * a) / g);
+        return p.g_slots * g + p.a_slots * a;
+    };
+    // Peers' sums land behind the rings where four slots of G and three of A, or as many as a short run uses, stay beside them (512 x 512 at r = 8 in fp32, a
+    // step a CTA: 4.7 us, in the rings 5.3).
+    p.push = push;
+    p.land = 0;
+    if (push && budget >= staged + std::min<size_t>(4, steps * T) * g + std::min<size_t>(3, std::max<size_t>(2, steps)) * a) p.land = (uint32_t)rings(budget - staged);
+    p.smem = p.land ? p.land + staged + 1024 : std::max(rings(budget), staged) + 1024;
     // no more CTAs on an SM than its tensor memory serves: the CTAs of a cluster wait for one another, so none may wait for columns
     uint32_t cols = 32;
     while ((int)cols < cols_used) cols <<= 1;
@@ -74,6 +86,10 @@ inline double gen_k1_cost(bool f32, int r, int T, int workers, double together, 
     const double step = std::max(latency, std::max(1.0, together) * std::max(700.0 * T, issue));
     return (double)waves * (4000.0 + (workers == 16 ? 2000.0 : 0.0) + (split > 1 ? 200.0 : 0.0) + (double)steps * step);
 }
+// The kernel that blends the sums of a split into the sketch: a microsecond of a chain, one more for every sixteen parts that it reads, and its bytes, of which
+// L2 takes and gives some 8 TB/s.  (In a chain, without and with it, us: 512 x 512 at r = 8 in fp32, sixteen parts, 3.6 and 5.6; the ragged set of eight matrices at r = 32, 33 parts
+// at most, 8.3 and 13.4, in fp32, 64 parts, 11.7 and 17.8.)
+inline double gen_fold_cost(int64_t parts, double floats) { return 2000.0 + 2300.0 * (double)((parts + 15) / 16) + 1.9 / 8000.0 * 4.0 * floats; }
 // Clusters of `size` CTAs of the compression kernel that can be resident (asked once per kind of launch: the kernel's variants
 // need the same registers, so one stands for all).
 inline int gen_k1_resident(const GenK1Plan& p, int size)
@@ -92,15 +108,13 @@ inline int gen_k1_resident(const GenK1Plan& p, int size)
     known.push_back({dev, p.workers, size, n, p.smem});
     return n;
 }
-// Tile shape and split with the shortest schedule.  Chosen once per shape and kept (64 of them).
-// clusters: the CTAs of a split form one (see GenJoin); without, any free slot will do, and more CTAs are resident.  A launch that leaves
+// Tile shape and split with the shortest schedule.  Chosen once per shape and manner of joining and kept (of 64 shapes).
+// push: the CTAs of a split form a cluster; without, any free slot will do, and more CTAs are resident.  A launch that leaves
 // half of the GPU free (beside) starts, in a chain of such launches, beside its predecessor and has the time to fill its ring of A; clusters
-// that do not also lose what single CTAs find in the gaps, about the time of making two tiles of A (1000 x 4097 at r = 64, a momentum step: 17.7 us in
-// clusters, 14.0 without and with a pass that scales the sketch).
-// chain: it stands behind launches like itself (compressions of a cycle).
-inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bool clusters, bool chain)
+// that do not also lose what single CTAs find in the gaps, about the time of making two tiles of A.
+inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bool push)
 {
-    struct Known { int dev, r; bool f32, clusters, chain; int64_t tiles, steps; GenK1Plan plan; };
+    struct Known { int dev, r; bool f32, push; int64_t tiles, steps; GenK1Plan plan; };
     static std::mutex mutex;
     static std::vector<Known> known;
     int dev = 0;
@@ -108,7 +122,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
     std::lock_guard<std::mutex> lock(mutex);
     if (tune_knob("FLORA_GEN_T", 0, 0, 4)) known.clear();        // (a sweep over shapes)
     for (const Known& k : known)
-        if (k.dev == dev && k.r == r && k.f32 == f32 && k.clusters == clusters && k.chain == chain && k.tiles == tiles && k.steps == steps) return k.plan;
+        if (k.dev == dev && k.r == r && k.f32 == f32 && k.push == push && k.tiles == tiles && k.steps == steps) return k.plan;
     const int K = f32 ? 32 : 64;
     GenK1Plan best;
     double least = 1e300;
@@ -121,29 +135,30 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
                     tune_knob("FLORA_GEN_WORKERS", workers, 8, 16) != workers)
                     continue;
                 GenK1Plan p;
-                if (!gen_k1_shape(p, f32, r, T, split > 1, workers == 16 ? 1 : 2, (steps + split - 1) / split)) continue;    // (registers: one CTA of sixteen warps)
+                if (!gen_k1_shape(p, f32, r, T, split > 1, push && split > 1, workers == 16 ? 1 : 2, (steps + split - 1) / split)) continue;    // (registers: one CTA of sixteen warps)
                 p.cluster = split;
                 p.workers = workers;
                 const int64_t groups = (tiles + T - 1) / T;
                 // (waves of row groups: what is left of a wave that is not full counts as one)
-                const int64_t resident = clusters ? gen_k1_resident(p, split) : (int64_t)sm_count() * p.per_sm;
-                const int64_t units = clusters ? groups : groups * split;
-                const double together = std::min<double>(p.per_sm, (double)(std::min(units, resident) * (clusters ? split : 1)) / sm_count());
+                const int64_t resident = push ? gen_k1_resident(p, split) : (int64_t)sm_count() * p.per_sm;
+                const int64_t units = push ? groups : groups * split;
+                const double together = std::min<double>(p.per_sm, (double)(std::min(units, resident) * (push ? split : 1)) / sm_count());
                 p.beside = 2 * groups * split <= (int64_t)sm_count() * p.per_sm;
                 double cost = gen_k1_cost(f32, r, T, workers, together, (units + resident - 1) / resident, (steps + split - 1) / split, split,
-                                          !clusters && (chain || r * K <= 2048) && p.beside && (steps + split - 1) / split <= p.a_slots);
-                if (clusters && split > 1 && !p.beside) cost += 1.25 * r * K;
+                                          !push && p.beside && (steps + split - 1) / split <= p.a_slots);
+                if (push && split > 1) cost += 200.0 + 25.0 * split + 30.0 * r + (p.beside ? 0.0 : 1.25 * r * K);
+                if (!push && split > 1) cost += gen_fold_cost(split, 128.0 * tiles * r * (2 * split + 2));
                 if (cost < least * 0.98) {
                     least = p.cost = cost;
                     best = p;
                 }
             }
     if (least > 1e299) {                                          // (one tile, no split, one CTA per SM fits every rank)
-        gen_k1_shape(best, f32, r, 1, false, 1, steps);
+        gen_k1_shape(best, f32, r, 1, false, false, 1, steps);
         best.workers = 16;
     }
-    if (known.size() >= 64) known.erase(known.begin());
-    known.push_back({dev, r, f32, clusters, chain, tiles, steps, best});
+    if (known.size() >= 2 * 64) known.erase(known.begin());
+    known.push_back({dev, r, f32, push, tiles, steps, best});
     return best;
 }
 
@@ -157,7 +172,6 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     cfg.blockDim = dim3((unsigned)gen_threads(WORKERS));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = st;
-    const int joining = p.ordered ? GEN_JOIN_ORDERED : b != 1.0f ? GEN_JOIN_SCALED : GEN_JOIN_PLAIN;
     // Tiles of A made before the wait: all slots where there is time for it, or where that takes half a microsecond a tile at most; one
     // otherwise, and the loads go out as soon as they may (1000 x 4097 at r = 64, all slots / one: 15.6 / 13.8 us; the ragged set of eight matrices at
     // r = 32, a compression: 11.2 / 13.5).
@@ -170,9 +184,9 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = p.cluster > 1 && joining != GEN_JOIN_PLAIN ? 2 : 1;
+    cfg.numAttrs = p.cluster > 1 && p.push ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, seeds, one, split, col0, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
-                              (int)p.sbs, p.g_slots, p.a_slots, p.cluster, joining, ahead);
+                              (int)p.sbs, p.g_slots, p.a_slots, p.cluster, p.push ? GEN_JOIN_PUSH : GEN_JOIN_SLICES, (int)p.land, ahead);
 }
 inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds,
                                         const GenMat& one, int split, int col0, int seed_base, int r, float a, float b, cudaStream_t st,
@@ -192,7 +206,7 @@ inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int cluste
 
 inline GenMat gen_mat(const flora_mat& big, const flora_mat& s)
 {
-    return GenMat{big.data, (float*)s.data, big.ld, s.ld, (int32_t)big.rows, (int32_t)big.cols};
+    return GenMat{big.data, (float*)s.data, big.ld, s.ld, (int32_t)big.rows, (int32_t)big.cols, nullptr};
 }
 // What the kernels index with 32 bits.
 inline bool gen_supported(const flora_mat& big) { return big.rows < (1ll << 31) - 1024 && big.cols < (1ll << 31) - 1024; }
@@ -205,9 +219,10 @@ inline bool gen_supported(const flora_mat& big) { return big.rows < (1ll << 31) 
 // r = 128 11.6 / 9.9, but 2816 x 1024 at r = 64 8.9 / 9.4 and 2048 x 2048 at r = 256 15.5 / 31.4.
 // A set of small matrices stops gaining a little earlier (its TMA kernels start once for all): `elements` of a set are counted
 // as 5/3.  (4 x 768 x 768 at r = 16: compress 11.1 / 7.0, decompress 6.6 / 6.0; 7 M elements at r = 16: 13.6 / 12.9 and 10.4 / 13.8.)
-// One matrix at a time, in a chain (with the TMA kernels and with these): bf16 1600 x 4800 at r = 16 12.2 / 9.2 (momentum 13.2 / 12.5), at r = 64 17.8 / 16.8, 6400 x 1600 at
-// r = 32 14.3 / 12.8, but 768 x 9216 10.8 / 11.5 and 4096 x 4096 at r = 64 17.3 / 22.0; 2048 x 2048 at r = 128 14.0 / 14.4; fp32 2048 x 2048 at r = 8 11.4 / 9.0, at
-// r = 128 21.3 / 19.7, but at r = 256 25.5 / 32.3 and 1024 x 4096 at r = 8 11.6 / 12.2.
+// One matrix at a time, in a chain (adding / momentum step with the TMA kernels, and with these): bf16 r = 16 1600 x 4800 12.3 / 13.2, 8.8, 2560 x 4096 12.7 / 14.2, 12.3; r = 32
+// 2560 x 4096 15.2 / 16.8, 14.5, 2048 x 5120 14.3 / 17.3, 14.2; r = 48 2048 x 4096 15.7 / 17.4, 13.8, but 2560 x 4096 15.6 / 17.4, 19.6 and 8192 x 1024 15.7 / 17.6,
+// 18.4; r = 64 2048 x 4096 16.7 / 18.4, 16.8, but 2560 x 4096 16.7 / 18.6, 19.3; fp32 2048 x 2048 at r = 8 11.7 / 12.7, 9.4, at r = 64 16.9 / 18.5, 16.4, at r = 128 21.2 / 23.1, 21.8, but at
+// r = 256 25.5 / 32.3.
 inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32, bool set)
 {
     const int knob = tune_knob("FLORA_GEN", -1, 0, 1);
@@ -216,7 +231,8 @@ inline bool gen_compress_quicker(int64_t elements, int64_t cols, int r, bool f32
     // split over a cluster, which only these kernels have.)
     if (f32) return (cols <= 3072 && elements <= (set || r > 128 ? 5 << 19 : 4 << 20)) || deterministic_flag().load();
     if (r > 64) return cols <= 4096 && elements <= 5 << 18;
-    return set ? cols <= 4096 && elements <= 4 << 20 : cols <= 5120 && elements <= 10 << 20;
+    if (set) return cols <= 4096 && elements <= 4 << 20;
+    return cols <= 5120 && (r <= 32 ? elements <= 10 << 20 : elements <= 8 << 20 && elements <= cols << 12);
 }
 // loose: TMA cannot address the sketch; the TMA kernel then reads a copy of its three parts.  (bf16 1224 x 4896 at r = 7 14.5 / 10.8, at r = 45 16.5 / 17.4, at r =
 // 255 28.7 / 49; 4096 x 11008 at r = 7 39.0 / 52.9.  Tight, 768 x 3072 at r = 96 14.4 / 11.2, 2048 x 2048 at r = 128 14.5 / 16.3.)
@@ -238,49 +254,33 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
     const int r = (int)S.cols;
     const int64_t pass = f32 ? GEN_F32_PASS_COLS : G.cols;
     const int64_t tiles = (G.rows + 127) / 128, steps = (std::min(G.cols, pass) + (f32 ? 31 : 63)) / (f32 ? 32 : 64);
-    const bool ordered = deterministic_flag().load() != 0;
-    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps, ordered, b == 1.0f);
-    // Rows that several CTAs add to are scaled by the launch itself, in clusters, or by a pass of its own in front of it, which takes one or two
-    // microseconds of a chain and the time of its bytes.  (Momentum step, in clusters / with a pass, us: 768 x 2304 at r = 16 5.5 / 6.4, but 2048 x 2048
-    // at r = 32 11.3 / 9, 3000 x 5001 at r = 18 in fp32 52.7 / 37.6.)
-    bool scale_first = false;
-    if (!ordered && p.cluster > 1 && b != 1.0f) {
-        const GenK1Plan c = gen_k1_choose(f32, r, tiles, steps, true, false);
-        scale_first = c.cost > p.cost + 3000.0 + 0.01 * (double)(G.rows * r);
-        if (!scale_first) p = c;
+    // Clusters, or single CTAs and a kernel that blends their sums in, by the cost model.  The former where bits are to be the same whatever memory is left,
+    // where the call is recorded into a graph and where there is no memory for the sums.
+    GenK1Plan p = gen_k1_choose(f32, r, tiles, steps, true);
+    GenMat mat = gen_mat(G, S);
+    void* sums = nullptr;
+    const int join = tune_knob("FLORA_GEN_JOIN", 0, 0, 2);
+    if (!deterministic_flag().load() && join != 1) {
+        const GenK1Plan q = gen_k1_choose(f32, r, tiles, steps, false);
+        if ((q.cost < p.cost || join == 2) && !capturing(st)) {
+            if (q.cluster == 1 || scratch_alloc(&sums, sizeof(float4) * (size_t)(q.cluster * fold_slice(G.rows, r)), st) == cudaSuccess) p = q;
+            else cudaGetLastError();
+        }
     }
-    const int64_t groups = (tiles + p.T - 1) / p.T;
+    mat.D = (float*)sums;
     p.aligned = gen_aligned(G);
-    p.ordered = ordered;
-    if (scale_first) {
-        TcMatrix one;
-        memset(&one, 0, sizeof(one));
-        one.S = (float*)S.data;
-        one.lds = S.ld;
-        one.n = (int32_t)G.rows;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(std::min(helper_blocks(G.rows * r), (unsigned)sm_count() * 6));
-        cfg.blockDim = dim3(256);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, scale_sketches_kernel<true>, (const TcMatrix*)nullptr, one, (const int*)nullptr, 0, r, b) != cudaSuccess) return FLORA_ERR_CUDA;
-        launches.fetch_add(1, std::memory_order_relaxed);
-        b = 1.0f;
-    }
     SeedTable table;
     table.s[0] = seed;
+    flora_status rc = FLORA_OK;
     int64_t col0 = 0;
     do {                                                          // (a matrix without columns: one launch, S <- b S)
-        const flora_status rc = gen_compress_launch(f32, p, (int)groups, nullptr, nullptr, table, gen_mat(G, S), p.cluster, (int)col0, 0, r, a,
-                                                    col0 ? 1.0f : b, st, launches);
-        if (rc) return rc;
+        rc = gen_compress_launch(f32, p, (int)((tiles + p.T - 1) / p.T), nullptr, nullptr, table, mat, p.cluster, (int)col0, 0, r, a, col0 ? 1.0f : b, st, launches);
+        if (rc == FLORA_OK && sums)
+            rc = fold_single(FoldMat{(float*)S.data, mat.D, S.ld, (int32_t)G.rows, 0, p.cluster, 0}, r, a, col0 ? 1.0f : b, sm_count(), st, launches);
         col0 += pass;
-    } while (col0 < G.cols);
-    return FLORA_OK;
+    } while (rc == FLORA_OK && col0 < G.cols);
+    if (sums && cudaFreeAsync(sums, st) != cudaSuccess && rc == FLORA_OK) rc = FLORA_ERR_CUDA;
+    return rc;
 }
 
 // Decompression: slabs of 128 columns for bf16 matrices whose rows move in 16-byte pieces, of 64 otherwise (an element-wise
@@ -358,13 +358,12 @@ struct GenSet {
     std::vector<GenMat> h_mats;                // one entry per matrix of the set (members filled in)
     GenMat* d_mats = nullptr;
     GenItem* d_k1 = nullptr;
-    GenItem* d_plain = nullptr;                // compression that only adds (b = 1): CTAs of a split form no clusters there
+    float* d_sums = nullptr;                   // compression by single CTAs (GEN_JOIN_SLICES): their sums, and the list of the kernel that blends them in
+    FoldItem* d_fold = nullptr;                // after each pass over columns
+    std::vector<int> fold_begin, pass_end;     // per pass: first item; the launches of the compression up to it
     GenK2Item* d_k2 = nullptr;
     int* d_share = nullptr;                    // decompression: per launch, the first item of every CTA and the end
     std::vector<int> begin, first_mat;         // compression: ranges of items per launch; decompression: where its table starts in d_share
-    std::vector<int> plain_begin, plain_first; // ... its ranges and first matrices
-    GenK1Plan plain;
-    std::vector<uint8_t> adds;                 // compression: launches behind the first columns of their matrices, which add to them
     std::vector<unsigned> grid;                // decompression: CTAs per launch
     int bn = 64;
     GenK1Plan plan;
@@ -377,7 +376,8 @@ inline void gen_set_free(GenSet& s)
 {
     if (s.d_mats) cudaFree(s.d_mats);
     if (s.d_k1) cudaFree(s.d_k1);
-    if (s.d_plain) cudaFree(s.d_plain);
+    if (s.d_sums) cudaFree(s.d_sums);
+    if (s.d_fold) cudaFree(s.d_fold);
     if (s.d_k2) cudaFree(s.d_k2);
     if (s.d_share) cudaFree(s.d_share);
     s = GenSet();
@@ -397,15 +397,15 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
     int count = 0;
-    auto launches_of = [&](std::vector<int>& begin, std::vector<int>& first_mat, auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
+    auto launches_of = [&](auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
         size_t u0 = 0;
         while (u0 < cuts.size()) {
             size_t u1 = u0;
             const int first = cuts[u0].mat;
             while (u1 < cuts.size() && cuts[u1].mat < first + SEEDS_PER_LAUNCH) ++u1;
             std::stable_sort(cuts.begin() + u0, cuts.begin() + u1, [](const Cut& x, const Cut& y) { return x.work > y.work; });
-            begin.push_back(count);
-            first_mat.push_back(first);
+            s.begin.push_back(count);
+            s.first_mat.push_back(first);
             for (size_t u = u0; u < u1; ++u, ++count) emit(cuts[u]);
             u0 = u1;
         }
@@ -428,7 +428,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         // One kind of CTA for the whole list: one tile, eight warps, two to an SM, where that fits (more tiles to share a tile of A
         // lose more to the longer step than they save: measured); per matrix as many CTAs along the columns as leave each about a
         // third of an SM's share of the work, and a single short wave on a small list.
-        const int per_sm = gen_k1_shape(s.plan, s.f32, s.r, 1, true, 2, GEN_A_SLOTS_MAX + 1) ? 2 : 1;
+        const int per_sm = gen_k1_shape(s.plan, s.f32, s.r, 1, true, true, 2, GEN_A_SLOTS_MAX + 1) ? 2 : 1;
         const int64_t share = std::max<int64_t>(2, total / (per_sm * sms * 3));
         std::vector<int> split(big.size(), 1);
         int cluster = 1;
@@ -481,30 +481,7 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         }
         most = tune_knob("FLORA_GEN_MOST", most, 1, GEN_MAX_SPLIT);
         cut_columns(most);
-        const int T = 1;
-        int64_t longest = 1;
-        for (int i : ids) longest = std::max(longest, (steps_of(i, 0) + split[i] - 1) / split[i]);
-        if (!gen_k1_shape(s.plan, s.f32, s.r, T, cluster > 1, per_sm, longest)) return FLORA_ERR_UNSUPPORTED;
-        s.plan.cluster = cluster;
-        s.plan.ordered = deterministic_flag().load() != 0;
-        std::vector<GenItem> items;
-        for (int64_t pass = 0; pass < passes; ++pass) {
-            cuts.clear();
-            for (int i : ids) {
-                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass), per = (int64_t)(cluster / split[i]) * T;
-                if (pass > 0 && steps == 0) continue;
-                for (int64_t t0 = 0; t0 < tiles; t0 += per)
-                    cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]),
-                                    {i, (int32_t)t0, split[i], s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0, 0}});
-            }
-            launches_of(s.begin, s.first_mat, [&](const Cut& c) { items.push_back(c.item); });
-            s.adds.resize(s.begin.size(), pass > 0 ? 1 : 0);
-        }
-        s.begin.push_back(count);
-        rc = upload(&s.d_k1, items, st);
-        if (rc || s.plan.ordered) return rc;
-        // Where nothing is to be scaled: single CTAs, and as many steps for each as make the shortest sum of waves.  (The ragged set of eight matrices
-        // at r = 32, a compression: 9.6 -> 8.4 us, in fp32 20.3 -> 11.7; 24 matrices of GPT-2-small shapes with an odd column 70.9 -> 65.4)
+        // Or single CTAs, and as many steps for each as make the shortest sum of waves.
         int64_t most_steps = 1;
         for (int i : ids) most_steps = std::max(most_steps, steps_of(i, 0));
         auto parts_of = [&](int i, int64_t per, int64_t pass) {
@@ -515,40 +492,83 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         int64_t best_per = most_steps;
         double least = 1e300;
         for (int64_t per = 1; per <= most_steps; per += std::max<int64_t>(1, per / 8)) {
-            int64_t ctas = 0, longest_run = 1;
+            int64_t ctas = 0, longest_run = 1, most_parts = 1;
+            double floats = 0;
             for (int i : ids) {
                 const int64_t parts = parts_of(i, per, 0);
                 ctas += (big[i].rows + 127) / 128 * parts;
                 longest_run = std::max(longest_run, (steps_of(i, 0) + parts - 1) / parts);
+                most_parts = std::max(most_parts, parts);
+                if (parts > 1) floats += (double)big[i].rows * s.r * (2 * parts + 2);
             }
             const int64_t slots = sms * per_sm, waves = (ctas + slots - 1) / slots;
             const double together = std::min<double>(per_sm, (double)ctas / sms);
-            const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, together, waves, longest_run, 2);
+            const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, together, waves, longest_run, 2) +
+                                (most_parts > 1 ? gen_fold_cost(most_parts, floats) : 0.0);
             if (cost < least * 0.98) {
                 least = cost;
                 best_per = per;
             }
         }
-        s.plain = s.plan;
-        int64_t longest_run = 1;
-        for (int i : ids) longest_run = std::max(longest_run, (steps_of(i, 0) + parts_of(i, best_per, 0) - 1) / parts_of(i, best_per, 0));
-        if (!gen_k1_shape(s.plain, s.f32, s.r, 1, true, per_sm, longest_run)) return FLORA_ERR_UNSUPPORTED;
-        s.plain.cluster = 1;
-        std::vector<GenItem> plain;
-        count = 0;
+        const int T = 1, join = tune_knob("FLORA_GEN_JOIN", 0, 0, 2);
+        // (Where two CTAs share an SM clusters do better than the model has it.  Model, clusters / slices in 1000 cycles, and us of a compression: ragged set of eight at r = 32
+        // 31 / 20 and 11.5 / 12.3, in fp32 44 / 24 and 21.9 / 18.5; three of 2000 to 5000 rows and odd columns at r = 32 30 / 18 and 21.4 / 17.1; 24 of
+        // GPT-2-small shapes and an odd column at r = 32 147 / 94 and 74 / 79; at r = 255, one CTA an SM, ragged set 74 / 54 and 78 / 54.)
+        bool slices = !deterministic_flag().load() && (join ? join == 2 : least < (per_sm == 2 ? 0.63 : 1.0) * shortest);
+        if (slices) {
+            size_t pieces = 0;
+            std::vector<size_t> at(big.size(), 0);
+            for (int i : ids) {
+                const int64_t parts = parts_of(i, best_per, 0);
+                at[i] = pieces;
+                if (parts > 1) pieces += (size_t)(parts * fold_slice(big[i].rows, s.r));
+            }
+            if (pieces && cudaMalloc((void**)&s.d_sums, sizeof(float4) * pieces) != cudaSuccess) {
+                cudaGetLastError();
+                s.d_sums = nullptr;
+                slices = false;                                   // no memory: clusters
+            } else {
+                for (int i : ids) s.h_mats[i].D = s.d_sums + 4 * at[i];
+            }
+        }
+        int64_t longest = 1;
+        for (int i : ids) {
+            const int64_t parts = slices ? parts_of(i, best_per, 0) : split[i];
+            longest = std::max(longest, (steps_of(i, 0) + parts - 1) / parts);
+        }
+        if (slices) cluster = 1;
+        if (!gen_k1_shape(s.plan, s.f32, s.r, T, true, cluster > 1, per_sm, longest)) return FLORA_ERR_UNSUPPORTED;
+        s.plan.cluster = cluster;
+        std::vector<GenItem> items;
+        std::vector<FoldItem> fold;
         for (int64_t pass = 0; pass < passes; ++pass) {
             cuts.clear();
+            s.fold_begin.push_back((int)fold.size());
             for (int i : ids) {
-                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass), parts = parts_of(i, best_per, pass);
+                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass);
+                const int32_t col0 = s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0;
                 if (pass > 0 && steps == 0) continue;
-                for (int64_t t0 = 0; t0 < tiles; ++t0)
-                    for (int64_t part = 0; part < parts; ++part)
-                        cuts.push_back({i, (steps + parts - 1) / parts, {i, (int32_t)t0, (int32_t)parts, s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0, (int32_t)part}});
+                if (slices) {
+                    const int64_t parts = parts_of(i, best_per, pass);
+                    for (int64_t t0 = 0; t0 < tiles; ++t0)
+                        for (int64_t part = 0; part < parts; ++part) cuts.push_back({i, (steps + parts - 1) / parts, {i, (int32_t)t0, (int32_t)parts, col0, (int32_t)part}});
+                    if (parts > 1)
+                        fold_cut(fold, FoldMat{s.h_mats[i].S, s.h_mats[i].D, s.h_mats[i].lds, (int32_t)big[i].rows, 0, (int32_t)parts, 0},
+                                 fold_slice(big[i].rows, s.r), fold_pieces_of_set(parts));
+                } else {
+                    const int64_t per = (int64_t)(cluster / split[i]) * T;
+                    for (int64_t t0 = 0; t0 < tiles; t0 += per)
+                        cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]), {i, (int32_t)t0, split[i], col0, 0}});
+                }
             }
-            launches_of(s.plain_begin, s.plain_first, [&](const Cut& c) { plain.push_back(c.item); });
+            launches_of([&](const Cut& c) { items.push_back(c.item); });
+            s.pass_end.push_back((int)s.begin.size());
         }
-        s.plain_begin.push_back(count);
-        return upload(&s.d_plain, plain, st);
+        s.begin.push_back(count);
+        s.fold_begin.push_back((int)fold.size());
+        rc = upload(&s.d_k1, items, st);
+        if (rc == FLORA_OK && slices) rc = upload(&s.d_mats, s.h_mats, st);
+        return rc ? rc : upload(&s.d_fold, fold, st);
     }
     // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
     bool aligned = true;
@@ -598,18 +618,17 @@ inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
 inline flora_status gen_set_compress(GenSet& s, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
     if (s.ready() && s.plan.aligned && !s.captured_aligned) s.captured_aligned = capturing(st);
-    if (b == 1.0f && s.d_plain) {
-        for (size_t l = 0; l + 1 < s.plain_begin.size(); ++l) {
-            const flora_status rc = gen_compress_launch(s.f32, s.plain, s.plain_begin[l + 1] - s.plain_begin[l], s.d_mats, s.d_plain + s.plain_begin[l],
-                                                        gen_seeds(s, seeds, s.plain_first[l]), GenMat{}, 1, 0, s.plain_first[l], s.r, a, b, st, launches);
+    size_t l = 0;
+    for (size_t pass = 0; pass < s.pass_end.size(); ++pass) {
+        const float scale = pass ? 1.0f : b;
+        for (; (int)l < s.pass_end[pass]; ++l) {
+            const flora_status rc = gen_compress_launch(s.f32, s.plan, s.begin[l + 1] - s.begin[l], s.d_mats, s.d_k1 + s.begin[l],
+                                                        gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, 0, s.first_mat[l], s.r, a, scale, st, launches);
             if (rc) return rc;
         }
-        return FLORA_OK;
-    }
-    for (size_t l = 0; l + 1 < s.begin.size(); ++l) {
-        const flora_status rc = gen_compress_launch(s.f32, s.plan, s.begin[l + 1] - s.begin[l], s.d_mats, s.d_k1 + s.begin[l],
-                                                    gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, 0, s.first_mat[l], s.r, a, s.adds[l] ? 1.0f : b, st,
-                                                    launches);
+        const int first = s.fold_begin[pass], items = s.fold_begin[pass + 1] - first;
+        if (items == 0) continue;
+        const flora_status rc = fold_launch(true, s.d_fold + first, items, FoldMat{}, 0, 0, s.r, a, scale, sm_count(), st, launches);
         if (rc) return rc;
     }
     return FLORA_OK;
@@ -642,7 +661,7 @@ inline flora_status gen_set_rebind(GenSet& s, const std::vector<flora_mat>& big,
         s.h_mats[i].big = big[i].data;
         aligned = aligned && gen_aligned(big[i]);
     }
-    s.plan.aligned = s.plain.aligned = aligned;
+    s.plan.aligned = aligned;
     return upload(&s.d_mats, s.h_mats, st);
 }
 

@@ -100,17 +100,11 @@ __device__ __forceinline__ void cluster_sync_some()
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// The two halves of that barrier, in the same manner.  relaxed: of threads whose writes another thread's release covers (it has met
-// them at a barrier of the CTA before).
+// The two halves of that barrier, in the same manner.
 __device__ __forceinline__ void cluster_arrive_release()
 {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_arrive_relaxed()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait_some()
 {
@@ -137,6 +131,13 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t ran
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
     return r;
 }
+// Stores 16 bytes into another CTA's shared memory, counted there on an mbarrier (both addresses from map_to_cta, of the same CTA).
+__device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar_cluster_addr)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar_cluster_addr)
+                 : "memory");
+}
 __device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -157,6 +158,29 @@ __device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t cluster_add
 // Waits on a barrier of this CTA on which other CTAs of the cluster (or the tensor core on their behalf) arrive.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) { return mbar_try_wait(bar, parity); }
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort) { return mbar_wait(bar, parity, abort); }
+// ... where what is waited for are stores by threads of the cluster (st_async_v4), which the wait acquires.  It goes on for its whole limit when another
+// thread of the CTA has given up: the stores come all the same.
+__device__ __forceinline__ bool mbar_wait_peers(uint32_t bar, uint32_t parity, volatile int* abort, unsigned long long limit_ns)
+{
+    unsigned long long t0 = 0;
+    for (uint32_t spin = 1;; ++spin) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (spin == 1) t0 = globaltimer();
+        if ((spin & 0xFF) == 0 && globaltimer() - t0 > limit_ns) {
+            *abort = 1;
+            atomicExch(&g_flora_error_word, 1);
+            return false;
+        }
+    }
+}
 // Bulk copy from this CTA's shared memory into a peer CTA's shared memory; the bytes are counted on the
 // peer's mbarrier.  Both addresses are 16-byte aligned, the size a multiple of 16.
 __device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster_addr, uint32_t src_local_addr, uint32_t bytes, uint32_t bar_cluster_addr)
@@ -219,12 +243,6 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-// Counts this thread at such a barrier without waiting there.
-__device__ __forceinline__ void named_barrier_arrive(uint32_t id, uint32_t nthreads)
-{
-    __syncwarp();
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 template <int N>
 __device__ __forceinline__ void tma_store_wait_read()
@@ -401,7 +419,6 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
 {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
-__device__ __forceinline__ void red_add(float* p, float a) { asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory"); }
 // 16-byte asynchronous copy global -> shared by the calling thread (both addresses 16-byte aligned), grouped and
 // awaited per thread.
 __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src)

@@ -23,7 +23,7 @@ def _projection(G, r, seed):
 
 
 def _check(states, gradients, calls, ratio, sums):
-    """calls: (beta or None, function); sums: error that the products' sums may have, of a product."""
+    """calls: (beta or None, function); sums: error that the products' sums may have, of a product, by its columns."""
     products = [G.double() @ _projection(G, S.shape[1], 40 + i).T for i, (G, S) in enumerate(zip(gradients, states))]
     start = [(torch.randn_like(S) * (ratio * p.norm().item() / p.numel() ** 0.5)) for S, p in zip(states, products)]
     for beta, call in calls:
@@ -33,7 +33,9 @@ def _check(states, gradients, calls, ratio, sums):
         a, b = (1.0, 1.0) if beta is None else (1.0 - torch.tensor(beta).item(), torch.tensor(beta).item())
         for i, (S, s, p) in enumerate(zip(states, start, products)):
             want = b * s.double() + a * p
-            assert ((S.double() - want).norm() <= 3e-8 * want.norm() + sums * a * p.norm()).item(), (beta, ratio, i)
+            m = gradients[i].shape[1]
+            launches = -(-m // 36864) if gradients[i].dtype == torch.float32 else 1        # (each takes so many columns of an fp32 matrix at most)
+            assert ((S.double() - want).norm() <= 3e-8 * launches ** 0.5 * want.norm() + sums(m) * a * p.norm()).item(), (beta, ratio, i)
     assert fb.flora_device_status() == 0
 
 
@@ -55,10 +57,32 @@ def _set(shapes, r, dtype, offset, ratio, sums):
 @pytest.mark.parametrize("ratio", [1, 1000])
 @pytest.mark.parametrize("n,m,r,offset", [(4096, 11008, 7, 0), (2048, 4096, 128, 1), (1224, 4896, 255, 0)])
 def test_sketches_that_tma_cannot_address(n, m, r, offset, ratio):
-    _single(n, m, r, "bf16", offset, ratio, 7e-8 * m / 64 / 8)
+    _single(n, m, r, "bf16", offset, ratio, lambda m: 7e-8 * m / 64 / 8)
 
 
 @pytest.mark.parametrize("ratio", [1, 1000])
 @pytest.mark.parametrize("r,offset", [(31, 0), (101, 0), (32, 1)])
 def test_sets_of_such_sketches(r, offset, ratio):
-    _set([(1192, 3576), (1192, 1192), (1192, 4768), (4768, 1192)] * 2, r, "bf16", offset, ratio, 7e-8 * 4768 / 64 / 2)
+    _set([(1192, 3576), (1192, 1192), (1192, 4768), (4768, 1192)] * 2, r, "bf16", offset, ratio, lambda m: 7e-8 * 4768 / 64 / 2)
+
+
+# The general kernels, by clusters and by single CTAs whose sums a second kernel adds up: what plain fp32 sums are off by (fp32), or 7e-8 per step of a CTA's part (bf16:
+# four parts at least where there are more than 512 columns, two in a set).  One row group and many, rows and ranks off the pieces of four, fp32 rows of two launches.
+def _general(dtype, parts):
+    return (lambda m: 1.8e-8 * max(m, 64) ** 0.5) if dtype == "f32" else (lambda m: 7e-8 * (m / 64 / (parts if m > 512 else 1) + 1))
+
+
+@pytest.mark.parametrize("ratio", [1, 1000])
+@pytest.mark.parametrize("n,m,r,dtype", [(512, 512, 8, "f32"), (300, 700, 33, "f32"), (3000, 5001, 18, "f32"), (3456, 145, 256, "f32"), (200, 40001, 24, "f32"),
+                                         (2048, 2048, 64, "f32"), (256, 384, 32, "bf16"), (95, 3057, 17, "bf16"), (1000, 4097, 64, "bf16"), (2048, 2048, 32, "bf16"),
+                                         (129, 520, 255, "bf16"), (3000, 2001, 128, "bf16")])
+def test_general_kernels(n, m, r, dtype, ratio):
+    _single(n, m, r, dtype, 0, ratio, _general(dtype, 4))
+
+
+@pytest.mark.parametrize("ratio", [1, 1000])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("r", [8, 33, 255])
+@pytest.mark.parametrize("shapes", [[(130, 70), (1000, 515), (257, 4097), (128, 64), (4000, 129), (768, 768), (10, 768), (50, 3072)], [(127, 4100), (64, 40001)]])
+def test_sets_of_general_kernels(shapes, r, dtype, ratio):
+    _set(shapes, r, dtype, 0, ratio, _general(dtype, 2))
