@@ -858,8 +858,8 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     // release_later: the caller frees the call's scratch (stream-ordered) itself, after it has put more work behind the
     // last kernel; nothing then stands between that kernel and the caller's next launch
     // ordered: set to true where the call's first work on the stream waits for everything before it (the table copy of several
-    // matrices).  One matrix has no such work: its gram kernel is launched early and waits itself, after its successor may have
-    // started, so a kernel behind the transfer may not take for granted that anything before the call is done.
+    // matrices; the clearing of T in front of the kernels of a few).  One matrix has no such work: its gram kernel is launched early and waits
+    // itself, after its successor may have started, so a kernel behind the transfer may not take for granted that anything before the call is done.
     if (release_later) *release_later = nullptr;
     if (ordered) *ordered = false;
     if (jobs.empty()) return FLORA_OK;
@@ -1036,6 +1036,9 @@ inline flora_status transfer_tc(std::vector<GramJob>& jobs, int r, float a, floa
     GramArg<GRAM_ONE> one;
     one.j[0] = jobs[0];
     if (list) {
+        // (T has been cleared; parts are one matrix's.  Only at low ranks: a compression that starts early takes SMs from the apply kernel, which in fp32 arithmetic is the
+        // longer one at high ranks.  Resampled step of three 2048 x 4096 and a small matrix, late / early: r = 32 42.2 / 38.0, r = 64 50.0 / 54.4, r = 128 74.6 / 82.7 us)
+        if (ordered) *ordered = ok && r <= 32;
         std::copy(jobs.begin(), jobs.end(), by_value.j);
         ok = ok && raise_smem_limit<gram_tc_kernel<GRAM_LIST>>();
         if (ok && n_items)

@@ -253,6 +253,36 @@ def test_resampled_step_of_one_matrix_waits_for_the_writer_of_its_gradient(n, m,
     assert fb.flora_device_status() == 0
 
 
+@pytest.mark.parametrize("r", [32, 128])
+def test_resampled_step_of_a_few_matrices_waits_for_the_writers_of_their_gradients(r):
+    """The same with a few matrices, one of which TMA cannot address: their transfer starts with the clearing of its scratch, which waits for
+    all earlier work, so that the compression behind it may read G before its own wait."""
+    shapes = [(2048, 4224), (130, 515), (40, 70)]
+    G = [torch.zeros(n, m, device=DEV, dtype=torch.bfloat16) for n, m in shapes]
+    D = [torch.randn(n, r, device=DEV) for n, _ in shapes]
+    M = [torch.randn(n, r, device=DEV) for n, _ in shapes]
+    M0 = [x.clone() for x in M]
+    fset, seeds = fb.FloraSet(G, None, M), [[s + i for i in range(len(shapes))] for s in (21, 31)]
+    for i in range(len(shapes)):
+        fb.flora_decompress_apply(G[i], D[i], 7, 0.0, 1.0)            # (plans)
+    for k in range(4):
+        for i in range(len(shapes)):
+            G[i].zero_()
+            M[i].copy_(M0[i])
+        for i in reversed(range(len(shapes))):
+            fb.flora_decompress_apply(G[i], D[i], 8 + k, -1.0, 1.0)   # G <- D A, the largest one last
+        fset.momentum_step_resampled(0.5, *seeds)
+        for i, (n, m) in enumerate(shapes):
+            want = M0[i].clone()
+            fb.flora_resample_transfer(want, m, "bf16", seeds[0][i], seeds[1][i])
+            torch.cuda.synchronize()
+            fb.flora_momentum_step(G[i], want, 0.5, seeds[1][i])
+            # (a single transfer reads sketches as tf32, whose ten bits are cut off: a product loses less than 2^-9)
+            assert rel_err(M[i].cpu().numpy(), want.cpu().numpy()) <= 2.0 ** -9, (k, i)
+    fset.close()
+    assert fb.flora_device_status() == 0
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_a_set_may_be_used_from_any_stream_as_soon_as_it_exists(dtype):
     """The tables of a set are copied behind whatever the default stream holds; a stream that is not ordered to it may use the set
