@@ -218,8 +218,8 @@ flora_status compress_single(const flora_mat* G, flora_mat* S, uint64_t seed, fl
             // (sums as short as those of the general kernels: the tensor core truncates them, 7e-8 of a sum lost per step of 64 columns)
             const int64_t steps = (G->cols + 63) / 64, parts = gen_k1_choose(false, r, (G->rows + 127) / 128, steps, true).cluster;
             flora_status rc = tc_compress_single(G, &sums, seed, 1.0f, 0.0f, st, g_launches, (steps + parts - 1) / parts);
-            const FoldMat fold{(float*)S->data, (const float*)sums.data, S->ld, (int32_t)S->rows, (int32_t)sums.ld, 1, 0};
-            if (rc == FLORA_OK) rc = fold_single(fold, r, a, b, sm_count(), st, g_launches);
+            const FoldMat fold{(float*)S->data, 0, S->ld, (int32_t)S->rows, (int32_t)sums.ld, 1, 0};
+            if (rc == FLORA_OK) rc = fold_single((const float*)sums.data, fold, r, a, b, sm_count(), st, g_launches);
             if (cudaFreeAsync(sums.data, st) != cudaSuccess && rc == FLORA_OK) rc = FLORA_ERR_CUDA;
             return rc;
         }
@@ -326,7 +326,7 @@ static flora_status set_build_beside(flora_set* s, const std::vector<uint8_t>& u
     float* D = s->d_sums;
     for (int i : ids) {
         flora_mat& m = S[(size_t)i];
-        fold_cut(fold, FoldMat{(float*)m.data, D, m.ld, (int32_t)m.rows, ld, 1, 0}, m.rows, fold_rows(rows, s->r, sm_count()));
+        fold_cut(fold, FoldMat{(float*)m.data, D - s->d_sums, m.ld, (int32_t)m.rows, ld, 1, 0}, m.rows, fold_rows(rows, s->r, sm_count()));
         m.data = D;
         m.ld = ld;
         D += m.rows * ld;
@@ -652,9 +652,9 @@ static flora_status beside_compress(flora_set* set, const uint64_t* seeds, float
     if (!tc.compress_ready || tc.off_tma) return tma_compress(set, tc, seeds, a, b, st, false);
     const bool alone = (size_t)set->beside == tc.members.size();
     flora_status rc = FLORA_OK;
-    if (!alone && b != 0.0f) rc = tc_scale_launch<false>(tc.d_mats, TcMatrix{}, set->d_beside, (size_t)set->beside, set->beside_most, set->r, 0.0f, true, st, g_launches);
+    if (!alone && b != 0.0f) rc = tc_scale_launch<false>(tc.d_mats, TcMatrix{}, set->d_beside, (size_t)set->beside, set->beside_most, fold_ld(set->r), 0.0f, true, st, g_launches);
     if (rc == FLORA_OK) rc = tc_set_compress(tc, seeds, a, alone ? 0.0f : b, st, g_launches, behind_own_transfer);
-    return rc ? rc : fold_launch(false, set->d_fold, set->fold_items, FoldMat{}, 0, 0, set->r, 1.0f, b, sm_count(), st, g_launches);
+    return rc ? rc : fold_launch(false, set->d_sums, set->d_fold, set->fold_items, FoldMat{}, 0, 0, set->r, 1.0f, b, sm_count(), st, g_launches);
 }
 
 // behind_own_transfer: the work before this call on the stream is the library's own transfer, which does not touch G and whose first

@@ -19,9 +19,10 @@ namespace flora {
 
 struct FoldMat {
     float* S;
-    // One part: rows of ldd floats, 16-byte aligned.  More: slices of fold_slice float4 each, as [row / 8][piece of four columns][row % 8], so that the
-    // threads that write them (a row each) and those that add them up (neighbouring rows, then pieces) touch whole lines.
-    const float* D;
+    // Where its sums start in the scratch, in floats.  One part: rows of ldd floats, 16-byte aligned.  More: slices of fold_slice float4 each, as
+    // [row / 8][piece of four columns][row % 8], so that the threads that write them (a row each) and those that add them up (neighbouring rows, then
+    // pieces) touch whole lines.
+    int64_t at;
     int64_t lds;
     int32_t n, ldd, parts, pad;
 };
@@ -82,9 +83,10 @@ __device__ __forceinline__ void store_some(float* p, const float4& v, bool vec, 
 // sixteen 5.4; few enough registers for a block to wait beside the compression's CTAs, and eight parts at a time, 700 x 2001 at r = 255 19 to 23, this way 16.5 (there it takes the
 // place of the compression behind it); four threads to a piece, a set of eight matrices at r = 255 86, this way 54; slices stored row by row, 3000 x 5001 at r = 128 54.7, as
 // lines of eight rows 47.
+// (sums: not __restrict__, which would let it be read through a path that does not see what was written since the kernel started.)
 template <bool SINGLE, bool SLICES>
-__global__ void __launch_bounds__(FOLD_THREADS, 1) fold_sums_kernel(const FoldItem* __restrict__ items, int n_items, const __grid_constant__ FoldMat single,
-                                                                        int64_t total_single, int count_single, int r, float a, float b)
+__global__ void __launch_bounds__(FOLD_THREADS, 1) fold_sums_kernel(const float* sums, const FoldItem* __restrict__ items, int n_items,
+                                                                        const __grid_constant__ FoldMat single, int64_t total_single, int count_single, int r, float a, float b)
 {
     ptx::grid_launch_dependents();
     const int tid = threadIdx.x, quads = (r + 3) >> 2;
@@ -103,7 +105,7 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) fold_sums_kernel(const FoldIt
         if (SLICES) {
             const int64_t slice = fold_slice(mat.n, r), row8 = item.first / (8 * quads);
             const int e_first = (int)(item.first - row8 * 8 * quads);
-            const float4* const D = reinterpret_cast<const float4*>(mat.D) + item.first;
+            const float4* const D = reinterpret_cast<const float4*>(sums + mat.at) + item.first;
             for (int e = tid; e < item.count; e += FOLD_THREADS) {
                 const int x = e_first + e, g = x / (8 * quads), j = 4 * ((x - 8 * quads * g) >> 3);
                 const int64_t row = (row8 + g) * 8 + (x & 7);
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) fold_sums_kernel(const FoldIt
                     const int e = e0 + FOLD_THREADS * u, i = e / quads, j = 4 * (e - i * quads);
                     s[u] = mat.S + (item.first + i) * mat.lds + j;
                     o[u] = load_some(s[u], true, b != 0.0f && e < total);
-                    v[u] = load_some(mat.D + (item.first + i) * mat.ldd + j, true, e < total);
+                    v[u] = load_some(sums + mat.at + (item.first + i) * mat.ldd + j, true, e < total);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) store_some(s[u], fold_blend(v[u], o[u], a, b), true, e0 + FOLD_THREADS * u < total);
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) fold_sums_kernel(const FoldIt
                     const int e = e0 + FOLD_THREADS * u, i = e / r, j = e - i * r;
                     s[u] = mat.S + (item.first + i) * mat.lds + j;
                     o[u] = b != 0.0f && e < total ? *s[u] : 0.0f;
-                    v[u] = e < total ? mat.D[(item.first + i) * mat.ldd + j] : 0.0f;
+                    v[u] = e < total ? sums[mat.at + (item.first + i) * mat.ldd + j] : 0.0f;
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) fold_sums_kernel(const FoldIt
 
 // Launched early: it waits itself, and what follows waits for it.  items: of matrices of a set, all of one kind; otherwise the one matrix, cut into
 // items of `count` of its `total` rows or pieces.
-inline flora_status fold_launch(bool slices, const FoldItem* items, int n_items, const FoldMat& one, int64_t total, int count, int r, float a, float b, int sms,
+inline flora_status fold_launch(bool slices, const float* sums, const FoldItem* items, int n_items, const FoldMat& one, int64_t total, int count, int r, float a, float b, int sms,
                                 cudaStream_t st, std::atomic<uint64_t>& launches)
 {
     cudaLaunchConfig_t cfg = {};
@@ -169,17 +171,17 @@ inline flora_status fold_launch(bool slices, const FoldItem* items, int n_items,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, items, n_items, one, total, count, r, a, b); };
+    auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, sums, items, n_items, one, total, count, r, a, b); };
     const cudaError_t e = items ? (slices ? go(fold_sums_kernel<false, true>) : go(fold_sums_kernel<false, false>))
                                 : (slices ? go(fold_sums_kernel<true, true>) : go(fold_sums_kernel<true, false>));
     launches.fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? FLORA_OK : FLORA_ERR_CUDA;
 }
-inline flora_status fold_single(const FoldMat& one, int r, float a, float b, int sms, cudaStream_t st, std::atomic<uint64_t>& launches)
+inline flora_status fold_single(const float* sums, const FoldMat& one, int r, float a, float b, int sms, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
     const bool slices = one.parts > 1;
     const int64_t total = slices ? fold_slice(one.n, r) : one.n, count = slices ? fold_pieces(total) : fold_rows(total, r, sms);
-    return fold_launch(slices, nullptr, (int)((total + count - 1) / count), one, total, (int)count, r, a, b, sms, st, launches);
+    return fold_launch(slices, sums, nullptr, (int)((total + count - 1) / count), one, total, (int)count, r, a, b, sms, st, launches);
 }
 
 }  // namespace flora

@@ -27,7 +27,7 @@ struct GenMat {            // a matrix with its sketch
     float* S;
     int64_t ld, lds;
     int32_t n, m;
-    float* D;              // compression: scratch for the sums of its parts (GEN_JOIN_SLICES)
+    int64_t slices;        // compression: where the sums of its parts start in the scratch (GEN_JOIN_SLICES, in pieces of four)
 };
 struct GenItem {           // compression: one cluster, or one CTA of a split whose CTAs form none
     int32_t mat;
@@ -147,7 +147,7 @@ __device__ __forceinline__ GenRows gen_rows(int tiles, int part, int split)
 // themselves and the small ones one or two others; the blocks are added up when they are read back.
 template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
 __global__ void __launch_bounds__(gen_threads(WORKERS), WORKERS == 8 ? 2 : 1)
-gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, const __grid_constant__ SeedTable seeds,
+gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__ items, float4* sums, const __grid_constant__ SeedTable seeds,
                     const __grid_constant__ GenMat single, int single_split, int single_col0, int seed_base, int r, float scale, float a, float b, int T, int sbs,
                     int g_slots, int a_slots, int cluster, int joining, int land, int ahead)
 {
@@ -590,7 +590,7 @@ gen_compress_kernel(const GenMat* __restrict__ mats, const GenItem* __restrict__
         } else {
             // (laid out for the kernel that adds the slices up, in lines of eight rows' pieces: FoldMat)
             const int quads = (r + 3) >> 2;
-            float4* const slice = reinterpret_cast<float4*>(mat.D) + (int64_t)part * fold_slice(mat.n, r);
+            float4* const slice = sums + mat.slices + (int64_t)part * fold_slice(mat.n, r);
             for (int t = 0; t < tiles; ++t) {
                 const int row = (tile0 + t) * 128 + (warp & 3) * 32 + lane;
                 float4* const dst = slice + (int64_t)(row >> 3) * quads * 8 + (row & 7);

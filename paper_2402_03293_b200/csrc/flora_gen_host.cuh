@@ -90,6 +90,8 @@ inline double gen_k1_cost(bool f32, int r, int T, int workers, double together, 
 // L2 takes and gives some 8 TB/s.  (In a chain, without and with it, us: 512 x 512 at r = 8 in fp32, sixteen parts, 3.6 and 5.6; the ragged set of eight matrices at r = 32, 33 parts
 // at most, 8.3 and 13.4, in fp32, 64 parts, 11.7 and 17.8.)
 inline double gen_fold_cost(int64_t parts, double floats) { return 2000.0 + 2300.0 * (double)((parts + 15) / 16) + 1.9 / 8000.0 * 4.0 * floats; }
+// Sums beside the sketches stay in L2 (126 MB), and in what the scratch pool keeps.
+constexpr size_t GEN_SUMS_MAX_BYTES = 48ull << 20;
 // Clusters of `size` CTAs of the compression kernel that can be resident (asked once per kind of launch: the kernel's variants
 // need the same registers, so one stands for all).
 inline int gen_k1_resident(const GenK1Plan& p, int size)
@@ -147,6 +149,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
                 double cost = gen_k1_cost(f32, r, T, workers, together, (units + resident - 1) / resident, (steps + split - 1) / split, split,
                                           !push && p.beside && (steps + split - 1) / split <= p.a_slots);
                 if (push && split > 1) cost += 200.0 + 25.0 * split + 30.0 * r + (p.beside ? 0.0 : 1.25 * r * K);
+                if (!push && split > 1 && 128.0 * tiles * r * 4 * split > (double)GEN_SUMS_MAX_BYTES) continue;
                 if (!push && split > 1) cost += gen_fold_cost(split, 128.0 * tiles * r * (2 * split + 2));
                 if (cost < least * 0.98) {
                     least = p.cost = cost;
@@ -163,7 +166,7 @@ inline GenK1Plan gen_k1_choose(bool f32, int r, int64_t tiles, int64_t steps, bo
 }
 
 template <bool SINGLE, bool F32, bool ALIGNED, int WORKERS>
-inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds, const GenMat& one,
+inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, float4* sums, const SeedTable& seeds, const GenMat& one,
                                  int split, int col0, int seed_base, int r, float a, float b, cudaStream_t st)
 {
     if (!raise_smem_limit<gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>>(true)) return cudaErrorInvalidValue;
@@ -185,14 +188,14 @@ inline cudaError_t gen_launch_k1(const GenK1Plan& p, int clusters, const GenMat*
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.cluster > 1 && p.push ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, seeds, one, split, col0, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
+    return cudaLaunchKernelEx(&cfg, gen_compress_kernel<SINGLE, F32, ALIGNED, WORKERS>, mats, items, sums, seeds, one, split, col0, seed_base, r, 1.0f / sqrtf((float)r), a, b, p.T,
                               (int)p.sbs, p.g_slots, p.a_slots, p.cluster, p.push ? GEN_JOIN_PUSH : GEN_JOIN_SLICES, (int)p.land, ahead);
 }
-inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, const SeedTable& seeds,
+inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int clusters, const GenMat* mats, const GenItem* items, float4* sums, const SeedTable& seeds,
                                         const GenMat& one, int split, int col0, int seed_base, int r, float a, float b, cudaStream_t st,
                                         std::atomic<uint64_t>& launches)
 {
-    auto go = [&](auto launch) { return launch(p, clusters, mats, items, seeds, one, split, col0, seed_base, r, a, b, st); };
+    auto go = [&](auto launch) { return launch(p, clusters, mats, items, sums, seeds, one, split, col0, seed_base, r, a, b, st); };
     cudaError_t e;
 #define FLORA_GEN_K1(SINGLE, F32, ALIGNED) (p.workers == 16 ? go(gen_launch_k1<SINGLE, F32, ALIGNED, 16>) : go(gen_launch_k1<SINGLE, F32, ALIGNED, 8>))
     if (items) e = f32 ? (p.aligned ? FLORA_GEN_K1(false, true, true) : FLORA_GEN_K1(false, true, false))
@@ -206,7 +209,7 @@ inline flora_status gen_compress_launch(bool f32, const GenK1Plan& p, int cluste
 
 inline GenMat gen_mat(const flora_mat& big, const flora_mat& s)
 {
-    return GenMat{big.data, (float*)s.data, big.ld, s.ld, (int32_t)big.rows, (int32_t)big.cols, nullptr};
+    return GenMat{big.data, (float*)s.data, big.ld, s.ld, (int32_t)big.rows, (int32_t)big.cols, 0};
 }
 // What the kernels index with 32 bits.
 inline bool gen_supported(const flora_mat& big) { return big.rows < (1ll << 31) - 1024 && big.cols < (1ll << 31) - 1024; }
@@ -257,7 +260,6 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
     // Clusters, or single CTAs and a kernel that blends their sums in, by the cost model.  The former where bits are to be the same whatever memory is left,
     // where the call is recorded into a graph and where there is no memory for the sums.
     GenK1Plan p = gen_k1_choose(f32, r, tiles, steps, true);
-    GenMat mat = gen_mat(G, S);
     void* sums = nullptr;
     const int join = tune_knob("FLORA_GEN_JOIN", 0, 0, 2);
     if (!deterministic_flag().load() && join != 1) {
@@ -267,16 +269,15 @@ inline flora_status gen_compress_single(const flora_mat& G, const flora_mat& S, 
             else cudaGetLastError();
         }
     }
-    mat.D = (float*)sums;
     p.aligned = gen_aligned(G);
     SeedTable table;
     table.s[0] = seed;
     flora_status rc = FLORA_OK;
     int64_t col0 = 0;
     do {                                                          // (a matrix without columns: one launch, S <- b S)
-        rc = gen_compress_launch(f32, p, (int)((tiles + p.T - 1) / p.T), nullptr, nullptr, table, mat, p.cluster, (int)col0, 0, r, a, col0 ? 1.0f : b, st, launches);
+        rc = gen_compress_launch(f32, p, (int)((tiles + p.T - 1) / p.T), nullptr, nullptr, (float4*)sums, table, gen_mat(G, S), p.cluster, (int)col0, 0, r, a, col0 ? 1.0f : b, st, launches);
         if (rc == FLORA_OK && sums)
-            rc = fold_single(FoldMat{(float*)S.data, mat.D, S.ld, (int32_t)G.rows, 0, p.cluster, 0}, r, a, col0 ? 1.0f : b, sm_count(), st, launches);
+            rc = fold_single((const float*)sums, FoldMat{(float*)S.data, 0, S.ld, (int32_t)G.rows, 0, p.cluster, 0}, r, a, col0 ? 1.0f : b, sm_count(), st, launches);
         col0 += pass;
     } while (rc == FLORA_OK && col0 < G.cols);
     if (sums && cudaFreeAsync(sums, st) != cudaSuccess && rc == FLORA_OK) rc = FLORA_ERR_CUDA;
@@ -358,9 +359,14 @@ struct GenSet {
     std::vector<GenMat> h_mats;                // one entry per matrix of the set (members filled in)
     GenMat* d_mats = nullptr;
     GenItem* d_k1 = nullptr;
-    float* d_sums = nullptr;                   // compression by single CTAs (GEN_JOIN_SLICES): their sums, and the list of the kernel that blends them in
-    FoldItem* d_fold = nullptr;                // after each pass over columns
-    std::vector<int> fold_begin, pass_end;     // per pass: first item; the launches of the compression up to it
+    // compression by single CTAs (GEN_JOIN_SLICES), where that is the quicker: their list, that of the kernel that blends their sums in after each pass over
+    // columns, and the bytes of the sums, which are borrowed for every call (made with the set they took a millisecond of its creation, and more)
+    GenItem* d_alone = nullptr;
+    FoldItem* d_fold = nullptr;
+    size_t sums_bytes = 0;
+    GenK1Plan alone;
+    std::vector<int> alone_begin, alone_first, alone_pass_end;
+    std::vector<int> fold_begin, pass_end;     // per pass: first item; the launches up to its end
     GenK2Item* d_k2 = nullptr;
     int* d_share = nullptr;                    // decompression: per launch, the first item of every CTA and the end
     std::vector<int> begin, first_mat;         // compression: ranges of items per launch; decompression: where its table starts in d_share
@@ -376,7 +382,7 @@ inline void gen_set_free(GenSet& s)
 {
     if (s.d_mats) cudaFree(s.d_mats);
     if (s.d_k1) cudaFree(s.d_k1);
-    if (s.d_sums) cudaFree(s.d_sums);
+    if (s.d_alone) cudaFree(s.d_alone);
     if (s.d_fold) cudaFree(s.d_fold);
     if (s.d_k2) cudaFree(s.d_k2);
     if (s.d_share) cudaFree(s.d_share);
@@ -397,15 +403,15 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
     struct Cut { int mat; int64_t work; GenItem item; };
     std::vector<Cut> cuts;
     int count = 0;
-    auto launches_of = [&](auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
+    auto launches_of = [&](std::vector<int>& begin, std::vector<int>& first_mat, auto emit) {         // ranges of at most SEEDS_PER_LAUNCH consecutive matrices, the largest items first
         size_t u0 = 0;
         while (u0 < cuts.size()) {
             size_t u1 = u0;
             const int first = cuts[u0].mat;
             while (u1 < cuts.size() && cuts[u1].mat < first + SEEDS_PER_LAUNCH) ++u1;
             std::stable_sort(cuts.begin() + u0, cuts.begin() + u1, [](const Cut& x, const Cut& y) { return x.work > y.work; });
-            s.begin.push_back(count);
-            s.first_mat.push_back(first);
+            begin.push_back(count);
+            first_mat.push_back(first);
             for (size_t u = u0; u < u1; ++u, ++count) emit(cuts[u]);
             u0 = u1;
         }
@@ -489,18 +495,22 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
             if (s.f32) per = std::min(per, gen_f32_chain(steps_of(i, 0)));
             return std::max<int64_t>(1, std::min<int64_t>(GEN_MAX_PARTS, (steps + per - 1) / per));
         };
-        int64_t best_per = most_steps;
+        int64_t best_per = 0;
         double least = 1e300;
         for (int64_t per = 1; per <= most_steps; per += std::max<int64_t>(1, per / 8)) {
             int64_t ctas = 0, longest_run = 1, most_parts = 1;
-            double floats = 0;
+            double floats = 0, pieces = 0;
             for (int i : ids) {
                 const int64_t parts = parts_of(i, per, 0);
                 ctas += (big[i].rows + 127) / 128 * parts;
                 longest_run = std::max(longest_run, (steps_of(i, 0) + parts - 1) / parts);
                 most_parts = std::max(most_parts, parts);
-                if (parts > 1) floats += (double)big[i].rows * s.r * (2 * parts + 2);
+                if (parts > 1) {
+                    floats += (double)big[i].rows * s.r * (2 * parts + 2);
+                    pieces += (double)(parts * fold_slice(big[i].rows, s.r));
+                }
             }
+            if (16.0 * pieces > (double)GEN_SUMS_MAX_BYTES) continue;
             const int64_t slots = sms * per_sm, waves = (ctas + slots - 1) / slots;
             const double together = std::min<double>(per_sm, (double)ctas / sms);
             const double cost = gen_k1_cost(s.f32, s.r, 1, s.plan.workers, together, waves, longest_run, 2) +
@@ -514,61 +524,65 @@ inline flora_status gen_set_build(GenSet& s, int kind, const std::vector<flora_m
         // (Where two CTAs share an SM clusters do better than the model has it.  Model, clusters / slices in 1000 cycles, and us of a compression: ragged set of eight at r = 32
         // 31 / 20 and 11.5 / 12.3, in fp32 44 / 24 and 21.9 / 18.5; three of 2000 to 5000 rows and odd columns at r = 32 30 / 18 and 21.4 / 17.1; 24 of
         // GPT-2-small shapes and an odd column at r = 32 147 / 94 and 74 / 79; at r = 255, one CTA an SM, ragged set 74 / 54 and 78 / 54.)
-        bool slices = !deterministic_flag().load() && (join ? join == 2 : least < (per_sm == 2 ? 0.63 : 1.0) * shortest);
-        if (slices) {
-            size_t pieces = 0;
-            std::vector<size_t> at(big.size(), 0);
-            for (int i : ids) {
-                const int64_t parts = parts_of(i, best_per, 0);
-                at[i] = pieces;
-                if (parts > 1) pieces += (size_t)(parts * fold_slice(big[i].rows, s.r));
-            }
-            if (pieces && cudaMalloc((void**)&s.d_sums, sizeof(float4) * pieces) != cudaSuccess) {
-                cudaGetLastError();
-                s.d_sums = nullptr;
-                slices = false;                                   // no memory: clusters
-            } else {
-                for (int i : ids) s.h_mats[i].D = s.d_sums + 4 * at[i];
-            }
-        }
+        const bool slices = !deterministic_flag().load() && best_per > 0 && (join ? join == 2 : least < (per_sm == 2 ? 0.63 : 1.0) * shortest);
         int64_t longest = 1;
-        for (int i : ids) {
-            const int64_t parts = slices ? parts_of(i, best_per, 0) : split[i];
-            longest = std::max(longest, (steps_of(i, 0) + parts - 1) / parts);
-        }
-        if (slices) cluster = 1;
+        for (int i : ids) longest = std::max(longest, (steps_of(i, 0) + split[i] - 1) / split[i]);
         if (!gen_k1_shape(s.plan, s.f32, s.r, T, true, cluster > 1, per_sm, longest)) return FLORA_ERR_UNSUPPORTED;
         s.plan.cluster = cluster;
         std::vector<GenItem> items;
-        std::vector<FoldItem> fold;
         for (int64_t pass = 0; pass < passes; ++pass) {
             cuts.clear();
-            s.fold_begin.push_back((int)fold.size());
             for (int i : ids) {
-                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass);
-                const int32_t col0 = s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0;
+                const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass), per = (int64_t)(cluster / split[i]) * T;
                 if (pass > 0 && steps == 0) continue;
-                if (slices) {
-                    const int64_t parts = parts_of(i, best_per, pass);
-                    for (int64_t t0 = 0; t0 < tiles; ++t0)
-                        for (int64_t part = 0; part < parts; ++part) cuts.push_back({i, (steps + parts - 1) / parts, {i, (int32_t)t0, (int32_t)parts, col0, (int32_t)part}});
-                    if (parts > 1)
-                        fold_cut(fold, FoldMat{s.h_mats[i].S, s.h_mats[i].D, s.h_mats[i].lds, (int32_t)big[i].rows, 0, (int32_t)parts, 0},
-                                 fold_slice(big[i].rows, s.r), fold_pieces_of_set(parts));
-                } else {
-                    const int64_t per = (int64_t)(cluster / split[i]) * T;
-                    for (int64_t t0 = 0; t0 < tiles; t0 += per)
-                        cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]), {i, (int32_t)t0, split[i], col0, 0}});
-                }
+                for (int64_t t0 = 0; t0 < tiles; t0 += per)
+                    cuts.push_back({i, std::min<int64_t>(T, tiles - t0) * ((steps + split[i] - 1) / split[i]),
+                                    {i, (int32_t)t0, split[i], s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0, 0}});
             }
-            launches_of([&](const Cut& c) { items.push_back(c.item); });
+            launches_of(s.begin, s.first_mat, [&](const Cut& c) { items.push_back(c.item); });
             s.pass_end.push_back((int)s.begin.size());
         }
         s.begin.push_back(count);
-        s.fold_begin.push_back((int)fold.size());
-        rc = upload(&s.d_k1, items, st);
-        if (rc == FLORA_OK && slices) rc = upload(&s.d_mats, s.h_mats, st);
-        return rc ? rc : upload(&s.d_fold, fold, st);
+        if (slices) {
+            int64_t pieces = 0;
+            longest = 1;
+            for (int i : ids) {
+                const int64_t parts = parts_of(i, best_per, 0);
+                s.h_mats[i].slices = pieces;
+                if (parts > 1) pieces += parts * fold_slice(big[i].rows, s.r);
+                longest = std::max(longest, (steps_of(i, 0) + parts - 1) / parts);
+            }
+            s.sums_bytes = sizeof(float4) * (size_t)pieces;
+            if (!gen_k1_shape(s.alone, s.f32, s.r, T, true, false, per_sm, longest)) return FLORA_ERR_UNSUPPORTED;
+            s.alone.workers = s.plan.workers;
+            s.alone.aligned = s.plan.aligned;
+            std::vector<GenItem> alone;
+            std::vector<FoldItem> fold;
+            count = 0;
+            for (int64_t pass = 0; pass < passes; ++pass) {
+                cuts.clear();
+                s.fold_begin.push_back((int)fold.size());
+                for (int i : ids) {
+                    const int64_t tiles = (big[i].rows + 127) / 128, steps = steps_of(i, pass), parts = parts_of(i, best_per, pass);
+                    if (pass > 0 && steps == 0) continue;
+                    for (int64_t t0 = 0; t0 < tiles; ++t0)
+                        for (int64_t part = 0; part < parts; ++part)
+                            cuts.push_back({i, (steps + parts - 1) / parts, {i, (int32_t)t0, (int32_t)parts, s.f32 ? (int32_t)(pass * GEN_F32_PASS_COLS) : 0, (int32_t)part}});
+                    if (parts > 1)
+                        fold_cut(fold, FoldMat{s.h_mats[i].S, 4 * s.h_mats[i].slices, s.h_mats[i].lds, (int32_t)big[i].rows, 0, (int32_t)parts, 0},
+                                 fold_slice(big[i].rows, s.r), fold_pieces_of_set(parts));
+                }
+                launches_of(s.alone_begin, s.alone_first, [&](const Cut& c) { alone.push_back(c.item); });
+                s.alone_pass_end.push_back((int)s.alone_begin.size());
+            }
+            s.alone_begin.push_back(count);
+            s.fold_begin.push_back((int)fold.size());
+            rc = upload(&s.d_alone, alone, st);
+            if (rc == FLORA_OK) rc = upload(&s.d_fold, fold, st);
+            if (rc == FLORA_OK) rc = upload(&s.d_mats, s.h_mats, st);
+            if (rc) return rc;
+        }
+        return upload(&s.d_k1, items, st);
     }
     // decompression: equal, contiguous shares of the (slab, tile) units of each launch's matrices
     bool aligned = true;
@@ -618,20 +632,27 @@ inline SeedTable gen_seeds(const GenSet& s, const uint64_t* seeds, int base)
 inline flora_status gen_set_compress(GenSet& s, const uint64_t* seeds, float a, float b, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
     if (s.ready() && s.plan.aligned && !s.captured_aligned) s.captured_aligned = capturing(st);
-    size_t l = 0;
-    for (size_t pass = 0; pass < s.pass_end.size(); ++pass) {
-        const float scale = pass ? 1.0f : b;
-        for (; (int)l < s.pass_end[pass]; ++l) {
-            const flora_status rc = gen_compress_launch(s.f32, s.plan, s.begin[l + 1] - s.begin[l], s.d_mats, s.d_k1 + s.begin[l],
-                                                        gen_seeds(s, seeds, s.first_mat[l]), GenMat{}, 1, 0, s.first_mat[l], s.r, a, scale, st, launches);
-            if (rc) return rc;
-        }
-        const int first = s.fold_begin[pass], items = s.fold_begin[pass + 1] - first;
-        if (items == 0) continue;
-        const flora_status rc = fold_launch(true, s.d_fold + first, items, FoldMat{}, 0, 0, s.r, a, scale, sm_count(), st, launches);
-        if (rc) return rc;
+    // (clusters where the call is recorded into a graph and where there is no memory for the sums)
+    void* sums = nullptr;
+    bool alone = s.d_alone && !capturing(st);
+    if (alone && s.sums_bytes && scratch_alloc(&sums, s.sums_bytes, st) != cudaSuccess) {
+        cudaGetLastError();
+        alone = false;
     }
-    return FLORA_OK;
+    const std::vector<int>&begin = alone ? s.alone_begin : s.begin, &first_mat = alone ? s.alone_first : s.first_mat, &pass_end = alone ? s.alone_pass_end : s.pass_end;
+    const GenItem* const items = alone ? s.d_alone : s.d_k1;
+    flora_status rc = FLORA_OK;
+    size_t l = 0;
+    for (size_t pass = 0; pass < pass_end.size() && rc == FLORA_OK; ++pass) {
+        const float scale = pass ? 1.0f : b;
+        for (; (int)l < pass_end[pass] && rc == FLORA_OK; ++l)
+            rc = gen_compress_launch(s.f32, alone ? s.alone : s.plan, begin[l + 1] - begin[l], s.d_mats, items + begin[l], (float4*)sums, gen_seeds(s, seeds, first_mat[l]),
+                                     GenMat{}, 1, 0, first_mat[l], s.r, a, scale, st, launches);
+        const int first = alone ? s.fold_begin[pass] : 0, folds = alone ? s.fold_begin[pass + 1] - first : 0;
+        if (rc == FLORA_OK && folds) rc = fold_launch(true, (const float*)sums, s.d_fold + first, folds, FoldMat{}, 0, 0, s.r, a, scale, sm_count(), st, launches);
+    }
+    if (sums && cudaFreeAsync(sums, st) != cudaSuccess && rc == FLORA_OK) rc = FLORA_ERR_CUDA;
+    return rc;
 }
 inline flora_status gen_set_decompress(const GenSet& s, const uint64_t* seeds, float step, cudaStream_t st, std::atomic<uint64_t>& launches)
 {
@@ -661,7 +682,7 @@ inline flora_status gen_set_rebind(GenSet& s, const std::vector<flora_mat>& big,
         s.h_mats[i].big = big[i].data;
         aligned = aligned && gen_aligned(big[i]);
     }
-    s.plan.aligned = aligned;
+    s.plan.aligned = s.alone.aligned = aligned;
     return upload(&s.d_mats, s.h_mats, st);
 }
 
