@@ -14,6 +14,7 @@
 #include <mutex>
 #include <new>
 
+#include "flora_fold.cuh"
 #include "flora_pair.cuh"
 #include "flora_pair_k2.cuh"
 #include "flora_pool.cuh"
@@ -1128,7 +1129,8 @@ inline flora_status tc_compress_launch(const TcSet& set, const TcMatrix* mats, c
         // rows that receive adds (from several CTAs, or from the pair kernel's reducing write-out): scale them by b first
         const size_t total = SINGLE ? 1 : scale_all ? set.members.size() : set.split_mats.size();
         const int* ids = scale_all ? set.d_members : set.d_split;        // (no list: every matrix of the set)
-        const flora_status rc = tc_scale_launch<SINGLE>(mats, one, ids, total, SINGLE ? state_bytes / 4 : most_sketch(set), r, b, early, st, launches);
+        // (ranks that are no multiple of four: sums in scratch, rows fold_ld(r) apart, which are cleared as they lie)
+        const flora_status rc = tc_scale_launch<SINGLE>(mats, one, ids, total, SINGLE ? state_bytes / 4 : most_sketch(set), b == 0.0f ? fold_ld(r) : r, b, early, st, launches);
         if (rc) return rc;
         if (scale_all) b = 1.0f;
     }
