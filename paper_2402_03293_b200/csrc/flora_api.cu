@@ -195,8 +195,12 @@ bool small_decompress(int64_t elements, int r, bool f32, bool loose)
 bool use_tc_compress(const flora_mat* big, const flora_mat* sketch, void* stream)
 {
     if (!sketch_writable(*sketch) && capturing(as_stream(stream))) return false;
-    return g_force_path.load(std::memory_order_relaxed) != 1 && tc_compress_supported(big, sketch) &&
-           !small_compress(big->rows * big->cols, big->cols, (int)sketch->cols, big->dtype == FLORA_F32, false);
+    if (g_force_path.load(std::memory_order_relaxed) == 1 || !tc_compress_supported(big, sketch)) return false;
+    // (neither for matrices a little above the size up to which those are the quicker)
+    if (big->dtype == FLORA_BF16 && sketch->cols <= 64 && big->cols <= 5120 && big->rows * big->cols <= 10 << 20 && g_force_path.load(std::memory_order_relaxed) != 2 &&
+        capturing(as_stream(stream)))
+        return false;
+    return !small_compress(big->rows * big->cols, big->cols, (int)sketch->cols, big->dtype == FLORA_F32, false);
 }
 bool use_tc_decompress(const flora_mat* big, const flora_mat* sketch, void* stream)
 {

@@ -106,7 +106,7 @@ __device__ __forceinline__ void store_quad(uint32_t addr, uint32_t part_bytes, f
 // 64 bf16 values) at a time.  Worker warps fetch the rows with plain 16-byte loads, two tiles ahead in registers (rows that start
 // off a 16-byte boundary: two aligned loads per piece, shifted together), cut fp32 values into parts and write operand
 // tiles; the same warps generate the step's tile of A while the loads are under way.  One thread issues the MMAs.
-// Where a matrix has too few rows to fill the GPU, `split` CTAs share its columns and add their sums to the sketch (GenJoin).
+// Where a matrix has too few rows to fill the GPU, `split` CTAs share its columns and bring their sums together (GenJoin).
 // ------------------------------------------------------------------------------------------------
 template <bool F32>
 struct GenK1 {

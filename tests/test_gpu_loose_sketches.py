@@ -156,3 +156,36 @@ def test_no_memory_for_the_copy_of_the_sketches():
         A = torch.empty(1, m, device=DEV)
         fb.flora_materialize_A(A, 3 + i)
         assert torch.equal(W[i], (-0.5 * A.bfloat16().float()).bfloat16().expand_as(W[i]))
+
+
+@pytest.mark.parametrize("r,ld", [(61, 64), (30, 32), (7, 8), (101, 104), (253, 256)])
+def test_what_lies_behind_a_row_is_not_read(r, ld):
+    """Ranks that are no multiple of four, rows 16 bytes apart: TMA reads such a sketch, and what is behind its rows (NaN) stays out of the weights."""
+    n, m = 256, 1024
+    buf = torch.full((n, ld), float("nan"), device=DEV)
+    S = buf[:, :r]
+    S.copy_(torch.randn(n, r, generator=torch.Generator().manual_seed(1)))
+    W = wl.gaussian_matrix(n, m, 4e-4, "bf16", 6).to(DEV)
+    W0 = W.clone()
+    fb.flora_decompress_apply(W, S, 14, 0.03, 1.0)
+    _weights_match(W, W0, S, 14, 0.03)
+    assert buf[:, r:].isnan().all()
+
+
+@pytest.mark.parametrize("n,m,r", [(2564, 4048, 48), (8200, 1016, 64)])
+def test_first_compressions_of_a_shape_inside_a_graph(n, m, r):
+    """Matrices a little above the size up to which the general kernels are the quicker: calls that a graph records first need no plan."""
+    fb.flora_debug_force_path(0)                                      # (shapes of their own: no plan of another test)
+    G, S = wl.gaussian_matrix(n, m, 1e-2, "bf16", 1).to(DEV), torch.zeros(n, r, device=DEV)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        fb.flora_momentum_step(G, S, 0.0, 3)
+        fb.flora_compress_accumulate(G, S, 3, r)
+    G2 = wl.gaussian_matrix(n, m, 1e-2, "bf16", 4).to(DEV)
+    G.copy_(G2)
+    graph.replay()
+    rows = np.arange(0, n, 257)
+    want = 2.0 * oracle_compress(G2[rows].contiguous(), torch.zeros(len(rows), r), 3)
+    assert rel_err(S[rows].cpu().numpy(), want) <= TOL["f32"]
+    del graph
