@@ -45,6 +45,10 @@
  *    flora_set_rebind_gradients and a single-matrix call that plans upload
  *    small tables from ordinary host memory that the call does not keep;
  *    do not record these into a CUDA graph.
+ *  - Scratch: a compression or an update may borrow some from the stream-ordered pool that the library owns, for
+ *    sums of parts of the columns (48 MB at most), sums beside a sketch that TMA cannot address or a copy of the
+ *    sketch.  A compression does without where there is none, and so does an update unless r > 64 and TMA can address
+ *    W and the sketch.
  *  - Errors are reported by the returned status only; arguments are checked
  *    before anything is launched, and a failed check launches nothing.
  *  - A[j,k] depends on (seed, j, k) only and on r only through the factor
@@ -165,9 +169,12 @@ typedef struct flora_set flora_set;
 
 /* count matrices; G[i] and W[i] are n_i x m_i with equal shape and dtype, S[i] (the sketch C or
  * M) is n_i x r f32 with the same r for all i.  W may be NULL if flora_set_decompress_apply is
- * never called, G may be NULL if no compression is.  Allocates a few hundred bytes of device
- * memory per matrix (descriptors and work lists) that flora_set_destroy frees.  The arrays
- * themselves are host memory and are copied. */
+ * never called, G may be NULL if no compression is.  Allocates device memory that flora_set_destroy
+ * frees: a few hundred bytes per matrix (descriptors and work lists); of bf16 weights above r = 64 a
+ * copy of their sketches, n x ceil(r/64)*64 x 2 bytes each, and three times that at any rank where
+ * TMA cannot address the sketch; of bf16 gradients, where it cannot, sums beside the sketch, as large as
+ * it.  Without memory for these sums or for three-part copies the set is made without them and is
+ * slower.  The arrays themselves are host memory and are copied. */
 flora_status flora_set_create(int count, const flora_mat* G, const flora_mat* W, const flora_mat* S, flora_set** out);
 flora_status flora_set_destroy(flora_set* set);
 
@@ -227,8 +234,8 @@ flora_status flora_set_read_weights_to_host(flora_set* set, void* const* host_W,
  * ------------------------------------------------------------------------------------------- */
 /* A is a function of (seed, j, k) alone, so every result is reproducible up to the order of floating-point
  * additions.  By default the work of one matrix may be split over CTAs that add their partial sums in arrival
- * order (compression over column ranges of a wide matrix; the r x r product of the transfer over column ranges),
- * which can change the last bits from run to run.  on != 0: sets created from now on give every row of a sketch a
+ * order (compression over column ranges of a wide matrix that TMA serves; the r x r product of the transfer over column
+ * ranges), which can change the last bits from run to run.  on != 0: sets created from now on give every row of a sketch a
  * single owner, and every transfer from now on sums its r x r product in one CTA per matrix, so that repeated runs
  * on the same inputs are bit-identical (slower on few, wide matrices).  (The r x r product of a single bf16 matrix is summed by up to
  * four clusters of CTAs and added up in a fixed order; that of a member of a set, or of fp32 operands, by one CTA per tile of it.)  Process-wide; default off. */
